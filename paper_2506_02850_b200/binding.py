@@ -1,15 +1,20 @@
-"""Thin ctypes binding of ``libmetok.so``: argument marshalling only.
+"""Thin binding of ``libmetok.so``: argument marshalling only.
 
 Every function here has the name of the C entry point it calls
 (``include/metok.h``), allocates the output tensors and the workspace with
 torch, passes raw device pointers and the current CUDA stream, and returns the
 outputs.  Nothing is computed in Python and there is no fallback: if the
 library is missing, or a call returns an error status, an exception is raised.
+
+The calls a program makes per video, per pruning layer and per cache go through
+``lib/_metok_calls.so`` (``csrc/host/calls.cpp``), which marshals natively; the
+others, and every symbol of the library for its own sake, through ctypes.
 """
 
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Dict, List, Optional, Sequence
 
@@ -17,6 +22,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "lib", "libmetok.so")
+CALLS_PATH = os.path.join(_PKG, "lib", "_metok_calls.so")
 
 F32, BF16 = 0, 1
 SIM_FLATTEN, SIM_MEANPOOL = 0, 1
@@ -110,6 +116,26 @@ def lib():
     return _lib_handle
 
 
+_calls_module = None
+_calls_bound = None                      # the library whose entry points the native calls use
+
+
+def _calls():
+    """The native calls, on the entry points of the library that lib() returns."""
+    global _calls_module, _calls_bound
+    h = _lib_handle if _lib_handle is not None else lib()
+    if h is not _calls_bound:
+        if _calls_module is None:
+            if not os.path.exists(CALLS_PATH):
+                raise RuntimeError(f"{CALLS_PATH} is missing: build it with `python -m paper_2506_02850_b200.build`")
+            spec = importlib.util.spec_from_file_location("_metok_calls", CALLS_PATH)
+            _calls_module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(_calls_module)
+        _calls_module.bind({name: _c.cast(getattr(h, name), _vp).value for name in _SIGNATURES})
+        _calls_bound = h
+    return _calls_module
+
+
 def _check(fn: str, status: int) -> None:
     if status != 0:
         L = lib()
@@ -140,18 +166,11 @@ def _cuda_contig(t: torch.Tensor, name: str) -> torch.Tensor:
     return t
 
 
-_ws_cache: Dict[tuple, torch.Tensor] = {}
-
-
 def workspace(nbytes: int, device) -> torch.Tensor:
     """A reusable scratch buffer per device and stream: calls on one stream never overlap,
     calls on different streams may, so they must not share scratch."""
-    key = (str(device), torch.cuda.current_stream(device).cuda_stream)
-    buf = _ws_cache.get(key)
-    if buf is None or buf.numel() < nbytes:
-        buf = torch.empty(max(nbytes, 1 << 20), dtype=torch.uint8, device=device)
-        _ws_cache[key] = buf
-    return buf
+    index = torch.device(device).index
+    return _calls().workspace(nbytes, torch.cuda.current_device() if index is None else index)
 
 
 # --------------------------------------------------------------------------- #
@@ -160,24 +179,10 @@ def workspace(nbytes: int, device) -> torch.Tensor:
 def metok_segment_events(feats: torch.Tensor, k: int, sim_mode: int = SIM_FLATTEN,
                          out: Optional[Dict[str, torch.Tensor]] = None) -> Dict[str, torch.Tensor]:
     """`out` (a dict returned by an earlier call with the same shapes) reuses its buffers."""
-    feats = _cuda_contig(feats, "feats")
-    T, N, d = feats.shape
-    dev = feats.device
-    L = lib()
-    if out is not None:
-        sims, boundaries, offsets, frame_event = out["_sims"], out["_boundaries"], out["_offsets"], out["frame_event"]
-    else:
-        sims = torch.empty(max(T - 1, 1), dtype=torch.float32, device=dev)
-        boundaries = torch.empty(max(k - 1, 1), dtype=torch.int32, device=dev)
-        offsets = torch.empty(max(k + 1, 2), dtype=torch.int32, device=dev)
-        frame_event = torch.empty(T, dtype=torch.int32, device=dev)
-    need = L.metok_segment_events_workspace_bytes(_dt(feats), T, N, d, sim_mode)
-    ws = workspace(need, dev)
-    st = L.metok_segment_events(_ptr(feats), _dt(feats), T, N, d, k, sim_mode, _ptr(sims), _ptr(boundaries),
-                                _ptr(offsets), _ptr(frame_event), _ptr(ws), ws.numel(), _stream())
-    _check("metok_segment_events", st)
-    return {"sims": sims[: T - 1], "boundaries": boundaries[: max(k - 1, 0)], "event_offsets": offsets[: k + 1],
-            "frame_event": frame_event, "_sims": sims, "_boundaries": boundaries, "_offsets": offsets}
+    res = _calls().segment_events(feats, k, sim_mode, out)
+    if type(res) is int:
+        _check("metok_segment_events", res)
+    return res
 
 
 def metok_segment_events_static(feats: torch.Tensor, k: int, sim_mode: int = SIM_FLATTEN) -> Dict[str, torch.Tensor]:
@@ -202,31 +207,10 @@ def metok_segment_score_events(feats: torch.Tensor, k: int, text_emb: torch.Tens
                                out: Optional[Dict[str, torch.Tensor]] = None) -> Dict[str, torch.Tensor]:
     """metok_segment_events (FLATTEN) plus the per-token text relevance and inverse norms of the
     same pass over `feats`; hand "token_score" / "token_inv_norm" on to metok_compress_vision."""
-    feats = _cuda_contig(feats, "feats")
-    text_emb = _cuda_contig(text_emb, "text_emb")
-    T, N, d = feats.shape
-    dev = feats.device
-    L = lib()
-    if out is None:
-        out = {
-            "_sims": torch.empty(max(T - 1, 1), dtype=torch.float32, device=dev),
-            "_boundaries": torch.empty(max(k - 1, 1), dtype=torch.int32, device=dev),
-            "_offsets": torch.empty(max(k + 1, 2), dtype=torch.int32, device=dev),
-            "frame_event": torch.empty(T, dtype=torch.int32, device=dev),
-            "token_score": torch.empty(T * N, dtype=torch.float32, device=dev),
-            "token_inv_norm": torch.empty(T * N, dtype=torch.float32, device=dev),
-        }
-    need = L.metok_segment_score_events_workspace_bytes(_dt(feats), T, N, d)
-    ws = workspace(need, dev)
-    st = L.metok_segment_score_events(_ptr(feats), _dt(feats), T, N, d, k, _ptr(text_emb), _ptr(out["_sims"]),
-                                      _ptr(out["_boundaries"]), _ptr(out["_offsets"]), _ptr(out["frame_event"]),
-                                      _ptr(out["token_score"]), _ptr(out["token_inv_norm"]), _ptr(ws), ws.numel(),
-                                      _stream())
-    _check("metok_segment_score_events", st)
-    out["sims"] = out["_sims"][: T - 1]
-    out["boundaries"] = out["_boundaries"][: max(k - 1, 0)]
-    out["event_offsets"] = out["_offsets"][: k + 1]
-    return out
+    res = _calls().segment_score_events(feats, k, text_emb, out)
+    if type(res) is int:
+        _check("metok_segment_score_events", res)
+    return res
 
 
 def vision_params(alpha: float, keep_key: float = 1.0, keep_nonkey: float = 1.0, event_agg: int = AGG_MEAN,
@@ -251,97 +235,29 @@ def metok_compress_vision(feats: torch.Tensor, event_offsets: torch.Tensor, text
                           key_frames: Optional[torch.Tensor] = None) -> Dict[str, torch.Tensor]:
     """`scored` (the result of metok_segment_score_events on the same feats and text) makes the call
     skip its own scoring pass over `feats`; `key_events` (uint8 [k] on the device) replaces the
-    call's own choice of key events, `key_frames` (uint8 [T], mode POOL) that of key frames."""
-    feats = _cuda_contig(feats, "feats")
-    event_offsets = _cuda_contig(event_offsets, "event_offsets")
-    text_emb = _cuda_contig(text_emb, "text_emb")
-    T, N, d = feats.shape
-    k = event_offsets.numel() - 1
-    dev = feats.device
-    L = lib()
-    if cap is None:
-        cap = metok_compress_vision_bound(T, N, k, p)
-    i32 = dict(dtype=torch.int32, device=dev)
-    if out is not None:
-        cap = out["out_src"].numel()
-    else:
-        out = {
-            "out_feats": torch.empty((cap, d), dtype=feats.dtype, device=dev),
-            "out_src": torch.empty(cap, **i32), "out_event": torch.empty(cap, **i32),
-            "out_members": torch.empty(cap, **i32), "assign": torch.empty(T * N, **i32),
-            "token_score": torch.empty(T * N, dtype=torch.float32, device=dev),
-            "frame_score": torch.empty(T, dtype=torch.float32, device=dev),
-            "event_score": torch.empty(k, dtype=torch.float32, device=dev),
-            "event_is_key": torch.empty(k, dtype=torch.uint8, device=dev),
-            "n_out": torch.zeros(1, **i32),
-        }
-    if scored is not None:
-        out["token_score"] = scored["token_score"]
-        p = VisionParams.from_buffer_copy(p)
-        p.token_inv_norm = scored["token_inv_norm"].data_ptr()
-    if key_events is not None:
-        key_events = _cuda_contig(key_events, "key_events")
-        if key_events.dtype != torch.uint8 or key_events.numel() != k:
-            raise ValueError("key_events must be uint8 [k]")
-        p = VisionParams.from_buffer_copy(p)
-        p.key_events_given = key_events.data_ptr()
-    if key_frames is not None:
-        key_frames = _cuda_contig(key_frames, "key_frames")
-        if key_frames.dtype != torch.uint8 or key_frames.numel() != T:
-            raise ValueError("key_frames must be uint8 [T]")
-        p = VisionParams.from_buffer_copy(p)
-        p.key_frames_given = key_frames.data_ptr()
-    need = L.metok_compress_vision_workspace_bytes(_dt(feats), T, N, d, k, cap, _c.byref(p))
-    ws = workspace(need, dev)
-    st = L.metok_compress_vision(_ptr(feats), _dt(feats), T, N, d, _ptr(event_offsets), k, _ptr(text_emb),
-                                 _c.byref(p), _ptr(out["out_feats"]), _ptr(out["out_src"]), _ptr(out["out_event"]),
-                                 _ptr(out["out_members"]), _ptr(out["assign"]), _ptr(out["token_score"]),
-                                 _ptr(out["frame_score"]), _ptr(out["event_score"]), _ptr(out["event_is_key"]),
-                                 _ptr(out["n_out"]), cap, _ptr(ws), ws.numel(), _stream())
-    _check("metok_compress_vision", st)
-    out["status"] = ws[:4].view(torch.int32)      # device status word (0, or -5 after a device-side timeout)
-    return out
+    call's own choice of key events, `key_frames` (uint8 [T], mode POOL) that of key frames.
+    "status" is the device status word (0, or -5 after a device-side timeout)."""
+    res = _calls().compress_vision(feats, event_offsets, text_emb, p, cap, out, scored, key_events, key_frames)
+    if type(res) is int:
+        _check("metok_compress_vision", res)
+    return res
 
 
 def metok_retention_budgets(alpha: float, r: float, stage: int, N0: Sequence[int]) -> List[int]:
-    n0 = (_c.c_int32 * 2)(int(N0[0]), int(N0[1]))
-    out = (_c.c_int32 * 2)()
-    _check("metok_retention_budgets", lib().metok_retention_budgets(alpha, r, stage, n0, out))
-    return [int(out[0]), int(out[1])]
+    res = _calls().retention_budgets(alpha, r, stage, N0)
+    if type(res) is int:
+        _check("metok_retention_budgets", res)
+    return res
 
 
 def metok_prefill_prune(q_text: torch.Tensor, k_all: torch.Tensor, hidden: Optional[torch.Tensor], vis_start: int,
                         n_vis: int, token_group: torch.Tensor, group_budget: Sequence[int], softmax_scale: float,
                         out: Optional[Dict[str, torch.Tensor]] = None) -> Dict[str, torch.Tensor]:
-    q_text = _cuda_contig(q_text, "q_text")
-    k_all = _cuda_contig(k_all, "k_all")
-    token_group = _cuda_contig(token_group, "token_group")
-    Hq, Lt, dh = q_text.shape
-    Hkv, S, _ = k_all.shape
-    dev = q_text.device
-    D = 0
-    if hidden is not None:
-        hidden = _cuda_contig(hidden, "hidden")
-        D = hidden.shape[1]
-    L = lib()
-    G = len(group_budget)
-    budgets = (_c.c_int32 * G)(*[int(b) for b in group_budget])
-    if out is None:
-        out = {
-            "scores": torch.empty(n_vis, dtype=torch.float32, device=dev),
-            "keep_idx": torch.empty(S, dtype=torch.int32, device=dev),
-            "S_out": torch.zeros(1, dtype=torch.int32, device=dev),
-            "hidden_out": None if hidden is None else torch.empty_like(hidden),
-        }
-    need = L.metok_prefill_prune_workspace_bytes(_dt(q_text), Hq, Hkv, Lt, S, dh, n_vis)
-    ws = workspace(need, dev)
-    st = L.metok_prefill_prune(_ptr(q_text), _ptr(k_all), _ptr(hidden), _dt(q_text), Hq, Hkv, Lt, S, dh, D, vis_start,
-                               n_vis, _ptr(token_group), G, budgets, softmax_scale, _ptr(out["scores"]),
-                               _ptr(out["keep_idx"]), _ptr(out["S_out"]), _ptr(out["hidden_out"]), _ptr(ws),
-                               ws.numel(), _stream())
-    _check("metok_prefill_prune", st)
-    out["status"] = ws[:4].view(torch.int32)      # device status word (0, or -5 after a device-side timeout)
-    return out
+    """"status" is the device status word (0, or -5 after a device-side timeout)."""
+    res = _calls().prefill_prune(q_text, k_all, hidden, vis_start, n_vis, token_group, group_budget, softmax_scale, out)
+    if type(res) is int:
+        _check("metok_prefill_prune", res)
+    return res
 
 
 def metok_attention_scores(q_text: torch.Tensor, k_all: torch.Tensor, vis_start: int, n_vis: int,
@@ -432,48 +348,14 @@ def metok_prefill_prune_schedule(q_texts: Sequence[torch.Tensor], k_alls: Sequen
     """The pruning levels chained in one call: per level the tensors of that layer (rows of the
     survivors of the level before, in order).  Returns one dict per level."""
     n_levels = len(q_texts)
-    token_group = _cuda_contig(token_group, "token_group")
-    n_vis = token_group.numel()
-    sizes = metok_prune_schedule_sizes(n_levels, alpha, r, N0)
-    Hq, Lt, dh = q_texts[0].shape
-    Hkv, S, _ = k_alls[0].shape
-    dev = token_group.device
-    D = 0 if hiddens is None else hiddens[0].shape[1]
-    i32 = dict(dtype=torch.int32, device=dev)
-    outs: List[Dict[str, torch.Tensor]] = []
     arr = (PruneLevel * n_levels)()
-    for s in range(n_levels):
-        q, k_ = _cuda_contig(q_texts[s], "q_text"), _cuda_contig(k_alls[s], "k_all")
-        S_s = S - n_vis + sizes[s]
-        if tuple(k_.shape) != (Hkv, S_s, dh):
-            raise ValueError(f"level {s + 1}: k_all must be {(Hkv, S_s, dh)}, got {tuple(k_.shape)}")
-        h = None if hiddens is None else _cuda_contig(hiddens[s], "hidden")
-        o = {
-            "scores": torch.empty(max(sizes[s], 1), dtype=torch.float32, device=dev),
-            "keep_idx": torch.empty(S_s, **i32), "S_out": torch.zeros(1, **i32),
-            "hidden_out": None if h is None else torch.empty_like(h),
-            "token_group": token_group if s == 0 else torch.empty(max(sizes[s], 1), **i32),
-            "origin": torch.empty(max(sizes[s], 1), **i32), "n_vis": sizes[s], "S": S_s,
-        }
-        arr[s] = PruneLevel(q.data_ptr(), k_.data_ptr(), None if h is None else h.data_ptr(),
-                            None if h is None else o["hidden_out"].data_ptr(), o["scores"].data_ptr(),
-                            o["keep_idx"].data_ptr(), o["S_out"].data_ptr(), o["token_group"].data_ptr(),
-                            o["origin"].data_ptr())
-        o["_inputs"] = (q, k_, h)                               # keep the tensors alive until the caller is done
-        outs.append(o)
-    n0 = (_c.c_int32 * 2)(int(N0[0]), int(N0[1]))
-    L = lib()
-    need = L.metok_prefill_prune_schedule_workspace_bytes(n_levels, _dt(q_texts[0]), Hq, Hkv, Lt, S, dh, n_vis, alpha, r, n0)
-    if need == 0:
-        _check("metok_prefill_prune_schedule", -1)
-    ws = workspace(need, dev)
-    status = torch.zeros(1, **i32)
-    st = L.metok_prefill_prune_schedule(arr, n_levels, _dt(q_texts[0]), Hq, Hkv, Lt, S, dh, D, vis_start, n_vis, alpha, r,
-                                        n0, softmax_scale, _ptr(status), _ptr(ws), ws.numel(), _stream())
-    _check("metok_prefill_prune_schedule", st)
+    outs = _calls().prefill_prune_schedule(q_texts, k_alls, hiddens, vis_start, token_group, alpha, r, N0, softmax_scale, arr)
+    if type(outs) is int:
+        _check("metok_prefill_prune_schedule", outs)
+    n_vis = token_group.numel()
+    plan = (arr, n_levels, k_alls[0].shape[1], n_vis, alpha, r, (_c.c_int32 * 2)(int(N0[0]), int(N0[1])))
     for o in outs:
-        o["status"] = status
-        o["_schedule"] = (arr, n_levels, S, n_vis, alpha, r, n0)
+        o["_schedule"] = plan
     return outs
 
 
@@ -499,30 +381,11 @@ def metok_kv_compact(k_layers: Sequence[torch.Tensor], v_layers: Sequence[torch.
                      scores: Optional[torch.Tensor] = None, keep_idx: Optional[torch.Tensor] = None,
                      keep_len: Optional[torch.Tensor] = None,
                      new_len: Optional[torch.Tensor] = None) -> Dict[str, torch.Tensor]:
-    nl = len(k_layers)
-    for t in list(k_layers) + list(v_layers):
-        _cuda_contig(t, "k/v layer")
-    Hkv, S_cap, dh = k_layers[0].shape
-    dev = k_layers[0].device
-    L = lib()
-    karr = (_vp * nl)(*[t.data_ptr() for t in k_layers])
-    varr = (_vp * nl)(*[t.data_ptr() for t in v_layers])
-    if keep_idx is None:
-        keep_idx = torch.empty((nl, S_cur), dtype=torch.int32, device=dev)
-        keep_len = torch.zeros(nl, dtype=torch.int32, device=dev)
-    if new_len is None:
-        new_len = torch.zeros(nl, dtype=torch.int32, device=dev)
-    per_layer = 0
-    if scores is not None:
-        scores = _cuda_contig(scores, "scores")
-        per_layer = 1 if scores.dim() == 2 else 0
-    need = L.metok_kv_compact_workspace_bytes(_dt(k_layers[0]), nl, Hkv, S_cur, dh, policy, n_vis)
-    ws = workspace(need, dev)
-    st = L.metok_kv_compact(karr, varr, _dt(k_layers[0]), nl, Hkv, S_cap, S_cur, dh, policy, l1, keep_ratio,
-                            vis_start, n_vis, _ptr(scores), per_layer, _ptr(keep_idx), _ptr(keep_len),
-                            _ptr(new_len), _ptr(ws), ws.numel(), _stream())
-    _check("metok_kv_compact", st)
-    return {"keep_idx": keep_idx, "keep_len": keep_len, "new_len": new_len, "status": ws[:4].view(torch.int32)}
+    res = _calls().kv_compact(k_layers, v_layers, S_cur, policy, vis_start, n_vis, l1, keep_ratio, scores, keep_idx, keep_len,
+                              new_len)
+    if type(res) is int:
+        _check("metok_kv_compact", res)
+    return res
 
 
 def metok_version() -> int:

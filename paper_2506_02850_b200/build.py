@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree: csrc/*.cu -> lib/libmetok.so (sm_100a only).
+"""Builds the CUDA library in-tree: csrc/*.cu -> lib/libmetok.so (sm_100a only), and the native half of
+binding.py: csrc/host/calls.cpp -> lib/_metok_calls.so.
 
 nvcc cross-compiles without a GPU, so this runs on any box with the CUDA toolkit.
 """
@@ -8,6 +9,7 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -18,6 +20,8 @@ LIB = os.path.join(LIBDIR, "libmetok.so")
 # the same sources with short device-side waits, a host switch that withholds one copy, and range checks
 # on every data-dependent index: exercises the time-out and unwind paths a normal run never reaches
 DEBUG_LIB = os.path.join(LIBDIR, "libmetok_debug.so")
+CALLS_SRC = os.path.join(CSRC, "host", "calls.cpp")
+CALLS_LIB = os.path.join(LIBDIR, "_metok_calls.so")
 DEBUG_DEFINES = ["-DMETOK_DEBUG_SHORT_WAIT", "-DMETOK_DEBUG_BOUNDS"]
 
 NVCC_FLAGS = [
@@ -45,8 +49,31 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_calls(force: bool = False, verbose: bool = False) -> str:
+    """Builds lib/_metok_calls.so against the installed torch."""
+    os.makedirs(LIBDIR, exist_ok=True)
+    header = os.path.join(os.path.dirname(PKG), "include", "metok.h")
+    if force or _stale(CALLS_LIB, [CALLS_SRC, header]):
+        from torch.utils import cpp_extension
+        cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+        includes = [sysconfig.get_paths()["include"], os.path.join(cuda, "include")] + cpp_extension.include_paths()
+        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden"]
+        for d in includes:
+            cmd += ["-isystem", d]
+        cmd += [CALLS_SRC, "-o", CALLS_LIB]
+        for d in cpp_extension.library_paths():
+            cmd += ["-L", d]
+        cmd += ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch", "-ltorch_python"]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if verbose or r.returncode != 0:
+            sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+        if r.returncode != 0:
+            raise RuntimeError("compiling the native calls failed: " + " ".join(cmd))
+    return CALLS_LIB
+
+
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, debug: bool = False) -> str:
-    """Builds lib/libmetok.so, or with debug=True lib/libmetok_debug.so (see DEBUG_DEFINES)."""
+    """Builds lib/libmetok.so and lib/_metok_calls.so, or with debug=True lib/libmetok_debug.so (see DEBUG_DEFINES)."""
     objdir = OBJDIR + ("_debug" if debug else "")
     lib = DEBUG_LIB if debug else LIB
     defines = DEBUG_DEFINES if debug else []
@@ -82,6 +109,8 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, 
         if r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
+    if not debug:
+        build_calls(force, verbose)
     return lib
 
 

@@ -1,4 +1,5 @@
 // Host-only helpers of the C ABI: status strings, last CUDA error, version.
+#include <atomic>
 #include <deque>
 #include <mutex>
 #include <string>
@@ -12,6 +13,45 @@
 namespace metok {
 static thread_local int g_last_cuda_error = 0;
 void set_last_cuda_error(int e) { g_last_cuda_error = e; }
+
+namespace {
+// (kernel, device) -> the dynamic shared memory it was last opted in to.  Entries are only ever added (there
+// are a few dozen kernels); readers take no lock.
+struct SmemOptIn { std::atomic<const void*> kernel{nullptr}; std::atomic<int> dev{-1}; std::atomic<size_t> bytes{0}; };
+constexpr int kSmemOptIns = 1024;
+SmemOptIn g_smem[kSmemOptIns];
+std::mutex g_smem_mu;
+}  // namespace
+
+int allow_smem_bytes(const void* kernel, size_t bytes) {
+    int dev = 0;
+    METOK_CUDA_TRY(cudaGetDevice(&dev));
+    const size_t h = (reinterpret_cast<uintptr_t>(kernel) >> 4) * 31 + (size_t)dev;
+    auto find = [&]() -> SmemOptIn* {
+        for (int i = 0; i < kSmemOptIns; ++i) {
+            SmemOptIn& e = g_smem[(h + i) % kSmemOptIns];
+            const void* k = e.kernel.load(std::memory_order_acquire);
+            if (!k) return nullptr;
+            if (k == kernel && e.dev.load(std::memory_order_relaxed) == dev) return &e;
+        }
+        return nullptr;
+    };
+    SmemOptIn* e = find();
+    if (e && e->bytes.load(std::memory_order_acquire) >= bytes) return METOK_OK;
+    std::lock_guard<std::mutex> lk(g_smem_mu);
+    e = find();
+    if (e && e->bytes.load(std::memory_order_acquire) >= bytes) return METOK_OK;   // another thread was faster: never lowered
+    METOK_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    for (int i = 0; !e && i < kSmemOptIns; ++i) {
+        SmemOptIn& f = g_smem[(h + i) % kSmemOptIns];
+        if (f.kernel.load(std::memory_order_relaxed)) continue;
+        f.dev.store(dev, std::memory_order_relaxed);
+        f.kernel.store(kernel, std::memory_order_release);
+        e = &f;
+    }
+    if (e) e->bytes.store(bytes, std::memory_order_release);
+    return METOK_OK;
+}
 
 bool g_profiling = false;
 namespace {

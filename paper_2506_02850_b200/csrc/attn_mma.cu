@@ -479,10 +479,8 @@ int launch_dh(const void* q_text, const void* k_all, const AttnMmaDims& dm, floa
     constexpr int KB = DH / 64;
     const size_t smem_st = (size_t)KB * (kStBM + kStStages * kStBN) * 128 + 1024;
     const size_t smem_cs = (size_t)KB * (dm.cs_nq + kCsStages * kCsBM) * 128 + 1024;
-    METOK_CUDA_TRY(cudaFuncSetAttribute(attn_stats_mma_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem_st));
-    METOK_CUDA_TRY(cudaFuncSetAttribute(attn_colsum_mma_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)((size_t)KB * (kCsMaxNQ + kCsStages * kCsBM) * 128 + 1024)));
+    METOK_ALLOW_SMEM(attn_stats_mma_kernel<DH>, smem_st);
+    METOK_ALLOW_SMEM(attn_colsum_mma_kernel<DH>, ((size_t)KB * (kCsMaxNQ + kCsStages * kCsBM) * 128 + 1024));
     {
         METOK_TIMED("attn_stats_mma_kernel", st);
         launch_chained(attn_stats_mma_kernel<DH>, dim3(dim3(dm.st_nsplit, dm.st_nrt, dm.Hkv)), dim3(kStThreads), smem_st, st, 

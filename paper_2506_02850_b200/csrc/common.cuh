@@ -25,6 +25,17 @@ void set_last_cuda_error(int e);
     } while (0)
 #define METOK_LAUNCH_CHECK() METOK_CUDA_TRY(cudaGetLastError())
 
+// Opts a kernel in to `bytes` of dynamic shared memory on the current device; asks the runtime only when that
+// is more than it was opted in to before (the request costs about as much host time as a third of a launch).
+int allow_smem_bytes(const void* kernel, size_t bytes);
+template <typename K>
+inline int allow_smem(K* kernel, size_t bytes) { return allow_smem_bytes(reinterpret_cast<const void*>(kernel), bytes); }
+#define METOK_ALLOW_SMEM(kernel, bytes)                                              \
+    do {                                                                             \
+        const int _rc = ::metok::allow_smem(kernel, bytes);                          \
+        if (_rc != METOK_OK) return _rc;                                             \
+    } while (0)
+
 // Brackets one kernel launch with CUDA events while profiling is on (see
 // metok_profile_begin); costs one predictable branch otherwise.
 extern bool g_profiling;

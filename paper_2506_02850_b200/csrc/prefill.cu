@@ -346,7 +346,7 @@ int launch_class_topk(const float* scores, size_t score_stride, const int32_t* t
     if (bl.fits) {
         auto kernel = (G == 1 && !token_group) ? block_topk_kernel<true> : block_topk_kernel<false>;
         if (bl.bytes > 32 * 1024)
-            METOK_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bl.bytes));
+            METOK_ALLOW_SMEM(kernel, bl.bytes);
         {
             METOK_TIMED("class_topk_kernel", st);
             launch_chained(kernel, dim3(problems), dim3(kBsThreads), bl.bytes, st, scores, score_stride, token_group, n_vis, G, bl, b, S,
@@ -358,8 +358,7 @@ int launch_class_topk(const float* scores, size_t score_stride, const int32_t* t
     const SelectLayout lay = select_layout(G, select_items_per_cta((long long)S));
     const int nthreads = select_threads(select_items_per_cta((long long)S));
     if (lay.bytes > 32 * 1024)                        // static + dynamic beyond 48 KiB needs the opt-in
-        METOK_CUDA_TRY(cudaFuncSetAttribute(class_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)lay.bytes));
+        METOK_ALLOW_SMEM(class_topk_kernel, lay.bytes);
     {
         METOK_TIMED("class_topk_kernel", st);
         class_topk_kernel<<<problems * kSelCluster, nthreads, lay.bytes, st>>>(
@@ -437,8 +436,7 @@ gather_rows_bulk_kernel(const uint8_t* __restrict__ src, uint8_t* __restrict__ d
 
 int launch_gather_rows_bulk(const void* src, void* dst, const int32_t* idx, const int32_t* n_rows, size_t row_bytes,
                             int src_rows, int32_t* status, const char* timer_name, cudaStream_t st) {
-    METOK_CUDA_TRY(cudaFuncSetAttribute(gather_rows_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)kGbSmemBytes));
+    METOK_ALLOW_SMEM(gather_rows_bulk_kernel, kGbSmemBytes);
     {
         METOK_TIMED(timer_name, st);
         launch_chained(gather_rows_bulk_kernel, dim3(kNumSMs * 6), dim3(32), kGbSmemBytes, st, 
@@ -509,8 +507,8 @@ template <typename T>
 static int launch_attn_scores(const void* q_text, const void* k_all, const AttnDims& dm, const PrefillWs& w,
                               float inv_rows, float* scores, cudaStream_t st) {
     const size_t smem = (size_t)2 * dm.dh * kAtLD * sizeof(float);
-    METOK_CUDA_TRY(cudaFuncSetAttribute(attn_stats_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    METOK_CUDA_TRY(cudaFuncSetAttribute(attn_colsum_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    METOK_ALLOW_SMEM(attn_stats_kernel<T>, smem);
+    METOK_ALLOW_SMEM(attn_colsum_kernel<T>, smem);
     dim3 grid(dm.nsplit, dm.nrt, dm.Hkv);
     {
         METOK_TIMED("attn_stats_kernel", st);

@@ -298,8 +298,7 @@ static int launch_segment(const void* feats, int Tn, int N, int d, int k, int si
     }
     const size_t smem = (size_t)Tn * 3 * sizeof(float);
     if (smem > 48 * 1024) {
-        METOK_CUDA_TRY(cudaFuncSetAttribute(seg_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem));
+        METOK_ALLOW_SMEM(seg_finish_kernel, smem);
     }
     {
         METOK_TIMED("seg_finish_kernel", st);
@@ -646,7 +645,7 @@ seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat1
 template <typename KernelT>
 static int seg_score_runs(KernelT kernel, size_t smem, int Tn, int N, int* frames_per_warp) {
     if (smem > 40 * 1024)
-        METOK_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        METOK_ALLOW_SMEM(kernel, smem);
     int per_sm = 0;
     METOK_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kFsThreads, smem));
     const long long slots = (long long)kNumSMs * (per_sm > 0 ? per_sm : 1) * (kFsThreads / 32);
@@ -670,7 +669,7 @@ static int launch_seg_score(const void* feats, const void* text, int Tn, int N, 
         const size_t smem_t = (size_t)nslice * 4 * sizeof(uint4) + (size_t)(kFsThreads / 32) * kFsDepth * kFsStageBytes;
         auto kernel = (d / 8) % (4 * kFsSlices) == 0 ? seg_score_mma_kernel<true> : seg_score_mma_kernel<false>;
         if (smem_t > 40 * 1024)
-            METOK_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_t));
+            METOK_ALLOW_SMEM(kernel, smem_t);
         nslab = ceil_div(N, kFsThreads / 32);              // the kernel adds the four positions of a CTA
         METOK_TIMED("seg_score_kernel", st);
         launch_chained(kernel, dim3(nslab * ceil_div(Tn, kFsFrames)), dim3(kFsThreads), smem_t, st, 
@@ -689,7 +688,7 @@ static int launch_seg_score(const void* feats, const void* text, int Tn, int N, 
     METOK_LAUNCH_CHECK();
     const size_t smem = (size_t)Tn * 3 * sizeof(float);
     if (smem > 48 * 1024)
-        METOK_CUDA_TRY(cudaFuncSetAttribute(seg_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        METOK_ALLOW_SMEM(seg_finish_kernel, smem);
     {
         METOK_TIMED("seg_finish_kernel", st);
         launch_chained(seg_finish_kernel, dim3(1), dim3(1024), smem, st, part_dot, part_nrm, nslab, Tn, k, sims, boundaries, event_offsets,

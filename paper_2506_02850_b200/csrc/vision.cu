@@ -1354,8 +1354,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         const int grid = min(ceil_div(Nv, 8), kNumSMs * 8);
         const size_t smem = (size_t)d * sizeof(float);
         if (smem > 48 * 1024)
-            METOK_CUDA_TRY(cudaFuncSetAttribute(tok_score_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)smem));
+            METOK_ALLOW_SMEM(tok_score_kernel<T>, smem);
         {
             METOK_TIMED("tok_score_kernel", st);
             tok_score_kernel<T><<<grid, 256, smem, st>>>(feats, text, Nv, d, token_score, w.inv_norm);
@@ -1375,8 +1374,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     pp.s1 = p->s1; pp.s2 = p->s2; pp.s1_nonkey = p->s1_nonkey; pp.s2_nonkey = p->s2_nonkey;
     const size_t plan_smem = (size_t)(k + Tn) * sizeof(float) + (size_t)k * (3 * sizeof(int) + 1);
     if (plan_smem > 40 * 1024)
-        METOK_CUDA_TRY(cudaFuncSetAttribute(event_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)plan_smem));
+        METOK_ALLOW_SMEM(event_plan_kernel, plan_smem);
     PlanClears clr;
     const bool merging = p->mode == METOK_MODE_TOPK_MERGE;
     clr.zero_a = mma ? w.best64 : nullptr;
@@ -1412,8 +1410,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         const BlockSelLayout bl = block_sel_layout(1, (long long)(Tn - (k - 1)) * N, 0);
         if (bl.fits) {
             if (bl.bytes > 32 * 1024)
-                METOK_CUDA_TRY(cudaFuncSetAttribute(event_block_topk_kernel,
-                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bl.bytes));
+                METOK_ALLOW_SMEM(event_block_topk_kernel, bl.bytes);
             METOK_TIMED("event_topk_kernel", st);
             launch_chained(event_block_topk_kernel, dim3(k), dim3(kBsThreads), bl.bytes, st, token_score, w.ev_lo, N, w.ev_budget, w.ev_out_off,
                                                                      bl, w.is_key, out_src, out_event, assign);
@@ -1421,8 +1418,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
             const SelectLayout lay = select_layout(1, select_items_per_cta((long long)(Tn - (k - 1)) * N));
             const int nthreads = select_threads(select_items_per_cta(2LL * Nv / k));
             if (lay.bytes > 32 * 1024)                    // static + dynamic beyond 48 KiB needs the opt-in
-                METOK_CUDA_TRY(cudaFuncSetAttribute(event_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                    (int)lay.bytes));
+                METOK_ALLOW_SMEM(event_topk_kernel, lay.bytes);
             METOK_TIMED("event_topk_kernel", st);
             event_topk_kernel<<<k * kSelCluster, nthreads, lay.bytes, st>>>(
                 token_score, w.ev_lo, N, w.ev_budget, w.ev_out_off, lay, w.is_key, out_src, out_event, assign);
@@ -1436,8 +1432,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         if (r2 != METOK_OK) return r2;
         r2 = make_tmap_bf16_2d(&tmA_half, feats, (uint64_t)Nv, (uint64_t)d, kMmaBM / 2);
         if (r2 != METOK_OK) return r2;
-        METOK_CUDA_TRY(cudaFuncSetAttribute(merge_assign_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)kMmaSmemBytes));
+        METOK_ALLOW_SMEM(merge_assign_mma_kernel, kMmaSmemBytes);
         {
             METOK_TIMED("merge_assign_mma_kernel", st);
             launch_chained(merge_assign_mma_kernel, dim3(kNumSMs), dim3(kMmaThreads), kMmaSmemBytes, st, 
@@ -1468,7 +1463,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     // rows in flight per CTA: a pass over a row moves at most seg0 bytes, the ring holds 24 KiB
     const uint32_t seg0 = (uint32_t)std::min<long long>(kAvgThreads * kAvgChunks, (long long)d * sizeof(T) / 16) * 16u;
     auto launch = [&](auto kernel) -> int {
-        METOK_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAvgSmemBytes));
+        METOK_ALLOW_SMEM(kernel, kAvgSmemBytes);
         {
             METOK_TIMED("merge_avg_kernel", st);
             launch_chained(kernel, dim3(kAvgFrontCtas + cap), dim3(kAvgThreads), kAvgSmemBytes, st,
