@@ -281,7 +281,7 @@ class_topk_kernel(const float* __restrict__ scores, size_t score_stride, const i
     auto emit = [&](int u, int rank) {
         for (int r = 0; r < replicas; ++r) keep[(size_t)r * keep_stride + rank] = u;
     };
-    const int total = cluster_compact(cx, p_lo, p_hi, flag, emit, sm);
+    const int total = cluster_compact(cx, p_lo, p_hi, flag, emit, [](int, int) {}, sm);
     if (cx.rank == 0) {
         for (int r = threadIdx.x; r < replicas; r += blockDim.x) {
             if (count_a) count_a[problem + r] = total;

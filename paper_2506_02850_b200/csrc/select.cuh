@@ -352,8 +352,9 @@ __device__ void cluster_select(SelectCtx& cx, int n, ClsF cls, ValF val, const i
 // problem.  Warps own contiguous ranges (counted first, written in a second sweep);
 // flag(u) is evaluated twice and must be pure.  Returns the total over the cluster.
 // Ends with a cluster barrier: no CTA leaves while another may still read its memory.
-template <typename FlagF, typename EmitF>
-__device__ int cluster_compact(SelectCtx& cx, int p_lo, int p_hi, FlagF flag, EmitF emit, SelectSmem& sm) {
+// skip(u, before) is called for the others, before = number of flagged positions before u.
+template <typename FlagF, typename EmitF, typename SkipF>
+__device__ int cluster_compact(SelectCtx& cx, int p_lo, int p_hi, FlagF flag, EmitF emit, SkipF skip, SelectSmem& sm) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nwarps = blockDim.x >> 5;
     const int n = p_hi - p_lo;
@@ -399,7 +400,9 @@ __device__ int cluster_compact(SelectCtx& cx, int p_lo, int p_hi, FlagF flag, Em
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const unsigned bal = __ballot_sync(0xFFFFFFFFu, f[u]);
-            if (f[u]) emit(b + u * 32 + lane, run + __popc(bal & ((1u << lane) - 1u)));
+            const int before = run + __popc(bal & ((1u << lane) - 1u));
+            if (f[u]) emit(b + u * 32 + lane, before);
+            else if (b + u * 32 + lane < hi) skip(b + u * 32 + lane, before);
             run += __popc(bal);
         }
     }

@@ -112,6 +112,7 @@ __device__ __forceinline__ int find_event(const int32_t* __restrict__ off, int k
 // Event scores, key events, per-event token budgets and output offsets.  One CTA.
 struct PlanParams {
     int Tn, N, k, n_key_events, event_agg, mode, tile_rows, chunk_cols;
+    int rows_with_keys;                         // the merge's row tiles run over all tokens of an event (1) or only over those that are no key token (0)
     int grid, s1, s2, s1_nonkey, s2_nonkey;     // POOL: side of the token grid and the four strides
     double keep_key, keep_nonkey, beta;
     const uint8_t* key_given;                   // the caller's key events, or null
@@ -121,7 +122,7 @@ struct PlanParams {
 // The workspace regions that later kernels of the call expect cleared: written here, at the start of
 // the call's first kernel, instead of by separate memset nodes (each costs the chain a launch).
 struct PlanClears {
-    void* zero_a; size_t zero_a_bytes;      // packed argmax per token (tensor-core path), may be null
+    void* zero_a; size_t zero_a_bytes;      // packed argmax per token, may be null
     void* zero_b; size_t zero_b_bytes;      // member bits, member counts, long-list counters
     void* ones;   size_t ones_bytes;        // output -> long-list index, all bits set = none
     int32_t* status;                        // device status word
@@ -144,7 +145,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
                   const int32_t* __restrict__ event_offsets, PlanParams pp,
                   float* __restrict__ event_score, uint8_t* __restrict__ event_is_key,
                   int32_t* __restrict__ ev_lo, int32_t* __restrict__ ev_budget, int32_t* __restrict__ ev_out_off,
-                  int32_t* __restrict__ ev_tile_off, int32_t* __restrict__ ev_unit_off,
+                  int32_t* __restrict__ ev_unit_off,
                   int32_t* __restrict__ frame_ev, int32_t* __restrict__ frame_stride,
                   int32_t* __restrict__ frame_off, int32_t* __restrict__ n_out, PlanClears clr) {
     grid_dep_wait();
@@ -237,18 +238,16 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
         }
         __syncthreads();
         if (tid == 0) {                                     // everything it reads is in shared memory
-            int slots = 0, tiles = 0, units = 0;
+            int slots = 0, units = 0;
             for (int e = 0; e < k; ++e) {
                 ev_out_off[e] = slots;
-                ev_tile_off[e] = tiles;
                 ev_unit_off[e] = units;
                 slots += s_bud[e];
-                const int t = ((s_evhi[e] - s_evlo[e]) * pp.N + pp.tile_rows - 1) / pp.tile_rows;
-                tiles += t;
+                const int rows = (s_evhi[e] - s_evlo[e]) * pp.N - (pp.rows_with_keys ? 0 : s_bud[e]);
+                const int t = (rows + pp.tile_rows - 1) / pp.tile_rows;
                 units += t * ((s_bud[e] + pp.chunk_cols - 1) / pp.chunk_cols);   // row tiles x key chunks
             }
             ev_out_off[k] = slots;
-            ev_tile_off[k] = tiles;
             ev_unit_off[k] = units;
             *n_out = slots;
         }
@@ -399,12 +398,13 @@ pool_kernel(const T* __restrict__ feats, int d, int N, int G, int Tn, const int3
     }
 }
 
-// Per-event key-token top-k: one cluster per event.
+// Per-event key-token top-k: one cluster per event.  `rest` lists the event's other tokens, from the event's first
+// token's place on.
 __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThreads)
 event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restrict__ ev_lo, int N,
                   const int32_t* __restrict__ ev_budget, const int32_t* __restrict__ ev_out_off, SelectLayout lay,
                   uint8_t* __restrict__ is_key, int32_t* __restrict__ out_src, int32_t* __restrict__ out_event,
-                  int32_t* __restrict__ assign) {
+                  int32_t* __restrict__ assign, int32_t* __restrict__ rest) {
     __shared__ SelectSmem sm;
     __shared__ int s_budget[1];
     extern __shared__ __align__(16) unsigned char sel_dyn[];
@@ -440,7 +440,8 @@ event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restri
         assign[lo + i] = slot;
     };
     for (int i = p_lo + threadIdx.x; i < p_hi; i += blockDim.x) is_key[lo + i] = flag(i) ? 1 : 0;
-    cluster_compact(cx, p_lo, p_hi, flag, emit, sm);
+    auto skip = [&](int i, int before) { rest[lo + i - before] = lo + i; };
+    cluster_compact(cx, p_lo, p_hi, flag, emit, skip, sm);
 }
 
 // The same by one CTA per event, when the largest event a segmentation can produce fits a
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(kBsThreads, 1)
 event_block_topk_kernel(const float* __restrict__ token_score, const int32_t* __restrict__ ev_lo, int N,
                         const int32_t* __restrict__ ev_budget, const int32_t* __restrict__ ev_out_off,
                         BlockSelLayout lay, uint8_t* __restrict__ is_key, int32_t* __restrict__ out_src,
-                        int32_t* __restrict__ out_event, int32_t* __restrict__ assign) {
+                        int32_t* __restrict__ out_event, int32_t* __restrict__ assign, int32_t* __restrict__ rest) {
     grid_dep_wait();
     __shared__ BlockSelSmem sm;
     __shared__ int s_budget[1];
@@ -480,6 +481,8 @@ event_block_topk_kernel(const float* __restrict__ token_score, const int32_t* __
                     out_event[slot] = e;
                     assign[lo + i] = slot;
                     ++slot;
+                } else {
+                    rest[lo + i - (slot - slot0)] = lo + i;
                 }
             }
         }
@@ -487,110 +490,129 @@ event_block_topk_kernel(const float* __restrict__ token_score, const int32_t* __
 }
 
 // --------------------------------------------------------------------------- //
-// Merge-assign, generic CUDA-core path (fp32 inputs, and any shape the tensor-core
-// path does not take).  CTA = 64 token rows of one event; loops over the event's
-// key tokens 64 at a time; fp32 accumulate; fused row argmax of dot * inv_norm(key).
+// Merge-assign on the CUDA cores (fp32 inputs; bf16 only when forced for debugging): fp32 products, added in
+// the order of the row, so every dot product is one chain of fused multiply-adds.
+//
+// Work unit = 64 of an event's tokens that are no key tokens x 64 of its key tokens; the units of all events form one list and
+// a CTA takes every gridDim-th.  A unit is done by 64 threads with 8 x 8 outputs each (rows ty + 8 i, keys
+// tx + 8 j).  Shared-memory reads and multiply-adds are nearly in balance there (a k costs a thread 64 bytes,
+// which is what 64 multiply-adds take to run), so rows and keys are kept as they lie (k contiguous, 8-byte reads
+// of two k; wider reads are no cheaper per byte: a k-major layout with 16-byte reads took 423 us) and come by
+// 16-byte asynchronous copies into two stages of 16 k, a row's pitch of 80 bytes (fp32) putting the eight keys
+// of a warp's read into different banks.  Rows past the tile's end are copies of another row: nobody reads
+// their results.  Small CTAs, six per SM, because the unit count is small: 61 frames of 169 tokens give 756
+// units.
+// 61 x 169 tokens, d = 1156, fp32: 755 us with 64-row CTAs of 4 x 4 outputs per thread that each walked all keys
+// of the event, 219 us now (0.76 of the multiply-adds: key tokens need no assignment).
+// Units of one row meet in a 64-bit atomicMax as in the tensor-core kernel: larger value, then lower slot.
 // --------------------------------------------------------------------------- //
-constexpr int kMergeTM = 64, kMergeTN = 64, kMergeTK = 32;
-
+constexpr int kSaTile = 64, kSaBK = 16, kSaThreads = 64, kSaCtasPerSm = 6;
 
 template <typename T>
-__global__ void __launch_bounds__(256)
-merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_t* __restrict__ ev_lo, int k,
-                         const int32_t* __restrict__ ev_out_off, const int32_t* __restrict__ ev_tile_off,
-                         const int32_t* __restrict__ out_src, const float* __restrict__ inv_norm,
-                         const uint8_t* __restrict__ is_key, int32_t* __restrict__ assign) {
-    constexpr int VN = Vec16<T>::N;
-    constexpr int CPR = kMergeTK / VN;      // 16-byte chunks per tile row
-    constexpr int LD = kMergeTM + 1;
-    __shared__ float As[kMergeTK][LD];
-    __shared__ float Bs[kMergeTK][LD];
-    __shared__ int s_src[kMergeTN];
-    __shared__ float s_inv[kMergeTN];
-    const int t = blockIdx.x;
-    if (t >= ev_tile_off[k]) return;
-    const int e = find_event(ev_tile_off, k, t);
-    const int row0 = ev_lo[e] * N + (t - ev_tile_off[e]) * kMergeTM;
-    const int row_end = ev_lo[e + 1] * N;
-    const int s0 = ev_out_off[e], s1 = ev_out_off[e + 1];
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-
-    float best_v[4];
-    int best_s[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { best_v[i] = -3.4e38f; best_s[i] = 0x7FFFFFFF; }
-
-    for (int n0 = s0; n0 < s1; n0 += kMergeTN) {
-        __syncthreads();
-        if (tid < kMergeTN) {
-            const int slot = n0 + tid;
-            const int src = slot < s1 ? out_src[slot] : -1;
-            s_src[tid] = src;
-            s_inv[tid] = src >= 0 ? inv_norm[src] : 0.f;
-        }
-        __syncthreads();
-        float acc[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-        for (int k0 = 0; k0 < d; k0 += kMergeTK) {
-            for (int c = tid; c < kMergeTM * CPR; c += 256) {
-                const int r = c / CPR, ch = c % CPR;
-                const int kk = k0 + ch * VN;
-                float va[VN], vb[VN];
-                const int row = row0 + r;
-                if (row < row_end && kk < d) Vec16<T>::load(feats + (size_t)row * d + kk, va);
-                else Vec16<T>::zero(va);
-                const int src = s_src[r];
-                if (src >= 0 && kk < d) Vec16<T>::load(feats + (size_t)src * d + kk, vb);
-                else Vec16<T>::zero(vb);
-#pragma unroll
-                for (int q = 0; q < VN; ++q) {
-                    As[ch * VN + q][r] = va[q];
-                    Bs[ch * VN + q][r] = vb[q];
-                }
-            }
-            __syncthreads();
-#pragma unroll 8
-            for (int kk = 0; kk < kMergeTK; ++kk) {
-                float a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {                 // ascending slot within this thread
-            const int col = tx + 16 * j;
-            const int slot = n0 + col;
-            if (slot < s1) {
-                const float inv = s_inv[col];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float v = acc[i][j] * inv;
-                    if (v > best_v[i]) { best_v[i] = v; best_s[i] = slot; }
-                }
-            }
-        }
+__device__ __forceinline__ float2 load_pair(const T* p) {
+    if constexpr (sizeof(T) == 4) {
+        return *reinterpret_cast<const float2*>(p);
+    } else {
+        const uint32_t w = *reinterpret_cast<const uint32_t*>(p);
+        return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
     }
-    // combine the 16 column owners of each row: larger value, then lower slot
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? kSaCtasPerSm : 4)
+merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_t* __restrict__ ev_lo, int k,
+                         const int32_t* __restrict__ ev_out_off, const int32_t* __restrict__ ev_unit_off,
+                         const int32_t* __restrict__ out_src, const int32_t* __restrict__ rest,
+                         const float* __restrict__ inv_norm, unsigned long long* __restrict__ best64) {
+    grid_dep_wait();
+    constexpr int CE = 16 / sizeof(T);              // elements per 16-byte chunk
+    constexpr int CPR = kSaBK / CE;                 // chunks per row and stage
+    constexpr int LD = kSaBK + CE;                  // row pitch in elements
+    constexpr int kCopies = 2 * kSaTile * CPR / kSaThreads;
+    constexpr int kRowStep = kSaThreads / CPR;      // rows between a thread's copies
+    constexpr uint32_t kStage = 2 * kSaTile * LD * sizeof(T), kCopyStep = kRowStep * LD * sizeof(T);
+    __shared__ __align__(16) T tile[2][2 * kSaTile][LD];    // rows 0..63 tokens, 64..127 keys
+    __shared__ float s_inv[kSaTile];
+    const int tid = threadIdx.x, ty = tid >> 3, tx = tid & 7;
+    const int crow = tid / CPR, cchunk = tid % CPR;
+    const uint32_t dst0 = sm100::smem_u32(&tile[0][crow][cchunk * CE]);
+    const int total = ev_unit_off[k];
+    const int ksteps = (d + kSaBK - 1) / kSaBK;
+    const uint32_t row_chunks = (uint32_t)(d / CE);
+    for (int unit = blockIdx.x; unit < total; unit += gridDim.x) {
+        const int e = find_event(ev_unit_off, k, unit);
+        const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0;
+        const int nchunks = (nk + kSaTile - 1) / kSaTile;
+        const int local = unit - ev_unit_off[e];
+        const int row_tile = local / nchunks, chunk = local - row_tile * nchunks;
+        const int row0 = ev_lo[e] * N + row_tile * kSaTile, row_end = ev_lo[e + 1] * N - nk;   // places in `rest`
+        const int key0 = s0 + chunk * kSaTile, key_end = s0 + nk;
+        const uint4* src[kCopies];                  // where this thread's copies of the first stage read
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) {
-            const float ov = __shfl_xor_sync(0xFFFFFFFFu, best_v[i], o);
-            const int os = __shfl_xor_sync(0xFFFFFFFFu, best_s[i], o);
-            if (ov > best_v[i] || (ov == best_v[i] && os < best_s[i])) { best_v[i] = ov; best_s[i] = os; }
+        for (int i = 0; i < kCopies; ++i) {
+            const int r = crow + kRowStep * i;
+            const int row = r < kSaTile ? rest[min(row0 + r, row_end - 1)] : out_src[min(key0 + r - kSaTile, key_end - 1)];
+            src[i] = reinterpret_cast<const uint4*>(feats) + (size_t)row * row_chunks + cchunk;
         }
-        const int row = row0 + ty + 16 * i;
-        if (tx == 0 && row < row_end && !is_key[row]) assign[row] = best_s[i];
+        __syncthreads();                            // the unit before is done with s_inv and both stages
+        s_inv[tid] = key0 + tid < key_end ? inv_norm[out_src[key0 + tid]] : 0.f;
+        auto issue = [&](int ks) {                  // into stage ks % 2; past the end of the rows: zeros
+            const uint32_t bytes = (uint32_t)(ks * CPR + cchunk) < row_chunks ? 16u : 0u;
+            const uint32_t dst = dst0 + (ks & 1) * kStage;
+            const int off = bytes ? ks * CPR : 0;
+#pragma unroll
+            for (int i = 0; i < kCopies; ++i) sm100::cp_async16_zfill(dst + i * kCopyStep, src[i] + off, bytes);
+            sm100::cp_async_commit();
+        };
+        float acc[8][8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+        issue(0);
+        for (int ks = 0; ks < ksteps; ++ks) {
+            sm100::cp_async_wait_all();
+            __syncthreads();                        // stage ks % 2 has landed for everybody; the other one has been read by everybody
+            if (ks + 1 < ksteps) issue(ks + 1);
+            const T* pa = &tile[ks & 1][ty][0];
+            const T* pb = &tile[ks & 1][kSaTile + tx][0];
+#pragma unroll
+            for (int kk = 0; kk < kSaBK; kk += 2) {
+                float2 a[8], b[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) a[i] = load_pair<T>(pa + 8 * i * LD + kk);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) b[j] = load_pair<T>(pb + 8 * j * LD + kk);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float best_v = -3.4e38f;
+            int best_s = 0x7FFFFFFF;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {           // ascending slots
+                const int slot = key0 + tx + 8 * j;
+                const float v = acc[i][j] * s_inv[tx + 8 * j];
+                if (slot < key_end && v > best_v) { best_v = v; best_s = slot; }
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) {       // the eight column owners of the row
+                const float ov = __shfl_xor_sync(0xFFFFFFFFu, best_v, o);
+                const int os = __shfl_xor_sync(0xFFFFFFFFu, best_s, o);
+                if (ov > best_v || (ov == best_v && os < best_s)) { best_v = ov; best_s = os; }
+            }
+            const int at = row0 + ty + 8 * i;
+            if (tx == 0 && at < row_end && best_s != 0x7FFFFFFF)
+                atomicMax(&best64[rest[at]], ((unsigned long long)float_key(best_v) << 32) | (unsigned long long)(~(uint32_t)best_s));
+        }
     }
 }
 
@@ -856,8 +878,7 @@ __host__ __device__ __forceinline__ int avg_block_tokens(int m) {
     return g < 256 ? 256 : g;
 }
 
-// assign[row] of every non-key token from the packed argmax (tensor-core path; best64 is null when
-// the CUDA-core kernel has written assign itself), and the member-block bits of every output token.
+// assign[row] of every non-key token from the packed argmax, and the member-block bits of every output token.
 __global__ void __launch_bounds__(256)
 merge_decode_kernel(const unsigned long long* __restrict__ best64, const uint8_t* __restrict__ is_key, int Nv,
                     int N, const int32_t* __restrict__ ev_lo, int k, int32_t* __restrict__ assign,
@@ -872,7 +893,7 @@ merge_decode_kernel(const unsigned long long* __restrict__ best64, const uint8_t
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= Nv) return;
     int slot;
-    if (best64 && !is_key[row]) {
+    if (!is_key[row]) {
         slot = (int32_t)(~(uint32_t)(best64[row] & 0xFFFFFFFFull));
         assign[row] = slot;
     } else {
@@ -1272,9 +1293,10 @@ struct VisionWs {
     int32_t* status;          // device status word, first in the workspace
     float* inv_norm;
     uint8_t* is_key;
-    int32_t *ev_lo, *ev_budget, *ev_out_off, *ev_tile_off, *ev_unit_off;
+    int32_t* rest;            // per event, from its first token's place on: its tokens that are no key token
+    int32_t *ev_lo, *ev_budget, *ev_out_off, *ev_unit_off;
     int32_t *frame_ev, *frame_stride, *frame_off;   // POOL mode
-    unsigned long long* best64;   // packed argmax per token (tensor-core path)
+    unsigned long long* best64;   // packed argmax per token (merging modes)
     unsigned long long* slot_blocks;   // per output token: which blocks of its event hold a member
     int32_t* slot_cnt;                 // per output token: members
     int32_t* long_counter;             // outputs with more than kAvgLong members ...
@@ -1289,20 +1311,20 @@ struct VisionWs {
     size_t zero_bytes;                 // slot_blocks .. long_done are cleared together
 };
 
-static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, bool mma) {
+static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, bool merging) {
     VisionWs w;
     w.status = cv.take<int32_t>(64);
     w.inv_norm = cv.take<float>((size_t)Tn * N);
     w.is_key = cv.take<uint8_t>((size_t)Tn * N);
+    w.rest = merging ? cv.take<int32_t>((size_t)Tn * N) : nullptr;
     w.ev_lo = cv.take<int32_t>((size_t)k + 1);
     w.ev_budget = cv.take<int32_t>((size_t)k + 1);
     w.ev_out_off = cv.take<int32_t>((size_t)k + 1);
-    w.ev_tile_off = cv.take<int32_t>((size_t)k + 1);
     w.ev_unit_off = cv.take<int32_t>((size_t)k + 1);
     w.frame_ev = cv.take<int32_t>((size_t)Tn);
     w.frame_stride = cv.take<int32_t>((size_t)Tn);
     w.frame_off = cv.take<int32_t>((size_t)Tn + 1);
-    w.best64 = mma ? cv.take<unsigned long long>((size_t)Tn * N) : nullptr;
+    w.best64 = merging ? cv.take<unsigned long long>((size_t)Tn * N) : nullptr;
     {
         const size_t n = (size_t)cap + 64;
         w.zero_bytes = n * 8 + n * 4 + (size_t)(64 + kAvgLongCapMax + 64) * 4;
@@ -1344,7 +1366,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     constexpr bool kBf16 = sizeof(T) == 2;
     const bool mma = kBf16 && use_mma_path(d) && p->mode == METOK_MODE_TOPK_MERGE;
     Carver cv(ws);
-    VisionWs w = carve_vision(cv, Tn, N, k, d, cap, mma);
+    VisionWs w = carve_vision(cv, Tn, N, k, d, cap, p->mode == METOK_MODE_TOPK_MERGE);
     // (the status word and the scratch that must start cleared are written by event_plan_kernel)
     if (const int rc = debug_arm(w.status, st)) return rc;
 
@@ -1364,8 +1386,9 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     PlanParams pp;
     pp.Tn = Tn; pp.N = N; pp.k = k;
     pp.n_key_events = min(k, ceilq(p->alpha * (double)k));
-    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? kMmaBM : kMergeTM;
-    pp.chunk_cols = kMmaBN;
+    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? kMmaBM : kSaTile;
+    pp.chunk_cols = mma ? kMmaBN : kSaTile;
+    pp.rows_with_keys = mma ? 1 : 0;
     pp.keep_key = p->keep_key; pp.keep_nonkey = p->keep_nonkey; pp.beta = p->beta;
     pp.key_given = p->key_events_given;
     pp.key_frames_given = p->key_frames_given;
@@ -1377,7 +1400,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         METOK_ALLOW_SMEM(event_plan_kernel, plan_smem);
     PlanClears clr;
     const bool merging = p->mode == METOK_MODE_TOPK_MERGE;
-    clr.zero_a = mma ? w.best64 : nullptr;
+    clr.zero_a = merging ? w.best64 : nullptr;
     clr.zero_a_bytes = (size_t)Nv * sizeof(unsigned long long);
     clr.zero_b = merging ? w.slot_blocks : nullptr;
     clr.zero_b_bytes = w.zero_bytes;
@@ -1388,7 +1411,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         METOK_TIMED("event_plan_kernel", st);
         launch_chained(event_plan_kernel, dim3(1 + kPlanFillCtas), dim3(1024), plan_smem, st, token_score, frame_score, event_offsets, pp, event_score,
                                                                   event_is_key, w.ev_lo, w.ev_budget, w.ev_out_off,
-                                                                  w.ev_tile_off, w.ev_unit_off, w.frame_ev,
+                                                                  w.ev_unit_off, w.frame_ev,
                                                                   w.frame_stride, w.frame_off, n_out, clr);
     }
     METOK_LAUNCH_CHECK();
@@ -1413,7 +1436,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
                 METOK_ALLOW_SMEM(event_block_topk_kernel, bl.bytes);
             METOK_TIMED("event_topk_kernel", st);
             launch_chained(event_block_topk_kernel, dim3(k), dim3(kBsThreads), bl.bytes, st, token_score, w.ev_lo, N, w.ev_budget, w.ev_out_off,
-                                                                     bl, w.is_key, out_src, out_event, assign);
+                                                                     bl, w.is_key, out_src, out_event, assign, w.rest);
         } else {
             const SelectLayout lay = select_layout(1, select_items_per_cta((long long)(Tn - (k - 1)) * N));
             const int nthreads = select_threads(select_items_per_cta(2LL * Nv / k));
@@ -1421,7 +1444,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
                 METOK_ALLOW_SMEM(event_topk_kernel, lay.bytes);
             METOK_TIMED("event_topk_kernel", st);
             event_topk_kernel<<<k * kSelCluster, nthreads, lay.bytes, st>>>(
-                token_score, w.ev_lo, N, w.ev_budget, w.ev_out_off, lay, w.is_key, out_src, out_event, assign);
+                token_score, w.ev_lo, N, w.ev_budget, w.ev_out_off, lay, w.is_key, out_src, out_event, assign, w.rest);
         }
         METOK_LAUNCH_CHECK();
     }
@@ -1441,19 +1464,15 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         }
         METOK_LAUNCH_CHECK();
     } else {
-        const int max_tiles = Nv / kMergeTM + k;
-        {
-            METOK_TIMED("merge_assign_simt_kernel", st);
-            merge_assign_simt_kernel<T><<<max_tiles, 256, 0, st>>>(feats, d, N, w.ev_lo, k, w.ev_out_off,
-                                                                   w.ev_tile_off, out_src, inv_norm, w.is_key,
-                                                                   assign);
-        }
+        METOK_TIMED("merge_assign_simt_kernel", st);
+        launch_chained(merge_assign_simt_kernel<T>, dim3(kNumSMs * kSaCtasPerSm), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
+                       w.ev_out_off, w.ev_unit_off, out_src, w.rest, inv_norm, w.best64);
         METOK_LAUNCH_CHECK();
     }
 
     {
         METOK_TIMED("merge_decode_kernel", st);
-        launch_chained(merge_decode_kernel, dim3(ceil_div(Nv, 256)), dim3(256), 0, st, mma ? w.best64 : nullptr, w.is_key, Nv, N, w.ev_lo, k,
+        launch_chained(merge_decode_kernel, dim3(ceil_div(Nv, 256)), dim3(256), 0, st, w.best64, w.is_key, Nv, N, w.ev_lo, k,
                                                                assign, w.slot_blocks, w.slot_cnt, w.long_index,
                                                                w.long_slot, w.long_counter, kAvgLong, avg_long_cap(d),
                                                                w.few_members, kAvgFew, w.heavy_index, w.heavy_slot,
@@ -1520,9 +1539,10 @@ extern "C" int metok_compress_vision_bound(int T, int N, int k, const metok_visi
 
 extern "C" size_t metok_compress_vision_workspace_bytes(int dtype, int T, int N, int d, int k, int cap,
                                                         const metok_vision_params* p) {
+    (void)dtype;
     if (T < 1 || N < 1 || k < 1 || d < 1 || cap < 0) return 0;
     Carver cv(nullptr);
-    carve_vision(cv, T, N, k, d, cap, dtype == METOK_BF16 && !(p && p->mode == METOK_MODE_POOL));
+    carve_vision(cv, T, N, k, d, cap, !(p && p->mode == METOK_MODE_POOL));
     return cv.total();
 }
 
