@@ -55,19 +55,29 @@ struct KernelTimer {
 // memory, which returns once that kernel has completed and its writes are visible.  Because every CTA
 // of every kernel launched this way waits first, completion of a kernel implies completion of all
 // kernels before it on the stream.  The launch error is picked up by METOK_LAUNCH_CHECK().
+// `cluster` > 1 launches clusters of that many CTAs along x.
 template <typename... P, typename... A>
-inline void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+inline void launch_chained_clusters(int cluster, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                    A&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     (void)cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+inline void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    launch_chained_clusters(1, kern, grid, block, smem, st, args...);
 }
 
 #ifdef __CUDACC__

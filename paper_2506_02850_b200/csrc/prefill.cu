@@ -4,7 +4,7 @@
 
 #include "common.cuh"
 #include "select.cuh"
-#include "select_block.cuh"
+#include "select_cluster.cuh"
 #include "launchers.h"
 #include "sm100.cuh"
 
@@ -290,49 +290,70 @@ class_topk_kernel(const float* __restrict__ scores, size_t score_stride, const i
     }
 }
 
-template <bool kOne>                     // kOne: one class and no class array
-__global__ void __launch_bounds__(kBsThreads, 1)
-block_topk_kernel(const float* __restrict__ scores, size_t score_stride, const int32_t* __restrict__ token_group,
-                  int n_vis, int G, BlockSelLayout lay, TopkBudgets budgets, int S, int vis_start,
-                  int32_t* __restrict__ keep_idx, size_t keep_stride, int replicas,
-                  int32_t* __restrict__ count_a, int32_t* __restrict__ count_b) {
+// The same for up to 81 920 items (select_cluster.cuh): a CTA or a cluster per problem.
+template <int IT, bool kCl, bool kOne>   // kOne: one class and no class array
+__global__ void __launch_bounds__(IT == kCsMaxItems ? kCsMaxItemsThreads : 1024)
+cs_topk_kernel(const float* __restrict__ scores, size_t score_stride, const int32_t* __restrict__ token_group,
+               int n_vis, int G, CsLayout lay, TopkBudgets budgets, int S, int vis_start,
+               int32_t* __restrict__ keep_idx, size_t keep_stride, int replicas,
+               int32_t* __restrict__ count_a, int32_t* __restrict__ count_b) {
+    cs_enter<kCl>();
     grid_dep_wait();
-    __shared__ BlockSelSmem sm;
+    __shared__ CsShared sm;
     extern __shared__ __align__(16) unsigned char sel_dyn[];
-    const int problem = blockIdx.x;
+    constexpr int C = kCl ? kCsMaxCluster : 1;
+    const int problem = blockIdx.x / C, rank = blockIdx.x - problem * C;
     const float* sc = scores + (size_t)problem * score_stride;
     int32_t* keep = keep_idx + (size_t)problem * keep_stride;
-    const int tid = threadIdx.x;
-    const BlockSelView sel = block_sel_run<kOne>(sm, sel_dyn, lay, sc, kOne ? nullptr : token_group, n_vis, G, budgets.v);
-    const uint32_t* mask = sel.mask;
-    const int* woff = sel.woff;
-    const int kept = sel.kept;
-    const int n4 = (n_vis + 3) >> 2;
-    const int vis_end = vis_start + n_vis;
-    // The kept positions in order.  Positions before and after the visual span are always kept;
-    // the kept visual items are first packed in shared memory (over the keys, which the masks
-    // have replaced) so that the list leaves in whole coalesced stores.
-    // One list may serve several layers: `replicas` copies, keep_stride apart.
-    int32_t* packed = reinterpret_cast<int32_t*>(sel.keys);
-    for (int q = tid; q < n4; q += kBsThreads) {
-        const uint32_t m = mask[q >> 3];
-        const int sh = (q & 7) * 4;
-        const uint32_t nib = (m >> sh) & 15u;
-        int rank = woff[q >> 3] + __popc(m & ((1u << sh) - 1u));
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if ((nib >> u) & 1u) packed[rank++] = vis_start + q * 4 + u;
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    const CsSlice sl = cs_slice<IT>(n_vis, rank, C);
+    auto load = [&](int i, float& v, int& c) {
+        v = sc[i];
+        c = 0;
+        if (!kOne) {
+            c = token_group[i];
+            if (c >= G) c = -1;
         }
+    };
+    int before, kept;
+    const uint32_t bits = cs_select<IT, kCl, kOne>(sm, sel_dyn, lay, G, budgets.v, rank, sl.i_first, sl.i_hi, load, &before, &kept);
+    // The kept positions in order; positions before and after the visual span are always kept.
+    const int outside = S - n_vis;
+    if (replicas == 1) {
+        cs_for_items<IT>(bits, vis_start + before, sl.i_first, sl.i_hi, [&](int, int i, int place, bool k) {
+            if (k) keep[place] = vis_start + i;
+        });
+        for (int i = rank * nthr + tid; i < outside; i += C * nthr)
+            keep[i < vis_start ? i : kept + i] = i < vis_start ? i : i + n_vis;
+    } else {
+        // One list serves several layers (`replicas` copies, keep_stride apart): the CTA's part of it is packed in
+        // shared memory (over the histograms, as much as they hold at a time), so that every copy leaves in
+        // coalesced stores.
+        int32_t* pack = reinterpret_cast<int32_t*>(sel_dyn);
+        const int room = 2 * G << lay.nb_log2;
+        int mine = 0;                                        // what this CTA keeps, and the place of its first item
+        for (int w = 0; w < (nthr >> 5); ++w) mine += sm.warp_tot[w];
+        const int first = sm.before;
+        for (int p0 = 0; p0 < mine; p0 += room) {
+            cs_for_items<IT>(bits, before - first - p0, sl.i_first, sl.i_hi, [&](int, int i, int place, bool k) {
+                if (k && place >= 0 && place < room) pack[place] = vis_start + i;
+            });
+            __syncthreads();
+            for (int i = tid; i < min(room, mine - p0); i += nthr) {
+                const int v = pack[i];
+                for (int l = 0; l < replicas; ++l) keep[(size_t)l * keep_stride + vis_start + first + p0 + i] = v;
+            }
+            __syncthreads();
+        }
+        for (int i = rank * nthr + tid; i < outside; i += C * nthr)
+            for (int l = 0; l < replicas; ++l)
+                keep[(size_t)l * keep_stride + (i < vis_start ? i : kept + i)] = i < vis_start ? i : i + n_vis;
     }
-    __syncthreads();
-    const int total = vis_start + kept + (S - vis_end);
-    for (int i = tid; i < total; i += kBsThreads) {
-        const int v = i < vis_start ? i : i < vis_start + kept ? packed[i - vis_start] : vis_end + (i - vis_start - kept);
-        for (int r = 0; r < replicas; ++r) keep[(size_t)r * keep_stride + i] = v;
-    }
-    for (int r = tid; r < replicas; r += kBsThreads) {
-        if (count_a) count_a[problem + r] = total;
-        if (count_b) count_b[problem + r] = total;
+    if (rank == 0) {
+        for (int l = tid; l < replicas; l += nthr) {
+            if (count_a) count_a[problem + l] = outside + kept;
+            if (count_b) count_b[problem + l] = outside + kept;
+        }
     }
 }
 
@@ -341,19 +362,24 @@ int launch_class_topk(const float* scores, size_t score_stride, const int32_t* t
                       int replicas, int32_t* count_a, int32_t* count_b, int problems, cudaStream_t st) {
     TopkBudgets b;
     for (int g = 0; g < METOK_MAX_GROUPS; ++g) b.v[g] = g < G ? budgets_host[g] : 0;
-    // problems whose keys fit one CTA's shared memory skip the cluster and its barriers
-    const BlockSelLayout bl = block_sel_layout(G, n_vis, S);
-    if (bl.fits) {
-        auto kernel = (G == 1 && !token_group) ? block_topk_kernel<true> : block_topk_kernel<false>;
-        if (bl.bytes > 32 * 1024)
-            METOK_ALLOW_SMEM(kernel, bl.bytes);
-        {
+    const CsPlan plan = cs_plan(n_vis);
+    if (plan.fits) {
+        const CsLayout lay = cs_layout(G, n_vis);
+        auto launch = [&](auto kernel) -> int {
+            if (lay.bytes > 40 * 1024) METOK_ALLOW_SMEM(kernel, lay.bytes);
             METOK_TIMED("class_topk_kernel", st);
-            launch_chained(kernel, dim3(problems), dim3(kBsThreads), bl.bytes, st, scores, score_stride, token_group, n_vis, G, bl, b, S,
-                                                           vis_start, keep_idx, keep_stride, replicas, count_a, count_b);
-        }
-        METOK_LAUNCH_CHECK();
-        return METOK_OK;
+            launch_chained_clusters(plan.C, kernel, dim3(problems * plan.C), dim3(plan.threads), lay.bytes, st, scores,
+                                    score_stride, token_group, n_vis, G, lay, b, S, vis_start, keep_idx, keep_stride,
+                                    replicas, count_a, count_b);
+            METOK_LAUNCH_CHECK();
+            return METOK_OK;
+        };
+        const bool one = G == 1 && !token_group;
+        if (plan.C == 1)
+            return one ? launch(cs_topk_kernel<4, false, true>) : launch(cs_topk_kernel<4, false, false>);
+        if (plan.items == 4)
+            return one ? launch(cs_topk_kernel<4, true, true>) : launch(cs_topk_kernel<4, true, false>);
+        return one ? launch(cs_topk_kernel<kCsMaxItems, true, true>) : launch(cs_topk_kernel<kCsMaxItems, true, false>);
     }
     const SelectLayout lay = select_layout(G, select_items_per_cta((long long)S));
     const int nthreads = select_threads(select_items_per_cta((long long)S));

@@ -5,7 +5,7 @@
 
 #include "common.cuh"
 #include "select.cuh"
-#include "select_block.cuh"
+#include "select_cluster.cuh"
 #include "sm100.cuh"
 #include "launchers.h"
 
@@ -444,49 +444,60 @@ event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restri
     cluster_compact(cx, p_lo, p_hi, flag, emit, skip, sm);
 }
 
-// The same by one CTA per event, when the largest event a segmentation can produce fits a
-// CTA's shared memory (select_block.cuh): no cluster barriers.
-__global__ void __launch_bounds__(kBsThreads, 1)
-event_block_topk_kernel(const float* __restrict__ token_score, const int32_t* __restrict__ ev_lo, int N,
-                        const int32_t* __restrict__ ev_budget, const int32_t* __restrict__ ev_out_off,
-                        BlockSelLayout lay, uint8_t* __restrict__ is_key, int32_t* __restrict__ out_src,
-                        int32_t* __restrict__ out_event, int32_t* __restrict__ assign, int32_t* __restrict__ rest) {
-    grid_dep_wait();
-    __shared__ BlockSelSmem sm;
-    __shared__ int s_budget[1];
-    extern __shared__ __align__(16) unsigned char sel_dyn[];
-    const int e = blockIdx.x;
-    const int lo = ev_lo[e] * N, hi = ev_lo[e + 1] * N;
-    const int n = hi - lo;
-    if (n <= 0) return;
-    const int tid = threadIdx.x;
-    if (tid == 0) s_budget[0] = ev_budget[e];
-    __syncthreads();
-    const BlockSelView sel = block_sel_run<true>(sm, sel_dyn, lay, token_score + lo, nullptr, n, 1, s_budget);
-    const int slot0 = ev_out_off[e];
-    const int n4 = (n + 3) >> 2;
-    for (int q = tid; q < n4; q += kBsThreads) {
-        const uint32_t m = sel.mask[q >> 3];
-        const int sh = (q & 7) * 4;
-        const uint32_t nib = (m >> sh) & 15u;
-        int slot = slot0 + sel.woff[q >> 3] + __popc(m & ((1u << sh) - 1u));
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = q * 4 + u;
-            if (i < n) {
-                const bool key = (nib >> u) & 1u;
-                is_key[lo + i] = key ? 1 : 0;
-                if (key) {
-                    out_src[slot] = lo + i;
-                    out_event[slot] = e;
-                    assign[lo + i] = slot;
-                    ++slot;
-                } else {
-                    rest[lo + i - (slot - slot0)] = lo + i;
-                }
-            }
+// The same when the largest event a segmentation can produce fits select_cluster.cuh.
+template <int IT, bool kCl>
+__device__ __forceinline__ void
+cs_event_topk(CsShared& sm, unsigned char* dyn, const CsLayout& lay, const float* __restrict__ sc, int lo, int n, int e,
+              int budget, int slot0, int rank, uint8_t* __restrict__ is_key, int32_t* __restrict__ out_src,
+              int32_t* __restrict__ out_event, int32_t* __restrict__ assign, int32_t* __restrict__ rest) {
+    const CsSlice sl = cs_slice<IT>(n, rank, kCl ? kCsMaxCluster : 1);
+    int before, kept;
+    const uint32_t bits = cs_select<IT, kCl, true>(sm, dyn, lay, 1, &budget, rank, sl.i_first, sl.i_hi,
+                                                   [&](int i, float& v, int& c) { v = sc[i]; c = 0; }, &before, &kept);
+    cs_for_items<IT>(bits, before, sl.i_first, sl.i_hi, [&](int, int i, int place, bool key) {
+        is_key[lo + i] = key ? 1 : 0;
+        if (key) {
+            out_src[slot0 + place] = lo + i;
+            out_event[slot0 + place] = e;
+            assign[lo + i] = slot0 + place;
+        } else {
+            rest[lo + i - place] = lo + i;
         }
+    });
+}
+
+template <int IT, bool kCl>
+__global__ void __launch_bounds__(IT == kCsMaxItems ? kCsMaxItemsThreads : 1024)
+cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restrict__ ev_lo, int N,
+                     const int32_t* __restrict__ ev_budget, const int32_t* __restrict__ ev_out_off, CsLayout lay,
+                     uint8_t* __restrict__ is_key, int32_t* __restrict__ out_src, int32_t* __restrict__ out_event,
+                     int32_t* __restrict__ assign, int32_t* __restrict__ rest) {
+    grid_dep_wait();
+    __shared__ CsShared sm;
+    extern __shared__ __align__(16) unsigned char sel_dyn[];
+    constexpr int C = kCl ? kCsMaxCluster : 1;
+    const int e = blockIdx.x / C, rank = blockIdx.x - e * C;
+    const int lo = ev_lo[e] * N, n = ev_lo[e + 1] * N - lo;
+    if (n <= 0) return;
+    const float* sc = token_score + lo;
+    const int budget = ev_budget[e], slot0 = ev_out_off[e];
+#define METOK_EVENT_TOPK(ITEMS, CLUSTER, RANK) \
+    cs_event_topk<ITEMS, CLUSTER>(sm, sel_dyn, lay, sc, lo, n, e, budget, slot0, RANK, is_key, out_src, out_event, assign, rest)
+    // most events are much shorter than the longest possible one: the cluster's first CTA takes them alone
+    const bool solo = !kCl || n <= min(kCsSolo, 4 * (int)blockDim.x);
+    if (solo) {
+        if (rank == 0) {
+            if (IT != 8 || n <= 4 * (int)blockDim.x) METOK_EVENT_TOPK(4, false, 0);
+            else METOK_EVENT_TOPK(8, false, 0);
+        }
+        return;
     }
+    if constexpr (kCl) {
+        cs_enter<true>();
+        if (IT == 4 || n <= 4 * C * (int)blockDim.x) METOK_EVENT_TOPK(4, true, rank);
+        else METOK_EVENT_TOPK(IT, true, rank);
+    }
+#undef METOK_EVENT_TOPK
 }
 
 // --------------------------------------------------------------------------- //
@@ -1428,16 +1439,25 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     }
 
     {
-        // the cache is sized for the longest event there can be, the thread count for twice the mean
         // an event has at most Tn - (k - 1) frames
-        const BlockSelLayout bl = block_sel_layout(1, (long long)(Tn - (k - 1)) * N, 0);
-        if (bl.fits) {
-            if (bl.bytes > 32 * 1024)
-                METOK_ALLOW_SMEM(event_block_topk_kernel, bl.bytes);
+        const long long longest = (long long)(Tn - (k - 1)) * N;
+        const CsPlan plan = cs_plan(longest);
+        if (plan.fits) {
+            const CsLayout lay = cs_layout(1, std::max(Nv / k, 2048));          // buckets for the mean event
             METOK_TIMED("event_topk_kernel", st);
-            launch_chained(event_block_topk_kernel, dim3(k), dim3(kBsThreads), bl.bytes, st, token_score, w.ev_lo, N, w.ev_budget, w.ev_out_off,
-                                                                     bl, w.is_key, out_src, out_event, assign, w.rest);
+            auto launch = [&](auto kernel, int C, int threads) {
+                launch_chained_clusters(C, kernel, dim3(k * C), dim3(threads), lay.bytes, st, token_score, w.ev_lo, N, w.ev_budget,
+                                        w.ev_out_off, lay, w.is_key, out_src, out_event, assign, w.rest);
+            };
+            // One CTA per event where that holds the longest one there can be.  Clusters, most of which come down to
+            // their first CTA, cost nothing while all of them are resident at once; with more events (61 of them: 488
+            // CTAs of 1024 threads, 9 us against 6) a CTA with eight items per thread is preferred as long as it can.
+            if (plan.C == 1) launch(cs_event_topk_kernel<4, false>, 1, plan.threads);
+            else if (longest <= 2 * kCsSolo && k * plan.C > kNumSMs) launch(cs_event_topk_kernel<8, false>, 1, 1024);
+            else if (plan.items == 4) launch(cs_event_topk_kernel<4, true>, plan.C, kCsSolo / 4);
+            else launch(cs_event_topk_kernel<kCsMaxItems, true>, plan.C, kCsMaxItemsThreads);
         } else {
+            // the cache is sized for the longest event there can be, the thread count for twice the mean
             const SelectLayout lay = select_layout(1, select_items_per_cta((long long)(Tn - (k - 1)) * N));
             const int nthreads = select_threads(select_items_per_cta(2LL * Nv / k));
             if (lay.bytes > 32 * 1024)                    // static + dynamic beyond 48 KiB needs the opt-in
