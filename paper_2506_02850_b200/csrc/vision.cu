@@ -1,6 +1,7 @@
 // metok_compress_vision: text relevance and key events (Eq. 5), per-event key-token
 // top-k, merge-assign of the remaining tokens and averaging.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 
 #include "common.cuh"
@@ -119,27 +120,6 @@ struct PlanParams {
     const uint8_t* key_frames_given;            // POOL: the caller's key frames, or null
 };
 
-// The workspace regions that later kernels of the call expect cleared: written here, at the start of
-// the call's first kernel, instead of by separate memset nodes (each costs the chain a launch).
-struct PlanClears {
-    void* zero_a; size_t zero_a_bytes;      // packed argmax per token, may be null
-    void* zero_b; size_t zero_b_bytes;      // member bits, member counts, long-list counters
-    void* ones;   size_t ones_bytes;        // output -> long-list index, all bits set = none
-    int32_t* status;                        // device status word
-};
-// part `part` of `parts` of the fill; p 16-byte aligned, bytes % 4 == 0
-__device__ __forceinline__ void block_fill(void* p, size_t bytes, uint32_t word, int part, int parts) {
-    if (!p) return;
-    uint4* q = reinterpret_cast<uint4*>(p);
-    const size_t n16 = bytes / 16;
-    for (size_t i = (size_t)part * blockDim.x + threadIdx.x; i < n16; i += (size_t)parts * blockDim.x)
-        q[i] = make_uint4(word, word, word, word);
-    uint32_t* t = reinterpret_cast<uint32_t*>(q + n16);
-    if (part == 0)
-        for (size_t i = threadIdx.x; i < (bytes - n16 * 16) / 4; i += blockDim.x) t[i] = word;
-}
-constexpr int kPlanFillCtas = 8;
-
 __global__ void __launch_bounds__(1024)
 event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ frame_score,
                   const int32_t* __restrict__ event_offsets, PlanParams pp,
@@ -147,16 +127,12 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
                   int32_t* __restrict__ ev_lo, int32_t* __restrict__ ev_budget, int32_t* __restrict__ ev_out_off,
                   int32_t* __restrict__ ev_unit_off,
                   int32_t* __restrict__ frame_ev, int32_t* __restrict__ frame_stride,
-                  int32_t* __restrict__ frame_off, int32_t* __restrict__ n_out, PlanClears clr) {
+                  int32_t* __restrict__ frame_off, int32_t* __restrict__ n_out, int32_t* __restrict__ counters, int n_counters,
+                  int32_t* __restrict__ status) {
     grid_dep_wait();
     extern __shared__ float s_score[];      // [k]
-    if (blockIdx.x > 0) {                   // CTAs 1 .. kPlanFillCtas only clear; CTA 0 plans
-        block_fill(clr.zero_a, clr.zero_a_bytes, 0u, (int)blockIdx.x - 1, kPlanFillCtas);
-        block_fill(clr.zero_b, clr.zero_b_bytes, 0u, (int)blockIdx.x - 1, kPlanFillCtas);
-        block_fill(clr.ones, clr.ones_bytes, 0xFFFFFFFFu, (int)blockIdx.x - 1, kPlanFillCtas);
-        return;
-    }
-    if (threadIdx.x == 0) *clr.status = 0;
+    if (threadIdx.x == 0) *status = 0;
+    for (int i = threadIdx.x; i < n_counters; i += blockDim.x) counters[i] = 0;   // what later kernels of the call count in
     __shared__ int s_scan[1024];
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int k = pp.k, Tn = pp.Tn;
@@ -398,13 +374,72 @@ pool_kernel(const T* __restrict__ feats, int d, int N, int G, int Tn, const int3
     }
 }
 
-// Per-event key-token top-k: one cluster per event.  `rest` lists the event's other tokens, from the event's first
-// token's place on.
+// --------------------------------------------------------------------------- //
+// Member lists.  The kernel that chooses the key tokens starts the list of every output token with its key
+// token; the merge-assign kernels add a token as soon as its output is known.  Per output: the number of members,
+// the first kAvgFew of them in order of arrival, a bit per block of the event that holds a member (an output
+// with more members is searched for there), and lists of the outputs with many.
+// --------------------------------------------------------------------------- //
+constexpr int kAvgFew = 128;       // members listed per output
+constexpr int kAvgHeavy = 16;      // outputs with more members are averaged by whole CTAs,
+constexpr int kAvgLong = kAvgFew;  // those with more than this in parts
+struct MemberLists {
+    unsigned long long* blocks;    // per output token: which blocks of its event hold a member
+    int32_t* count;                // per output token: members
+    int32_t* few;                  // per output token: its first kAvgFew members
+    int32_t *heavy_slot, *long_slot;         // the outputs with more than kAvgHeavy (kAvgLong) members
+    int32_t *heavy_counter, *long_counter;   // and how many there are
+};
+// An event's tokens are cut into at most 64 blocks of this many tokens.
+__host__ __device__ __forceinline__ int avg_block_tokens(int m) {
+    const int g = (((m + 63) / 64) + 3) & ~3;
+    return g < 256 ? 256 : g;
+}
+// Token `row`, the i-th of its event of m tokens, is the key token of output `slot`.
+__device__ __forceinline__ void members_start(const MemberLists& ml, int slot, int row, int i, int m) {
+    ml.count[slot] = 1;
+    ml.few[(size_t)slot * kAvgFew] = row;
+    ml.blocks[slot] = 1ull << (i / avg_block_tokens(m));
+}
+// It joins output `slot`.  (Which place of the list or index an output gets depends on arrival order, what is computed
+// from the lists does not.)
+__device__ __forceinline__ void members_join(const MemberLists& ml, int slot, int row, int i, int m) {
+    atomicOr(&ml.blocks[slot], 1ull << (i / avg_block_tokens(m)));
+    const int pos = atomicAdd(&ml.count[slot], 1);
+    if (pos < kAvgFew) ml.few[(size_t)slot * kAvgFew + pos] = row;
+    if (pos == kAvgHeavy) ml.heavy_slot[atomicAdd(ml.heavy_counter, 1)] = slot;
+    if (pos == kAvgLong) ml.long_slot[atomicAdd(ml.long_counter, 1)] = slot;
+}
+// What the kernels that choose the key tokens write per token: whether it is one, its output if so, its place in the
+// list of the others if not, and the cleared scratch of its merge.
+struct TokenOut {
+    uint8_t* is_key;
+    int32_t *out_src, *out_event, *assign;
+    int32_t* rest;                 // per event, from its first token's place on: its tokens that are no key token
+    unsigned long long* best64;    // packed argmax of the token's similarities
+    int32_t* tile_done;            // at a row tile's first token: key chunks of the tile that are done
+    MemberLists ml;
+};
+__device__ __forceinline__ void token_out(const TokenOut& o, int lo, int n, int i, int e, int slot0, int place, bool key) {
+    o.is_key[lo + i] = key ? 1 : 0;
+    o.best64[lo + i] = 0ull;
+    o.tile_done[lo + i] = 0;
+    if (key) {
+        const int slot = slot0 + place;
+        o.out_src[slot] = lo + i;
+        o.out_event[slot] = e;
+        o.assign[lo + i] = slot;
+        members_start(o.ml, slot, lo + i, i, n);
+    } else {
+        o.rest[lo + i - place] = lo + i;
+    }
+}
+
+// Per-event key-token top-k: one cluster per event.
 __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThreads)
 event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restrict__ ev_lo, int N,
                   const int32_t* __restrict__ ev_budget, const int32_t* __restrict__ ev_out_off, SelectLayout lay,
-                  uint8_t* __restrict__ is_key, int32_t* __restrict__ out_src, int32_t* __restrict__ out_event,
-                  int32_t* __restrict__ assign, int32_t* __restrict__ rest) {
+                  TokenOut out) {
     __shared__ SelectSmem sm;
     __shared__ int s_budget[1];
     extern __shared__ __align__(16) unsigned char sel_dyn[];
@@ -433,14 +468,8 @@ event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restri
     cluster_select(cx, n, cls, val, s_budget, sm);
     const int slot0 = ev_out_off[e];
     auto flag = [&](int i) { return is_selected(sm, 0, item_at(cx, i - p_lo, cls, val).key, i); };
-    auto emit = [&](int i, int rank) {
-        const int slot = slot0 + rank;
-        out_src[slot] = lo + i;
-        out_event[slot] = e;
-        assign[lo + i] = slot;
-    };
-    for (int i = p_lo + threadIdx.x; i < p_hi; i += blockDim.x) is_key[lo + i] = flag(i) ? 1 : 0;
-    auto skip = [&](int i, int before) { rest[lo + i - before] = lo + i; };
+    auto emit = [&](int i, int rank) { token_out(out, lo, n, i, e, slot0, rank, true); };
+    auto skip = [&](int i, int before) { token_out(out, lo, n, i, e, slot0, before, false); };
     cluster_compact(cx, p_lo, p_hi, flag, emit, skip, sm);
 }
 
@@ -448,30 +477,20 @@ event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restri
 template <int IT, bool kCl>
 __device__ __forceinline__ void
 cs_event_topk(CsShared& sm, unsigned char* dyn, const CsLayout& lay, const float* __restrict__ sc, int lo, int n, int e,
-              int budget, int slot0, int rank, uint8_t* __restrict__ is_key, int32_t* __restrict__ out_src,
-              int32_t* __restrict__ out_event, int32_t* __restrict__ assign, int32_t* __restrict__ rest) {
+              int budget, int slot0, int rank, const TokenOut& out) {
     const CsSlice sl = cs_slice<IT>(n, rank, kCl ? kCsMaxCluster : 1);
     int before, kept;
     const uint32_t bits = cs_select<IT, kCl, true>(sm, dyn, lay, 1, &budget, rank, sl.i_first, sl.i_hi,
                                                    [&](int i, float& v, int& c) { v = sc[i]; c = 0; }, &before, &kept);
-    cs_for_items<IT>(bits, before, sl.i_first, sl.i_hi, [&](int, int i, int place, bool key) {
-        is_key[lo + i] = key ? 1 : 0;
-        if (key) {
-            out_src[slot0 + place] = lo + i;
-            out_event[slot0 + place] = e;
-            assign[lo + i] = slot0 + place;
-        } else {
-            rest[lo + i - place] = lo + i;
-        }
-    });
+    cs_for_items<IT>(bits, before, sl.i_first, sl.i_hi,
+                     [&](int, int i, int place, bool key) { token_out(out, lo, n, i, e, slot0, place, key); });
 }
 
 template <int IT, bool kCl>
 __global__ void __launch_bounds__(IT == kCsMaxItems ? kCsMaxItemsThreads : 1024)
 cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restrict__ ev_lo, int N,
                      const int32_t* __restrict__ ev_budget, const int32_t* __restrict__ ev_out_off, CsLayout lay,
-                     uint8_t* __restrict__ is_key, int32_t* __restrict__ out_src, int32_t* __restrict__ out_event,
-                     int32_t* __restrict__ assign, int32_t* __restrict__ rest) {
+                     TokenOut out) {
     grid_dep_wait();
     __shared__ CsShared sm;
     extern __shared__ __align__(16) unsigned char sel_dyn[];
@@ -482,7 +501,7 @@ cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __res
     const float* sc = token_score + lo;
     const int budget = ev_budget[e], slot0 = ev_out_off[e];
 #define METOK_EVENT_TOPK(ITEMS, CLUSTER, RANK) \
-    cs_event_topk<ITEMS, CLUSTER>(sm, sel_dyn, lay, sc, lo, n, e, budget, slot0, RANK, is_key, out_src, out_event, assign, rest)
+    cs_event_topk<ITEMS, CLUSTER>(sm, sel_dyn, lay, sc, lo, n, e, budget, slot0, RANK, out)
     // most events are much shorter than the longest possible one: the cluster's first CTA takes them alone
     const bool solo = !kCl || n <= min(kCsSolo, 4 * (int)blockDim.x);
     if (solo) {
@@ -533,9 +552,9 @@ template <typename T>
 __global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? kSaCtasPerSm : 4)
 merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_t* __restrict__ ev_lo, int k,
                          const int32_t* __restrict__ ev_out_off, const int32_t* __restrict__ ev_unit_off,
-                         const int32_t* __restrict__ out_src, const int32_t* __restrict__ rest,
-                         const float* __restrict__ inv_norm, unsigned long long* __restrict__ best64) {
+                         const float* __restrict__ inv_norm, TokenOut out) {
     grid_dep_wait();
+    const int32_t *out_src = out.out_src, *rest = out.rest;
     constexpr int CE = 16 / sizeof(T);              // elements per 16-byte chunk
     constexpr int CPR = kSaBK / CE;                 // chunks per row and stage
     constexpr int LD = kSaBK + CE;                  // row pitch in elements
@@ -622,9 +641,22 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
             }
             const int at = row0 + ty + 8 * i;
             if (tx == 0 && at < row_end && best_s != 0x7FFFFFFF)
-                atomicMax(&best64[rest[at]], ((unsigned long long)float_key(best_v) << 32) | (unsigned long long)(~(uint32_t)best_s));
+                atomicMax(&out.best64[rest[at]], ((unsigned long long)float_key(best_v) << 32) | (unsigned long long)(~(uint32_t)best_s));
         }
     }
+}
+
+// After it: every token that is no key token to its output.  (In the tensor-core kernel the CTA that does a row tile's last
+// chunk does this; here that cost 15 us at 61 frames, this kernel takes 5.)
+__global__ void __launch_bounds__(256)
+merge_join_kernel(int Nv, int N, const int32_t* __restrict__ ev_lo, int k, const int32_t* __restrict__ ev_out_off, TokenOut out) {
+    grid_dep_wait();
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= Nv || out.is_key[row]) return;
+    const int e = find_event(ev_lo, k, row / N);
+    const int lo = ev_lo[e] * N, slot = (int32_t)(~(uint32_t)(out.best64[row] & 0xFFFFFFFFull));
+    out.assign[row] = slot;
+    if (slot >= ev_out_off[e] && slot < ev_out_off[e + 1]) members_join(out.ml, slot, row, row - lo, ev_lo[e + 1] * N - lo);
 }
 
 
@@ -650,35 +682,44 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
 //              slice (one per row half), and commits to the ring / accumulator barriers;
 //   warps 2-9: epilogue, four warps per row half -- read the accumulator with
 //              tcgen05.ld, scale each column by 1/|key|, take the (value, slot) argmax of
-//              the thread's row over the chunk.
+//              the thread's row over the chunk, and add the row's token to its output's member
+//              list once all chunks are known.
 // Chunks of one row tile may be handled by different CTAs: a row's result is combined
 // with a 64-bit atomicMax on (order-preserving key of the value) << 32 | ~slot, which
 // does not depend on the order of arrival (larger value first, then the lower slot).
 // Every wait is bounded; on a timeout the CTA unwinds and writes METOK_ERR_TIMEOUT.
 // --------------------------------------------------------------------------- //
-constexpr int kMmaBM = 256, kMmaBK = 64, kMmaBN = 256, kMmaStages = 3;
+constexpr int kMmaBM = 256, kMmaBK = 64, kMmaBN = 256, kMmaMaxStages = 6;
 constexpr int kMmaThreads = 448;
 constexpr int kMmaKeyThreads = 128;                        // warps 10-13
-constexpr uint32_t kMmaABytes = kMmaBM * kMmaBK * 2;       // 32 KiB
-constexpr uint32_t kMmaBBytes = kMmaBN * kMmaBK * 2;       // 32 KiB
-constexpr size_t kMmaSmemBytes = (size_t)kMmaStages * (kMmaABytes + kMmaBBytes) + 1024;
+constexpr uint32_t kMmaRingBytes = 192 * 1024;
+constexpr size_t kMmaSmemBytes = kMmaRingBytes + 1024;
+// Unit shape of a launch: up to bm token rows (128 or 256) x up to bn keys (a multiple of 16), and what follows from it.
+struct MmaTile {
+    int bm, bn, stages;
+    uint32_t a_bytes, stage_bytes;
+};
 
-struct MergeUnit { int row0, row_end, col0, nvalid; };     // rows of V; first key slot and number of keys
+struct MergeUnit { int row_lo, row0, row_end, col0, nvalid, nchunks, slot0, slot_end; };   // the event's first row, the unit's rows; first key slot and number of keys; the event's chunks and slots
 
 __device__ __forceinline__ MergeUnit merge_unit(int u, const int32_t* __restrict__ ev_unit_off,
                                                 const int32_t* __restrict__ ev_lo,
-                                                const int32_t* __restrict__ ev_out_off, int k, int N) {
+                                                const int32_t* __restrict__ ev_out_off, int k, int N, const MmaTile& mt) {
     const int e = find_event(ev_unit_off, k, u);
     const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0;
-    const int nchunks = (nk + kMmaBN - 1) / kMmaBN;
+    const int nchunks = (nk + mt.bn - 1) / mt.bn;
     const int cols = (((nk + nchunks - 1) / nchunks) + 15) & ~15;       // equal chunks, whole MMA columns
     const int local = u - ev_unit_off[e];
     const int tile = local / nchunks, c = local - tile * nchunks;
     MergeUnit m;
-    m.row0 = ev_lo[e] * N + tile * kMmaBM;
+    m.row_lo = ev_lo[e] * N;
+    m.row0 = m.row_lo + tile * mt.bm;
     m.row_end = ev_lo[e + 1] * N;
     m.col0 = s0 + c * cols;
     m.nvalid = min(cols, nk - c * cols);
+    m.nchunks = nchunks;
+    m.slot0 = s0;
+    m.slot_end = s0 + nk;
     return m;
 }
 
@@ -686,16 +727,17 @@ __global__ void __launch_bounds__(kMmaThreads, 1)
 merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA_half,
                         const __nv_bfloat16* __restrict__ feats, int d, int N,
                         const int32_t* __restrict__ ev_lo, int k, const int32_t* __restrict__ ev_out_off,
-                        const int32_t* __restrict__ ev_unit_off, const int32_t* __restrict__ out_src,
-                        const float* __restrict__ inv_norm, const uint8_t* __restrict__ is_key,
-                        unsigned long long* __restrict__ best64, int32_t* __restrict__ status) {
+                        const int32_t* __restrict__ ev_unit_off, const float* __restrict__ inv_norm, MmaTile mt,
+                        TokenOut out, int32_t* __restrict__ status) {
     grid_dep_wait();
     using namespace sm100;
+    const int32_t* out_src = out.out_src;
     extern __shared__ uint8_t smem_dyn[];
-    __shared__ __align__(8) uint64_t full_bar[kMmaStages], empty_bar[kMmaStages], tfull_bar, tempty_bar, drain_bar;
+    __shared__ __align__(8) uint64_t full_bar[kMmaMaxStages], empty_bar[kMmaMaxStages], tfull_bar, tempty_bar, drain_bar;
     __shared__ uint32_t s_tmem_base;
-    __shared__ int s_abort;
-    __shared__ float s_keyinv[2][kMmaBN];
+    __shared__ int s_abort, s_last;
+    __shared__ __align__(16) float s_keyinv[2][kMmaBN];
+    const int kMmaStages = mt.stages;
 
     const int total_units = ev_unit_off[k];
     if ((int)blockIdx.x >= total_units) return;
@@ -734,16 +776,16 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             uint32_t ph = 0;
             bool ok = true;
             for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
-                const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N);
-                const bool two = mu.row_end - mu.row0 > 128;           // both row halves hold rows of the event
+                const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
+                const bool two = mt.bm > 128 && mu.row_end - mu.row0 > 128;   // both row halves hold rows of the event
                 const CUtensorMap* a0 = two ? &tmA : &tmA_half;
-                const uint32_t tx = two ? kMmaABytes : kMmaABytes / 2;
+                const uint32_t tx = (two ? 256u : 128u) * kMmaBK * 2;
                 for (int ks = 0; ks < ksteps; ++ks) {
                     if (!mbar_wait(smem_u32(&empty_bar[0]) + 8u * s, ph ^ 1u, abort_flag)) { ok = false; break; }
                     const uint32_t fb = smem_u32(&full_bar[0]) + 8u * s;
                     mbar_arrive_expect_tx(fb, tx);
                     if (!(dbg_withhold(status, kDbgMergeAssign) && blockIdx.x == 0 && issued == 0))   // debug builds: one copy never sent
-                        tma_load_2d(smem_base + (uint32_t)s * (kMmaABytes + kMmaBBytes), a0, ks * kMmaBK, mu.row0, fb);
+                        tma_load_2d(smem_base + (uint32_t)s * mt.stage_bytes, a0, ks * kMmaBK, mu.row0, fb);
                     ++issued;
                     if (++s == kMmaStages) { s = 0; ph ^= 1u; }
                 }
@@ -762,11 +804,11 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             uint32_t ph = 0;
             bool ok = true;
             const uint32_t a_lo0 = desc_k128_lo(smem_base);
-            constexpr uint32_t kStageWords = (kMmaABytes + kMmaBBytes) >> 4, kBWords = kMmaABytes >> 4,
-                               kHalfWords = (kMmaABytes / 2) >> 4;
+            const uint32_t kStageWords = mt.stage_bytes >> 4, kBWords = mt.a_bytes >> 4;
+            constexpr uint32_t kHalfWords = (128 * kMmaBK * 2) >> 4;
             for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++n) {
-                const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N);
-                const bool two = mu.row_end - mu.row0 > 128;
+                const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
+                const bool two = mt.bm > 128 && mu.row_end - mu.row0 > 128;
                 if (!mbar_wait(smem_u32(&tempty_bar), ((uint32_t)n & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t idesc = make_idesc_bf16(128, (mu.nvalid + 15) & ~15);
@@ -804,12 +846,12 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         // position c ^ (r % 8).  Rows past the chunk's keys up to the next multiple of 16 (the MMA's
         // column count) are written as zeros; rows beyond are not touched.
         const int pt = (int)threadIdx.x - 320, c = pt & 7, rsub = pt >> 3;
-        const uint32_t dst0 = smem_base + kMmaABytes + (uint32_t)rsub * 128u + (uint32_t)((c ^ (rsub & 7)) << 4);   // (r % 8) == (rsub % 8)
+        const uint32_t dst0 = smem_base + mt.a_bytes + (uint32_t)rsub * 128u + (uint32_t)((c ^ (rsub & 7)) << 4);   // (r % 8) == (rsub % 8)
         int s = 0;
         uint32_t ph = 0;
         bool ok = true;
         for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
-            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N);
+            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
             const int npad = (mu.nvalid + 15) & ~15;
             const __nv_bfloat16* src[16];
 #pragma unroll
@@ -820,7 +862,7 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             }
             for (int ks = 0; ks < ksteps; ++ks) {
                 if (!mbar_wait(smem_u32(&empty_bar[0]) + 8u * s, ph ^ 1u, abort_flag)) { ok = false; break; }
-                const uint32_t dst = dst0 + (uint32_t)s * (kMmaABytes + kMmaBBytes);
+                const uint32_t dst = dst0 + (uint32_t)s * mt.stage_bytes;
                 // a K slice that reaches past d (d is a multiple of 8, not of 64) reads zeros there
                 const bool in_k = ks * kMmaBK + c * 8 < d;
 #pragma unroll
@@ -842,37 +884,90 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         bool ok = true;
         int n = 0;
         for (int u = blockIdx.x; u < total_units; u += gridDim.x, ++n) {
-            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N);
+            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
             const int b = n & 1;                                    // s_keyinv alternates: a slow warp may still read the last one
             s_keyinv[b][et] = (et < mu.nvalid) ? inv_norm[out_src[mu.col0 + et]] : 0.f;
             named_bar_sync(1, 256);
             if (ok && !mbar_wait(smem_u32(&tfull_bar), (uint32_t)n & 1u, abort_flag)) ok = false;
             ok = __all_sync(0xFFFFFFFFu, ok);                      // tcgen05.ld below is warp-collective
-            if (!ok) continue;                                     // keep meeting the others at the named barrier
-            tc_fence_after();
             const int row = mu.row0 + half * 128 + grp * 32 + lane;
+            // the second accumulator of a short unit holds nothing
+            const bool mine = half == 0 || (mt.bm > 128 && mu.row_end - mu.row0 > 128);
             float best_v = -3.4e38f;
             int best_c = 0;
-            if (half == 0 || mu.row_end - mu.row0 > 128) {          // the second accumulator of a short unit holds nothing
-                const uint32_t t_row = tmem_base + ((uint32_t)(grp * 32) << 16) + (uint32_t)half * kMmaBN;
-                for (int c0 = 0; c0 < mu.nvalid; c0 += 32) {
-                    float v[32];
-                    tmem_ld32(t_row + (uint32_t)c0, v);
+            if (ok) {
+                tc_fence_after();
+                if (mine) {
+                    // Row argmax.  An element costs an instruction or two: four products and their maximum, and only if
+                    // that beats the row's best are the four kept, so that the column is found once at the end (the
+                    // first column of the first group that reached the maximum, as a scan in column order finds it).
+                    const uint32_t t_row = tmem_base + ((uint32_t)(grp * 32) << 16) + (uint32_t)half * kMmaBN;
+                    float b0 = 0.f, b1 = 0.f, b2 = 0.f;
+                    uint32_t raw[2][32];
+                    auto fold = [&](int c0, const uint32_t (&r)[32]) {
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int col = c0 + j;
-                        const float val = v[j] * s_keyinv[b][col];
-                        if (col < mu.nvalid && val > best_v) { best_v = val; best_c = col; }
+                        for (int j = 0; j < 32; j += 4) {
+                            const float4 ki = *reinterpret_cast<const float4*>(&s_keyinv[b][c0 + j]);
+                            const float p0 = __uint_as_float(r[j]) * ki.x, p1 = __uint_as_float(r[j + 1]) * ki.y,
+                                        p2 = __uint_as_float(r[j + 2]) * ki.z, p3 = __uint_as_float(r[j + 3]) * ki.w;
+                            const float m4 = fmaxf(fmaxf(p0, p1), fmaxf(p2, p3));
+                            if (m4 > best_v) { best_v = m4; best_c = c0 + j; b0 = p0; b1 = p1; b2 = p2; }
+                        }
+                    };
+                    const int full = mu.nvalid & ~31;
+                    if (full > 0) tmem_ld32_issue(t_row, raw[0]);
+#pragma unroll 1
+                    for (int c0 = 0; c0 < full; c0 += 64) {         // the next 32 columns are fetched while these are reduced
+                        tmem_ld32_wait(raw[0]);
+                        if (c0 + 32 < full) tmem_ld32_issue(t_row + (uint32_t)c0 + 32u, raw[1]);
+                        fold(c0, raw[0]);
+                        if (c0 + 32 < full) {
+                            tmem_ld32_wait(raw[1]);
+                            if (c0 + 64 < full) tmem_ld32_issue(t_row + (uint32_t)c0 + 64u, raw[0]);
+                            fold(c0 + 32, raw[1]);
+                        }
+                    }
+                    if (best_v > -3.4e38f) best_c += b0 == best_v ? 0 : b1 == best_v ? 1 : b2 == best_v ? 2 : 3;
+                    if (full < mu.nvalid) {
+                        float v[32];
+                        tmem_ld32(t_row + (uint32_t)full, v);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            const float val = v[j] * s_keyinv[b][(full + j) & (kMmaBN - 1)];
+                            if (full + j < mu.nvalid && val > best_v) { best_v = val; best_c = full + j; }
+                        }
                     }
                 }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&tempty_bar));
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&tempty_bar));
-            if (row < mu.row_end && !is_key[row]) {
-                const unsigned long long packed =
-                    ((unsigned long long)float_key(best_v) << 32) | (unsigned long long)(~(uint32_t)(mu.col0 + best_c));
-                atomicMax(&best64[row], packed);
+            // (a warp that gave up keeps meeting the others at the named barriers)
+            const bool have = ok && mine && row < mu.row_end && !out.is_key[row];
+            int slot = mu.col0 + best_c;
+            bool last = true;
+            if (mu.nchunks > 1) {
+                // the chunks of a row tile meet in an order-independent maximum; whoever comes last has the result
+                if (have)
+                    atomicMax(&out.best64[row], ((unsigned long long)float_key(best_v) << 32) | (unsigned long long)(~(uint32_t)slot));
+                __threadfence();
+                named_bar_sync(1, 256);
+                if (et == 0) s_last = atomicAdd(&out.tile_done[mu.row0], 1) == mu.nchunks - 1;
+                named_bar_sync(1, 256);
+                last = s_last;
+                if (have && last) {
+                    __threadfence();
+                    slot = (int32_t)(~(uint32_t)(__ldcg(&out.best64[row]) & 0xFFFFFFFFull));
+                }
+            }
+            if (have && last) {
+                out.assign[row] = slot;
+                // a token whose unit gave up on a wait has no maximum: it stays out of every member list (the call's
+                // status word says that the results are not valid)
+                if (slot >= mu.slot0 && slot < mu.slot_end) {
+                    const int lo = mu.row_lo;
+                    members_join(out.ml, slot, row, row - lo, mu.row_end - lo);
+                }
             }
         }
     }
@@ -882,419 +977,440 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     if (threadIdx.x == 0 && s_abort) *status = METOK_ERR_TIMEOUT;
 }
 
-// An event's tokens are cut into at most 64 blocks of this many tokens; per output token one
-// bit per block says whether the block holds a member.
-__host__ __device__ __forceinline__ int avg_block_tokens(int m) {
-    const int g = (((m + 63) / 64) + 3) & ~3;
-    return g < 256 ? 256 : g;
-}
-
-// assign[row] of every non-key token from the packed argmax, and the member-block bits of every output token.
-__global__ void __launch_bounds__(256)
-merge_decode_kernel(const unsigned long long* __restrict__ best64, const uint8_t* __restrict__ is_key, int Nv,
-                    int N, const int32_t* __restrict__ ev_lo, int k, int32_t* __restrict__ assign,
-                    unsigned long long* __restrict__ slot_blocks, int32_t* __restrict__ slot_cnt,
-                    int32_t* __restrict__ long_index, int32_t* __restrict__ long_slot,
-                    int32_t* __restrict__ long_counter, int long_threshold, int long_cap,
-                    int32_t* __restrict__ few_members, int few_cap, int32_t* __restrict__ heavy_index,
-                    int32_t* __restrict__ heavy_slot, int32_t* __restrict__ heavy_counter, int heavy_threshold,
-                    int heavy_cap,
-                    const int32_t* __restrict__ n_out) {
-    grid_dep_wait();
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= Nv) return;
-    int slot;
-    if (!is_key[row]) {
-        slot = (int32_t)(~(uint32_t)(best64[row] & 0xFFFFFFFFull));
-        assign[row] = slot;
-    } else {
-        slot = assign[row];
-    }
-    // a token whose unit gave up on a wait has no maximum: it stays out of every member list (the
-    // call's status word already says that the results are not valid)
-    if (slot < 0 || slot >= *n_out) return;
-    const int e = find_event(ev_lo, k, row / N);
-    const int lo = ev_lo[e] * N, m = ev_lo[e + 1] * N - lo;
-    atomicOr(&slot_blocks[slot], 1ull << ((row - lo) / avg_block_tokens(m)));
-    // member count; the token that takes an output past the threshold books scratch for it (which
-    // scratch an output gets depends on arrival order, what is computed in it does not)
-    const int pos = atomicAdd(&slot_cnt[slot], 1);
-    if (pos < few_cap) few_members[(size_t)slot * few_cap + pos] = row;   // the first few_cap arrivals are listed
-    if (pos == heavy_threshold) {                             // many members: an output to be started early
-        const int hh = atomicAdd(heavy_counter, 1);
-        heavy_index[slot] = hh;
-        if (hh < heavy_cap) heavy_slot[hh] = slot;
-    }
-    if (pos == long_threshold) {
-        const int l = atomicAdd(long_counter, 1);
-        long_index[slot] = l;
-        if (l < long_cap) long_slot[l] = slot;
-    }
-}
-
 // --------------------------------------------------------------------------- //
-// Averaging: one CTA per output token.  Only the blocks of the event that hold a member
-// (one bit each, set by merge_decode) are searched: their `assign` entries are read in
-// passes in which every thread takes a contiguous run (16-byte loads, all issued before
-// the first is looked at), the matches are packed in token order by one block-wide
-// scan, and the member rows are then added in that order (so the
-// summation order is fixed).  The rows come in by bulk copies into shared memory, up to
-// kAvgStages rows at once (usually all members of an output), so that the bytes in
-// flight do not depend on registers.  fp32 sum, one division, one rounding.
+// Averaging: a warp per (output, piece of its row).  The member rows' pieces come by 16-byte asynchronous copies into
+// a ring of the warp's own, a stream that runs on from piece to piece, are added in token order in fp32, divided and
+// rounded once.  No barrier wider than the warp.  What bounds it is not the memory (a warp waits for its copies a
+// tenth of its time) but the fixed cost of a row and of a piece, so these are kept short and independent of each other:
+// with a CTA per output, a CTA lived about 4 us for its dependent round trips (list, rows) however short the rows were,
+// and 14 775 outputs of 2 KB rows shared 1184 CTA slots: 91 us between kernels of a replayed graph, 37 now; 3693 outputs
+// of 7 KB rows take the 29 us they took.  The grid is what fits at once; a warp takes its first pieces by its number and
+// the later ones from a counter, a piece ahead.  Rows are averaged from their last piece to their first, and outputs from
+// the last down: the merge-assign pass before this one sweeps the columns of all rows together and leaves the last ones
+// in L2.
+//
+// Outputs with many members would set the kernel's time if a warp took one late, so they come first and a CTA each: its
+// warps take a quarter of the members and their sums are added in warp order.  More than kAvgLong members are not all
+// listed: they are found by searching the event's blocks that hold one, in up to kAvgParts parts (a CTA each, an equal
+// share of the search per warp), and the last part to finish adds the parts' sums in part order.  Such an item is a
+// chain of some ten round trips, 15 to 25 us while the rest of the kernel keeps the memory busy, so its loads are
+// issued together where they can be and every piece of the row is an item of its own.
 // --------------------------------------------------------------------------- //
 constexpr int kAvgThreads = 128;
-constexpr int kAvgChunks = 4;      // 16-byte chunks per thread per pass over d
-constexpr int kAvgQuads = 5;       // 16-byte groups of `assign` per thread and pass
-constexpr int kAvgStages = 3;      // member rows in flight when a pass over a row fills a stage (more than 4 KiB); the same
-                                   // bytes hold 6 or 12 shorter rows (template parameter NST of the kernel)
-constexpr int kAvgList = 512;      // members listed at a time
-constexpr int kAvgStageBytes = kAvgThreads * kAvgChunks * 16;
-constexpr size_t kAvgSmemBytes = (size_t)kAvgStages * kAvgStageBytes + 128;
-constexpr int kAvgFew = 32;        // outputs with at most this many members get them listed by merge_decode (a warp ranks them)
-constexpr int kAvgHeavy = 16;      // outputs with more members than this are listed to be started first
-constexpr int kAvgLong = 32;       // outputs with more members than this (= kAvgFew: the others need no search) are split ...
-constexpr int kAvgParts = 8;       // ... over up to this many CTAs (fp32 partial sums, added in part order)
-constexpr int kAvgLongCapMax = 1024;   // most long outputs that get scratch for their partial sums ...
+constexpr int kAvgWarps = kAvgThreads / 32;
+constexpr int kAvgCtasPerSm = 5;
+constexpr int kAvgRing = 8192;         // bytes per warp
+constexpr int kAvgList = 160;          // members of a long output's part listed at a time per warp: 32 kept over plus a pass of 128
+constexpr int kAvgParts = 16;
+constexpr int kAvgLongCapMax = 1024;   // most long outputs that get scratch for their parts' sums ...
 constexpr size_t kAvgLongBytes = (size_t)32 << 20;   // ... within this much scratch
-constexpr int kAvgHeavyCap = 2048;  // outputs with more than kAvgHeavy members that are listed to be started first
-constexpr int kAvgFrontCtas = 8 * kNumSMs;   // CTAs at the front of the grid that take the listed outputs and parts
+constexpr size_t kAvgSmemBytes = (size_t)kAvgWarps * kAvgRing + 128;
 // long outputs that get scratch: as many as kAvgLongBytes hold (kAvgParts rows of d floats each)
 __host__ __device__ inline int avg_long_cap(int d) {
     const long long c = (long long)(kAvgLongBytes / ((size_t)kAvgParts * (size_t)d * sizeof(float)));
     return (int)(c < 64 ? 64 : c > kAvgLongCapMax ? kAvgLongCapMax : c);
 }
-// parts of an output with `count` > kAvgLong members: about eight members each if they lie evenly
+// parts of an output with `count` > kAvgLong members: about eight members per warp if they lie evenly
 __host__ __device__ inline int avg_parts(int count) {
-    const int p = (count + 7) / 8;
+    const int p = (count + 8 * kAvgWarps - 1) / (8 * kAvgWarps);
     return p < kAvgParts ? p : kAvgParts;
 }
 
-// One (output, part): the members of output c in this part's share of the search, added in token order.
-// What a CTA needs to know about its output before it can fetch a row; the loads are independent of
-// one another, so a caller issues them together with whatever else it has to look up about the output.
-struct AvgMeta {
-    int count, few_tok, li, e;
-    unsigned long long blocks;
+// most pieces a row is cut into (1 KB each, of fp32 or bf16)
+__host__ __device__ inline int avg_max_pieces(int d) { return (d + 255) / 256; }
+
+struct AvgArgs {
+    int d, N, Nv, nseg, seg_chunks;      // a row is cut into nseg pieces of up to seg_chunks 16-byte chunks
+    const int32_t *ev_lo, *out_event, *assign;
+    MemberLists ml;
+    float* long_sums;
+    int32_t *long_done, *next_item, *next;   // parts finished per long output and piece; the next item and piece to take
+    const int32_t* n_out;
+    int32_t *out_members, *status;
 };
-__device__ __forceinline__ AvgMeta avg_meta(int c, const int32_t* __restrict__ slot_cnt,
-                                            const int32_t* __restrict__ few_members,
-                                            const int32_t* __restrict__ long_index,
-                                            const int32_t* __restrict__ out_event,
-                                            const unsigned long long* __restrict__ slot_blocks) {
-    AvgMeta m;
+
+struct AvgPiece { int out, seg, n, pad; int row[kAvgHeavy]; };   // a piece of the stream: its output, piece of the row, members
+constexpr int kAvgQueue = 16;            // a power of two above the R + 1 pieces that R rows can belong to
+
+// The warp's ring of R stages, a barrier each with the parity of its next completion.
+template <int R>
+struct AvgRing {
+    static constexpr uint32_t kStage = kAvgRing / R;
+    static constexpr int kChunks = kStage / 512;             // 16-byte chunks of a row's piece per lane
+    const uint8_t* mem;                  // generic address
+    uint32_t mem_u32, bar_u32, phase;
+    volatile int* abort_flag;
+};
+
+// Starts the copies of chunks [ch0, ch0 + nch) of V's row `row` into a stage; one arrival per lane.
+template <typename T, int R>
+__device__ __forceinline__ void avg_issue(AvgRing<R>& ring, int st, const T* __restrict__ feats, const AvgArgs& ar, int row,
+                                          int ch0, int nch, bool withhold) {
+    using namespace sm100;
     const int lane = threadIdx.x & 31;
-    m.few_tok = lane < kAvgFew ? few_members[(size_t)c * kAvgFew + lane] : 0;
-    m.count = slot_cnt[c];
-    m.li = long_index[c];
-    m.e = out_event[c];
-    m.blocks = slot_blocks[c];
-    return m;
+    const uint32_t row_chunks = (uint32_t)(ar.d * (int)sizeof(T) / 16);
+    const uint4* src = reinterpret_cast<const uint4*>(feats) + (size_t)dbg_bound(row, ar.Nv, ar.status) * row_chunks + ch0 + lane;
+    const uint32_t dst = ring.mem_u32 + (uint32_t)st * AvgRing<R>::kStage + (uint32_t)lane * 16u;
+#pragma unroll
+    for (int u = 0; u < AvgRing<R>::kChunks; ++u)
+        if (u * 32 + lane < nch) cp_async16_zfill(dst + u * 512u, src + u * 32, 16u);
+    if (!(withhold && lane == 0)) cp_async_arrive_noinc(ring.bar_u32 + 8u * st);   // debug builds: one lane's copies never reported
+}
+// Waits for a stage and adds it to acc.  A lane reads only what it has copied itself.  False, for the whole warp, when a
+// wait has given up: nobody may go on alone, the warp's shuffles would read lanes that have left.
+template <typename T, int R>
+__device__ __forceinline__ bool avg_take(AvgRing<R>& ring, int st, float (&acc)[AvgRing<R>::kChunks][16 / sizeof(T)]) {
+    const int lane = threadIdx.x & 31;
+    const bool ok = sm100::mbar_wait(ring.bar_u32 + 8u * st, (ring.phase >> st) & 1u, ring.abort_flag);
+    ring.phase ^= 1u << st;
+    if (!__all_sync(0xFFFFFFFFu, ok)) return false;
+    // chunks past the piece's end add whatever the stage holds to sums that nobody stores: no branches
+    const uint4* row = reinterpret_cast<const uint4*>(ring.mem + st * AvgRing<R>::kStage) + lane;
+    uint4 raw[AvgRing<R>::kChunks];
+#pragma unroll
+    for (int u = 0; u < AvgRing<R>::kChunks; ++u) raw[u] = row[u * 32];
+#pragma unroll
+    for (int u = 0; u < AvgRing<R>::kChunks; ++u) {
+        const uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if constexpr (sizeof(T) == 4) {
+                acc[u][i] += __uint_as_float(w[i]);
+            } else {
+                acc[u][2 * i] += __uint_as_float(w[i] << 16);
+                acc[u][2 * i + 1] += __uint_as_float(w[i] & 0xFFFF0000u);
+            }
+        }
+    }
+    return true;
+}
+// acc += all nlist rows of the list (in shared memory, the same for the whole warp), in its order.
+template <typename T, int R>
+__device__ __forceinline__ void avg_add_rows(AvgRing<R>& ring, const T* __restrict__ feats, const AvgArgs& ar, const int* list,
+                                             int nlist, int ch0, int nch, float (&acc)[AvgRing<R>::kChunks][16 / sizeof(T)]) {
+    for (int m = 0; m < nlist && m < R; ++m) avg_issue<T, R>(ring, m, feats, ar, list[m], ch0, nch, false);
+    int st = 0;
+    for (int m = 0; m < nlist; ++m) {
+        if (!avg_take<T, R>(ring, st, acc)) break;
+        if (m + R < nlist) avg_issue<T, R>(ring, st, feats, ar, list[m + R], ch0, nch, false);
+        st = st + 1 == R ? 0 : st + 1;
+    }
+    __syncwarp();                                            // the list may be written again
 }
 
-template <typename T, int NST>
-__device__ __forceinline__ void
-merge_avg_item(int c, int part, const AvgMeta& meta, uint32_t& phase, uint8_t* avg_dyn, uint64_t* s_bar, int* s_list, int* s_wtot,
-               int* s_blocks, int* s_abort_p, int* s_last_p,
-               const T* __restrict__ feats, int d, int N, int Nv, const int32_t* __restrict__ ev_lo,
-               const int32_t* __restrict__ out_event, const int32_t* __restrict__ assign,
-               const unsigned long long* __restrict__ slot_blocks, const int32_t* __restrict__ slot_cnt,
-               const int32_t* __restrict__ long_index, const int32_t* __restrict__ few_members,
-               float* __restrict__ long_sums, int32_t* __restrict__ long_done, T* __restrict__ out_feats, int32_t* __restrict__ out_members,
-               int32_t* __restrict__ status) {
-    using namespace sm100;
-    constexpr int VN = Vec16<T>::N;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int& s_abort = *s_abort_p;
-    int& s_last = *s_last_p;
-    // an output with at most kAvgFew members has them listed by merge_decode (in arrival order):
-    // fetched together with the output's other data, no search of `assign`
-    const int few_tok = meta.few_tok;
-    const int count = meta.count;
-    const bool few = count <= kAvgFew;
-    int li = meta.li;
-    if (li >= avg_long_cap(d)) li = -1;                        // no scratch left: one CTA does it all
-    const int nparts = li >= 0 ? avg_parts(count) : 1;
-    const int e = meta.e;
-    const int lo = ev_lo[e] * N, hi = ev_lo[e + 1] * N;
-    const int nchunk = d / VN;
-    const int4* assign4 = reinterpret_cast<const int4*>(assign);
-    const uint32_t stage0 = (smem_u32(avg_dyn) + 127u) & ~127u;
-    constexpr int nst = NST;
-    constexpr uint32_t stage_stride = (uint32_t)(kAvgStages * kAvgStageBytes) / NST;   // a pass over a row moves no more
-    // the blocks to search, in order; a block is searched as bt/4 + 1 groups of four tokens (its
-    // first token need not start a group)
-    const unsigned long long blocks = meta.blocks;
-    const int nblk = __popcll(blocks);
-    const int bt = avg_block_tokens(hi - lo), qpb = bt / 4 + 1;
-    const int total_q = nblk * qpb;
-    // a part takes an equal share of the groups to search (not of the members): what it finds there
-    // it adds up, so an output's search is done once however many parts it has
-    const int q_per = (total_q + nparts - 1) / nparts;
-    const int q_begin = min(total_q, part * q_per), q_end = min(total_q, q_begin + q_per);
-    if (few) {
-        if (warp == 0) {                                       // into token order: rank = members before it
-            const int mine = lane < count ? few_tok : 0x7FFFFFFF;
-            int rank = 0;
-            for (int j = 0; j < count; ++j) rank += __shfl_sync(0xFFFFFFFFu, mine, j) < mine;
-            if (lane < count) s_list[rank] = mine;
+template <typename T>
+__device__ __forceinline__ void avg_store(T* out, const float* sum, float inv) {
+    constexpr int VN = 16 / sizeof(T);
+    alignas(16) T tmp[VN];
+#pragma unroll
+    for (int q = 0; q < VN; ++q) from_float(tmp[q], sum[q] * inv);
+    *reinterpret_cast<uint4*>(out) = *reinterpret_cast<const uint4*>(tmp);
+}
+
+// The four warps' sums of chunks [ch0, ch0 + nch), added in warp order: handed chunk by chunk to f(chunk, sum).  They
+// go through the rings' memory, into which no copy is in flight any more.
+template <typename T, int CH, typename F>
+__device__ __forceinline__ void avg_cta_sum(uint8_t* cta_mem, const float (&acc)[CH][16 / sizeof(T)], int nch, F f) {
+    constexpr int VN = 16 / sizeof(T), kPiece = CH * 32 * VN;   // floats per warp: at most kAvgRing bytes
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* sums = reinterpret_cast<float*>(cta_mem);
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < CH; ++u)
+#pragma unroll
+        for (int q = 0; q < VN; ++q) sums[warp * kPiece + (u * 32 + lane) * VN + q] = acc[u][q];
+    __syncthreads();
+    for (int i = threadIdx.x; i < nch; i += kAvgThreads) {
+        float t[VN];
+#pragma unroll
+        for (int q = 0; q < VN; ++q) {
+            t[q] = sums[i * VN + q];
+#pragma unroll
+            for (int w = 1; w < kAvgWarps; ++w) t[q] += sums[w * kPiece + i * VN + q];
         }
-    } else if (tid == 0) {
-        unsigned long long mm = blocks;
-        for (int i = 0; mm; ++i, mm &= mm - 1) s_blocks[i] = __ffsll((long long)mm) - 1;
+        f(i, t);
     }
     __syncthreads();
-    volatile int* abort_flag = &s_abort;
-    for (int cb = 0; cb < nchunk; cb += kAvgThreads * kAvgChunks) {
-        const uint32_t seg_bytes = (uint32_t)min(kAvgThreads * kAvgChunks, nchunk - cb) * 16u;
-        float acc[kAvgChunks][VN];
+}
+
+// Output c, all of whose `count` <= kAvgFew members are listed, by the whole CTA.
+template <typename T, int R>
+__device__ __forceinline__ void avg_heavy(AvgRing<R>& ring, const T* __restrict__ feats, T* __restrict__ out_feats, const AvgArgs& ar,
+                                          int c, int count, int seg, int* list, uint8_t* cta_mem) {
+    constexpr int VN = 16 / sizeof(T), CH = AvgRing<R>::kChunks;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ch0 = seg * ar.seg_chunks, nch = min(ar.seg_chunks, ar.d / VN - ch0);
+    // every thread ranks one member against all (they are read again and again from L1), every warp lists its quarter
+    static_assert(kAvgFew == kAvgThreads, "one member per thread");
+    const int32_t* few = ar.ml.few + (size_t)c * kAvgFew;
+    int* s_few = reinterpret_cast<int*>(cta_mem);            // no copy is in flight yet
+    if (threadIdx.x < count) s_few[threadIdx.x] = few[threadIdx.x];
+    __syncthreads();
+    const int share = (count + kAvgWarps - 1) / kAvgWarps, from = min(count, warp * share), n = min(count, from + share) - from;
+    for (int x = lane; x < count; x += 32) {
+        const int tok = s_few[x];
+        int rank = 0;
+#pragma unroll 8
+        for (int j = 0; j < count; ++j) rank += s_few[j] < tok;
+        if (rank >= from && rank < from + n) list[rank - from] = tok;
+    }
+    __syncthreads();
+    float acc[CH][VN] = {};
+    avg_add_rows<T, R>(ring, feats, ar, list, n, ch0, nch, acc);
+    const float inv = 1.0f / (float)count;
+    avg_cta_sum<T, CH>(cta_mem, acc, nch,
+                            [&](int i, const float* t) { avg_store<T>(out_feats + (size_t)c * ar.d + (size_t)(ch0 + i) * VN, t, inv); });
+    if (seg == 0 && threadIdx.x == 0) ar.out_members[c] = count;
+}
+
+// Part `part` of piece `seg` of output c with `count` > kAvgLong members, by the whole CTA; li: its place in the scratch of
+// the parts' sums, -1: none, one part.
+template <typename T, int R>
+__device__ __forceinline__ void avg_long(AvgRing<R>& ring, const T* __restrict__ feats, T* __restrict__ out_feats, const AvgArgs& ar,
+                                         int c, int count, int part, int nparts, int li, int seg, int* list, uint8_t* cta_mem,
+                                         unsigned char* s_block, int* s_last) {
+    constexpr int VN = 16 / sizeof(T), CH = AvgRing<R>::kChunks;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int e = ar.out_event[c];
+    const unsigned long long blocks = ar.ml.blocks[c];
+    const int lo = ar.ev_lo[e] * ar.N, hi = ar.ev_lo[e + 1] * ar.N;
+    const int ch0 = seg * ar.seg_chunks, nch = min(ar.seg_chunks, ar.d / VN - ch0);
+    if (tid < 64 && ((blocks >> tid) & 1ull)) s_block[__popcll(blocks & ((1ull << tid) - 1ull))] = (unsigned char)tid;
+    __syncthreads();
+    // the search runs over the flagged blocks' groups of four tokens (a block's first token need not start a group)
+    const int bt = avg_block_tokens(hi - lo), qpb = bt / 4 + 1, total_q = __popcll(blocks) * qpb;
+    const int share = (total_q + nparts * kAvgWarps - 1) / (nparts * kAvgWarps);
+    const int q_begin = min(total_q, (part * kAvgWarps + warp) * share), q_end = min(total_q, q_begin + share);
+    const int4* assign4 = reinterpret_cast<const int4*>(ar.assign);
+    float acc[CH][VN] = {};
+    int n = 0;                                               // members listed and not yet added
+    for (int q0 = q_begin; q0 < q_end; q0 += 128) {
+        unsigned match[4];                                   // of four rounds of 32 groups; bit i: token i of the lane's group is a member
+        int first[4];
+        int4 a[4];
+        int j_lo[4], j_hi[4];
 #pragma unroll
-        for (int u = 0; u < kAvgChunks; ++u) Vec16<T>::zero(acc[u]);
-        // the listed members' rows, nst in flight, added in list order
-        auto consume = [&](int nlist) {
-        // a ring: row m goes to stage m % nst; the stage is refilled with row m + nst as
-        // soon as every thread has added row m, so nst rows stay in flight until the list ends
-        auto issue = [&](int m) {
-            const int j = m % nst;                             // nst is a constant: no division
-            const uint32_t bar = smem_u32(&s_bar[j]);
-            mbar_arrive_expect_tx(bar, seg_bytes);
-            const long long src_row = dbg_bound(s_list[m], Nv, status);
-            if (!(dbg_withhold(status, kDbgMergeAvg) && blockIdx.x == (unsigned)kAvgFrontCtas && m == 0 && cb == 0))   // debug builds: one copy never sent
-                bulk_load(stage0 + (uint32_t)j * stage_stride, feats + (size_t)src_row * d + (size_t)cb * VN, seg_bytes, bar);
-        };
-        if (tid == 0)
-            for (int m = 0; m < nlist && m < nst; ++m) issue(m);
-        for (int m = 0; m < nlist; ++m) {
-            const int j = m % nst;
-            const bool ok = mbar_wait(smem_u32(&s_bar[j]), (phase >> j) & 1u, abort_flag);
-            phase ^= 1u << j;
-            if (ok) {
-                const uint8_t* row = avg_dyn + (stage0 - smem_u32(avg_dyn)) + (size_t)j * stage_stride;
-#pragma unroll
-                for (int u = 0; u < kAvgChunks; ++u) {
-                    const int ch = cb + u * kAvgThreads + tid;
-                    if (ch < nchunk) {
-                        const uint4 raw = *reinterpret_cast<const uint4*>(row + (size_t)(u * kAvgThreads + tid) * 16);
-                        float v[VN];
-                        if constexpr (sizeof(T) == 4) {
-                            v[0] = __uint_as_float(raw.x); v[1] = __uint_as_float(raw.y);
-                            v[2] = __uint_as_float(raw.z); v[3] = __uint_as_float(raw.w);
-                        } else {
-                            const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                v[2 * i]     = __uint_as_float(w4[i] << 16);
-                                v[2 * i + 1] = __uint_as_float(w4[i] & 0xFFFF0000u);
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < VN; ++q) acc[u][q] += v[q];
-                    }
+        for (int x = 0; x < 4; ++x) {
+            const int qf = q0 + x * 32 + lane;
+            a[x] = make_int4(-1, -1, -1, -1);
+            first[x] = j_lo[x] = j_hi[x] = 0;
+            if (qf < q_end) {
+                const int bi = qf / qpb;
+                j_lo[x] = lo + (int)s_block[bi] * bt;
+                j_hi[x] = min(j_lo[x] + bt, hi);
+                const int q = (j_lo[x] >> 2) + (qf - bi * qpb);
+                first[x] = q * 4;
+                if (q * 4 + 3 < ar.Nv) {
+                    a[x] = assign4[q];
+                } else {                                     // the array ends inside this group
+                    if (q * 4 + 0 < ar.Nv) a[x].x = ar.assign[q * 4 + 0];
+                    if (q * 4 + 1 < ar.Nv) a[x].y = ar.assign[q * 4 + 1];
+                    if (q * 4 + 2 < ar.Nv) a[x].z = ar.assign[q * 4 + 2];
                 }
             }
-            __syncthreads();                                   // every thread is done with stage j
-            if (tid == 0 && m + nst < nlist && !*abort_flag) issue(m + nst);
         }
-        };
-        if (few) {
-            consume(count);                                    // s_list holds them already
-        } else {
-        // a thread's run is qpt consecutive groups: as few as cover the search in one pass
-        const int qpt = max(1, min(kAvgQuads, (q_end - q_begin + kAvgThreads - 1) / kAvgThreads));
-        for (int qs = q_begin; qs < q_end; qs += kAvgThreads * qpt) {
-            int4 a[kAvgQuads];
-            int qidx[kAvgQuads], j_lo[kAvgQuads], j_hi[kAvgQuads];   // group index; the block's token range
 #pragma unroll
-            for (int u = 0; u < kAvgQuads; ++u) {
-                const int qf = qs + tid * qpt + u;
-                a[u] = make_int4(-1, -1, -1, -1);
-                qidx[u] = 0; j_lo[u] = 0; j_hi[u] = 0;
-                if (u < qpt && qf < q_end) {
-                    const int bi = qf / qpb, wq = qf - bi * qpb;
-                    const int st = lo + s_blocks[bi] * bt;
-                    const int q = (st >> 2) + wq;
-                    qidx[u] = q; j_lo[u] = st; j_hi[u] = min(st + bt, hi);
-                    if (q * 4 + 3 < Nv) {
-                        a[u] = assign4[q];
-                    } else {                                   // the array ends inside this group
-                        if (q * 4 + 0 < Nv) a[u].x = assign[q * 4 + 0];
-                        if (q * 4 + 1 < Nv) a[u].y = assign[q * 4 + 1];
-                        if (q * 4 + 2 < Nv) a[u].z = assign[q * 4 + 2];
-                    }
-                }
-            }
-            unsigned match = 0;                                // bit 4u+i: token 4*qidx[u]+i belongs to output c
+        for (int x = 0; x < 4; ++x) {
+            const int j = first[x];
+            match[x] = (unsigned)(a[x].x == c && j + 0 >= j_lo[x] && j + 0 < j_hi[x]) << 0 |
+                       (unsigned)(a[x].y == c && j + 1 >= j_lo[x] && j + 1 < j_hi[x]) << 1 |
+                       (unsigned)(a[x].z == c && j + 2 >= j_lo[x] && j + 2 < j_hi[x]) << 2 |
+                       (unsigned)(a[x].w == c && j + 3 >= j_lo[x] && j + 3 < j_hi[x]) << 3;
+        }
 #pragma unroll
-            for (int u = 0; u < kAvgQuads; ++u) {
-                if (u >= qpt) break;
-                const int j = qidx[u] * 4;
-                match |= (unsigned)(a[u].x == c && j + 0 >= j_lo[u] && j + 0 < j_hi[u]) << (4 * u + 0);
-                match |= (unsigned)(a[u].y == c && j + 1 >= j_lo[u] && j + 1 < j_hi[u]) << (4 * u + 1);
-                match |= (unsigned)(a[u].z == c && j + 2 >= j_lo[u] && j + 2 < j_hi[u]) << (4 * u + 2);
-                match |= (unsigned)(a[u].w == c && j + 3 >= j_lo[u] && j + 3 < j_hi[u]) << (4 * u + 3);
-            }
-            const int mine = __popc(match);
+        for (int x = 0; x < 4; ++x) {
+            const int mine = __popc(match[x]);
             int incl = mine;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
                 if (lane >= o) incl += v;
             }
-            if (lane == 31) s_wtot[warp] = incl;
-            __syncthreads();
-            int before = incl - mine, total = 0;               // rank of this thread's first member in the pass
+            int r = n + incl - mine;
 #pragma unroll
-            for (int w = 0; w < kAvgThreads / 32; ++w) {
-                const int v = s_wtot[w];
-                if (w < warp) before += v;
-                total += v;
-            }
-            // the members of the pass, listed kAvgList at a time
-            for (int b0 = 0; b0 < total; b0 += kAvgList) {
-                const int nlist = min(kAvgList, total - b0);
-                {
-                    unsigned mm = match;
-                    int r = before;
-                    while (mm) {
-                        const int b = __ffs(mm) - 1;
-                        mm &= mm - 1;
-                        if (r >= b0 && r < b0 + nlist) s_list[r - b0] = qidx[b >> 2] * 4 + (b & 3);
-                        ++r;
-                    }
-                }
-                __syncthreads();
-                consume(nlist);
-            }
-            __syncthreads();                                   // s_wtot and s_list are reused by the next pass
-        }
-        }
-        if (nparts == 1) {
-            const float inv = 1.0f / (float)count;
-#pragma unroll
-            for (int u = 0; u < kAvgChunks; ++u) {
-                const int ch = cb + u * kAvgThreads + tid;
-                if (ch < nchunk) {
-                    T* o = out_feats + (size_t)c * d + (size_t)ch * VN;
-                    alignas(16) T tmp[VN];
-#pragma unroll
-                    for (int q = 0; q < VN; ++q) from_float(tmp[q], acc[u][q] * inv);
-                    *reinterpret_cast<uint4*>(o) = *reinterpret_cast<const uint4*>(tmp);
-                }
-            }
-        } else {
-            float* ps = long_sums + ((size_t)li * kAvgParts + part) * d;
-#pragma unroll
-            for (int u = 0; u < kAvgChunks; ++u) {
-                const int ch = cb + u * kAvgThreads + tid;
-                if (ch < nchunk) {
-#pragma unroll
-                    for (int q = 0; q < VN; ++q) ps[(size_t)ch * VN + q] = acc[u][q];
-                }
+            for (int i = 0; i < 4; ++i)
+                if ((match[x] >> i) & 1u) list[r++] = first[x] + i;
+            n += __shfl_sync(0xFFFFFFFFu, incl, 31);
+            __syncwarp();
+            if (n > kAvgList - 128) {                        // the next round might not fit
+                avg_add_rows<T, R>(ring, feats, ar, list, n, ch0, nch, acc);
+                n = 0;
             }
         }
     }
-    if (part == 0 && tid == 0) out_members[c] = count;
-    if (tid == 0 && s_abort) *status = METOK_ERR_TIMEOUT;
-    if (nparts > 1) {
-        // the last part to finish adds the partial sums in part order
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) s_last = atomicAdd(&long_done[li], 1) == nparts - 1;
-        __syncthreads();
-        if (s_last) {
-            __threadfence();
-            const float inv = 1.0f / (float)count;
-            const float* ps = long_sums + (size_t)li * kAvgParts * d;
-            // four elements per thread and trip, the parts' loads all in flight, added in part order
-            // (d is a multiple of 4: rows are whole 16-byte chunks)
-            for (int i = tid * 4; i < d; i += kAvgThreads * 4) {
-                float4 v[kAvgParts];
-#pragma unroll
-                for (int q = 0; q < kAvgParts; ++q)
-                    v[q] = q < nparts ? __ldcg(reinterpret_cast<const float4*>(ps + (size_t)q * d + i))
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
-                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int q = 0; q < kAvgParts; ++q) {
-                    if (q < nparts) { a.x += v[q].x; a.y += v[q].y; a.z += v[q].z; a.w += v[q].w; }
-                }
-                T* o = out_feats + (size_t)c * d + i;
-                from_float(o[0], a.x * inv); from_float(o[1], a.y * inv);
-                from_float(o[2], a.z * inv); from_float(o[3], a.w * inv);
-            }
-        }
-    }
-}
-
-template <typename T, int NST>
-__global__ void __launch_bounds__(kAvgThreads, 8)
-merge_avg_kernel(const T* __restrict__ feats, int d, int N, int Nv, const int32_t* __restrict__ ev_lo,
-                 const int32_t* __restrict__ out_event, const int32_t* __restrict__ assign,
-                 const unsigned long long* __restrict__ slot_blocks, const int32_t* __restrict__ slot_cnt,
-                 const int32_t* __restrict__ long_index, const int32_t* __restrict__ long_slot,
-                 const int32_t* __restrict__ long_counter, const int32_t* __restrict__ few_members,
-                 const int32_t* __restrict__ heavy_index, const int32_t* __restrict__ heavy_slot,
-                 const int32_t* __restrict__ heavy_counter,
-                 float* __restrict__ long_sums, int32_t* __restrict__ long_done, int front_ctas, const int32_t* __restrict__ n_out,
-                 T* __restrict__ out_feats, int32_t* __restrict__ out_members, int32_t* __restrict__ status) {
-    grid_dep_wait();
-    using namespace sm100;
-    extern __shared__ uint8_t avg_dyn[];
-    __shared__ __align__(8) uint64_t s_bar[NST];
-    __shared__ int s_list[kAvgList];
-    __shared__ int s_wtot[kAvgThreads / 32];
-    __shared__ int s_blocks[64];
-    __shared__ int s_abort, s_last;
-    // A CTA adds the rows of its output about three at a time, one memory latency per three rows:
-    // an output with many members lasts many times longer than the usual one, and would set the
-    // kernel's time if it started late.  So merge_decode lists every output with more than kAvgHeavy
-    // members, and the first front_ctas CTAs of the grid take the listed work round-robin, before the
-    // other outputs' CTAs start: the outputs with more than kAvgLong members part by part (up to
-    // kAvgParts parts, each an equal share of the blocks to search, partial sums combined in part
-    // order by the last part to finish), the others whole (their members are listed: no search).
-    // A listed output's own CTA leaves at once.  The other CTAs start
-    // in index order and take the outputs from the last one down, so that this pass begins with the
-    // rows of V that the preceding (ascending) pass left in L2.
-    const int tid = threadIdx.x;
-    const int long_cap = avg_long_cap(d);
-    if (tid == 32) {                                           // not thread 0: it is busy with the block list below
-        for (int j = 0; j < NST; ++j) mbar_init(smem_u32(&s_bar[j]), 1);
-        s_abort = 0;
-        mbar_fence_init();
-    }
-    uint32_t phase = 0;                                        // bit j: parity of the next completion of barrier j
-#define METOK_AVG_ITEM(C, PART, META)                                                                                     \
-    merge_avg_item<T, NST>(C, PART, META, phase, avg_dyn, s_bar, s_list, s_wtot, s_blocks, &s_abort, &s_last, feats, d, N, Nv,  \
-                      ev_lo, out_event, assign, slot_blocks, slot_cnt, long_index, few_members, long_sums, long_done,  \
-                      out_feats, out_members, status)
-    if ((int)blockIdx.x >= front_ctas) {
-        const int c = *n_out - 1 - ((int)blockIdx.x - front_ctas);
-        if (c < 0) return;
-        // everything about output c in one round trip: whether it is listed, and what its own CTA needs if not
-        const int hh = heavy_index[c];
-        const AvgMeta meta = avg_meta(c, slot_cnt, few_members, long_index, out_event, slot_blocks);
-        if ((hh >= 0 && hh < kAvgHeavyCap) || (meta.li >= 0 && meta.li < long_cap)) return;   // listed: the front CTAs have it
-        METOK_AVG_ITEM(c, 0, meta);
+    avg_add_rows<T, R>(ring, feats, ar, list, n, ch0, nch, acc);
+    const float inv = 1.0f / (float)count;
+    if (seg == 0 && part == 0 && tid == 0) ar.out_members[c] = count;
+    if (nparts == 1) {
+        avg_cta_sum<T, CH>(cta_mem, acc, nch,
+                                [&](int i, const float* t) { avg_store<T>(out_feats + (size_t)c * ar.d + (size_t)(ch0 + i) * VN, t, inv); });
         return;
     }
-    const int n_long = min(*long_counter, long_cap), n_heavy = min(*heavy_counter, kAvgHeavyCap);
-    const int n_items = n_long * kAvgParts + n_heavy;
-    for (int it = (int)blockIdx.x; it < n_items; it += front_ctas) {
-        int c, part;
-        if (it < n_long * kAvgParts) {
-            c = long_slot[it / kAvgParts];
-            part = it % kAvgParts;
-            if (part >= avg_parts(slot_cnt[c])) continue;
-        } else {
-            c = heavy_slot[it - n_long * kAvgParts];
-            part = 0;
-            const int li = long_index[c];
-            if (li >= 0 && li < long_cap) continue;            // split into parts: taken above
+    float* sums = ar.long_sums + (size_t)li * kAvgParts * ar.d + (size_t)ch0 * VN;
+    avg_cta_sum<T, CH>(cta_mem, acc, nch, [&](int i, const float* t) {
+#pragma unroll
+        for (int q = 0; q < VN; q += 4)
+            *reinterpret_cast<float4*>(sums + (size_t)part * ar.d + i * VN + q) = make_float4(t[q], t[q + 1], t[q + 2], t[q + 3]);
+    });
+    // the last part to finish adds the parts' sums in part order
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) *s_last = atomicAdd(&ar.long_done[li * ar.nseg + seg], 1) == nparts - 1;
+    __syncthreads();
+    if (*s_last) {
+        __threadfence();
+        for (int i = tid; i < nch; i += kAvgThreads) {
+            float t[VN];
+#pragma unroll
+            for (int q = 0; q < VN; q += 4) {
+                float4 v[kAvgParts];
+#pragma unroll
+                for (int x = 0; x < kAvgParts; ++x)
+                    v[x] = x < nparts ? __ldcg(reinterpret_cast<const float4*>(sums + (size_t)x * ar.d + i * VN + q))
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+                float4 sum = v[0];
+#pragma unroll
+                for (int x = 1; x < kAvgParts; ++x) {
+                    if (x < nparts) { sum.x += v[x].x; sum.y += v[x].y; sum.z += v[x].z; sum.w += v[x].w; }
+                }
+                t[q] = sum.x; t[q + 1] = sum.y; t[q + 2] = sum.z; t[q + 3] = sum.w;
+            }
+            avg_store<T>(out_feats + (size_t)c * ar.d + (size_t)(ch0 + i) * VN, t, inv);
         }
-        const AvgMeta meta = avg_meta(c, slot_cnt, few_members, long_index, out_event, slot_blocks);
-        METOK_AVG_ITEM(c, part, meta);
-        __syncthreads();                                       // the shared lists are reused by the next item
     }
-#undef METOK_AVG_ITEM
+    __syncthreads();
+}
+
+template <typename T, int R>
+__global__ void __launch_bounds__(kAvgThreads, kAvgCtasPerSm)
+merge_avg_kernel(const T* __restrict__ feats, T* __restrict__ out_feats, AvgArgs ar) {
+    grid_dep_wait();
+    using namespace sm100;
+    constexpr int VN = 16 / sizeof(T), CH = AvgRing<R>::kChunks;
+    extern __shared__ uint8_t avg_dyn[];
+    __shared__ __align__(8) uint64_t s_bar[kAvgWarps][R];
+    __shared__ AvgPiece s_piece[kAvgWarps][kAvgQueue];
+    __shared__ int s_list[kAvgWarps][kAvgList];
+    __shared__ int s_abort, s_last, s_next;
+    __shared__ unsigned char s_block[64];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint8_t* cta_mem = avg_dyn + ((128u - (smem_u32(avg_dyn) & 127u)) & 127u);
+    AvgRing<R> ring;
+    ring.mem = cta_mem + warp * kAvgRing;
+    ring.mem_u32 = smem_u32(ring.mem);
+    ring.bar_u32 = smem_u32(&s_bar[warp][0]);
+    ring.phase = 0u;
+    ring.abort_flag = &s_abort;
+    if (lane == 0) {
+        for (int j = 0; j < R; ++j) mbar_init(ring.bar_u32 + 8u * j, 32);
+        if (warp == 0) s_abort = 0;
+        mbar_fence_init();
+    }
+    __syncthreads();
+    const int n_out = *ar.n_out, n_long = *ar.ml.long_counter, n_heavy = *ar.ml.heavy_counter;
+    // the outputs with many members, a CTA per item: (part, output, piece), then (output, piece)
+    const int per_part = n_long * ar.nseg, n_split = per_part * kAvgParts, n_items = n_split + n_heavy * ar.nseg;
+    bool stop = false;                                       // a wait has given up: the same for the whole CTA
+    for (int it = (int)blockIdx.x; it < n_items && !stop;) {
+        if (tid == 0) s_next = n_items > (int)gridDim.x ? (int)gridDim.x + atomicAdd(ar.next_item, 1) : n_items;
+        if (it < n_split) {
+            const int part = it / per_part, sub = it - part * per_part, back = sub / n_long, li = sub - back * n_long;
+            const int c = ar.ml.long_slot[li], count = ar.ml.count[c];
+            const bool scratch = li < avg_long_cap(ar.d);
+            const int nparts = scratch ? avg_parts(count) : 1;
+            if (part < nparts)
+                avg_long<T, R>(ring, feats, out_feats, ar, c, count, part, nparts, scratch ? li : -1, ar.nseg - 1 - back, s_list[warp],
+                                 cta_mem, s_block, &s_last);
+        } else {
+            const int x = it - n_split, back = x / n_heavy, h = x - back * n_heavy;
+            const int c = ar.ml.heavy_slot[h], count = ar.ml.count[c];
+            if (count <= kAvgLong) avg_heavy<T, R>(ring, feats, out_feats, ar, c, count, ar.nseg - 1 - back, s_list[warp], cta_mem);
+        }
+        __syncthreads();
+        it = s_next;
+        stop = s_abort != 0;                                 // nobody waits for copies between these two barriers
+        __syncthreads();
+    }
+    // The others, a warp per piece: the last piece of every row first, then the one before it and so on (see above), from
+    // the last output down.  A stream of rows that runs on from piece to piece: R of them are on their way while one is added, whichever
+    // piece they belong to; the list of the piece after the one being issued has been fetched, and the number of the
+    // one after that.  Pieces being issued or added stand in a queue in shared memory.
+    const int total = n_out * ar.nseg, nchunk = ar.d / VN;
+    AvgPiece* queue = s_piece[warp];
+    int a_out = 0, a_seg = 0, a_n = -1, a_tok = 0;           // the piece ahead: n = 0: taken elsewhere, -1: no more pieces
+    auto fetch = [&](int t) {
+        a_n = -1;
+        if (t < total) {
+            const int back = t / n_out;
+            a_seg = ar.nseg - 1 - back;
+            a_out = n_out - 1 - (t - back * n_out);
+            a_tok = lane < kAvgHeavy ? ar.ml.few[(size_t)a_out * kAvgFew + lane] : 0;
+            a_n = ar.ml.count[a_out];
+            if (a_n > kAvgHeavy) a_n = 0;
+        }
+    };
+    // A warp's first two pieces are fixed: all warps at one counter at once would stand in line for 5 us.
+    const int warps = (int)gridDim.x * kAvgWarps, me = (int)blockIdx.x * kAvgWarps + warp;
+    auto take = [&]() { return lane == 0 ? 2 * warps + atomicAdd(ar.next, 1) : 0; };
+    fetch(me);
+    int ticket = me + warps;
+    bool withhold = dbg_withhold(ar.status, kDbgMergeAvg);   // debug builds: of every warp's first row
+    int i_piece = -1, i_n = 0, i_at = 0, i_ch0 = 0, i_nch = 0;   // issued: rows [0, i_at) of piece i_piece of the stream
+    auto issue_next = [&](int st) {                          // the next row of the stream; false: there is none
+        if (i_at == i_n) {
+            while (a_n == 0) {
+                fetch(__shfl_sync(0xFFFFFFFFu, ticket, 0));
+                ticket = take();
+            }
+            if (a_n < 0) return false;
+            // the members into token order: rank = members before it
+            AvgPiece& q = queue[++i_piece & (kAvgQueue - 1)];
+            const int key = lane < a_n ? a_tok : 0x7FFFFFFF;
+            int rank = 0;
+            for (int j = 0; j < a_n; j += 4) {               // four at a time: lanes past the list hold the largest integer
+#pragma unroll
+                for (int x = 0; x < 4; ++x) rank += __shfl_sync(0xFFFFFFFFu, key, j + x) < key;
+            }
+            if (lane < a_n) q.row[rank] = key;
+            if (lane == 0) { q.out = a_out; q.seg = a_seg; q.n = a_n; }
+            __syncwarp();
+            i_n = a_n;
+            i_at = 0;
+            i_ch0 = a_seg * ar.seg_chunks;
+            i_nch = min(ar.seg_chunks, nchunk - i_ch0);
+            fetch(__shfl_sync(0xFFFFFFFFu, ticket, 0));
+            ticket = take();
+        }
+        avg_issue<T, R>(ring, st, feats, ar, queue[i_piece & (kAvgQueue - 1)].row[i_at], i_ch0, i_nch, withhold);
+        withhold = false;
+        ++i_at;
+        return true;
+    };
+    int flying = 0;
+    if (!stop)
+        for (int m = 0; m < R; ++m) flying += issue_next(m) ? 1 : 0;
+    int st = 0;
+    for (int piece = 0; flying > 0; ++piece) {
+        const AvgPiece& q = queue[piece & (kAvgQueue - 1)];
+        const int out = q.out, seg = q.seg, n = q.n, ch0 = seg * ar.seg_chunks, nch = min(ar.seg_chunks, nchunk - ch0);
+        float acc[CH][VN] = {};
+        bool ok = true;                                      // the same for the whole warp
+        for (int m = 0; m < n && ok; ++m) {
+            ok = avg_take<T, R>(ring, st, acc);
+            if (ok && !issue_next(st)) --flying;
+            st = st + 1 == R ? 0 : st + 1;
+        }
+        if (!ok) break;
+        const float inv = 1.0f / (float)n;
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+            const int ch = u * 32 + lane;
+            if (ch < nch) avg_store<T>(out_feats + (size_t)out * ar.d + (size_t)(ch0 + ch) * VN, acc[u], inv);
+        }
+        if (seg == 0 && lane == 0) ar.out_members[out] = n;
+    }
+    cp_async_wait_all();                                     // nothing may land after the CTA's shared memory is gone
+    if (lane == 0 && s_abort) *ar.status = METOK_ERR_TIMEOUT;
 }
 
 // --------------------------------------------------------------------------- //
@@ -1303,31 +1419,21 @@ merge_avg_kernel(const T* __restrict__ feats, int d, int N, int Nv, const int32_
 struct VisionWs {
     int32_t* status;          // device status word, first in the workspace
     float* inv_norm;
-    uint8_t* is_key;
-    int32_t* rest;            // per event, from its first token's place on: its tokens that are no key token
     int32_t *ev_lo, *ev_budget, *ev_out_off, *ev_unit_off;
     int32_t *frame_ev, *frame_stride, *frame_off;   // POOL mode
-    unsigned long long* best64;   // packed argmax per token (merging modes)
-    unsigned long long* slot_blocks;   // per output token: which blocks of its event hold a member
-    int32_t* slot_cnt;                 // per output token: members
-    int32_t* long_counter;             // outputs with more than kAvgLong members ...
-    int32_t* long_done;                // ... parts of each that have finished
-    int32_t* long_index;               // output -> index among the long ones, -1 otherwise
-    int32_t* long_slot;                // and back
-    int32_t* heavy_counter;            // outputs with more than kAvgHeavy members ...
-    int32_t* heavy_index;              // ... output -> index among them, -1 otherwise (directly after long_index)
-    int32_t* heavy_slot;               // ... and back
-    int32_t* few_members;              // per output token: its first kAvgFew members, in arrival order
-    float* long_sums;                  // partial sums of their parts
-    size_t zero_bytes;                 // slot_blocks .. long_done are cleared together
+    uint8_t* is_key;          // the rest: merging modes (TokenOut, MemberLists, AvgArgs)
+    int32_t *rest, *tile_done;
+    unsigned long long* best64;
+    MemberLists ml;
+    float* long_sums;
+    int32_t *long_done, *avg_next;
+    int n_counters;           // the counters are cleared together: long, heavy, avg_next and long_done
 };
 
 static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, bool merging) {
-    VisionWs w;
+    VisionWs w = {};
     w.status = cv.take<int32_t>(64);
     w.inv_norm = cv.take<float>((size_t)Tn * N);
-    w.is_key = cv.take<uint8_t>((size_t)Tn * N);
-    w.rest = merging ? cv.take<int32_t>((size_t)Tn * N) : nullptr;
     w.ev_lo = cv.take<int32_t>((size_t)k + 1);
     w.ev_budget = cv.take<int32_t>((size_t)k + 1);
     w.ev_out_off = cv.take<int32_t>((size_t)k + 1);
@@ -1335,24 +1441,53 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
     w.frame_ev = cv.take<int32_t>((size_t)Tn);
     w.frame_stride = cv.take<int32_t>((size_t)Tn);
     w.frame_off = cv.take<int32_t>((size_t)Tn + 1);
-    w.best64 = merging ? cv.take<unsigned long long>((size_t)Tn * N) : nullptr;
-    {
+    if (merging) {
         const size_t n = (size_t)cap + 64;
-        w.zero_bytes = n * 8 + n * 4 + (size_t)(64 + kAvgLongCapMax + 64) * 4;
-        unsigned char* z = cv.take<unsigned char>(w.zero_bytes);
-        w.slot_blocks = reinterpret_cast<unsigned long long*>(z);
-        w.slot_cnt = reinterpret_cast<int32_t*>(z + n * 8);
-        w.long_counter = w.slot_cnt + n;
-        w.long_done = w.long_counter + 64;
-        w.heavy_counter = w.long_done + kAvgLongCapMax;
-        w.long_index = cv.take<int32_t>(2 * n);         // long_index, then heavy_index: filled with -1 together
-        w.heavy_index = w.long_index + n;
-        w.heavy_slot = cv.take<int32_t>(kAvgHeavyCap);
-        w.long_slot = cv.take<int32_t>(kAvgLongCapMax);
-        w.few_members = cv.take<int32_t>(n * kAvgFew);
+        w.is_key = cv.take<uint8_t>((size_t)Tn * N);
+        w.rest = cv.take<int32_t>((size_t)Tn * N);
+        w.tile_done = cv.take<int32_t>((size_t)Tn * N);
+        w.best64 = cv.take<unsigned long long>((size_t)Tn * N);
+        w.ml.blocks = cv.take<unsigned long long>(n);
+        w.ml.count = cv.take<int32_t>(n);
+        w.ml.few = cv.take<int32_t>(n * kAvgFew);
+        w.ml.heavy_slot = cv.take<int32_t>(n);
+        w.ml.long_slot = cv.take<int32_t>(n);
+        w.n_counters = 4 + avg_long_cap(d) * avg_max_pieces(d);
+        w.ml.long_counter = cv.take<int32_t>((size_t)w.n_counters);
+        w.ml.heavy_counter = w.ml.long_counter + 1;
+        w.avg_next = w.ml.long_counter + 2;              // two: items, pieces
+        w.long_done = w.ml.long_counter + 4;
         w.long_sums = cv.take<float>((size_t)avg_long_cap(d) * kAvgParts * d);
     }
     return w;
+}
+
+// The shape of a merge unit.  An SM is fed about 118 KB per us from L2 and a tensor instruction of 128 x bn x 16 takes
+// bn * 0.27 ns (at least 24 ns), so large units do more per byte (256 x 256: 0.56 us per K block of 64 for 64 KB) --
+// but a launch lasts as long as the SM with the most of them, and with few events small units spread better: 32 frames
+// of 144 tokens in four events are 40 units of 256 x 173 or 76 of 128 x 173.  The shape with the
+// shortest estimated launch is taken, from the mean event; 1.5 us per unit for its start and its argmax.
+static MmaTile choose_mma_tile(int Nv, int k, int d, double keep) {
+    static const struct { int bm, bn; } shapes[] = {{256, 256}, {256, 128}, {128, 256}, {128, 128}, {128, 64}};
+    const int m = ceil_div(Nv, k), keys = std::max(1, (int)(keep * m)), ksteps = ceil_div(d, kMmaBK);
+    MmaTile best = {};
+    double best_us = 0.0;
+    for (const auto& s : shapes) {
+        const int chunks = ceil_div(keys, s.bn), cols = (ceil_div(keys, chunks) + 15) & ~15;
+        // events differ in length, and long ones have more row tiles and more chunks: half as many chunks again as the mean
+        const double units = k == 1 ? (double)ceil_div(Nv, s.bm) * chunks : ((double)Nv / s.bm + 0.5 * k) * (1.5 * keys / s.bn + 0.5);
+        const double fill = (s.bm + cols) * kMmaBK * 2 / 118e3, mma = (s.bm / 128) * 4 * std::max(0.024, cols * 0.272e-3);
+        const double us = std::ceil(units / kNumSMs) * (ksteps * std::max(fill, mma) + 1.5);
+        if (best.bm == 0 || us < 0.97 * best_us) {                  // the larger one unless it is clearly slower
+            best_us = us;
+            best.bm = s.bm;
+            best.bn = s.bn;
+        }
+    }
+    best.a_bytes = (uint32_t)best.bm * kMmaBK * 2;
+    best.stage_bytes = best.a_bytes + (uint32_t)best.bn * kMmaBK * 2;
+    best.stages = std::min<int>(kMmaMaxStages, kMmaRingBytes / best.stage_bytes);
+    return best;
 }
 
 // The tensor-core merge path needs bf16 rows that TMA can address (16-byte row pitch);
@@ -1394,11 +1529,12 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         }
         METOK_LAUNCH_CHECK();
     }
+    const MmaTile tile = choose_mma_tile(Nv, k, d, p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey);
     PlanParams pp;
     pp.Tn = Tn; pp.N = N; pp.k = k;
     pp.n_key_events = min(k, ceilq(p->alpha * (double)k));
-    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? kMmaBM : kSaTile;
-    pp.chunk_cols = mma ? kMmaBN : kSaTile;
+    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? tile.bm : kSaTile;
+    pp.chunk_cols = mma ? tile.bn : kSaTile;
     pp.rows_with_keys = mma ? 1 : 0;
     pp.keep_key = p->keep_key; pp.keep_nonkey = p->keep_nonkey; pp.beta = p->beta;
     pp.key_given = p->key_events_given;
@@ -1409,21 +1545,11 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     const size_t plan_smem = (size_t)(k + Tn) * sizeof(float) + (size_t)k * (3 * sizeof(int) + 1);
     if (plan_smem > 40 * 1024)
         METOK_ALLOW_SMEM(event_plan_kernel, plan_smem);
-    PlanClears clr;
-    const bool merging = p->mode == METOK_MODE_TOPK_MERGE;
-    clr.zero_a = merging ? w.best64 : nullptr;
-    clr.zero_a_bytes = (size_t)Nv * sizeof(unsigned long long);
-    clr.zero_b = merging ? w.slot_blocks : nullptr;
-    clr.zero_b_bytes = w.zero_bytes;
-    clr.ones = merging ? w.long_index : nullptr;
-    clr.ones_bytes = 2 * ((size_t)cap + 64) * sizeof(int32_t);
-    clr.status = w.status;
     {
         METOK_TIMED("event_plan_kernel", st);
-        launch_chained(event_plan_kernel, dim3(1 + kPlanFillCtas), dim3(1024), plan_smem, st, token_score, frame_score, event_offsets, pp, event_score,
-                                                                  event_is_key, w.ev_lo, w.ev_budget, w.ev_out_off,
-                                                                  w.ev_unit_off, w.frame_ev,
-                                                                  w.frame_stride, w.frame_off, n_out, clr);
+        launch_chained(event_plan_kernel, dim3(1), dim3(1024), plan_smem, st, token_score, frame_score, event_offsets, pp, event_score,
+                       event_is_key, w.ev_lo, w.ev_budget, w.ev_out_off, w.ev_unit_off, w.frame_ev, w.frame_stride, w.frame_off,
+                       n_out, w.ml.long_counter, w.n_counters, w.status);
     }
     METOK_LAUNCH_CHECK();
 
@@ -1438,6 +1564,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         return METOK_OK;
     }
 
+    const TokenOut to = {w.is_key, out_src, out_event, assign, w.rest, w.best64, w.tile_done, w.ml};
     {
         // an event has at most Tn - (k - 1) frames
         const long long longest = (long long)(Tn - (k - 1)) * N;
@@ -1447,7 +1574,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
             METOK_TIMED("event_topk_kernel", st);
             auto launch = [&](auto kernel, int C, int threads) {
                 launch_chained_clusters(C, kernel, dim3(k * C), dim3(threads), lay.bytes, st, token_score, w.ev_lo, N, w.ev_budget,
-                                        w.ev_out_off, lay, w.is_key, out_src, out_event, assign, w.rest);
+                                        w.ev_out_off, lay, to);
             };
             // One CTA per event where that holds the longest one there can be.  Clusters, most of which come down to
             // their first CTA, cost nothing while all of them are resident at once; with more events (61 of them: 488
@@ -1464,7 +1591,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
                 METOK_ALLOW_SMEM(event_topk_kernel, lay.bytes);
             METOK_TIMED("event_topk_kernel", st);
             event_topk_kernel<<<k * kSelCluster, nthreads, lay.bytes, st>>>(
-                token_score, w.ev_lo, N, w.ev_budget, w.ev_out_off, lay, w.is_key, out_src, out_event, assign, w.rest);
+                token_score, w.ev_lo, N, w.ev_budget, w.ev_out_off, lay, to);
         }
         METOK_LAUNCH_CHECK();
     }
@@ -1479,44 +1606,48 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         {
             METOK_TIMED("merge_assign_mma_kernel", st);
             launch_chained(merge_assign_mma_kernel, dim3(kNumSMs), dim3(kMmaThreads), kMmaSmemBytes, st, 
-                tmA, tmA_half, reinterpret_cast<const __nv_bfloat16*>(feats), d, N, w.ev_lo, k, w.ev_out_off, w.ev_unit_off, out_src, inv_norm, w.is_key, w.best64,
-                w.status);
+                tmA, tmA_half, reinterpret_cast<const __nv_bfloat16*>(feats), d, N, w.ev_lo, k, w.ev_out_off, w.ev_unit_off, inv_norm,
+                tile, to, w.status);
         }
         METOK_LAUNCH_CHECK();
     } else {
-        METOK_TIMED("merge_assign_simt_kernel", st);
-        launch_chained(merge_assign_simt_kernel<T>, dim3(kNumSMs * kSaCtasPerSm), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
-                       w.ev_out_off, w.ev_unit_off, out_src, w.rest, inv_norm, w.best64);
+        {
+            METOK_TIMED("merge_assign_simt_kernel", st);
+            launch_chained(merge_assign_simt_kernel<T>, dim3(kNumSMs * kSaCtasPerSm), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
+                           w.ev_out_off, w.ev_unit_off, inv_norm, to);
+        }
+        METOK_LAUNCH_CHECK();
+        {
+            METOK_TIMED("merge_join_kernel", st);
+            launch_chained(merge_join_kernel, dim3(ceil_div(Nv, 256)), dim3(256), 0, st, Nv, N, w.ev_lo, k, w.ev_out_off, to);
+        }
         METOK_LAUNCH_CHECK();
     }
 
-    {
-        METOK_TIMED("merge_decode_kernel", st);
-        launch_chained(merge_decode_kernel, dim3(ceil_div(Nv, 256)), dim3(256), 0, st, w.best64, w.is_key, Nv, N, w.ev_lo, k,
-                                                               assign, w.slot_blocks, w.slot_cnt, w.long_index,
-                                                               w.long_slot, w.long_counter, kAvgLong, avg_long_cap(d),
-                                                               w.few_members, kAvgFew, w.heavy_index, w.heavy_slot,
-                                                               w.heavy_counter, kAvgHeavy, kAvgHeavyCap, n_out);
-    }
-    METOK_LAUNCH_CHECK();
-    // rows in flight per CTA: a pass over a row moves at most seg0 bytes, the ring holds 24 KiB
-    const uint32_t seg0 = (uint32_t)std::min<long long>(kAvgThreads * kAvgChunks, (long long)d * sizeof(T) / 16) * 16u;
+    // Pieces of up to 2 KB, or of 1 KB (so that twice as many copies of a row list are in flight per warp) when the rows
+    // are that short or 2 KB pieces would leave half of the warps without one.
+    AvgArgs ar = {};
+    const int nchunk = d * (int)sizeof(T) / 16;
+    const int warps = kNumSMs * kAvgCtasPerSm * kAvgWarps;
+    const bool small = nchunk <= 64 || (long long)cap * ceil_div(nchunk, 128) < warps / 2;
+    ar.nseg = ceil_div(nchunk, small ? 64 : 128);
+    ar.seg_chunks = ceil_div(nchunk, ar.nseg);
+    ar.d = d; ar.N = N; ar.Nv = Nv;
+    ar.ev_lo = w.ev_lo; ar.out_event = out_event; ar.assign = assign;
+    ar.ml = w.ml;
+    ar.long_sums = w.long_sums; ar.long_done = w.long_done; ar.next_item = w.avg_next; ar.next = w.avg_next + 1;
+    ar.n_out = n_out; ar.out_members = out_members; ar.status = w.status;
+    const int grid = (int)std::min<long long>(kNumSMs * kAvgCtasPerSm, ((long long)cap * ar.nseg + kAvgWarps - 1) / kAvgWarps);
     auto launch = [&](auto kernel) -> int {
         METOK_ALLOW_SMEM(kernel, kAvgSmemBytes);
         {
             METOK_TIMED("merge_avg_kernel", st);
-            launch_chained(kernel, dim3(kAvgFrontCtas + cap), dim3(kAvgThreads), kAvgSmemBytes, st,
-                feats, d, N, Nv, w.ev_lo, out_event, assign, w.slot_blocks, w.slot_cnt, w.long_index, w.long_slot,
-                w.long_counter, w.few_members, w.heavy_index, w.heavy_slot, w.heavy_counter, w.long_sums, w.long_done,
-                kAvgFrontCtas, n_out, out_feats, out_members,
-                w.status);
+            launch_chained(kernel, dim3(grid), dim3(kAvgThreads), kAvgSmemBytes, st, feats, out_feats, ar);
         }
         METOK_LAUNCH_CHECK();
         return METOK_OK;
     };
-    if (seg0 > (uint32_t)kAvgStageBytes / 2) return launch(merge_avg_kernel<T, kAvgStages>);
-    if (seg0 > (uint32_t)kAvgStageBytes / 4) return launch(merge_avg_kernel<T, 2 * kAvgStages>);
-    return launch(merge_avg_kernel<T, 4 * kAvgStages>);
+    return small ? launch(merge_avg_kernel<T, 8>) : launch(merge_avg_kernel<T, 4>);
 }
 
 }  // namespace metok
