@@ -37,6 +37,7 @@ template <typename T>
 __global__ void __launch_bounds__(kSegThreads)
 seg_partial_kernel(const T* __restrict__ feats, int Tn, long long chunks_per_frame, int frames_per_cta,
                    float* __restrict__ part_dot, float* __restrict__ part_nrm) {
+    grid_dep_wait();
     constexpr int VN = Vec16<T>::N;
     constexpr int NW = kSegThreads / 32;
     __shared__ float s_nn[kSegMaxRun + 1][NW], s_dp[kSegMaxRun + 1][NW];
@@ -102,6 +103,7 @@ seg_partial_kernel(const T* __restrict__ feats, int Tn, long long chunks_per_fra
 template <typename T>
 __global__ void __launch_bounds__(128)
 seg_mean_kernel(const T* __restrict__ feats, int N, int d, float* __restrict__ mean) {
+    grid_dep_wait();
     constexpr int VN = Vec16<T>::N;
     const int f = blockIdx.y;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -124,6 +126,7 @@ seg_mean_kernel(const T* __restrict__ feats, int N, int d, float* __restrict__ m
 __global__ void __launch_bounds__(256)
 seg_meandot_kernel(const float* __restrict__ mean, int Tn, int d, float* __restrict__ part_dot,
                    float* __restrict__ part_nrm) {
+    grid_dep_wait();
     __shared__ float red[2][8];
     const int f = blockIdx.x;
     const float* a = mean + (size_t)f * d;
@@ -157,9 +160,11 @@ seg_finish_kernel(const float* __restrict__ part_dot, const float* __restrict__ 
                   int32_t* __restrict__ event_offsets, int32_t* __restrict__ frame_event) {
     grid_dep_wait();
     extern __shared__ float sm_f[];
-    float* s_sim = sm_f;                                   // [Tn]   (Tn-1 used)
-    float* s_nrm = sm_f + Tn;                              // [Tn]
-    int* s_flag = reinterpret_cast<int*>(sm_f + 2 * Tn);   // [Tn]  boundary after frame i
+    const int Tp = (Tn + 3) & ~3;
+    float* s_sim = sm_f;                                   // [Tp]   (Tn-1 used)
+    float* s_nrm = sm_f + Tp;                              // [Tp]   norms, later the similarities' keys
+    uint32_t* s_simkey = reinterpret_cast<uint32_t*>(s_nrm);
+    int* s_flag = reinterpret_cast<int*>(sm_f + 2 * Tp);   // [Tp]  boundary after frame i
     __shared__ int s_scan[32];
     const int tid = threadIdx.x, nthr = blockDim.x;
 
@@ -202,27 +207,48 @@ seg_finish_kernel(const float* __restrict__ part_dot, const float* __restrict__ 
         __syncthreads();
     }
     __syncthreads();
+    // Integer keys give a total order even with non-finite similarities (a NaN ranks as the largest value), so exactly
+    // k-1 boundaries are flagged whatever the input holds.
     for (int i = tid; i < Tn - 1; i += nthr) {
         const float c = s_sim[i] / (s_nrm[i] * s_nrm[i + 1]);
         s_sim[i] = c;
         sims[i] = c;
     }
     __syncthreads();
+    for (int i = tid; i < Tp; i += nthr) s_simkey[i] = i < Tn - 1 ? sim_key(s_sim[i]) : 0xFFFFFFFFu;
+    __syncthreads();
+    // Rank by counting: P lanes share a frame, each compares it with every P-th group of four keys; in the groups before
+    // the frame's own an equal key ranks lower, in those after it higher.  (One thread per frame, comparing floats one by
+    // one: 25 us of this kernel at 512 frames.)
     const int nb = k - 1;
-    for (int i = tid; i < Tn; i += nthr) {
-        int flag = 0;
+    const int p_log2 = Tn > 512 ? 0 : Tn > 256 ? 1 : Tn > 128 ? 2 : 3, P = 1 << p_log2;
+    for (int i0 = 0; i0 < Tn; i0 += nthr >> p_log2) {
+        const int i = i0 + (tid >> p_log2), part = tid & (P - 1);
+        int rank = 0;
         if (i < Tn - 1 && nb > 0) {
-            // integer keys give a total order even with non-finite similarities (a NaN ranks as the
-            // largest value), so exactly k-1 boundaries are flagged whatever the input holds
-            const uint32_t v = sim_key(s_sim[i]);
-            int rank = 0;
-            for (int j = 0; j < Tn - 1; ++j) {
-                const uint32_t w = sim_key(s_sim[j]);
-                rank += (w < v) || (w == v && j < i);
+            const uint32_t v = s_simkey[i];
+            const uint4* keys4 = reinterpret_cast<const uint4*>(s_simkey);
+            const int own = i >> 2, nq = (Tn + 2) >> 2;
+            int q = part;
+#pragma unroll 4
+            for (; q < own; q += P) {
+                const uint4 w = keys4[q];
+                rank += (w.x <= v) + (w.y <= v) + (w.z <= v) + (w.w <= v);
             }
-            flag = rank < nb;
+            if (q == own) {
+                const uint4 w = keys4[q];
+                const int r = i & 3;
+                rank += (w.x < v || (w.x == v && 0 < r)) + (w.y < v || (w.y == v && 1 < r)) + (w.z < v || (w.z == v && 2 < r)) + (w.w < v);
+                q += P;
+            }
+#pragma unroll 4
+            for (; q < nq; q += P) {
+                const uint4 w = keys4[q];
+                rank += (w.x < v) + (w.y < v) + (w.z < v) + (w.w < v);
+            }
         }
-        s_flag[i] = flag;
+        for (int o = 1; o < P; o <<= 1) rank += __shfl_xor_sync(0xFFFFFFFFu, rank, o);
+        if (part == 0 && i < Tn) s_flag[i] = i < Tn - 1 && rank < nb;
     }
     __syncthreads();
     // exclusive scan of the flags: contiguous ranges per thread, a shuffle scan inside each warp,
@@ -275,8 +301,8 @@ static int launch_segment(const void* feats, int Tn, int N, int d, int k, int si
         dim3 grid(nslab, ceil_div(Tn, fpc));
         {
             METOK_TIMED("seg_partial_kernel", st);
-            seg_partial_kernel<T><<<grid, kSegThreads, 0, st>>>(reinterpret_cast<const T*>(feats), Tn, chunks, fpc,
-                                                            part_dot, part_nrm);
+            launch_chained(seg_partial_kernel<T>, grid, dim3(kSegThreads), 0, st, reinterpret_cast<const T*>(feats), Tn, chunks, fpc,
+                           part_dot, part_nrm);
         }
         METOK_LAUNCH_CHECK();
     } else {
@@ -287,16 +313,16 @@ static int launch_segment(const void* feats, int Tn, int N, int d, int k, int si
         dim3 grid(ceil_div(d / VN, 128), Tn);
         {
             METOK_TIMED("seg_mean_kernel", st);
-            seg_mean_kernel<T><<<grid, 128, 0, st>>>(reinterpret_cast<const T*>(feats), N, d, mean);
+            launch_chained(seg_mean_kernel<T>, grid, dim3(128), 0, st, reinterpret_cast<const T*>(feats), N, d, mean);
         }
         METOK_LAUNCH_CHECK();
         {
             METOK_TIMED("seg_meandot_kernel", st);
-            seg_meandot_kernel<<<Tn, 256, 0, st>>>(mean, Tn, d, part_dot, part_nrm);
+            launch_chained(seg_meandot_kernel, dim3(Tn), dim3(256), 0, st, mean, Tn, d, part_dot, part_nrm);
         }
         METOK_LAUNCH_CHECK();
     }
-    const size_t smem = (size_t)Tn * 3 * sizeof(float);
+    const size_t smem = (size_t)((Tn + 3) & ~3) * 3 * sizeof(float);
     if (smem > 48 * 1024) {
         METOK_ALLOW_SMEM(seg_finish_kernel, smem);
     }
@@ -392,6 +418,7 @@ __global__ void __launch_bounds__(kFsThreads, 3)
 seg_score_kernel(const T* __restrict__ feats, const T* __restrict__ text, int Tn, int N, int d, int frames_per_warp,
                  float* __restrict__ part_dot, float* __restrict__ part_nrm, float* __restrict__ token_score,
                  float* __restrict__ inv_norm) {
+    grid_dep_wait();
     constexpr int VN = Vec16<T>::N;
     extern __shared__ float s_t[];                 // [d], in planes of 4 floats per chunk (conflict-free 16-byte reads)
                                                    // then [warps][nchunk] raw 16-byte chunks: the previous frame's row
@@ -681,12 +708,12 @@ static int launch_seg_score(const void* feats, const void* text, int Tn, int N, 
         if (rc != METOK_OK) return rc;
         const int warps = N * ceil_div(Tn, fpw);
         METOK_TIMED("seg_score_kernel", st);
-        seg_score_kernel<T, kCH><<<ceil_div(warps, kFsThreads / 32), kFsThreads, smem_t, st>>>(
+        launch_chained(seg_score_kernel<T, kCH>, dim3(ceil_div(warps, kFsThreads / 32)), dim3(kFsThreads), smem_t, st,
             reinterpret_cast<const T*>(feats), reinterpret_cast<const T*>(text), Tn, N, d, fpw, part_dot, part_nrm,
             token_score, inv_norm);
     }
     METOK_LAUNCH_CHECK();
-    const size_t smem = (size_t)Tn * 3 * sizeof(float);
+    const size_t smem = (size_t)((Tn + 3) & ~3) * 3 * sizeof(float);
     if (smem > 48 * 1024)
         METOK_ALLOW_SMEM(seg_finish_kernel, smem);
     {

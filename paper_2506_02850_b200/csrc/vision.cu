@@ -14,86 +14,68 @@ namespace metok {
 
 // --------------------------------------------------------------------------- //
 // token_score[j] = <x_j, t> / (max(|x_j|, eps) * max(|t|, eps)); also 1/max(|x_j|, eps).
-// One warp per token row, 16-byte loads, four chunks in flight per lane.
+// One warp per token row, 16-byte loads, eight chunks of the row in flight per lane.  The text's chunks are read
+// beside them (they stay in L1), so a CTA has nothing to prepare: with the text laid out in shared memory first, a
+// CTA of 64 rows x 196 tokens x 1152 spent more time on that than on its rows (11.5 us; MEASURED_TS now).
 // --------------------------------------------------------------------------- //
+template <typename T>
+__device__ __forceinline__ void widen_chunk(const uint4& r, float (&v)[16 / sizeof(T)]) {
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if constexpr (sizeof(T) == 4) {
+            v[i] = __uint_as_float(w[i]);
+        } else {
+            v[2 * i]     = __uint_as_float(w[i] << 16);
+            v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+        }
+    }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256)
 tok_score_kernel(const T* __restrict__ feats, const T* __restrict__ text, int Nv, int d,
                  float* __restrict__ token_score, float* __restrict__ inv_norm) {
+    grid_dep_wait();
     constexpr int VN = Vec16<T>::N;
-    extern __shared__ float s_t[];                 // [d]
-    __shared__ float s_red[8];
-    __shared__ float s_tn;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nchunk = d / VN;
-    // t is stored in planes of 4 floats per chunk so that a lane's 16-byte reads
-    // of consecutive chunks are bank-conflict free
-    for (int i = tid; i < d; i += 256) {
-        const int c = i / VN, q = i % VN;
-        s_t[(q >> 2) * (nchunk * 4) + c * 4 + (q & 3)] = to_float(text[i]);
-    }
-    __syncthreads();
-    float a = 0.f;
-    for (int i = tid; i < d; i += 256) a = fmaf(s_t[i], s_t[i], a);
-    a = warp_sum(a);
-    if (lane == 0) s_red[warp] = a;
-    __syncthreads();
-    if (tid == 0) {
-        float s = 0.f;
-        for (int w = 0; w < 8; ++w) s += s_red[w];
-        s_tn = fmaxf(sqrtf(s), kEps);
-    }
-    __syncthreads();
-    const float tn = s_tn;
+    const uint4* t4 = reinterpret_cast<const uint4*>(text);
     // rows from the last one down: the pass before this one (segmentation) streams V upwards
     // and leaves its tail in L2
     for (int rr = blockIdx.x * 8 + warp; rr < Nv; rr += gridDim.x * 8) {
         const int row = Nv - 1 - rr;
-        const T* x = feats + (size_t)row * d;
-        float nn = 0.f, dt = 0.f;
+        const uint4* x4 = reinterpret_cast<const uint4*>(feats) + (size_t)row * nchunk;
+        float nn = 0.f, dt = 0.f, tt = 0.f;
         constexpr int U = 8;                        // 16-byte chunks in flight per lane
         for (int c0 = 0; c0 < nchunk; c0 += 32 * U) {
             uint4 raw[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int c = c0 + u * 32 + lane;
-                raw[u] = c < nchunk ? __ldg(reinterpret_cast<const uint4*>(x) + c) : make_uint4(0u, 0u, 0u, 0u);
+                raw[u] = c < nchunk ? __ldg(x4 + c) : make_uint4(0u, 0u, 0u, 0u);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int c = c0 + u * 32 + lane;
                 if (c < nchunk) {
-                    float v[VN];
-                    if constexpr (sizeof(T) == 4) {
-                        v[0] = __uint_as_float(raw[u].x); v[1] = __uint_as_float(raw[u].y);
-                        v[2] = __uint_as_float(raw[u].z); v[3] = __uint_as_float(raw[u].w);
-                    } else {
-                        const uint32_t w[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+                    float v[VN], t[VN];
+                    widen_chunk<T>(raw[u], v);
+                    widen_chunk<T>(__ldg(t4 + c), t);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            v[2 * i]     = __uint_as_float(w[i] << 16);
-                            v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-                        }
-                    }
-#pragma unroll
-                    for (int h = 0; h < VN / 4; ++h) {
-                        const float4 tt = reinterpret_cast<const float4*>(s_t + h * (nchunk * 4))[c];
-                        nn = fmaf(v[4 * h + 0], v[4 * h + 0], nn);
-                        dt = fmaf(v[4 * h + 0], tt.x, dt);
-                        nn = fmaf(v[4 * h + 1], v[4 * h + 1], nn);
-                        dt = fmaf(v[4 * h + 1], tt.y, dt);
-                        nn = fmaf(v[4 * h + 2], v[4 * h + 2], nn);
-                        dt = fmaf(v[4 * h + 2], tt.z, dt);
-                        nn = fmaf(v[4 * h + 3], v[4 * h + 3], nn);
-                        dt = fmaf(v[4 * h + 3], tt.w, dt);
+                    for (int i = 0; i < VN; ++i) {
+                        nn = fmaf(v[i], v[i], nn);
+                        dt = fmaf(v[i], t[i], dt);
+                        tt = fmaf(t[i], t[i], tt);
                     }
                 }
             }
         }
         nn = warp_sum(nn);
         dt = warp_sum(dt);
+        tt = warp_sum(tt);
         if (lane == 0) {
-            const float n = fmaxf(sqrtf(nn), kEps);
+            const float n = fmaxf(sqrtf(nn), kEps), tn = fmaxf(sqrtf(tt), kEps);
             token_score[row] = dt / (n * tn);
             inv_norm[row] = 1.0f / n;
         }
@@ -110,7 +92,8 @@ __device__ __forceinline__ int find_event(const int32_t* __restrict__ off, int k
     return lo;
 }
 
-// Event scores, key events, per-event token budgets and output offsets.  One CTA.
+// Event scores, key events, per-event token budgets and output offsets.  One CTA; with many frames a cluster, whose
+// other CTAs only average frames for it (512 frames: 13.4 us with one CTA, MEASURED_EP with four).
 struct PlanParams {
     int Tn, N, k, n_key_events, event_agg, mode, tile_rows, chunk_cols;
     int rows_with_keys;                         // the merge's row tiles run over all tokens of an event (1) or only over those that are no key token (0)
@@ -129,11 +112,13 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
                   int32_t* __restrict__ frame_ev, int32_t* __restrict__ frame_stride,
                   int32_t* __restrict__ frame_off, int32_t* __restrict__ n_out, int32_t* __restrict__ counters, int n_counters,
                   int32_t* __restrict__ status) {
+    const int C = (int)gridDim.x, rank = (int)blockIdx.x;
+    if (C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     grid_dep_wait();
     extern __shared__ float s_score[];      // [k]
-    if (threadIdx.x == 0) *status = 0;
-    for (int i = threadIdx.x; i < n_counters; i += blockDim.x) counters[i] = 0;   // what later kernels of the call count in
-    __shared__ int s_scan[1024];
+    if (rank == 0 && threadIdx.x == 0) *status = 0;
+    for (int i = rank * 1024 + threadIdx.x; i < n_counters; i += C * 1024) counters[i] = 0;   // what later kernels of the call count in
+    __shared__ int s_scan[32];
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int k = pp.k, Tn = pp.Tn;
     // frame_score[f] = mean of the frame's N token scores; eight lanes per frame (a lane's loads are
@@ -142,12 +127,18 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
     int* s_evlo = reinterpret_cast<int*>(s_frame + Tn);     // [k] first frame of the event, clamped
     int* s_evhi = s_evlo + k;                                // [k] one past its last frame
     int* s_bud = s_evhi + k;                                 // [k] budget of the event
-    unsigned char* s_key = reinterpret_cast<unsigned char*>(s_bud + k);   // [k]
-    for (int f0 = 0; f0 < Tn; f0 += nthr >> 3) {
+    int* s_units = s_bud + k;                                // [k] merge units of the event
+    unsigned char* s_key = reinterpret_cast<unsigned char*>(s_units + k);   // [k]
+    float* s_frame0 = s_frame;              // the first CTA's
+    if (C > 1) {
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // everybody has started
+        s_frame0 = cg::this_cluster().map_shared_rank(s_frame, 0);
+    }
+    for (int f0 = rank * (nthr >> 3); f0 < Tn; f0 += C * (nthr >> 3)) {
         const int f = f0 + (tid >> 3), part = tid & 7;
         float s = 0.f;
         if (f < Tn) {
-            constexpr int kB = 6;                           // loads in flight; the additions keep their order
+            constexpr int kB = 9;                           // loads in flight; the additions keep their order
             for (int p0 = part; p0 < pp.N; p0 += 8 * kB) {
                 float x[kB];
 #pragma unroll
@@ -160,11 +151,18 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
         if (f < Tn && part == 0) {
-            s_frame[f] = s / (float)pp.N;
-            frame_score[f] = s_frame[f];
+            s /= (float)pp.N;
+            s_frame0[f] = s;
+            frame_score[f] = s;
         }
     }
-    __syncthreads();
+    if (C > 1) {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (rank > 0) return;
+    } else {
+        __syncthreads();
+    }
     for (int e = tid; e < k; e += nthr) {
         int lo = min(max(event_offsets[e], 0), Tn);
         int hi = min(max(event_offsets[e + 1], lo), Tn);
@@ -177,10 +175,12 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
             s = -3.0e38f;
         } else if (pp.event_agg == METOK_AGG_MEAN) {
             float a = 0.f;
+#pragma unroll 8
             for (int f = lo; f < hi; ++f) a += s_frame[f];
             s = a / (float)(hi - lo);
         } else {
             float a = s_frame[lo];
+#pragma unroll 8
             for (int f = lo + 1; f < hi; ++f) a = fmaxf(a, s_frame[f]);
             s = a;
         }
@@ -211,21 +211,32 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
             if (b > m) b = m;
             ev_budget[e] = (int)b;
             s_bud[e] = (int)b;
+            const int rows = m - (pp.rows_with_keys ? 0 : (int)b);
+            s_units[e] = (rows + pp.tile_rows - 1) / pp.tile_rows * (((int)b + pp.chunk_cols - 1) / pp.chunk_cols);   // row tiles x key chunks
         }
         __syncthreads();
-        if (tid == 0) {                                     // everything it reads is in shared memory
+        if (tid < 32) {                                     // offsets: one warp, 32 events at a time
             int slots = 0, units = 0;
-            for (int e = 0; e < k; ++e) {
-                ev_out_off[e] = slots;
-                ev_unit_off[e] = units;
-                slots += s_bud[e];
-                const int rows = (s_evhi[e] - s_evlo[e]) * pp.N - (pp.rows_with_keys ? 0 : s_bud[e]);
-                const int t = (rows + pp.tile_rows - 1) / pp.tile_rows;
-                units += t * ((s_bud[e] + pp.chunk_cols - 1) / pp.chunk_cols);   // row tiles x key chunks
+            for (int e0 = 0; e0 < k; e0 += 32) {
+                const int e = e0 + tid, b = e < k ? s_bud[e] : 0, u = e < k ? s_units[e] : 0;
+                int bi = b, ui = u;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(0xFFFFFFFFu, bi, o), y = __shfl_up_sync(0xFFFFFFFFu, ui, o);
+                    if (tid >= o) { bi += x; ui += y; }
+                }
+                if (e < k) {
+                    ev_out_off[e] = slots + bi - b;
+                    ev_unit_off[e] = units + ui - u;
+                }
+                slots += __shfl_sync(0xFFFFFFFFu, bi, 31);
+                units += __shfl_sync(0xFFFFFFFFu, ui, 31);
             }
-            ev_out_off[k] = slots;
-            ev_unit_off[k] = units;
-            *n_out = slots;
+            if (tid == 0) {
+                ev_out_off[k] = slots;
+                ev_unit_off[k] = units;
+                *n_out = slots;
+            }
         }
     } else {
         // Algorithm 1: key frames = the ceil(beta * len) best-scored frames of every event (ties to the
@@ -250,12 +261,13 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
             if (nk < 1) nk = 1;
             if (nk > len) nk = len;
             const float v = s_frame[f];
-            int rank = 0;
+            int better = 0;
+#pragma unroll 8
             for (int j = lo; j < hi; ++j) {
                 const float w = s_frame[j];
-                rank += (w > v) || (w == v && j < f);
+                better += (w > v) || (w == v && j < f);
             }
-            const bool key_frame = pp.key_frames_given ? pp.key_frames_given[f] != 0 : rank < (int)nk;
+            const bool key_frame = pp.key_frames_given ? pp.key_frames_given[f] != 0 : better < (int)nk;
             frame_stride[f] = event_is_key[e] ? (key_frame ? pp.s1 : pp.s2) : (key_frame ? pp.s1_nonkey : pp.s2_nonkey);
         }
         __syncthreads();
@@ -267,110 +279,85 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
             const int go = (pp.grid + frame_stride[f] - 1) / frame_stride[f];
             local += go * go;
         }
-        s_scan[tid] = local;
-        __syncthreads();
-        for (int off = 1; off < nthr; off <<= 1) {
-            const int v = (tid >= off) ? s_scan[tid - off] : 0;
-            __syncthreads();
-            s_scan[tid] += v;
-            __syncthreads();
+        const int lane = tid & 31, warp = tid >> 5;
+        int incl = local;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += v;
         }
-        int run = s_scan[tid] - local;
+        if (lane == 31) s_scan[warp] = incl;
+        __syncthreads();
+        const int wt = s_scan[lane];
+        const int total = __reduce_add_sync(0xFFFFFFFFu, wt);
+        int run = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? wt : 0) + incl - local;
         for (int f = lo; f < hi; ++f) {
             frame_off[f] = run;
             const int go = (pp.grid + frame_stride[f] - 1) / frame_stride[f];
             run += go * go;
         }
-        if (tid == nthr - 1) { frame_off[Tn] = s_scan[tid]; *n_out = s_scan[tid]; }
+        if (tid == 0) { frame_off[Tn] = total; *n_out = total; }
     }
 }
 
 // --------------------------------------------------------------------------- //
-// Adaptive pooling (Algorithm 1): one CTA per output token = one window of one frame's
-// G x G token grid, window = stride, edge windows clipped to the grid.  The window's
-// cells are added in row-major order in fp32 (two rows of V in flight per thread),
-// divided by their number and rounded once.
+// Adaptive pooling (Algorithm 1): an output token = one window of one frame's G x G token grid, window = stride,
+// edge windows clipped to the grid.  A thread owns one 16-byte chunk of one window: the cells are added in row-major
+// order in fp32, divided by their number and rounded once.  A CTA takes a share of a frame's (window, chunk) pairs, so
+// the frame's stride and offset are looked up once, every load is one of consecutive 16-byte chunks, and what is in
+// flight is four loads of every thread of the chip.  (A CTA per window, two rows in flight, at 128 registers: 40 us
+// for 64 frames of 196 tokens of 1152; MEASURED_PO now.)
 // --------------------------------------------------------------------------- //
-constexpr int kPoolThreads = 128;
-constexpr int kPoolChunks = 4;
+constexpr int kPoolThreads = 256;
 
 template <typename T>
 __global__ void __launch_bounds__(kPoolThreads)
-pool_kernel(const T* __restrict__ feats, int d, int N, int G, int Tn, const int32_t* __restrict__ frame_off,
-            const int32_t* __restrict__ frame_stride, const int32_t* __restrict__ frame_ev,
-            const int32_t* __restrict__ n_out, T* __restrict__ out_feats, int32_t* __restrict__ out_src,
-            int32_t* __restrict__ out_event, int32_t* __restrict__ out_members, int32_t* __restrict__ assign) {
+pool_kernel(const T* __restrict__ feats, int d, int N, int G, const int32_t* __restrict__ frame_off,
+            const int32_t* __restrict__ frame_stride, const int32_t* __restrict__ frame_ev, T* __restrict__ out_feats,
+            int32_t* __restrict__ out_src, int32_t* __restrict__ out_event, int32_t* __restrict__ out_members,
+            int32_t* __restrict__ assign) {
+    grid_dep_wait();
     constexpr int VN = Vec16<T>::N;
-    const int o = blockIdx.x;
-    if (o >= *n_out) return;
-    const int f = find_event(frame_off, Tn, o);
-    const int w = o - frame_off[f];
-    const int s = frame_stride[f];
-    const int go = (G + s - 1) / s;
-    const int r0 = (w / go) * s, r1 = min(G, r0 + s);
-    const int c0 = (w % go) * s, c1 = min(G, c0 + s);
-    const int wc = c1 - c0, cells = (r1 - r0) * wc;
-    const int tid = threadIdx.x;
-    const int nchunk = d / VN;
-    const size_t frame_base = (size_t)f * N;
-    auto cell_token = [&](int i) { return frame_base + (size_t)(r0 + i / wc) * G + (c0 + i % wc); };
-    for (int cb = 0; cb < nchunk; cb += kPoolThreads * kPoolChunks) {
-        float acc[kPoolChunks][VN];
+    const int f = blockIdx.y, s = frame_stride[f], off = frame_off[f], e = frame_ev[f];
+    const int go = (G + s - 1) / s, nchunk = d / VN, items = go * go * nchunk;
+    const uint4* frame = reinterpret_cast<const uint4*>(feats) + (size_t)f * N * nchunk;
+    for (int it = blockIdx.x * kPoolThreads + threadIdx.x; it < items; it += gridDim.x * kPoolThreads) {
+        const int w = it / nchunk, c = it - w * nchunk, wy = w / go, wx = w - wy * go;
+        const int r0 = wy * s, c0 = wx * s, wc = min(G, c0 + s) - c0, cells = (min(G, r0 + s) - r0) * wc;
+        const int first = r0 * G + c0, o = off + w;
+        float acc[VN];
+        Vec16<T>::zero(acc);
+        int cell = first, col = 0;                          // the next cell to load
+        for (int i = 0; i < cells; i += 4) {
+            uint4 raw[4];
 #pragma unroll
-        for (int u = 0; u < kPoolChunks; ++u) Vec16<T>::zero(acc[u]);
-        int i = 0;
-        for (; i + 1 < cells; i += 2) {
-            const T* x0 = feats + cell_token(i) * d;
-            const T* x1 = feats + cell_token(i + 1) * d;
-            float v0[kPoolChunks][VN], v1[kPoolChunks][VN];
-#pragma unroll
-            for (int u = 0; u < kPoolChunks; ++u) {
-                const int ch = cb + u * kPoolThreads + tid;
-                if (ch < nchunk) {
-                    Vec16<T>::load(x0 + (size_t)ch * VN, v0[u]);
-                    Vec16<T>::load(x1 + (size_t)ch * VN, v1[u]);
-                }
+            for (int u = 0; u < 4; ++u) {
+                raw[u] = i + u < cells ? __ldg(frame + (size_t)cell * nchunk + c) : make_uint4(0u, 0u, 0u, 0u);
+                ++cell;
+                if (++col == wc) { col = 0; cell += G - wc; }
             }
 #pragma unroll
-            for (int u = 0; u < kPoolChunks; ++u) {
-                const int ch = cb + u * kPoolThreads + tid;
-                if (ch < nchunk) {
+            for (int u = 0; u < 4; ++u) {
+                float v[VN];
+                widen_chunk<T>(raw[u], v);
+                if (i + u < cells) {
 #pragma unroll
-                    for (int q = 0; q < VN; ++q) acc[u][q] = (acc[u][q] + v0[u][q]) + v1[u][q];
-                }
-            }
-        }
-        if (i < cells) {
-            const T* x0 = feats + cell_token(i) * d;
-#pragma unroll
-            for (int u = 0; u < kPoolChunks; ++u) {
-                const int ch = cb + u * kPoolThreads + tid;
-                if (ch < nchunk) {
-                    float v0[VN];
-                    Vec16<T>::load(x0 + (size_t)ch * VN, v0);
-#pragma unroll
-                    for (int q = 0; q < VN; ++q) acc[u][q] += v0[q];
+                    for (int q = 0; q < VN; ++q) acc[q] += v[q];
                 }
             }
         }
         const float inv = 1.0f / (float)cells;
+        alignas(16) T tmp[VN];
 #pragma unroll
-        for (int u = 0; u < kPoolChunks; ++u) {
-            const int ch = cb + u * kPoolThreads + tid;
-            if (ch < nchunk) {
-                T* dst = out_feats + (size_t)o * d + (size_t)ch * VN;
-                alignas(16) T tmp[VN];
-#pragma unroll
-                for (int q = 0; q < VN; ++q) from_float(tmp[q], acc[u][q] * inv);
-                *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(tmp);
-            }
+        for (int q = 0; q < VN; ++q) from_float(tmp[q], acc[q] * inv);
+        reinterpret_cast<uint4*>(out_feats)[(size_t)o * nchunk + c] = *reinterpret_cast<const uint4*>(tmp);
+        // the window's cells are told their output by the first of its threads
+        for (int i = c; i < cells; i += nchunk) assign[(size_t)f * N + (r0 + i / wc) * G + c0 + i % wc] = o;
+        if (c == 0) {
+            out_src[o] = f * N + first;
+            out_event[o] = e;
+            out_members[o] = cells;
         }
-    }
-    for (int i = tid; i < cells; i += kPoolThreads) assign[cell_token(i)] = o;
-    if (tid == 0) {
-        out_src[o] = (int32_t)cell_token(0);
-        out_event[o] = frame_ev[f];
-        out_members[o] = cells;
     }
 }
 
@@ -440,6 +427,7 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThread
 event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restrict__ ev_lo, int N,
                   const int32_t* __restrict__ ev_budget, const int32_t* __restrict__ ev_out_off, SelectLayout lay,
                   TokenOut out) {
+    grid_dep_wait();
     __shared__ SelectSmem sm;
     __shared__ int s_budget[1];
     extern __shared__ __align__(16) unsigned char sel_dyn[];
@@ -1519,13 +1507,10 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     // Eq. 5 per token, unless the caller brings the scores and norms from metok_segment_score_events
     const float* inv_norm = p->token_inv_norm ? p->token_inv_norm : w.inv_norm;
     if (!p->token_inv_norm) {
-        const int grid = min(ceil_div(Nv, 8), kNumSMs * 8);
-        const size_t smem = (size_t)d * sizeof(float);
-        if (smem > 48 * 1024)
-            METOK_ALLOW_SMEM(tok_score_kernel<T>, smem);
         {
             METOK_TIMED("tok_score_kernel", st);
-            tok_score_kernel<T><<<grid, 256, smem, st>>>(feats, text, Nv, d, token_score, w.inv_norm);
+            launch_chained(tok_score_kernel<T>, dim3(min(ceil_div(Nv, 8), kNumSMs * 32)), dim3(256), 0, st, feats, text, Nv, d,
+                           token_score, w.inv_norm);
         }
         METOK_LAUNCH_CHECK();
     }
@@ -1542,12 +1527,14 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     pp.grid = 1;
     while (pp.grid * pp.grid < N) ++pp.grid;
     pp.s1 = p->s1; pp.s2 = p->s2; pp.s1_nonkey = p->s1_nonkey; pp.s2_nonkey = p->s2_nonkey;
-    const size_t plan_smem = (size_t)(k + Tn) * sizeof(float) + (size_t)k * (3 * sizeof(int) + 1);
+    const size_t plan_smem = (size_t)(k + Tn) * sizeof(float) + (size_t)k * (4 * sizeof(int) + 1);
+    // more CTAs than one as soon as one would need more than two rounds for the frames
+    const int plan_ctas = Tn <= 256 ? 1 : Tn <= 512 ? 4 : 8;
     if (plan_smem > 40 * 1024)
         METOK_ALLOW_SMEM(event_plan_kernel, plan_smem);
     {
         METOK_TIMED("event_plan_kernel", st);
-        launch_chained(event_plan_kernel, dim3(1), dim3(1024), plan_smem, st, token_score, frame_score, event_offsets, pp, event_score,
+        launch_chained_clusters(plan_ctas, event_plan_kernel, dim3(plan_ctas), dim3(1024), plan_smem, st, token_score, frame_score, event_offsets, pp, event_score,
                        event_is_key, w.ev_lo, w.ev_budget, w.ev_out_off, w.ev_unit_off, w.frame_ev, w.frame_stride, w.frame_off,
                        n_out, w.ml.long_counter, w.n_counters, w.status);
     }
@@ -1556,9 +1543,13 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     if (p->mode == METOK_MODE_POOL) {
         {
             METOK_TIMED("pool_kernel", st);
-            pool_kernel<T><<<cap, kPoolThreads, 0, st>>>(feats, d, N, pp.grid, Tn, w.frame_off, w.frame_stride,
-                                                     w.frame_ev, n_out, out_feats, out_src, out_event, out_members,
-                                                     assign);
+            // about sixteen CTAs per SM, but no more per frame than its largest number of pairs fills
+            const int smin = std::min(std::min(p->s1, p->s2), std::min(p->s1_nonkey, p->s2_nonkey));
+            const int side = ceil_div(pp.grid, smin);
+            const int most = (int)std::min<long long>(ceil_div(kNumSMs * 16, Tn),
+                                                      ((long long)side * side * (d * (int)sizeof(T) / 16) + kPoolThreads - 1) / kPoolThreads);
+            launch_chained(pool_kernel<T>, dim3(std::max(1, most), Tn), dim3(kPoolThreads), 0, st, feats, d, N, pp.grid, w.frame_off,
+                           w.frame_stride, w.frame_ev, out_feats, out_src, out_event, out_members, assign);
         }
         METOK_LAUNCH_CHECK();
         return METOK_OK;
@@ -1590,7 +1581,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
             if (lay.bytes > 32 * 1024)                    // static + dynamic beyond 48 KiB needs the opt-in
                 METOK_ALLOW_SMEM(event_topk_kernel, lay.bytes);
             METOK_TIMED("event_topk_kernel", st);
-            event_topk_kernel<<<k * kSelCluster, nthreads, lay.bytes, st>>>(
+            launch_chained(event_topk_kernel, dim3(k * kSelCluster), dim3(nthreads), lay.bytes, st,
                 token_score, w.ev_lo, N, w.ev_budget, w.ev_out_off, lay, to);
         }
         METOK_LAUNCH_CHECK();
