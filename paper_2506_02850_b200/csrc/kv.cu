@@ -42,6 +42,7 @@ struct KvPtrs {
 __global__ void __launch_bounds__(256)
 kv_paper_lists_kernel(int S_cur, int vis_start, int n_vis, int l1, int32_t* __restrict__ keep_idx,
                       int32_t* __restrict__ keep_len, int32_t* __restrict__ new_len) {
+    grid_dep_wait();
     const int layer = blockIdx.x;
     int32_t* keep = keep_idx + (size_t)layer * S_cur;
     int n;
@@ -57,6 +58,43 @@ kv_paper_lists_kernel(int S_cur, int vis_start, int n_vis, int l1, int32_t* __re
     if (threadIdx.x == 0) { keep_len[layer] = n; new_len[layer] = n; }
 }
 
+// PAPER policy when no more rows follow the visual span than it holds (the rule: a question is shorter than its video):
+// every row that moves comes from beyond the new length, so one kernel writes the lists and moves the rows, a
+// contiguous piece per slab.  (Three launches, the lists read back row by row: 12.3 us for 6272 + 80 rows in 28 layers;
+// 4.2 now, one pass of a replayed graph.)  The CTAs of a layer's slabs share the writing of its list.
+__global__ void __launch_bounds__(256)
+kv_paper_kernel(KvPtrs ptrs, int layer0, int Hkv, int S_cap, int S_cur, int row_chunks, int vis_start, int n_vis, int l1,
+                int32_t* __restrict__ keep_idx, int32_t* __restrict__ keep_len, int32_t* __restrict__ new_len,
+                int32_t* __restrict__ status) {
+    grid_dep_wait();
+    const int slab = blockIdx.y, head = slab % Hkv, which = (slab / Hkv) & 1, ll = slab / (2 * Hkv), layer = layer0 + ll;
+    const int tail = S_cur - (vis_start + n_vis), n = layer < l1 ? S_cur : vis_start + tail;
+    if (layer >= l1) {
+        uint4* base = reinterpret_cast<uint4*>(which ? ptrs.v[ll] : ptrs.k[ll]) + (size_t)head * S_cap * row_chunks;
+        uint4* dst = base + (size_t)vis_start * row_chunks;
+        const uint4* src = dst + (size_t)n_vis * row_chunks;
+        const int total = n_vis > 0 ? tail * row_chunks : 0;
+        constexpr int U = 4;
+        for (int g0 = blockIdx.x * 256 * U + threadIdx.x; g0 < total; g0 += gridDim.x * 256 * U) {
+            uint4 v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (g0 + u * 256 < total) v[u] = src[g0 + u * 256];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (g0 + u * 256 < total) dst[g0 + u * 256] = v[u];
+        }
+    }
+    int32_t* keep = keep_idx + (size_t)layer * S_cur;
+    const int part = (which * Hkv + head) * gridDim.x + blockIdx.x, parts = 2 * Hkv * gridDim.x;
+    for (int i = part * 256 + threadIdx.x; i < n; i += parts * 256) keep[i] = layer < l1 || i < vis_start ? i : i + n_vis;
+    if (part == 0 && threadIdx.x == 0) {
+        keep_len[layer] = n;
+        new_len[layer] = n;
+        if (layer == 0) *status = METOK_OK;
+    }
+}
+
 // GIVEN policy: the caller's lists are checked before anything is indexed through them.  One CTA
 // per layer reads only the list itself: 0 <= length <= S_cur, entries strictly ascending inside
 // [0, S_cur).  valid[layer] says whether the layer may be compacted; a layer with a bad list is
@@ -64,6 +102,7 @@ kv_paper_lists_kernel(int S_cur, int vis_start, int n_vis, int l1, int32_t* __re
 __global__ void __launch_bounds__(256)
 kv_check_lists_kernel(int S_cur, const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ keep_len,
                       int32_t* __restrict__ new_len, int32_t* __restrict__ valid) {
+    grid_dep_wait();
     __shared__ int s_bad;
     const int layer = blockIdx.x;
     const int n = keep_len[layer];
@@ -210,6 +249,7 @@ __global__ void __cluster_dims__(kKvCluster, 1, 1) __launch_bounds__(kKvThreads)
 kv_gather_kernel(KvPtrs ptrs, int layer0, int Hkv, int S_cap, int S_cur, int row_chunks,
                  const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ keep_len,
                  const int32_t* __restrict__ haz) {
+    grid_dep_wait();
     cg::cluster_group cluster = cg::this_cluster();
     const int crank = (int)cluster.block_rank();
     const int slab = blockIdx.x / kKvCluster;            // (layer_local, which, head)
@@ -287,6 +327,15 @@ static KvWs carve_kv(Carver& cv, int L, int Hkv, int S_cur, int row_chunks) {
     return w;
 }
 
+static KvPtrs kv_ptrs(void* const* k_layers, void* const* v_layers, int l0, int nl) {
+    KvPtrs p;
+    for (int l = 0; l < kKvMaxLayersPerLaunch; ++l) {
+        p.k[l] = l < nl ? k_layers[l0 + l] : nullptr;
+        p.v[l] = l < nl ? v_layers[l0 + l] : nullptr;
+    }
+    return p;
+}
+
 }  // namespace metok
 
 using namespace metok;
@@ -332,10 +381,27 @@ extern "C" int metok_kv_compact(void* const* k_layers, void* const* v_layers, in
     // (-1: not known); lists that keep all rows cause no copying
     int kept_bound = -1;
     if (policy == METOK_KV_PAPER) {
+        if (S_cur - (vis_start + n_vis) <= n_vis) {                // one kernel: nothing moves into a row that is still to be read
+            for (int l0 = 0; l0 < L; l0 += kKvMaxLayersPerLaunch) {
+                const int nl = (L - l0) < kKvMaxLayersPerLaunch ? (L - l0) : kKvMaxLayersPerLaunch;
+                const KvPtrs ptrs = kv_ptrs(k_layers, v_layers, l0, nl);
+                const int slabs = nl * 2 * Hkv;
+                // a CTA per 1024 chunks of a slab, up to eight CTAs per SM
+                const long long want = ((long long)(S_cur - vis_start - n_vis) * row_chunks + 1023) / 1024, room = 8 * kNumSMs / slabs;
+                const int split = (int)(want < 1 || room < 1 ? 1 : want < room ? want : room);
+                {
+                    METOK_TIMED("kv_paper_kernel", st);
+                    launch_chained(kv_paper_kernel, dim3(split, slabs), dim3(256), 0, st, ptrs, l0, Hkv, S_cap, S_cur, row_chunks,
+                                   vis_start, n_vis, l1, keep_idx, keep_len, new_len, w.status);
+                }
+                METOK_LAUNCH_CHECK();
+            }
+            return METOK_OK;
+        }
         kept_bound = S_cur - n_vis;
         {
             METOK_TIMED("kv_paper_lists_kernel", st);
-            kv_paper_lists_kernel<<<L, 256, 0, st>>>(S_cur, vis_start, n_vis, l1, keep_idx, keep_len, new_len);
+            launch_chained(kv_paper_lists_kernel, dim3(L), dim3(256), 0, st, S_cur, vis_start, n_vis, l1, keep_idx, keep_len, new_len);
         }
         METOK_LAUNCH_CHECK();
     } else if (policy == METOK_KV_TOPK) {
@@ -351,18 +417,14 @@ extern "C" int metok_kv_compact(void* const* k_layers, void* const* v_layers, in
     } else {
         {
             METOK_TIMED("kv_check_lists_kernel", st);
-            kv_check_lists_kernel<<<L, 256, 0, st>>>(S_cur, keep_idx, keep_len, new_len, w.valid);
+            launch_chained(kv_check_lists_kernel, dim3(L), dim3(256), 0, st, S_cur, keep_idx, keep_len, new_len, w.valid);
         }
         METOK_LAUNCH_CHECK();
     }
     const int32_t* valid = policy == METOK_KV_GIVEN ? w.valid : nullptr;
     for (int l0 = 0; l0 < L; l0 += kKvMaxLayersPerLaunch) {
         const int nl = (L - l0) < kKvMaxLayersPerLaunch ? (L - l0) : kKvMaxLayersPerLaunch;
-        KvPtrs ptrs;
-        for (int l = 0; l < kKvMaxLayersPerLaunch; ++l) {
-            ptrs.k[l] = l < nl ? k_layers[l0 + l] : nullptr;
-            ptrs.v[l] = l < nl ? v_layers[l0 + l] : nullptr;
-        }
+        const KvPtrs ptrs = kv_ptrs(k_layers, v_layers, l0, nl);
         const int slabs = nl * 2 * Hkv;
         {
             METOK_TIMED("kv_stage_kernel", st);
@@ -381,7 +443,7 @@ extern "C" int metok_kv_compact(void* const* k_layers, void* const* v_layers, in
         if (kept_bound < 0 || kept_bound > w.stage_rows) {
             {
                 METOK_TIMED("kv_gather_kernel", st);
-                kv_gather_kernel<<<slabs * kKvCluster, kKvThreads, 0, st>>>(ptrs, l0, Hkv, S_cap, S_cur, row_chunks,
+                launch_chained(kv_gather_kernel, dim3(slabs * kKvCluster), dim3(kKvThreads), 0, st, ptrs, l0, Hkv, S_cap, S_cur, row_chunks,
                                                                         keep_idx, keep_len, w.haz);
             }
             METOK_LAUNCH_CHECK();

@@ -16,7 +16,7 @@ namespace metok {
 // token_score[j] = <x_j, t> / (max(|x_j|, eps) * max(|t|, eps)); also 1/max(|x_j|, eps).
 // One warp per token row, 16-byte loads, eight chunks of the row in flight per lane.  The text's chunks are read
 // beside them (they stay in L1), so a CTA has nothing to prepare: with the text laid out in shared memory first, a
-// CTA of 64 rows x 196 tokens x 1152 spent more time on that than on its rows (11.5 us; MEASURED_TS now).
+// CTA of 64 rows x 196 tokens x 1152 spent more time on that than on its rows (11.5 us; 8.4 now).
 // --------------------------------------------------------------------------- //
 template <typename T>
 __device__ __forceinline__ void widen_chunk(const uint4& r, float (&v)[16 / sizeof(T)]) {
@@ -93,7 +93,7 @@ __device__ __forceinline__ int find_event(const int32_t* __restrict__ off, int k
 }
 
 // Event scores, key events, per-event token budgets and output offsets.  One CTA; with many frames a cluster, whose
-// other CTAs only average frames for it (512 frames: 13.4 us with one CTA, MEASURED_EP with four).
+// other CTAs only average frames for it (512 frames: 13.4 us with one CTA, 6.5 with four).
 struct PlanParams {
     int Tn, N, k, n_key_events, event_agg, mode, tile_rows, chunk_cols;
     int rows_with_keys;                         // the merge's row tiles run over all tokens of an event (1) or only over those that are no key token (0)
@@ -306,7 +306,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
 // order in fp32, divided by their number and rounded once.  A CTA takes a share of a frame's (window, chunk) pairs, so
 // the frame's stride and offset are looked up once, every load is one of consecutive 16-byte chunks, and what is in
 // flight is four loads of every thread of the chip.  (A CTA per window, two rows in flight, at 128 registers: 40 us
-// for 64 frames of 196 tokens of 1152; MEASURED_PO now.)
+// for 64 frames of 196 tokens of 1152; about 9 now.)
 // --------------------------------------------------------------------------- //
 constexpr int kPoolThreads = 256;
 

@@ -1,0 +1,90 @@
+"""Branches that depend on sizes, at the sizes where they change: the finishing step of the segmentation (lanes per frame),
+the frame averages of the event plan (one CTA or a cluster), the paper's K/V rule (one kernel as long as no more rows
+follow the visual span than it holds), and member lists around the sizes at which averaging changes its way."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import metok_oracle as O
+from paper_2506_02850_b200 import binding as B
+
+from . import runners as R
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 5, 127, 128, 129, 131, 256, 257, 511, 512, 513, 1025, 2050])
+def test_segmentation_finish_and_event_plan_at_their_edges(T):
+    rng = np.random.default_rng(T)
+    N, d = 9, 16
+    V = rng.standard_normal((T, N, d)).astype(np.float32)
+    if T > 8:
+        V[T // 2] = V[T // 2 - 1]                                       # equal similarities: ties go to the lower index
+        V[T // 2 + 1] = V[T // 2 - 1]
+    t = rng.standard_normal(d).astype(np.float32)
+    V += 0.5 * t                                                        # scores away from zero
+    for k in sorted({1, min(T, 2), max(1, T // 3), T}):
+        R.segment_case(V, "f32", k)
+        offs = np.sort(rng.choice(np.arange(1, T), size=k - 1, replace=False)) if k > 1 else np.zeros(0, np.int64)
+        offs = np.concatenate([[0], offs, [T]]).astype(np.int32)
+        R.compress_case(V, t, offs, "f32", 0.5, 0.3, 0.2, check_features=False)
+        R.pool_case(V, t, offs, "f32", 0.5, 0.4, (2, 3, 1, 5))
+
+
+@pytest.mark.parametrize("L,S_vis,vis_start,tail,l1", [
+    (3, 40, 0, 0, 1), (3, 40, 5, 40, 0), (3, 40, 5, 41, 0), (3, 40, 0, 39, 3), (70, 33, 3, 7, 65), (2, 0, 4, 9, 0), (2, 600, 1, 260, 1),
+])
+@pytest.mark.parametrize("dh,dtype", [(64, torch.bfloat16), (24, torch.float32)])
+def test_kv_paper_rule_in_place(L, S_vis, vis_start, tail, l1, dh, dtype):
+    S = vis_start + S_vis + tail
+    Hkv, S_cap = 2, S + 3
+    g = torch.Generator(device="cuda").manual_seed(S + L)
+    ks = [torch.randn((Hkv, S_cap, dh), device="cuda", generator=g).to(dtype) for _ in range(L)]
+    vs = [torch.randn((Hkv, S_cap, dh), device="cuda", generator=g).to(dtype) for _ in range(L)]
+    old = [x.clone() for x in ks + vs]
+    got = B.metok_kv_compact(ks, vs, S, B.KV_PAPER, vis_start, S_vis, l1=l1)
+    torch.cuda.synchronize()
+    want = O.kv_select(O.KV_PAPER, L, S, vis_start, S_vis, l1=l1)
+    assert int(got["status"].item()) == 0
+    for layer in range(L):
+        n = len(want[layer])
+        assert int(got["new_len"][layer].item()) == n == int(got["keep_len"][layer].item())
+        assert np.array_equal(got["keep_idx"][layer, :n].cpu().numpy(), want[layer])
+        idx = torch.from_numpy(np.asarray(want[layer], dtype=np.int64)).cuda()
+        for x, o in ((ks[layer], old[layer]), (vs[layer], old[L + layer])):
+            assert torch.equal(x[:, :n], o[:, idx])
+
+
+@pytest.mark.parametrize("count", [15, 16, 17, 18, 127, 128, 129, 130, 300, 700])
+@pytest.mark.parametrize("d,dtype", [(8, torch.bfloat16), (520, torch.bfloat16), (1032, torch.bfloat16), (260, torch.float32)])
+def test_averages_of_chosen_member_counts(count, d, dtype):
+    """One event, three key tokens, `count` tokens that are closest to the second: the means in token order."""
+    rng = np.random.default_rng(count + d)
+    base = np.eye(3, d) * 4.0 + 0.5
+    who = np.array([0, 1, 2] + [1] * (count - 1))
+    rng.shuffle(who)
+    V = base[who] + 0.05 * rng.standard_normal((who.size, d))
+    first = [int(np.nonzero(who == i)[0][0]) for i in range(3)]
+    V[first] *= 1.5
+    t = V[first].sum(0) / np.linalg.norm(V[first].sum(0))               # the three are not the best scored by themselves:
+    Vd = torch.from_numpy(V.astype(np.float32)).to(dtype).cuda()[None]   # their scores are handed over
+    td = torch.from_numpy(t.astype(np.float32)).to(dtype).cuda()
+    score = torch.zeros(who.size, device="cuda")
+    score[first] = torch.tensor([3.0, 2.0, 1.0], device="cuda")
+    inv = 1.0 / Vd[0].float().norm(dim=1)
+    got = B.metok_compress_vision(Vd, torch.tensor([0, 1], dtype=torch.int32, device="cuda"), td,
+                                  B.vision_params(1.0, 3.0 / who.size, 3.0 / who.size),
+                                  scored={"token_score": score, "token_inv_norm": inv})
+    torch.cuda.synchronize()
+    assert int(got["n_out"].item()) == 3 and int(got["status"].item()) == 0
+    assert got["out_src"][:3].tolist() == sorted(first)
+    slot_of = {int(who[s]): i for i, s in enumerate(sorted(first))}
+    want_assign = np.array([slot_of[int(w)] for w in who])
+    assert np.array_equal(got["assign"].cpu().numpy(), want_assign)
+    x = Vd[0].double().cpu().numpy()
+    for i in range(3):
+        mean = x[want_assign == i].mean(0)
+        assert int(got["out_members"][i].item()) == int((want_assign == i).sum())
+        out = got["out_feats"][i].double().cpu().numpy()
+        assert np.linalg.norm(out - mean) <= (5e-3 if dtype == torch.bfloat16 else 1e-5) * np.linalg.norm(mean)
