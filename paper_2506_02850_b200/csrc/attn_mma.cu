@@ -16,9 +16,14 @@
 //            too.  Only key tiles that touch the visual span are visited.
 //
 // Warp roles in both: warp 0 = TMA producer, warp 1 = MMA issuer (one elected lane),
-// the others = epilogue: four (stats) or two (colsum) warps per TMEM lane quadrant, each
-// taking a quarter or half of the columns.  Two accumulators in TMEM (2 x 256 columns) so
+// the others = epilogue: four warps per TMEM lane quadrant, each taking a quarter of the
+// columns.  Two accumulators in TMEM (2 x 256 columns) so
 // that the epilogue of tile i overlaps the MMA of tile i+1.  Every wait is bounded.
+//
+// What bounds both is the exponentials and what goes with them: 16 a clock on an SM's special-function units, so every
+// fourth pair is taken on the FMA pipe, the multiply-adds and sums are done two at a time (half the issue slots), stats
+// takes no maximum after its first tile, and a warp empties its part of the accumulator before the arithmetic, so that
+// the next product never waits for it.  28 heads, 128 queries, 73 856 keys of 128: stats 85 -> 74 us, colsum 91 -> 80.
 #include "common.cuh"
 #include "launchers.h"
 #include "sm100.cuh"
@@ -27,18 +32,17 @@ namespace metok {
 
 namespace {
 
-constexpr int kAmThreads = 320;
-constexpr int kAmEpiWarps = 8;
-constexpr int kStEpiWarps = 16;           // stats: four warps per TMEM lane quadrant, 64 columns of a tile each
-constexpr int kStThreads = 64 + kStEpiWarps * 32;
+constexpr int kEpiWarps = 16;             // four warps per TMEM lane quadrant, a quarter of a tile's columns each
+constexpr int kThreads = 64 + kEpiWarps * 32;
 constexpr float kLog2e = 1.4426950408889634f;
+template <int V> struct Int { static constexpr int value = V; };
 constexpr float kNegInf = -3.0e38f;       // finite stand-in: keeps (m_old - m_new) free of inf - inf
 
 constexpr int kStBM = 128;                // stats: query rows per CTA
 constexpr int kStBN = 256;                // stats: keys per tile
 constexpr int kStStages = 2;
 constexpr int kCsBM = 128;                // colsum: keys per tile
-constexpr int kCsMaxNQ = 256;             // colsum: query rows per chunk (multiple of 16)
+constexpr int kCsMaxNQ = 256;             // colsum: query rows per chunk (multiple of 32)
 constexpr int kCsStages = 4;
 constexpr int kStMinTiles = 2;            // fewest key tiles a stats CTA is started for
 constexpr int kCsMinTiles = 3;            // the same for colsum
@@ -67,7 +71,7 @@ __host__ AttnMmaDims make_mma_dims(int Hq, int Hkv, int Lt, int S, int vis_start
     dm.st_per = ceil_div(dm.st_tiles, ns);
     dm.st_nsplit = ceil_div(dm.st_tiles, dm.st_per);   // every split owns at least one tile
     dm.cs_nchunk = ceil_div(dm.R, kCsMaxNQ);
-    dm.cs_nq = ceil_div(ceil_div(dm.R, dm.cs_nchunk), 16) * 16;
+    dm.cs_nq = ceil_div(ceil_div(dm.R, dm.cs_nchunk), 32) * 32;       // quarters of whole 8-column groups
     dm.cs_t0 = vis_start / kCsBM;
     dm.cs_tiles = (vis_start + n_vis - 1) / kCsBM - dm.cs_t0 + 1;
     ns = kNumSMs / (Hkv * dm.cs_nchunk);
@@ -79,11 +83,27 @@ __host__ AttnMmaDims make_mma_dims(int Hq, int Hkv, int Lt, int S, int vis_start
     return dm;
 }
 
+// Sum of 2^(v[j] * sc + add) over the 32 columns; every fourth pair's exponentials on the FMA pipe.
+__device__ __forceinline__ float exp2_sum32(const uint32_t (&v)[32], uint64_t sc, uint64_t add) {
+    using namespace sm100;
+    uint64_t s0 = 0ull, s1 = 0ull;                             // {0.f, 0.f}
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        const uint64_t x = fma_pair(pair(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), sc, add);
+        const uint64_t e = (j & 3) == 3 ? exp2_fma_pair(x) : exp2_pair(x);
+        if (j & 1) s1 = add_pair(s1, e);
+        else s0 = add_pair(s0, e);
+    }
+    float a, b;
+    unpair(add_pair(s0, s1), a, b);
+    return a + b;
+}
+
 // --------------------------------------------------------------------------- //
 // stats
 // --------------------------------------------------------------------------- //
 template <int DH>
-__global__ void __launch_bounds__(kStThreads, 1)
+__global__ void __launch_bounds__(kThreads, 1)
 attn_stats_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                       AttnMmaDims dm, float* __restrict__ part_m, float* __restrict__ part_l,
                       int32_t* __restrict__ status) {
@@ -117,7 +137,7 @@ attn_stats_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         mbar_init(smem_u32(&q_bar), 1);
         mbar_init(smem_u32(&drain_bar), 1);
         for (int s = 0; s < kStStages; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&tfull_bar[b]), 1); mbar_init(smem_u32(&tempty_bar[b]), kStEpiWarps); }
+        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&tfull_bar[b]), 1); mbar_init(smem_u32(&tempty_bar[b]), kEpiWarps); }
         s_abort = 0;
         mbar_fence_init();
     }
@@ -205,60 +225,64 @@ attn_stats_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             const bool masked = u_tile + kStBN - 1 > text_start;       // some query cannot see some key of the tile
             uint32_t raw[2][32];
             tmem_ld32_issue(taddr, raw[0]);
-#pragma unroll
-            for (int ci = 0; ci < kStBN / 128; ++ci) {
-                // the next 32 columns are fetched while these are reduced
-                const int c0 = ci * 32;
-                tmem_ld32_wait(raw[ci & 1]);
-                if (ci + 1 < kStBN / 128) tmem_ld32_issue(taddr + (uint32_t)(c0 + 32), raw[(ci + 1) & 1]);
-                float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(raw[ci & 1][j]);
-                float a0 = 0.f, a1 = 0.f;
-                float m_new;
-                if (masked) {                                  // hidden keys add exactly nothing
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = (u0 + c0 + j <= limit) ? v[j] * sc : kNegInf;
-                    float cm = v[0];
-#pragma unroll
-                    for (int j = 1; j < 32; ++j) cm = fmaxf(cm, v[j]);
-                    m_new = fmaxf(m_run, cm);
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) a0 += (v[j] > kNegInf) ? fast_exp2(v[j] - m_new) : 0.f;
-                } else {
-                    // the scale is positive: the maximum of the raw logits, scaled, is the maximum of the
-                    // scaled ones, and scaling folds into the exponent's multiply-add
-                    float t16[16];                             // a tree: the maximum is five steps deep, not 31
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) t16[j] = fmaxf(v[2 * j], v[2 * j + 1]);
-#pragma unroll
-                    for (int w = 8; w >= 1; w >>= 1) {
-#pragma unroll
-                        for (int j = 0; j < w; ++j) t16[j] = fmaxf(t16[j], t16[j + w]);
-                    }
-                    const float cm = t16[0];
-                    m_new = fmaxf(m_run, cm * sc);
-                    const float neg_m = -m_new;
-#pragma unroll
-                    for (int j = 0; j < 32; j += 4) {           // every fourth exponential on the FMA pipe
-                        a0 += fast_exp2(fmaf(v[j], sc, neg_m));
-                        a1 += fast_exp2(fmaf(v[j + 1], sc, neg_m));
-                        a0 += fast_exp2(fmaf(v[j + 2], sc, neg_m));
-                        a1 += exp2_fma(fmaf(v[j + 3], sc, neg_m));
-                    }
-                }
-                l_run = l_run * fast_exp2(m_run - m_new) + (a0 + a1);
-                m_run = m_new;
-            }
-            tc_fence_before();
+            // A row's (m_run, l_run) stands for l_run * 2^m_run, and any reference m_run that its logits do not exceed by
+            // the exponent range will do: the first tile's maximum stays, later tiles only add 2^(logit - m_run), with no
+            // maximum taken.  A chunk whose sum leaves the range (a logit 60 octaves above the reference) is done again
+            // against its own maximum.
+            const bool plain = !masked && it > 0;
+            tmem_ld32_issue(taddr + 32u, raw[1]);
+            tmem_ld32_wait(raw[0]);
+            tmem_ld32_wait(raw[1]);
+            tc_fence_before();                                 // the accumulator is free before the arithmetic
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&tempty_bar[b]));
+#pragma unroll
+            for (int ci = 0; ci < kStBN / 128; ++ci) {
+                const int c0 = ci * 32;
+                bool redo = !plain;
+                if (plain) {
+                    const float sum = exp2_sum32(raw[ci & 1], pair(sc, sc), pair(-m_run, -m_run));
+                    redo = __any_sync(0xFFFFFFFFu, !(sum < 1.0e18f));
+                    if (!redo) l_run += sum;
+                }
+                if (redo) {
+                    float v[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(raw[ci & 1][j]);
+                    float sum = 0.f;
+                    float m_new;
+                    if (masked) {                              // hidden keys add exactly nothing
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] = (u0 + c0 + j <= limit) ? v[j] * sc : kNegInf;
+                        float cm = v[0];
+#pragma unroll
+                        for (int j = 1; j < 32; ++j) cm = fmaxf(cm, v[j]);
+                        m_new = fmaxf(m_run, cm);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) sum += (v[j] > kNegInf) ? fast_exp2(v[j] - m_new) : 0.f;
+                    } else {
+                        // the scale is positive: the maximum of the raw logits, scaled, is the maximum of the scaled ones
+                        float t16[16];                         // a tree: the maximum is five steps deep, not 31
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) t16[j] = fmaxf(v[2 * j], v[2 * j + 1]);
+#pragma unroll
+                        for (int w = 8; w >= 1; w >>= 1) {
+#pragma unroll
+                            for (int j = 0; j < w; ++j) t16[j] = fmaxf(t16[j], t16[j + w]);
+                        }
+                        m_new = fmaxf(m_run, t16[0] * sc);
+                        sum = exp2_sum32(raw[ci & 1], pair(sc, sc), pair(-m_new, -m_new));
+                    }
+                    l_run = l_run * fast_exp2(m_run - m_new) + sum;
+                    m_run = m_new;
+                }
+            }
         }
         // the four column quarters of a row are merged here, in quarter order: one pair per row and split
         const int rl = quad * 32 + lane;
         s_pm[part][rl] = m_run;
         s_pl[part][rl] = l_run;
-        asm volatile("bar.sync 1, %0;" ::"n"(kStEpiWarps * 32) : "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
         if (part == 0 && ok && valid) {
             float M = s_pm[0][rl];
 #pragma unroll
@@ -281,7 +305,7 @@ attn_stats_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 // colsum
 // --------------------------------------------------------------------------- //
 template <int DH>
-__global__ void __launch_bounds__(kAmThreads, 1)
+__global__ void __launch_bounds__(kThreads, 1)
 attn_colsum_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                        AttnMmaDims dm, const float* __restrict__ part_m, const float* __restrict__ part_l,
                        float* __restrict__ part_col, int32_t* __restrict__ status) {
@@ -295,6 +319,8 @@ attn_colsum_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         tempty_bar[2];
     __shared__ uint32_t s_tmem_base;
     __shared__ int s_abort;
+    __shared__ float s_part[4][3][kCsBM];                      // sums of the column quarters 1 to 3 per key, of four tiles
+    __shared__ __align__(8) uint64_t part_bar[4][4];           // [tile % 4][lane quadrant]: its three warps have written them
     __shared__ __align__(16) float s_nlse[kCsMaxNQ];           // -(log-sum-exp) per query row of the chunk, log2 units
 
     const int split = blockIdx.x, chunk = blockIdx.y, g = blockIdx.z;
@@ -313,8 +339,12 @@ attn_colsum_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         mbar_init(smem_u32(&q_bar), 1);
         mbar_init(smem_u32(&drain_bar), 1);
         for (int s = 0; s < kCsStages; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&tfull_bar[b]), 1); mbar_init(smem_u32(&tempty_bar[b]), kAmEpiWarps); }
+        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&tfull_bar[b]), 1); mbar_init(smem_u32(&tempty_bar[b]), kEpiWarps); }
         s_abort = 0;
+        mbar_fence_init();
+    }
+    if (warp == 2 && lane < 16) {
+        mbar_init(smem_u32(&part_bar[lane >> 2][lane & 3]), 3);
         mbar_fence_init();
     }
     if (warp == 1) {
@@ -380,84 +410,112 @@ attn_colsum_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         }
     } else {
         // The epilogue warps first turn the key-split partials into the log-sum-exp of the chunk's
-        // query rows, one row per thread, while the producer's first copies and the first MMA are
-        // already under way; nobody else reads s_nlse, so a barrier among these 256 threads is enough.
+        // query rows, two threads per row, while the producer's first copies and the first MMA are
+        // already under way; nobody else reads s_nlse, so a barrier among these threads is enough.
         {
-            const int c = threadIdx.x - 64;                    // 0 .. kCsMaxNQ - 1
+            static_assert(kEpiWarps * 32 == 2 * kCsMaxNQ, "two threads per row");
+            const int c = (threadIdx.x - 64) >> 1, odd = threadIdx.x & 1;   // two threads per row: its even and its odd splits
             const int r = chunk * NQ + c;
-            float nl = kNegInf;                                // rows past R contribute exp2(x - 3e38) = 0
-            if (c < NQ && r < dm.R) {
-                const int ns2 = dm.st_nsplit;                  // one (max, sum) pair per key split
-                const float* pm = part_m + (size_t)g * ns2 * dm.R + r;
-                const float* pl = part_l + (size_t)g * ns2 * dm.R + r;
-                float M = kNegInf, Z = 0.f;                    // running maximum and sum, partials in order
-                for (int s0 = 0; s0 < ns2; s0 += 8) {
-                    float m8[8], l8[8];
+            const bool row = c < NQ && r < dm.R;
+            const int ns2 = row ? dm.st_nsplit : 0;            // one (max, sum) pair per key split
+            const float* pm = part_m + (size_t)g * dm.st_nsplit * dm.R + r;
+            const float* pl = part_l + (size_t)g * dm.st_nsplit * dm.R + r;
+            float M = kNegInf, Z = 0.f;                        // running maximum and sum, partials in order
+            for (int s0 = odd; s0 < ns2; s0 += 16) {
+                float m8[8], l8[8];
 #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const bool in = s0 + u < ns2;
-                        m8[u] = in ? pm[(size_t)(s0 + u) * dm.R] : kNegInf;
-                        l8[u] = in ? pl[(size_t)(s0 + u) * dm.R] : 0.f;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const float Mn = fmaxf(M, m8[u]);
-                        Z = Z * exp2f(M - Mn) + l8[u] * exp2f(m8[u] - Mn);
-                        M = Mn;
-                    }
+                for (int u = 0; u < 8; ++u) {
+                    const bool in = s0 + 2 * u < ns2;
+                    m8[u] = in ? pm[(size_t)(s0 + 2 * u) * dm.R] : kNegInf;
+                    l8[u] = in ? pl[(size_t)(s0 + 2 * u) * dm.R] : 0.f;
                 }
-                nl = -(M + log2f(Z));
+                float Mn = M;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) Mn = fmaxf(Mn, m8[u]);
+                Z *= exp2f(M - Mn);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) Z += l8[u] * exp2f(m8[u] - Mn);
+                M = Mn;
             }
-            s_nlse[c] = nl;
-            asm volatile("bar.sync 1, 256;" ::: "memory");
+            const float Mo = __shfl_xor_sync(0xFFFFFFFFu, M, 1), Zo = __shfl_xor_sync(0xFFFFFFFFu, Z, 1);
+            const float Mn = fmaxf(M, Mo);
+            const float ze = odd ? Zo : Z, me = odd ? Mo : M, zo = odd ? Z : Zo, mo = odd ? M : Mo;
+            Z = ze * exp2f(me - Mn) + zo * exp2f(mo - Mn);
+            // rows past R contribute exp2(x - 3e38) = 0
+            if (!odd) s_nlse[c] = row ? -(Mn + log2f(Z)) : kNegInf;
+            asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
         }
         const int quad = warp & 3;
-        const int half = (warp - 2) >> 2;
-        const int h0 = ((NQ / 16 + 1) / 2) * 16;               // first column of the second half
-        const int c_lo = half ? h0 : 0, c_hi = half ? NQ : h0;
+        const int part = (warp - 2) >> 2;                      // column quarter
+        const int width = NQ >> 2, c_lo = part * width;        // 8 .. 64 columns
         const float sc = dm.scale_log2;
+        const uint64_t sc2 = pair(sc, sc);
         const int vis_end = dm.vis_start + dm.n_vis;
-        float* plane = part_col + ((size_t)(g * dm.cs_nchunk + chunk) * 2 + half) * dm.n_vis;
+        float* plane = part_col + (size_t)(g * dm.cs_nchunk + chunk) * dm.n_vis;
         bool ok = true;
         for (int it = 0; it < nt; ++it) {
             const int b = it & 1;
             if (!mbar_wait(smem_u32(&tfull_bar[b]), (uint32_t)(it >> 1) & 1u, abort_flag)) ok = false;
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
-            tc_fence_after();
-            const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * kCsMaxNQ);
-            float a0 = 0.f, a1 = 0.f;
-            int c = c_lo;
-#pragma unroll 1
-            for (; c + 32 <= c_hi; c += 32) {
-                float v[32];
-                tmem_ld32(taddr + (uint32_t)c, v);
+            float sum;
+            {
+                tc_fence_after();
+                // the whole quarter into registers, so that the accumulator is free before the arithmetic (columns past
+                // the quarter are loaded too, and not used)
+                const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * kCsMaxNQ + c_lo);
+                uint32_t raw[2][32];
+                tmem_ld32_issue(taddr, raw[0]);
+                if (width > 32) tmem_ld32_issue(taddr + 32u, raw[1]);
+                tmem_ld32_wait(raw[0]);
+                tmem_ld32_wait(raw[1]);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&tempty_bar[b]));
+                uint64_t s0 = 0ull, s1 = 0ull;                 // {0.f, 0.f}
+                const float* nlse = &s_nlse[c_lo];
+                // the quarter's n columns, a constant in each case: no branch between them, so that their exponentials overlap
+                auto fold = [&](auto n_) {
+                    constexpr int n = decltype(n_)::value;
 #pragma unroll
-                for (int j = 0; j < 32; j += 4) {
-                    const float4 nl = *reinterpret_cast<const float4*>(&s_nlse[c + j]);
-                    a0 += fast_exp2(fmaf(v[j], sc, nl.x));
-                    a1 += fast_exp2(fmaf(v[j + 1], sc, nl.y));
-                    a0 += fast_exp2(fmaf(v[j + 2], sc, nl.z));
-                    a1 += exp2_fma(fmaf(v[j + 3], sc, nl.w));     // every fourth exponential on the FMA pipe
+                    for (int c = 0; c < n; c += 4) {
+                        const uint32_t* r = &raw[c >> 5][c & 31];
+                        const ulonglong2 nl = *reinterpret_cast<const ulonglong2*>(nlse + c);
+                        const uint64_t x0 = fma_pair(pair(__uint_as_float(r[0]), __uint_as_float(r[1])), sc2, nl.x);
+                        const uint64_t x1 = fma_pair(pair(__uint_as_float(r[2]), __uint_as_float(r[3])), sc2, nl.y);
+                        s0 = add_pair(s0, exp2_pair(x0));
+                        s1 = add_pair(s1, (c & 4) ? exp2_fma_pair(x1) : exp2_pair(x1));   // every fourth pair on the FMA pipe
+                    }
+                };
+                switch (width >> 3) {
+                    case 1: fold(Int<8>()); break;
+                    case 2: fold(Int<16>()); break;
+                    case 3: fold(Int<24>()); break;
+                    case 4: fold(Int<32>()); break;
+                    case 5: fold(Int<40>()); break;
+                    case 6: fold(Int<48>()); break;
+                    case 7: fold(Int<56>()); break;
+                    default: fold(Int<64>()); break;
                 }
+                float a0, a1;
+                unpair(add_pair(s0, s1), a0, a1);
+                sum = a0 + a1;
             }
-            if (c < c_hi) {                                    // halves are multiples of 16 columns
-                float v[16];
-                tmem_ld16(taddr + (uint32_t)c, v);
-#pragma unroll
-                for (int j = 0; j < 16; j += 4) {
-                    const float4 nl = *reinterpret_cast<const float4*>(&s_nlse[c + j]);
-                    a0 += fast_exp2(fmaf(v[j], sc, nl.x));
-                    a1 += fast_exp2(fmaf(v[j + 1], sc, nl.y));
-                    a0 += fast_exp2(fmaf(v[j + 2], sc, nl.z));
-                    a1 += exp2_fma(fmaf(v[j + 3], sc, nl.w));     // every fourth exponential on the FMA pipe
-                }
+            // The four quarters meet at the first one's warp, in quarter order.  Four buffers: whoever is at tile it + 4 has
+            // its accumulator from the first quarter's warps, which gave it back at tile it + 2, after tile it.  (A
+            // barrier of all 16 warps per tile put their loads and their arithmetic in step: 92 us at 73 728 keys.)
+            const int slot = it & 3, col = quad * 32 + lane;
+            const uint32_t pb = smem_u32(&part_bar[slot][quad]);
+            if (part > 0) {
+                s_part[slot][part - 1][col] = sum;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(pb);
+            } else {
+                if (ok && !mbar_wait(pb, (uint32_t)(it >> 2) & 1u, abort_flag)) ok = false;
+                const int u = (t_lo + it) * kCsBM + col;
+                if (ok && u >= dm.vis_start && u < vis_end)
+                    plane[u - dm.vis_start] = ((sum + s_part[slot][0][col]) + s_part[slot][1][col]) + s_part[slot][2][col];
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&tempty_bar[b]));
-            const int u = (t_lo + it) * kCsBM + quad * 32 + lane;
-            if (u >= dm.vis_start && u < vis_end) plane[u - dm.vis_start] = a0 + a1;
         }
     }
     tc_fence_before();
@@ -483,13 +541,13 @@ int launch_dh(const void* q_text, const void* k_all, const AttnMmaDims& dm, floa
     METOK_ALLOW_SMEM(attn_colsum_mma_kernel<DH>, ((size_t)KB * (kCsMaxNQ + kCsStages * kCsBM) * 128 + 1024));
     {
         METOK_TIMED("attn_stats_mma_kernel", st);
-        launch_chained(attn_stats_mma_kernel<DH>, dim3(dim3(dm.st_nsplit, dm.st_nrt, dm.Hkv)), dim3(kStThreads), smem_st, st, 
+        launch_chained(attn_stats_mma_kernel<DH>, dim3(dim3(dm.st_nsplit, dm.st_nrt, dm.Hkv)), dim3(kThreads), smem_st, st, 
             tmQs, tmKs, dm, part_m, part_l, status);
     }
     METOK_LAUNCH_CHECK();
     {
         METOK_TIMED("attn_colsum_mma_kernel", st);
-        launch_chained(attn_colsum_mma_kernel<DH>, dim3(dim3(dm.cs_nsplit, dm.cs_nchunk, dm.Hkv)), dim3(kAmThreads), smem_cs, st, 
+        launch_chained(attn_colsum_mma_kernel<DH>, dim3(dim3(dm.cs_nsplit, dm.cs_nchunk, dm.Hkv)), dim3(kThreads), smem_cs, st, 
             tmQc, tmKc, dm, part_m, part_l, part_col, status);
     }
     METOK_LAUNCH_CHECK();
@@ -502,7 +560,7 @@ void attn_mma_workspace(int Hq, int Hkv, int Lt, int S, int n_vis, size_t* n_par
                         int* n_planes) {
     const AttnMmaDims dm = make_mma_dims(Hq, Hkv, Lt, S, 0, n_vis, 1.f);
     *n_part_ml = (size_t)Hkv * dm.st_nsplit * 2 * dm.R;
-    *n_planes = Hkv * dm.cs_nchunk * 2;
+    *n_planes = Hkv * dm.cs_nchunk;
     *n_part_col = (size_t)(*n_planes) * n_vis;
 }
 

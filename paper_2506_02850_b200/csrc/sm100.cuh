@@ -200,28 +200,13 @@ __device__ __forceinline__ void tmem_ld32_wait(uint32_t (&r)[32]) {
         : "memory");
 }
 
-// 16 consecutive fp32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // 2^x on the special-function unit (about 2 ulp; results below 2^-126 flush to zero).
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// 2^x for x <= 0 on the FMA pipe instead of the special-function unit: round x to an integer with
+// 2^x for x < 127 on the FMA pipe instead of the special-function unit: round x to an integer with
 // the 1.5 * 2^23 trick, a degree-5 polynomial for 2^f on f in [-0.5, 0.5] (relative error 2e-7, that
 // of ex2.approx), and the integer added to the exponent.  Used for a share of an epilogue's
 // exponentials so that both pipes work.
@@ -236,6 +221,48 @@ __device__ __forceinline__ float exp2_fma(float x) {
     p = fmaf(p, f, 0.6931470036506653f);
     p = fmaf(p, f, 1.0f);
     return __int_as_float(__float_as_int(p) + (__float_as_int(t) << 23));
+}
+
+// ---- pairs of floats in 64-bit registers: one instruction for two multiply-adds or additions -------------------------
+// (the FMA pipe does them at the same rate per element; what a pair saves is the issue slot)
+__device__ __forceinline__ uint64_t pair(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpair(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma_pair(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_pair(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// 2^x of both halves on the special-function unit, and on the FMA pipe (exp2_fma).
+__device__ __forceinline__ uint64_t exp2_pair(uint64_t x) {
+    float a, b;
+    unpair(x, a, b);
+    return pair(fast_exp2(a), fast_exp2(b));
+}
+__device__ __forceinline__ uint64_t exp2_fma_pair(uint64_t x) {
+    float a, b;
+    unpair(x, a, b);
+    x = pair(fmaxf(a, -125.0f), fmaxf(b, -125.0f));
+    const uint64_t t = add_pair(x, pair(12582912.0f, 12582912.0f));
+    const uint64_t f = fma_pair(add_pair(t, pair(-12582912.0f, -12582912.0f)), pair(-1.0f, -1.0f), x);
+    uint64_t p = pair(0.001326472731307149f, 0.001326472731307149f);
+    p = fma_pair(p, f, pair(0.009671512991189957f, 0.009671512991189957f));
+    p = fma_pair(p, f, pair(0.05550733581185341f, 0.05550733581185341f));
+    p = fma_pair(p, f, pair(0.24022242426872253f, 0.24022242426872253f));
+    p = fma_pair(p, f, pair(0.6931470036506653f, 0.6931470036506653f));
+    p = fma_pair(p, f, pair(1.0f, 1.0f));
+    float p0, p1, t0, t1;
+    unpair(p, p0, p1);
+    unpair(t, t0, t1);
+    return pair(__int_as_float(__float_as_int(p0) + (__float_as_int(t0) << 23)), __int_as_float(__float_as_int(p1) + (__float_as_int(t1) << 23)));
 }
 
 // Shared-memory matrix descriptor of a K-major tile stored as rows of 128 bytes

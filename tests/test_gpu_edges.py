@@ -88,3 +88,26 @@ def test_averages_of_chosen_member_counts(count, d, dtype):
         assert int(got["out_members"][i].item()) == int((want_assign == i).sum())
         out = got["out_feats"][i].double().cpu().numpy()
         assert np.linalg.norm(out - mean) <= (5e-3 if dtype == torch.bfloat16 else 1e-5) * np.linalg.norm(mean)
+
+
+@pytest.mark.parametrize("Hq,Hkv,Lt,dh,n_vis,jump", [
+    (1, 1, 1, 64, 40, 0), (2, 1, 8, 64, 127, 0), (4, 2, 33, 128, 700, 0), (14, 2, 120, 64, 900, 0),   # one row up to several chunks of rows
+    (2, 1, 16, 128, 1500, 90), (1, 1, 9, 64, 3000, 300), (4, 4, 5, 128, 2600, 1000),                  # logits that leave the first tile's range
+])
+def test_attention_scores_whose_logits_grow_along_the_keys(Hq, Hkv, Lt, dh, n_vis, jump):
+    rng = np.random.default_rng(n_vis)
+    S = n_vis + Lt
+    u = rng.standard_normal(dh)
+    u /= np.linalg.norm(u)
+    Q = (0.3 * rng.standard_normal((Hq, Lt, dh)) + 4.0 * u).astype(np.float32)
+    K = (0.3 * rng.standard_normal((Hkv, S, dh))).astype(np.float32)
+    # `jump` octaves (in units of the exponent) between the first and the last visual keys, in three steps
+    step = np.floor(np.arange(S) * 3.0 / S) / 2.0
+    K += (jump * np.log(2.0) * dh ** 0.5 / 4.0 * step)[None, :, None].astype(np.float32) * u.astype(np.float32)
+    K[:, -Lt:] *= 0.0
+    Qb, Kb = (torch.from_numpy(x).to(torch.bfloat16) for x in (Q, K))
+    want = O.attention_scores(Qb.float().numpy(), Kb.float().numpy(), 0, n_vis, dh ** -0.5)
+    got = B.metok_attention_scores(Qb.cuda(), Kb.cuda(), 0, n_vis, dh ** -0.5)
+    torch.cuda.synchronize()
+    err = np.abs(got.double().cpu().numpy() - want).max() / want.max()
+    assert err < 2e-4, err
