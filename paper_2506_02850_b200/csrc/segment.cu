@@ -395,19 +395,16 @@ extern "C" int metok_segment_events(const void* feats, int dtype, int T, int N, 
 // flight) and the sums run on the tensor cores.  A warp owns one position and
 // EIGHT consecutive frames; a stage holds 512 contiguous bytes of those eight rows and
 // of the frame before them (one copy instruction per row, 16 bytes per lane: the memory
-// system sees long pieces of a row).  A stage is consumed as eight 64-byte slices.  Lane
-// (g, q) = (lane / 4, lane % 4) reads chunk q of frame g's
-// slice: the 16 bytes, as they lie in memory (dwords m0..m3), are the A operand of
-// m16n8k16 mma, which gives row g of A the k-slots (m0, m2) and row 8 + g the slots
-// (m1, m3).  The other vector is the B operand, whose two registers pair with (m0, m2)
-// in the upper half of C and with (m1, m3) in the lower half: with B = (y0, y2) the
-// diagonal element C[g][g] adds the products of the even dwords of frame g's slice, with
-// B = (y1, y3) C[8 + g][g] those of the odd dwords -- the order of k inside a dot product
-// is free as long as both operands use the same one.  Two mma per slice and vector pair,
-// accumulated over the slices of the row: at the end the lane that holds C[g][g] has the
-// complete sum of frame g, with no shuffle and no widening.  The previous frame's slice
-// is the same slice of the row before it in the stage.  Products of bf16 are exact in fp32 and
-// the sums are fp32; the off-diagonal entries are never read.
+// system sees long pieces of a row).  All three sums come out of one m16n8k16 mma per 16
+// elements: B is the eight frames (columns), A the same eight frames (rows 0-7), the text
+// (row 8) and the frame before the run (row 9; rows 10-15 repeat the text and are not
+// read).  C then holds the squared norms on its diagonal, the dots of neighbouring frames
+// next to it, <text, frame> in row 8 and the first frame's dot with its predecessor at
+// C[9][0].  One ldmatrix brings A as it is needed, and two of its four registers are B.
+// Products of bf16 are exact in fp32 and the sums are fp32 (two accumulators, even and
+// odd steps).  The kernel is meant to be bound by HBM; with a separate mma for each of the
+// three sums and each half of a 16-byte chunk (54 instructions per 64 bytes of a row, eight
+// warps an SM) it was bound by instruction latency: 512 x 144 rows of 1024 in 41 us.
 // --------------------------------------------------------------------------- //
 namespace metok {
 
@@ -514,6 +511,14 @@ __device__ __forceinline__ void mma_bf16_m16n8k16(float (&c)[4], const uint4& a,
         : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
+// Four 8 x 8 matrices of 16-bit elements; lane l names row l % 8 of matrix l / 8 (16 bytes).
+__device__ __forceinline__ uint4 ldmatrix_x4(uint32_t row) {
+    uint4 r;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(row) : "memory");
+    return r;
+}
+
 // 16-byte asynchronous copy global -> shared that bypasses L1; src_bytes = 0 writes zeros.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
@@ -522,15 +527,15 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+constexpr int kFsCtasPerSm = 2;                    // what the rings leave room for
 constexpr int kFsDepth = 4;                        // stages of a warp's ring
 constexpr int kFsFrames = 8;                       // frames per warp = row groups of the mma tile
 constexpr int kFsSlices = 8;                       // 64-byte slices of a row per stage: 512 contiguous bytes
-constexpr int kFsRowPitch = kFsSlices * 64 + 64;   // bytes between a stage's rows (see the bank note in the kernel)
+constexpr int kFsRowPitch = kFsSlices * 64 + 16;   // bytes between a stage's rows (see the bank note in the kernel)
 constexpr int kFsStageBytes = (kFsFrames + 1) * kFsRowPitch;
 
-// Shared memory: the text embedding as 16-byte chunks with the dwords in the order
-// (0, 2, 1, 3), zero-padded to whole slices; then per warp kFsDepth stages of nine rows
-// (512 bytes of frame f0 - 1, then of frames f0 .. f0 + 7).
+// Shared memory: the text embedding, zero-padded to whole slices; then per warp kFsDepth
+// stages of nine rows (512 bytes of frame f0 - 1, then of frames f0 .. f0 + 7).
 template <bool kFull>                               // kFull: the row is a whole number of 512-byte pieces
 __global__ void __launch_bounds__(kFsThreads)
 seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat16* __restrict__ text, int Tn, int N,
@@ -538,16 +543,84 @@ seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat1
                      float* __restrict__ token_score, float* __restrict__ inv_norm) {
     grid_dep_wait();
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    __shared__ float s_red[kFsThreads / 32];
+    constexpr int kFsWarps = kFsThreads / 32;
+    __shared__ float s_red[kFsWarps];
     __shared__ float s_tn;
+    __shared__ float s_nn[2][kFsWarps][kFsFrames], s_dp[2][kFsWarps][kFsFrames];   // alternate from unit to unit
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nchunk = d / 8;
     const int nslice = (nchunk + 3) >> 2;
+    const int nsuper = (nslice + kFsSlices - 1) / kFsSlices;
     uint4* s_text = reinterpret_cast<uint4*>(s_dyn);
+    // A unit is eight frames of four consecutive positions, one per warp: their norms and dots are added in the CTA
+    // (in warp order), so that seg_finish has a quarter of the partial sums to read.  Units run position first.
+    const int pgroups = (N + kFsWarps - 1) / kFsWarps;
+    const int nunits = pgroups * ((Tn + kFsFrames - 1) / kFsFrames);
+    const int g = lane >> 2, q = lane & 3;
+    const size_t frame_pitch = (size_t)N * nchunk;          // 16-byte chunks from a frame's row to the next frame's
+    // Copies: a stage holds 512 contiguous bytes (eight 64-byte slices) of each of the nine rows -- the
+    // frame before the run, then the run's eight frames.  One copy instruction moves a row's 512 bytes
+    // (16 per lane), so what reaches the memory system is long contiguous pieces of a row.  Rows of a
+    // stage lie kFsRowPitch bytes apart: 16 more than a multiple of 128, so that the eight rows of an
+    // 8 x 8 matrix lie in different banks.
+    unsigned char* ring = s_dyn + (size_t)nslice * 4 * sizeof(uint4) + (size_t)warp * kFsDepth * kFsStageBytes;
+    const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + (uint32_t)lane * 16u;
+    // ldmatrix: lanes 0-7 and 16-23 name the frames' rows (first and second 16 bytes of a step), lanes 9 and 25 the
+    // row of the frame before them, the other lanes the text
+    const bool on_text = (lane & 8) != 0 && (lane & 7) != 1;
+    const uint32_t ld_row = dst - (uint32_t)lane * 16u + (uint32_t)((lane & 8) ? 0 : (lane & 7) + 1) * kFsRowPitch + (uint32_t)(lane >> 4) * 16u;
+    const uint32_t ld_text = static_cast<uint32_t>(__cvta_generic_to_shared(s_text)) + (uint32_t)(lane >> 4) * 16u;
+    // the copies run kFsDepth - 1 pieces ahead of the sums, into the next units too
+    int i_unit = blockIdx.x, i_left = 0, i_lo = 0, i_hi = 0;
+    int i_chunk = lane;                                     // this lane's chunk of the next piece's rows
+    uint32_t i_stage = 0;
+    const uint4* i_src = nullptr;                           // that chunk of row i_lo, the first of the nine rows that exists
+    auto issue_unit = [&]() {
+        const int run = i_unit / pgroups;
+        // an idle warp repeats the last position and writes nothing
+        const int p = min((i_unit - run * pgroups) * kFsWarps + warp, N - 1);
+        const int f0 = run * kFsFrames;
+        i_lo = f0 == 0 ? 1 : 0;                             // row 0: the frame before the run
+        i_hi = min(kFsFrames + 1, Tn - f0 + 1);
+        i_left = nsuper;
+        i_chunk = lane;
+        i_src = reinterpret_cast<const uint4*>(feats) + ((size_t)(f0 - 1 + i_lo) * N + p) * (size_t)nchunk + lane;
+    };
+    auto issue = [&]() {                                    // one group per call
+        if (i_unit < nunits) {
+            const bool in = kFull || i_chunk < nchunk;
+            const uint4* src = in ? i_src : reinterpret_cast<const uint4*>(feats);
+            const size_t step = in ? frame_pitch : 0;
+            const uint32_t to = dst + i_stage;
+            if (i_hi - i_lo == kFsFrames + 1) {
+#pragma unroll
+                for (int r = 0; r <= kFsFrames; ++r, src += step) cp_async16(to + r * kFsRowPitch, src, in ? 16u : 0u);
+            } else {                                        // rows that do not exist are written as zeros (0 bytes read)
+#pragma unroll 1
+                for (int r = 0; r <= kFsFrames; ++r) {
+                    const bool ok = r >= i_lo && r < i_hi;
+                    cp_async16(to + r * kFsRowPitch, src, ok && in ? 16u : 0u);
+                    if (ok && r + 1 < i_hi) src += step;
+                }
+            }
+            i_stage = i_stage == (kFsDepth - 1) * kFsStageBytes ? 0u : i_stage + kFsStageBytes;
+            i_chunk += kFsSlices * 4;
+            i_src += kFsSlices * 4;
+            if (--i_left == 0) {
+                i_unit += gridDim.x;
+                if (i_unit < nunits) issue_unit();
+            }
+        }
+        cp_async_commit();
+    };
+    if (i_unit < nunits) issue_unit();
+#pragma unroll 1
+    for (int j = 0; j < kFsDepth - 1; ++j) issue();
+
     float a = 0.f;
     for (int c = tid; c < nslice * 4; c += kFsThreads) {
         const uint4 r = c < nchunk ? __ldg(reinterpret_cast<const uint4*>(text) + c) : make_uint4(0u, 0u, 0u, 0u);
-        s_text[c] = make_uint4(r.x, r.z, r.y, r.w);
+        s_text[c] = r;
         const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -561,110 +634,68 @@ seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat1
     __syncthreads();
     if (tid == 0) {
         float sum = 0.f;
-        for (int w = 0; w < kFsThreads / 32; ++w) sum += s_red[w];
+        for (int w = 0; w < kFsWarps; ++w) sum += s_red[w];
         s_tn = fmaxf(sqrtf(sum), kEps);
     }
     __syncthreads();
     const float tn = s_tn;
-    // the CTA owns eight frames and four consecutive positions, one per warp: their norms and dots are
-    // added here (in warp order), so that seg_finish has a quarter of the partial sums to read
-    constexpr int kFsWarps = kFsThreads / 32;
-    const int pgroups = (N + kFsWarps - 1) / kFsWarps;
-    const int run = blockIdx.x / pgroups, pg = blockIdx.x - run * pgroups;
-    const int p_raw = pg * kFsWarps + warp;
-    const bool has_p = p_raw < N;
-    const int p = has_p ? p_raw : N - 1;                    // an idle warp repeats the last position and writes nothing
-    const int f0 = run * kFsFrames;
-    const int g = lane >> 2, q = lane & 3;
-    const int f = f0 + g;                                   // this lane's frame
-    const bool has_f = f < Tn;
-    // Copies: a stage holds 512 contiguous bytes (eight 64-byte slices) of each of the nine rows -- the
-    // frame before the run, then the run's eight frames.  One copy instruction moves a row's 512 bytes
-    // (16 per lane), so what reaches the memory system is long contiguous pieces of a row.  Rows of a
-    // stage lie kFsRowPitch bytes apart: with 16 words more than a multiple of 32 the 16-byte reads of
-    // the eight lanes of a quarter warp (two frames, four chunks each) fall into different banks.
-    const uint4* row0 = reinterpret_cast<const uint4*>(feats) + ((size_t)max(f0 - 1, 0) * N + p) * (size_t)nchunk;
-    const size_t frame_pitch = (size_t)N * nchunk;          // 16-byte chunks from a frame's row to the next frame's
-    const int nsuper = (nslice + kFsSlices - 1) / kFsSlices;
-    unsigned char* ring = s_dyn + (size_t)nslice * 4 * sizeof(uint4) + (size_t)warp * kFsDepth * kFsStageBytes;
-    const unsigned char* mine = ring + (g + 1) * kFsRowPitch + q * 16;
-    const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + (uint32_t)lane * 16u;
-    const uint4* tq = s_text + q;
-    // 512-byte piece `sup` of the nine rows into stage `stage` (a constant where the caller is unrolled); one group per call
-    auto issue = [&](int sup, int stage) {
-        if (sup < nsuper) {
-            const int c = sup * 32 + lane;                  // this lane's chunk of every row
-            const bool in = c < nchunk;
-#pragma unroll
-            for (int r = 0; r <= kFsFrames; ++r) {
-                const int fr = f0 - 1 + r;                  // r = 0: the frame before the run
-                const bool ok = in && fr >= 0 && fr < Tn;
-                const uint4* src = ok ? row0 + (size_t)(fr - max(f0 - 1, 0)) * frame_pitch + c : row0;
-                cp_async16(dst + stage * kFsStageBytes + r * kFsRowPitch, src, ok ? 16u : 0u);   // 0 bytes read = zeros written
-            }
-        }
-        cp_async_commit();
-    };
-#pragma unroll
-    for (int j = 0; j < kFsDepth - 1; ++j) issue(j, j);
-    // accumulators: [0] pairs the even dwords (diagonal of the upper half), [1] the odd ones (lower half)
-    float cn[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-    float cp[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-    float ct[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+
+    uint32_t stage = 0;
+    int par = 0;
 #pragma unroll 1
-    for (int base = 0; base < nsuper; base += kFsDepth) {
+    for (int unit = blockIdx.x; unit < nunits; unit += gridDim.x, par ^= 1) {
+        const int run = unit / pgroups, pg = unit - run * pgroups;
+        const int p = pg * kFsWarps + warp;
+        const int f0 = run * kFsFrames;
+        const int f = f0 + g;                               // this lane's frame
+        const bool has = p < N && f < Tn;
+        float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};   // even and odd steps of 16 elements
+#pragma unroll 1
+        for (int sup = 0; sup < nsuper; ++sup) {
+            cp_async_wait<kFsDepth - 2>();                  // this lane's copies of the piece have landed
+            __syncwarp();                                   // ... and every lane's; the piece before it has been read by all
+            issue();                                        // into the stage that held the piece before
+            const uint32_t at = on_text ? ld_text + (uint32_t)sup * (kFsSlices * 64u) : ld_row + stage;
+            stage = stage == (kFsDepth - 1) * kFsStageBytes ? 0u : stage + kFsStageBytes;
 #pragma unroll
-        for (int j = 0; j < kFsDepth; ++j) {
-            const int sup = base + j;
-            if (sup < nsuper) {                             // the same for the whole warp
-                cp_async_wait<kFsDepth - 2>();              // this lane's copies of the piece have landed
-                __syncwarp();                               // ... and every lane's; the piece before it has been read by all
-                issue(sup + kFsDepth - 1, (j + kFsDepth - 1) % kFsDepth);     // into the stage that held the piece before
-#pragma unroll
-                for (int i = 0; i < kFsSlices; ++i) {
-                    const int sl = sup * kFsSlices + i;
-                    if (kFull || sl < nslice) {
-                        const uint4 x = *reinterpret_cast<const uint4*>(mine + j * kFsStageBytes + i * 64);
-                        const uint4 pv = *reinterpret_cast<const uint4*>(mine + j * kFsStageBytes + i * 64 - kFsRowPitch);
-                        const uint4 tt = tq[sl * 4];
-                        const uint4 xs = make_uint4(x.x, x.z, x.y, x.w);
-                        mma_bf16_m16n8k16(cn[0], x, xs.x, xs.y);
-                        mma_bf16_m16n8k16(cn[1], x, xs.z, xs.w);
-                        mma_bf16_m16n8k16(cp[0], pv, xs.x, xs.y);
-                        mma_bf16_m16n8k16(cp[1], pv, xs.z, xs.w);
-                        mma_bf16_m16n8k16(ct[0], x, tt.x, tt.y);
-                        mma_bf16_m16n8k16(ct[1], x, tt.z, tt.w);
-                    }
+            for (int i = 0; i < kFsSlices; ++i) {
+                if (kFull || sup * kFsSlices + i < nslice) {
+                    const uint4 x0 = ldmatrix_x4(at + i * 64u), x1 = ldmatrix_x4(at + i * 64u + 32u);
+                    mma_bf16_m16n8k16(acc[0], x0, x0.x, x0.z);
+                    mma_bf16_m16n8k16(acc[1], x1, x1.x, x1.z);
                 }
             }
         }
-    }
-    cp_async_wait<0>();
-    // the diagonal element of group g sits in the lane with q == g / 2, at column g % 2
-    __shared__ float s_nn[kFsWarps][kFsFrames], s_dp[kFsWarps][kFsFrames];
-    if (q == (g >> 1)) {
-        const bool odd = g & 1;
-        const float nn = odd ? cn[0][1] + cn[1][3] : cn[0][0] + cn[1][2];
-        const float dp = odd ? cp[0][1] + cp[1][3] : cp[0][0] + cp[1][2];
-        const float dt = odd ? ct[0][1] + ct[1][3] : ct[0][0] + ct[1][2];
-        s_nn[warp][g] = has_p && has_f ? nn : 0.f;
-        s_dp[warp][g] = has_p && has_f ? dp : 0.f;
-        if (has_p && has_f) {
-            const size_t r = (size_t)f * N + p;
-            const float n = fmaxf(sqrtf(nn), kEps);
-            token_score[r] = dt / (n * tn);
-            inv_norm[r] = 1.0f / n;
+        // lane (g, q) holds columns 2q and 2q + 1 of rows g and 8 + g
+        float c[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) c[i] = acc[0][i] + acc[1][i];
+        // <text, frame g> is C[8][g], in lane (0, g / 2)
+        const float t0 = __shfl_sync(0xFFFFFFFFu, c[2], g >> 1), t1 = __shfl_sync(0xFFFFFFFFu, c[3], g >> 1);
+        if (q == (g >> 1)) {                                // C[g][g]
+            const float nn = g & 1 ? c[1] : c[0];
+            s_nn[par][warp][g] = has ? nn : 0.f;
+            if (has) {
+                const size_t r = (size_t)f * N + p;
+                const float n = fmaxf(sqrtf(nn), kEps);
+                token_score[r] = (g & 1 ? t1 : t0) / (n * tn);
+                inv_norm[r] = 1.0f / n;
+            }
+        }
+        // s_dp[j]: frame f0 + j with the frame before it, C[j - 1][j]; for the run's first frame C[9][0]
+        if (g < 7 && q == ((g + 1) >> 1)) s_dp[par][warp][g + 1] = p < N ? (g & 1 ? c[0] : c[1]) : 0.f;
+        if (lane == 4) s_dp[par][warp][0] = p < N ? c[2] : 0.f;
+        __syncthreads();
+        if (tid < kFsFrames && f0 + tid < Tn) {
+            float nn = 0.f, dp = 0.f;
+#pragma unroll
+            for (int w = 0; w < kFsWarps; ++w) { nn += s_nn[par][w][tid]; dp += s_dp[par][w][tid]; }
+            const int ff = f0 + tid;
+            part_nrm[(size_t)pg * Tn + ff] = nn;
+            if (ff > 0) part_dot[(size_t)pg * Tn + (ff - 1)] = dp;    // dots of frames ff-1 and ff, four positions
         }
     }
-    __syncthreads();
-    if (tid < kFsFrames && f0 + tid < Tn) {
-        float nn = 0.f, dp = 0.f;
-#pragma unroll
-        for (int w = 0; w < kFsWarps; ++w) { nn += s_nn[w][tid]; dp += s_dp[w][tid]; }
-        const int ff = f0 + tid;
-        part_nrm[(size_t)pg * Tn + ff] = nn;
-        if (ff > 0) part_dot[(size_t)pg * Tn + (ff - 1)] = dp;    // dots of frames ff-1 and ff, four positions
-    }
+    cp_async_wait<0>();
 }
 
 // Frame runs sized so that all warps are resident at once: a second, partly filled wave of
@@ -699,7 +730,7 @@ static int launch_seg_score(const void* feats, const void* text, int Tn, int N, 
             METOK_ALLOW_SMEM(kernel, smem_t);
         nslab = ceil_div(N, kFsThreads / 32);              // the kernel adds the four positions of a CTA
         METOK_TIMED("seg_score_kernel", st);
-        launch_chained(kernel, dim3(nslab * ceil_div(Tn, kFsFrames)), dim3(kFsThreads), smem_t, st, 
+        launch_chained(kernel, dim3(std::min(nslab * ceil_div(Tn, kFsFrames), kNumSMs * kFsCtasPerSm)), dim3(kFsThreads), smem_t, st,
             reinterpret_cast<const __nv_bfloat16*>(feats), reinterpret_cast<const __nv_bfloat16*>(text), Tn, N, d,
             part_dot, part_nrm, token_score, inv_norm);
     } else {

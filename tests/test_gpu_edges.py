@@ -111,3 +111,19 @@ def test_attention_scores_whose_logits_grow_along_the_keys(Hq, Hkv, Lt, dh, n_vi
     torch.cuda.synchronize()
     err = np.abs(got.double().cpu().numpy() - want).max() / want.max()
     assert err < 2e-4, err
+
+
+@pytest.mark.parametrize("T,N,d", [(1, 1, 8), (8, 4, 256), (9, 5, 264), (7, 3, 1032), (33, 241, 248), (250, 75, 40), (131, 150, 520)])
+def test_one_pass_segmentation_units(T, N, d):
+    """Eight frames of four positions are a unit, a CTA takes every 296th: one unit, ragged ones, several per CTA."""
+    rng = np.random.default_rng(T * N + d)
+    V = O.round_bf16(rng.standard_normal((T, N, d)).astype(np.float32))
+    t = O.round_bf16(rng.standard_normal(d).astype(np.float32))
+    got = B.metok_segment_score_events(torch.from_numpy(V).cuda().bfloat16(), 1, torch.from_numpy(t).cuda().bfloat16())
+    x = V.astype(np.float64)
+    norm = np.sqrt((x ** 2).sum(-1))
+    frame = np.sqrt((norm ** 2).sum(-1))
+    sims = np.einsum("tnd,tnd->t", x[:-1], x[1:]) / (frame[:-1] * frame[1:])
+    assert np.allclose(got["sims"].cpu().numpy(), sims, rtol=1e-4, atol=2e-5)
+    assert np.allclose(got["token_score"].cpu().numpy().reshape(T, N), x @ t / (norm * np.linalg.norm(t)), rtol=1e-4, atol=2e-5)
+    assert np.allclose(got["token_inv_norm"].cpu().numpy().reshape(T, N), 1.0 / norm, rtol=1e-5)
