@@ -1121,30 +1121,30 @@ __device__ __forceinline__ void avg_cta_sum(uint8_t* cta_mem, const float (&acc)
     __syncthreads();
 }
 
-// Output c, all of whose `count` <= kAvgFew members are listed, by the whole CTA.
+// Output c, all of whose `count` <= kAvgFew members are listed, by the whole CTA; few: entry threadIdx.x of its list.
 template <typename T, int R>
 __device__ __forceinline__ void avg_heavy(AvgRing<R>& ring, const T* __restrict__ feats, T* __restrict__ out_feats, const AvgArgs& ar,
-                                          int c, int count, int seg, int* list, uint8_t* cta_mem) {
+                                          int c, int count, int few, int seg, int* sorted, uint8_t* cta_mem) {
     constexpr int VN = 16 / sizeof(T), CH = AvgRing<R>::kChunks;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int warp = threadIdx.x >> 5;
     const int ch0 = seg * ar.seg_chunks, nch = min(ar.seg_chunks, ar.d / VN - ch0);
-    // every thread ranks one member against all (they are read again and again from L1), every warp lists its quarter
+    // every thread ranks one member against all, every warp adds a quarter of the sorted list
     static_assert(kAvgFew == kAvgThreads, "one member per thread");
-    const int32_t* few = ar.ml.few + (size_t)c * kAvgFew;
-    int* s_few = reinterpret_cast<int*>(cta_mem);            // no copy is in flight yet
-    if (threadIdx.x < count) s_few[threadIdx.x] = few[threadIdx.x];
+    int4* s_few = reinterpret_cast<int4*>(cta_mem);          // no copy is in flight yet
+    const int tok = threadIdx.x < count ? few : 0x7FFFFFFF;  // lanes past the list hold the largest integer
+    reinterpret_cast<int*>(s_few)[threadIdx.x] = tok;
+    __syncthreads();
+    int rank = 0;
+#pragma unroll 4
+    for (int j = 0; j < (count + 3) / 4; ++j) {
+        const int4 x = s_few[j];
+        rank += (x.x < tok) + (x.y < tok) + (x.z < tok) + (x.w < tok);
+    }
+    if (threadIdx.x < count) sorted[rank] = tok;
     __syncthreads();
     const int share = (count + kAvgWarps - 1) / kAvgWarps, from = min(count, warp * share), n = min(count, from + share) - from;
-    for (int x = lane; x < count; x += 32) {
-        const int tok = s_few[x];
-        int rank = 0;
-#pragma unroll 8
-        for (int j = 0; j < count; ++j) rank += s_few[j] < tok;
-        if (rank >= from && rank < from + n) list[rank - from] = tok;
-    }
-    __syncthreads();
     float acc[CH][VN] = {};
-    avg_add_rows<T, R>(ring, feats, ar, list, n, ch0, nch, acc);
+    avg_add_rows<T, R>(ring, feats, ar, sorted + from, n, ch0, nch, acc);
     const float inv = 1.0f / (float)count;
     avg_cta_sum<T, CH>(cta_mem, acc, nch,
                             [&](int i, const float* t) { avg_store<T>(out_feats + (size_t)c * ar.d + (size_t)(ch0 + i) * VN, t, inv); });
@@ -1311,8 +1311,8 @@ merge_avg_kernel(const T* __restrict__ feats, T* __restrict__ out_feats, AvgArgs
                                  cta_mem, s_block, &s_last);
         } else {
             const int x = it - n_split, back = x / n_heavy, h = x - back * n_heavy;
-            const int c = ar.ml.heavy_slot[h], count = ar.ml.count[c];
-            if (count <= kAvgLong) avg_heavy<T, R>(ring, feats, out_feats, ar, c, count, ar.nseg - 1 - back, s_list[warp], cta_mem);
+            const int c = ar.ml.heavy_slot[h], count = ar.ml.count[c], few = ar.ml.few[(size_t)c * kAvgFew + tid];
+            if (count <= kAvgLong) avg_heavy<T, R>(ring, feats, out_feats, ar, c, count, few, ar.nseg - 1 - back, &s_list[0][0], cta_mem);
         }
         __syncthreads();
         it = s_next;
@@ -1337,18 +1337,28 @@ merge_avg_kernel(const T* __restrict__ feats, T* __restrict__ out_feats, AvgArgs
             if (a_n > kAvgHeavy) a_n = 0;
         }
     };
-    // A warp's first two pieces are fixed: all warps at one counter at once would stand in line for 5 us.
-    const int warps = (int)gridDim.x * kAvgWarps, me = (int)blockIdx.x * kAvgWarps + warp;
-    auto take = [&]() { return lane == 0 ? 2 * warps + atomicAdd(ar.next, 1) : 0; };
-    fetch(me);
-    int ticket = me + warps;
+    // A warp's first two pieces are fixed: all warps at one counter at once would stand in line for 5 us.  A CTA that had
+    // an item comes late: unless there are pieces enough for everybody, its warps take what is left, or their fixed pieces
+    // would be the last to be done (4009 outputs of 208 bytes, 72 of them such items: 22 -> 16 us; with five pieces a
+    // warp the two round trips to the counter cost 1 us).
+    const int n_busy = total < 4 * (int)gridDim.x * kAvgWarps ? min(n_items, (int)gridDim.x) : 0, warps = ((int)gridDim.x - n_busy) * kAvgWarps;
+    auto take = [&](int n) { return lane == 0 ? 2 * warps + atomicAdd(ar.next, n) : 0; };
+    int ticket;
+    if ((int)blockIdx.x >= n_busy) {
+        const int me = ((int)blockIdx.x - n_busy) * kAvgWarps + warp;
+        fetch(me);
+        ticket = me + warps;
+    } else {
+        ticket = __shfl_sync(0xFFFFFFFFu, take(2), 0);
+        fetch(ticket++);
+    }
     bool withhold = dbg_withhold(ar.status, kDbgMergeAvg);   // debug builds: of every warp's first row
     int i_piece = -1, i_n = 0, i_at = 0, i_ch0 = 0, i_nch = 0;   // issued: rows [0, i_at) of piece i_piece of the stream
     auto issue_next = [&](int st) {                          // the next row of the stream; false: there is none
         if (i_at == i_n) {
             while (a_n == 0) {
                 fetch(__shfl_sync(0xFFFFFFFFu, ticket, 0));
-                ticket = take();
+                ticket = take(1);
             }
             if (a_n < 0) return false;
             // the members into token order: rank = members before it
@@ -1367,7 +1377,7 @@ merge_avg_kernel(const T* __restrict__ feats, T* __restrict__ out_feats, AvgArgs
             i_ch0 = a_seg * ar.seg_chunks;
             i_nch = min(ar.seg_chunks, nchunk - i_ch0);
             fetch(__shfl_sync(0xFFFFFFFFu, ticket, 0));
-            ticket = take();
+            ticket = take(1);
         }
         avg_issue<T, R>(ring, st, feats, ar, queue[i_piece & (kAvgQueue - 1)].row[i_at], i_ch0, i_nch, withhold);
         withhold = false;
@@ -1628,7 +1638,9 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     ar.ml = w.ml;
     ar.long_sums = w.long_sums; ar.long_done = w.long_done; ar.next_item = w.avg_next; ar.next = w.avg_next + 1;
     ar.n_out = n_out; ar.out_members = out_members; ar.status = w.status;
-    const int grid = (int)std::min<long long>(kNumSMs * kAvgCtasPerSm, ((long long)cap * ar.nseg + kAvgWarps - 1) / kAvgWarps);
+    // a warp per piece, and CTAs for the outputs with many members, which there may be Nv / (kAvgHeavy + 1) of
+    const long long pieces = (long long)cap * ar.nseg, heavy = std::min<long long>(kNumSMs, (long long)Nv / (kAvgHeavy + 1) * ar.nseg);
+    const int grid = (int)std::min<long long>(kNumSMs * kAvgCtasPerSm, (pieces + kAvgWarps - 1) / kAvgWarps + heavy);
     auto launch = [&](auto kernel) -> int {
         METOK_ALLOW_SMEM(kernel, kAvgSmemBytes);
         {
