@@ -511,20 +511,21 @@ cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __res
 // Merge-assign on the CUDA cores (fp32 inputs; bf16 only when forced for debugging): fp32 products, added in
 // the order of the row, so every dot product is one chain of fused multiply-adds.
 //
-// Work unit = 64 of an event's tokens that are no key tokens x 64 of its key tokens; the units of all events form one list and
-// a CTA takes every gridDim-th.  A unit is done by 64 threads with 8 x 8 outputs each (rows ty + 8 i, keys
-// tx + 8 j).  Shared-memory reads and multiply-adds are nearly in balance there (a k costs a thread 64 bytes,
-// which is what 64 multiply-adds take to run), so rows and keys are kept as they lie (k contiguous, 8-byte reads
-// of two k; wider reads are no cheaper per byte: a k-major layout with 16-byte reads took 423 us) and come by
-// 16-byte asynchronous copies into two stages of 16 k, a row's pitch of 80 bytes (fp32) putting the eight keys
-// of a warp's read into different banks.  Rows past the tile's end are copies of another row: nobody reads
-// their results.  Small CTAs, six per SM, because the unit count is small: 61 frames of 169 tokens give 756
-// units.
+// Work unit = 8 P of an event's tokens that are no key tokens x 8 P of its key tokens (P = 2, 4 or 8: choose_simt_outputs);
+// the units of all events form one list, a CTA takes its first by its number and the others from a counter.  A unit is
+// done by 64 threads with P x P outputs each (rows ty + 8 i, keys tx + 8 j).  Shared-memory reads and multiply-adds are
+// nearly in balance at P = 8 (a k costs a thread 64 bytes, which is what 64 multiply-adds take to run), so rows and keys
+// are kept as they lie (k contiguous, 8-byte reads of two k; wider reads are no cheaper per byte: a k-major layout with
+// 16-byte reads took 423 us) and come by 16-byte asynchronous copies into two stages of 16 k (three or four are no
+// faster), a row's pitch of 80 bytes (fp32) putting the eight keys of a warp's read into different banks.  Rows past the
+// tile's end are copies of another row: nobody reads their results.  Small CTAs, several per SM, because the unit count
+// is small.
 // 61 x 169 tokens, d = 1156, fp32: 755 us with 64-row CTAs of 4 x 4 outputs per thread that each walked all keys
-// of the event, 219 us now (0.76 of the multiply-adds: key tokens need no assignment).
+// of the event, 204 us now (0.76 of the multiply-adds: key tokens need no assignment).
 // Units of one row meet in a 64-bit atomicMax as in the tensor-core kernel: larger value, then lower slot.
 // --------------------------------------------------------------------------- //
-constexpr int kSaTile = 64, kSaBK = 16, kSaThreads = 64, kSaCtasPerSm = 6;
+constexpr int kSaBK = 16, kSaThreads = 64;
+constexpr int sa_ctas_per_sm(int pt) { return pt == 8 ? 6 : pt == 4 ? 10 : 12; }
 
 template <typename T>
 __device__ __forceinline__ float2 load_pair(const T* p) {
@@ -536,28 +537,30 @@ __device__ __forceinline__ float2 load_pair(const T* p) {
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? kSaCtasPerSm : 4)
+template <typename T, int PT>                       // PT x PT outputs per thread
+__global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? sa_ctas_per_sm(PT) : 4)
 merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_t* __restrict__ ev_lo, int k,
                          const int32_t* __restrict__ ev_out_off, const int32_t* __restrict__ ev_unit_off,
-                         const float* __restrict__ inv_norm, TokenOut out) {
+                         const float* __restrict__ inv_norm, int32_t* __restrict__ next, TokenOut out) {
     grid_dep_wait();
     const int32_t *out_src = out.out_src, *rest = out.rest;
+    constexpr int kSaTile = 8 * PT;
     constexpr int CE = 16 / sizeof(T);              // elements per 16-byte chunk
     constexpr int CPR = kSaBK / CE;                 // chunks per row and stage
     constexpr int LD = kSaBK + CE;                  // row pitch in elements
     constexpr int kCopies = 2 * kSaTile * CPR / kSaThreads;
     constexpr int kRowStep = kSaThreads / CPR;      // rows between a thread's copies
     constexpr uint32_t kStage = 2 * kSaTile * LD * sizeof(T), kCopyStep = kRowStep * LD * sizeof(T);
-    __shared__ __align__(16) T tile[2][2 * kSaTile][LD];    // rows 0..63 tokens, 64..127 keys
+    __shared__ __align__(16) T tile[2][2 * kSaTile][LD];    // the tokens' rows, then the keys'
     __shared__ float s_inv[kSaTile];
+    __shared__ int s_next;
     const int tid = threadIdx.x, ty = tid >> 3, tx = tid & 7;
     const int crow = tid / CPR, cchunk = tid % CPR;
     const uint32_t dst0 = sm100::smem_u32(&tile[0][crow][cchunk * CE]);
     const int total = ev_unit_off[k];
     const int ksteps = (d + kSaBK - 1) / kSaBK;
     const uint32_t row_chunks = (uint32_t)(d / CE);
-    for (int unit = blockIdx.x; unit < total; unit += gridDim.x) {
+    for (int unit = blockIdx.x; unit < total; unit = s_next) {
         const int e = find_event(ev_unit_off, k, unit);
         const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0;
         const int nchunks = (nk + kSaTile - 1) / kSaTile;
@@ -573,7 +576,8 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
             src[i] = reinterpret_cast<const uint4*>(feats) + (size_t)row * row_chunks + cchunk;
         }
         __syncthreads();                            // the unit before is done with s_inv and both stages
-        s_inv[tid] = key0 + tid < key_end ? inv_norm[out_src[key0 + tid]] : 0.f;
+        if (tid == 0) s_next = total > (int)gridDim.x ? (int)gridDim.x + atomicAdd(next, 1) : total;
+        if (tid < kSaTile) s_inv[tid] = key0 + tid < key_end ? inv_norm[out_src[key0 + tid]] : 0.f;
         auto issue = [&](int ks) {                  // into stage ks % 2; past the end of the rows: zeros
             const uint32_t bytes = (uint32_t)(ks * CPR + cchunk) < row_chunks ? 16u : 0u;
             const uint32_t dst = dst0 + (ks & 1) * kStage;
@@ -582,11 +586,11 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
             for (int i = 0; i < kCopies; ++i) sm100::cp_async16_zfill(dst + i * kCopyStep, src[i] + off, bytes);
             sm100::cp_async_commit();
         };
-        float acc[8][8];
+        float acc[PT][PT];
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < PT; ++i)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+            for (int j = 0; j < PT; ++j) acc[i][j] = 0.f;
         issue(0);
         for (int ks = 0; ks < ksteps; ++ks) {
             sm100::cp_async_wait_all();
@@ -596,27 +600,27 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
             const T* pb = &tile[ks & 1][kSaTile + tx][0];
 #pragma unroll
             for (int kk = 0; kk < kSaBK; kk += 2) {
-                float2 a[8], b[8];
+                float2 a[PT], b[PT];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) a[i] = load_pair<T>(pa + 8 * i * LD + kk);
+                for (int i = 0; i < PT; ++i) a[i] = load_pair<T>(pa + 8 * i * LD + kk);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) b[j] = load_pair<T>(pb + 8 * j * LD + kk);
+                for (int j = 0; j < PT; ++j) b[j] = load_pair<T>(pb + 8 * j * LD + kk);
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < PT; ++i)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+                    for (int j = 0; j < PT; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < PT; ++i)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                    for (int j = 0; j < PT; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
             }
         }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < PT; ++i) {
             float best_v = -3.4e38f;
             int best_s = 0x7FFFFFFF;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {           // ascending slots
+            for (int j = 0; j < PT; ++j) {           // ascending slots
                 const int slot = key0 + tx + 8 * j;
                 const float v = acc[i][j] * s_inv[tx + 8 * j];
                 if (slot < key_end && v > best_v) { best_v = v; best_s = slot; }
@@ -1424,8 +1428,8 @@ struct VisionWs {
     unsigned long long* best64;
     MemberLists ml;
     float* long_sums;
-    int32_t *long_done, *avg_next;
-    int n_counters;           // the counters are cleared together: long, heavy, avg_next and long_done
+    int32_t *long_done, *avg_next, *unit_next;
+    int n_counters;           // the counters are cleared together: long, heavy, avg_next, unit_next and long_done
 };
 
 static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, bool merging) {
@@ -1450,11 +1454,12 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
         w.ml.few = cv.take<int32_t>(n * kAvgFew);
         w.ml.heavy_slot = cv.take<int32_t>(n);
         w.ml.long_slot = cv.take<int32_t>(n);
-        w.n_counters = 4 + avg_long_cap(d) * avg_max_pieces(d);
+        w.n_counters = 5 + avg_long_cap(d) * avg_max_pieces(d);
         w.ml.long_counter = cv.take<int32_t>((size_t)w.n_counters);
         w.ml.heavy_counter = w.ml.long_counter + 1;
         w.avg_next = w.ml.long_counter + 2;              // two: items, pieces
-        w.long_done = w.ml.long_counter + 4;
+        w.unit_next = w.ml.long_counter + 4;
+        w.long_done = w.ml.long_counter + 5;
         w.long_sums = cv.take<float>((size_t)avg_long_cap(d) * kAvgParts * d);
     }
     return w;
@@ -1486,6 +1491,18 @@ static MmaTile choose_mma_tile(int Nv, int k, int d, double keep) {
     best.stage_bytes = best.a_bytes + (uint32_t)best.bn * kMmaBK * 2;
     best.stages = std::min<int>(kMmaMaxStages, kMmaRingBytes / best.stage_bytes);
     return best;
+}
+
+// Outputs per thread (a side of the square) of the CUDA-core kernel, from the number of 64 x 64 units of the mean event.
+// Few of them leave SMs idle and last as long as one unit's chain of d steps: 16 x 16 units are then the fastest (5 frames
+// of 164 tokens, d = 2104, about 26 units: 161 us the call with 64 x 64, 76 with 32 x 32, 69 with 16 x 16; at about 94
+// units 146, 106 and 120).  Many small units read shared memory as fast as it goes and spread evenly; units of 64 x 64 do
+// a sixth more work in the same time but only where one round of CTAs does them all and is well filled (262 us against
+// 290 at 756 units; past the 888 places 308 against 290) -- events differ in length, hence not up to the last place.
+static int choose_simt_outputs(int Nv, int k, double keep) {
+    const double m = (double)Nv / k, keys = std::max(1.0, keep * m), units = ((m - keys) / 64 + 0.5) * (keys / 64 + 0.5) * k;
+    const double places = kNumSMs * sa_ctas_per_sm(8);
+    return units < kNumSMs / 2 ? 2 : units < places * 2 / 3 || units > places * 0.9 ? 4 : 8;
 }
 
 // The tensor-core merge path needs bf16 rows that TMA can address (16-byte row pitch);
@@ -1524,12 +1541,14 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         }
         METOK_LAUNCH_CHECK();
     }
-    const MmaTile tile = choose_mma_tile(Nv, k, d, p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey);
+    const double keep = p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey;
+    const MmaTile tile = choose_mma_tile(Nv, k, d, keep);
+    const int simt_pt = choose_simt_outputs(Nv, k, keep);
     PlanParams pp;
     pp.Tn = Tn; pp.N = N; pp.k = k;
     pp.n_key_events = min(k, ceilq(p->alpha * (double)k));
-    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? tile.bm : kSaTile;
-    pp.chunk_cols = mma ? tile.bn : kSaTile;
+    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? tile.bm : 8 * simt_pt;
+    pp.chunk_cols = mma ? tile.bn : 8 * simt_pt;
     pp.rows_with_keys = mma ? 1 : 0;
     pp.keep_key = p->keep_key; pp.keep_nonkey = p->keep_nonkey; pp.beta = p->beta;
     pp.key_given = p->key_events_given;
@@ -1614,8 +1633,9 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     } else {
         {
             METOK_TIMED("merge_assign_simt_kernel", st);
-            launch_chained(merge_assign_simt_kernel<T>, dim3(kNumSMs * kSaCtasPerSm), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
-                           w.ev_out_off, w.ev_unit_off, inv_norm, to);
+            auto kernel = simt_pt == 8 ? merge_assign_simt_kernel<T, 8> : simt_pt == 4 ? merge_assign_simt_kernel<T, 4> : merge_assign_simt_kernel<T, 2>;
+            launch_chained(kernel, dim3(kNumSMs * sa_ctas_per_sm(simt_pt)), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
+                           w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to);
         }
         METOK_LAUNCH_CHECK();
         {

@@ -127,3 +127,17 @@ def test_one_pass_segmentation_units(T, N, d):
     assert np.allclose(got["sims"].cpu().numpy(), sims, rtol=1e-4, atol=2e-5)
     assert np.allclose(got["token_score"].cpu().numpy().reshape(T, N), x @ t / (norm * np.linalg.norm(t)), rtol=1e-4, atol=2e-5)
     assert np.allclose(got["token_inv_norm"].cpu().numpy().reshape(T, N), 1.0 / norm, rtol=1e-5)
+
+
+@pytest.mark.parametrize("T,N,k,d,keep", [(3, 5, 3, 4, 0.4), (8, 16, 2, 64, 0.5), (13, 127, 2, 36, 0.42), (61, 169, 7, 20, 0.25), (40, 225, 3, 20, 0.3)])
+def test_fp32_merge_units(T, N, k, d, keep):
+    """Units of 16 x 16, 32 x 32 and 64 x 64, one round of CTAs and more."""
+    rng = np.random.default_rng(T * N + d)
+    V = rng.standard_normal((T, N, d)).astype(np.float32)
+    t = rng.standard_normal(d).astype(np.float32)
+    V += 0.5 * t
+    offs = np.sort(rng.choice(np.arange(1, T), size=k - 1, replace=False))
+    offs = np.concatenate([[0], offs, [T]]).astype(np.int32)
+    rep = R.compress_case(V, t, offs, "f32", 0.5, keep, keep)
+    assert rep["key_mismatches"] <= rep["key_near_ties"]
+    assert rep["assign_mismatches"] <= rep["assign_near_ties"]
