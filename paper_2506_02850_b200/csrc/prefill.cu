@@ -1,11 +1,13 @@
 // metok_prefill_prune: text->visual attention scores at a pruning layer, class-wise
 // top-k under the Eq. 6/7 budgets, and compaction of the surviving hidden states.
+#include <algorithm>
 #include <cstdlib>
 
 #include "common.cuh"
 #include "select.cuh"
 #include "select_cluster.cuh"
 #include "launchers.h"
+#include "simt_tile.cuh"
 #include "sm100.cuh"
 
 namespace metok {
@@ -20,195 +22,183 @@ namespace metok {
 // per-row running (max, sum) over a split of the columns, pass 2 recomputes the
 // logits, normalises, and sums each column over the rows of the tile.
 // Everything is reduced in a fixed order (no float atomics).
+//
+// A CTA of 64 threads takes a tile of 32 rows and a run of tiles of 32 keys (SimtTile with 4 x 4 outputs per thread); a
+// thread keeps the running (max, sum) of its four rows over its own keys and they meet once, at the end of the run.  What
+// bounds it is the rate of multiply-adds and shared-memory reads together, at small sizes the chain over the head
+// dimension.  Tiles of 64 x 64 read less but fill the chip worse (28 heads x 30 rows x 6080 keys, fp32, the whole pruning
+// call: 222 us with 64 x 64 tiles of 4 x 4 scalar reads per thread and 256 threads, 133 with SimtTile<8>, 126 as it is;
+// 40 heads x 16 rows x 3016 keys: 265, 166, 100; 14 heads x 7 rows x 2041 keys: 30.8, 33.5, 27); of 16 x 16 only
+// where a KV head has 16 rows or fewer (92 for the second case).
 // --------------------------------------------------------------------------- //
-constexpr int kAtTM = 64, kAtTN = 64;
-constexpr int kAtLD = 65;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kNegInf = -3.0e38f;   // finite stand-in: keeps (m_old - m_new) free of inf - inf
+constexpr int kAtPT = 4, kAtTile = 8 * kAtPT;   // outputs per thread and tile (a side of the square)
+constexpr int kAtMaxSplits = 128;
 
 struct AttnDims {
-    int Hq, Hkv, Lt, S, dh, vis_start, n_vis, rep, R, nrt, nsplit, tiles_n;
+    int Hq, Hkv, Lt, S, dh, vis_start, n_vis, rep, R, nrt, nsplit, per, tiles_n;   // nsplit runs of `per` key tiles
     float scale_log2;
 };
 
-template <typename T>
-__device__ __forceinline__ void load_tile_transposed(const T* __restrict__ base, int row0, int row_end, int dh,
-                                                     float* __restrict__ dst /*[dh][kAtLD]*/) {
-    constexpr int VN = Vec16<T>::N;
-    const int cpr = dh / VN;
-    for (int c = threadIdx.x; c < kAtTM * cpr; c += blockDim.x) {
-        const int r = c / cpr, ch = c % cpr;
-        float v[VN];
-        const int row = row0 + r;
-        if (row < row_end) Vec16<T>::load(base + (size_t)row * dh + ch * VN, v);
-        else Vec16<T>::zero(v);
+// This thread's copies of a tile's query rows (they stay the same) and of the key rows from u0 on; rows past the end are
+// copies of the last one, whose results nobody uses.
+template <typename Tile, typename T>
+__device__ __forceinline__ void attn_tile_sources(const T* Qg, const T* Kg, const AttnDims& dm, int rt, int u0, bool first,
+                                                  const uint4* (&src)[Tile::kCopies]) {
+    const size_t row_chunks = (size_t)(dm.dh / Tile::CE);
 #pragma unroll
-        for (int q = 0; q < VN; ++q) dst[(ch * VN + q) * kAtLD + r] = v[q];
-    }
-}
-
-__device__ __forceinline__ void tile_logits(const float* __restrict__ Qs, const float* __restrict__ Ks, int dh,
-                                            int ty, int tx, float (&acc)[4][4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 4
-    for (int kk = 0; kk < dh; ++kk) {
-        float a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = Qs[kk * kAtLD + ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = Ks[kk * kAtLD + tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    for (int i = 0; i < Tile::kCopies; ++i) {
+        const int r = Tile::copy_row(i);
+        if (r >= kAtTile)
+            src[i] = reinterpret_cast<const uint4*>(Kg) + (size_t)min(u0 + r - kAtTile, dm.S - 1) * row_chunks + Tile::copy_chunk();
+        else if (first)
+            src[i] = reinterpret_cast<const uint4*>(Qg) + (size_t)min(rt * kAtTile + r, dm.R - 1) * row_chunks + Tile::copy_chunk();
     }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? sa_ctas_per_sm(kAtPT) : 4)
 attn_stats_kernel(const T* __restrict__ q_text, const T* __restrict__ k_all, AttnDims dm,
                   float* __restrict__ part_m, float* __restrict__ part_l) {
     grid_dep_wait();
-    extern __shared__ float smem[];
-    float* Qs = smem;
-    float* Ks = smem + dm.dh * kAtLD;
+    using Tile = SimtTile<T, kAtPT>;
+    constexpr int PT = kAtPT;
+    __shared__ __align__(16) Tile tile;
     const int split = blockIdx.x, rt = blockIdx.y, g = blockIdx.z;
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;
     const T* Qg = q_text + (size_t)g * dm.R * dm.dh;
     const T* Kg = k_all + (size_t)g * dm.S * dm.dh;
     const int text_start = dm.S - dm.Lt;
-    load_tile_transposed<T>(Qg, rt * kAtTM, dm.R, dm.dh, Qs);
-
-    int limit[4];
-    float m_run[4], l_run[4];
+    int limit[PT];
+    float m_run[PT], l_run[PT];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = rt * kAtTM + ty + 16 * i;
+    for (int i = 0; i < PT; ++i) {
+        const int r = rt * kAtTile + ty + 8 * i;
         limit[i] = r < dm.R ? text_start + (r % dm.Lt) : -1;    // last visible key
         m_run[i] = kNegInf;
         l_run[i] = 0.f;
     }
-    const int per = (dm.tiles_n + dm.nsplit - 1) / dm.nsplit;
-    const int t_lo = split * per, t_hi = min(dm.tiles_n, t_lo + per);
+    const int t_lo = split * dm.per, t_hi = min(dm.tiles_n, t_lo + dm.per);
+    const int ksteps = Tile::steps(dm.dh);
+    const uint32_t dst0 = tile.copy_dst();
+    const uint4* src[Tile::kCopies];
     for (int tn = t_lo; tn < t_hi; ++tn) {
+        const int u0 = tn * kAtTile;
+        attn_tile_sources<Tile>(Qg, Kg, dm, rt, u0, tn == t_lo, src);
         __syncthreads();
-        load_tile_transposed<T>(Kg, tn * kAtTN, dm.S, dm.dh, Ks);
-        __syncthreads();
-        float acc[4][4];
-        tile_logits(Qs, Ks, dm.dh, ty, tx, acc);
+        float acc[PT][PT];
+        tile.dots(src, dm.dh / Tile::CE, ksteps, dst0, acc);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float tmax = kNegInf;
+        for (int i = 0; i < PT; ++i) {
+            float m_new = m_run[i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int u = tn * kAtTN + tx + 16 * j;
-                acc[i][j] = (u <= limit[i]) ? acc[i][j] * dm.scale_log2 : kNegInf;
-                tmax = fmaxf(tmax, acc[i][j]);
+            for (int j = 0; j < PT; ++j) {
+                acc[i][j] = (u0 + tx + 8 * j <= limit[i]) ? acc[i][j] * dm.scale_log2 : kNegInf;
+                m_new = fmaxf(m_new, acc[i][j]);
             }
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xFFFFFFFFu, tmax, o));
-            const float m_new = fmaxf(m_run[i], tmax);
             float s = 0.f;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) s += (acc[i][j] > kNegInf) ? exp2f(acc[i][j] - m_new) : 0.f;
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+            for (int j = 0; j < PT; ++j) s += (acc[i][j] > kNegInf) ? exp2f(acc[i][j] - m_new) : 0.f;
             l_run[i] = l_run[i] * exp2f(m_run[i] - m_new) + s;
             m_run[i] = m_new;
         }
     }
-    if (tx == 0) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = rt * kAtTM + ty + 16 * i;
-            if (r < dm.R) {
-                const size_t o = ((size_t)g * dm.nsplit + split) * dm.R + r;
-                part_m[o] = m_run[i];
-                part_l[o] = l_run[i];
-            }
+    for (int i = 0; i < PT; ++i) {
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {                       // the eight threads of the row
+            const float m2 = __shfl_xor_sync(0xFFFFFFFFu, m_run[i], o), l2 = __shfl_xor_sync(0xFFFFFFFFu, l_run[i], o);
+            const float m = fmaxf(m_run[i], m2);
+            l_run[i] = l_run[i] * exp2f(m_run[i] - m) + l2 * exp2f(m2 - m);
+            m_run[i] = m;
+        }
+        const int r = rt * kAtTile + ty + 8 * i;
+        if (tx == 0 && r < dm.R) {
+            const size_t o = ((size_t)g * dm.nsplit + split) * dm.R + r;
+            part_m[o] = m_run[i];
+            part_l[o] = l_run[i];
         }
     }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? sa_ctas_per_sm(kAtPT) : 4)
 attn_colsum_kernel(const T* __restrict__ q_text, const T* __restrict__ k_all, AttnDims dm,
                    const float* __restrict__ part_m, const float* __restrict__ part_l,
                    float* __restrict__ part_col) {
     grid_dep_wait();
-    extern __shared__ float smem[];
-    float* Qs = smem;
-    float* Ks = smem + dm.dh * kAtLD;
-    __shared__ float s_M[kAtTM], s_invZ[kAtTM];
-    __shared__ float s_col[8][kAtTN];
+    using Tile = SimtTile<T, kAtPT>;
+    constexpr int PT = kAtPT;
+    __shared__ __align__(16) Tile tile;
+    __shared__ float s_M[kAtTile], s_invZ[kAtTile];
+    __shared__ float s_col[2][kAtTile];
     const int split = blockIdx.x, rt = blockIdx.y, g = blockIdx.z;
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, warp = tid >> 5;
+    const int tid = threadIdx.x, ty = tid >> 3, tx = tid & 7, warp = tid >> 5, lane = tid & 31;
     const T* Qg = q_text + (size_t)g * dm.R * dm.dh;
     const T* Kg = k_all + (size_t)g * dm.S * dm.dh;
-    const int text_start = dm.S - dm.Lt;
-    load_tile_transposed<T>(Qg, rt * kAtTM, dm.R, dm.dh, Qs);
-    if (tid < kAtTM) {
-        const int r = rt * kAtTM + tid;
+    const int text_start = dm.S - dm.Lt, vis_end = dm.vis_start + dm.n_vis;
+    const int t_lo = max(split * dm.per, dm.vis_start / kAtTile);                                    // tiles with a visual column
+    const int t_hi = min(min(dm.tiles_n, split * dm.per + dm.per), (vis_end + kAtTile - 1) / kAtTile);
+    if (t_lo >= t_hi) return;
+    if (tid < kAtTile) {
+        const int r = rt * kAtTile + tid;
         float M = kNegInf, Z = 0.f;
         if (r < dm.R) {
-            for (int s = 0; s < dm.nsplit; ++s) M = fmaxf(M, part_m[((size_t)g * dm.nsplit + s) * dm.R + r]);
-            for (int s = 0; s < dm.nsplit; ++s) {
-                const size_t o = ((size_t)g * dm.nsplit + s) * dm.R + r;
-                Z += part_l[o] * exp2f(part_m[o] - M);
+            const size_t o = (size_t)g * dm.nsplit * dm.R + r;
+            for (int s0 = 0; s0 < dm.nsplit; s0 += 8) {         // eight runs' loads in flight
+                float m[8], l[8], M8 = M;
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                    const bool in = s0 + x < dm.nsplit;
+                    m[x] = in ? part_m[o + (size_t)(s0 + x) * dm.R] : kNegInf;
+                    l[x] = in ? part_l[o + (size_t)(s0 + x) * dm.R] : 0.f;
+                    M8 = fmaxf(M8, m[x]);
+                }
+                Z *= exp2f(M - M8);
+#pragma unroll
+                for (int x = 0; x < 8; ++x) Z += l[x] * exp2f(m[x] - M8);
+                M = M8;
             }
         }
         s_M[tid] = M;
         s_invZ[tid] = Z > 0.f ? 1.0f / Z : 0.f;
     }
     __syncthreads();
-    int limit[4];
-    float rM[4], rI[4];
+    int limit[PT];
+    float rM[PT], rI[PT];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int rl = ty + 16 * i;
-        const int r = rt * kAtTM + rl;
+    for (int i = 0; i < PT; ++i) {
+        const int rl = ty + 8 * i;
+        const int r = rt * kAtTile + rl;
         limit[i] = r < dm.R ? text_start + (r % dm.Lt) : -1;
         rM[i] = s_M[rl];
         rI[i] = s_invZ[rl];
     }
-    const int per = (dm.tiles_n + dm.nsplit - 1) / dm.nsplit;
-    const int t_lo = split * per, t_hi = min(dm.tiles_n, t_lo + per);
-    const int vis_end = dm.vis_start + dm.n_vis;
+    const int ksteps = Tile::steps(dm.dh);
+    const uint32_t dst0 = tile.copy_dst();
+    const uint4* src[Tile::kCopies];
     for (int tn = t_lo; tn < t_hi; ++tn) {
-        const int u0 = tn * kAtTN;
-        if (u0 >= vis_end || u0 + kAtTN <= dm.vis_start) continue;     // no visual column in this tile
-        __syncthreads();
-        load_tile_transposed<T>(Kg, u0, dm.S, dm.dh, Ks);
-        __syncthreads();
-        float acc[4][4];
-        tile_logits(Qs, Ks, dm.dh, ty, tx, acc);
-        float cs[4];
+        const int u0 = tn * kAtTile;
+        attn_tile_sources<Tile>(Qg, Kg, dm, rt, u0, tn == t_lo, src);
+        float acc[PT][PT];
+        tile.dots(src, dm.dh / Tile::CE, ksteps, dst0, acc);      // (the barrier below: nobody reads the tile before)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int u = u0 + tx + 16 * j;
+        for (int j = 0; j < PT; ++j) {
+            const int u = u0 + tx + 8 * j;
             float c = 0.f;
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < PT; ++i)
                 c += (u <= limit[i]) ? exp2f(acc[i][j] * dm.scale_log2 - rM[i]) * rI[i] : 0.f;
-            c += __shfl_xor_sync(0xFFFFFFFFu, c, 16);            // the warp's two row groups
-            cs[j] = c;
-        }
-        if ((tid & 31) < 16) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) s_col[warp][tx + 16 * j] = cs[j];
+            c += __shfl_xor_sync(0xFFFFFFFFu, c, 8);             // the warp's four row groups
+            c += __shfl_xor_sync(0xFFFFFFFFu, c, 16);
+            if (lane < 8) s_col[warp][tx + 8 * j] = c;
         }
         __syncthreads();
-        if (tid < kAtTN) {
+        if (tid < kAtTile) {
             const int u = u0 + tid;
-            if (u >= dm.vis_start && u < vis_end) {
-                float c = 0.f;
-#pragma unroll
-                for (int w = 0; w < 8; ++w) c += s_col[w][tid];
-                part_col[((size_t)g * dm.nrt + rt) * dm.n_vis + (u - dm.vis_start)] = c;
-            }
+            if (u >= dm.vis_start && u < vis_end)
+                part_col[((size_t)g * dm.nrt + rt) * dm.n_vis + (u - dm.vis_start)] = s_col[0][tid] + s_col[1][tid];
         }
     }
 }
@@ -481,13 +471,12 @@ static AttnDims make_dims(int Hq, int Hkv, int Lt, int S, int dh, int vis_start,
     dm.Hq = Hq; dm.Hkv = Hkv; dm.Lt = Lt; dm.S = S; dm.dh = dh; dm.vis_start = vis_start; dm.n_vis = n_vis;
     dm.rep = Hq / Hkv;
     dm.R = dm.rep * Lt;
-    dm.nrt = ceil_div(dm.R, kAtTM);
-    dm.tiles_n = ceil_div(S, kAtTN);
-    int ns = ceil_div(4 * kNumSMs, dm.nrt * Hkv);
-    if (ns > dm.tiles_n) ns = dm.tiles_n;
-    if (ns < 1) ns = 1;
-    if (ns > 64) ns = 64;
-    dm.nsplit = ns;
+    dm.nrt = ceil_div(dm.R, kAtTile);
+    dm.tiles_n = ceil_div(S, kAtTile);
+    // as many runs of key tiles as give every place on the chip one, no more: a last round would cost as much as the others
+    const int most = std::max(1, std::min(kAtMaxSplits, kNumSMs * sa_ctas_per_sm(kAtPT) / (dm.nrt * Hkv)));
+    dm.per = ceil_div(dm.tiles_n, most);
+    dm.nsplit = ceil_div(dm.tiles_n, dm.per);
     dm.scale_log2 = scale * kLog2e;
     return dm;
 }
@@ -535,21 +524,17 @@ static int launch_score_reduce(const PrefillWs& w, const AttnDims& dm, float inv
 template <typename T>
 static int launch_attn_scores(const void* q_text, const void* k_all, const AttnDims& dm, const PrefillWs& w,
                               float inv_rows, float* scores, cudaStream_t st) {
-    const size_t smem = (size_t)2 * dm.dh * kAtLD * sizeof(float);
-    METOK_ALLOW_SMEM(attn_stats_kernel<T>, smem);
-    METOK_ALLOW_SMEM(attn_colsum_kernel<T>, smem);
     dim3 grid(dm.nsplit, dm.nrt, dm.Hkv);
     {
         METOK_TIMED("attn_stats_kernel", st);
-        launch_chained(attn_stats_kernel<T>, grid, dim3(256), smem, st, reinterpret_cast<const T*>(q_text), reinterpret_cast<const T*>(k_all),
-                                                  dm, w.part_m, w.part_l);
+        launch_chained(attn_stats_kernel<T>, grid, dim3(kSaThreads), 0, st, reinterpret_cast<const T*>(q_text), reinterpret_cast<const T*>(k_all),
+                       dm, w.part_m, w.part_l);
     }
     METOK_LAUNCH_CHECK();
     {
         METOK_TIMED("attn_colsum_kernel", st);
-        launch_chained(attn_colsum_kernel<T>, grid, dim3(256), smem, st, reinterpret_cast<const T*>(q_text),
-                                                   reinterpret_cast<const T*>(k_all), dm, w.part_m, w.part_l,
-                                                   w.part_col);
+        launch_chained(attn_colsum_kernel<T>, grid, dim3(kSaThreads), 0, st, reinterpret_cast<const T*>(q_text),
+                       reinterpret_cast<const T*>(k_all), dm, w.part_m, w.part_l, w.part_col);
     }
     METOK_LAUNCH_CHECK();
     return launch_score_reduce(w, dm, inv_rows, scores, st);

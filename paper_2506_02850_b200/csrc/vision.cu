@@ -7,6 +7,7 @@
 #include "common.cuh"
 #include "select.cuh"
 #include "select_cluster.cuh"
+#include "simt_tile.cuh"
 #include "sm100.cuh"
 #include "launchers.h"
 
@@ -512,31 +513,12 @@ cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __res
 // the order of the row, so every dot product is one chain of fused multiply-adds.
 //
 // Work unit = 8 P of an event's tokens that are no key tokens x 8 P of its key tokens (P = 2, 4 or 8: choose_simt_outputs);
-// the units of all events form one list, a CTA takes its first by its number and the others from a counter.  A unit is
-// done by 64 threads with P x P outputs each (rows ty + 8 i, keys tx + 8 j).  Shared-memory reads and multiply-adds are
-// nearly in balance at P = 8 (a k costs a thread 64 bytes, which is what 64 multiply-adds take to run), so rows and keys
-// are kept as they lie (k contiguous, 8-byte reads of two k; wider reads are no cheaper per byte: a k-major layout with
-// 16-byte reads took 423 us) and come by 16-byte asynchronous copies into two stages of 16 k (three or four are no
-// faster), a row's pitch of 80 bytes (fp32) putting the eight keys of a warp's read into different banks.  Rows past the
-// tile's end are copies of another row: nobody reads their results.  Small CTAs, several per SM, because the unit count
-// is small.
+// the units of all events form one list, a CTA takes its first by its number and the others from a counter; the dot
+// products of a unit are SimtTile's.  Rows past a unit's end are copies of another row: nobody reads their results.
 // 61 x 169 tokens, d = 1156, fp32: 755 us with 64-row CTAs of 4 x 4 outputs per thread that each walked all keys
 // of the event, 204 us now (0.76 of the multiply-adds: key tokens need no assignment).
 // Units of one row meet in a 64-bit atomicMax as in the tensor-core kernel: larger value, then lower slot.
 // --------------------------------------------------------------------------- //
-constexpr int kSaBK = 16, kSaThreads = 64;
-constexpr int sa_ctas_per_sm(int pt) { return pt == 8 ? 6 : pt == 4 ? 10 : 12; }
-
-template <typename T>
-__device__ __forceinline__ float2 load_pair(const T* p) {
-    if constexpr (sizeof(T) == 4) {
-        return *reinterpret_cast<const float2*>(p);
-    } else {
-        const uint32_t w = *reinterpret_cast<const uint32_t*>(p);
-        return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
-    }
-}
-
 template <typename T, int PT>                       // PT x PT outputs per thread
 __global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? sa_ctas_per_sm(PT) : 4)
 merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_t* __restrict__ ev_lo, int k,
@@ -544,22 +526,15 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
                          const float* __restrict__ inv_norm, int32_t* __restrict__ next, TokenOut out) {
     grid_dep_wait();
     const int32_t *out_src = out.out_src, *rest = out.rest;
-    constexpr int kSaTile = 8 * PT;
-    constexpr int CE = 16 / sizeof(T);              // elements per 16-byte chunk
-    constexpr int CPR = kSaBK / CE;                 // chunks per row and stage
-    constexpr int LD = kSaBK + CE;                  // row pitch in elements
-    constexpr int kCopies = 2 * kSaTile * CPR / kSaThreads;
-    constexpr int kRowStep = kSaThreads / CPR;      // rows between a thread's copies
-    constexpr uint32_t kStage = 2 * kSaTile * LD * sizeof(T), kCopyStep = kRowStep * LD * sizeof(T);
-    __shared__ __align__(16) T tile[2][2 * kSaTile][LD];    // the tokens' rows, then the keys'
+    using Tile = SimtTile<T, PT>;
+    constexpr int kSaTile = Tile::kTile, kCopies = Tile::kCopies;
+    __shared__ __align__(16) Tile tile;
     __shared__ float s_inv[kSaTile];
     __shared__ int s_next;
     const int tid = threadIdx.x, ty = tid >> 3, tx = tid & 7;
-    const int crow = tid / CPR, cchunk = tid % CPR;
-    const uint32_t dst0 = sm100::smem_u32(&tile[0][crow][cchunk * CE]);
     const int total = ev_unit_off[k];
-    const int ksteps = (d + kSaBK - 1) / kSaBK;
-    const uint32_t row_chunks = (uint32_t)(d / CE);
+    const int row_chunks = d / Tile::CE, ksteps = Tile::steps(d);
+    const uint32_t dst0 = tile.copy_dst();
     for (int unit = blockIdx.x; unit < total; unit = s_next) {
         const int e = find_event(ev_unit_off, k, unit);
         const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0;
@@ -571,50 +546,15 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
         const uint4* src[kCopies];                  // where this thread's copies of the first stage read
 #pragma unroll
         for (int i = 0; i < kCopies; ++i) {
-            const int r = crow + kRowStep * i;
+            const int r = Tile::copy_row(i);
             const int row = r < kSaTile ? rest[min(row0 + r, row_end - 1)] : out_src[min(key0 + r - kSaTile, key_end - 1)];
-            src[i] = reinterpret_cast<const uint4*>(feats) + (size_t)row * row_chunks + cchunk;
+            src[i] = reinterpret_cast<const uint4*>(feats) + (size_t)row * row_chunks + Tile::copy_chunk();
         }
         __syncthreads();                            // the unit before is done with s_inv and both stages
         if (tid == 0) s_next = total > (int)gridDim.x ? (int)gridDim.x + atomicAdd(next, 1) : total;
         if (tid < kSaTile) s_inv[tid] = key0 + tid < key_end ? inv_norm[out_src[key0 + tid]] : 0.f;
-        auto issue = [&](int ks) {                  // into stage ks % 2; past the end of the rows: zeros
-            const uint32_t bytes = (uint32_t)(ks * CPR + cchunk) < row_chunks ? 16u : 0u;
-            const uint32_t dst = dst0 + (ks & 1) * kStage;
-            const int off = bytes ? ks * CPR : 0;
-#pragma unroll
-            for (int i = 0; i < kCopies; ++i) sm100::cp_async16_zfill(dst + i * kCopyStep, src[i] + off, bytes);
-            sm100::cp_async_commit();
-        };
         float acc[PT][PT];
-#pragma unroll
-        for (int i = 0; i < PT; ++i)
-#pragma unroll
-            for (int j = 0; j < PT; ++j) acc[i][j] = 0.f;
-        issue(0);
-        for (int ks = 0; ks < ksteps; ++ks) {
-            sm100::cp_async_wait_all();
-            __syncthreads();                        // stage ks % 2 has landed for everybody; the other one has been read by everybody
-            if (ks + 1 < ksteps) issue(ks + 1);
-            const T* pa = &tile[ks & 1][ty][0];
-            const T* pb = &tile[ks & 1][kSaTile + tx][0];
-#pragma unroll
-            for (int kk = 0; kk < kSaBK; kk += 2) {
-                float2 a[PT], b[PT];
-#pragma unroll
-                for (int i = 0; i < PT; ++i) a[i] = load_pair<T>(pa + 8 * i * LD + kk);
-#pragma unroll
-                for (int j = 0; j < PT; ++j) b[j] = load_pair<T>(pb + 8 * j * LD + kk);
-#pragma unroll
-                for (int i = 0; i < PT; ++i)
-#pragma unroll
-                    for (int j = 0; j < PT; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-#pragma unroll
-                for (int i = 0; i < PT; ++i)
-#pragma unroll
-                    for (int j = 0; j < PT; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-            }
-        }
+        tile.dots(src, row_chunks, ksteps, dst0, acc);
 #pragma unroll
         for (int i = 0; i < PT; ++i) {
             float best_v = -3.4e38f;

@@ -141,3 +141,19 @@ def test_fp32_merge_units(T, N, k, d, keep):
     rep = R.compress_case(V, t, offs, "f32", 0.5, keep, keep)
     assert rep["key_mismatches"] <= rep["key_near_ties"]
     assert rep["assign_mismatches"] <= rep["assign_near_ties"]
+
+
+@pytest.mark.parametrize("Hq,Hkv,Lt,dh,vis_start,n_vis", [
+    (1, 1, 1, 4, 0, 1), (2, 2, 31, 20, 33, 1), (3, 1, 11, 64, 31, 33), (8, 2, 8, 100, 64, 159), (40, 40, 3, 128, 5, 90),
+    (1, 1, 2, 8, 0, 9000), (4, 1, 33, 12, 700, 3000),                    # more key tiles than runs of them
+])
+def test_fp32_attention_scores_at_tile_edges(Hq, Hkv, Lt, dh, vis_start, n_vis):
+    rng = np.random.default_rng(n_vis + dh)
+    S = vis_start + n_vis + Lt + 2
+    Q = (2.0 * rng.standard_normal((Hq, Lt, dh))).astype(np.float32)
+    K = rng.standard_normal((Hkv, S, dh)).astype(np.float32)
+    want = O.attention_scores(Q, K, vis_start, n_vis, dh ** -0.5)
+    got = B.metok_attention_scores(torch.from_numpy(Q).cuda(), torch.from_numpy(K).cuda(), vis_start, n_vis, dh ** -0.5)
+    torch.cuda.synchronize()
+    err = np.abs(got.double().cpu().numpy() - want).max() / want.max()
+    assert err < 1e-5, err
