@@ -32,9 +32,10 @@ __device__ __forceinline__ void widen16(const uint4& r, float (&v)[16 / sizeof(T
 }
 
 constexpr int kSegMaxRun = 16;    // frames per CTA at most
+constexpr int kSegCtasPerSm = 4;  // by its registers
 
 template <typename T>
-__global__ void __launch_bounds__(kSegThreads)
+__global__ void __launch_bounds__(kSegThreads, kSegCtasPerSm)
 seg_partial_kernel(const T* __restrict__ feats, int Tn, long long chunks_per_frame, int frames_per_cta,
                    float* __restrict__ part_dot, float* __restrict__ part_nrm) {
     grid_dep_wait();
@@ -294,8 +295,16 @@ static int launch_segment(const void* feats, int Tn, int N, int d, int k, int si
     if (sim_mode == METOK_SIM_FLATTEN) {
         const long long chunks = (long long)N * d / VN;
         nslab = (int)((chunks + kSegThreads * kSegUnroll - 1) / (kSegThreads * kSegUnroll));
-        int fpc = kSegMaxRun;
-        while (fpc > 1 && (long long)nslab * ceil_div(Tn, fpc) < 4 * kNumSMs) fpc >>= 1;
+        // Frames per CTA: the run with the fewest frames read one after the other, over all rounds of CTAs; a CTA reads one
+        // frame more than it owns and takes about another frame's time to start (64 x 196 x 1152: two frames a CTA were two
+        // rounds, four are one; 375 x 256 x 1872: sixteen left the third round half empty, thirteen fill it).
+        int fpc = 1;
+        long long best = -1;
+        for (int f = 1; f <= kSegMaxRun; ++f) {
+            const long long ctas = (long long)nslab * ceil_div(Tn, f), rounds = (ctas + kSegCtasPerSm * kNumSMs - 1) / (kSegCtasPerSm * kNumSMs);
+            const long long cost = rounds * (f + 2);
+            if (best < 0 || cost <= best) { best = cost; fpc = f; }
+        }
         part_dot = cv.take<float>((size_t)nslab * Tn);
         part_nrm = cv.take<float>((size_t)nslab * Tn);
         dim3 grid(nslab, ceil_div(Tn, fpc));
