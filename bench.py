@@ -44,29 +44,12 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # captures (profiles/), keyed by (scope/kernel, workload); a kernel changed since its capture is left out
 # (its stage then reports traffic null).
 NCU_TRAFFIC_BYTES = {
-    ("segment/seg_score_kernel", "frames128"): 136371200,
-    ("segment/seg_finish_kernel", "frames128"): 58624,
-    ("compress/event_plan_kernel", "frames128"): 131584,
-    ("compress/event_topk_kernel", "frames128"): 132352,
-    ("compress/merge_assign_mma_kernel", "frames128"): 137563392,
-    ("compress/merge_decode_kernel", "frames128"): 279808,
-    ("compress/merge_avg_kernel", "frames128"): 147466752,
-    ("prefill1/attn_stats_mma_kernel", "frames128"): 19438592,
-    ("prefill1/attn_colsum_mma_kernel", "frames128"): 19495680,
     ("prefill1/attn_score_reduce_kernel", "frames128"): 1189120,
-    ("prefill1/class_topk_kernel", "frames128"): 217856,
     ("prefill1/gather_rows_kernel", "frames128"): 53984512,
-    ("prefill2/attn_stats_mma_kernel", "frames128"): 7494656,
-    ("prefill2/attn_colsum_mma_kernel", "frames128"): 7568128,
     ("prefill2/attn_score_reduce_kernel", "frames128"): 442880,
-    ("prefill2/class_topk_kernel", "frames128"): 124928,
     ("prefill2/gather_rows_kernel", "frames128"): 15964672,
-    ("prefill3/attn_stats_mma_kernel", "frames128"): 2776576,
-    ("prefill3/attn_colsum_mma_kernel", "frames128"): 2791936,
     ("prefill3/attn_score_reduce_kernel", "frames128"): 147456,
-    ("prefill3/class_topk_kernel", "frames128"): 87808,
     ("prefill3/gather_rows_kernel", "frames128"): 473344,
-    ("kv/class_topk_kernel", "frames128"): 139776,
     ("kv/kv_stage_kernel", "frames128"): 4828160,
     ("kv/kv_copy_kernel", "frames128"): 100829184,
 }
@@ -324,7 +307,7 @@ class Workload:
                 "bound": "tensor+hbm", "flops": float(np.sum(2.0 * (lens - k_e) * k_e * d)),
                 "bytes": float(Nv + n_out) * d * b,
                 "kernels": ["compress/merge_assign_mma_kernel", "compress/merge_assign_simt_kernel",
-                            "compress/merge_decode_kernel", "compress/merge_avg_kernel"]}
+                            "compress/merge_join_kernel", "compress/merge_avg_kernel"]}
         for i, s in enumerate(self.stages, start=1):
             kept = cfg.Lt + sum(min(bg, int((s["groups"] == g).sum().item())) for g, bg in enumerate(s["budgets"]))
             st[f"a5 attention scores, level {i}"] = {
@@ -342,7 +325,7 @@ class Workload:
             st["a8 K/V lists"] = {"bound": "latency", "bytes": 4.0 * Nv + 4.0 * cfg.L * kv_rows,
                                   "kernels": ["kv/class_topk_kernel", "kv/kv_paper_lists_kernel", "kv/kv_check_lists_kernel"]}
             st["a9 K/V in-place gather"] = {"bound": "hbm", "bytes": 2.0 * kv_rows * cfg.dh * b * 2 * cfg.Hkv * cfg.L,
-                                            "kernels": ["kv/kv_stage_kernel", "kv/kv_copy_kernel", "kv/kv_gather_kernel"]}
+                                            "kernels": ["kv/kv_stage_kernel", "kv/kv_copy_kernel", "kv/kv_gather_kernel", "kv/kv_paper_kernel"]}
         return st
 
 
