@@ -625,6 +625,7 @@ constexpr int kMmaBM = 256, kMmaBK = 64, kMmaBN = 256, kMmaMaxStages = 6;
 constexpr int kMmaThreads = 448;
 constexpr int kMmaKeyThreads = 128;                        // warps 10-13
 constexpr uint32_t kMmaRingBytes = 192 * 1024;
+constexpr int kMmaEvents = 512;                            // up to as many events' offsets are kept in shared memory
 constexpr size_t kMmaSmemBytes = kMmaRingBytes + 1024;
 // Unit shape of a launch: up to bm token rows (128 or 256) x up to bn keys (a multiple of 16), and what follows from it.
 struct MmaTile {
@@ -634,9 +635,9 @@ struct MmaTile {
 
 struct MergeUnit { int row_lo, row0, row_end, col0, nvalid, nchunks, slot0, slot_end; };   // the event's first row, the unit's rows; first key slot and number of keys; the event's chunks and slots
 
-__device__ __forceinline__ MergeUnit merge_unit(int u, const int32_t* __restrict__ ev_unit_off,
-                                                const int32_t* __restrict__ ev_lo,
-                                                const int32_t* __restrict__ ev_out_off, int k, int N, const MmaTile& mt) {
+__device__ __forceinline__ MergeUnit merge_unit(int u, const int32_t* ev_unit_off,
+                                                const int32_t* ev_lo,
+                                                const int32_t* ev_out_off, int k, int N, const MmaTile& mt) {
     const int e = find_event(ev_unit_off, k, u);
     const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0;
     const int nchunks = (nk + mt.bn - 1) / mt.bn;
@@ -658,8 +659,8 @@ __device__ __forceinline__ MergeUnit merge_unit(int u, const int32_t* __restrict
 __global__ void __launch_bounds__(kMmaThreads, 1)
 merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA_half,
                         const __nv_bfloat16* __restrict__ feats, int d, int N,
-                        const int32_t* __restrict__ ev_lo, int k, const int32_t* __restrict__ ev_out_off,
-                        const int32_t* __restrict__ ev_unit_off, const float* __restrict__ inv_norm, MmaTile mt,
+                        const int32_t* ev_lo, int k, const int32_t* ev_out_off,
+                        const int32_t* ev_unit_off, const float* __restrict__ inv_norm, MmaTile mt,
                         TokenOut out, int32_t* __restrict__ status) {
     grid_dep_wait();
     using namespace sm100;
@@ -671,6 +672,22 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     __shared__ __align__(16) float s_keyinv[2][kMmaBN];
     const int kMmaStages = mt.stages;
 
+    // The events' offsets: every role looks a unit up, in a chain of log2(k) + 2 dependent reads that the copies of a
+    // unit's first stages wait for (400 x 100 tokens of 512 in 100 events: 86.7 us the whole path with the reads from
+    // global memory, 85.4 from shared memory; 127 x 174 of 1992 in 19: 193.5 and 192.6).
+    __shared__ int32_t s_off[3][kMmaEvents + 1];
+    if (k <= kMmaEvents) {
+        for (int i = threadIdx.x; i <= k; i += kMmaThreads) {
+            const int32_t a = ev_unit_off[i], b = ev_lo[i], c = ev_out_off[i];
+            s_off[0][i] = a;
+            s_off[1][i] = b;
+            s_off[2][i] = c;
+        }
+        __syncthreads();
+        ev_unit_off = s_off[0];
+        ev_lo = s_off[1];
+        ev_out_off = s_off[2];
+    }
     const int total_units = ev_unit_off[k];
     if ((int)blockIdx.x >= total_units) return;
     const int ksteps = (d + kMmaBK - 1) / kMmaBK;
@@ -819,10 +836,11 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
             const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
             const int b = n & 1;                                    // s_keyinv alternates: a slow warp may still read the last one
             s_keyinv[b][et] = (et < mu.nvalid) ? inv_norm[out_src[mu.col0 + et]] : 0.f;
+            const int row = mu.row0 + half * 128 + grp * 32 + lane;
+            const bool is_key = row >= mu.row_end || out.is_key[row];   // on its way while the products are made
             named_bar_sync(1, 256);
             if (ok && !mbar_wait(smem_u32(&tfull_bar), (uint32_t)n & 1u, abort_flag)) ok = false;
             ok = __all_sync(0xFFFFFFFFu, ok);                      // tcgen05.ld below is warp-collective
-            const int row = mu.row0 + half * 128 + grp * 32 + lane;
             // the second accumulator of a short unit holds nothing
             const bool mine = half == 0 || (mt.bm > 128 && mu.row_end - mu.row0 > 128);
             float best_v = -3.4e38f;
@@ -875,7 +893,7 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                 if (lane == 0) mbar_arrive(smem_u32(&tempty_bar));
             }
             // (a warp that gave up keeps meeting the others at the named barriers)
-            const bool have = ok && mine && row < mu.row_end && !out.is_key[row];
+            const bool have = ok && mine && !is_key;
             int slot = mu.col0 + best_c;
             bool last = true;
             if (mu.nchunks > 1) {
