@@ -404,16 +404,17 @@ extern "C" int metok_segment_events(const void* feats, int dtype, int T, int N, 
 // flight) and the sums run on the tensor cores.  A warp owns one position and
 // EIGHT consecutive frames; a stage holds 512 contiguous bytes of those eight rows and
 // of the frame before them (one copy instruction per row, 16 bytes per lane: the memory
-// system sees long pieces of a row).  All three sums come out of one m16n8k16 mma per 16
-// elements: B is the eight frames (columns), A the same eight frames (rows 0-7), the text
-// (row 8) and the frame before the run (row 9; rows 10-15 repeat the text and are not
-// read).  C then holds the squared norms on its diagonal, the dots of neighbouring frames
-// next to it, <text, frame> in row 8 and the first frame's dot with its predecessor at
-// C[9][0].  One ldmatrix brings A as it is needed, and two of its four registers are B.
-// Products of bf16 are exact in fp32 and the sums are fp32 (two accumulators, even and
-// odd steps).  The kernel is meant to be bound by HBM; with a separate mma for each of the
-// three sums and each half of a 16-byte chunk (54 instructions per 64 bytes of a row, eight
-// warps an SM) it was bound by instruction latency: 512 x 144 rows of 1024 in 41 us.
+// system sees long pieces of a row).  A stage is consumed as eight 64-byte slices, two m16n8k16 mma each, and all three
+// sums come out of the same mma: B is the eight frames (columns), A the same eight frames (rows 0-7), the text (row 8) and
+// the frame before the run (row 9; rows 10-15 repeat the text and are not read).  C then holds the squared norms on its
+// diagonal, the dots of neighbouring frames next to it, <text, frame> in row 8 and the first frame's dot with its
+// predecessor at C[9][0].  Lane (g, q) = (lane / 4, lane % 4) reads chunk q of frame g's slice (dwords m0..m3) and chunk q
+// of row 8 + g (t0..t3); the order of k inside a dot product is free as long as both operands use the same one, so the
+// first mma takes (m0, t0, m2, t2) as A and (m0, m2) as B, the second the odd dwords: nothing is rearranged between lanes.
+// Products of bf16 are exact in fp32 and the sums are fp32 (an accumulator for the even dwords, one for the odd ones).
+// The kernel is meant to be bound by HBM; with separate mma for each of the three sums (54 instructions per 64 bytes
+// of a row, eight warps an SM) it was bound by instruction latency: 512 x 144 rows of 1024 in 41.7 us, 31 now; 128 x 144 of
+// 3584 30.7 and 27.
 // --------------------------------------------------------------------------- //
 namespace metok {
 
@@ -520,14 +521,6 @@ __device__ __forceinline__ void mma_bf16_m16n8k16(float (&c)[4], const uint4& a,
         : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
-// Four 8 x 8 matrices of 16-bit elements; lane l names row l % 8 of matrix l / 8 (16 bytes).
-__device__ __forceinline__ uint4 ldmatrix_x4(uint32_t row) {
-    uint4 r;
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(row) : "memory");
-    return r;
-}
-
 // 16-byte asynchronous copy global -> shared that bypasses L1; src_bytes = 0 writes zeros.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
@@ -540,7 +533,7 @@ constexpr int kFsCtasPerSm = 2;                    // what the rings leave room 
 constexpr int kFsDepth = 4;                        // stages of a warp's ring
 constexpr int kFsFrames = 8;                       // frames per warp = row groups of the mma tile
 constexpr int kFsSlices = 8;                       // 64-byte slices of a row per stage: 512 contiguous bytes
-constexpr int kFsRowPitch = kFsSlices * 64 + 16;   // bytes between a stage's rows (see the bank note in the kernel)
+constexpr int kFsRowPitch = kFsSlices * 64 + 64;   // bytes between a stage's rows (see the bank note in the kernel)
 constexpr int kFsStageBytes = (kFsFrames + 1) * kFsRowPitch;
 
 // Shared memory: the text embedding, zero-padded to whole slices; then per warp kFsDepth
@@ -570,15 +563,13 @@ seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat1
     // Copies: a stage holds 512 contiguous bytes (eight 64-byte slices) of each of the nine rows -- the
     // frame before the run, then the run's eight frames.  One copy instruction moves a row's 512 bytes
     // (16 per lane), so what reaches the memory system is long contiguous pieces of a row.  Rows of a
-    // stage lie kFsRowPitch bytes apart: 16 more than a multiple of 128, so that the eight rows of an
-    // 8 x 8 matrix lie in different banks.
+    // stage lie kFsRowPitch bytes apart: with 16 words more than a multiple of 32 the 16-byte reads of
+    // the eight lanes of a quarter warp (two frames, four chunks each) fall into different banks.
     unsigned char* ring = s_dyn + (size_t)nslice * 4 * sizeof(uint4) + (size_t)warp * kFsDepth * kFsStageBytes;
     const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + (uint32_t)lane * 16u;
-    // ldmatrix: lanes 0-7 and 16-23 name the frames' rows (first and second 16 bytes of a step), lanes 9 and 25 the
-    // row of the frame before them, the other lanes the text
-    const bool on_text = (lane & 8) != 0 && (lane & 7) != 1;
-    const uint32_t ld_row = dst - (uint32_t)lane * 16u + (uint32_t)((lane & 8) ? 0 : (lane & 7) + 1) * kFsRowPitch + (uint32_t)(lane >> 4) * 16u;
-    const uint32_t ld_text = static_cast<uint32_t>(__cvta_generic_to_shared(s_text)) + (uint32_t)(lane >> 4) * 16u;
+    const unsigned char* mine = ring + (g + 1) * kFsRowPitch + q * 16;
+    // row 8 + g of A: the frame before the run (g = 1) or the text
+    const unsigned char* other = g == 1 ? ring + q * 16 : reinterpret_cast<const unsigned char*>(s_text) + q * 16;
     // the copies run kFsDepth - 1 pieces ahead of the sums, into the next units too
     int i_unit = blockIdx.x, i_left = 0, i_lo = 0, i_hi = 0;
     int i_chunk = lane;                                     // this lane's chunk of the next piece's rows
@@ -658,20 +649,22 @@ seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat1
         const int f0 = run * kFsFrames;
         const int f = f0 + g;                               // this lane's frame
         const bool has = p < N && f < Tn;
-        float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};   // even and odd steps of 16 elements
+        float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};   // even and odd dwords
 #pragma unroll 1
         for (int sup = 0; sup < nsuper; ++sup) {
             cp_async_wait<kFsDepth - 2>();                  // this lane's copies of the piece have landed
             __syncwarp();                                   // ... and every lane's; the piece before it has been read by all
             issue();                                        // into the stage that held the piece before
-            const uint32_t at = on_text ? ld_text + (uint32_t)sup * (kFsSlices * 64u) : ld_row + stage;
+            const unsigned char* at = mine + stage;
+            const unsigned char* at2 = other + (g == 1 ? (int)stage : sup * (kFsSlices * 64));
             stage = stage == (kFsDepth - 1) * kFsStageBytes ? 0u : stage + kFsStageBytes;
 #pragma unroll
             for (int i = 0; i < kFsSlices; ++i) {
                 if (kFull || sup * kFsSlices + i < nslice) {
-                    const uint4 x0 = ldmatrix_x4(at + i * 64u), x1 = ldmatrix_x4(at + i * 64u + 32u);
-                    mma_bf16_m16n8k16(acc[0], x0, x0.x, x0.z);
-                    mma_bf16_m16n8k16(acc[1], x1, x1.x, x1.z);
+                    const uint4 x = *reinterpret_cast<const uint4*>(at + i * 64);
+                    const uint4 y = *reinterpret_cast<const uint4*>(at2 + i * 64);
+                    mma_bf16_m16n8k16(acc[0], make_uint4(x.x, y.x, x.z, y.z), x.x, x.z);
+                    mma_bf16_m16n8k16(acc[1], make_uint4(x.y, y.y, x.w, y.w), x.y, x.w);
                 }
             }
         }
