@@ -100,9 +100,11 @@ seg_partial_kernel(const T* __restrict__ feats, int Tn, long long chunks_per_fra
     }
 }
 
-// MEANPOOL: mean over the N tokens of each frame, per 16-byte column chunk.
+// MEANPOOL: mean over the N tokens of each frame, a thread per 16-byte column chunk, sixteen rows' loads in flight (one
+// at a time, a thread's chain of N round trips was what the kernel lasted), added in row order.
+constexpr int kMeanThreads = 64, kMeanRows = 16;
 template <typename T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kMeanThreads)
 seg_mean_kernel(const T* __restrict__ feats, int N, int d, float* __restrict__ mean) {
     grid_dep_wait();
     constexpr int VN = Vec16<T>::N;
@@ -112,11 +114,20 @@ seg_mean_kernel(const T* __restrict__ feats, int N, int d, float* __restrict__ m
     const T* base = feats + ((size_t)f * N) * d + (size_t)c * VN;
     float acc[VN];
     Vec16<T>::zero(acc);
-    for (int p = 0; p < N; ++p) {
-        float v[VN];
-        Vec16<T>::load(base + (size_t)p * d, v);
+    for (int p0 = 0; p0 < N; p0 += kMeanRows) {
+        uint4 raw[kMeanRows];
 #pragma unroll
-        for (int e = 0; e < VN; ++e) acc[e] += v[e];
+        for (int u = 0; u < kMeanRows; ++u)
+            if (p0 + u < N) raw[u] = __ldg(reinterpret_cast<const uint4*>(base + (size_t)(p0 + u) * d));
+#pragma unroll
+        for (int u = 0; u < kMeanRows; ++u) {
+            if (p0 + u < N) {
+                float v[VN];
+                widen16<T>(raw[u], v);
+#pragma unroll
+                for (int e = 0; e < VN; ++e) acc[e] += v[e];
+            }
+        }
     }
     const float inv = 1.0f / (float)N;
 #pragma unroll
@@ -319,10 +330,10 @@ static int launch_segment(const void* feats, int Tn, int N, int d, int k, int si
         part_dot = cv.take<float>((size_t)Tn);
         part_nrm = cv.take<float>((size_t)Tn);
         float* mean = cv.take<float>((size_t)Tn * d);
-        dim3 grid(ceil_div(d / VN, 128), Tn);
+        dim3 grid(ceil_div(d / VN, kMeanThreads), Tn);
         {
             METOK_TIMED("seg_mean_kernel", st);
-            launch_chained(seg_mean_kernel<T>, grid, dim3(128), 0, st, reinterpret_cast<const T*>(feats), N, d, mean);
+            launch_chained(seg_mean_kernel<T>, grid, dim3(kMeanThreads), 0, st, reinterpret_cast<const T*>(feats), N, d, mean);
         }
         METOK_LAUNCH_CHECK();
         {

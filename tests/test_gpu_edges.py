@@ -157,3 +157,10 @@ def test_fp32_attention_scores_at_tile_edges(Hq, Hkv, Lt, dh, vis_start, n_vis):
     torch.cuda.synchronize()
     err = np.abs(got.double().cpu().numpy() - want).max() / want.max()
     assert err < 1e-5, err
+
+
+@pytest.mark.parametrize("N", [1, 15, 16, 17, 33])
+@pytest.mark.parametrize("d,dtype", [(8, "bf16"), (520, "bf16"), (516, "f32")])
+def test_segmentation_by_mean_frames_around_sixteen_rows(N, d, dtype):
+    V = np.random.default_rng(N * d).standard_normal((7, N, d)).astype(np.float32)
+    R.segment_case(O.round_bf16(V).astype(np.float32) if dtype == "bf16" else V, dtype, 3, sim_mode=1)
