@@ -83,14 +83,15 @@ __host__ AttnMmaDims make_mma_dims(int Hq, int Hkv, int Lt, int S, int vis_start
     return dm;
 }
 
-// Sum of 2^(v[j] * sc + add) over the 32 columns; every fourth pair's exponentials on the FMA pipe.
+// Sum of 2^(v[j] * sc + add) over the 32 columns; every fourth pair's exponentials on the FMA pipe.  Wherever an exponent is
+// above the range the sum is above 1e18, never below it.
 __device__ __forceinline__ float exp2_sum32(const uint32_t (&v)[32], uint64_t sc, uint64_t add) {
     using namespace sm100;
     uint64_t s0 = 0ull, s1 = 0ull;                             // {0.f, 0.f}
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
         const uint64_t x = fma_pair(pair(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), sc, add);
-        const uint64_t e = (j & 3) == 3 ? exp2_fma_pair(x) : exp2_pair(x);
+        const uint64_t e = (j & 3) == 3 ? exp2_fma_pair<true>(x) : exp2_pair(x);
         if (j & 1) s1 = add_pair(s1, e);
         else s0 = add_pair(s0, e);
     }
@@ -242,7 +243,7 @@ attn_stats_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 bool redo = !plain;
                 if (plain) {
                     const float sum = exp2_sum32(raw[ci & 1], pair(sc, sc), pair(-m_run, -m_run));
-                    redo = __any_sync(0xFFFFFFFFu, !(sum < 1.0e18f));
+                    redo = __any_sync(0xFFFFFFFFu, !(sum >= 0.f && sum < 1.0e18f));
                     if (!redo) l_run += sum;
                 }
                 if (redo) {
@@ -484,7 +485,7 @@ attn_colsum_mma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                         const uint64_t x0 = fma_pair(pair(__uint_as_float(r[0]), __uint_as_float(r[1])), sc2, nl.x);
                         const uint64_t x1 = fma_pair(pair(__uint_as_float(r[2]), __uint_as_float(r[3])), sc2, nl.y);
                         s0 = add_pair(s0, exp2_pair(x0));
-                        s1 = add_pair(s1, (c & 4) ? exp2_fma_pair(x1) : exp2_pair(x1));   // every fourth pair on the FMA pipe
+                        s1 = add_pair(s1, (c & 4) ? exp2_fma_pair<false>(x1) : exp2_pair(x1));   // every fourth pair on the FMA pipe; no logit is above the row's log-sum-exp
                     }
                 };
                 switch (width >> 3) {

@@ -241,16 +241,26 @@ __device__ __forceinline__ uint64_t add_pair(uint64_t a, uint64_t b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-// 2^x of both halves on the special-function unit, and on the FMA pipe (exp2_fma).
+// 2^x of both halves on the special-function unit, and on the FMA pipe (exp2_fma).  There the exponent is added as an
+// integer, which from x = 129 on runs into the sign bit: a huge argument would look like a small result.  kAbove: arguments
+// may be that large; they are held to 126, so that what comes out is 2^126 (two minima per pair: both passes of the attention
+// scores over 73 728 keys, 28 heads and 128 queries 163.8 -> 166 us with them in the first).
 __device__ __forceinline__ uint64_t exp2_pair(uint64_t x) {
     float a, b;
     unpair(x, a, b);
     return pair(fast_exp2(a), fast_exp2(b));
 }
+template <bool kAbove>
 __device__ __forceinline__ uint64_t exp2_fma_pair(uint64_t x) {
     float a, b;
     unpair(x, a, b);
-    x = pair(fmaxf(a, -125.0f), fmaxf(b, -125.0f));
+    a = fmaxf(a, -125.0f);
+    b = fmaxf(b, -125.0f);
+    if constexpr (kAbove) {
+        a = fminf(a, 126.0f);
+        b = fminf(b, 126.0f);
+    }
+    x = pair(a, b);
     const uint64_t t = add_pair(x, pair(12582912.0f, 12582912.0f));
     const uint64_t f = fma_pair(add_pair(t, pair(-12582912.0f, -12582912.0f)), pair(-1.0f, -1.0f), x);
     uint64_t p = pair(0.001326472731307149f, 0.001326472731307149f);

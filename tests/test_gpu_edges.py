@@ -113,6 +113,27 @@ def test_attention_scores_whose_logits_grow_along_the_keys(Hq, Hkv, Lt, dh, n_vi
     assert err < 2e-4, err
 
 
+@pytest.mark.parametrize("octaves", [50, 100, 128, 129, 130, 200, 255, 300, 400])
+@pytest.mark.parametrize("part", [0, 3])
+def test_attention_scores_with_one_key_far_above_the_first_tile(octaves, part):
+    """One key per head, each head another column of a 32-key chunk, in a key tile whose sums are taken against an earlier
+    tile's maximum: its logit leaves the range of every way in which a column's exponential is computed."""
+    H, Lt, dh, n_vis = 32, 4, 64, 1024                                  # five tiles of 256 keys, two per CTA: the second is 256..511
+    rng = np.random.default_rng(octaves + part)
+    Q = (0.3 * rng.standard_normal((H, Lt, dh))).astype(np.float32)
+    K = (0.3 * rng.standard_normal((H, n_vis + Lt, dh))).astype(np.float32)
+    Q[:, :, 0] = 8.0
+    K[:, :, 0] = 0.0
+    key = 256 + 64 * part + 32 * (part & 1) + np.arange(H)              # head h: column h of the chunk
+    K[np.arange(H), key, 0] = octaves * np.log(2.0)                     # times 8 / sqrt(64)
+    Qb, Kb = (torch.from_numpy(x).to(torch.bfloat16) for x in (Q, K))
+    want = O.attention_scores(Qb.float().numpy(), Kb.float().numpy(), 0, n_vis, dh ** -0.5)
+    got = B.metok_attention_scores(Qb.cuda(), Kb.cuda(), 0, n_vis, dh ** -0.5)
+    torch.cuda.synchronize()
+    err = np.abs(got.double().cpu().numpy() - want).max() / want.max()  # every raised key holds about 1/32 of the sum
+    assert err < 2e-4, err
+
+
 @pytest.mark.parametrize("T,N,d", [(1, 1, 8), (8, 4, 256), (9, 5, 264), (7, 3, 1032), (33, 241, 248), (250, 75, 40), (131, 150, 520)])
 def test_one_pass_segmentation_units(T, N, d):
     """Eight frames of four positions are a unit, a CTA takes every 296th: one unit, ragged ones, several per CTA."""
