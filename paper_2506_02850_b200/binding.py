@@ -236,7 +236,8 @@ def metok_compress_vision(feats: torch.Tensor, event_offsets: torch.Tensor, text
     """`scored` (the result of metok_segment_score_events on the same feats and text) makes the call
     skip its own scoring pass over `feats`; `key_events` (uint8 [k] on the device) replaces the
     call's own choice of key events, `key_frames` (uint8 [T], mode POOL) that of key frames.
-    "status" is the device status word (0, or -5 after a device-side timeout)."""
+    "status" is the device status word (0, -1 if `event_offsets` descend, or -5 after a device-side
+    timeout)."""
     res = _calls().compress_vision(feats, event_offsets, text_emb, p, cap, out, scored, key_events, key_frames)
     if type(res) is int:
         _check("metok_compress_vision", res)

@@ -95,6 +95,9 @@ __device__ __forceinline__ int find_event(const int32_t* __restrict__ off, int k
 
 // Event scores, key events, per-event token budgets and output offsets.  One CTA; with many frames a cluster, whose
 // other CTAs only average frames for it (512 frames: 13.4 us with one CTA, 6.5 with four).
+// The offsets are the caller's memory: they are held to [0, Tn], and where they descend (events that overlap would want
+// more outputs than the caller has room for) an offset is raised to the largest before it and the call's status word says
+// METOK_ERR_INVALID_ARG.  Events of no frames are taken as they are: no key token, no output.
 struct PlanParams {
     int Tn, N, k, n_key_events, event_agg, mode, tile_rows, chunk_cols;
     int rows_with_keys;                         // the merge's row tiles run over all tokens of an event (1) or only over those that are no key token (0)
@@ -125,11 +128,11 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
     // frame_score[f] = mean of the frame's N token scores; eight lanes per frame (a lane's loads are
     // independent), fixed shuffle tree; the scores stay in shared memory for the event loops below
     float* s_frame = s_score + k;           // [Tn]
-    int* s_evlo = reinterpret_cast<int*>(s_frame + Tn);     // [k] first frame of the event, clamped
-    int* s_evhi = s_evlo + k;                                // [k] one past its last frame
-    int* s_bud = s_evhi + k;                                 // [k] budget of the event
+    int* s_off = reinterpret_cast<int*>(s_frame + Tn);      // [k + 1] event_offsets, clamped
+    int* s_bud = s_off + k + 1;                              // [k] budget of the event
     int* s_units = s_bud + k;                                // [k] merge units of the event
     unsigned char* s_key = reinterpret_cast<unsigned char*>(s_units + k);   // [k]
+    for (int e = tid; e <= k; e += nthr) s_off[e] = min(max(event_offsets[e], 0), Tn);
     float* s_frame0 = s_frame;              // the first CTA's
     if (C > 1) {
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // everybody has started
@@ -164,13 +167,12 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
     } else {
         __syncthreads();
     }
+    bool descends = false;
     for (int e = tid; e < k; e += nthr) {
-        int lo = min(max(event_offsets[e], 0), Tn);
-        int hi = min(max(event_offsets[e + 1], lo), Tn);
+        const int lo = s_off[e], hi = s_off[e + 1];
+        descends |= hi < lo;
         ev_lo[e] = lo;
         if (e == k - 1) ev_lo[k] = hi;
-        s_evlo[e] = lo;
-        s_evhi[e] = hi;
         float s;
         if (hi <= lo) {
             s = -3.0e38f;
@@ -188,7 +190,16 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
         s_score[e] = s;
         event_score[e] = s;
     }
-    __syncthreads();
+    if (__syncthreads_or(descends)) {
+        if (tid == 0) {
+            for (int e = 1; e <= k; ++e) {
+                s_off[e] = max(s_off[e], s_off[e - 1]);
+                ev_lo[e] = s_off[e];
+            }
+            *status = METOK_ERR_INVALID_ARG;
+        }
+        __syncthreads();
+    }
     for (int e = tid; e < k; e += nthr) {
         const float v = s_score[e];
         int rank = 0;
@@ -203,7 +214,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
     __syncthreads();
     if (pp.mode == METOK_MODE_TOPK_MERGE) {
         for (int e = tid; e < k; e += nthr) {
-            const int m = (s_evhi[e] - s_evlo[e]) * pp.N;
+            const int m = (s_off[e + 1] - s_off[e]) * pp.N;
             const double ratio = s_key[e] ? pp.keep_key : pp.keep_nonkey;
             const double c = ratio * (double)m - 1e-9;
             long long b = (long long)c;
@@ -246,16 +257,12 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
         for (int f = tid; f < Tn; f += nthr) frame_ev[f] = 0;
         __syncthreads();
         for (int e = tid; e < k; e += nthr) {
-            const int lo = min(max(event_offsets[e], 0), Tn);
-            const int hi = min(max(event_offsets[e + 1], lo), Tn);
-            for (int f = lo; f < hi; ++f) frame_ev[f] = e;
+            for (int f = s_off[e]; f < s_off[e + 1]; ++f) frame_ev[f] = e;
         }
         __syncthreads();
         for (int f = tid; f < Tn; f += nthr) {
             const int e = frame_ev[f];
-            const int lo = min(max(event_offsets[e], 0), Tn);
-            const int hi = min(max(event_offsets[e + 1], lo), Tn);
-            const int len = hi - lo;
+            const int lo = s_off[e], hi = s_off[e + 1], len = hi - lo;
             const double c = pp.beta * (double)len - 1e-9;
             long long nk = (long long)c;
             if ((double)nk < c) nk += 1;
@@ -462,7 +469,51 @@ event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restri
     cluster_compact(cx, p_lo, p_hi, flag, emit, skip, sm);
 }
 
-// The same when the largest event a segmentation can produce fits select_cluster.cuh.
+// The same when the largest event a segmentation can produce fits select_cluster.cuh.  It has Tn - (k - 1) frames; offsets
+// with empty events can hold a longer one, which one CTA does from memory (cs_event_topk_long).
+__device__ __noinline__ void cs_event_topk_long(unsigned char* dyn, const float* __restrict__ sc, int lo, int n, int e, int budget,
+                                                int slot0, const TokenOut& out) {
+    uint32_t* hist = reinterpret_cast<uint32_t*>(dyn);                   // [256]: the layout's two sets of buckets are at least 512 words
+    uint32_t* warp_kept = hist + 256;                                    // [32]
+    uint32_t* state = warp_kept + 32;                                    // the digit found, items to take inside it
+    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
+    auto key_of = [&](int i) { return cs_key64(float_key(sc[i]), (uint32_t)i); };
+    // the budget-th largest key, eight bits at a time; keys are unique
+    unsigned long long thr = 0ull;
+    uint32_t need = (uint32_t)budget;
+    for (int shift = 56; budget < n && shift >= 0; shift -= 8) {
+        for (int b = tid; b < 256; b += nthr) hist[b] = 0u;
+        __syncthreads();
+        for (int i = tid; i < n; i += nthr) {
+            const unsigned long long key = key_of(i);
+            if (((key ^ thr) >> shift) < 256ull) atomicAdd(&hist[(uint32_t)(key >> shift) & 255u], 1u);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t b = 255u, left = need;
+            while (b > 0u && hist[b] < left) left -= hist[b--];
+            state[0] = b;
+            state[1] = left;
+        }
+        __syncthreads();
+        thr |= (unsigned long long)state[0] << shift;
+        need = state[1];
+    }
+    uint32_t base = 0u;                                                  // kept before the round's first item
+    for (int i0 = 0; i0 < n; i0 += nthr) {
+        const int i = i0 + tid;
+        const bool keep = i < n && key_of(i) >= thr;
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, keep);
+        if (lane == 0) warp_kept[warp] = (uint32_t)__popc(bal);
+        __syncthreads();
+        const uint32_t kept = lane < nwarps ? warp_kept[lane] : 0u;
+        const uint32_t before = base + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? kept : 0u) + __popc(bal & ((1u << lane) - 1u));
+        if (i < n) token_out(out, lo, n, i, e, slot0, (int)before, keep);
+        base += __reduce_add_sync(0xFFFFFFFFu, kept);
+        __syncthreads();
+    }
+}
+
 template <int IT, bool kCl>
 __device__ __forceinline__ void
 cs_event_topk(CsShared& sm, unsigned char* dyn, const CsLayout& lay, const float* __restrict__ sc, int lo, int n, int e,
@@ -479,7 +530,7 @@ template <int IT, bool kCl>
 __global__ void __launch_bounds__(IT == kCsMaxItems ? kCsMaxItemsThreads : 1024)
 cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restrict__ ev_lo, int N,
                      const int32_t* __restrict__ ev_budget, const int32_t* __restrict__ ev_out_off, CsLayout lay,
-                     TokenOut out) {
+                     const __grid_constant__ TokenOut out) {
     grid_dep_wait();
     __shared__ CsShared sm;
     extern __shared__ __align__(16) unsigned char sel_dyn[];
@@ -491,6 +542,10 @@ cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __res
     const int budget = ev_budget[e], slot0 = ev_out_off[e];
 #define METOK_EVENT_TOPK(ITEMS, CLUSTER, RANK) \
     cs_event_topk<ITEMS, CLUSTER>(sm, sel_dyn, lay, sc, lo, n, e, budget, slot0, RANK, out)
+    if (n > IT * C * (int)blockDim.x) {
+        if (rank == 0) cs_event_topk_long(sel_dyn, sc, lo, n, e, budget, slot0, out);
+        return;
+    }
     // most events are much shorter than the longest possible one: the cluster's first CTA takes them alone
     const bool solo = !kCl || n <= min(kCsSolo, 4 * (int)blockDim.x);
     if (solo) {
@@ -1514,7 +1569,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     pp.grid = 1;
     while (pp.grid * pp.grid < N) ++pp.grid;
     pp.s1 = p->s1; pp.s2 = p->s2; pp.s1_nonkey = p->s1_nonkey; pp.s2_nonkey = p->s2_nonkey;
-    const size_t plan_smem = (size_t)(k + Tn) * sizeof(float) + (size_t)k * (4 * sizeof(int) + 1);
+    const size_t plan_smem = (size_t)(k + Tn) * sizeof(float) + (size_t)k * (3 * sizeof(int) + 1) + sizeof(int);
     // more CTAs than one as soon as one would need more than two rounds for the frames
     const int plan_ctas = Tn <= 256 ? 1 : Tn <= 512 ? 4 : 8;
     if (plan_smem > 40 * 1024)
@@ -1544,7 +1599,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
 
     const TokenOut to = {w.is_key, out_src, out_event, assign, w.rest, w.best64, w.tile_done, w.ml};
     {
-        // an event has at most Tn - (k - 1) frames
+        // an event has at most Tn - (k - 1) frames if none is empty; cs_event_topk_long takes one that has more
         const long long longest = (long long)(Tn - (k - 1)) * N;
         const CsPlan plan = cs_plan(longest);
         if (plan.fits) {

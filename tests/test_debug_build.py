@@ -155,3 +155,14 @@ def test_no_index_leaves_its_range(debug_lib, case):
     words = B.workspace(1, Vd.device)[:16].view(torch.int32)
     assert int(words[0].item()) == 0 and int(words[2].item()) == 0
     _prefill_equal(pf, _normal_prefill(args))
+
+
+@pytest.mark.parametrize("offs", [[0, 0, 0, 10], [0, 10, 10, 10], [0, 7, 3, 10], [0, 10, 0, 10], [10, 0, 0, 0]])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_no_index_leaves_its_range_whatever_the_offsets(debug_lib, offs, dtype):
+    Vd, _, td, p = _vision_case(seed=21)
+    got = B.metok_compress_vision(Vd.to(dtype), torch.tensor(offs, dtype=torch.int32).cuda(), td.to(dtype), p)
+    torch.cuda.synchronize()
+    words = B.workspace(1, Vd.device)[:16].view(torch.int32)
+    assert int(words[0].item()) == (0 if sorted(offs) == offs else -1) and int(words[2].item()) == 0
+    assert int(got["n_out"].item()) <= B.metok_compress_vision_bound(10, 64, 3, p)

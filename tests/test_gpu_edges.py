@@ -185,3 +185,63 @@ def test_fp32_attention_scores_at_tile_edges(Hq, Hkv, Lt, dh, vis_start, n_vis):
 def test_segmentation_by_mean_frames_around_sixteen_rows(N, d, dtype):
     V = np.random.default_rng(N * d).standard_normal((7, N, d)).astype(np.float32)
     R.segment_case(O.round_bf16(V).astype(np.float32) if dtype == "bf16" else V, dtype, 3, sim_mode=1)
+
+
+@pytest.mark.parametrize("T,N,k", [
+    (40, 36, 30), (40, 1, 40), (120, 100, 60), (100, 360, 10), (100, 900, 10), (100, 1000, 10),   # each way of choosing key tokens
+])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_empty_events_and_one_longer_than_the_others_leave_room_for(T, N, k, dtype):
+    g = torch.Generator(device="cuda").manual_seed(T * N + k)
+    V = torch.randn((T, N, 8), device="cuda", generator=g).to(dtype)
+    t = torch.randn(8, device="cuda", generator=g).to(dtype)
+    lens = [0] * k
+    lens[k // 3], lens[k - 1] = T - 1, 1                                # the others hold no frame
+    offs = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    flags = np.zeros(k, np.uint8)
+    flags[[k // 3, 1]] = 1                                              # an empty one among the key events
+    kept = [k // 3, k - 1]
+    p = B.vision_params(0.5, 0.03, 0.02)
+
+    def call(offsets, key_events):
+        return B.metok_compress_vision(V, torch.from_numpy(offsets).cuda(), t, p, key_events=torch.from_numpy(key_events).cuda())
+
+    got, plain = call(offs, flags), call(np.array([0, T - 1, T], np.int32), flags[kept])
+    torch.cuda.synchronize()
+    n = int(plain["n_out"].item())
+    assert int(got["status"].item()) == 0 and int(got["n_out"].item()) == n
+    # the key tokens: the best scored of each event, the lower index on equal scores
+    score = got["token_score"].cpu().numpy()
+    want = []
+    for lo, hi, keep in ((0, (T - 1) * N, 0.03), ((T - 1) * N, T * N, 0.02)):
+        best = np.argsort(-score[lo:hi], kind="stable")[:max(1, int(np.ceil(keep * (hi - lo) - 1e-9)))]
+        want.append(np.sort(best) + lo)
+    assert np.array_equal(got["out_src"][:n].cpu().numpy(), np.concatenate(want))
+    assert torch.equal(got["out_event"][:n], torch.tensor(kept, device="cuda", dtype=torch.int32)[plain["out_event"][:n].long()])
+    for name in ("out_src", "out_members", "out_feats"):
+        assert torch.equal(got[name][:n], plain[name][:n]), name
+    assert torch.equal(got["assign"], plain["assign"])
+
+
+@pytest.mark.parametrize("offs", [[0, 30, 10, 40], [0, 40, 0, 40], [0, 41, -7, 40], [40, 40, 40, 0], [2 ** 31 - 1, -2 ** 31, 5, 40]])
+@pytest.mark.parametrize("mode", ["merge", "pool"])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_offsets_that_descend_are_refused_on_the_device(offs, mode, dtype):
+    """The status word says so, nothing is written past the rows that the bound promises, and the next call is clean."""
+    T, N, k = 40, 16, 3
+    g = torch.Generator(device="cuda").manual_seed(5)
+    V = torch.randn((T, N, 64), device="cuda", generator=g).to(dtype)
+    t = torch.randn(64, device="cuda", generator=g).to(dtype)
+    p = B.vision_params(0.5, 0.25, 0.25, mode=B.MODE_POOL if mode == "pool" else B.MODE_TOPK_MERGE)
+    good = torch.tensor([0, 10, 30, 40], dtype=torch.int32, device="cuda")
+    want = {key: v.clone() for key, v in B.metok_compress_vision(V, good, t, p).items() if torch.is_tensor(v)}
+    got = B.metok_compress_vision(V, torch.tensor(offs, dtype=torch.int32, device="cuda"), t, p)
+    torch.cuda.synchronize()
+    assert int(got["status"].item()) == -1
+    assert 0 <= int(got["n_out"].item()) <= got["out_src"].numel()
+    again = B.metok_compress_vision(V, good, t, p)
+    torch.cuda.synchronize()
+    n = int(want["n_out"].item())
+    assert int(again["status"].item()) == 0 and int(again["n_out"].item()) == n
+    for name in ("out_src", "out_event", "out_members", "out_feats"):
+        assert torch.equal(again[name][:n], want[name][:n]), name
