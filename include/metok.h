@@ -187,7 +187,8 @@ METOK_API int metok_segment_score_events(const void* feats, int dtype, int T, in
  *
  *   feats         DEVICE [T][N][d]                       (input)
  *   event_offsets DEVICE int32 [k+1] (from metok_segment_events, or the caller's own:  (input)
- *                 ascending in [0, T], events of no frames allowed.  Offsets outside [0, T] are
+ *                 ascending in [0, T], events of no frames allowed; tokens of frames that lie in
+ *                 no event have no part in the merge, their assign is not written.  Offsets outside [0, T] are
  *                 clamped; if they descend, the device status word (first int32 of ws, valid after
  *                 the stream is synchronised) reads METOK_ERR_INVALID_ARG and the results are not
  *                 valid, but nothing outside the caller's buffers is touched)

@@ -641,9 +641,10 @@ merge_join_kernel(int Nv, int N, const int32_t* __restrict__ ev_lo, int k, const
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= Nv || out.is_key[row]) return;
     const int e = find_event(ev_lo, k, row / N);
-    const int lo = ev_lo[e] * N, slot = (int32_t)(~(uint32_t)(out.best64[row] & 0xFFFFFFFFull));
+    const int lo = ev_lo[e] * N, hi = ev_lo[e + 1] * N, slot = (int32_t)(~(uint32_t)(out.best64[row] & 0xFFFFFFFFull));
+    if (row < lo || row >= hi) return;              // a token of no event (offsets that leave frames out): its scratch is not this call's
     out.assign[row] = slot;
-    if (slot >= ev_out_off[e] && slot < ev_out_off[e + 1]) members_join(out.ml, slot, row, row - lo, ev_lo[e + 1] * N - lo);
+    if (slot >= ev_out_off[e] && slot < ev_out_off[e + 1]) members_join(out.ml, slot, row, row - lo, hi - lo);
 }
 
 

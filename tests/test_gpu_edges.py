@@ -245,3 +245,23 @@ def test_offsets_that_descend_are_refused_on_the_device(offs, mode, dtype):
     assert int(again["status"].item()) == 0 and int(again["n_out"].item()) == n
     for name in ("out_src", "out_event", "out_members", "out_feats"):
         assert torch.equal(again[name][:n], want[name][:n]), name
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_frames_of_no_event_take_no_part(dtype):
+    T, N = 40, 24
+    g = torch.Generator(device="cuda").manual_seed(8)
+    V = torch.randn((T, N, 64), device="cuda", generator=g).to(dtype)
+    t = torch.randn(64, device="cuda", generator=g).to(dtype)
+    p = B.vision_params(0.5, 0.25, 0.25)
+    call = lambda v, offs: B.metok_compress_vision(v, torch.tensor(offs, dtype=torch.int32, device="cuda"), t, p)
+    want = call(V[5:35].contiguous(), [0, 15, 30])
+    call(V, [0, 20, 40])                                                # leaves its own scratch in the workspace
+    got = call(V, [5, 20, 35])
+    torch.cuda.synchronize()
+    n = int(want["n_out"].item())
+    assert int(got["status"].item()) == 0 and int(got["n_out"].item()) == n
+    assert torch.equal(got["out_src"][:n], want["out_src"][:n] + 5 * N)
+    for name in ("out_event", "out_members", "out_feats"):
+        assert torch.equal(got[name][:n], want[name][:n]), name
+    assert torch.equal(got["assign"][5 * N:35 * N], want["assign"])
