@@ -560,7 +560,7 @@ int launch_dh(const void* q_text, const void* k_all, const AttnMmaDims& dm, floa
 void attn_mma_workspace(int Hq, int Hkv, int Lt, int S, int n_vis, size_t* n_part_ml, size_t* n_part_col,
                         int* n_planes) {
     const AttnMmaDims dm = make_mma_dims(Hq, Hkv, Lt, S, 0, n_vis, 1.f);
-    *n_part_ml = (size_t)Hkv * dm.st_nsplit * 2 * dm.R;
+    *n_part_ml = (size_t)Hkv * dm.st_nsplit * dm.R;
     *n_planes = Hkv * dm.cs_nchunk;
     *n_part_col = (size_t)(*n_planes) * n_vis;
 }

@@ -8,6 +8,7 @@
 // partial sums go to the workspace and are added in a fixed order by the finishing
 // kernel, so the result does not depend on scheduling.
 #include "common.cuh"
+#include "sm100.cuh"
 
 namespace metok {
 
@@ -532,14 +533,6 @@ __device__ __forceinline__ void mma_bf16_m16n8k16(float (&c)[4], const uint4& a,
         : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
-// 16-byte asynchronous copy global -> shared that bypasses L1; src_bytes = 0 writes zeros.
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 constexpr int kFsCtasPerSm = 2;                    // what the rings leave room for
 constexpr int kFsDepth = 4;                        // stages of a warp's ring
 constexpr int kFsFrames = 8;                       // frames per warp = row groups of the mma tile
@@ -605,12 +598,12 @@ seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat1
             const uint32_t to = dst + i_stage;
             if (i_hi - i_lo == kFsFrames + 1) {
 #pragma unroll
-                for (int r = 0; r <= kFsFrames; ++r, src += step) cp_async16(to + r * kFsRowPitch, src, in ? 16u : 0u);
+                for (int r = 0; r <= kFsFrames; ++r, src += step) sm100::cp_async16_zfill(to + r * kFsRowPitch, src, in ? 16u : 0u);
             } else {                                        // rows that do not exist are written as zeros (0 bytes read)
 #pragma unroll 1
                 for (int r = 0; r <= kFsFrames; ++r) {
                     const bool ok = r >= i_lo && r < i_hi;
-                    cp_async16(to + r * kFsRowPitch, src, ok && in ? 16u : 0u);
+                    sm100::cp_async16_zfill(to + r * kFsRowPitch, src, ok && in ? 16u : 0u);
                     if (ok && r + 1 < i_hi) src += step;
                 }
             }
@@ -622,7 +615,7 @@ seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat1
                 if (i_unit < nunits) issue_unit();
             }
         }
-        cp_async_commit();
+        sm100::cp_async_commit();
     };
     if (i_unit < nunits) issue_unit();
 #pragma unroll 1
@@ -663,7 +656,7 @@ seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat1
         float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};   // even and odd dwords
 #pragma unroll 1
         for (int sup = 0; sup < nsuper; ++sup) {
-            cp_async_wait<kFsDepth - 2>();                  // this lane's copies of the piece have landed
+            sm100::cp_async_wait<kFsDepth - 2>();           // this lane's copies of the piece have landed
             __syncwarp();                                   // ... and every lane's; the piece before it has been read by all
             issue();                                        // into the stage that held the piece before
             const unsigned char* at = mine + stage;
@@ -708,7 +701,7 @@ seg_score_mma_kernel(const __nv_bfloat16* __restrict__ feats, const __nv_bfloat1
             if (ff > 0) part_dot[(size_t)pg * Tn + (ff - 1)] = dp;    // dots of frames ff-1 and ff, four positions
         }
     }
-    cp_async_wait<0>();
+    sm100::cp_async_wait_all();
 }
 
 // Frame runs sized so that all warps are resident at once: a second, partly filled wave of

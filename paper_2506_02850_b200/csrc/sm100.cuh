@@ -106,6 +106,9 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint32_t bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Waits until all but the newest `kPending` groups of this thread have landed; wait_all: all of its copies.
+template <int kPending>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ---- tcgen05 / TMEM --------------------------------------------------------------
@@ -206,23 +209,6 @@ __device__ __forceinline__ float fast_exp2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// 2^x for x < 127 on the FMA pipe instead of the special-function unit: round x to an integer with
-// the 1.5 * 2^23 trick, a degree-5 polynomial for 2^f on f in [-0.5, 0.5] (relative error 2e-7, that
-// of ex2.approx), and the integer added to the exponent.  Used for a share of an epilogue's
-// exponentials so that both pipes work.
-__device__ __forceinline__ float exp2_fma(float x) {
-    x = fmaxf(x, -125.0f);
-    const float t = x + 12582912.0f;
-    const float f = x - (t - 12582912.0f);
-    float p = 0.001326472731307149f;
-    p = fmaf(p, f, 0.009671512991189957f);
-    p = fmaf(p, f, 0.05550733581185341f);
-    p = fmaf(p, f, 0.24022242426872253f);
-    p = fmaf(p, f, 0.6931470036506653f);
-    p = fmaf(p, f, 1.0f);
-    return __int_as_float(__float_as_int(p) + (__float_as_int(t) << 23));
-}
-
 // ---- pairs of floats in 64-bit registers: one instruction for two multiply-adds or additions -------------------------
 // (the FMA pipe does them at the same rate per element; what a pair saves is the issue slot)
 __device__ __forceinline__ uint64_t pair(float lo, float hi) {
@@ -241,15 +227,18 @@ __device__ __forceinline__ uint64_t add_pair(uint64_t a, uint64_t b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-// 2^x of both halves on the special-function unit, and on the FMA pipe (exp2_fma).  There the exponent is added as an
-// integer, which from x = 129 on runs into the sign bit: a huge argument would look like a small result.  kAbove: arguments
-// may be that large; they are held to 126, so that what comes out is 2^126 (two minima per pair: both passes of the attention
-// scores over 73 728 keys, 28 heads and 128 queries 163.8 -> 166 us with them in the first).
+// 2^x of both halves on the special-function unit.
 __device__ __forceinline__ uint64_t exp2_pair(uint64_t x) {
     float a, b;
     unpair(x, a, b);
     return pair(fast_exp2(a), fast_exp2(b));
 }
+// The same for x < 127 on the FMA pipe: round x to an integer with the 1.5 * 2^23 trick, a degree-5 polynomial for 2^f on f in
+// [-0.5, 0.5] (relative error 2e-7, that of ex2.approx), and the integer added to the exponent.  Used for a share of an
+// epilogue's exponentials so that both pipes work.  The addition runs into the sign bit from x = 129 on: a huge argument
+// would look like a small result.  kAbove: arguments may be that large; they are held to 126, so that what comes out is
+// 2^126 (two minima per pair: both passes of the attention scores over 73 728 keys, 28 heads and 128 queries take 158 us
+// instead of 155.6 with them in the first).
 template <bool kAbove>
 __device__ __forceinline__ uint64_t exp2_fma_pair(uint64_t x) {
     float a, b;
@@ -292,16 +281,6 @@ __device__ __forceinline__ uint64_t make_desc_k128(uint32_t smem_addr_bytes) {
 // Instruction descriptor: A, B bf16 K-major, D fp32, shape M x N.
 __host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ bool elect_one() {
-    uint32_t pred;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "elect.sync _|p, 0xFFFFFFFF;\n\t"
-        "selp.b32 %0, 1, 0, p;\n\t}"
-        : "=r"(pred));
-    return pred != 0;
 }
 
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
