@@ -100,6 +100,7 @@ __device__ __forceinline__ int find_event(const int32_t* __restrict__ off, int k
 // METOK_ERR_INVALID_ARG.  Events of no frames are taken as they are: no key token, no output.
 struct PlanParams {
     int Tn, N, k, n_key_events, event_agg, mode, tile_rows, chunk_cols;
+    int wide_min, wide_max;                     // CUDA-core merge: units of 64 x 64 instead if there are this many of them (wide_max 0: never)
     int rows_with_keys;                         // the merge's row tiles run over all tokens of an event (1) or only over those that are no key token (0)
     int grid, s1, s2, s1_nonkey, s2_nonkey;     // POOL: side of the token grid and the four strides
     double keep_key, keep_nonkey, beta;
@@ -112,7 +113,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
                   const int32_t* __restrict__ event_offsets, PlanParams pp,
                   float* __restrict__ event_score, uint8_t* __restrict__ event_is_key,
                   int32_t* __restrict__ ev_lo, int32_t* __restrict__ ev_budget, int32_t* __restrict__ ev_out_off,
-                  int32_t* __restrict__ ev_unit_off,
+                  int32_t* ev_unit_off, int32_t* ev_wide_off,
                   int32_t* __restrict__ frame_ev, int32_t* __restrict__ frame_stride,
                   int32_t* __restrict__ frame_off, int32_t* __restrict__ n_out, int32_t* __restrict__ counters, int n_counters,
                   int32_t* __restrict__ status) {
@@ -123,6 +124,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
     if (rank == 0 && threadIdx.x == 0) *status = 0;
     for (int i = rank * 1024 + threadIdx.x; i < n_counters; i += C * 1024) counters[i] = 0;   // what later kernels of the call count in
     __shared__ int s_scan[32];
+    __shared__ int s_wide;
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int k = pp.k, Tn = pp.Tn;
     // frame_score[f] = mean of the frame's N token scores; eight lanes per frame (a lane's loads are
@@ -132,7 +134,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
     int* s_bud = s_off + k + 1;                              // [k] budget of the event
     int* s_units = s_bud + k;                                // [k] merge units of the event
     unsigned char* s_key = reinterpret_cast<unsigned char*>(s_units + k);   // [k]
-    for (int e = tid; e <= k; e += nthr) s_off[e] = min(max(event_offsets[e], 0), Tn);
+    const int off0 = tid <= k ? event_offsets[tid] : 0;     // on its way while the frames are averaged
     float* s_frame0 = s_frame;              // the first CTA's
     if (C > 1) {
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // everybody has started
@@ -160,6 +162,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
             frame_score[f] = s;
         }
     }
+    for (int e = tid; e <= k; e += nthr) s_off[e] = min(max(e == tid ? off0 : event_offsets[e], 0), Tn);
     if (C > 1) {
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -213,6 +216,10 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
     }
     __syncthreads();
     if (pp.mode == METOK_MODE_TOPK_MERGE) {
+        auto units = [&](int m, int b, int rows, int cols) {                 // row tiles x key chunks
+            return (m - (pp.rows_with_keys ? 0 : b) + rows - 1) / rows * ((b + cols - 1) / cols);
+        };
+        bool wide = false;
         for (int e = tid; e < k; e += nthr) {
             const int m = (s_off[e + 1] - s_off[e]) * pp.N;
             const double ratio = s_key[e] ? pp.keep_key : pp.keep_nonkey;
@@ -223,10 +230,21 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
             if (b > m) b = m;
             ev_budget[e] = (int)b;
             s_bud[e] = (int)b;
-            const int rows = m - (pp.rows_with_keys ? 0 : (int)b);
-            s_units[e] = (rows + pp.tile_rows - 1) / pp.tile_rows * (((int)b + pp.chunk_cols - 1) / pp.chunk_cols);   // row tiles x key chunks
+            s_units[e] = units(m, (int)b, pp.tile_rows, pp.chunk_cols);
+        }
+        if (pp.wide_max > 0) {
+            if (tid == 0) s_wide = 0;
+            __syncthreads();
+            int n = 0;
+            for (int e = tid; e < k; e += nthr) n += units((s_off[e + 1] - s_off[e]) * pp.N, s_bud[e], 64, 64);
+            if (n > 0) atomicAdd(&s_wide, n);
+            __syncthreads();
+            wide = s_wide >= pp.wide_min && s_wide <= pp.wide_max;
+            if (wide)
+                for (int e = tid; e < k; e += nthr) s_units[e] = units((s_off[e + 1] - s_off[e]) * pp.N, s_bud[e], 64, 64);
         }
         __syncthreads();
+        int32_t* unit_off = wide ? ev_wide_off : ev_unit_off;   // the other list is empty
         if (tid < 32) {                                     // offsets: one warp, 32 events at a time
             int slots = 0, units = 0;
             for (int e0 = 0; e0 < k; e0 += 32) {
@@ -239,14 +257,15 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
                 }
                 if (e < k) {
                     ev_out_off[e] = slots + bi - b;
-                    ev_unit_off[e] = units + ui - u;
+                    unit_off[e] = units + ui - u;
                 }
                 slots += __shfl_sync(0xFFFFFFFFu, bi, 31);
                 units += __shfl_sync(0xFFFFFFFFu, ui, 31);
             }
             if (tid == 0) {
                 ev_out_off[k] = slots;
-                ev_unit_off[k] = units;
+                (wide ? ev_unit_off : ev_wide_off)[k] = 0;
+                unit_off[k] = units;
                 *n_out = slots;
             }
         }
@@ -567,7 +586,8 @@ cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __res
 // Merge-assign on the CUDA cores (fp32 inputs; bf16 only when forced for debugging): fp32 products, added in
 // the order of the row, so every dot product is one chain of fused multiply-adds.
 //
-// Work unit = 8 P of an event's tokens that are no key tokens x 8 P of its key tokens (P = 2, 4 or 8: choose_simt_outputs);
+// Work unit = 8 P of an event's tokens that are no key tokens x 8 P of its key tokens (P = 2, 4 or 8: choose_simt_tile; where
+// the exact count decides, both kernels are launched and one finds no units);
 // the units of all events form one list, a CTA takes its first by its number and the others from a counter; the dot
 // products of a unit are SimtTile's.  Rows past a unit's end are copies of another row: nobody reads their results.
 // 61 x 169 tokens, d = 1156, fp32: 755 us with 64-row CTAs of 4 x 4 outputs per thread that each walked all keys
@@ -1435,7 +1455,7 @@ merge_avg_kernel(const T* __restrict__ feats, T* __restrict__ out_feats, AvgArgs
 struct VisionWs {
     int32_t* status;          // device status word, first in the workspace
     float* inv_norm;
-    int32_t *ev_lo, *ev_budget, *ev_out_off, *ev_unit_off;
+    int32_t *ev_lo, *ev_budget, *ev_out_off, *ev_unit_off, *ev_wide_off;   // ev_wide_off: ev_unit_off for units of 64 x 64
     int32_t *frame_ev, *frame_stride, *frame_off;   // POOL mode
     uint8_t* is_key;          // the rest: merging modes (TokenOut, MemberLists, AvgArgs)
     int32_t *rest, *tile_done;
@@ -1454,6 +1474,7 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
     w.ev_budget = cv.take<int32_t>((size_t)k + 1);
     w.ev_out_off = cv.take<int32_t>((size_t)k + 1);
     w.ev_unit_off = cv.take<int32_t>((size_t)k + 1);
+    w.ev_wide_off = cv.take<int32_t>((size_t)k + 1);
     w.frame_ev = cv.take<int32_t>((size_t)Tn);
     w.frame_stride = cv.take<int32_t>((size_t)Tn);
     w.frame_off = cv.take<int32_t>((size_t)Tn + 1);
@@ -1508,15 +1529,26 @@ static MmaTile choose_mma_tile(int Nv, int k, int d, double keep) {
 }
 
 // Outputs per thread (a side of the square) of the CUDA-core kernel, from the number of 64 x 64 units of the mean event.
-// Few of them leave SMs idle and last as long as one unit's chain of d steps: 16 x 16 units are then the fastest (5 frames
-// of 164 tokens, d = 2104, about 26 units: 161 us the call with 64 x 64, 76 with 32 x 32, 69 with 16 x 16; at about 94
-// units 146, 106 and 120).  Many small units read shared memory as fast as it goes and spread evenly; units of 64 x 64 do
-// a sixth more work in the same time but only where one round of CTAs does them all and is well filled (262 us against
-// 290 at 756 units; past the 888 places 308 against 290) -- events differ in length, hence not up to the last place.
-static int choose_simt_outputs(int Nv, int k, double keep) {
+// Few of them leave SMs idle and last as long as one unit's chain of d steps: 16 x 16 units are then the fastest.  The whole
+// call with 16 x 16 / 32 x 32 / 64 x 64, at that many units: 169 tokens of 1156, 34 units 42 / 48 / 96 us, 57: 51 / 49 / 96,
+// 103: 82 / 70 / 98; 100 tokens of 512, 36: 29 / 32 / 52, 75: 39 / 42 / 55, 98: 48 / 44 / 57.  From there on 32 x 32, except
+// where one round of CTAs does all 64 x 64 units and is well filled (they do a sixth more work in the same time; 32 x 32 /
+// 64 x 64 by their exact number: 690: 239 / 242 us, 738: 236 / 240, 766: 254 / 241, 784: 208 / 197, 846: 271 / 243,
+// 882: 130 / 117, 895: 130 / 184, 950: 294 / 375, 1056: 353 / 433 -- places = 888).  The estimate does not know the events'
+// lengths: within 2/3 and 0.9 of the places only one call in five has its exact number between 5/6 and all of them, and
+// with Zipf lengths 64 x 64 by the estimate alone took up to 35 % longer.  So there event_plan_kernel counts, and both
+// kernels are launched, 32 x 32 first (59 frames of 169 tokens of 1156, Zipf: 427 -> 318 us; 58 of 144 of 1024: 356 -> 243).
+// The second one costs nothing measurable where it finds no units, the first one 2 to 3.5 us where it finds none.
+struct SimtTileChoice { int outputs, wide_min, wide_max; };
+static SimtTileChoice choose_simt_tile(int Nv, int k, double keep) {
     const double m = (double)Nv / k, keys = std::max(1.0, keep * m), units = ((m - keys) / 64 + 0.5) * (keys / 64 + 0.5) * k;
-    const double places = kNumSMs * sa_ctas_per_sm(8);
-    return units < kNumSMs / 2 ? 2 : units < places * 2 / 3 || units > places * 0.9 ? 4 : 8;
+    const int places = kNumSMs * sa_ctas_per_sm(8);
+    SimtTileChoice c = {units < kNumSMs / 2 ? 2 : 4, 0, 0};
+    if (units >= places * 2 / 3 && units <= places * 0.9) {
+        c.wide_min = places * 5 / 6;
+        c.wide_max = places;
+    }
+    return c;
 }
 
 // The tensor-core merge path needs bf16 rows that TMA can address (16-byte row pitch);
@@ -1557,12 +1589,13 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     }
     const double keep = p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey;
     const MmaTile tile = choose_mma_tile(Nv, k, d, keep);
-    const int simt_pt = choose_simt_outputs(Nv, k, keep);
+    const SimtTileChoice simt = choose_simt_tile(Nv, k, keep);
     PlanParams pp;
     pp.Tn = Tn; pp.N = N; pp.k = k;
     pp.n_key_events = min(k, ceilq(p->alpha * (double)k));
-    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? tile.bm : 8 * simt_pt;
-    pp.chunk_cols = mma ? tile.bn : 8 * simt_pt;
+    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? tile.bm : 8 * simt.outputs;
+    pp.chunk_cols = mma ? tile.bn : 8 * simt.outputs;
+    pp.wide_min = simt.wide_min; pp.wide_max = mma ? 0 : simt.wide_max;
     pp.rows_with_keys = mma ? 1 : 0;
     pp.keep_key = p->keep_key; pp.keep_nonkey = p->keep_nonkey; pp.beta = p->beta;
     pp.key_given = p->key_events_given;
@@ -1578,7 +1611,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     {
         METOK_TIMED("event_plan_kernel", st);
         launch_chained_clusters(plan_ctas, event_plan_kernel, dim3(plan_ctas), dim3(1024), plan_smem, st, token_score, frame_score, event_offsets, pp, event_score,
-                       event_is_key, w.ev_lo, w.ev_budget, w.ev_out_off, w.ev_unit_off, w.frame_ev, w.frame_stride, w.frame_off,
+                       event_is_key, w.ev_lo, w.ev_budget, w.ev_out_off, w.ev_unit_off, w.ev_wide_off, w.frame_ev, w.frame_stride, w.frame_off,
                        n_out, w.ml.long_counter, w.n_counters, w.status);
     }
     METOK_LAUNCH_CHECK();
@@ -1645,13 +1678,19 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         }
         METOK_LAUNCH_CHECK();
     } else {
-        {
-            METOK_TIMED("merge_assign_simt_kernel", st);
-            auto kernel = simt_pt == 8 ? merge_assign_simt_kernel<T, 8> : simt_pt == 4 ? merge_assign_simt_kernel<T, 4> : merge_assign_simt_kernel<T, 2>;
-            launch_chained(kernel, dim3(kNumSMs * sa_ctas_per_sm(simt_pt)), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
-                           w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to);
-        }
-        METOK_LAUNCH_CHECK();
+        auto assign_units = [&](auto kernel, int outputs, const int32_t* unit_off) -> int {
+            {
+                METOK_TIMED("merge_assign_simt_kernel", st);
+                launch_chained(kernel, dim3(kNumSMs * sa_ctas_per_sm(outputs)), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
+                               w.ev_out_off, unit_off, inv_norm, w.unit_next, to);
+            }
+            METOK_LAUNCH_CHECK();
+            return METOK_OK;
+        };
+        int rc = simt.outputs == 2 ? assign_units(merge_assign_simt_kernel<T, 2>, 2, w.ev_unit_off)
+                                   : assign_units(merge_assign_simt_kernel<T, 4>, 4, w.ev_unit_off);
+        if (rc == METOK_OK && pp.wide_max > 0) rc = assign_units(merge_assign_simt_kernel<T, 8>, 8, w.ev_wide_off);
+        if (rc != METOK_OK) return rc;
         {
             METOK_TIMED("merge_join_kernel", st);
             launch_chained(merge_join_kernel, dim3(ceil_div(Nv, 256)), dim3(256), 0, st, Nv, N, w.ev_lo, k, w.ev_out_off, to);

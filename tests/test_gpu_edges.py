@@ -164,6 +164,23 @@ def test_fp32_merge_units(T, N, k, d, keep):
     assert rep["assign_mismatches"] <= rep["assign_near_ties"]
 
 
+@pytest.mark.parametrize("N,keep,lens,units", [
+    (170, 0.25, [9, 12, 8, 11, 5], 612), (91, 0.25, [14, 41], 735), (84, 0.3, [24, 36], 740),        # 740 to 888 units of 64 x 64
+    (87, 0.25, [7, 47, 15], 888), (126, 0.25, [4, 12, 22, 23], 891), (128, 0.25, [3, 1, 10, 27, 25], 1155),   # are done as such
+])
+def test_fp32_merge_units_by_their_exact_number(N, keep, lens, units):
+    m = N * np.array(lens)
+    b = np.ceil(keep * m - 1e-9)
+    assert (np.ceil((m - b) / 64) * np.ceil(b / 64)).sum() == units
+    rng = np.random.default_rng(units)
+    V = rng.standard_normal((sum(lens), N, 20)).astype(np.float32)
+    t = rng.standard_normal(20).astype(np.float32)
+    V += 0.5 * t
+    rep = R.compress_case(V, t, np.concatenate([[0], np.cumsum(lens)]).astype(np.int32), "f32", 0.5, keep, keep)
+    assert rep["key_mismatches"] <= rep["key_near_ties"]
+    assert rep["assign_mismatches"] <= rep["assign_near_ties"]
+
+
 @pytest.mark.parametrize("Hq,Hkv,Lt,dh,vis_start,n_vis", [
     (1, 1, 1, 4, 0, 1), (2, 2, 31, 20, 33, 1), (3, 1, 11, 64, 31, 33), (8, 2, 8, 100, 64, 159), (40, 40, 3, 128, 5, 90),
     (1, 1, 2, 8, 0, 9000), (4, 1, 33, 12, 700, 3000),                    # more key tiles than runs of them
