@@ -394,7 +394,7 @@ pool_kernel(const T* __restrict__ feats, int d, int N, int G, const int32_t* __r
 // the first kAvgFew of them in order of arrival, a bit per block of the event that holds a member (an output
 // with more members is searched for there), and lists of the outputs with many.
 // --------------------------------------------------------------------------- //
-constexpr int kAvgFew = 128;       // members listed per output
+constexpr int kAvgFew = 128;       // members listed per output: 512 bytes of workspace each, whatever the output holds (see carve_vision)
 constexpr int kAvgHeavy = 16;      // outputs with more members are averaged by whole CTAs,
 constexpr int kAvgLong = kAvgFew;  // those with more than this in parts
 struct MemberLists {
@@ -1479,6 +1479,8 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
     w.frame_stride = cv.take<int32_t>((size_t)Tn);
     w.frame_off = cv.take<int32_t>((size_t)Tn + 1);
     if (merging) {
+        // 528 bytes per output, most of it the member list, beside rows of usually 2 KB and more: 7.5 MB for 512 frames of
+        // 144 tokens of which a fifth is kept, 300 MB for 8192 frames of which half is
         const size_t n = (size_t)cap + 64;
         w.is_key = cv.take<uint8_t>((size_t)Tn * N);
         w.rest = cv.take<int32_t>((size_t)Tn * N);
@@ -1504,7 +1506,11 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
 // bn * 0.27 ns (at least 24 ns), so large units do more per byte (256 x 256: 0.56 us per K block of 64 for 64 KB) --
 // but a launch lasts as long as the SM with the most of them, and with few events small units spread better: 32 frames
 // of 144 tokens in four events are 40 units of 256 x 173 or 76 of 128 x 173.  The shape with the
-// shortest estimated launch is taken, from the mean event; 1.5 us per unit for its start and its argmax.
+// shortest estimated launch is taken; 1.5 us per unit for its start and its argmax.
+// The number of units is a guess from the mean event, with half as many key chunks again for the long ones, because the
+// offsets are on the device: for the shape taken, four in five of 400 calls drawn over 4 to 512 frames lie between 0.56 and
+// 1.33 of the real number (median 1.0).  It is too high where events are of like length (32 frames: 96 for 76 units of
+// 128 x 256; 128 frames: 148 for 112 of 256 x 256) and too low for Zipf lengths (512 frames: 591 for 1468).
 static MmaTile choose_mma_tile(int Nv, int k, int d, double keep) {
     static const struct { int bm, bn; } shapes[] = {{256, 256}, {256, 128}, {128, 256}, {128, 128}, {128, 64}};
     const int m = ceil_div(Nv, k), keys = std::max(1, (int)(keep * m)), ksteps = ceil_div(d, kMmaBK);
@@ -1512,7 +1518,6 @@ static MmaTile choose_mma_tile(int Nv, int k, int d, double keep) {
     double best_us = 0.0;
     for (const auto& s : shapes) {
         const int chunks = ceil_div(keys, s.bn), cols = (ceil_div(keys, chunks) + 15) & ~15;
-        // events differ in length, and long ones have more row tiles and more chunks: half as many chunks again as the mean
         const double units = k == 1 ? (double)ceil_div(Nv, s.bm) * chunks : ((double)Nv / s.bm + 0.5 * k) * (1.5 * keys / s.bn + 0.5);
         const double fill = (s.bm + cols) * kMmaBK * 2 / 118e3, mma = (s.bm / 128) * 4 * std::max(0.024, cols * 0.272e-3);
         const double us = std::ceil(units / kNumSMs) * (ksteps * std::max(fill, mma) + 1.5);
