@@ -44,14 +44,30 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # captures (profiles/), keyed by (scope/kernel, workload); a kernel changed since its capture is left out
 # (its stage then reports traffic null).
 NCU_TRAFFIC_BYTES = {
-    ("prefill1/attn_score_reduce_kernel", "frames128"): 1189120,
-    ("prefill1/gather_rows_kernel", "frames128"): 53984512,
-    ("prefill2/attn_score_reduce_kernel", "frames128"): 442880,
+    ("segment/seg_score_kernel", "frames128"): 135844352,
+    ("segment/seg_finish_kernel", "frames128"): 61952,
+    ("compress/event_plan_kernel", "frames128"): 133376,
+    ("compress/event_topk_kernel", "frames128"): 140544,
+    ("compress/merge_assign_mma_kernel", "frames128"): 135850496,
+    ("compress/merge_avg_kernel", "frames128"): 140172032,
+    ("prefill1/attn_stats_mma_kernel", "frames128"): 19441152,
+    ("prefill1/attn_colsum_mma_kernel", "frames128"): 19510272,
+    ("prefill1/attn_score_reduce_kernel", "frames128"): 599040,
+    ("prefill1/class_topk_kernel", "frames128"): 211968,
+    ("prefill1/gather_rows_kernel", "frames128"): 53216768,
+    ("prefill2/attn_stats_mma_kernel", "frames128"): 7497472,
+    ("prefill2/attn_colsum_mma_kernel", "frames128"): 7582720,
+    ("prefill2/attn_score_reduce_kernel", "frames128"): 225792,
+    ("prefill2/class_topk_kernel", "frames128"): 119040,
     ("prefill2/gather_rows_kernel", "frames128"): 15964672,
-    ("prefill3/attn_score_reduce_kernel", "frames128"): 147456,
-    ("prefill3/gather_rows_kernel", "frames128"): 473344,
-    ("kv/kv_stage_kernel", "frames128"): 4828160,
-    ("kv/kv_copy_kernel", "frames128"): 100829184,
+    ("prefill3/attn_stats_mma_kernel", "frames128"): 2778880,
+    ("prefill3/attn_colsum_mma_kernel", "frames128"): 2806528,
+    ("prefill3/attn_score_reduce_kernel", "frames128"): 78336,
+    ("prefill3/class_topk_kernel", "frames128"): 66560,
+    ("prefill3/gather_rows_kernel", "frames128"): 473088,
+    ("kv/class_topk_kernel", "frames128"): 135680,
+    ("kv/kv_stage_kernel", "frames128"): 4830464,
+    ("kv/kv_copy_kernel", "frames128"): 100684032,
 }
 
 
