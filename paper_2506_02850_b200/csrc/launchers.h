@@ -28,8 +28,16 @@ int launch_gather_rows_bulk(const void* src, void* dst, const int32_t* idx, cons
 // (each) and of part_col.  `status` receives METOK_ERR_TIMEOUT if a device-side wait gave up.
 void attn_mma_workspace(int Hq, int Hkv, int Lt, int S, int n_vis, size_t* n_part_ml, size_t* n_part_col,
                         int* n_planes);
-int launch_attn_scores_mma(const void* q_text, const void* k_all, int Hq, int Hkv, int Lt, int S, int dh,
-                           int vis_start, int n_vis, float scale, float* part_m, float* part_l, float* part_col,
-                           int32_t* status, cudaStream_t st);
+// One call scores up to kMaxPruneLevels levels in its two launches: the same heads and text queries, keys and scratch of
+// their own.  Besides the status word it clears the class counts behind it.
+constexpr int kMaxPruneLevels = 3;
+constexpr int kStatusCounts = 4;                   // words of the status area: tokens of classes 0 and 1
+struct AttnScoreCall {
+    const void *q_text, *k_all;
+    int S, vis_start, n_vis;
+    float *part_m, *part_l, *part_col;
+};
+int launch_attn_scores_mma(const AttnScoreCall* calls, int n, int Hq, int Hkv, int Lt, int dh, float scale, int32_t* status,
+                           cudaStream_t st);
 
 }  // namespace metok

@@ -203,11 +203,31 @@ attn_colsum_kernel(const T* __restrict__ q_text, const T* __restrict__ k_all, At
     }
 }
 
+// scores[j] = inv_rows * (sum of the planes, in their order), for up to kMaxPruneLevels levels at once.  With `group`, the
+// blocks of the first level also write origin[j] = j and count the tokens of classes 0 and 1.
+struct ReduceLevel { const float* part_col; float* scores; int n_vis, block0; };   // block0: the level's first block
+struct ReduceArgs {
+    ReduceLevel lv[kMaxPruneLevels];
+    int nparts;
+    float inv_rows;
+    const int32_t* group;
+    int32_t *origin, *counts;
+};
 __global__ void __launch_bounds__(256)
-attn_score_reduce_kernel(const float* __restrict__ part_col, int nparts, int n_vis, float inv_rows,
-                         float* __restrict__ scores) {
+attn_score_reduce_kernel(ReduceArgs ra) {
     grid_dep_wait();
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    int level = 0;
+#pragma unroll
+    for (int l = 1; l < kMaxPruneLevels; ++l) level += (int)blockIdx.x >= ra.lv[l].block0;
+    const ReduceLevel lv = ra.lv[level];
+    const float* part_col = lv.part_col;
+    const int n_vis = lv.n_vis, nparts = ra.nparts, j = ((int)blockIdx.x - lv.block0) * 256 + (int)threadIdx.x;
+    if (ra.group && level == 0) {
+        const int g = j < n_vis ? ra.group[j] : -1;
+        const int c0 = __syncthreads_count(g == 0), c1 = __syncthreads_count(g == 1);
+        if (threadIdx.x < 2) atomicAdd(&ra.counts[threadIdx.x], threadIdx.x == 0 ? c0 : c1);
+        if (j < n_vis) ra.origin[j] = j;
+    }
     if (j >= n_vis) return;
     float a = 0.f;
     int p = 0;
@@ -219,7 +239,7 @@ attn_score_reduce_kernel(const float* __restrict__ part_col, int nparts, int n_v
         for (int u = 0; u < 8; ++u) a += v[u];
     }
     for (; p < nparts; ++p) a += part_col[(size_t)p * n_vis + j];
-    scores[j] = a * inv_rows;
+    lv.scores[j] = a * ra.inv_rows;
 }
 
 // --------------------------------------------------------------------------- //
@@ -390,54 +410,56 @@ int launch_class_topk(const float* scores, size_t score_stride, const int32_t* t
 
 // --------------------------------------------------------------------------- //
 // hidden_out[i] = hidden[keep_idx[i]], i < *S_out.  Rows are whole 16-byte chunks.
-// The gather is driven by the copy engine: one thread per CTA moves (row, 8 KiB segment)
+// The gather is driven by the copy engine: a worker is one thread, which moves (row, 8 KiB segment)
 // items global -> shared -> global with bulk copies, kGbStages items in flight; no registers
 // or warps are spent on the data.
 constexpr int kGbStages = 4;
 constexpr uint32_t kGbSegBytes = 8192;
-constexpr size_t kGbSmemBytes = (size_t)kGbStages * kGbSegBytes + 128;
+constexpr size_t kGbWorkerBytes = (size_t)kGbStages * kGbSegBytes;
+constexpr size_t kGbSmemBytes = kGbWorkerBytes + 128;
 
-__global__ void __launch_bounds__(32)
-gather_rows_bulk_kernel(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst,
-                        const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ n_rows,
-                        uint32_t row_bytes, int src_rows, int32_t* __restrict__ status) {
-    grid_dep_wait();
+constexpr int kGatherWorkersMax = 6;      // workers of a CTA, and of an SM
+struct GatherRows {
+    const uint8_t* src;
+    uint8_t* dst;
+    const int32_t *keep_idx, *n_rows;
+    uint32_t row_bytes;
+    int src_rows;
+    int32_t *status, *call_status;       // METOK_ERR_TIMEOUT to the first, and to the second if that is given and still 0
+};
+
+// Worker `first` of `stride`; stage0: its kGbWorkerBytes of shared memory, bars and abort_flag its own.
+__device__ __forceinline__ void gather_rows_worker(const GatherRows& ga, long long first, long long stride, uint32_t stage0,
+                                                   uint64_t* bars, volatile int* abort_flag) {
     using namespace sm100;
-    extern __shared__ uint8_t gb_dyn[];
-    __shared__ __align__(8) uint64_t s_bar[kGbStages];
-    __shared__ int s_abort;
-    if (threadIdx.x != 0) return;
-    const uint32_t stage0 = (smem_u32(gb_dyn) + 127u) & ~127u;
-    for (int j = 0; j < kGbStages; ++j) mbar_init(smem_u32(&s_bar[j]), 1);
-    s_abort = 0;
+    for (int j = 0; j < kGbStages; ++j) mbar_init(smem_u32(&bars[j]), 1);
+    *abort_flag = 0;
     mbar_fence_init();
-    const int nseg = (int)((row_bytes + kGbSegBytes - 1) / kGbSegBytes);
-    const long long items = (long long)(*n_rows) * nseg;
-    const long long first = blockIdx.x, stride = gridDim.x;
-    const long long mine = first < items ? (items - first + stride - 1) / stride : 0;   // items of this CTA
+    const int nseg = (int)((ga.row_bytes + kGbSegBytes - 1) / kGbSegBytes);
+    const long long items = (long long)(*ga.n_rows) * nseg;
+    const long long mine = first < items ? (items - first + stride - 1) / stride : 0;   // items of this worker
     auto issue_load = [&](long long k) {
         const long long it = first + k * stride;
         const int i = (int)(it / nseg), sg = (int)(it - (long long)i * nseg);
         const uint32_t off = (uint32_t)sg * kGbSegBytes;
-        const uint32_t bytes = min(kGbSegBytes, row_bytes - off);
-        const uint32_t bar = smem_u32(&s_bar[k % kGbStages]);
+        const uint32_t bytes = min(kGbSegBytes, ga.row_bytes - off);
+        const uint32_t bar = smem_u32(&bars[k % kGbStages]);
         mbar_arrive_expect_tx(bar, bytes);
-        const long long row = dbg_bound(keep_idx[i], src_rows, status);
-        if (!(dbg_withhold(status, kDbgGatherRows) && blockIdx.x == 0 && k == 0))   // debug builds: one copy never sent
-            bulk_load(stage0 + (uint32_t)(k % kGbStages) * kGbSegBytes, src + (size_t)row * row_bytes + off, bytes, bar);
+        const long long row = dbg_bound(ga.keep_idx[i], ga.src_rows, ga.status);
+        if (!(dbg_withhold(ga.status, kDbgGatherRows) && first == 0 && k == 0))   // debug builds: one copy never sent
+            bulk_load(stage0 + (uint32_t)(k % kGbStages) * kGbSegBytes, ga.src + (size_t)row * ga.row_bytes + off, bytes, bar);
     };
-    volatile int* abort_flag = &s_abort;
     for (long long k = 0; k < mine && k < kGbStages; ++k) issue_load(k);
     bool ok = true;
     for (long long k = 0; k < mine; ++k) {
         const int s = (int)(k % kGbStages);
-        if (!mbar_wait(smem_u32(&s_bar[s]), (uint32_t)(k / kGbStages) & 1u, abort_flag)) { ok = false; break; }
+        if (!mbar_wait(smem_u32(&bars[s]), (uint32_t)(k / kGbStages) & 1u, abort_flag)) { ok = false; break; }
         const long long it = first + k * stride;
         const int i = (int)(it / nseg), sg = (int)(it - (long long)i * nseg);
         const uint32_t off = (uint32_t)sg * kGbSegBytes;
-        const uint32_t bytes = min(kGbSegBytes, row_bytes - off);
+        const uint32_t bytes = min(kGbSegBytes, ga.row_bytes - off);
         fence_proxy_async();
-        bulk_store(dst + (size_t)i * row_bytes + off, stage0 + (uint32_t)s * kGbSegBytes, bytes);
+        bulk_store(ga.dst + (size_t)i * ga.row_bytes + off, stage0 + (uint32_t)s * kGbSegBytes, bytes);
         bulk_commit();
         // the stage of the item before this one is free once its store has read it
         if (k >= 1 && k - 1 + kGbStages < mine) {
@@ -448,22 +470,35 @@ gather_rows_bulk_kernel(const uint8_t* __restrict__ src, uint8_t* __restrict__ d
     bulk_wait_all();
     if (!ok) {
         // loads still in flight must land before the shared memory goes away
-        for (int j = 0; j < kGbStages; ++j) mbar_wait(smem_u32(&s_bar[j]), 0u, abort_flag);
-        *status = METOK_ERR_TIMEOUT;
+        for (int j = 0; j < kGbStages; ++j) mbar_wait(smem_u32(&bars[j]), 0u, abort_flag);
+        *ga.status = METOK_ERR_TIMEOUT;
+        if (ga.call_status) atomicCAS(ga.call_status, METOK_OK, METOK_ERR_TIMEOUT);
     }
 }
 
-int launch_gather_rows_bulk(const void* src, void* dst, const int32_t* idx, const int32_t* n_rows, size_t row_bytes,
-                            int src_rows, int32_t* status, const char* timer_name, cudaStream_t st) {
+__global__ void __launch_bounds__(32)
+gather_rows_bulk_kernel(const __grid_constant__ GatherRows ga) {
+    grid_dep_wait();
+    extern __shared__ uint8_t gb_dyn[];
+    __shared__ __align__(8) uint64_t s_bar[kGbStages];
+    __shared__ int s_abort;
+    if (threadIdx.x != 0) return;
+    gather_rows_worker(ga, blockIdx.x, gridDim.x, (sm100::smem_u32(gb_dyn) + 127u) & ~127u, s_bar, &s_abort);
+}
+
+static int launch_gather(const GatherRows& ga, const char* timer_name, cudaStream_t st) {
     METOK_ALLOW_SMEM(gather_rows_bulk_kernel, kGbSmemBytes);
     {
         METOK_TIMED(timer_name, st);
-        launch_chained(gather_rows_bulk_kernel, dim3(kNumSMs * 6), dim3(32), kGbSmemBytes, st, 
-            reinterpret_cast<const uint8_t*>(src), reinterpret_cast<uint8_t*>(dst), idx, n_rows, (uint32_t)row_bytes,
-            src_rows, status);
+        launch_chained(gather_rows_bulk_kernel, dim3(kNumSMs * 6), dim3(32), kGbSmemBytes, st, ga);
     }
     METOK_LAUNCH_CHECK();
     return METOK_OK;
+}
+int launch_gather_rows_bulk(const void* src, void* dst, const int32_t* idx, const int32_t* n_rows, size_t row_bytes,
+                            int src_rows, int32_t* status, const char* timer_name, cudaStream_t st) {
+    return launch_gather({reinterpret_cast<const uint8_t*>(src), reinterpret_cast<uint8_t*>(dst), idx, n_rows, (uint32_t)row_bytes,
+                          src_rows, status, nullptr}, timer_name, st);
 }
 
 static AttnDims make_dims(int Hq, int Hkv, int Lt, int S, int dh, int vis_start, int n_vis, float scale) {
@@ -511,19 +546,40 @@ static PrefillWs carve_prefill(Carver& cv, const AttnDims& dm, bool mma) {
     return w;
 }
 
-static int launch_score_reduce(const PrefillWs& w, const AttnDims& dm, float inv_rows, float* scores, cudaStream_t st) {
+// One level's scoring as run_attention_scores takes it.
+struct ScoreLevel {
+    const void *q_text, *k_all;
+    AttnDims dm;
+    PrefillWs w;                  // all levels of a call have the same status area
+    float* scores;
+};
+
+static int launch_score_reduce(const ScoreLevel* lv, int n, float inv_rows, const int32_t* group, int32_t* origin, cudaStream_t st) {
+    ReduceArgs ra = {};
+    int blocks = 0;
+    for (int l = 0; l < kMaxPruneLevels; ++l) {
+        ra.lv[l].block0 = l < n ? blocks : 0x7FFFFFFF;
+        if (l >= n) continue;
+        ra.lv[l].part_col = lv[l].w.part_col;
+        ra.lv[l].scores = lv[l].scores;
+        ra.lv[l].n_vis = lv[l].dm.n_vis;
+        blocks += ceil_div(lv[l].dm.n_vis, 256);
+    }
+    ra.nparts = lv[0].w.n_planes;                             // the same heads and queries on every level
+    ra.inv_rows = inv_rows;
+    ra.group = group;
+    ra.origin = origin;
+    ra.counts = lv[0].w.status + kStatusCounts;
     {
         METOK_TIMED("attn_score_reduce_kernel", st);
-        launch_chained(attn_score_reduce_kernel, dim3(ceil_div(dm.n_vis, 256)), dim3(256), 0, st, w.part_col, w.n_planes,
-                       dm.n_vis, inv_rows, scores);
+        launch_chained(attn_score_reduce_kernel, dim3(blocks), dim3(256), 0, st, ra);
     }
     METOK_LAUNCH_CHECK();
     return METOK_OK;
 }
 
 template <typename T>
-static int launch_attn_scores(const void* q_text, const void* k_all, const AttnDims& dm, const PrefillWs& w,
-                              float inv_rows, float* scores, cudaStream_t st) {
+static int launch_attn_passes(const void* q_text, const void* k_all, const AttnDims& dm, const PrefillWs& w, cudaStream_t st) {
     dim3 grid(dm.nsplit, dm.nrt, dm.Hkv);
     {
         METOK_TIMED("attn_stats_kernel", st);
@@ -537,27 +593,38 @@ static int launch_attn_scores(const void* q_text, const void* k_all, const AttnD
                        reinterpret_cast<const T*>(k_all), dm, w.part_m, w.part_l, w.part_col);
     }
     METOK_LAUNCH_CHECK();
-    return launch_score_reduce(w, dm, inv_rows, scores, st);
+    return METOK_OK;
 }
 
 }  // namespace metok
 
 using namespace metok;
 
-// a5 as the calls run it: the status word cleared, then the two passes and the plane sum;
-// scores[j] = inv_rows * (sum over this call's heads and text queries of the probabilities).
-static int run_attention_scores(const void* q_text, const void* k_all, int dtype, const AttnDims& dm,
-                                const PrefillWs& w, float softmax_scale, float inv_rows, float* scores,
-                                cudaStream_t st) {
-    const bool mma = use_mma_attn(dtype, dm.dh);
-    if (!mma) METOK_CUDA_TRY(cudaMemsetAsync(w.status, 0, sizeof(int32_t), st));   // else attn_stats_mma_kernel clears it
-    if (mma) {
-        const int rc = launch_attn_scores_mma(q_text, k_all, dm.Hq, dm.Hkv, dm.Lt, dm.S, dm.dh, dm.vis_start, dm.n_vis,
-                                              softmax_scale, w.part_m, w.part_l, w.part_col, w.status, st);
-        return rc == METOK_OK ? launch_score_reduce(w, dm, inv_rows, scores, st) : rc;
+// a5 as the calls run it, for one level or several: the status word and the class counts cleared, then the two passes and
+// the plane sum; scores[j] = inv_rows * (sum over this call's heads and text queries of the probabilities).  group, origin:
+// see attn_score_reduce_kernel.
+static int run_attention_scores(const ScoreLevel* lv, int n, int dtype, float softmax_scale, float inv_rows, const int32_t* group,
+                                int32_t* origin, cudaStream_t st) {
+    const AttnDims& dm = lv[0].dm;
+    int32_t* status = lv[0].w.status;
+    if (use_mma_attn(dtype, dm.dh)) {                         // attn_stats_mma_kernel does the clearing
+        AttnScoreCall calls[kMaxPruneLevels];
+        for (int l = 0; l < n; ++l)
+            calls[l] = {lv[l].q_text, lv[l].k_all, lv[l].dm.S, lv[l].dm.vis_start, lv[l].dm.n_vis, lv[l].w.part_m, lv[l].w.part_l,
+                        lv[l].w.part_col};
+        const int rc = launch_attn_scores_mma(calls, n, dm.Hq, dm.Hkv, dm.Lt, dm.dh, softmax_scale, status, st);
+        if (rc != METOK_OK) return rc;
+    } else {
+        // (words 1 and 2 belong to debug builds)
+        METOK_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
+        if (group) METOK_CUDA_TRY(cudaMemsetAsync(status + kStatusCounts, 0, 2 * sizeof(int32_t), st));
+        for (int l = 0; l < n; ++l) {
+            const int rc = dtype == METOK_F32 ? launch_attn_passes<float>(lv[l].q_text, lv[l].k_all, lv[l].dm, lv[l].w, st)
+                                              : launch_attn_passes<__nv_bfloat16>(lv[l].q_text, lv[l].k_all, lv[l].dm, lv[l].w, st);
+            if (rc != METOK_OK) return rc;
+        }
     }
-    return dtype == METOK_F32 ? launch_attn_scores<float>(q_text, k_all, dm, w, inv_rows, scores, st)
-                              : launch_attn_scores<__nv_bfloat16>(q_text, k_all, dm, w, inv_rows, scores, st);
+    return launch_score_reduce(lv, n, inv_rows, group, origin, st);
 }
 
 extern "C" size_t metok_prefill_prune_workspace_bytes(int dtype, int Hq, int Hkv, int Lt, int S, int dh, int n_vis) {
@@ -613,7 +680,8 @@ extern "C" int metok_prefill_prune(const void* q_text, const void* k_all, const 
     PrefillWs w = carve_prefill(cv, dm, use_mma_attn(dtype, dh));
     int rc = debug_arm(w.status, st);
     if (rc != METOK_OK) return rc;
-    rc = run_attention_scores(q_text, k_all, dtype, dm, w, softmax_scale, 1.0f / (float)(Hq * Lt), scores, st);
+    const ScoreLevel lv = {q_text, k_all, dm, w, scores};
+    rc = run_attention_scores(&lv, 1, dtype, softmax_scale, 1.0f / (float)(Hq * Lt), nullptr, nullptr, st);
     if (rc != METOK_OK) return rc;
     rc = launch_class_topk(scores, 0, token_group, n_vis, G, group_budget, S, vis_start, keep_idx, 0, 1, S_out,
                            nullptr, 1, st);
@@ -645,8 +713,8 @@ extern "C" int metok_attention_scores(const void* q_text, const void* k_all, int
     PrefillWs w = carve_prefill(cv, dm, use_mma_attn(dtype, dh));
     const float inv_rows = 1.0f / (float)(rows_total ? rows_total : Hq * Lt);
     if (const int rc = debug_arm(w.status, reinterpret_cast<cudaStream_t>(stream))) return rc;
-    return run_attention_scores(q_text, k_all, dtype, dm, w, softmax_scale, inv_rows, scores,
-                                reinterpret_cast<cudaStream_t>(stream));
+    const ScoreLevel lv = {q_text, k_all, dm, w, scores};
+    return run_attention_scores(&lv, 1, dtype, softmax_scale, inv_rows, nullptr, nullptr, reinterpret_cast<cudaStream_t>(stream));
 }
 
 extern "C" size_t metok_prune_by_scores_workspace_bytes(void) { return 1024; }
@@ -702,63 +770,168 @@ extern "C" int metok_retention_budgets(double alpha, double r, int stage, const 
 // --------------------------------------------------------------------------- //
 namespace metok {
 
-// One CTA: origin[i] = i, and the class counts of the first level against the caller's N0.  Eight groups of four tokens in
-// flight per thread (18 432 tokens: 11 us with one token at a time).
-__global__ void __launch_bounds__(1024)
-schedule_init_kernel(const int32_t* __restrict__ token_group, int n_vis, int n0_key, int n0_nonkey,
-                     int32_t* __restrict__ origin, int32_t* __restrict__ status) {
-    grid_dep_wait();
-    __shared__ int s_cnt[2];
-    if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
-    __syncthreads();
-    int c0 = 0, c1 = 0;
-    const bool vec = ((reinterpret_cast<uintptr_t>(token_group) | reinterpret_cast<uintptr_t>(origin)) & 15) == 0;
-    const int n4 = vec ? n_vis >> 2 : 0;
-    constexpr int U = 8;
-    for (int q0 = threadIdx.x; q0 < n4; q0 += 1024 * U) {
-        int4 g[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) g[u] = q0 + u * 1024 < n4 ? reinterpret_cast<const int4*>(token_group)[q0 + u * 1024] : make_int4(-1, -1, -1, -1);
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int q = q0 + u * 1024;
-            c0 += (g[u].x == 0) + (g[u].y == 0) + (g[u].z == 0) + (g[u].w == 0);
-            c1 += (g[u].x == 1) + (g[u].y == 1) + (g[u].z == 1) + (g[u].w == 1);
-            if (q < n4) reinterpret_cast<int4*>(origin)[q] = make_int4(4 * q, 4 * q + 1, 4 * q + 2, 4 * q + 3);
-        }
+// What a level hands to the next one and to the caller.
+struct ScheduleHand {
+    const int32_t *group, *origin;                    // of this level's tokens; origin null: the first level, token i is i
+    int32_t *group_next, *origin_next;                // of the next level's n_next tokens; null: no next level
+    int n_next;
+    const int32_t* level_status;                      // the attention passes' status word and the class counts behind it
+    int32_t* status;                                  // the caller's: written on the first level, later only if still 0
+    bool first;
+    int n0_key, n0_nonkey, n_vis;
+};
+__device__ __forceinline__ void schedule_check(const ScheduleHand& h) {
+    if (h.first) {
+        const int c0 = h.level_status[kStatusCounts], c1 = h.level_status[kStatusCounts + 1];
+        *h.status = c0 == h.n0_key && c1 == h.n0_nonkey && c0 + c1 == h.n_vis ? *h.level_status : METOK_ERR_INVALID_ARG;
+    } else if (*h.level_status != METOK_OK) {
+        atomicCAS(h.status, METOK_OK, *h.level_status);
     }
-    for (int i = 4 * n4 + threadIdx.x; i < n_vis; i += 1024) {
-        origin[i] = i;
-        const int g = token_group[i];
-        c0 += g == 0;
-        c1 += g == 1;
-    }
-    c0 = __reduce_add_sync(0xFFFFFFFFu, c0);
-    c1 = __reduce_add_sync(0xFFFFFFFFu, c1);
-    if ((threadIdx.x & 31) == 0) { atomicAdd(&s_cnt[0], c0); atomicAdd(&s_cnt[1], c1); }
-    __syncthreads();
-    if (threadIdx.x == 0)
-        *status = (s_cnt[0] == n0_key && s_cnt[1] == n0_nonkey && s_cnt[0] + s_cnt[1] == n_vis) ? METOK_OK
-                                                                                                 : METOK_ERR_INVALID_ARG;
 }
 
-// Class and origin of the i-th surviving visual token: the keep list holds every position before
-// the visual span, so its entry vis_start + i is that token's position at the level before.
+// One level of a schedule: the class-wise selection of up to 81 920 items (as cs_topk_kernel), class and origin of every
+// survivor for the next level, and beside it the hidden rows of the level before.  CTAs 0 .. C - 1 select; each of the others runs
+// `workers` gather workers.  The selection is a chain of latencies in eight SMs or one and the gather is bound by memory, so
+// one hides the other (18 432 tokens, three levels: 8 + 16, 7.5 + 7.6 and 5 + 4 us one after the other, and 3 us for every
+// launch between that handed classes and origins on).
+template <int IT, bool kCl>
+__global__ void __launch_bounds__(IT == kCsMaxItems ? kCsMaxItemsThreads : 1024)
+schedule_select_kernel(const float* __restrict__ sc, int n_vis, CsLayout lay, TopkBudgets budgets, int S, int vis_start,
+                       int32_t* __restrict__ keep, int32_t* __restrict__ S_out, const __grid_constant__ ScheduleHand hand,
+                       const __grid_constant__ GatherRows ga, int workers) {
+    cs_enter<kCl>();
+    grid_dep_wait();
+    constexpr int C = kCl ? kCsMaxCluster : 1;
+    __shared__ CsShared sm;
+    __shared__ __align__(8) uint64_t s_bar[kGatherWorkersMax][kGbStages];
+    __shared__ int s_abort[kGatherWorkersMax];
+    extern __shared__ __align__(16) unsigned char sel_dyn[];
+    const int tid = threadIdx.x, nthr = blockDim.x, rank = blockIdx.x;
+    if (rank >= C) {
+        const int w = tid >> 5;
+        if (w < workers && (tid & 31) == 0)
+            gather_rows_worker(ga, (long long)(rank - C) * workers + w, (long long)(gridDim.x - C) * workers,
+                               ((sm100::smem_u32(sel_dyn) + 127u) & ~127u) + (uint32_t)(w * kGbWorkerBytes), s_bar[w], &s_abort[w]);
+        __syncwarp();
+        if constexpr (kCl) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // of cs_enter()
+        return;
+    }
+    if (rank == 0 && tid == 0) schedule_check(hand);
+    const int32_t* group = hand.group;
+    const CsSlice sl = cs_slice<IT>(n_vis, rank, C);
+    auto load = [&](int i, float& v, int& c) {
+        v = sc[i];
+        c = group[i];
+        if (c >= 2) c = -1;
+    };
+    int before, kept;
+    const uint32_t bits = cs_select<IT, kCl, false>(sm, sel_dyn, lay, 2, budgets.v, rank, sl.i_first, sl.i_hi, load, &before, &kept);
+    const int outside = S - n_vis;
+    cs_for_items<IT>(bits, before, sl.i_first, sl.i_hi, [&](int, int i, int place, bool k) {
+        if (!k) return;
+        keep[vis_start + place] = vis_start + i;
+        if (hand.group_next && place < hand.n_next) {
+            hand.group_next[place] = group[i];
+            hand.origin_next[place] = hand.origin ? hand.origin[i] : i;
+        }
+    });
+    for (int i = rank * nthr + tid; i < outside; i += C * nthr)
+        keep[i < vis_start ? i : kept + i] = i < vis_start ? i : i + n_vis;
+    if (hand.group_next)                                      // fewer survivors than N0 says (the status word says so)
+        for (int i = kept + rank * nthr + tid; i < hand.n_next; i += C * nthr) {
+            hand.group_next[i] = group[n_vis - 1];
+            hand.origin_next[i] = hand.origin ? hand.origin[n_vis - 1] : n_vis - 1;
+        }
+    if (rank == 0 && tid == 0) *S_out = outside + kept;
+}
+
+// After a selection by select.cuh (a level of more than 81 920 tokens): class and origin of the i-th surviving visual token.
+// The keep list holds every position before the visual span, so its entry vis_start + i is that token's position.
 __global__ void __launch_bounds__(256)
-schedule_propagate_kernel(const int32_t* __restrict__ keep_idx, int vis_start, int n_cur, int n_next,
-                          const int32_t* __restrict__ group, const int32_t* __restrict__ origin,
-                          int32_t* __restrict__ group_next, int32_t* __restrict__ origin_next,
-                          const int32_t* __restrict__ level_status, int32_t* __restrict__ status) {
+schedule_propagate_kernel(const int32_t* __restrict__ keep_idx, int vis_start, int n_cur, const __grid_constant__ ScheduleHand hand) {
     grid_dep_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    // a level that gave up on a wait leaves its code in its own status word, which the next level
-    // clears: the first failure is kept in the caller's
-    if (i == 0 && *level_status != METOK_OK && *status == METOK_OK) *status = *level_status;
-    if (i >= n_next) return;
+    if (i == 0) schedule_check(hand);
+    if (!hand.group_next || i >= hand.n_next) return;
     int j = keep_idx[vis_start + i] - vis_start;
     j = j < 0 ? 0 : (j >= n_cur ? n_cur - 1 : j);            // only reached with a wrong N0 (status says so)
-    group_next[i] = group[j];
-    origin_next[i] = origin[j];
+    hand.group_next[i] = hand.group[j];
+    hand.origin_next[i] = hand.origin ? hand.origin[j] : j;
+}
+
+// The selection of one level; `ga` (may be null): the gather that runs beside it.
+static int launch_schedule_select(const float* scores, int n_vis, const int32_t* budget, int S, int vis_start, int32_t* keep_idx,
+                                  int32_t* S_out, const ScheduleHand& hand, const GatherRows* ga, cudaStream_t st) {
+    const CsPlan plan = cs_plan(n_vis);
+    if (!plan.fits) {
+        int rc = ga ? launch_gather(*ga, "gather_rows_kernel", st) : METOK_OK;
+        if (rc == METOK_OK)
+            rc = launch_class_topk(scores, 0, hand.group, n_vis, 2, budget, S, vis_start, keep_idx, 0, 1, S_out, nullptr, 1, st);
+        if (rc != METOK_OK) return rc;
+        METOK_TIMED("schedule_propagate_kernel", st);
+        launch_chained(schedule_propagate_kernel, dim3(std::max(1, ceil_div(hand.n_next, 256))), dim3(256), 0, st, keep_idx, vis_start,
+                       n_vis, hand);
+        METOK_LAUNCH_CHECK();
+        return METOK_OK;
+    }
+    TopkBudgets b = {};
+    b.v[0] = budget[0];
+    b.v[1] = budget[1];
+    const CsLayout lay = cs_layout(2, n_vis);
+    // The gather's CTAs have the selection's threads and registers: one that is alone on its SM holds six workers (the copies
+    // in flight that the gather has when it is launched alone), one of two holds three.
+    const int workers = std::min(plan.threads / 32, plan.threads > (plan.items == 4 ? 512 : 320) ? kGatherWorkersMax : kGatherWorkersMax / 2);
+    size_t smem = lay.bytes;
+    int grid = plan.C;
+    GatherRows none = {};
+    if (ga) {
+        smem = std::max(smem, workers * kGbWorkerBytes + 128);
+        const int ctas = kNumSMs * kGatherWorkersMax / workers;
+        grid += (ctas - plan.C) / plan.C * plan.C;
+    }
+    auto launch = [&](auto kernel) -> int {
+        if (smem > 32 * 1024) METOK_ALLOW_SMEM(kernel, smem);
+        METOK_TIMED("schedule_select_kernel", st);
+        launch_chained_clusters(plan.C, kernel, dim3(grid), dim3(plan.threads), smem, st, scores, n_vis, lay, b, S, vis_start, keep_idx,
+                                S_out, hand, ga ? *ga : none, workers);
+        METOK_LAUNCH_CHECK();
+        return METOK_OK;
+    };
+    if (plan.C == 1) return launch(schedule_select_kernel<4, false>);
+    if (plan.items == 4) return launch(schedule_select_kernel<4, true>);
+    return launch(schedule_select_kernel<kCsMaxItems, true>);
+}
+
+// Whether the levels' scoring and selection may run ahead of the gathers before them: no array that one level writes is
+// read or written by another, except hidden rows, whose gathers stay in order.
+static bool schedule_levels_apart(const metok_prune_level* lv, int n, const int32_t* sizes, int S, int n_vis, int Hq, int Hkv, int Lt,
+                                  int dh, int D, int eb) {
+    struct Range { uintptr_t lo, hi; };
+    auto range = [](const void* p, size_t bytes) { return Range{(uintptr_t)p, p ? (uintptr_t)p + bytes : (uintptr_t)p}; };
+    auto meet = [](const Range& a, const Range& b) { return a.lo < b.hi && b.lo < a.hi; };
+    Range w[kMaxPruneLevels][5], r[kMaxPruneLevels][4];
+    for (int s = 0; s < n; ++s) {
+        const size_t nv = sizes[s], rows = (size_t)(S - n_vis + sizes[s]);
+        w[s][0] = range(lv[s].scores, nv * 4);
+        w[s][1] = range(lv[s].keep_idx, rows * 4);
+        w[s][2] = range(lv[s].S_out, 4);
+        w[s][3] = range(lv[s].origin, nv * 4);
+        w[s][4] = range(lv[s].token_group, nv * 4);           // (written where s > 0)
+        r[s][0] = range(lv[s].q_text, (size_t)Hq * Lt * dh * eb);
+        r[s][1] = range(lv[s].k_all, (size_t)Hkv * rows * dh * eb);
+        r[s][2] = range(lv[s].hidden, rows * D * eb);
+        r[s][3] = range(lv[s].hidden_out, rows * D * eb);
+    }
+    for (int a = 0; a < n; ++a)
+        for (int b = 0; b < n; ++b) {
+            if (a == b) continue;
+            for (const Range& x : w[a]) {
+                for (const Range& y : w[b]) if (meet(x, y)) return false;
+                for (const Range& y : r[b]) if (meet(x, y)) return false;
+            }
+            if (meet(r[a][3], r[b][0]) || meet(r[a][3], r[b][1])) return false;
+        }
+    return true;
 }
 
 }  // namespace metok
@@ -839,13 +1012,13 @@ extern "C" size_t metok_prefill_prune_schedule_workspace_bytes(int n_levels, int
                                                                const int32_t* N0) {
     int32_t sizes[4];
     if (metok_prune_schedule_sizes(n_levels, alpha, r, N0, sizes) != METOK_OK || sizes[0] != n_vis) return 0;
-    size_t need = 0;
+    Carver cv(nullptr);
     for (int s = 0; s < n_levels; ++s) {
-        const size_t b = metok_prefill_prune_workspace_bytes(dtype, Hq, Hkv, Lt, S - n_vis + sizes[s], dh, sizes[s]);
-        if (b == 0) return 0;
-        need = b > need ? b : need;
+        const int S_s = S - n_vis + sizes[s];
+        if (metok_prefill_prune_workspace_bytes(dtype, Hq, Hkv, Lt, S_s, dh, sizes[s]) == 0) return 0;
+        carve_prefill(cv, make_dims(Hq, Hkv, Lt, S_s, dh, 0, sizes[s], 1.f), use_mma_attn(dtype, dh));
     }
-    return need;
+    return cv.total();
 }
 
 extern "C" int metok_prefill_prune_schedule(const metok_prune_level* levels, int n_levels, int dtype, int Hq, int Hkv,
@@ -872,33 +1045,50 @@ extern "C" int metok_prefill_prune_schedule(const metok_prune_level* levels, int
                                     lv.keep_idx, lv.S_out, lv.hidden_out, ws, ws_bytes);
         if (rc != METOK_OK) return rc;
     }
+    if (ws_bytes < metok_prefill_prune_schedule_workspace_bytes(n_levels, dtype, Hq, Hkv, Lt, S, dh, n_vis, alpha, r, N0))
+        return METOK_ERR_WORKSPACE;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    {
-        METOK_TIMED("schedule_init_kernel", st);
-        launch_chained(schedule_init_kernel, dim3(1), dim3(1024), 0, st, levels[0].token_group, n_vis, N0[0], N0[1], levels[0].origin, status);
+    const int eb = dtype == METOK_F32 ? 4 : 2;
+    const bool apart = schedule_levels_apart(levels, n_levels, sizes, S, n_vis, Hq, Hkv, Lt, dh, D, eb);
+    ScoreLevel sl[kMaxPruneLevels];
+    Carver cv(ws);
+    for (int s = 0; s < n_levels; ++s) {
+        const AttnDims dm = make_dims(Hq, Hkv, Lt, S - n_vis + sizes[s], dh, vis_start, sizes[s], softmax_scale);
+        sl[s] = {levels[s].q_text, levels[s].k_all, dm, carve_prefill(cv, dm, use_mma_attn(dtype, dh)), levels[s].scores};
+        if (s > 0) sl[s].w.status = sl[0].w.status;
     }
-    METOK_LAUNCH_CHECK();
+    int32_t* level_status = sl[0].w.status;
+    rc = debug_arm(level_status, st);
+    if (rc != METOK_OK) return rc;
+    // Nothing but the classes, origins and row numbers passes from level to level, so all levels are scored first, in the
+    // launches of one.  Buffers that levels share make the levels follow one another.
+    const float inv_rows = 1.0f / (float)(Hq * Lt);
+    GatherRows pending = {};                                  // the hidden rows of the level before
     for (int s = 0; s < n_levels; ++s) {
         const metok_prune_level& lv = levels[s];
         int32_t budget[2];
         rc = metok_retention_budgets(alpha, r, s + 1, N0, budget);
         if (rc != METOK_OK) return rc;
-        const int S_s = S - n_vis + sizes[s];
-        rc = metok_prefill_prune(lv.q_text, lv.k_all, lv.hidden, dtype, Hq, Hkv, Lt, S_s, dh, D, vis_start, sizes[s],
-                                 lv.token_group, 2, budget, softmax_scale, lv.scores, lv.keep_idx, lv.S_out,
-                                 lv.hidden_out, ws, ws_bytes, stream);
-        if (rc != METOK_OK) return rc;
-        // the level's status word (start of the workspace, cleared again by the next level) is folded
-        // into the caller's; this kernel also hands classes and origins to the next level
-        const bool more = s + 1 < n_levels;
-        const metok_prune_level& nx = levels[more ? s + 1 : s];
-        {
-            METOK_TIMED("schedule_propagate_kernel", st);
-            launch_chained(schedule_propagate_kernel, dim3(more ? ceil_div(sizes[s + 1], 256) : 1), dim3(256), 0, st,
-                lv.keep_idx, vis_start, sizes[s], more ? sizes[s + 1] : 0, lv.token_group, lv.origin, nx.token_group,
-                nx.origin, reinterpret_cast<const int32_t*>(ws), status);
+        if (s == 0 || !apart) {
+            if (pending.src) rc = launch_gather(pending, "gather_rows_kernel", st);
+            pending = {};
+            if (rc == METOK_OK)
+                rc = run_attention_scores(sl + s, apart ? n_levels : 1, dtype, softmax_scale, inv_rows, s == 0 ? lv.token_group : nullptr,
+                                          lv.origin, st);
+            if (rc != METOK_OK) return rc;
         }
-        METOK_LAUNCH_CHECK();
+        const bool more = s + 1 < n_levels;
+        const ScheduleHand hand = {lv.token_group, s == 0 ? nullptr : lv.origin, more ? levels[s + 1].token_group : nullptr,
+                                   more ? levels[s + 1].origin : nullptr, more ? sizes[s + 1] : 0, level_status,
+                                   status, s == 0, N0[0], N0[1], n_vis};
+        const int S_s = S - n_vis + sizes[s];
+        rc = launch_schedule_select(lv.scores, sizes[s], budget, S_s, vis_start, lv.keep_idx, lv.S_out, hand,
+                                    pending.src ? &pending : nullptr, st);
+        if (rc != METOK_OK) return rc;
+        pending = {};
+        if (lv.hidden)
+            pending = {reinterpret_cast<const uint8_t*>(lv.hidden), reinterpret_cast<uint8_t*>(lv.hidden_out), lv.keep_idx, lv.S_out,
+                       (uint32_t)((size_t)D * eb), S_s, level_status, status};
     }
-    return METOK_OK;
+    return pending.src ? launch_gather(pending, "gather_rows_kernel", st) : METOK_OK;
 }

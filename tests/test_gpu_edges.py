@@ -282,3 +282,85 @@ def test_frames_of_no_event_take_no_part(dtype):
     for name in ("out_event", "out_members", "out_feats"):
         assert torch.equal(got[name][:n], want[name][:n]), name
     assert torch.equal(got["assign"][5 * N:35 * N], want["assign"])
+
+
+def _schedule_case(n_vis, Lt, vis_start, r, dh, D, dtype, seed, Hq=4, Hkv=2):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    group = (torch.rand(n_vis, device="cuda", generator=g) < 0.5).to(torch.int32)
+    N0 = [int((group == 0).sum()), int((group == 1).sum())]
+    sizes = B.metok_prune_schedule_sizes(3, 0.5, r, N0)
+    rows = [vis_start + n + Lt for n in sizes[:3]]
+    q = [(0.3 * torch.randn((Hq, Lt, dh), device="cuda", generator=g)).to(dtype) for _ in range(3)]
+    k = [(0.3 * torch.randn((Hkv, S, dh), device="cuda", generator=g)).to(dtype) for S in rows]
+    h = [torch.randn((S, D), device="cuda", generator=g).to(dtype) for S in rows]
+    return group, N0, sizes, rows, q, k, h
+
+
+def _levels_one_by_one(case, vis_start, r, scale):
+    """The schedule as three pruning calls, classes and origins handed on by the host."""
+    group, N0, sizes, rows, q, k, h = case
+    origin = torch.arange(sizes[0], dtype=torch.int32, device="cuda")
+    out = []
+    for s in range(3):
+        lv = B.metok_prefill_prune(q[s], k[s], h[s], vis_start, sizes[s], group, B.metok_retention_budgets(0.5, r, s + 1, N0), scale)
+        out.append((lv["scores"].clone(), lv["keep_idx"][:vis_start + sizes[s + 1] + q[s].shape[1]].clone(), lv["hidden_out"].clone(),
+                    group, origin))
+        assert int(lv["S_out"].item()) == vis_start + sizes[s + 1] + q[s].shape[1]
+        kept = lv["keep_idx"][vis_start:vis_start + sizes[s + 1]].long() - vis_start
+        group, origin = group[kept].contiguous(), origin[kept]
+    return out
+
+
+# one CTA or a cluster selects (4096), three or six gather workers beside it, 16 items per thread, more items than a cluster holds
+@pytest.mark.parametrize("n_vis,r,dtype,dh", [
+    (40, 0.7, torch.bfloat16, 64), (4096, 0.8, torch.bfloat16, 128), (4097, 0.9, torch.bfloat16, 64), (5500, 0.9, torch.float32, 24),
+    (18432, 0.5, torch.bfloat16, 128), (30001, 0.95, torch.bfloat16, 64), (50000, 0.8, torch.bfloat16, 64), (82000, 0.6, torch.bfloat16, 64),
+])
+def test_schedule_equals_the_levels_called_one_by_one(n_vis, r, dtype, dh):
+    vis_start, D, scale = 5, 264, dh ** -0.5
+    case = _schedule_case(n_vis, 7, vis_start, r, dh, D, dtype, n_vis)
+    group, N0, sizes, rows, q, k, h = case
+    want = _levels_one_by_one(case, vis_start, r, scale)
+    got = B.metok_prefill_prune_schedule(q, k, h, vis_start, group, 0.5, r, N0, scale)
+    torch.cuda.synchronize()
+    for s, (scores, keep, hidden, grp, origin) in enumerate(want):
+        lv, n = got[s], len(keep)
+        assert int(lv["status"].item()) == 0 and int(lv["S_out"].item()) == n
+        assert torch.equal(lv["scores"], scores) and torch.equal(lv["keep_idx"][:n], keep)
+        assert torch.equal(lv["hidden_out"][:n].view(torch.uint8), hidden[:n].view(torch.uint8))
+        assert torch.equal(lv["origin"], origin) and torch.equal(lv["token_group"], grp)
+
+
+@pytest.mark.parametrize("dtype,dh", [(torch.bfloat16, 64), (torch.float32, 24)])
+def test_schedule_levels_that_share_buffers(dtype, dh):
+    """One scores, keep-list and S_out array for all levels, and a level's hidden rows where the level before left them."""
+    import ctypes as c
+    n_vis, r, vis_start, D, Lt = 6000, 0.8, 3, 264, 7
+    group, N0, sizes, rows, q, k, h = case = _schedule_case(n_vis, Lt, vis_start, r, dh, D, dtype, 1)
+    want = _levels_one_by_one((group, N0, sizes, rows, q, k, h), vis_start, r, dh ** -0.5)
+    lib, S, dt = B.lib(), rows[0], B.BF16 if dtype == torch.bfloat16 else B.F32
+    n0 = (c.c_int32 * 2)(*N0)
+    scores = torch.empty(n_vis, device="cuda")
+    keep, s_out, status = (torch.empty(n, dtype=torch.int32, device="cuda") for n in (S, 1, 1))
+    groups = [group] + [torch.empty(n, dtype=torch.int32, device="cuda") for n in sizes[1:3]]
+    origins = [torch.empty(n, dtype=torch.int32, device="cuda") for n in sizes[:3]]
+    a, b = h[0].clone(), torch.empty_like(h[0])                          # hidden rows go to and fro
+    arr = (B.PruneLevel * 3)()
+    for s in range(3):
+        arr[s].q_text, arr[s].k_all = q[s].data_ptr(), k[s].data_ptr()
+        arr[s].hidden, arr[s].hidden_out = (a, b)[s & 1].data_ptr(), (b, a)[s & 1].data_ptr()
+        arr[s].scores, arr[s].keep_idx, arr[s].S_out = scores.data_ptr(), keep.data_ptr(), s_out.data_ptr()
+        arr[s].token_group, arr[s].origin = groups[s].data_ptr(), origins[s].data_ptr()
+    ws = torch.empty(lib.metok_prefill_prune_schedule_workspace_bytes(3, dt, 4, 2, Lt, S, dh, n_vis, 0.5, r, n0), dtype=torch.uint8,
+                     device="cuda")
+    assert lib.metok_prefill_prune_schedule(arr, 3, dt, 4, 2, Lt, S, dh, D, vis_start, n_vis, 0.5, r, n0, dh ** -0.5, status.data_ptr(),
+                                            ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream) == 0
+    torch.cuda.synchronize()
+    n = vis_start + sizes[3] + Lt
+    assert int(status.item()) == 0 and int(s_out.item()) == n
+    assert torch.equal(scores[:sizes[2]], want[2][0]) and torch.equal(keep[:n], want[2][1])
+    rows_kept = torch.arange(rows[0], device="cuda")                     # of the first level's hidden rows
+    for s in range(3):
+        rows_kept = rows_kept[want[s][1].long()]
+        assert torch.equal(origins[s], want[s][4]) and torch.equal(groups[s], want[s][3])
+    assert torch.equal(b[:n].view(torch.uint8), h[0][rows_kept].view(torch.uint8))
