@@ -1,0 +1,525 @@
+// Merge-assign of fp32 features on the tensor cores.  Included by vision.cu after the member lists.
+//
+// A float is the sum of three bf16 numbers, its leading, middle and trailing eight significant bits (x = h + m + l exactly,
+// by truncation), so a product of two floats is the sum of nine products of bf16 numbers, each exact in the tensor core's
+// fp32.  Six are made: hh, hm, mh, mm, hl, lh; the three left out (ml, lm, ll) are below 2^-23 of the product.  What would
+// lose precision is the accumulator, which the tensor core cuts off instead of rounding: the sums of hh are therefore taken
+// out of tensor memory after every two steps, four additions, and added up in registers with rounding, and the
+// other five, 2^-8 of the whole, have an accumulator of their own.
+//
+// Which key token is the most similar is decided by the fp32 chain all the same.  The tensor cores find, for every token, the key
+// with the largest similarity and the others that are within f3_margin of it; where there are any (a few per cent of the tokens),
+// merge_join_f32_kernel makes these products again as one chain of fused multiply-adds and takes the largest, so that the
+// assignment is the one that merge_assign_simt_kernel finds.
+//
+// merge_planes_kernel writes the three planes of every token into the workspace, the tokens that are no key tokens and the key
+// tokens of an event apart, in the order and the swizzle in which a step's tiles lie in shared memory;
+// merge_assign_f32_mma_kernel then brings a step of a unit in with two bulk copies.  (Splitting the rows inside the second kernel,
+// where they were needed, was bound by the latency of the scattered loads: 95 us at 61 x 169 tokens of 1156.)
+#pragma once
+
+namespace metok {
+
+constexpr int kF3BM = 128, kF3BN = 256, kF3BK = 32;           // most tokens and keys of a unit; elements per step
+constexpr int kF3MaxStages = 8;
+constexpr int kF3MinD = 60;                                   // narrowest rows that this has been compared with 64 bits at
+// Steps whose hh add up in tensor memory.  A row of few steps has little else to round: one, or its error would be above that
+// of the CUDA cores' chain.  Relative error of the cosines against 64 bits, root mean square (largest), chain / here: width
+// 60: 5.5e-8 (6.3e-7) / 4.6e-8 (2.8e-7); 96: 6.1e-8 / 5.2e-8; 512: 7.7e-8 (1.3e-6) / 4.3e-8 (3.6e-7); 1156: 1.5e-7 (1.6e-6) / 8.3e-8
+// (5.7e-7); 2048: 1.8e-7 / 1.1e-7; 3580: 2.3e-7 (2.9e-6) / 1.7e-7 (9.6e-7).  One step everywhere costs 2.5 us at 61 x 169 x 1156.
+__device__ __forceinline__ int f3_segment(int d) { return d < 96 ? 1 : 2; }
+constexpr int kF3EpiWarps = 16, kF3Threads = kF3EpiWarps * 32 + 64;
+constexpr uint32_t kF3RowBytes = 3 * kF3BK * 2;               // a row's share of a step: three planes
+constexpr uint32_t kF3ABytes = kF3BM * kF3RowBytes, kF3RingBytes = 3 * (kF3ABytes + kF3BN * kF3RowBytes);
+constexpr size_t kF3SmemBytes = kF3RingBytes + 1024;
+constexpr int kF3Events = 512;                                // up to as many events' offsets are kept in shared memory
+
+// Where the planes of an event lie.  Tokens that are no key tokens: tiles of 128 rows, the event's first at f3_tile0; a tile is
+// [step][plane][128 rows][64 bytes].  Key tokens: groups of 16 rows, the first at f3_group0; a unit's keys are whole groups,
+// [step][plane][rows][64 bytes].  Both are rounded down from the rows before the event, plus one per event before, so that
+// events never overlap whatever their sizes.
+__host__ __device__ inline long long f3_tile0(long long rest_before, int e) { return rest_before / kF3BM + e; }
+__host__ __device__ inline long long f3_group0(long long keys_before, int e) { return keys_before / 16 + e; }
+__host__ __device__ inline int f3_steps(int d) { return (d + kF3BK - 1) / kF3BK; }
+__host__ __device__ inline size_t f3_a_bytes(long long Nv, int k, int d) { return (size_t)(f3_tile0(Nv, k) + 1) * kF3ABytes * f3_steps(d); }
+__host__ __device__ inline size_t f3_b_bytes(long long cap, int k, int d) { return (size_t)(f3_group0(cap, k) + 1) * 16 * kF3RowBytes * f3_steps(d); }
+struct F3Planes { uint8_t *a, *b; };
+
+// The chain's error and the tensor cores' together, twice (for the two keys that are compared), with a factor of two to three to spare: the largest
+// errors of a cosine against 64 bits, chain + here: width 60: 6.3e-7 + 2.8e-7, margin 4.1e-6; 1156: 1.6e-6 + 5.7e-7, 1.5e-5;
+// 3580: 2.9e-6 + 9.6e-7, 2.5e-5.
+__device__ __forceinline__ float f3_margin(int d) { return 1.0e-6f + 4.0e-7f * sqrtf((float)d); }
+// A token's candidates beside the best one so far (best64, whose packing they share): at most kF3Cands are listed, and a
+// count of kF3All or more stands for all keys of the event (a norm that is no finite number).  Key tokens that are copies
+// of one another (frames that repeat) would fill the lists: of those with the same similarity and the same hash the first counts.
+constexpr int kF3Cands = 7, kF3All = 1 << 16;
+struct F3Cands {
+    unsigned long long* list;                                 // [token][kF3Cands + 1]
+    int32_t* count;                                           // [token], cleared with the merge's scratch
+    uint32_t* hash;                                           // [slot] of the key token's row
+};
+__device__ __forceinline__ unsigned long long f3_pack(float v, int slot) {
+    return ((unsigned long long)float_key(v) << 32) | (unsigned long long)(~(uint32_t)slot);
+}
+__device__ __forceinline__ float f3_value(unsigned long long p) {
+    const uint32_t k = (uint32_t)(p >> 32);
+    return __uint_as_float(k & 0x80000000u ? k & 0x7FFFFFFFu : ~k);
+}
+__device__ __forceinline__ int f3_slot(unsigned long long p) { return (int)~(uint32_t)p; }
+__device__ __forceinline__ void f3_push(const F3Cands& ca, int row, unsigned long long p) {
+    const int at = atomicAdd(&ca.count[row], 1);
+    if (at < kF3Cands) ca.list[(size_t)row * (kF3Cands + 1) + at] = p;
+}
+
+// An event's key tokens in equal chunks of whole sixteens.
+__device__ __forceinline__ int f3_chunk(int nk, int nchunks) { return ((nk + nchunks - 1) / nchunks + 15) & ~15; }
+struct F3Unit {
+    int at, rows, col0, cols;                                 // rest[at .. at + rows), slots [col0, col0 + cols)
+    long long tile, group;                                    // its rows' tile, its keys' first group
+};
+__device__ __forceinline__ F3Unit f3_unit(int u, const int32_t* ev_unit_off, const int32_t* ev_lo, const int32_t* ev_out_off, int k, int N, int bn) {
+    const int e = find_event(ev_unit_off, k, u);
+    const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0, lo = ev_lo[e] * N, hi = ev_lo[e + 1] * N;
+    const int nchunks = (nk + bn - 1) / bn, size = f3_chunk(nk, nchunks);
+    const int local = u - ev_unit_off[e], tile = local / nchunks, c = local - tile * nchunks;
+    F3Unit x;
+    x.at = lo + tile * kF3BM;
+    x.rows = min(kF3BM, hi - nk - x.at);
+    x.col0 = s0 + c * size;
+    x.cols = min(size, nk - c * size);
+    x.tile = f3_tile0(lo - s0, e) + tile;
+    x.group = f3_group0(s0, e) + c * (size / 16);
+    return x;
+}
+
+// A 64-byte-swizzled K-major tile: rows of 64 bytes, groups of eight rows 512 bytes apart.
+__device__ __forceinline__ constexpr uint32_t desc_k64_hi() { return (uint32_t)(512 >> 4) | (1u << 14) | (4u << 29); }
+__device__ __forceinline__ void umma_bf16_k64(uint32_t d_tmem, uint32_t a_addr, uint32_t b_addr, uint32_t idesc, uint32_t accumulate) {
+    const uint32_t a_lo = sm100::desc_k128_lo(a_addr), b_lo = sm100::desc_k128_lo(b_addr);
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 da, {%1, %3};\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_k64_hi()), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// The three planes' four elements of x: two words each.
+__device__ __forceinline__ void f3_split(const uint4& x, uint2& h, uint2& m, uint2& l) {
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+    uint32_t r1[4], r2[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float a = __uint_as_float(w[i]) - __uint_as_float(w[i] & 0xFFFF0000u);
+        r1[i] = __float_as_uint(a);
+        r2[i] = __float_as_uint(a - __uint_as_float(r1[i] & 0xFFFF0000u));
+    }
+    h = make_uint2(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632));
+    m = make_uint2(__byte_perm(r1[0], r1[1], 0x7632), __byte_perm(r1[2], r1[3], 0x7632));
+    l = make_uint2(__byte_perm(r2[0], r2[1], 0x7632), __byte_perm(r2[2], r2[3], 0x7632));
+}
+
+// The planes of all tokens.  Four rows per warp, eight threads and 128 bytes of a row each, so that 256 bytes of a plane leave
+// together; kF3Ahead steps of loads in flight per thread.  blockIdx.y: a share of the steps.  In a plane row r lies at
+// r * 64 bytes and its 16-byte piece p at position p ^ (r / 2 % 4).
+constexpr int kF3Ahead = 6;
+__global__ void __launch_bounds__(256)
+merge_planes_kernel(const float* __restrict__ feats, int Nv, int d, int N, const int32_t* ev_lo, int k, const int32_t* ev_out_off,
+                    TokenOut out, F3Planes pl, F3Cands ca, int bn, int steps_per_cta, int32_t* __restrict__ status) {
+    grid_dep_wait();
+    __shared__ int32_t s_lo[kF3Events + 1], s_out[kF3Events + 1];
+    const long long all = (long long)ev_lo[k] * N, first = (long long)ev_lo[0] * N;
+    if (k <= kF3Events) {
+        for (int i = threadIdx.x; i <= k; i += blockDim.x) {
+            s_lo[i] = ev_lo[i];
+            s_out[i] = ev_out_off[i];
+        }
+        __syncthreads();
+        ev_lo = s_lo;
+        ev_out_off = s_out;
+    }
+    const long long i = (long long)blockIdx.x * 32 + (threadIdx.x >> 3);   // a place: an event's other tokens, then its key tokens
+    if (i < first || i >= all) return;
+    const int e = find_event(ev_lo, k, (int)(i / N));
+    const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0, lo = ev_lo[e] * N, nr = ev_lo[e + 1] * N - lo - nk, x = (int)i - lo;
+    uint8_t* dst;
+    uint32_t plane;                                           // bytes of a plane; three of them are a step
+    int r, row, slot = -1;
+    if (x < nr) {
+        r = x % kF3BM;
+        row = out.rest[lo + x];
+        dst = pl.a + (size_t)(f3_tile0(lo - s0, e) + x / kF3BM) * kF3ABytes * f3_steps(d);
+        plane = kF3BM * 64;
+    } else {
+        const int j = x - nr, nchunks = (nk + bn - 1) / bn, size = f3_chunk(nk, nchunks), c = j / size;
+        r = j - c * size;
+        slot = s0 + j;
+        row = out.out_src[slot];
+        dst = pl.b + (size_t)(f3_group0(s0, e) + c * (size / 16)) * 16 * kF3RowBytes * f3_steps(d);
+        plane = (uint32_t)((min(size, nk - c * size) + 15) & ~15) * 64u;
+    }
+    row = (int)dbg_bound(row, all, status);
+    const int c = threadIdx.x & 7;
+    dst += (uint32_t)r * 64u + (uint32_t)(((c >> 1) ^ ((r >> 1) & 3)) << 4) + (uint32_t)(c & 1) * 8u;
+    const float* src = feats + (size_t)row * d + c * 4;
+    const int k_lo = (int)blockIdx.y * steps_per_cta, k_hi = min(f3_steps(d), k_lo + steps_per_cta);
+    uint32_t hash = 0;                                        // a sum of the elements' bits with odd weights
+    for (int k0 = k_lo; k0 < k_hi; k0 += kF3Ahead) {
+        uint4 v[kF3Ahead];
+#pragma unroll
+        for (int u = 0; u < kF3Ahead; ++u) {                  // the last step may reach past d (a multiple of 4): zeros there
+            const int at = (k0 + u) * kF3BK;
+            v[u] = k0 + u < k_hi && at + c * 4 < d ? __ldg(reinterpret_cast<const uint4*>(src + at)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int u = 0; u < kF3Ahead; ++u) {
+            if (k0 + u >= k_hi) continue;
+            const uint32_t w = (uint32_t)((k0 + u) * 8 + c) * 0x9E3779B2u + 1u;
+            hash += (v[u].x * 3u + v[u].y * 0x85EBCA6Bu + v[u].z * 0xC2B2AE35u + v[u].w * 0x27D4EB2Fu) * w;
+            uint2 h, m, l;
+            f3_split(v[u], h, m, l);
+            uint8_t* o = dst + (size_t)(k0 + u) * 3 * plane;
+            *reinterpret_cast<uint2*>(o) = h;
+            *reinterpret_cast<uint2*>(o + plane) = m;
+            *reinterpret_cast<uint2*>(o + 2 * plane) = l;
+        }
+    }
+    if (slot >= 0) atomicAdd(&ca.hash[slot], hash);
+}
+
+// Work unit = up to 128 of an event's tokens that are no key tokens x up to 256 of its key tokens (equal chunks of its keys);
+// a persistent CTA takes every gridDim-th unit of the list of all events.
+//   warp 16    : brings a step's tiles in, one bulk copy for the tokens and one for the keys;
+//   warp 17    : issues tcgen05.mma (M = 128, N = the chunk's keys, K = 16), twelve per step of 32 elements: hh last, so that its
+//                accumulator may still be read while the others of the next step are made;
+//   warps 0-15 : epilogue, four TMEM lane quadrants x four quarters of the columns: a thread adds up 64 columns of its row, scales
+//                them by 1/|key| and takes their (value, slot) argmax; the quarters and the chunks of a row meet in a 64-bit atomicMax
+//                (larger value, then lower slot), and whichever of two falls behind there, or beside it in the quarter, by less
+//                than the margin is listed.
+// Shared memory bounds it: a step of 128 x 256 writes 72 KB and its products read 144 KB, 0.89 us at 128 bytes a clock beside 0.84
+// us of tensor time.  Every wait is bounded; on a timeout the CTA unwinds and writes METOK_ERR_TIMEOUT.
+__global__ void __launch_bounds__(kF3Threads, 1)
+merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int32_t* ev_out_off,
+                            const int32_t* ev_unit_off, const float* __restrict__ inv_norm, TokenOut out, F3Planes pl, F3Cands ca, int bn,
+                            int32_t* __restrict__ status) {
+    grid_dep_wait();
+    using namespace sm100;
+    const int32_t *out_src = out.out_src, *rest = out.rest;
+    extern __shared__ uint8_t smem_dyn[];
+    __shared__ __align__(8) uint64_t full_bar[kF3MaxStages], empty_bar[kF3MaxStages], hfull_bar, hempty_bar, sfull_bar, sempty_bar, drain_bar;
+    __shared__ uint32_t s_tmem_base;
+    __shared__ int s_abort;
+    __shared__ __align__(16) float s_keyinv[2][kF3BN];
+    const int total_units = ev_unit_off[k];
+    if ((int)blockIdx.x >= total_units) return;
+    const int ksteps = f3_steps(d), segment = f3_segment(d), nseg = (ksteps + segment - 1) / segment;
+    const uint32_t stage_bytes = kF3ABytes + (uint32_t)bn * kF3RowBytes;
+    const int stages = min(kF3MaxStages, (int)(kF3RingBytes / stage_bytes));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
+        mbar_init(smem_u32(&hfull_bar), 1);
+        mbar_init(smem_u32(&hempty_bar), kF3EpiWarps);
+        mbar_init(smem_u32(&sfull_bar), 1);
+        mbar_init(smem_u32(&sempty_bar), kF3EpiWarps);
+        mbar_init(smem_u32(&drain_bar), 1);
+        s_abort = 0;
+        mbar_fence_init();
+    }
+    if (warp == kF3EpiWarps + 1) {
+        tmem_alloc(smem_u32(&s_tmem_base), 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = s_tmem_base;                   // columns 0 ..: the sums of hh, 256 ..: the others'
+    volatile int* abort_flag = &s_abort;
+
+    if (warp == kF3EpiWarps) {
+        if (lane == 0) {
+            int s = 0, issued = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
+                const F3Unit un = f3_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, bn);
+                const uint32_t b_bytes = (uint32_t)((un.cols + 15) & ~15) * kF3RowBytes;
+                const uint8_t* a = pl.a + (size_t)un.tile * kF3ABytes * ksteps;
+                const uint8_t* b = pl.b + (size_t)un.group * 16 * kF3RowBytes * ksteps;
+                for (int ks = 0; ks < ksteps; ++ks, a += kF3ABytes, b += b_bytes) {
+                    if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
+                    const uint32_t fb = smem_u32(&full_bar[s]), dst = smem_base + (uint32_t)s * stage_bytes;
+                    mbar_arrive_expect_tx(fb, kF3ABytes + b_bytes);
+                    bulk_load(dst, a, kF3ABytes, fb);
+                    if (!(dbg_withhold(status, kDbgMergeAssign) && blockIdx.x == 0 && issued == 0))   // debug builds: one copy never sent
+                        bulk_load(dst + kF3ABytes, b, b_bytes, fb);
+                    ++issued;
+                    if (++s == stages) { s = 0; ph ^= 1u; }
+                }
+            }
+            // every copy has landed before the CTA's shared memory goes away
+            for (int back = 1; back <= stages && back <= issued; ++back) {
+                const int j = issued - back;
+                mbar_wait(smem_u32(&full_bar[j % stages]), (uint32_t)(j / stages) & 1u, abort_flag);
+            }
+        }
+    } else if (warp == kF3EpiWarps + 1) {
+        if (lane == 0) {
+            int s = 0, n = 0, seg = 0;                        // stage; units and segments so far
+            uint32_t ph = 0;
+            bool ok = true;
+            const uint32_t d_hh = tmem_base, d_small = tmem_base + kF3BN;
+            for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++n) {
+                const F3Unit un = f3_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, bn);
+                const uint32_t cols = (uint32_t)(un.cols + 15) & ~15u, idesc = make_idesc_bf16(kF3BM, (int)cols);
+                constexpr uint32_t kA = kF3BM * 64;           // a plane of the tokens, and of the keys
+                const uint32_t kB = cols * 64;
+                for (int ks = 0; ks < ksteps; ++ks) {
+                    if (!mbar_wait(smem_u32(&full_bar[s]), ph, abort_flag)) { ok = false; break; }
+                    if (ks == 0 && !mbar_wait(smem_u32(&sempty_bar), ((uint32_t)n & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t a = smem_base + (uint32_t)s * stage_bytes, b = a + kF3ABytes;
+#pragma unroll
+                    for (int kk = 0; kk < kF3BK / 16; ++kk) {
+                        const uint32_t ah = a + 32u * kk, bh = b + 32u * kk;
+                        umma_bf16_k64(d_small, ah + kA, bh + kB, idesc, ks > 0 || kk > 0 ? 1u : 0u);
+                        umma_bf16_k64(d_small, ah, bh + 2 * kB, idesc, 1u);
+                        umma_bf16_k64(d_small, ah + 2 * kA, bh, idesc, 1u);
+                        umma_bf16_k64(d_small, ah, bh + kB, idesc, 1u);
+                        umma_bf16_k64(d_small, ah + kA, bh, idesc, 1u);
+                    }
+                    const bool opens = (ks & (segment - 1)) == 0;
+                    if (opens) {
+                        if (!mbar_wait(smem_u32(&hempty_bar), ((uint32_t)seg & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+                        tc_fence_after();
+                    }
+#pragma unroll
+                    for (int kk = 0; kk < kF3BK / 16; ++kk) umma_bf16_k64(d_hh, a + 32u * kk, b + 32u * kk, idesc, !opens || kk > 0 ? 1u : 0u);
+                    umma_commit(smem_u32(&empty_bar[s]));
+                    if (++s == stages) { s = 0; ph ^= 1u; }
+                    if ((ks & (segment - 1)) == segment - 1 || ks == ksteps - 1) {
+                        umma_commit(smem_u32(&hfull_bar));
+                        ++seg;
+                    }
+                }
+                if (ok) umma_commit(smem_u32(&sfull_bar));
+            }
+            if (!ok) {                                        // wait until whatever was issued has retired
+                umma_commit(smem_u32(&drain_bar));
+                mbar_wait(smem_u32(&drain_bar), 0u, abort_flag);
+            }
+        }
+    } else {
+        const int quad = warp & 3, part = warp >> 2;          // TMEM lanes 32 * quad ..., columns 64 * part ...
+        const int et = threadIdx.x, c0 = 64 * part;
+        bool ok = true;
+        int n = 0, seg = 0;
+        const float margin = f3_margin(d);
+        for (int u = blockIdx.x; u < total_units; u += gridDim.x, ++n) {
+            const F3Unit un = f3_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, bn);
+            float* keyinv = s_keyinv[n & 1];                  // alternates: a slow warp may still read the last one
+            if (et < kF3BN) keyinv[et] = et < un.cols ? inv_norm[out_src[un.col0 + et]] : 1.f;
+            const int r = quad * 32 + lane;
+            const int row = r < un.rows ? rest[un.at + r] : -1;
+            const float rinv = row >= 0 ? inv_norm[row] : 1.f;
+            named_bar_sync(1, kF3EpiWarps * 32);
+            const bool mine = c0 < un.cols;                   // the same for the whole warp
+            const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
+            float sum[64];
+#pragma unroll
+            for (int j = 0; j < 64; ++j) sum[j] = 0.f;
+            auto take = [&](uint32_t col, uint32_t bar, uint32_t parity, uint32_t free_bar) {
+                if (ok && !mbar_wait(bar, parity, abort_flag)) ok = false;
+                ok = __all_sync(0xFFFFFFFFu, ok);             // tcgen05.ld below is warp-collective
+                if (!ok) return;
+                if (mine) {
+                    tc_fence_after();
+#pragma unroll
+                    for (int x = 0; x < 64; x += 16) {
+                        float v[16];
+                        tmem_ld16(t_row + col + (uint32_t)x, v);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) sum[x + j] += v[j];
+                    }
+                    tc_fence_before();
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(free_bar);
+            };
+            for (int i = 0; i < nseg; ++i, ++seg) take(0u, smem_u32(&hfull_bar), (uint32_t)seg & 1u, smem_u32(&hempty_bar));
+            take(kF3BN, smem_u32(&sfull_bar), (uint32_t)n & 1u, smem_u32(&sempty_bar));
+            if (ok && mine && row >= 0) {
+                float best_v = -3.4e38f, least = rinv;        // zero: a norm beyond the largest float, of the token or of a key
+                int best_c = -1;
+#pragma unroll
+                for (int j = 0; j < 64; ++j) {
+                    const float ki = keyinv[c0 + j], v = c0 + j < un.cols ? sum[j] * ki : -3.4e38f;
+                    least = fminf(least, ki);
+                    sum[j] = v;
+                    if (v > best_v) { best_v = v; best_c = c0 + j; }
+                }
+                if (least == 0.f) atomicAdd(&ca.count[row], kF3All);
+                if (best_c >= 0) {
+                    const unsigned long long me = f3_pack(best_v, un.col0 + best_c), old = atomicMax(&out.best64[row], me);
+                    const float old_v = old ? f3_value(old) : -3.4e38f, from = fmaxf(best_v, old_v) - margin / rinv;
+                    if (best_v >= from && old_v >= from && !(old_v == best_v && ca.hash[f3_slot(old)] == ca.hash[f3_slot(me)]))
+                        f3_push(ca, row, old > me ? me : old);
+                    uint32_t close[2] = {0u, 0u};             // the others of these columns
+#pragma unroll
+                    for (int j = 0; j < 64; ++j)
+                        if (sum[j] >= from) close[j >> 5] |= 1u << (j & 31);
+#pragma unroll
+                    for (int w = 0; w < 2; ++w) {
+#pragma unroll 1
+                        for (uint32_t left = close[w]; left; left &= left - 1) {
+                            const int c = c0 + 32 * w + __ffs(left) - 1;
+                            float v = 0.f;
+#pragma unroll
+                            for (int j = 32 * w; j < 32 * w + 32; ++j) v = c0 + j == c ? sum[j] : v;
+                            if (c != best_c && c < un.cols && !(v == best_v && ca.hash[un.col0 + c] == ca.hash[f3_slot(me)]))
+                                f3_push(ca, row, f3_pack(v, un.col0 + c));
+                        }
+                    }
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == kF3EpiWarps + 1) tmem_dealloc(tmem_base, 512);
+    if (threadIdx.x == 0 && s_abort) *status = METOK_ERR_TIMEOUT;
+}
+
+// The token's key among its candidates, and the token into that output's member list.  A CTA looks at 16 tokens, eight lanes
+// each, a candidate per lane; those whose products have to be made again are listed and its warps take one each: 256 elements
+// of the token and of its candidates go through shared memory, the next 256 on their way, and a lane per candidate runs its
+// chain over them.  What bounds it is the latency of these steps one after the other.
+constexpr int kF3JoinWarps = 4, kF3JoinPiece = 64;            // float4s of a row at a time
+__device__ __forceinline__ float f3_chain4(const float4& x, const float4& y, float a) {
+    return fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, a))));
+}
+struct F3Again { int row, lo, hi, s0, s1, n, slot[kF3Cands + 1]; };   // n candidates, 0: all keys of the event
+__device__ __forceinline__ void f3_join(const TokenOut& out, int slot, int row, int lo, int hi, int s0, int s1) {
+    out.assign[row] = slot;
+    if (slot >= s0 && slot < s1) members_join(out.ml, slot, row, row - lo, hi - lo);
+}
+__global__ void __launch_bounds__(kF3JoinWarps * 32)
+merge_join_f32_kernel(const float* __restrict__ feats, int Nv, int d, int N, const int32_t* ev_lo, int k, const int32_t* ev_out_off,
+                      const float* __restrict__ inv_norm, TokenOut out, F3Cands ca) {
+    grid_dep_wait();
+    __shared__ float4 s_row[kF3JoinWarps][kF3Cands + 2][kF3JoinPiece];   // the token, then its candidates
+    __shared__ int32_t s_lo[kF3Events + 1], s_out[kF3Events + 1];
+    __shared__ F3Again s_again[kF3JoinWarps * 4];
+    __shared__ int s_n;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & 7;
+    const int row = (blockIdx.x * kF3JoinWarps + warp) * 4 + (lane >> 3);
+    bool is_rest = row < Nv && !out.is_key[row];
+    if (threadIdx.x == 0) s_n = 0;
+    if (k <= kF3Events) {
+        for (int i = threadIdx.x; i <= k; i += blockDim.x) {
+            s_lo[i] = ev_lo[i];
+            s_out[i] = ev_out_off[i];
+        }
+        ev_lo = s_lo;
+        ev_out_off = s_out;
+    }
+    __syncthreads();
+    {
+        int lo = 0, hi = 0, s0 = 0, s1 = 0, count = 0;
+        float inv = 1.f;
+        unsigned long long mine = 0;                          // this lane's candidate; the last of the eight: the best
+        if (is_rest) {
+            count = ca.count[row];
+            inv = inv_norm[row];
+            if (sub == kF3Cands) mine = out.best64[row];
+            const int e = find_event(ev_lo, k, row / N);
+            lo = ev_lo[e] * N;
+            hi = ev_lo[e + 1] * N;
+            s0 = ev_out_off[e];
+            s1 = ev_out_off[e + 1];
+            is_rest = row >= lo && row < hi;                  // else a token of no event: its scratch is not this call's
+            if (is_rest && sub < count && count <= kF3Cands) mine = ca.list[(size_t)row * (kF3Cands + 1) + sub];
+        }
+        const unsigned long long best = __shfl_sync(0xFFFFFFFFu, mine, lane | 7);
+        const bool cand = is_rest && mine && f3_value(mine) >= f3_value(best) - f3_margin(d) / inv;
+        const uint32_t set = (__ballot_sync(0xFFFFFFFFu, cand) >> (lane & 24)) & 0xFFu;
+        const bool all = count > kF3Cands, again = is_rest && (all || __popc(set) > 1);
+        int at = again && sub == 0 ? atomicAdd(&s_n, 1) : 0;
+        at = __shfl_sync(0xFFFFFFFFu, at, lane & 24);
+        if (again) {
+            F3Again& x = s_again[at];
+            if (sub == 0) { x.row = row; x.lo = lo; x.hi = hi; x.s0 = s0; x.s1 = s1; x.n = all ? 0 : __popc(set); }
+            if (cand) x.slot[__popc(set & ((1u << sub) - 1u))] = f3_slot(mine);
+        } else if (is_rest && sub == 0) {
+            f3_join(out, best ? f3_slot(best) : -1, row, lo, hi, s0, s1);
+        }
+    }
+    __syncthreads();
+    for (int t = warp; t < s_n; t += kF3JoinWarps) {
+        const F3Again& x = s_again[t];
+        const int n4 = d >> 2, nc = x.n;
+        const float4* x4 = reinterpret_cast<const float4*>(feats + (size_t)x.row * d);
+        unsigned long long won = 0;
+        if (nc == 0) {                                        // a key of the event per lane
+            for (int s = x.s0 + lane; s < x.s1; s += 32) {
+                const int key = out.out_src[s];
+                const float4* y4 = reinterpret_cast<const float4*>(feats + (size_t)key * d);
+                float a = 0.f;
+#pragma unroll 4
+                for (int i = 0; i < n4; ++i) a = f3_chain4(__ldg(x4 + i), __ldg(y4 + i), a);
+                const float v = a * inv_norm[key];
+                if (v > -3.4e38f) {
+                    const unsigned long long p = f3_pack(v, s);
+                    won = p > won ? p : won;
+                }
+            }
+        } else {
+            const int slot = lane < nc ? x.slot[lane] : -1, key = lane < nc ? out.out_src[slot] : 0;
+            const float4* y4[kF3Cands + 1];
+#pragma unroll
+            for (int j = 0; j <= kF3Cands; ++j) y4[j] = reinterpret_cast<const float4*>(feats + (size_t)__shfl_sync(0xFFFFFFFFu, key, j) * d);
+            const float key_inv = lane < nc ? inv_norm[key] : 0.f;
+            constexpr int U = kF3JoinPiece / 32;
+            float4 next[kF3Cands + 2][U];
+            auto fetch = [&](int i0) {
+                const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int i = i0 + 32 * u + lane;
+                    next[0][u] = i < n4 ? __ldg(x4 + i) : zero;
+#pragma unroll
+                    for (int j = 0; j <= kF3Cands; ++j) next[j + 1][u] = j < nc && i < n4 ? __ldg(y4[j] + i) : zero;
+                }
+            };
+            fetch(0);
+            float a = 0.f;
+            for (int i0 = 0; i0 < n4; i0 += kF3JoinPiece) {
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j <= kF3Cands + 1; ++j)
+                    if (j <= nc) {
+#pragma unroll
+                        for (int u = 0; u < U; ++u) s_row[warp][j][32 * u + lane] = next[j][u];
+                    }
+                __syncwarp();
+                fetch(i0 + kF3JoinPiece);
+                if (lane < nc) {                              // (past the row's end: zeros, which change nothing)
+#pragma unroll 8
+                    for (int i = 0; i < kF3JoinPiece; ++i) a = f3_chain4(s_row[warp][0][i], s_row[warp][lane + 1][i], a);
+                }
+            }
+            if (lane < nc) {
+                const float v = a * key_inv;
+                if (v > -3.4e38f) won = f3_pack(v, slot);
+            }
+        }
+        const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(won >> 32));
+        const uint32_t low = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(won >> 32) == top ? (uint32_t)won : 0u);
+        if (lane == 0) f3_join(out, top ? (int)~low : -1, x.row, x.lo, x.hi, x.s0, x.s1);
+    }
+}
+
+}  // namespace metok

@@ -2,11 +2,9 @@
 // others tx + 8 j; ty = thread / 8, tx = thread % 8).  fp32 products, added in the order of the row: every dot product is
 // one chain of fused multiply-adds.
 //
-// Shared-memory reads and multiply-adds are nearly in balance at P = 8 (a k costs a thread 64 bytes, which is what 64
-// multiply-adds take to run), so rows are kept as they lie (k contiguous, 8-byte reads of two k; wider reads are no cheaper
-// per byte: a k-major layout with 16-byte reads took 423 us where this one takes 204) and come by 16-byte asynchronous
-// copies into two stages of 16 k (three or four are no faster), a row's pitch of 80 bytes (fp32) putting the eight rows of
-// a warp's read into different banks.  Small CTAs, several per SM: sa_ctas_per_sm.
+// Rows are kept as they lie (k contiguous, 8-byte reads of two k; wider reads are no cheaper per byte) and come by 16-byte
+// asynchronous copies into two stages of 16 k (three or four are no faster), a row's pitch of 80 bytes (fp32) putting the eight
+// rows of a warp's read into different banks.  Small CTAs, several per SM: sa_ctas_per_sm.
 #pragma once
 #include "common.cuh"
 #include "sm100.cuh"
@@ -14,7 +12,7 @@
 namespace metok {
 
 constexpr int kSaBK = 16, kSaThreads = 64;
-constexpr int sa_ctas_per_sm(int pt) { return pt == 8 ? 6 : pt == 4 ? 10 : 12; }
+constexpr int sa_ctas_per_sm(int pt) { return pt == 4 ? 10 : 12; }
 
 template <typename T>
 __device__ __forceinline__ float2 load_pair(const T* p) {

@@ -100,7 +100,6 @@ __device__ __forceinline__ int find_event(const int32_t* __restrict__ off, int k
 // METOK_ERR_INVALID_ARG.  Events of no frames are taken as they are: no key token, no output.
 struct PlanParams {
     int Tn, N, k, n_key_events, event_agg, mode, tile_rows, chunk_cols;
-    int wide_min, wide_max;                     // CUDA-core merge: units of 64 x 64 instead if there are this many of them (wide_max 0: never)
     int rows_with_keys;                         // the merge's row tiles run over all tokens of an event (1) or only over those that are no key token (0)
     int grid, s1, s2, s1_nonkey, s2_nonkey;     // POOL: side of the token grid and the four strides
     double keep_key, keep_nonkey, beta;
@@ -113,7 +112,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
                   const int32_t* __restrict__ event_offsets, PlanParams pp,
                   float* __restrict__ event_score, uint8_t* __restrict__ event_is_key,
                   int32_t* __restrict__ ev_lo, int32_t* __restrict__ ev_budget, int32_t* __restrict__ ev_out_off,
-                  int32_t* ev_unit_off, int32_t* ev_wide_off,
+                  int32_t* ev_unit_off,
                   int32_t* __restrict__ frame_ev, int32_t* __restrict__ frame_stride,
                   int32_t* __restrict__ frame_off, int32_t* __restrict__ n_out, int32_t* __restrict__ counters, int n_counters,
                   int32_t* __restrict__ status) {
@@ -124,7 +123,6 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
     if (rank == 0 && threadIdx.x == 0) *status = 0;
     for (int i = rank * 1024 + threadIdx.x; i < n_counters; i += C * 1024) counters[i] = 0;   // what later kernels of the call count in
     __shared__ int s_scan[32];
-    __shared__ int s_wide;
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int k = pp.k, Tn = pp.Tn;
     // frame_score[f] = mean of the frame's N token scores; eight lanes per frame (a lane's loads are
@@ -219,7 +217,6 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
         auto units = [&](int m, int b, int rows, int cols) {                 // row tiles x key chunks
             return (m - (pp.rows_with_keys ? 0 : b) + rows - 1) / rows * ((b + cols - 1) / cols);
         };
-        bool wide = false;
         for (int e = tid; e < k; e += nthr) {
             const int m = (s_off[e + 1] - s_off[e]) * pp.N;
             const double ratio = s_key[e] ? pp.keep_key : pp.keep_nonkey;
@@ -232,19 +229,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
             s_bud[e] = (int)b;
             s_units[e] = units(m, (int)b, pp.tile_rows, pp.chunk_cols);
         }
-        if (pp.wide_max > 0) {
-            if (tid == 0) s_wide = 0;
-            __syncthreads();
-            int n = 0;
-            for (int e = tid; e < k; e += nthr) n += units((s_off[e + 1] - s_off[e]) * pp.N, s_bud[e], 64, 64);
-            if (n > 0) atomicAdd(&s_wide, n);
-            __syncthreads();
-            wide = s_wide >= pp.wide_min && s_wide <= pp.wide_max;
-            if (wide)
-                for (int e = tid; e < k; e += nthr) s_units[e] = units((s_off[e + 1] - s_off[e]) * pp.N, s_bud[e], 64, 64);
-        }
         __syncthreads();
-        int32_t* unit_off = wide ? ev_wide_off : ev_unit_off;   // the other list is empty
         if (tid < 32) {                                     // offsets: one warp, 32 events at a time
             int slots = 0, units = 0;
             for (int e0 = 0; e0 < k; e0 += 32) {
@@ -257,15 +242,14 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
                 }
                 if (e < k) {
                     ev_out_off[e] = slots + bi - b;
-                    unit_off[e] = units + ui - u;
+                    ev_unit_off[e] = units + ui - u;
                 }
                 slots += __shfl_sync(0xFFFFFFFFu, bi, 31);
                 units += __shfl_sync(0xFFFFFFFFu, ui, 31);
             }
             if (tid == 0) {
                 ev_out_off[k] = slots;
-                (wide ? ev_unit_off : ev_wide_off)[k] = 0;
-                unit_off[k] = units;
+                ev_unit_off[k] = units;
                 *n_out = slots;
             }
         }
@@ -431,7 +415,8 @@ struct TokenOut {
     int32_t *out_src, *out_event, *assign;
     int32_t* rest;                 // per event, from its first token's place on: its tokens that are no key token
     unsigned long long* best64;    // packed argmax of the token's similarities
-    int32_t* tile_done;            // at a row tile's first token: key chunks of the tile that are done
+    int32_t* tile_done;            // at a row tile's first token: key chunks of the tile that are done (fp32 on the tensor cores: candidates of the token)
+    uint32_t* key_hash;            // fp32 on the tensor cores, else null: per output, hash of its key token
     MemberLists ml;
 };
 __device__ __forceinline__ void token_out(const TokenOut& o, int lo, int n, int i, int e, int slot0, int place, bool key) {
@@ -443,6 +428,7 @@ __device__ __forceinline__ void token_out(const TokenOut& o, int lo, int n, int 
         o.out_src[slot] = lo + i;
         o.out_event[slot] = e;
         o.assign[lo + i] = slot;
+        if (o.key_hash) o.key_hash[slot] = 0u;
         members_start(o.ml, slot, lo + i, i, n);
     } else {
         o.rest[lo + i - place] = lo + i;
@@ -586,12 +572,10 @@ cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __res
 // Merge-assign on the CUDA cores (fp32 inputs; bf16 only when forced for debugging): fp32 products, added in
 // the order of the row, so every dot product is one chain of fused multiply-adds.
 //
-// Work unit = 8 P of an event's tokens that are no key tokens x 8 P of its key tokens (P = 2, 4 or 8: choose_simt_tile; where
-// the exact count decides, both kernels are launched and one finds no units);
+// Work unit = 8 P of an event's tokens that are no key tokens x 8 P of its key tokens (P = 2 or 4: choose_simt_outputs);
 // the units of all events form one list, a CTA takes its first by its number and the others from a counter; the dot
 // products of a unit are SimtTile's.  Rows past a unit's end are copies of another row: nobody reads their results.
-// 61 x 169 tokens, d = 1156, fp32: 755 us with 64-row CTAs of 4 x 4 outputs per thread that each walked all keys
-// of the event, 204 us now (0.76 of the multiply-adds: key tokens need no assignment).
+// 16 x 169 tokens in two events, d = 1156: the call takes 99 us.  Larger problems go to merge_f32.cuh.
 // Units of one row meet in a 64-bit atomicMax as in the tensor-core kernel: larger value, then lower slot.
 // --------------------------------------------------------------------------- //
 template <typename T, int PT>                       // PT x PT outputs per thread
@@ -652,6 +636,10 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
         }
     }
 }
+
+}  // namespace metok
+#include "merge_f32.cuh"
+namespace metok {
 
 // After it: every token that is no key token to its output.  (In the tensor-core kernel the CTA that does a row tile's last
 // chunk does this; here that cost 15 us at 61 frames, this kernel takes 5.)
@@ -1455,18 +1443,21 @@ merge_avg_kernel(const T* __restrict__ feats, T* __restrict__ out_feats, AvgArgs
 struct VisionWs {
     int32_t* status;          // device status word, first in the workspace
     float* inv_norm;
-    int32_t *ev_lo, *ev_budget, *ev_out_off, *ev_unit_off, *ev_wide_off;   // ev_wide_off: ev_unit_off for units of 64 x 64
+    int32_t *ev_lo, *ev_budget, *ev_out_off, *ev_unit_off;
     int32_t *frame_ev, *frame_stride, *frame_off;   // POOL mode
     uint8_t* is_key;          // the rest: merging modes (TokenOut, MemberLists, AvgArgs)
     int32_t *rest, *tile_done;
     unsigned long long* best64;
     MemberLists ml;
     float* long_sums;
+    F3Planes planes;          // fp32 merge on the tensor cores; so are the candidates' lists and the hashes
+    unsigned long long* cands;
+    uint32_t* key_hash;
     int32_t *long_done, *avg_next, *unit_next;
     int n_counters;           // the counters are cleared together: long, heavy, avg_next, unit_next and long_done
 };
 
-static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, bool merging) {
+static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, bool merging, bool planes) {
     VisionWs w = {};
     w.status = cv.take<int32_t>(64);
     w.inv_norm = cv.take<float>((size_t)Tn * N);
@@ -1474,7 +1465,6 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
     w.ev_budget = cv.take<int32_t>((size_t)k + 1);
     w.ev_out_off = cv.take<int32_t>((size_t)k + 1);
     w.ev_unit_off = cv.take<int32_t>((size_t)k + 1);
-    w.ev_wide_off = cv.take<int32_t>((size_t)k + 1);
     w.frame_ev = cv.take<int32_t>((size_t)Tn);
     w.frame_stride = cv.take<int32_t>((size_t)Tn);
     w.frame_off = cv.take<int32_t>((size_t)Tn + 1);
@@ -1498,6 +1488,12 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
         w.unit_next = w.ml.long_counter + 4;
         w.long_done = w.ml.long_counter + 5;
         w.long_sums = cv.take<float>((size_t)avg_long_cap(d) * kAvgParts * d);
+        if (planes) {
+            w.planes.a = cv.take<uint8_t>(f3_a_bytes((long long)Tn * N, k, d));
+            w.planes.b = cv.take<uint8_t>(f3_b_bytes(cap, k, d));
+            w.cands = cv.take<unsigned long long>((size_t)Tn * N * (kF3Cands + 1));
+            w.key_hash = cv.take<uint32_t>(n);
+        }
     }
     return w;
 }
@@ -1533,34 +1529,49 @@ static MmaTile choose_mma_tile(int Nv, int k, int d, double keep) {
     return best;
 }
 
-// Outputs per thread (a side of the square) of the CUDA-core kernel, from the number of 64 x 64 units of the mean event.
-// Few of them leave SMs idle and last as long as one unit's chain of d steps: 16 x 16 units are then the fastest.  The whole
-// call with 16 x 16 / 32 x 32 / 64 x 64, at that many units: 169 tokens of 1156, 34 units 42 / 48 / 96 us, 57: 51 / 49 / 96,
-// 103: 82 / 70 / 98; 100 tokens of 512, 36: 29 / 32 / 52, 75: 39 / 42 / 55, 98: 48 / 44 / 57.  From there on 32 x 32, except
-// where one round of CTAs does all 64 x 64 units and is well filled (they do a sixth more work in the same time; 32 x 32 /
-// 64 x 64 by their exact number: 690: 239 / 242 us, 738: 236 / 240, 766: 254 / 241, 784: 208 / 197, 846: 271 / 243,
-// 882: 130 / 117, 895: 130 / 184, 950: 294 / 375, 1056: 353 / 433 -- places = 888).  The estimate does not know the events'
-// lengths: within 2/3 and 0.9 of the places only one call in five has its exact number between 5/6 and all of them, and
-// with Zipf lengths 64 x 64 by the estimate alone took up to 35 % longer.  So there event_plan_kernel counts, and both
-// kernels are launched, 32 x 32 first (59 frames of 169 tokens of 1156, Zipf: 427 -> 318 us; 58 of 144 of 1024: 356 -> 243).
-// The second one costs nothing measurable where it finds no units, the first one 2 to 3.5 us where it finds none.
-struct SimtTileChoice { int outputs, wide_min, wide_max; };
-static SimtTileChoice choose_simt_tile(int Nv, int k, double keep) {
-    const double m = (double)Nv / k, keys = std::max(1.0, keep * m), units = ((m - keys) / 64 + 0.5) * (keys / 64 + 0.5) * k;
-    const int places = kNumSMs * sa_ctas_per_sm(8);
-    SimtTileChoice c = {units < kNumSMs / 2 ? 2 : 4, 0, 0};
-    if (units >= places * 2 / 3 && units <= places * 0.9) {
-        c.wide_min = places * 5 / 6;
-        c.wide_max = places;
-    }
-    return c;
-}
-
 // The tensor-core merge path needs bf16 rows that TMA can address (16-byte row pitch);
 // METOK_DEBUG_FORCE_SIMT=1 in the environment selects the CUDA-core kernels (debugging aid).
-static bool use_mma_path(int d) {
-    static const bool force_simt = [] { const char* e = getenv("METOK_DEBUG_FORCE_SIMT"); return e && e[0] == '1'; }();
-    return !force_simt && d % 8 == 0;
+static bool force_simt() {
+    static const bool force = [] { const char* e = getenv("METOK_DEBUG_FORCE_SIMT"); return e && e[0] == '1'; }();
+    return force;
+}
+static bool use_mma_path(int d) { return !force_simt() && d % 8 == 0; }
+
+// Outputs per thread (a side of the square) of the CUDA-core kernel, from the number of 64 x 64 units of the mean event.
+// Few of them leave SMs idle and last as long as one unit's chain of d steps: 16 x 16 units are then the fastest.  The whole
+// call with 16 x 16 / 32 x 32, at that many units: 169 tokens of 1156, 34 units 42 / 48 us, 57: 51 / 49, 103: 82 / 70; 100 tokens
+// of 512, 36: 29 / 32, 75: 39 / 42, 98: 48 / 44.  (Larger units would pay only for rows so short that fp32 stays on the CUDA
+// cores however many units there are.)
+static int choose_simt_outputs(int Nv, int k, double keep) {
+    const double m = (double)Nv / k, keys = std::max(1.0, keep * m), units = ((m - keys) / 64 + 0.5) * (keys / 64 + 0.5) * k;
+    return units < kNumSMs / 2 ? 2 : 4;
+}
+
+// The fp32 merge: on the tensor cores (keys per unit; see merge_f32.cuh) or 0, on the CUDA cores.  Both times are estimated for
+// the mean event.  Tensor cores: the planes read and written at 5.2 TB/s, then rounds of units, a step of which takes what its
+// tensor instructions or its shared-memory traffic take, then the chains of the near ties; the events' lengths are not known
+// here, so that units are counted as 1.3 times the estimate where fewer keys per unit would just fit a round.  CUDA cores: 64 us
+// per 10^9 multiply-adds (and 3 us in favour of what needs no planes).  The whole call on the CUDA cores / on the tensor cores,
+// frames x tokens x width in events, keep: 24 x 100 x 512 in 3, 0.3: 56 / 58 us; 40 x 100 x 512 in 4: 67 / 61; 64 x 100 x 512 in 7: 104 / 66;
+// 20 x 64 x 2048 in 2: 80 / 95; 50 x 64 x 2048 in 4: 140 / 122; 14 x 144 x 3584 in 2, 0.2: 174 / 175; 20 x 144 x 3584 in 2: 225 / 183;
+// 128 x 64 x 128 in 6: 61 / 54; 61 x 169 x 1156 in 7, 0.25: 265 / 133.
+// The planes take one and a half times the memory of the features, and the share of the key tokens as much again, so beyond kF3MaxBytes
+// the CUDA cores do it.
+constexpr size_t kF3MaxBytes = (size_t)1 << 30;
+static int choose_f3(int Nv, int k, int d, int cap, double keep) {
+    if (d < kF3MinD || f3_a_bytes(Nv, k, d) + f3_b_bytes(cap, k, d) > kF3MaxBytes) return 0;
+    const double m = (double)Nv / k, keys = std::max(1.0, keep * m), rest = m - keys;
+    double best = 0.0;
+    int best_bn = 0;
+    for (const int bn : {256, 128, 64}) {
+        const double units = k * (rest / kF3BM + 0.5) * (keys / bn + 0.5) * (bn < 256 ? 1.3 : 1.0);
+        const double cols = std::min(256.0, std::ceil(keys / std::ceil(keys / bn) / 16) * 16);
+        const double mma = 12 * std::max(0.024, cols * 0.272e-3), smem = ((kF3BM + cols) * kF3RowBytes + 12 * (4096 + 32 * cols)) / 243e3;
+        const double us = std::ceil(units / kNumSMs) * (f3_steps(d) * std::max(mma, smem) + 3.0);
+        if (!best_bn || us < 0.9 * best) { best_bn = bn; best = us; }
+    }
+    best += 11.0 + 0.004 * d + (double)Nv * d * 10.0 / 5.2e6;
+    return best < 3.0 + 64e-9 * k * rest * keys * d ? best_bn : 0;
 }
 
 static bool ratio_ok(double r) { return r > 0.0 && r <= 1.0; }
@@ -1578,7 +1589,9 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     constexpr bool kBf16 = sizeof(T) == 2;
     const bool mma = kBf16 && use_mma_path(d) && p->mode == METOK_MODE_TOPK_MERGE;
     Carver cv(ws);
-    VisionWs w = carve_vision(cv, Tn, N, k, d, cap, p->mode == METOK_MODE_TOPK_MERGE);
+    const double keep = p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey;
+    const int f3_bn = kBf16 || p->mode != METOK_MODE_TOPK_MERGE || force_simt() ? 0 : choose_f3(Nv, k, d, cap, keep);
+    VisionWs w = carve_vision(cv, Tn, N, k, d, cap, p->mode == METOK_MODE_TOPK_MERGE, f3_bn > 0);
     // (the status word and the scratch that must start cleared are written by event_plan_kernel)
     if (const int rc = debug_arm(w.status, st)) return rc;
 
@@ -1592,15 +1605,13 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         }
         METOK_LAUNCH_CHECK();
     }
-    const double keep = p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey;
     const MmaTile tile = choose_mma_tile(Nv, k, d, keep);
-    const SimtTileChoice simt = choose_simt_tile(Nv, k, keep);
+    const int simt = choose_simt_outputs(Nv, k, keep);
     PlanParams pp;
     pp.Tn = Tn; pp.N = N; pp.k = k;
     pp.n_key_events = min(k, ceilq(p->alpha * (double)k));
-    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? tile.bm : 8 * simt.outputs;
-    pp.chunk_cols = mma ? tile.bn : 8 * simt.outputs;
-    pp.wide_min = simt.wide_min; pp.wide_max = mma ? 0 : simt.wide_max;
+    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? tile.bm : f3_bn ? kF3BM : 8 * simt;
+    pp.chunk_cols = mma ? tile.bn : f3_bn ? f3_bn : 8 * simt;
     pp.rows_with_keys = mma ? 1 : 0;
     pp.keep_key = p->keep_key; pp.keep_nonkey = p->keep_nonkey; pp.beta = p->beta;
     pp.key_given = p->key_events_given;
@@ -1616,7 +1627,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     {
         METOK_TIMED("event_plan_kernel", st);
         launch_chained_clusters(plan_ctas, event_plan_kernel, dim3(plan_ctas), dim3(1024), plan_smem, st, token_score, frame_score, event_offsets, pp, event_score,
-                       event_is_key, w.ev_lo, w.ev_budget, w.ev_out_off, w.ev_unit_off, w.ev_wide_off, w.frame_ev, w.frame_stride, w.frame_off,
+                       event_is_key, w.ev_lo, w.ev_budget, w.ev_out_off, w.ev_unit_off, w.frame_ev, w.frame_stride, w.frame_off,
                        n_out, w.ml.long_counter, w.n_counters, w.status);
     }
     METOK_LAUNCH_CHECK();
@@ -1636,7 +1647,8 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         return METOK_OK;
     }
 
-    const TokenOut to = {w.is_key, out_src, out_event, assign, w.rest, w.best64, w.tile_done, w.ml};
+    const TokenOut to = {w.is_key, out_src, out_event, assign, w.rest, w.best64, w.tile_done, w.key_hash, w.ml};
+    const F3Cands cands = {w.cands, w.tile_done, w.key_hash};
     {
         // an event has at most Tn - (k - 1) frames if none is empty; cs_event_topk_long takes one that has more
         const long long longest = (long long)(Tn - (k - 1)) * N;
@@ -1683,24 +1695,48 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         }
         METOK_LAUNCH_CHECK();
     } else {
-        auto assign_units = [&](auto kernel, int outputs, const int32_t* unit_off) -> int {
+        if constexpr (!kBf16) {
+            if (f3_bn) {
+                // the planes: about eight CTAs per SM, rows in shares of their steps where there are few
+                const int steps = f3_steps(d), shares = std::min(steps, std::max(1, kNumSMs * 8 * 32 / Nv)), per = ceil_div(steps, shares);
+                {
+                    METOK_TIMED("merge_planes_kernel", st);
+                    launch_chained(merge_planes_kernel, dim3(ceil_div(Nv, 32), ceil_div(steps, per)), dim3(256), 0, st, feats, Nv, d, N,
+                                   w.ev_lo, k, w.ev_out_off, to, w.planes, cands, f3_bn, per, w.status);
+                }
+                METOK_LAUNCH_CHECK();
+                METOK_ALLOW_SMEM(merge_assign_f32_mma_kernel, kF3SmemBytes);
+                {
+                    METOK_TIMED("merge_assign_f32_mma_kernel", st);
+                    launch_chained(merge_assign_f32_mma_kernel, dim3(kNumSMs), dim3(kF3Threads), kF3SmemBytes, st, d, N, w.ev_lo, k,
+                                   w.ev_out_off, w.ev_unit_off, inv_norm, to, w.planes, cands, f3_bn, w.status);
+                }
+                METOK_LAUNCH_CHECK();
+                {
+                    METOK_TIMED("merge_join_f32_kernel", st);
+                    launch_chained(merge_join_f32_kernel, dim3(ceil_div(Nv, 4 * kF3JoinWarps)), dim3(kF3JoinWarps * 32), 0, st, feats, Nv,
+                                   d, N, w.ev_lo, k, w.ev_out_off, inv_norm, to, cands);
+                }
+                METOK_LAUNCH_CHECK();
+            }
+        }
+        if (!f3_bn) {
             {
                 METOK_TIMED("merge_assign_simt_kernel", st);
-                launch_chained(kernel, dim3(kNumSMs * sa_ctas_per_sm(outputs)), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
-                               w.ev_out_off, unit_off, inv_norm, w.unit_next, to);
+                auto assign_units = [&](auto kernel) {
+                    launch_chained(kernel, dim3(kNumSMs * sa_ctas_per_sm(simt)), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
+                                   w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to);
+                };
+                if (simt == 2) assign_units(merge_assign_simt_kernel<T, 2>);
+                else assign_units(merge_assign_simt_kernel<T, 4>);
             }
             METOK_LAUNCH_CHECK();
-            return METOK_OK;
-        };
-        int rc = simt.outputs == 2 ? assign_units(merge_assign_simt_kernel<T, 2>, 2, w.ev_unit_off)
-                                   : assign_units(merge_assign_simt_kernel<T, 4>, 4, w.ev_unit_off);
-        if (rc == METOK_OK && pp.wide_max > 0) rc = assign_units(merge_assign_simt_kernel<T, 8>, 8, w.ev_wide_off);
-        if (rc != METOK_OK) return rc;
-        {
-            METOK_TIMED("merge_join_kernel", st);
-            launch_chained(merge_join_kernel, dim3(ceil_div(Nv, 256)), dim3(256), 0, st, Nv, N, w.ev_lo, k, w.ev_out_off, to);
+            {
+                METOK_TIMED("merge_join_kernel", st);
+                launch_chained(merge_join_kernel, dim3(ceil_div(Nv, 256)), dim3(256), 0, st, Nv, N, w.ev_lo, k, w.ev_out_off, to);
+            }
+            METOK_LAUNCH_CHECK();
         }
-        METOK_LAUNCH_CHECK();
     }
 
     // Pieces of up to 2 KB, or of 1 KB (so that twice as many copies of a row list are in flight per warp) when the rows
@@ -1771,10 +1807,13 @@ extern "C" int metok_compress_vision_bound(int T, int N, int k, const metok_visi
 
 extern "C" size_t metok_compress_vision_workspace_bytes(int dtype, int T, int N, int d, int k, int cap,
                                                         const metok_vision_params* p) {
-    (void)dtype;
     if (T < 1 || N < 1 || k < 1 || d < 1 || cap < 0) return 0;
     Carver cv(nullptr);
-    carve_vision(cv, T, N, k, d, cap, !(p && p->mode == METOK_MODE_POOL));
+    const bool merging = !(p && p->mode == METOK_MODE_POOL);
+    bool planes = merging && dtype == METOK_F32 && !force_simt() && (long long)T * N <= 0x7FFFFFFFLL / 2;
+    if (planes && p) planes = choose_f3(T * N, k, d, cap, p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey) > 0;
+    else if (planes) planes = f3_a_bytes((long long)T * N, k, d) + f3_b_bytes(cap, k, d) <= kF3MaxBytes;
+    carve_vision(cv, T, N, k, d, cap, merging, planes);
     return cv.total();
 }
 

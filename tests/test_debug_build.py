@@ -91,6 +91,23 @@ def test_wait_runs_out_in_the_stage1_kernels_and_the_next_call_is_clean(debug_li
         _vision_equal(again, want)
 
 
+def test_fp32_merge_on_the_tensor_cores_wait_and_indices(debug_lib):
+    Vd, offs, td, p = _vision_case(T=10, N=400, d=1032)                  # fp32 and enough for the tensor cores
+    Vd, td = Vd.float(), td.float()
+    want = {k_: (v.clone() if isinstance(v, torch.Tensor) else v) for k_, v in _normal_vision(Vd, offs, td, p).items()}
+    assert debug_lib.metok_debug_set(1, MERGE_ASSIGN) == 0
+    got = B.metok_compress_vision(Vd, offs, td, p)
+    torch.cuda.synchronize()
+    assert int(got["status"].item()) == TIMEOUT
+    assert debug_lib.metok_debug_set(1, 0) == 0
+    again = B.metok_compress_vision(Vd, offs, td, p)
+    torch.cuda.synchronize()
+    words = B.workspace(1, Vd.device)[:16].view(torch.int32)
+    assert int(words[0].item()) == 0 and int(words[2].item()) == 0
+    n = int(again["n_out"].item())
+    assert torch.equal(again["assign"], want["assign"]) and torch.equal(again["out_feats"][:n], want["out_feats"][:n])
+
+
 def test_wait_runs_out_in_the_prefill_kernels_and_the_next_call_is_clean(debug_lib):
     args = _prefill_case()
     want = {k_: (v.clone() if isinstance(v, torch.Tensor) else v) for k_, v in _normal_prefill(args).items()}

@@ -364,3 +364,84 @@ def test_schedule_levels_that_share_buffers(dtype, dh):
         rows_kept = rows_kept[want[s][1].long()]
         assert torch.equal(origins[s], want[s][4]) and torch.equal(groups[s], want[s][3])
     assert torch.equal(b[:n].view(torch.uint8), h[0][rows_kept].view(torch.uint8))
+
+
+# fp32 features wide and many enough for the tensor cores: tiles of 128 other tokens and chunks of up to 256 key tokens of an event, at
+# their last row and the one behind it; steps of 32 elements with 4, 28 and 32 in the last; an event of one frame
+@pytest.mark.parametrize("N,d,keep,lens", [
+    (160, 644, 0.2, [16]), (161, 640, 0.2, [10, 6]), (257, 636, 0.25, [8, 8, 2]), (255, 516, 0.25, [4, 8, 1]), (256, 516, 0.5, [4, 4]),
+    (300, 100, 0.4, [9, 1, 20, 2]), (100, 516, 0.3, [64]), (32, 516, 0.9, [70, 60]),
+])
+def test_fp32_merge_on_the_tensor_cores(N, d, keep, lens):
+    rng = np.random.default_rng(N + d)
+    T = sum(lens)
+    V = rng.standard_normal((T, N, d)).astype(np.float32)
+    V *= np.exp(rng.uniform(-6.0, 6.0, (T, N, 1))).astype(np.float32)    # rows of very different size
+    t = rng.standard_normal(d).astype(np.float32)
+    rep = R.compress_case(V, t, np.concatenate([[0], np.cumsum(lens)]).astype(np.int32), "f32", 0.5, keep, keep)
+    assert rep["key_mismatches"] <= rep["key_near_ties"]
+    assert rep["assign_mismatches"] <= rep["assign_near_ties"]
+
+
+def _fp32_merge_case(seed=9, T=16, N=160, d=644, keep=0.2):
+    rng = np.random.default_rng(seed)
+    V = rng.standard_normal((T * N, d)).astype(np.float32)
+    t = rng.standard_normal(d).astype(np.float32)
+    inv = 1.0 / np.maximum(np.sqrt((V.astype(np.float64) ** 2).sum(1)), 1e-8)
+    score = (V.astype(np.float64) @ t) * inv / np.linalg.norm(t)
+
+    def run(feats, norms):
+        scored = {"token_score": torch.from_numpy(score.astype(np.float32)).cuda(), "token_inv_norm": torch.from_numpy(norms.astype(np.float32)).cuda()}
+        got = B.metok_compress_vision(torch.from_numpy(feats.reshape(T, N, d)).cuda(), torch.tensor([0, T], dtype=torch.int32, device="cuda"),
+                                      torch.from_numpy(t).cuda(), B.vision_params(0.5, keep, keep), scored=scored)
+        torch.cuda.synchronize()
+        assert int(got["status"].item()) == 0
+        return got["out_src"][:int(got["n_out"].item())].cpu().numpy(), got["assign"].cpu().numpy()
+    return V, inv, run
+
+
+def test_fp32_merge_of_rows_that_are_no_numbers():
+    """A token with an infinity joins the first key token whose product is +inf, one with a NaN joins none; a key token that
+    is no number is joined by none; nobody else changes."""
+    V, inv, run = _fp32_merge_case()
+    src, clean = run(V, inv)
+    rest = np.setdiff1d(np.arange(len(V)), src)
+    up, down, both, nan = rest[[3, 200, 700, 1500]]
+    bad, norms = V.copy(), inv.copy()
+    bad[up, 5], bad[down, 643], bad[nan, 17] = np.inf, -np.inf, np.nan
+    bad[both, 1], bad[both, 2] = np.inf, -np.inf
+    norms[[up, down, both]], norms[nan] = 0.0, 1e8                       # as the scoring pass leaves them
+    for key in (None, 40, 300):                                          # and a key token of the first or the second chunk
+        if key is not None:
+            bad[src[key], 9], norms[src[key]] = np.inf, 0.0
+        s, a = run(bad, norms)
+        keys, finite = bad[src], norms[src] > 0
+        assert np.array_equal(s, src)
+        assert a[up] == np.flatnonzero((keys[:, 5] > 0) & finite)[0] and a[down] == np.flatnonzero((keys[:, 643] < 0) & finite)[0]
+        assert a[both] == np.flatnonzero((keys[:, 1] > 0) & (keys[:, 2] < 0) & finite)[0]
+        assert a[nan] == -1
+        same = np.setdiff1d(rest, [up, down, both, nan])
+        same = same[finite[clean[same]]]
+        assert np.array_equal(a[same], clean[same]) and finite[a[np.setdiff1d(rest, [nan])]].all()
+
+
+@pytest.mark.parametrize("copies", [1, 4, 16])
+def test_fp32_merge_decides_near_ties_as_the_chain_of_multiply_adds(copies):
+    """Key tokens that differ by little, and copies: the key with the largest chain of fp32 multiply-adds, the first of equal ones."""
+    V, inv, run = _fp32_merge_case(seed=copies)
+    src, _ = run(V, inv)
+    rng = np.random.default_rng(copies)
+    close = V.copy()
+    for j in range(0, len(src) - copies, copies + 1):                    # groups of equal keys and one a few ulps away
+        close[src[j + 1:j + copies]] = close[src[j]]
+        close[src[j + copies]] = close[src[j]] * (1.0 + 3e-7 * rng.integers(-2, 3, V.shape[1])).astype(np.float32)
+    rest = np.setdiff1d(np.arange(len(V)), src)[::7]
+    close[rest] = close[src[rng.integers(0, len(src), len(rest))]] + 0.1 * V[rest]
+    s, a = run(close, inv)
+    assert np.array_equal(s, src)
+    x, y = close[rest].astype(np.longdouble), close[src].astype(np.longdouble)
+    acc = np.zeros((len(rest), len(src)), dtype=np.float32)
+    for i in range(V.shape[1]):                                          # a fused multiply-add is one rounding of the exact sum
+        acc = (acc.astype(np.longdouble) + np.outer(x[:, i], y[:, i])).astype(np.float32)
+    want = (acc * inv[src].astype(np.float32)[None]).argmax(1)
+    assert np.array_equal(a[rest], want)
