@@ -60,12 +60,16 @@ __device__ __forceinline__ void attn_tile_sources(const T* Qg, const T* Kg, cons
 template <typename T>
 __global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? sa_ctas_per_sm(kAtPT) : 4)
 attn_stats_kernel(const T* __restrict__ q_text, const T* __restrict__ k_all, AttnDims dm,
-                  float* __restrict__ part_m, float* __restrict__ part_l) {
+                  float* __restrict__ part_m, float* __restrict__ part_l, int32_t* __restrict__ status) {
     grid_dep_wait();
     using Tile = SimtTile<T, kAtPT>;
     constexpr int PT = kAtPT;
     __shared__ __align__(16) Tile tile;
     const int split = blockIdx.x, rt = blockIdx.y, g = blockIdx.z;
+    if (status && split == 0 && rt == 0 && g == 0 && threadIdx.x == 0) {     // as in attn_stats_mma_kernel
+        *status = 0;
+        status[kStatusCounts] = status[kStatusCounts + 1] = 0;
+    }
     const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;
     const T* Qg = q_text + (size_t)g * dm.R * dm.dh;
     const T* Kg = k_all + (size_t)g * dm.S * dm.dh;
@@ -203,26 +207,29 @@ attn_colsum_kernel(const T* __restrict__ q_text, const T* __restrict__ k_all, At
     }
 }
 
-// scores[j] = inv_rows * (sum of the planes, in their order), for up to kMaxPruneLevels levels at once.  With `group`, the
-// blocks of the first level also write origin[j] = j and count the tokens of classes 0 and 1.
+// scores[j] = inv_rows * (sum of the planes, in their order), for one level or for all levels of a schedule.  With several,
+// the blocks of the first also write origin[j] = j and count the tokens of classes 0 and 1.  (The kernel is so short that what
+// one level does not need is left out at compile time: 2.8 us with one, 3.6 with the levels looked up.)
 struct ReduceLevel { const float* part_col; float* scores; int n_vis, block0; };   // block0: the level's first block
+template <int NL>
 struct ReduceArgs {
-    ReduceLevel lv[kMaxPruneLevels];
+    ReduceLevel lv[NL];
     int nparts;
     float inv_rows;
-    const int32_t* group;
+    const int32_t* group;                                     // several levels, else null
     int32_t *origin, *counts;
 };
+template <int NL>
 __global__ void __launch_bounds__(256)
-attn_score_reduce_kernel(ReduceArgs ra) {
+attn_score_reduce_kernel(const __grid_constant__ ReduceArgs<NL> ra) {
     grid_dep_wait();
     int level = 0;
 #pragma unroll
-    for (int l = 1; l < kMaxPruneLevels; ++l) level += (int)blockIdx.x >= ra.lv[l].block0;
-    const ReduceLevel lv = ra.lv[level];
-    const float* part_col = lv.part_col;
-    const int n_vis = lv.n_vis, nparts = ra.nparts, j = ((int)blockIdx.x - lv.block0) * 256 + (int)threadIdx.x;
-    if (ra.group && level == 0) {
+    for (int l = 1; l < NL; ++l) level += (int)blockIdx.x >= ra.lv[l].block0;
+    const float* __restrict__ part_col = ra.lv[level].part_col;
+    const int n_vis = ra.lv[level].n_vis, nparts = ra.nparts;
+    const int j = ((int)blockIdx.x - (NL > 1 ? ra.lv[level].block0 : 0)) * 256 + (int)threadIdx.x;
+    if (NL > 1 && level == 0) {
         const int g = j < n_vis ? ra.group[j] : -1;
         const int c0 = __syncthreads_count(g == 0), c1 = __syncthreads_count(g == 1);
         if (threadIdx.x < 2) atomicAdd(&ra.counts[threadIdx.x], threadIdx.x == 0 ? c0 : c1);
@@ -239,7 +246,7 @@ attn_score_reduce_kernel(ReduceArgs ra) {
         for (int u = 0; u < 8; ++u) a += v[u];
     }
     for (; p < nparts; ++p) a += part_col[(size_t)p * n_vis + j];
-    lv.scores[j] = a * ra.inv_rows;
+    ra.lv[level].scores[j] = a * ra.inv_rows;
 }
 
 // --------------------------------------------------------------------------- //
@@ -303,13 +310,45 @@ class_topk_kernel(const float* __restrict__ scores, size_t score_stride, const i
     }
 }
 
+// Where the selection adds the planes itself, a launch less: few planes, of which four are in flight (40 of 200 tokens: 18.1
+// us the call with the sum apart, 19.5 inside), and little to read per CTA (bytes).  14 heads in two planes, 6272 tokens:
+// 23.3 -> 22.3 us replayed; 28 in eight, 800 tokens: 21.7 -> 21.5, 8000: 32.5 -> 32.2, 18 432: the same, and left apart.
+constexpr int kPlanesInside = 8, kPlaneBytesInside = 64 * 1024;
+// The scores of one level as the attention passes leave them: n planes to be added in their order (n 0: they are added already).
+struct ScorePlanes { const float* part_col; int n; float inv_rows; float* scores; };
+// This thread's items i_first + 32 j < i_hi of the n_vis: their planes added and the scores written.
+template <int IT>
+__device__ __forceinline__ void add_planes(const ScorePlanes& pl, int n_vis, int i_first, int i_hi, float (&v)[IT]) {
+#pragma unroll
+    for (int j = 0; j < IT; ++j) v[j] = 0.f;
+    constexpr int U = 4;                                      // planes whose loads are in flight
+    for (int p0 = 0; p0 < pl.n; p0 += U) {
+        float x[U][IT];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int j = 0; j < IT; ++j)
+                x[u][j] = p0 + u < pl.n && i_first + 32 * j < i_hi ? pl.part_col[(size_t)(p0 + u) * n_vis + i_first + 32 * j] : 0.f;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int j = 0; j < IT; ++j)
+                if (p0 + u < pl.n) v[j] += x[u][j];
+    }
+#pragma unroll
+    for (int j = 0; j < IT; ++j) {
+        v[j] *= pl.inv_rows;
+        if (i_first + 32 * j < i_hi) pl.scores[i_first + 32 * j] = v[j];
+    }
+}
+
 // The same for up to 81 920 items (select_cluster.cuh): a CTA or a cluster per problem.
-template <int IT, bool kCl, bool kOne>   // kOne: one class and no class array
+template <int IT, bool kCl, bool kOne, bool kPlanes>   // kOne: one class and no class array; kPlanes: the scores are still in planes
 __global__ void __launch_bounds__(IT == kCsMaxItems ? kCsMaxItemsThreads : 1024)
 cs_topk_kernel(const float* __restrict__ scores, size_t score_stride, const int32_t* __restrict__ token_group,
                int n_vis, int G, CsLayout lay, TopkBudgets budgets, int S, int vis_start,
                int32_t* __restrict__ keep_idx, size_t keep_stride, int replicas,
-               int32_t* __restrict__ count_a, int32_t* __restrict__ count_b) {
+               int32_t* __restrict__ count_a, int32_t* __restrict__ count_b, ScorePlanes pl) {
     cs_enter<kCl>();
     grid_dep_wait();
     __shared__ CsShared sm;
@@ -320,8 +359,10 @@ cs_topk_kernel(const float* __restrict__ scores, size_t score_stride, const int3
     int32_t* keep = keep_idx + (size_t)problem * keep_stride;
     const int tid = threadIdx.x, nthr = blockDim.x;
     const CsSlice sl = cs_slice<IT>(n_vis, rank, C);
+    float added[kPlanes ? IT : 1] = {};
+    if constexpr (kPlanes) add_planes<IT>(pl, n_vis, sl.i_first, sl.i_hi, added);
     auto load = [&](int i, float& v, int& c) {
-        v = sc[i];
+        v = kPlanes ? added[(i - sl.i_first) >> 5] : sc[i];
         c = 0;
         if (!kOne) {
             c = token_group[i];
@@ -370,9 +411,18 @@ cs_topk_kernel(const float* __restrict__ scores, size_t score_stride, const int3
     }
 }
 
+static int class_topk(const float* scores, size_t score_stride, const int32_t* token_group, int n_vis, int G,
+                      const int32_t* budgets_host, int S, int vis_start, int32_t* keep_idx, size_t keep_stride,
+                      int replicas, int32_t* count_a, int32_t* count_b, int problems, const ScorePlanes& pl, cudaStream_t st);
 int launch_class_topk(const float* scores, size_t score_stride, const int32_t* token_group, int n_vis, int G,
                       const int32_t* budgets_host, int S, int vis_start, int32_t* keep_idx, size_t keep_stride,
                       int replicas, int32_t* count_a, int32_t* count_b, int problems, cudaStream_t st) {
+    return class_topk(scores, score_stride, token_group, n_vis, G, budgets_host, S, vis_start, keep_idx, keep_stride, replicas, count_a,
+                      count_b, problems, {}, st);
+}
+static int class_topk(const float* scores, size_t score_stride, const int32_t* token_group, int n_vis, int G,
+                      const int32_t* budgets_host, int S, int vis_start, int32_t* keep_idx, size_t keep_stride,
+                      int replicas, int32_t* count_a, int32_t* count_b, int problems, const ScorePlanes& pl, cudaStream_t st) {
     TopkBudgets b;
     for (int g = 0; g < METOK_MAX_GROUPS; ++g) b.v[g] = g < G ? budgets_host[g] : 0;
     const CsPlan plan = cs_plan(n_vis);
@@ -383,16 +433,17 @@ int launch_class_topk(const float* scores, size_t score_stride, const int32_t* t
             METOK_TIMED("class_topk_kernel", st);
             launch_chained_clusters(plan.C, kernel, dim3(problems * plan.C), dim3(plan.threads), lay.bytes, st, scores,
                                     score_stride, token_group, n_vis, G, lay, b, S, vis_start, keep_idx, keep_stride,
-                                    replicas, count_a, count_b);
+                                    replicas, count_a, count_b, pl);
             METOK_LAUNCH_CHECK();
             return METOK_OK;
         };
         const bool one = G == 1 && !token_group;
+        if (pl.n > 0) return plan.C == 1 ? launch(cs_topk_kernel<4, false, false, true>) : launch(cs_topk_kernel<4, true, false, true>);
         if (plan.C == 1)
-            return one ? launch(cs_topk_kernel<4, false, true>) : launch(cs_topk_kernel<4, false, false>);
+            return one ? launch(cs_topk_kernel<4, false, true, false>) : launch(cs_topk_kernel<4, false, false, false>);
         if (plan.items == 4)
-            return one ? launch(cs_topk_kernel<4, true, true>) : launch(cs_topk_kernel<4, true, false>);
-        return one ? launch(cs_topk_kernel<kCsMaxItems, true, true>) : launch(cs_topk_kernel<kCsMaxItems, true, false>);
+            return one ? launch(cs_topk_kernel<4, true, true, false>) : launch(cs_topk_kernel<4, true, false, false>);
+        return one ? launch(cs_topk_kernel<kCsMaxItems, true, true, false>) : launch(cs_topk_kernel<kCsMaxItems, true, false, false>);
     }
     const SelectLayout lay = select_layout(G, select_items_per_cta((long long)S));
     const int nthreads = select_threads(select_items_per_cta((long long)S));
@@ -554,10 +605,11 @@ struct ScoreLevel {
     float* scores;
 };
 
+template <int NL>
 static int launch_score_reduce(const ScoreLevel* lv, int n, float inv_rows, const int32_t* group, int32_t* origin, cudaStream_t st) {
-    ReduceArgs ra = {};
+    ReduceArgs<NL> ra = {};
     int blocks = 0;
-    for (int l = 0; l < kMaxPruneLevels; ++l) {
+    for (int l = 0; l < NL; ++l) {
         ra.lv[l].block0 = l < n ? blocks : 0x7FFFFFFF;
         if (l >= n) continue;
         ra.lv[l].part_col = lv[l].w.part_col;
@@ -572,19 +624,19 @@ static int launch_score_reduce(const ScoreLevel* lv, int n, float inv_rows, cons
     ra.counts = lv[0].w.status + kStatusCounts;
     {
         METOK_TIMED("attn_score_reduce_kernel", st);
-        launch_chained(attn_score_reduce_kernel, dim3(blocks), dim3(256), 0, st, ra);
+        launch_chained(attn_score_reduce_kernel<NL>, dim3(blocks), dim3(256), 0, st, ra);
     }
     METOK_LAUNCH_CHECK();
     return METOK_OK;
 }
 
 template <typename T>
-static int launch_attn_passes(const void* q_text, const void* k_all, const AttnDims& dm, const PrefillWs& w, cudaStream_t st) {
+static int launch_attn_passes(const void* q_text, const void* k_all, const AttnDims& dm, const PrefillWs& w, int32_t* clear, cudaStream_t st) {
     dim3 grid(dm.nsplit, dm.nrt, dm.Hkv);
     {
         METOK_TIMED("attn_stats_kernel", st);
         launch_chained(attn_stats_kernel<T>, grid, dim3(kSaThreads), 0, st, reinterpret_cast<const T*>(q_text), reinterpret_cast<const T*>(k_all),
-                       dm, w.part_m, w.part_l);
+                       dm, w.part_m, w.part_l, clear);
     }
     METOK_LAUNCH_CHECK();
     {
@@ -603,11 +655,10 @@ using namespace metok;
 // a5 as the calls run it, for one level or several: the status word and the class counts cleared, then the two passes and
 // the plane sum; scores[j] = inv_rows * (sum over this call's heads and text queries of the probabilities).  group, origin:
 // see attn_score_reduce_kernel.
-static int run_attention_scores(const ScoreLevel* lv, int n, int dtype, float softmax_scale, float inv_rows, const int32_t* group,
-                                int32_t* origin, cudaStream_t st) {
+static int run_attention_passes(const ScoreLevel* lv, int n, int dtype, float softmax_scale, cudaStream_t st) {
     const AttnDims& dm = lv[0].dm;
     int32_t* status = lv[0].w.status;
-    if (use_mma_attn(dtype, dm.dh)) {                         // attn_stats_mma_kernel does the clearing
+    if (use_mma_attn(dtype, dm.dh)) {                         // (the first stats kernel does the clearing)
         AttnScoreCall calls[kMaxPruneLevels];
         for (int l = 0; l < n; ++l)
             calls[l] = {lv[l].q_text, lv[l].k_all, lv[l].dm.S, lv[l].dm.vis_start, lv[l].dm.n_vis, lv[l].w.part_m, lv[l].w.part_l,
@@ -615,16 +666,21 @@ static int run_attention_scores(const ScoreLevel* lv, int n, int dtype, float so
         const int rc = launch_attn_scores_mma(calls, n, dm.Hq, dm.Hkv, dm.Lt, dm.dh, softmax_scale, status, st);
         if (rc != METOK_OK) return rc;
     } else {
-        // (words 1 and 2 belong to debug builds)
-        METOK_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
-        if (group) METOK_CUDA_TRY(cudaMemsetAsync(status + kStatusCounts, 0, 2 * sizeof(int32_t), st));
         for (int l = 0; l < n; ++l) {
-            const int rc = dtype == METOK_F32 ? launch_attn_passes<float>(lv[l].q_text, lv[l].k_all, lv[l].dm, lv[l].w, st)
-                                              : launch_attn_passes<__nv_bfloat16>(lv[l].q_text, lv[l].k_all, lv[l].dm, lv[l].w, st);
+            int32_t* clear = l == 0 ? status : nullptr;
+            const int rc = dtype == METOK_F32 ? launch_attn_passes<float>(lv[l].q_text, lv[l].k_all, lv[l].dm, lv[l].w, clear, st)
+                                              : launch_attn_passes<__nv_bfloat16>(lv[l].q_text, lv[l].k_all, lv[l].dm, lv[l].w, clear, st);
             if (rc != METOK_OK) return rc;
         }
     }
-    return launch_score_reduce(lv, n, inv_rows, group, origin, st);
+    return METOK_OK;
+}
+static int run_attention_scores(const ScoreLevel* lv, int n, int dtype, float softmax_scale, float inv_rows, const int32_t* group,
+                                int32_t* origin, cudaStream_t st) {
+    const int rc = run_attention_passes(lv, n, dtype, softmax_scale, st);
+    if (rc != METOK_OK) return rc;
+    return group ? launch_score_reduce<kMaxPruneLevels>(lv, n, inv_rows, group, origin, st)
+                 : launch_score_reduce<1>(lv, 1, inv_rows, nullptr, nullptr, st);
 }
 
 extern "C" size_t metok_prefill_prune_workspace_bytes(int dtype, int Hq, int Hkv, int Lt, int S, int dh, int n_vis) {
@@ -681,10 +737,15 @@ extern "C" int metok_prefill_prune(const void* q_text, const void* k_all, const 
     int rc = debug_arm(w.status, st);
     if (rc != METOK_OK) return rc;
     const ScoreLevel lv = {q_text, k_all, dm, w, scores};
-    rc = run_attention_scores(&lv, 1, dtype, softmax_scale, 1.0f / (float)(Hq * Lt), nullptr, nullptr, st);
+    const float inv_rows = 1.0f / (float)(Hq * Lt);
+    const CsPlan plan = cs_plan(n_vis);
+    const bool inside = plan.fits && plan.items == 4 && w.n_planes <= kPlanesInside &&
+                        (long long)w.n_planes * n_vis * 4 <= (long long)plan.C * kPlaneBytesInside;
+    rc = inside ? run_attention_passes(&lv, 1, dtype, softmax_scale, st)
+                : run_attention_scores(&lv, 1, dtype, softmax_scale, inv_rows, nullptr, nullptr, st);
     if (rc != METOK_OK) return rc;
-    rc = launch_class_topk(scores, 0, token_group, n_vis, G, group_budget, S, vis_start, keep_idx, 0, 1, S_out,
-                           nullptr, 1, st);
+    rc = class_topk(scores, 0, token_group, n_vis, G, group_budget, S, vis_start, keep_idx, 0, 1, S_out, nullptr, 1,
+                    {w.part_col, inside ? w.n_planes : 0, inv_rows, scores}, st);
     if (rc != METOK_OK) return rc;
     if (hidden) {
         rc = launch_gather_rows_bulk(hidden, hidden_out, keep_idx, S_out, (size_t)D * eb, S, w.status, "gather_rows_kernel",

@@ -445,3 +445,26 @@ def test_fp32_merge_decides_near_ties_as_the_chain_of_multiply_adds(copies):
         acc = (acc.astype(np.longdouble) + np.outer(x[:, i], y[:, i])).astype(np.float32)
     want = (acc * inv[src].astype(np.float32)[None]).argmax(1)
     assert np.array_equal(a[rest], want)
+
+
+# the selection adds the score planes itself (up to eight of them, 64 KB per CTA: 8 KV heads to 2048 tokens in one CTA, to 16 384 in a
+# cluster) or a launch before it does; both against the scores computed alone
+@pytest.mark.parametrize("Hq,Hkv,Lt,n_vis", [(8, 8, 3, 1), (8, 8, 3, 2048), (8, 8, 3, 2049), (9, 9, 3, 40), (2, 2, 5, 4096), (2, 2, 5, 4097), (8, 8, 3, 16384),
+                                             (8, 8, 3, 16385), (4, 1, 200, 33000)])
+@pytest.mark.parametrize("dtype,dh", [(torch.bfloat16, 64), (torch.float32, 8)])
+def test_score_planes_inside_the_selection(Hq, Hkv, Lt, n_vis, dtype, dh):
+    g = torch.Generator(device="cuda").manual_seed(n_vis + Hq)
+    S = n_vis + Lt + 2
+    q = torch.randn((Hq, Lt, dh), device="cuda", generator=g).to(dtype)
+    k = torch.randn((Hkv, S, dh), device="cuda", generator=g).to(dtype)
+    group = (torch.rand(n_vis, device="cuda", generator=g) < 0.4).to(torch.int32)
+    hidden = torch.randn((S, 16), device="cuda", generator=g).to(dtype)
+    budgets = [(int((group == c).sum()) + 1) // 2 for c in (0, 1)]
+    got = B.metok_prefill_prune(q, k, hidden, 2, n_vis, group, budgets, dh ** -0.5)
+    scores = B.metok_attention_scores(q, k, 2, n_vis, dh ** -0.5)
+    want = B.metok_prune_by_scores(scores, hidden, S, 2, group, budgets)
+    torch.cuda.synchronize()
+    n = int(want["S_out"].item())
+    assert int(got["status"].item()) == 0 and int(got["S_out"].item()) == n == S - n_vis + sum(budgets)
+    assert torch.equal(got["scores"], scores) and torch.equal(got["keep_idx"][:n], want["keep_idx"][:n])
+    assert torch.equal(got["hidden_out"][:n].view(torch.uint8), want["hidden_out"][:n].view(torch.uint8))
