@@ -755,7 +755,7 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     const int total_units = ev_unit_off[k];
     if ((int)blockIdx.x >= total_units) return;
     const int ksteps = (d + kMmaBK - 1) / kMmaBK;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
 
@@ -779,78 +779,91 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
 
-    // The two single-thread loops below run once per K step with nothing to hide their latency:
-    // stage and phase are counted (no division), addresses and descriptor words only move by adds.
+    // The loops of warps 0 and 1 run once per K step with nothing to hide their latency: stage and phase are counted (no
+    // division), addresses and descriptor words only move by adds, and the whole warp takes every step while one elected
+    // thread issues, so that all of these stay in uniform registers.  (Inside a branch of lane 0 a step cost the issuing
+    // thread some 1000 clocks, as long as its products: 250 for a wait that is over, 75 per product, 100 for the commit.  The
+    // launch, 32 x 144 tokens of 1024 / 128 x 144 of 3584 / 512 x 144 of 1024: 20.5 / 49.5 / 138.5 us, 18.9 / 47.3 / 129.2 now.)
+    const int units = __shfl_sync(0xFFFFFFFFu, total_units, 0);
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             prefetch_tmap(&tmA);
             prefetch_tmap(&tmA_half);
-            int s = 0, issued = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
-                const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
-                const bool two = mt.bm > 128 && mu.row_end - mu.row0 > 128;   // both row halves hold rows of the event
-                const CUtensorMap* a0 = two ? &tmA : &tmA_half;
-                const uint32_t tx = (two ? 256u : 128u) * kMmaBK * 2;
-                for (int ks = 0; ks < ksteps; ++ks) {
-                    if (!mbar_wait(smem_u32(&empty_bar[0]) + 8u * s, ph ^ 1u, abort_flag)) { ok = false; break; }
-                    const uint32_t fb = smem_u32(&full_bar[0]) + 8u * s;
+        }
+        __syncwarp();
+        int s = 0, issued = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
+            const int row0 = __shfl_sync(0xFFFFFFFFu, mu.row0, 0), rows = __shfl_sync(0xFFFFFFFFu, mu.row_end, 0) - row0;
+            const bool two = mt.bm > 128 && rows > 128;                   // both row halves hold rows of the event
+            const CUtensorMap* a0 = two ? &tmA : &tmA_half;
+            const uint32_t tx = (two ? 256u : 128u) * kMmaBK * 2;
+            for (int ks = 0; ks < ksteps; ++ks) {
+                if (!mbar_wait_warp(smem_u32(&empty_bar[0]) + 8u * s, ph ^ 1u, abort_flag)) { ok = false; break; }
+                const uint32_t fb = smem_u32(&full_bar[0]) + 8u * s;
+                if (elect_one()) {
                     mbar_arrive_expect_tx(fb, tx);
                     if (!(dbg_withhold(status, kDbgMergeAssign) && blockIdx.x == 0 && issued == 0))   // debug builds: one copy never sent
-                        tma_load_2d(smem_base + (uint32_t)s * mt.stage_bytes, a0, ks * kMmaBK, mu.row0, fb);
-                    ++issued;
-                    if (++s == kMmaStages) { s = 0; ph ^= 1u; }
+                        tma_load_2d(smem_base + (uint32_t)s * mt.stage_bytes, a0, ks * kMmaBK, row0, fb);
                 }
+                __syncwarp();
+                ++issued;
+                if (++s == kMmaStages) { s = 0; ph ^= 1u; }
             }
-            if (!ok) {
-                // let the copies already issued land before the CTA's shared memory goes away
-                for (int back = 1; back <= kMmaStages && back <= issued; ++back) {
-                    const int j = issued - back;
-                    mbar_wait(smem_u32(&full_bar[j % kMmaStages]), (uint32_t)(j / kMmaStages) & 1u, abort_flag);
-                }
+        }
+        if (!ok) {
+            // let the copies already issued land before the CTA's shared memory goes away
+            for (int back = 1; back <= kMmaStages && back <= issued; ++back) {
+                const int j = issued - back;
+                mbar_wait_warp(smem_u32(&full_bar[j % kMmaStages]), (uint32_t)(j / kMmaStages) & 1u, abort_flag);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            int s = 0, n = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            const uint32_t a_lo0 = desc_k128_lo(smem_base);
-            const uint32_t kStageWords = mt.stage_bytes >> 4, kBWords = mt.a_bytes >> 4;
-            constexpr uint32_t kHalfWords = (128 * kMmaBK * 2) >> 4;
-            for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++n) {
-                const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
-                const bool two = mt.bm > 128 && mu.row_end - mu.row0 > 128;
-                if (!mbar_wait(smem_u32(&tempty_bar), ((uint32_t)n & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+        int s = 0, n = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
+        const uint32_t a_lo0 = desc_k128_lo(smem_base);
+        const uint32_t kStageWords = mt.stage_bytes >> 4, kBWords = mt.a_bytes >> 4;
+        constexpr uint32_t kHalfWords = (128 * kMmaBK * 2) >> 4;
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++n) {
+            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
+            const bool two = mt.bm > 128 && __shfl_sync(0xFFFFFFFFu, mu.row_end - mu.row0, 0) > 128;
+            if (!mbar_wait_warp(smem_u32(&tempty_bar), ((uint32_t)n & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t idesc = make_idesc_bf16(128, __shfl_sync(0xFFFFFFFFu, (mu.nvalid + 15) & ~15, 0));
+            for (int ks = 0; ks < ksteps; ++ks) {
+                if (!mbar_wait_warp(smem_u32(&full_bar[0]) + 8u * s, ph, abort_flag)) { ok = false; break; }
+                fence_proxy_async();                             // the key rows were written by ordinary (non-bulk) copies
                 tc_fence_after();
-                const uint32_t idesc = make_idesc_bf16(128, (mu.nvalid + 15) & ~15);
-                for (int ks = 0; ks < ksteps; ++ks) {
-                    if (!mbar_wait(smem_u32(&full_bar[0]) + 8u * s, ph, abort_flag)) { ok = false; break; }
-                    fence_proxy_async();                             // the key rows were written by ordinary (non-bulk) copies
-                    tc_fence_after();
-                    const uint32_t a_lo = a_lo0 + (uint32_t)s * kStageWords, b_lo = a_lo + kBWords;
-                    const uint32_t acc0 = ks != 0 ? 1u : 0u;
+                const uint32_t a_lo = a_lo0 + (uint32_t)s * kStageWords, b_lo = a_lo + kBWords;
+                const uint32_t acc0 = ks != 0 ? 1u : 0u;
+                if (elect_one()) {
                     if (two) {                                       // rows 128..255 of the tile: 16 KiB further on
 #pragma unroll
                         for (int kk = 0; kk < kMmaBK / 16; ++kk) {
-                            umma_bf16_words(tmem_base, a_lo + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
-                            umma_bf16_words(tmem_base + kMmaBN, a_lo + kHalfWords + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
+                            umma_bf16_words(tmem, a_lo + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
+                            umma_bf16_words(tmem + kMmaBN, a_lo + kHalfWords + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
                         }
                     } else {
 #pragma unroll
                         for (int kk = 0; kk < kMmaBK / 16; ++kk)
-                            umma_bf16_words(tmem_base, a_lo + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
+                            umma_bf16_words(tmem, a_lo + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
                     }
                     umma_commit(smem_u32(&empty_bar[0]) + 8u * s);   // frees the stage when these MMAs retire
-                    if (++s == kMmaStages) { s = 0; ph ^= 1u; }
                 }
-                if (ok) umma_commit(smem_u32(&tfull_bar));         // both accumulators of this unit complete
+                __syncwarp();
+                if (++s == kMmaStages) { s = 0; ph ^= 1u; }
             }
-            if (!ok) {                                             // wait until whatever was issued has retired
-                umma_commit(smem_u32(&drain_bar));
-                mbar_wait(smem_u32(&drain_bar), 0u, abort_flag);
-            }
+            if (ok && elect_one()) umma_commit(smem_u32(&tfull_bar));   // both accumulators of this unit complete
+            __syncwarp();
+        }
+        if (!ok) {                                             // wait until whatever was issued has retired
+            if (elect_one()) umma_commit(smem_u32(&drain_bar));
+            __syncwarp();
+            mbar_wait_warp(smem_u32(&drain_bar), 0u, abort_flag);
         }
     } else if (warp >= 10) {
         // Key producers.  Thread pt copies 16-byte chunk c = pt % 8 of the rows r = pt / 8 + 16 i,
