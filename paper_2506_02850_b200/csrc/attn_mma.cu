@@ -214,7 +214,7 @@ attn_stats_mma_kernel(const __grid_constant__ AttnBatch<NL> ab, int32_t* __restr
         *status = 0;
         status[kStatusCounts] = status[kStatusCounts + 1] = 0;
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     const uint32_t q_addr = smem_base;
@@ -237,60 +237,72 @@ attn_stats_mma_kernel(const __grid_constant__ AttnBatch<NL> ab, int32_t* __restr
     tc_fence_after();
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
 
+    // Warps 0 and 1, here and in the colsum kernel, stay whole and one elected thread issues: addresses and descriptors are then
+    // in uniform registers.  (In a branch of lane 0 an issue loop costs some 75 clocks per product.  One level of 73 728 keys,
+    // 28 heads x 128 queries: 239.1 us the whole call, 234.7 now; three levels from 18 432: 89.2 -> 86.7; 6272: 23.6 -> 23.2.)
     AttnItem item = {};
     if (warp == 0) {
-        if (lane == 0) {
 #pragma unroll
-            for (int l = 0; l < NL; ++l) { prefetch_tmap(&ab.q[l]); prefetch_tmap(&ab.k[l]); }
-            int it = 0, n = 0;                                 // tiles and items so far
-            bool ok = true;
-            for (; ok && stats_item(ab, n, item); ++n) {
-                const AttnMmaDims& dm = ab.lv[item.level].dm;
-                const CUtensorMap *tmQ = &ab.q[item.level], *tmK = &ab.k[item.level];
-                // the item that had this buffer is done with its query tile
-                const int qb = n % kQBufs;
-                const uint32_t qph = (uint32_t)(n / kQBufs) & 1u;
-                if (!mbar_wait(smem_u32(&q_free_bar[qb]), qph ^ 1u, abort_flag)) { ok = false; break; }
+        for (int l = 0; l < NL; ++l)
+            if (elect_one()) { prefetch_tmap(&ab.q[l]); prefetch_tmap(&ab.k[l]); }
+        __syncwarp();
+        int it = 0, n = 0;                                 // tiles and items so far
+        bool ok = true;
+        for (; ok && stats_item(ab, n, item); ++n) {
+            const AttnMmaDims& dm = ab.lv[item.level].dm;
+            const CUtensorMap *tmQ = &ab.q[item.level], *tmK = &ab.k[item.level];
+            // the item that had this buffer is done with its query tile
+            const int qb = n % kQBufs;
+            const uint32_t qph = (uint32_t)(n / kQBufs) & 1u;
+            if (!mbar_wait_warp(smem_u32(&q_free_bar[qb]), qph ^ 1u, abort_flag)) { ok = false; break; }
+            if (elect_one()) {
                 mbar_arrive_expect_tx(smem_u32(&q_bar[qb]), kQBytes);
 #pragma unroll
                 for (int kb = 0; kb < KB; ++kb)
                     tma_load_2d(q_addr + qb * kQBytes + kb * kQBlk, tmQ, kb * 64, item.g * dm.R + item.row * kStBM, smem_u32(&q_bar[qb]));
-                for (int t = item.t_lo; t < item.t_lo + item.nt; ++t, ++it) {
-                    const int s = it % kStStages;
-                    const uint32_t ph = (uint32_t)(it / kStStages) & 1u;
-                    if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
-                    const uint32_t fb = smem_u32(&full_bar[s]);
-                    mbar_arrive_expect_tx(fb, kKBytes);
-                    if (dbg_withhold(status, kDbgAttnStats) && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && it == 0) continue;   // debug builds: one copy never sent
-#pragma unroll
-                    for (int kb = 0; kb < KB; ++kb)
-                        tma_load_2d(k_addr(s) + kb * kKBlk, tmK, kb * 64, item.g * dm.S + t * kStBN, fb);
-                }
             }
-            // every copy issued has landed before the CTA's shared memory goes away, whichever way the
-            // other warps leave (in a normal run these waits are over already)
-            for (int j = n > kQBufs ? n - kQBufs : 0; j < n; ++j)
-                mbar_wait(smem_u32(&q_bar[j % kQBufs]), (uint32_t)(j / kQBufs) & 1u, abort_flag);
-            for (int back = 1; back <= kStStages && back <= it; ++back) {
-                const int j = it - back;
-                mbar_wait(smem_u32(&full_bar[j % kStStages]), (uint32_t)(j / kStStages) & 1u, abort_flag);
+            __syncwarp();
+            for (int t = item.t_lo; t < item.t_lo + item.nt; ++t, ++it) {
+                const int s = it % kStStages;
+                const uint32_t ph = (uint32_t)(it / kStStages) & 1u;
+                if (!mbar_wait_warp(smem_u32(&empty_bar[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
+                const uint32_t fb = smem_u32(&full_bar[s]);
+                const bool held = dbg_withhold(status, kDbgAttnStats) && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && it == 0;   // debug builds: one copy never sent
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(fb, kKBytes);
+                    if (!held) {
+#pragma unroll
+                        for (int kb = 0; kb < KB; ++kb)
+                            tma_load_2d(k_addr(s) + kb * kKBlk, tmK, kb * 64, item.g * dm.S + t * kStBN, fb);
+                    }
+                }
+                __syncwarp();
             }
         }
+        // every copy issued has landed before the CTA's shared memory goes away, whichever way the
+        // other warps leave (in a normal run these waits are over already)
+        for (int j = n > kQBufs ? n - kQBufs : 0; j < n; ++j)
+            mbar_wait_warp(smem_u32(&q_bar[j % kQBufs]), (uint32_t)(j / kQBufs) & 1u, abort_flag);
+        for (int back = 1; back <= kStStages && back <= it; ++back) {
+            const int j = it - back;
+            mbar_wait_warp(smem_u32(&full_bar[j % kStStages]), (uint32_t)(j / kStStages) & 1u, abort_flag);
+        }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = make_idesc_bf16(kStBM, kStBN);
-            bool ok = true;
-            int it = 0;
-            for (int n = 0; ok && stats_item(ab, n, item); ++n) {
-                const int qb = n % kQBufs;
-                ok = mbar_wait(smem_u32(&q_bar[qb]), (uint32_t)(n / kQBufs) & 1u, abort_flag);
-                for (const int end = it + item.nt; it < end && ok; ++it) {
-                    const int b = it & 1, s = it % kStStages;
-                    if (!mbar_wait(smem_u32(&tempty_bar[b]), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-                    if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(it / kStStages) & 1u, abort_flag)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + (uint32_t)b * kStBN;
+        constexpr uint32_t idesc = make_idesc_bf16(kStBM, kStBN);
+        bool ok = true;
+        int it = 0;
+        for (int n = 0; ok && stats_item(ab, n, item); ++n) {
+            const int qb = n % kQBufs;
+            ok = mbar_wait_warp(smem_u32(&q_bar[qb]), (uint32_t)(n / kQBufs) & 1u, abort_flag);
+            for (const int end = it + item.nt; it < end && ok; ++it) {
+                const int b = it & 1, s = it % kStStages;
+                if (!mbar_wait_warp(smem_u32(&tempty_bar[b]), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+                if (!mbar_wait_warp(smem_u32(&full_bar[s]), (uint32_t)(it / kStStages) & 1u, abort_flag)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t d_tmem = tmem + (uint32_t)b * kStBN;
+                if (elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < DH / 16; ++kk) {
                         const uint64_t ad = make_desc_k128(q_addr + qb * kQBytes + (kk >> 2) * kQBlk + (kk & 3) * 32);
@@ -300,12 +312,15 @@ attn_stats_mma_kernel(const __grid_constant__ AttnBatch<NL> ab, int32_t* __restr
                     umma_commit(smem_u32(&empty_bar[s]));
                     umma_commit(smem_u32(&tfull_bar[b]));
                 }
-                if (ok) umma_commit(smem_u32(&q_free_bar[qb]));
+                __syncwarp();
             }
-            if (!ok) {                                         // wait until whatever was issued has retired
-                umma_commit(smem_u32(&drain_bar));
-                mbar_wait(smem_u32(&drain_bar), 0u, abort_flag);
-            }
+            if (ok && elect_one()) umma_commit(smem_u32(&q_free_bar[qb]));
+            __syncwarp();
+        }
+        if (!ok) {                                         // wait until whatever was issued has retired
+            if (elect_one()) umma_commit(smem_u32(&drain_bar));
+            __syncwarp();
+            mbar_wait_warp(smem_u32(&drain_bar), 0u, abort_flag);
         }
     } else {
         const int quad = warp & 3;                             // TMEM lanes 32*quad .. 32*quad+31
@@ -438,7 +453,7 @@ attn_colsum_mma_kernel(const __grid_constant__ AttnBatch<NL> ab, int32_t* __rest
     const uint32_t kQBlk = (uint32_t)NQ * 128;
     const uint32_t kQBytes = KB * kQBlk;
     const int stages = NL > 1 ? cs_stages(NQ, DH) : kCsStages;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     const uint32_t q_addr = smem_base;
@@ -465,6 +480,7 @@ attn_colsum_mma_kernel(const __grid_constant__ AttnBatch<NL> ab, int32_t* __rest
     tc_fence_after();
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
 
     AttnItem item = {};
     int at = 0, at_end = 1;
@@ -473,54 +489,62 @@ attn_colsum_mma_kernel(const __grid_constant__ AttnBatch<NL> ab, int32_t* __rest
         at_end = (int)((long long)ab.first[NL] * (blockIdx.x + 1) / gridDim.x);
     }
     if (warp == 0) {
-        if (lane == 0) {
 #pragma unroll
-            for (int l = 0; l < NL; ++l) { prefetch_tmap(&ab.q[l]); prefetch_tmap(&ab.k[l]); }
-            int it = 0, n = 0;                                 // as in the stats kernel
-            bool ok = true;
-            for (; ok && colsum_item(ab, at, at_end, item); ++n) {
-                const AttnMmaDims& dm = ab.lv[item.level].dm;
-                const CUtensorMap *tmQ = &ab.q[item.level], *tmK = &ab.k[item.level];
-                const int qb = n % kQBufs;
-                const uint32_t qph = (uint32_t)(n / kQBufs) & 1u;
-                if (!mbar_wait(smem_u32(&q_free_bar[qb]), qph ^ 1u, abort_flag)) { ok = false; break; }
+        for (int l = 0; l < NL; ++l)
+            if (elect_one()) { prefetch_tmap(&ab.q[l]); prefetch_tmap(&ab.k[l]); }
+        __syncwarp();
+        int it = 0, n = 0;                                 // as in the stats kernel
+        bool ok = true;
+        for (; ok && colsum_item(ab, at, at_end, item); ++n) {
+            const AttnMmaDims& dm = ab.lv[item.level].dm;
+            const CUtensorMap *tmQ = &ab.q[item.level], *tmK = &ab.k[item.level];
+            const int qb = n % kQBufs;
+            const uint32_t qph = (uint32_t)(n / kQBufs) & 1u;
+            if (!mbar_wait_warp(smem_u32(&q_free_bar[qb]), qph ^ 1u, abort_flag)) { ok = false; break; }
+            if (elect_one()) {
                 mbar_arrive_expect_tx(smem_u32(&q_bar[qb]), kQBytes);
 #pragma unroll
                 for (int kb = 0; kb < KB; ++kb)
                     tma_load_2d(q_addr + qb * kQBytes + kb * kQBlk, tmQ, kb * 64, item.g * dm.R + item.row * NQ, smem_u32(&q_bar[qb]));
-                for (int t = item.t_lo; t < item.t_lo + item.nt; ++t, ++it) {
-                    const int s = it % stages;
-                    const uint32_t ph = (uint32_t)(it / stages) & 1u;
-                    if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
-                    const uint32_t fb = smem_u32(&full_bar[s]);
-                    mbar_arrive_expect_tx(fb, kKBytes);
-                    if (dbg_withhold(status, kDbgAttnColsum) && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && it == 0) continue;   // debug builds: one copy never sent
-#pragma unroll
-                    for (int kb = 0; kb < KB; ++kb)
-                        tma_load_2d(k_addr(s) + kb * kKBlk, tmK, kb * 64, item.g * dm.S + t * kCsBM, fb);
-                }
             }
-            for (int j = n > kQBufs ? n - kQBufs : 0; j < n; ++j)
-                mbar_wait(smem_u32(&q_bar[j % kQBufs]), (uint32_t)(j / kQBufs) & 1u, abort_flag);
-            for (int back = 1; back <= stages && back <= it; ++back) {
-                const int j = it - back;
-                mbar_wait(smem_u32(&full_bar[j % stages]), (uint32_t)(j / stages) & 1u, abort_flag);
+            __syncwarp();
+            for (int t = item.t_lo; t < item.t_lo + item.nt; ++t, ++it) {
+                const int s = it % stages;
+                const uint32_t ph = (uint32_t)(it / stages) & 1u;
+                if (!mbar_wait_warp(smem_u32(&empty_bar[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
+                const uint32_t fb = smem_u32(&full_bar[s]);
+                const bool held = dbg_withhold(status, kDbgAttnColsum) && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && it == 0;   // debug builds: one copy never sent
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(fb, kKBytes);
+                    if (!held) {
+#pragma unroll
+                        for (int kb = 0; kb < KB; ++kb)
+                            tma_load_2d(k_addr(s) + kb * kKBlk, tmK, kb * 64, item.g * dm.S + t * kCsBM, fb);
+                    }
+                }
+                __syncwarp();
             }
         }
+        for (int j = n > kQBufs ? n - kQBufs : 0; j < n; ++j)
+            mbar_wait_warp(smem_u32(&q_bar[j % kQBufs]), (uint32_t)(j / kQBufs) & 1u, abort_flag);
+        for (int back = 1; back <= stages && back <= it; ++back) {
+            const int j = it - back;
+            mbar_wait_warp(smem_u32(&full_bar[j % stages]), (uint32_t)(j / stages) & 1u, abort_flag);
+        }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_bf16(kCsBM, NQ);
-            bool ok = true;
-            int it = 0;
-            for (int n = 0; ok && colsum_item(ab, at, at_end, item); ++n) {
-                const int qb = n % kQBufs;
-                ok = mbar_wait(smem_u32(&q_bar[qb]), (uint32_t)(n / kQBufs) & 1u, abort_flag);
-                for (const int end = it + item.nt; it < end && ok; ++it) {
-                    const int b = it & 1, s = it % stages;
-                    if (!mbar_wait(smem_u32(&tempty_bar[b]), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-                    if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(it / stages) & 1u, abort_flag)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + (uint32_t)b * kCsMaxNQ;
+        const uint32_t idesc = make_idesc_bf16(kCsBM, NQ);
+        bool ok = true;
+        int it = 0;
+        for (int n = 0; ok && colsum_item(ab, at, at_end, item); ++n) {
+            const int qb = n % kQBufs;
+            ok = mbar_wait_warp(smem_u32(&q_bar[qb]), (uint32_t)(n / kQBufs) & 1u, abort_flag);
+            for (const int end = it + item.nt; it < end && ok; ++it) {
+                const int b = it & 1, s = it % stages;
+                if (!mbar_wait_warp(smem_u32(&tempty_bar[b]), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+                if (!mbar_wait_warp(smem_u32(&full_bar[s]), (uint32_t)(it / stages) & 1u, abort_flag)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t d_tmem = tmem + (uint32_t)b * kCsMaxNQ;
+                if (elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < DH / 16; ++kk) {
                         const uint64_t ad = make_desc_k128(k_addr(s) + (kk >> 2) * kKBlk + (kk & 3) * 32);
@@ -530,12 +554,15 @@ attn_colsum_mma_kernel(const __grid_constant__ AttnBatch<NL> ab, int32_t* __rest
                     umma_commit(smem_u32(&empty_bar[s]));
                     umma_commit(smem_u32(&tfull_bar[b]));
                 }
-                if (ok) umma_commit(smem_u32(&q_free_bar[qb]));
+                __syncwarp();
             }
-            if (!ok) {
-                umma_commit(smem_u32(&drain_bar));
-                mbar_wait(smem_u32(&drain_bar), 0u, abort_flag);
-            }
+            if (ok && elect_one()) umma_commit(smem_u32(&q_free_bar[qb]));
+            __syncwarp();
+        }
+        if (!ok) {
+            if (elect_one()) umma_commit(smem_u32(&drain_bar));
+            __syncwarp();
+            mbar_wait_warp(smem_u32(&drain_bar), 0u, abort_flag);
         }
     } else {
         // The epilogue warps first turn the key-split partials into the log-sum-exp of the chunk's

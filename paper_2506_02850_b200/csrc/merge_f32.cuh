@@ -217,7 +217,7 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
     const int ksteps = f3_steps(d), segment = f3_segment(d), nseg = (ksteps + segment - 1) / segment;
     const uint32_t stage_bytes = kF3ABytes + (uint32_t)bn * kF3RowBytes;
     const int stages = min(kF3MaxStages, (int)(kF3RingBytes / stage_bytes));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
@@ -239,49 +239,53 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
     const uint32_t tmem_base = s_tmem_base;                   // columns 0 ..: the sums of hh, 256 ..: the others'
     volatile int* abort_flag = &s_abort;
 
+    // The loops of these two warps: the whole warp takes every step and one elected thread issues, so that stage, addresses and
+    // descriptors stay in uniform registers (see merge_assign_mma_kernel; 61 x 169 tokens of 1156: 140.0 -> 136.5 us the whole path).
+    const int units = __shfl_sync(0xFFFFFFFFu, total_units, 0);
     if (warp == kF3EpiWarps) {
-        if (lane == 0) {
-            int s = 0, issued = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
-                const F3Unit un = f3_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, bn);
-                const uint32_t b_bytes = (uint32_t)((un.cols + 15) & ~15) * kF3RowBytes;
-                const uint8_t* a = pl.a + (size_t)un.tile * kF3ABytes * ksteps;
-                const uint8_t* b = pl.b + (size_t)un.group * 16 * kF3RowBytes * ksteps;
-                for (int ks = 0; ks < ksteps; ++ks, a += kF3ABytes, b += b_bytes) {
-                    if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
-                    const uint32_t fb = smem_u32(&full_bar[s]), dst = smem_base + (uint32_t)s * stage_bytes;
+        int s = 0, issued = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+            const F3Unit un = f3_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, bn);
+            const uint32_t b_bytes = (uint32_t)((un.cols + 15) & ~15) * kF3RowBytes;
+            const uint8_t* a = pl.a + (size_t)un.tile * kF3ABytes * ksteps;
+            const uint8_t* b = pl.b + (size_t)un.group * 16 * kF3RowBytes * ksteps;
+            for (int ks = 0; ks < ksteps; ++ks, a += kF3ABytes, b += b_bytes) {
+                if (!mbar_wait_warp(smem_u32(&empty_bar[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
+                const uint32_t fb = smem_u32(&full_bar[s]), dst = smem_base + (uint32_t)s * stage_bytes;
+                if (elect_one()) {
                     mbar_arrive_expect_tx(fb, kF3ABytes + b_bytes);
                     bulk_load(dst, a, kF3ABytes, fb);
                     if (!(dbg_withhold(status, kDbgMergeAssign) && blockIdx.x == 0 && issued == 0))   // debug builds: one copy never sent
                         bulk_load(dst + kF3ABytes, b, b_bytes, fb);
-                    ++issued;
-                    if (++s == stages) { s = 0; ph ^= 1u; }
                 }
-            }
-            // every copy has landed before the CTA's shared memory goes away
-            for (int back = 1; back <= stages && back <= issued; ++back) {
-                const int j = issued - back;
-                mbar_wait(smem_u32(&full_bar[j % stages]), (uint32_t)(j / stages) & 1u, abort_flag);
+                __syncwarp();
+                ++issued;
+                if (++s == stages) { s = 0; ph ^= 1u; }
             }
         }
+        // every copy has landed before the CTA's shared memory goes away
+        for (int back = 1; back <= stages && back <= issued; ++back) {
+            const int j = issued - back;
+            mbar_wait_warp(smem_u32(&full_bar[j % stages]), (uint32_t)(j / stages) & 1u, abort_flag);
+        }
     } else if (warp == kF3EpiWarps + 1) {
-        if (lane == 0) {
-            int s = 0, n = 0, seg = 0;                        // stage; units and segments so far
-            uint32_t ph = 0;
-            bool ok = true;
-            const uint32_t d_hh = tmem_base, d_small = tmem_base + kF3BN;
-            for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x, ++n) {
-                const F3Unit un = f3_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, bn);
-                const uint32_t cols = (uint32_t)(un.cols + 15) & ~15u, idesc = make_idesc_bf16(kF3BM, (int)cols);
-                constexpr uint32_t kA = kF3BM * 64;           // a plane of the tokens, and of the keys
-                const uint32_t kB = cols * 64;
-                for (int ks = 0; ks < ksteps; ++ks) {
-                    if (!mbar_wait(smem_u32(&full_bar[s]), ph, abort_flag)) { ok = false; break; }
-                    if (ks == 0 && !mbar_wait(smem_u32(&sempty_bar), ((uint32_t)n & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t a = smem_base + (uint32_t)s * stage_bytes, b = a + kF3ABytes;
+        int s = 0, n = 0, seg = 0;                            // stage; units and segments so far
+        uint32_t ph = 0;
+        bool ok = true;
+        const uint32_t d_hh = __shfl_sync(0xFFFFFFFFu, tmem_base, 0), d_small = d_hh + kF3BN;
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++n) {
+            const F3Unit un = f3_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, bn);
+            const uint32_t cols = __shfl_sync(0xFFFFFFFFu, (uint32_t)(un.cols + 15) & ~15u, 0), idesc = make_idesc_bf16(kF3BM, (int)cols);
+            constexpr uint32_t kA = kF3BM * 64;               // a plane of the tokens, and of the keys
+            const uint32_t kB = cols * 64;
+            for (int ks = 0; ks < ksteps; ++ks) {
+                if (!mbar_wait_warp(smem_u32(&full_bar[s]), ph, abort_flag)) { ok = false; break; }
+                if (ks == 0 && !mbar_wait_warp(smem_u32(&sempty_bar), ((uint32_t)n & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t a = smem_base + (uint32_t)s * stage_bytes, b = a + kF3ABytes;
+                if (elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < kF3BK / 16; ++kk) {
                         const uint32_t ah = a + 32u * kk, bh = b + 32u * kk;
@@ -291,26 +295,31 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
                         umma_bf16_k64(d_small, ah, bh + kB, idesc, 1u);
                         umma_bf16_k64(d_small, ah + kA, bh, idesc, 1u);
                     }
-                    const bool opens = (ks & (segment - 1)) == 0;
-                    if (opens) {
-                        if (!mbar_wait(smem_u32(&hempty_bar), ((uint32_t)seg & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-                        tc_fence_after();
-                    }
+                }
+                __syncwarp();
+                const bool opens = (ks & (segment - 1)) == 0;
+                if (opens) {
+                    if (!mbar_wait_warp(smem_u32(&hempty_bar), ((uint32_t)seg & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+                    tc_fence_after();
+                }
+                const bool closes = (ks & (segment - 1)) == segment - 1 || ks == ksteps - 1;
+                if (elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < kF3BK / 16; ++kk) umma_bf16_k64(d_hh, a + 32u * kk, b + 32u * kk, idesc, !opens || kk > 0 ? 1u : 0u);
                     umma_commit(smem_u32(&empty_bar[s]));
-                    if (++s == stages) { s = 0; ph ^= 1u; }
-                    if ((ks & (segment - 1)) == segment - 1 || ks == ksteps - 1) {
-                        umma_commit(smem_u32(&hfull_bar));
-                        ++seg;
-                    }
+                    if (closes) umma_commit(smem_u32(&hfull_bar));
                 }
-                if (ok) umma_commit(smem_u32(&sfull_bar));
+                __syncwarp();
+                if (++s == stages) { s = 0; ph ^= 1u; }
+                if (closes) ++seg;
             }
-            if (!ok) {                                        // wait until whatever was issued has retired
-                umma_commit(smem_u32(&drain_bar));
-                mbar_wait(smem_u32(&drain_bar), 0u, abort_flag);
-            }
+            if (ok && elect_one()) umma_commit(smem_u32(&sfull_bar));
+            __syncwarp();
+        }
+        if (!ok) {                                            // wait until whatever was issued has retired
+            if (elect_one()) umma_commit(smem_u32(&drain_bar));
+            __syncwarp();
+            mbar_wait_warp(smem_u32(&drain_bar), 0u, abort_flag);
         }
     } else {
         const int quad = warp & 3, part = warp >> 2;          // TMEM lanes 32 * quad ..., columns 64 * part ...
