@@ -6,10 +6,9 @@
 //
 // Fast path.  A source row at or beyond n is never written by anybody, so it can be
 // read at any time.  Only the first h rows of the list, h = #{i : keep[i] < n}, have
-// their source inside the destination region.  Those h rows are first copied to a
-// staging area in the workspace (one kernel), then every row is written from its
-// source or from the staging area (a second kernel) -- no ordering inside either
-// kernel, any number of CTAs per slab.  With a keep ratio r about r*n rows are staged.
+// their source inside the destination region.  Those h rows are read, into registers or a
+// staging area in the workspace, by the CTAs of the slab's cluster before a cluster barrier behind
+// which every row is written.  With a keep ratio r about r*n rows are concerned.
 //
 // General path (h larger than the staging area: lists that keep most rows).  Rows are
 // moved in rounds of consecutive destination rows; a round's sources all lie at or
@@ -20,6 +19,8 @@
 // One thread-block cluster owns one (layer, K|V, head) slab; the read->write
 // ordering inside a round is a hardware cluster barrier (no spinning on memory).
 #include <cooperative_groups.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "launchers.h"
@@ -128,8 +129,8 @@ kv_check_lists_kernel(int S_cur, const int32_t* __restrict__ keep_idx, const int
 // ---- fast path ------------------------------------------------------------------
 constexpr int kKvFastThreads = 256;
 constexpr int kKvFastUnroll = 8;          // 16-byte chunks in flight per thread
-constexpr int kKvStageSplit = 2;          // CTAs per slab in the staging kernel
-constexpr int kKvCopySplit = 4;           // CTAs per slab in the copy kernel
+constexpr int kKvCtasPerSm = 4;           // (64 registers)
+constexpr int kKvMaxSplit = 8;            // most CTAs per slab, a cluster
 constexpr size_t kKvStageBudget = (size_t)128 << 20;   // bytes of workspace the staging area may take
 
 // First index of the ascending list keep[0..n) whose value is >= n; whole warp, 32-ary search.
@@ -158,13 +159,20 @@ __device__ __forceinline__ SlabId slab_of(int slab, int Hkv) {
     return s;
 }
 
-// Copies the rows whose source lies inside the destination region to the staging area and
-// records h per layer (-1: too many for the staging area, the general path takes the layer).
-__global__ void __launch_bounds__(kKvFastThreads)
-kv_stage_kernel(KvPtrs ptrs, int layer0, int Hkv, int S_cap, int S_cur, int row_chunks,
-                const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ keep_len, int stage_rows,
-                int32_t* __restrict__ haz, uint4* __restrict__ stage, const int32_t* __restrict__ valid,
-                int n_layers, int32_t* __restrict__ status) {
+// A cluster per slab moves the slab's rows; its CTAs take runs of 2048 pieces of 16 bytes in turn.  Rows whose
+// source lies at or beyond the new length (all but the first h) are never written before they are read.  The others are
+// read by everybody before anybody writes: those of a CTA's first run into registers, later ones into the staging area,
+// which the same thread reads again; then a cluster barrier, behind which the first run's loads of all rows land.
+// Records h per layer (-1: too many for the staging area, the general path takes the layer).
+// What bounds it is HBM, with scattered rows of 256 bytes.  Staging and copying as two kernels, the copy with four CTAs
+// per slab in one and a half waves, took (call, cold, us) for 28 layers x 4 heads of 18 432 + 64 rows, 6.5 / 15 / 30 / 50 %
+// kept: 52.2 / 98.3 / 196.6 / 469.0, this 46.0 / 87.0 / 185.3 / 472.1; 40 layers x 40 heads of 2751 rows 108.5 and 85.0, one
+// layer of one head of 63 606 rows 148.4 and 70.6.
+__global__ void __launch_bounds__(kKvFastThreads, kKvCtasPerSm)
+kv_move_kernel(KvPtrs ptrs, int layer0, int Hkv, int S_cap, int S_cur, int row_chunks,
+               const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ keep_len, int stage_rows,
+               int32_t* __restrict__ haz, uint4* stage, const int32_t* __restrict__ valid,
+               int n_layers, int32_t* __restrict__ status) {
     grid_dep_wait();
     __shared__ int s_h;
     const SlabId id = slab_of(blockIdx.y, Hkv);
@@ -178,69 +186,67 @@ kv_stage_kernel(KvPtrs ptrs, int layer0, int Hkv, int S_cap, int S_cur, int row_
                 if (!valid[l]) st = METOK_ERR_INVALID_ARG;
         *status = st;
     }
-    if (valid && !valid[layer]) {                          // nothing is indexed through a rejected list
+    if (valid && !valid[layer]) {                          // nothing is indexed through a rejected list (uniform per cluster)
         if (lead) haz[layer] = -2;
         return;
     }
     const int32_t* keep = keep_idx + (size_t)layer * S_cur;
     const int n = keep_len[layer];
-    if (threadIdx.x < 32) {
-        const int h = (n > 0 && n < S_cur) ? warp_lower_bound(keep, n, threadIdx.x) : 0;
-        if (threadIdx.x == 0) s_h = h;
+    if (n <= 0 || n >= S_cur) {                            // nothing to keep, or nothing dropped
+        if (lead) haz[layer] = 0;
+        return;
     }
-    __syncthreads();
-    const int h = s_h;
-    const bool fast = h <= stage_rows;
-    if (lead) haz[layer] = fast ? h : -1;
-    if (!fast || h == 0) return;
-    const uint4* base = reinterpret_cast<const uint4*>(id.which ? ptrs.v[id.ll] : ptrs.k[id.ll]) +
-                        (size_t)id.head * S_cap * row_chunks;
-    uint4* dst = stage + ((size_t)(layer * 2 + id.which) * Hkv + id.head) * (size_t)stage_rows * row_chunks;
-    const int total = h * row_chunks;
-    for (int gc = blockIdx.x * kKvFastThreads + threadIdx.x; gc < total; gc += kKvStageSplit * kKvFastThreads) {
-        const int i = gc / row_chunks, c = gc - i * row_chunks;
-        const int src = keep[i];
-        if (src != i) dst[gc] = base[(size_t)src * row_chunks + c];
-    }
-}
-
-// Every kept row from its source (at or beyond the new length: never written) or from the
-// staging area.
-__global__ void __launch_bounds__(kKvFastThreads)
-kv_copy_kernel(KvPtrs ptrs, int layer0, int Hkv, int S_cap, int S_cur, int row_chunks,
-               const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ keep_len, int stage_rows,
-               const int32_t* __restrict__ haz, const uint4* __restrict__ stage) {
-    grid_dep_wait();
-    const SlabId id = slab_of(blockIdx.y, Hkv);
-    const int layer = layer0 + id.ll;
-    const int h = haz[layer];
-    const int n = keep_len[layer];
-    if (h < 0 || n >= S_cur) return;
-    const int32_t* keep = keep_idx + (size_t)layer * S_cur;
     uint4* base = reinterpret_cast<uint4*>(id.which ? ptrs.v[id.ll] : ptrs.k[id.ll]) +
                   (size_t)id.head * S_cap * row_chunks;
-    const uint4* stg = stage + ((size_t)(layer * 2 + id.which) * Hkv + id.head) * (size_t)stage_rows * row_chunks;
+    uint4* stg = stage + ((size_t)(layer * 2 + id.which) * Hkv + id.head) * (size_t)stage_rows * row_chunks;
     const int total = n * row_chunks;
     constexpr int kStep = kKvFastThreads * kKvFastUnroll;
-    for (int g0 = blockIdx.x * kStep; g0 < total; g0 += kKvCopySplit * kStep) {
-        uint4 v[kKvFastUnroll];
-        int at[kKvFastUnroll];                            // destination chunk, -1: nothing to store
+    uint4 v[kKvFastUnroll];
+    unsigned some = 0;                                     // which of them there are to store
+    auto load = [&](int g0, int h) {
+        some = 0;
 #pragma unroll
         for (int u = 0; u < kKvFastUnroll; ++u) {
             const int gc = g0 + u * kKvFastThreads + threadIdx.x;
-            at[u] = -1;
             if (gc < total) {
                 const int i = gc / row_chunks, c = gc - i * row_chunks;
                 const int src = keep[i];
                 if (src != i) {
                     v[u] = i < h ? stg[gc] : base[(size_t)src * row_chunks + c];
-                    at[u] = gc;
+                    some |= 1u << u;
                 }
             }
         }
+    };
+    const int g_first = blockIdx.x * kStep, stride = gridDim.x * kStep;
+    load(g_first, 0);                                      // all from their sources
+    if (threadIdx.x < 32) {
+        const int h = warp_lower_bound(keep, n, threadIdx.x);
+        if (threadIdx.x == 0) s_h = h;
+    }
+    __syncthreads();
+    const int h = s_h;
+    if (lead) haz[layer] = h <= stage_rows ? h : -1;
+    if (h > stage_rows) return;                            // uniform per cluster
+    for (int gc = g_first + stride + (int)threadIdx.x, u = 0; gc < h * row_chunks;) {
+        const int i = gc / row_chunks, c = gc - i * row_chunks, src = keep[i];
+        if (src != i) stg[gc] = base[(size_t)src * row_chunks + c];
+        if (++u < kKvFastUnroll) {
+            gc += kKvFastThreads;
+        } else {
+            u = 0;
+            gc += stride - (kKvFastUnroll - 1) * kKvFastThreads;
+        }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    for (int g0 = g_first;;) {
 #pragma unroll
         for (int u = 0; u < kKvFastUnroll; ++u)
-            if (at[u] >= 0) base[at[u]] = v[u];
+            if (some >> u & 1u) base[g0 + u * kKvFastThreads + threadIdx.x] = v[u];
+        g0 += stride;
+        if (g0 >= total) break;
+        load(g0, h);
     }
 }
 
@@ -426,17 +432,16 @@ extern "C" int metok_kv_compact(void* const* k_layers, void* const* v_layers, in
         const int nl = (L - l0) < kKvMaxLayersPerLaunch ? (L - l0) : kKvMaxLayersPerLaunch;
         const KvPtrs ptrs = kv_ptrs(k_layers, v_layers, l0, nl);
         const int slabs = nl * 2 * Hkv;
+        // a cluster of as many CTAs per slab as keep all of them resident at once: two waves cost more than fewer loads in
+        // flight (224 slabs with clusters of four: 58.4 us instead of 46.0), and clusters that are no power of two leave SMs
+        // unused (192 slabs with clusters of three: 50.2 us instead of 44.6)
+        int split = 1;
+        while (2 * split <= kKvMaxSplit && 2 * split * slabs <= kNumSMs * kKvCtasPerSm) split *= 2;
         {
-            METOK_TIMED("kv_stage_kernel", st);
-            launch_chained(kv_stage_kernel, dim3(dim3(kKvStageSplit, slabs)), dim3(kKvFastThreads), 0, st, 
+            METOK_TIMED("kv_move_kernel", st);
+            launch_chained_clusters(split, kv_move_kernel, dim3(split, slabs), dim3(kKvFastThreads), 0, st,
                 ptrs, l0, Hkv, S_cap, S_cur, row_chunks, keep_idx, keep_len, w.stage_rows, w.haz, w.stage, valid, L,
                 w.status);
-        }
-        METOK_LAUNCH_CHECK();
-        {
-            METOK_TIMED("kv_copy_kernel", st);
-            launch_chained(kv_copy_kernel, dim3(dim3(kKvCopySplit, slabs)), dim3(kKvFastThreads), 0, st, 
-                ptrs, l0, Hkv, S_cap, S_cur, row_chunks, keep_idx, keep_len, w.stage_rows, w.haz, w.stage);
         }
         METOK_LAUNCH_CHECK();
         // h <= list length: when every list is known to fit the staging area, no layer takes the general path

@@ -56,6 +56,37 @@ def test_kv_paper_rule_in_place(L, S_vis, vis_start, tail, l1, dh, dtype):
             assert torch.equal(x[:, :n], o[:, idx])
 
 
+@pytest.mark.parametrize("L,Hkv", [(1, 1), (10, 4), (10, 8), (38, 4)])             # clusters of 8, 4, 2 and 1 CTAs
+@pytest.mark.parametrize("S", [1, 129, 1100, 3000])                                # in registers, staged, and beyond the staging area
+@pytest.mark.parametrize("lists", ["dense", "some", "front", "back", "one", "all"])
+def test_kv_rows_given_move_in_place(L, Hkv, S, lists):
+    g = torch.Generator().manual_seed(S + L)
+    dh, cap = 128, S + 3
+    cache = torch.randint(-2 ** 15, 2 ** 15, (L, 2, Hkv, cap, dh), generator=g, dtype=torch.int16).cuda()
+    keep = torch.zeros((L, S), dtype=torch.int32)
+    lens = torch.zeros(L, dtype=torch.int32)
+    for l in range(L):
+        draw = torch.rand(S, generator=g)
+        mask = {"dense": draw < 0.9, "some": draw < 0.1, "front": torch.arange(S) < (S + 1) // 2, "back": torch.arange(S) >= S // 2,
+                "one": torch.arange(S) == S - 1, "all": draw < 2}[lists]
+        rows = mask.nonzero().flatten().to(torch.int32)
+        keep[l, :len(rows)] = rows
+        lens[l] = len(rows)
+    want = cache.clone()
+    for l in range(L):
+        n = int(lens[l])
+        want[l, :, :, :n] = cache[l][:, :, keep[l, :n].long().cuda()]
+    kv = cache.view(torch.bfloat16)
+    r = B.metok_kv_compact([kv[l, 0] for l in range(L)], [kv[l, 1] for l in range(L)], S, B.KV_GIVEN, 0, 0,
+                           keep_idx=keep.cuda(), keep_len=lens.cuda())
+    torch.cuda.synchronize()
+    assert torch.equal(r["new_len"].cpu(), lens)
+    for l in range(L):
+        n = int(lens[l])
+        assert torch.equal(cache[l, :, :, :n], want[l, :, :, :n])
+        assert torch.equal(cache[l, :, :, S:], want[l, :, :, S:])                  # rows beyond the cache's length are not touched
+
+
 @pytest.mark.parametrize("count", [15, 16, 17, 18, 127, 128, 129, 130, 300, 700])
 @pytest.mark.parametrize("d,dtype", [(8, torch.bfloat16), (520, torch.bfloat16), (1032, torch.bfloat16), (260, torch.float32)])
 def test_averages_of_chosen_member_counts(count, d, dtype):
