@@ -377,7 +377,7 @@ static int launch_segment(const void* feats, int Tn, int N, int d, int k, int si
         METOK_LAUNCH_CHECK();
     }
     const size_t smem = (size_t)((Tn + 3) & ~3) * 3 * sizeof(float);
-    if (smem > 48 * 1024)                                  // more than 256 frames, then: a cluster
+    if (smem > 32 * 1024)                                  // with the kernel's own 8.3 KB; more than 256 frames, so a cluster
         METOK_ALLOW_SMEM(seg_finish_kernel<true>, smem);
     {
         METOK_TIMED("seg_finish_kernel", st);
@@ -783,8 +783,8 @@ static int launch_seg_score(const void* feats, const void* text, int Tn, int N, 
     }
     METOK_LAUNCH_CHECK();
     const size_t smem = (size_t)((Tn + 3) & ~3) * 3 * sizeof(float);
-    if (smem > 48 * 1024)
-        METOK_ALLOW_SMEM(seg_finish_kernel<true>, smem);       // more than 256 frames, then: a cluster
+    if (smem > 32 * 1024)                                  // with the kernel's own 8.3 KB; more than 256 frames, so a cluster
+        METOK_ALLOW_SMEM(seg_finish_kernel<true>, smem);
     {
         METOK_TIMED("seg_finish_kernel", st);
         launch_chained_clusters(finish_ctas(Tn), finish_ctas(Tn) > 1 ? seg_finish_kernel<true> : seg_finish_kernel<false>, dim3(finish_ctas(Tn)), dim3(1024), smem, st, part_dot, part_nrm, nslab, Tn, k, sims, boundaries, event_offsets,

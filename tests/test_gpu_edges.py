@@ -32,6 +32,20 @@ def test_segmentation_finish_and_event_plan_at_their_edges(T):
         R.pool_case(V, t, offs, "f32", 0.5, 0.4, (2, 3, 1, 5))
 
 
+@pytest.mark.parametrize("T", [3400, 3404, 3405, 4096, 4097, 8192])    # 12 bytes a frame and the kernel's own 8.3 KB against 48 KB
+def test_segmentation_finish_around_48_kb_of_shared_memory(T):
+    rng = np.random.default_rng(T)
+    V = rng.standard_normal((T, 1, 8)).astype(np.float32)
+    V += V[:1]
+    R.segment_case(V, "f32", T // 7)
+    feats = torch.from_numpy(V).cuda().bfloat16()
+    got = B.metok_segment_score_events(feats, T // 7, feats[0, 0].clone())
+    want = B.metok_segment_events(feats, T // 7)
+    torch.cuda.synchronize()
+    assert len(torch.unique(got["boundaries"][:T // 7 - 1])) == T // 7 - 1
+    assert torch.allclose(got["sims"][:T - 1], want["sims"][:T - 1], rtol=0, atol=1e-5)
+
+
 @pytest.mark.parametrize("L,S_vis,vis_start,tail,l1", [
     (3, 40, 0, 0, 1), (3, 40, 5, 40, 0), (3, 40, 5, 41, 0), (3, 40, 0, 39, 3), (70, 33, 3, 7, 65), (2, 0, 4, 9, 0), (2, 600, 1, 260, 1),
 ])
