@@ -1589,12 +1589,18 @@ static int choose_f3(int Nv, int k, int d, int cap, double keep) {
 
 static bool ratio_ok(double r) { return r > 0.0 && r <= 1.0; }
 
+static size_t vision_ws_bytes(int Tn, int N, int k, int d, int cap, bool merging, bool planes) {
+    Carver cv(nullptr);
+    carve_vision(cv, Tn, N, k, d, cap, merging, planes);
+    return cv.total();
+}
+
 template <typename T>
 static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t* event_offsets, int k,
                          const void* text_, const metok_vision_params* p, void* out_feats_, int32_t* out_src,
                          int32_t* out_event, int32_t* out_members, int32_t* assign, float* token_score,
                          float* frame_score, float* event_score, uint8_t* event_is_key, int32_t* n_out, int cap,
-                         void* ws, cudaStream_t st) {
+                         void* ws, size_t ws_bytes, cudaStream_t st) {
     const T* feats = reinterpret_cast<const T*>(feats_);
     const T* text = reinterpret_cast<const T*>(text_);
     T* out_feats = reinterpret_cast<T*>(out_feats_);
@@ -1603,7 +1609,9 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     const bool mma = kBf16 && use_mma_path(d) && p->mode == METOK_MODE_TOPK_MERGE;
     Carver cv(ws);
     const double keep = p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey;
-    const int f3_bn = kBf16 || p->mode != METOK_MODE_TOPK_MERGE || force_simt() ? 0 : choose_f3(Nv, k, d, cap, keep);
+    int f3_bn = kBf16 || p->mode != METOK_MODE_TOPK_MERGE || force_simt() ? 0 : choose_f3(Nv, k, d, cap, keep);
+    // a workspace sized for other ratios, for which there were no planes: the CUDA cores find the same assignment
+    if (f3_bn && ws_bytes < vision_ws_bytes(Tn, N, k, d, cap, true, true)) f3_bn = 0;
     VisionWs w = carve_vision(cv, Tn, N, k, d, cap, p->mode == METOK_MODE_TOPK_MERGE, f3_bn > 0);
     // (the status word and the scratch that must start cleared are written by event_plan_kernel)
     if (const int rc = debug_arm(w.status, st)) return rc;
@@ -1821,13 +1829,11 @@ extern "C" int metok_compress_vision_bound(int T, int N, int k, const metok_visi
 extern "C" size_t metok_compress_vision_workspace_bytes(int dtype, int T, int N, int d, int k, int cap,
                                                         const metok_vision_params* p) {
     if (T < 1 || N < 1 || k < 1 || d < 1 || cap < 0) return 0;
-    Carver cv(nullptr);
     const bool merging = !(p && p->mode == METOK_MODE_POOL);
     bool planes = merging && dtype == METOK_F32 && !force_simt() && (long long)T * N <= 0x7FFFFFFFLL / 2;
     if (planes && p) planes = choose_f3(T * N, k, d, cap, p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey) > 0;
     else if (planes) planes = f3_a_bytes((long long)T * N, k, d) + f3_b_bytes(cap, k, d) <= kF3MaxBytes;
-    carve_vision(cv, T, N, k, d, cap, merging, planes);
-    return cv.total();
+    return vision_ws_bytes(T, N, k, d, cap, merging, planes);
 }
 
 extern "C" int metok_compress_vision(const void* feats, int dtype, int T, int N, int d,
@@ -1849,14 +1855,14 @@ extern "C" int metok_compress_vision(const void* feats, int dtype, int T, int N,
     if (bound < 0 || cap < bound) return METOK_ERR_INVALID_ARG;
     const int eb = dtype == METOK_F32 ? 4 : 2;
     if (((long long)d * eb) % 16 != 0 || T > 8192) return METOK_ERR_UNSUPPORTED;
-    const size_t need = metok_compress_vision_workspace_bytes(dtype, T, N, d, k, cap, p);
+    const size_t need = vision_ws_bytes(T, N, k, d, cap, p->mode != METOK_MODE_POOL, false);
     if (!ws || ws_bytes < need || !aligned16(ws)) return METOK_ERR_WORKSPACE;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (dtype == METOK_F32)
         return launch_vision<float>(feats, T, N, d, event_offsets, k, text_emb, p, out_feats, out_src, out_event,
                                     out_members, assign, token_score, frame_score, event_score, event_is_key,
-                                    n_out, cap, ws, st);
+                                    n_out, cap, ws, ws_bytes, st);
     return launch_vision<__nv_bfloat16>(feats, T, N, d, event_offsets, k, text_emb, p, out_feats, out_src,
                                         out_event, out_members, assign, token_score, frame_score, event_score,
-                                        event_is_key, n_out, cap, ws, st);
+                                        event_is_key, n_out, cap, ws, ws_bytes, st);
 }

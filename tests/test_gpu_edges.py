@@ -513,3 +513,38 @@ def test_score_planes_inside_the_selection(Hq, Hkv, Lt, n_vis, dtype, dh):
     assert int(got["status"].item()) == 0 and int(got["S_out"].item()) == n == S - n_vis + sum(budgets)
     assert torch.equal(got["scores"], scores) and torch.equal(got["keep_idx"][:n], want["keep_idx"][:n])
     assert torch.equal(got["hidden_out"][:n].view(torch.uint8), want["hidden_out"][:n].view(torch.uint8))
+
+
+def test_fp32_merge_with_a_workspace_sized_for_another_ratio():
+    """The planes depend on the keep ratio; a workspace without room for them takes the CUDA cores and the same assignment."""
+    import ctypes as c
+    rng = np.random.default_rng(3)
+    T, N, d, k = 40, 160, 644, 2
+    V = torch.from_numpy(rng.standard_normal((T, N, d)).astype(np.float32)).cuda()
+    t = torch.from_numpy(rng.standard_normal(d).astype(np.float32)).cuda()
+    offs = torch.tensor([0, 17, T], dtype=torch.int32, device="cuda")
+    p, lib = B.vision_params(0.5, 0.2, 0.2), B.lib()
+    want = {n: v.clone() for n, v in B.metok_compress_vision(V, offs, t, p).items() if isinstance(v, torch.Tensor)}
+    cap = B.metok_compress_vision_bound(T, N, k, p)
+    size = lambda q: lib.metok_compress_vision_workspace_bytes(B.F32, T, N, d, k, cap, c.byref(q))
+    small, full = size(B.vision_params(0.5, 0.001, 0.001)), size(p)
+    assert small < full
+    i32 = lambda n: torch.empty(n, dtype=torch.int32, device="cuda")
+    for n_bytes in (small, full - 1, full):
+        ws = torch.zeros(n_bytes, dtype=torch.uint8, device="cuda")
+        feats, f32 = torch.empty((cap, d), device="cuda"), [torch.empty(n, device="cuda") for n in (T * N, T, k)]
+        src, event, members, assign, n_out = i32(cap), i32(cap), i32(cap), i32(T * N), i32(1)
+        is_key = torch.empty(k, dtype=torch.uint8, device="cuda")
+        assert lib.metok_compress_vision(V.data_ptr(), B.F32, T, N, d, offs.data_ptr(), k, t.data_ptr(), c.byref(p), feats.data_ptr(),
+                                         src.data_ptr(), event.data_ptr(), members.data_ptr(), assign.data_ptr(), f32[0].data_ptr(),
+                                         f32[1].data_ptr(), f32[2].data_ptr(), is_key.data_ptr(), n_out.data_ptr(), cap, ws.data_ptr(),
+                                         n_bytes, torch.cuda.current_stream().cuda_stream) == 0
+        torch.cuda.synchronize()
+        n = int(n_out.item())
+        assert int(ws[:4].view(torch.int32).item()) == 0 and n == int(want["n_out"].item())
+        assert torch.equal(assign, want["assign"]) and torch.equal(src[:n], want["out_src"][:n])
+        assert torch.equal(feats[:n], want["out_feats"][:n])
+    assert lib.metok_compress_vision(V.data_ptr(), B.F32, T, N, d, offs.data_ptr(), k, t.data_ptr(), c.byref(p), feats.data_ptr(),
+                                     src.data_ptr(), event.data_ptr(), members.data_ptr(), assign.data_ptr(), f32[0].data_ptr(),
+                                     f32[1].data_ptr(), f32[2].data_ptr(), is_key.data_ptr(), n_out.data_ptr(), cap, ws.data_ptr(),
+                                     small - 1, torch.cuda.current_stream().cuda_stream) == -3
