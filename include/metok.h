@@ -327,7 +327,8 @@ METOK_API int metok_retention_budgets(double alpha, double r, int stage, const i
  *
  *   Errors: those of metok_prefill_prune per level; INVALID_ARG also for
  *   n_levels outside [1, 3], N0 not summing to n_vis, or a level without visual
- *   tokens.  Workspace: that of all levels together (..._schedule_workspace_bytes; 0 = invalid).
+ *   tokens.  Workspace: that of all levels together (..._schedule_workspace_bytes; 0 = invalid), or of the
+ *   largest one (metok_prefill_prune_workspace_bytes), with which they follow one another.
  *   Levels may share buffers as separate calls may (hidden of one = hidden_out of the one before, one
  *   scores array for all); arrays of their own let all levels be scored in one launch.
  * ------------------------------------------------------------------------- */

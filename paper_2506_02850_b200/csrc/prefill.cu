@@ -1106,15 +1106,16 @@ extern "C" int metok_prefill_prune_schedule(const metok_prune_level* levels, int
                                     lv.keep_idx, lv.S_out, lv.hidden_out, ws, ws_bytes);
         if (rc != METOK_OK) return rc;
     }
-    if (ws_bytes < metok_prefill_prune_schedule_workspace_bytes(n_levels, dtype, Hq, Hkv, Lt, S, dh, n_vis, alpha, r, N0))
-        return METOK_ERR_WORKSPACE;
+    // scratch for the largest level only: the levels follow one another and use it in turn
+    const bool shared = ws_bytes < metok_prefill_prune_schedule_workspace_bytes(n_levels, dtype, Hq, Hkv, Lt, S, dh, n_vis, alpha, r, N0);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const int eb = dtype == METOK_F32 ? 4 : 2;
-    const bool apart = schedule_levels_apart(levels, n_levels, sizes, S, n_vis, Hq, Hkv, Lt, dh, D, eb);
+    const bool apart = !shared && schedule_levels_apart(levels, n_levels, sizes, S, n_vis, Hq, Hkv, Lt, dh, D, eb);
     ScoreLevel sl[kMaxPruneLevels];
     Carver cv(ws);
     for (int s = 0; s < n_levels; ++s) {
         const AttnDims dm = make_dims(Hq, Hkv, Lt, S - n_vis + sizes[s], dh, vis_start, sizes[s], softmax_scale);
+        if (shared) cv = Carver(ws);
         sl[s] = {levels[s].q_text, levels[s].k_all, dm, carve_prefill(cv, dm, use_mma_attn(dtype, dh)), levels[s].scores};
         if (s > 0) sl[s].w.status = sl[0].w.status;
     }

@@ -548,3 +548,37 @@ def test_fp32_merge_with_a_workspace_sized_for_another_ratio():
                                      src.data_ptr(), event.data_ptr(), members.data_ptr(), assign.data_ptr(), f32[0].data_ptr(),
                                      f32[1].data_ptr(), f32[2].data_ptr(), is_key.data_ptr(), n_out.data_ptr(), cap, ws.data_ptr(),
                                      small - 1, torch.cuda.current_stream().cuda_stream) == -3
+
+
+@pytest.mark.parametrize("dtype,dh", [(torch.bfloat16, 64), (torch.float32, 24)])
+def test_schedule_with_scratch_for_its_largest_level(dtype, dh):
+    import ctypes as c
+    n_vis, r, vis_start, D, Lt = 6000, 0.8, 3, 264, 7
+    group, N0, sizes, rows, q, k, h = case = _schedule_case(n_vis, Lt, vis_start, r, dh, D, dtype, 2)
+    want = _levels_one_by_one(case, vis_start, r, dh ** -0.5)
+    lib, S, dt = B.lib(), rows[0], B.BF16 if dtype == torch.bfloat16 else B.F32
+    n0, dev = (c.c_int32 * 2)(*N0), "cuda"
+    i32 = lambda n: torch.empty(n, dtype=torch.int32, device=dev)
+    status, keep, s_out, origins = i32(1), [i32(n) for n in rows], i32(3), [i32(n) for n in sizes[:3]]
+    scores, outs = [torch.empty(n, device=dev) for n in sizes[:3]], [torch.empty_like(x) for x in h]
+    groups = [group] + [i32(n) for n in sizes[1:3]]
+    arr = (B.PruneLevel * 3)()
+    for s in range(3):
+        arr[s].q_text, arr[s].k_all, arr[s].hidden, arr[s].hidden_out = q[s].data_ptr(), k[s].data_ptr(), h[s].data_ptr(), outs[s].data_ptr()
+        arr[s].scores, arr[s].keep_idx, arr[s].S_out = scores[s].data_ptr(), keep[s].data_ptr(), s_out[s:].data_ptr()
+        arr[s].token_group, arr[s].origin = groups[s].data_ptr(), origins[s].data_ptr()
+    size = lib.metok_prefill_prune_workspace_bytes(dt, 4, 2, Lt, S, dh, n_vis)
+    assert size < lib.metok_prefill_prune_schedule_workspace_bytes(3, dt, 4, 2, Lt, S, dh, n_vis, 0.5, r, n0)
+    ws = torch.empty(size, dtype=torch.uint8, device=dev)
+
+    def call(n_bytes):
+        return lib.metok_prefill_prune_schedule(arr, 3, dt, 4, 2, Lt, S, dh, D, vis_start, n_vis, 0.5, r, n0, dh ** -0.5,
+                                                status.data_ptr(), ws.data_ptr(), n_bytes, torch.cuda.current_stream().cuda_stream)
+    assert call(size - 1) == -3 and call(size) == 0
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    for s, (w_scores, w_keep, w_hidden, w_group, w_origin) in enumerate(want):
+        n = len(w_keep)
+        assert int(s_out[s].item()) == n and torch.equal(scores[s], w_scores) and torch.equal(keep[s][:n], w_keep)
+        assert torch.equal(outs[s][:n].view(torch.uint8), w_hidden[:n].view(torch.uint8))
+        assert torch.equal(groups[s], w_group) and torch.equal(origins[s], w_origin)
