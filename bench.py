@@ -44,30 +44,28 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # captures (profiles/), keyed by (scope/kernel, workload); a kernel changed since its capture is left out
 # (its stage then reports traffic null).
 NCU_TRAFFIC_BYTES = {
-    ("segment/seg_score_kernel", "frames128"): 135844352,
+    ("segment/seg_score_kernel", "frames128"): 136150000,
     ("segment/seg_finish_kernel", "frames128"): 61952,
     ("compress/event_plan_kernel", "frames128"): 133376,
     ("compress/event_topk_kernel", "frames128"): 140544,
-    ("compress/merge_assign_mma_kernel", "frames128"): 135850496,
-    ("compress/merge_avg_kernel", "frames128"): 140172032,
+    ("compress/merge_assign_mma_kernel", "frames128"): 136140000,
+    ("compress/merge_avg_kernel", "frames128"): 140182000,
     ("prefill1/attn_stats_mma_kernel", "frames128"): 19441152,
     ("prefill1/attn_colsum_mma_kernel", "frames128"): 19510272,
     ("prefill1/attn_score_reduce_kernel", "frames128"): 599040,
     ("prefill1/class_topk_kernel", "frames128"): 211968,
-    ("prefill1/gather_rows_kernel", "frames128"): 53216768,
+    ("prefill1/gather_rows_kernel", "frames128"): 55006000,
     ("prefill2/attn_stats_mma_kernel", "frames128"): 7497472,
     ("prefill2/attn_colsum_mma_kernel", "frames128"): 7582720,
-    ("prefill2/attn_score_reduce_kernel", "frames128"): 225792,
-    ("prefill2/class_topk_kernel", "frames128"): 119040,
+    ("prefill2/class_topk_kernel", "frames128"): 310000,
     ("prefill2/gather_rows_kernel", "frames128"): 15964672,
     ("prefill3/attn_stats_mma_kernel", "frames128"): 2778880,
     ("prefill3/attn_colsum_mma_kernel", "frames128"): 2806528,
-    ("prefill3/attn_score_reduce_kernel", "frames128"): 78336,
-    ("prefill3/class_topk_kernel", "frames128"): 66560,
+    ("prefill3/attn_score_reduce_kernel", "frames128"): 79000,
+    ("prefill3/class_topk_kernel", "frames128"): 67000,
     ("prefill3/gather_rows_kernel", "frames128"): 473088,
     ("kv/class_topk_kernel", "frames128"): 135680,
-    ("kv/kv_stage_kernel", "frames128"): 4830464,
-    ("kv/kv_copy_kernel", "frames128"): 100684032,
+    ("kv/kv_move_kernel", "frames128"): 100054000,
 }
 
 
@@ -322,8 +320,9 @@ class Workload:
             st["a4 merge-assign, averaging"] = {
                 "bound": "tensor+hbm", "flops": float(np.sum(2.0 * (lens - k_e) * k_e * d)),
                 "bytes": float(Nv + n_out) * d * b,
-                "kernels": ["compress/merge_assign_mma_kernel", "compress/merge_assign_simt_kernel",
-                            "compress/merge_join_kernel", "compress/merge_avg_kernel"]}
+                "kernels": ["compress/merge_assign_mma_kernel", "compress/merge_planes_kernel", "compress/merge_assign_f32_mma_kernel",
+                            "compress/merge_join_f32_kernel", "compress/merge_assign_simt_kernel", "compress/merge_join_kernel",
+                            "compress/merge_avg_kernel"]}
         for i, s in enumerate(self.stages, start=1):
             kept = cfg.Lt + sum(min(bg, int((s["groups"] == g).sum().item())) for g, bg in enumerate(s["budgets"]))
             st[f"a5 attention scores, level {i}"] = {
@@ -341,7 +340,7 @@ class Workload:
             st["a8 K/V lists"] = {"bound": "latency", "bytes": 4.0 * Nv + 4.0 * cfg.L * kv_rows,
                                   "kernels": ["kv/class_topk_kernel", "kv/kv_paper_lists_kernel", "kv/kv_check_lists_kernel"]}
             st["a9 K/V in-place gather"] = {"bound": "hbm", "bytes": 2.0 * kv_rows * cfg.dh * b * 2 * cfg.Hkv * cfg.L,
-                                            "kernels": ["kv/kv_stage_kernel", "kv/kv_copy_kernel", "kv/kv_gather_kernel", "kv/kv_paper_kernel"]}
+                                            "kernels": ["kv/kv_move_kernel", "kv/kv_gather_kernel", "kv/kv_paper_kernel"]}
         return st
 
 
@@ -829,6 +828,7 @@ def main():
     if "a4 merge-assign, averaging" in sw:
         a4 = sw["a4 merge-assign, averaging"]
         put_work("compress/merge_assign_mma_kernel", "tensor", a4["flops"])
+        put_work("compress/merge_assign_f32_mma_kernel", "tensor", a4["flops"])
         put_work("compress/merge_assign_simt_kernel", "tensor", a4["flops"])
         put_work("compress/merge_avg_kernel", "hbm", a4["bytes"])
     if "a1+a2 segmentation, text relevance" in sw:
@@ -839,7 +839,7 @@ def main():
             put_work(f"prefill{i}/{k_}", "tensor", a5["flops"] / 2)
         put_work(f"prefill{i}/gather_rows_kernel", "hbm", a7["bytes"])
     if "a9 K/V in-place gather" in sw:
-        put_work("kv/kv_copy_kernel", "hbm", sw["a9 K/V in-place gather"]["bytes"])
+        put_work("kv/kv_move_kernel", "hbm", sw["a9 K/V in-place gather"]["bytes"])
     roofline = None
     if kernel_work:
         top = max(kernel_work, key=lambda k_: kern_us[k_])
