@@ -52,12 +52,26 @@ __device__ __forceinline__ float f3_margin(int d) { return 1.0e-6f + 4.0e-7f * s
 // A token's candidates beside the best one so far (best64, whose packing they share): at most kF3Cands are listed, and a
 // count of kF3All or more stands for all keys of the event (a norm that is no finite number).  Key tokens that are copies
 // of one another (frames that repeat) would fill the lists: of those with the same similarity and the same hash the first counts.
+// The hash is a sum over a row's 16-byte pieces, each multiplied with keys of its place: a sum of the bits alone, whatever their
+// weights, is the same for rows of few significant bits that differ (any even number of flipped signs), and such rows tie.
 constexpr int kF3Cands = 7, kF3All = 1 << 16;
 struct F3Cands {
     unsigned long long* list;                                 // [token][kF3Cands + 1]
     int32_t* count;                                           // [token], cleared with the merge's scratch
-    uint32_t* hash;                                           // [slot] of the key token's row
+    unsigned long long* hash;                                 // [slot] of the key token's row and the inverse of its norm
 };
+// A piece's share: two products of pairs of words, each word with a key of its own that depends on the place.  A thread's sum of
+// them is mixed once, so that the sums of different threads do not cancel.
+__device__ __forceinline__ unsigned long long f3_piece(const uint4& x, uint32_t place) {
+    uint32_t m = (place + 1u) * 0x6A09E667u;                  // odd constants: leading fractional bits of square roots
+    m = (m ^ (m >> 15)) * 0xBB67AE85u;
+    return (unsigned long long)(x.x + m * 0x3C6EF373u) * (x.y + m * 0xA54FF53Bu) +
+           (unsigned long long)(x.z + m * 0x510E527Fu) * (x.w + m * 0x9B05688Du);
+}
+__device__ __forceinline__ unsigned long long f3_mix(unsigned long long z) {
+    z = (z ^ (z >> 32)) * 0x1F83D9ABFB41BD6Bull;
+    return z ^ (z >> 29);
+}
 __device__ __forceinline__ unsigned long long f3_pack(float v, int slot) {
     return ((unsigned long long)float_key(v) << 32) | (unsigned long long)(~(uint32_t)slot);
 }
@@ -127,7 +141,8 @@ __device__ __forceinline__ void f3_split(const uint4& x, uint2& h, uint2& m, uin
 constexpr int kF3Ahead = 6;
 __global__ void __launch_bounds__(256)
 merge_planes_kernel(const float* __restrict__ feats, int Nv, int d, int N, const int32_t* ev_lo, int k, const int32_t* ev_out_off,
-                    TokenOut out, F3Planes pl, F3Cands ca, int bn, int steps_per_cta, int32_t* __restrict__ status) {
+                    const float* __restrict__ inv_norm, TokenOut out, F3Planes pl, F3Cands ca, int bn, int steps_per_cta,
+                    int32_t* __restrict__ status) {
     grid_dep_wait();
     __shared__ int32_t s_lo[kF3Events + 1], s_out[kF3Events + 1];
     const long long all = (long long)ev_lo[k] * N, first = (long long)ev_lo[0] * N;
@@ -165,7 +180,8 @@ merge_planes_kernel(const float* __restrict__ feats, int Nv, int d, int N, const
     dst += (uint32_t)r * 64u + (uint32_t)(((c >> 1) ^ ((r >> 1) & 3)) << 4) + (uint32_t)(c & 1) * 8u;
     const float* src = feats + (size_t)row * d + c * 4;
     const int k_lo = (int)blockIdx.y * steps_per_cta, k_hi = min(f3_steps(d), k_lo + steps_per_cta);
-    uint32_t hash = 0;                                        // a sum of the elements' bits with odd weights
+    unsigned long long hash = 0;
+    const float inv = slot >= 0 && k_lo == 0 ? inv_norm[row] : 0.f;
     for (int k0 = k_lo; k0 < k_hi; k0 += kF3Ahead) {
         uint4 v[kF3Ahead];
 #pragma unroll
@@ -176,8 +192,7 @@ merge_planes_kernel(const float* __restrict__ feats, int Nv, int d, int N, const
 #pragma unroll
         for (int u = 0; u < kF3Ahead; ++u) {
             if (k0 + u >= k_hi) continue;
-            const uint32_t w = (uint32_t)((k0 + u) * 8 + c) * 0x9E3779B2u + 1u;
-            hash += (v[u].x * 3u + v[u].y * 0x85EBCA6Bu + v[u].z * 0xC2B2AE35u + v[u].w * 0x27D4EB2Fu) * w;
+            if (slot >= 0) hash += f3_piece(v[u], (uint32_t)((k0 + u) * 8 + c));
             uint2 h, m, l;
             f3_split(v[u], h, m, l);
             uint8_t* o = dst + (size_t)(k0 + u) * 3 * plane;
@@ -186,7 +201,13 @@ merge_planes_kernel(const float* __restrict__ feats, int Nv, int d, int N, const
             *reinterpret_cast<uint2*>(o + 2 * plane) = l;
         }
     }
-    if (slot >= 0) atomicAdd(&ca.hash[slot], hash);
+    if (slot >= 0) {                                          // (the eight threads of a row are in one case)
+        const uint32_t row_lanes = 0xFFu << (threadIdx.x & 24);
+        hash = f3_mix(hash + (c == 0 ? __float_as_uint(inv) : 0u));
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) hash += __shfl_xor_sync(row_lanes, hash, o);
+        if (c == 0) atomicAdd(&ca.hash[slot], hash);
+    }
 }
 
 // Work unit = up to 128 of an event's tokens that are no key tokens x up to 256 of its key tokens (equal chunks of its keys);

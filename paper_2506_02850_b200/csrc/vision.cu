@@ -416,7 +416,7 @@ struct TokenOut {
     int32_t* rest;                 // per event, from its first token's place on: its tokens that are no key token
     unsigned long long* best64;    // packed argmax of the token's similarities
     int32_t* tile_done;            // at a row tile's first token: key chunks of the tile that are done (fp32 on the tensor cores: candidates of the token)
-    uint32_t* key_hash;            // fp32 on the tensor cores, else null: per output, hash of its key token
+    unsigned long long* key_hash;  // fp32 on the tensor cores, else null: per output, hash of its key token
     MemberLists ml;
 };
 __device__ __forceinline__ void token_out(const TokenOut& o, int lo, int n, int i, int e, int slot0, int place, bool key) {
@@ -428,7 +428,7 @@ __device__ __forceinline__ void token_out(const TokenOut& o, int lo, int n, int 
         o.out_src[slot] = lo + i;
         o.out_event[slot] = e;
         o.assign[lo + i] = slot;
-        if (o.key_hash) o.key_hash[slot] = 0u;
+        if (o.key_hash) o.key_hash[slot] = 0ull;
         members_start(o.ml, slot, lo + i, i, n);
     } else {
         o.rest[lo + i - place] = lo + i;
@@ -1465,7 +1465,7 @@ struct VisionWs {
     float* long_sums;
     F3Planes planes;          // fp32 merge on the tensor cores; so are the candidates' lists and the hashes
     unsigned long long* cands;
-    uint32_t* key_hash;
+    unsigned long long* key_hash;
     int32_t *long_done, *avg_next, *unit_next;
     int n_counters;           // the counters are cleared together: long, heavy, avg_next, unit_next and long_done
 };
@@ -1505,7 +1505,7 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
             w.planes.a = cv.take<uint8_t>(f3_a_bytes((long long)Tn * N, k, d));
             w.planes.b = cv.take<uint8_t>(f3_b_bytes(cap, k, d));
             w.cands = cv.take<unsigned long long>((size_t)Tn * N * (kF3Cands + 1));
-            w.key_hash = cv.take<uint32_t>(n);
+            w.key_hash = cv.take<unsigned long long>(n);
         }
     }
     return w;
@@ -1723,7 +1723,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
                 {
                     METOK_TIMED("merge_planes_kernel", st);
                     launch_chained(merge_planes_kernel, dim3(ceil_div(Nv, 32), ceil_div(steps, per)), dim3(256), 0, st, feats, Nv, d, N,
-                                   w.ev_lo, k, w.ev_out_off, to, w.planes, cands, f3_bn, per, w.status);
+                                   w.ev_lo, k, w.ev_out_off, inv_norm, to, w.planes, cands, f3_bn, per, w.status);
                 }
                 METOK_LAUNCH_CHECK();
                 METOK_ALLOW_SMEM(merge_assign_f32_mma_kernel, kF3SmemBytes);

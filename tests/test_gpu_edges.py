@@ -582,3 +582,36 @@ def test_schedule_with_scratch_for_its_largest_level(dtype, dh):
         assert int(s_out[s].item()) == n and torch.equal(scores[s], w_scores) and torch.equal(keep[s][:n], w_keep)
         assert torch.equal(outs[s][:n].view(torch.uint8), w_hidden[:n].view(torch.uint8))
         assert torch.equal(groups[s], w_group) and torch.equal(origins[s], w_origin)
+
+
+def _chains(x, y, inv):
+    """x[i] . y[j] as one chain of fp32 fused multiply-adds, times inv[j]; a fused multiply-add is one rounding of the exact sum."""
+    x, y = x.astype(np.longdouble), y.astype(np.longdouble)
+    acc = np.zeros((len(x), len(y)), dtype=np.float32)
+    for i in range(x.shape[1]):
+        acc = (acc.astype(np.longdouble) + np.outer(x[:, i], y[:, i])).astype(np.float32)
+    return acc * inv.astype(np.float32)[None]
+
+
+@pytest.mark.parametrize("kind", ["signs", "few bits"])
+def test_fp32_merge_of_key_tokens_that_tie_but_are_no_copies(kind):
+    """Rows of few significant bits: all key tokens have the same product with a token, but for the chain's roundings."""
+    V, inv, run = _fp32_merge_case(seed=21)
+    src, _ = run(V, inv)
+    rng = np.random.default_rng(5)
+    n, d = V.shape
+    rest = np.setdiff1d(np.arange(n), src)
+    tied = np.empty_like(V)
+    if kind == "signs":                                                  # tokens +-c, keys with 100 signs of them flipped
+        tied[:] = np.float32(1.312744140625) * np.sign(rng.standard_normal(d)).astype(np.float32)
+        for j in src:
+            tied[j, rng.permutation(d)[:100]] *= -1
+    else:                                                                # tokens of equal elements, keys of the same eight values
+        tied[:] = rng.uniform(1.0, 2.0, (n, 1)).astype(np.float32)
+        for j in src:
+            tied[j] = rng.permutation(np.resize(np.arange(1, 9) / 4, d)).astype(np.float32)
+    norms = 1.0 / np.sqrt((tied.astype(np.float64) ** 2).sum(1))
+    s, a = run(tied, norms)
+    assert np.array_equal(s, src)
+    some = rest[::41]
+    assert np.array_equal(a[some], _chains(tied[some], tied[src], norms[src]).argmax(1))
