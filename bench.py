@@ -321,7 +321,7 @@ class Workload:
                 "bound": "tensor+hbm", "flops": float(np.sum(2.0 * (lens - k_e) * k_e * d)),
                 "bytes": float(Nv + n_out) * d * b,
                 "kernels": ["compress/merge_assign_mma_kernel", "compress/merge_planes_kernel", "compress/merge_assign_f32_mma_kernel",
-                            "compress/merge_join_f32_kernel", "compress/merge_assign_simt_kernel", "compress/merge_join_kernel",
+                            "compress/merge_join_f32_kernel", "compress/merge_again_kernel", "compress/merge_assign_simt_kernel", "compress/merge_join_kernel",
                             "compress/merge_avg_kernel"]}
         for i, s in enumerate(self.stages, start=1):
             kept = cfg.Lt + sum(min(bg, int((s["groups"] == g).sum().item())) for g, bg in enumerate(s["budgets"]))

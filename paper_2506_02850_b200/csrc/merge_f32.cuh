@@ -8,9 +8,9 @@
 // other five, 2^-8 of the whole, have an accumulator of their own.
 //
 // Which key token is the most similar is decided by the fp32 chain all the same.  The tensor cores find, for every token, the key
-// with the largest similarity and the others that are within f3_margin of it; where there are any (a few per cent of the tokens),
-// merge_join_f32_kernel makes these products again as one chain of fused multiply-adds and takes the largest, so that the
-// assignment is the one that merge_assign_simt_kernel finds.
+// with the largest similarity and the others that are within f3_margin of it; where there are any (a few per cent of the tokens
+// where frames differ by a tenth, nearly all in still video), these products are made again as one chain of fused multiply-adds and
+// the largest is taken: merge_join_f32_kernel lists such tokens and merge_assign_simt_kernel, which has the same chains, does them.
 //
 // merge_planes_kernel writes the three planes of every token into the workspace, the tokens that are no key tokens and the key
 // tokens of an event apart, in the order and the swizzle in which a step's tiles lie in shared memory;
@@ -54,7 +54,10 @@ __device__ __forceinline__ float f3_margin(int d) { return 1.0e-6f + 4.0e-7f * s
 // of one another (frames that repeat) would fill the lists: of those with the same similarity and the same hash the first counts.
 // The hash is a sum over a row's 16-byte pieces, each multiplied with keys of its place: a sum of the bits alone, whatever their
 // weights, is the same for rows of few significant bits that differ (any even number of flipped signs), and such rows tie.
-constexpr int kF3Cands = 7, kF3All = 1 << 16;
+constexpr int kF3Cands = 31, kF3All = 1 << 30, kF3NonZero = 1 << 29;
+// Inverse norms from here on are those of rows at or below the norms' lower clamp: zeros, mostly, for which all keys are alike.
+// Where such a row is none of zeros, merge_planes_kernel adds kF3NonZero to its count.
+constexpr float kF3TinyInv = 9.9e7f;
 struct F3Cands {
     unsigned long long* list;                                 // [token][kF3Cands + 1]
     int32_t* count;                                           // [token], cleared with the merge's scratch
@@ -80,10 +83,27 @@ __device__ __forceinline__ float f3_value(unsigned long long p) {
     return __uint_as_float(k & 0x80000000u ? k & 0x7FFFFFFFu : ~k);
 }
 __device__ __forceinline__ int f3_slot(unsigned long long p) { return (int)~(uint32_t)p; }
-__device__ __forceinline__ void f3_push(const F3Cands& ca, int row, unsigned long long p) {
+__device__ __forceinline__ bool f3_push(const F3Cands& ca, int row, unsigned long long p) {   // false: the list is full
     const int at = atomicAdd(&ca.count[row], 1);
-    if (at < kF3Cands) ca.list[(size_t)row * (kF3Cands + 1) + at] = p;
+    if (at >= kF3Cands) return false;
+    ca.list[(size_t)row * (kF3Cands + 1) + at] = p;
+    return true;
 }
+
+// What merge_join_f32_kernel leaves to merge_assign_simt_kernel.  Tokens with a few near keys: `near`, their candidates (the best
+// one with them) in their lists.  Tokens to be done with all keys of their event: in `rest` (nobody
+// reads what was there any more) from the event's first place on, in tiles of kF3AgainRows that are opened as they come.
+constexpr int kF3AgainRows = 32, kF3UnitBits = 40;
+struct F3Again {
+    int4* near;                                               // token, event, number of candidates
+    int32_t* n_near;
+    int32_t* rows;                                            // [event]: tokens in tiles
+    unsigned long long* tiles;                                // tiles << kF3UnitBits | units (tile x chunk of kF3AgainRows keys)
+    unsigned long long* next;                                 // units taken beyond the first of every CTA
+    long long* unit0;                                         // [tile]: units before it
+    int32_t *event, *place, *done;                            // [tile]: its event, its first row's place in `rest`, chunks done
+};
+__host__ __device__ inline size_t f3_again_tiles(long long Nv, int k) { return (size_t)(Nv / kF3AgainRows + k); }
 
 // An event's key tokens in equal chunks of whole sixteens.
 __device__ __forceinline__ int f3_chunk(int nk, int nchunks) { return ((nk + nchunks - 1) / nchunks + 15) & ~15; }
@@ -181,7 +201,8 @@ merge_planes_kernel(const float* __restrict__ feats, int Nv, int d, int N, const
     const float* src = feats + (size_t)row * d + c * 4;
     const int k_lo = (int)blockIdx.y * steps_per_cta, k_hi = min(f3_steps(d), k_lo + steps_per_cta);
     unsigned long long hash = 0;
-    const float inv = slot >= 0 && k_lo == 0 ? inv_norm[row] : 0.f;
+    const float inv = inv_norm[row];
+    uint32_t bits = 0u;                                       // of all elements, without their signs
     for (int k0 = k_lo; k0 < k_hi; k0 += kF3Ahead) {
         uint4 v[kF3Ahead];
 #pragma unroll
@@ -193,6 +214,7 @@ merge_planes_kernel(const float* __restrict__ feats, int Nv, int d, int N, const
         for (int u = 0; u < kF3Ahead; ++u) {
             if (k0 + u >= k_hi) continue;
             if (slot >= 0) hash += f3_piece(v[u], (uint32_t)((k0 + u) * 8 + c));
+            bits |= (v[u].x | v[u].y | v[u].z | v[u].w) << 1;
             uint2 h, m, l;
             f3_split(v[u], h, m, l);
             uint8_t* o = dst + (size_t)(k0 + u) * 3 * plane;
@@ -203,11 +225,12 @@ merge_planes_kernel(const float* __restrict__ feats, int Nv, int d, int N, const
     }
     if (slot >= 0) {                                          // (the eight threads of a row are in one case)
         const uint32_t row_lanes = 0xFFu << (threadIdx.x & 24);
-        hash = f3_mix(hash + (c == 0 ? __float_as_uint(inv) : 0u));
+        hash = f3_mix(hash + (c == 0 && k_lo == 0 ? __float_as_uint(inv) : 0u));
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1) hash += __shfl_xor_sync(row_lanes, hash, o);
         if (c == 0) atomicAdd(&ca.hash[slot], hash);
     }
+    if (inv >= kF3TinyInv && bits) atomicOr(&ca.count[row], kF3NonZero);
 }
 
 // Work unit = up to 128 of an event's tokens that are no key tokens x up to 256 of its key tokens (equal chunks of its keys);
@@ -391,12 +414,14 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
                     sum[j] = v;
                     if (v > best_v) { best_v = v; best_c = c0 + j; }
                 }
-                if (least == 0.f) atomicAdd(&ca.count[row], kF3All);
+                const bool whole = least == 0.f || rinv >= kF3TinyInv;
+                if (whole) atomicOr(&ca.count[row], kF3All);
                 if (best_c >= 0) {
                     const unsigned long long me = f3_pack(best_v, un.col0 + best_c), old = atomicMax(&out.best64[row], me);
                     const float old_v = old ? f3_value(old) : -3.4e38f, from = fmaxf(best_v, old_v) - margin / rinv;
-                    if (best_v >= from && old_v >= from && !(old_v == best_v && ca.hash[f3_slot(old)] == ca.hash[f3_slot(me)]))
-                        f3_push(ca, row, old > me ? me : old);
+                    bool room = !whole;
+                    if (room && best_v >= from && old_v >= from && !(old_v == best_v && ca.hash[f3_slot(old)] == ca.hash[f3_slot(me)]))
+                        room = f3_push(ca, row, old > me ? me : old);
                     uint32_t close[2] = {0u, 0u};             // the others of these columns
 #pragma unroll
                     for (int j = 0; j < 64; ++j)
@@ -404,13 +429,13 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
 #pragma unroll
                     for (int w = 0; w < 2; ++w) {
 #pragma unroll 1
-                        for (uint32_t left = close[w]; left; left &= left - 1) {
+                        for (uint32_t left = close[w]; left && room; left &= left - 1) {
                             const int c = c0 + 32 * w + __ffs(left) - 1;
                             float v = 0.f;
 #pragma unroll
                             for (int j = 32 * w; j < 32 * w + 32; ++j) v = c0 + j == c ? sum[j] : v;
                             if (c != best_c && c < un.cols && !(v == best_v && ca.hash[un.col0 + c] == ca.hash[f3_slot(me)]))
-                                f3_push(ca, row, f3_pack(v, un.col0 + c));
+                                room = f3_push(ca, row, f3_pack(v, un.col0 + c));
                         }
                     }
                 }
@@ -423,132 +448,175 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
     if (threadIdx.x == 0 && s_abort) *status = METOK_ERR_TIMEOUT;
 }
 
-// The token's key among its candidates, and the token into that output's member list.  A CTA looks at 16 tokens, eight lanes
-// each, a candidate per lane; those whose products have to be made again are listed and its warps take one each: 256 elements
-// of the token and of its candidates go through shared memory, the next 256 on their way, and a lane per candidate runs its
-// chain over them.  What bounds it is the latency of these steps one after the other.
-constexpr int kF3JoinWarps = 4, kF3JoinPiece = 64;            // float4s of a row at a time
-__device__ __forceinline__ float f3_chain4(const float4& x, const float4& y, float a) {
-    return fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, a))));
-}
-struct F3Again { int row, lo, hi, s0, s1, n, slot[kF3Cands + 1]; };   // n candidates, 0: all keys of the event
+// The token's key where it is certain, and the token into that output's member list; the others are listed (F3Again).
+// Candidates are read by a warp per token, which tokens do not share: what bounds many of them is the reading of their rows.  A
+// tile reads all keys of the event, but for 32 tokens, and a key per token costs kF3KeysPerCand times less there (61 x 169 x 1156
+// in seven events, all tokens: nine candidates each 57 us, all 368 keys 205; 64 x 100 x 512: ten 23, all 250 keys 55); so a
+// token with more than kF3Few candidates goes there if that outweighs the keys that are none.  Those whose list is full go there
+// too, and those with a norm that is no finite number.
+// The call with frames of an event that differ by 0.1 / 0.01 / 0.001 / 0.0001, with a third of the tokens zero and with tokens
+// that are all alike but for 0.001: 61 x 169 x 1156 in one event 275 / 317 / 331 / 1625 / 279 / 1650 us, on the CUDA cores 1346
+// whatever they are; in seven 118 / 121 / 144 / 175 / 118 / 332, on the CUDA cores 257.  What is left above the CUDA cores is the
+// planes and the products that decided nothing.
+constexpr int kF3JoinThreads = 128, kF3Few = 8, kF3KeysPerCand = 12;
 __device__ __forceinline__ void f3_join(const TokenOut& out, int slot, int row, int lo, int hi, int s0, int s1) {
     out.assign[row] = slot;
     if (slot >= s0 && slot < s1) members_join(out.ml, slot, row, row - lo, hi - lo);
 }
-__global__ void __launch_bounds__(kF3JoinWarps * 32)
-merge_join_f32_kernel(const float* __restrict__ feats, int Nv, int d, int N, const int32_t* ev_lo, int k, const int32_t* ev_out_off,
-                      const float* __restrict__ inv_norm, TokenOut out, F3Cands ca) {
+__global__ void __launch_bounds__(kF3JoinThreads)
+merge_join_f32_kernel(int Nv, int d, int N, const int32_t* ev_lo, int k, const int32_t* ev_out_off, const float* __restrict__ inv_norm,
+                      TokenOut out, F3Cands ca, F3Again ag) {
     grid_dep_wait();
-    __shared__ float4 s_row[kF3JoinWarps][kF3Cands + 2][kF3JoinPiece];   // the token, then its candidates
     __shared__ int32_t s_lo[kF3Events + 1], s_out[kF3Events + 1];
-    __shared__ F3Again s_again[kF3JoinWarps * 4];
-    __shared__ int s_n;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & 7;
-    const int row = (blockIdx.x * kF3JoinWarps + warp) * 4 + (lane >> 3);
-    bool is_rest = row < Nv && !out.is_key[row];
-    if (threadIdx.x == 0) s_n = 0;
+    const int row = blockIdx.x * kF3JoinThreads + threadIdx.x, lane = threadIdx.x & 31;
+    bool is_rest = row < Nv;
+    int count = 0;
+    float inv = 1.f;
+    unsigned long long best = 0;
+    if (is_rest) {                                            // (a key token's are not used)
+        count = ca.count[row];
+        inv = inv_norm[row];
+        best = out.best64[row];
+        is_rest = !out.is_key[row];
+    }
     if (k <= kF3Events) {
-        for (int i = threadIdx.x; i <= k; i += blockDim.x) {
+        for (int i = threadIdx.x; i <= k; i += kF3JoinThreads) {
             s_lo[i] = ev_lo[i];
             s_out[i] = ev_out_off[i];
         }
+        __syncthreads();
         ev_lo = s_lo;
         ev_out_off = s_out;
     }
-    __syncthreads();
-    {
-        int lo = 0, hi = 0, s0 = 0, s1 = 0, count = 0;
-        float inv = 1.f;
-        unsigned long long mine = 0;                          // this lane's candidate; the last of the eight: the best
-        if (is_rest) {
-            count = ca.count[row];
-            inv = inv_norm[row];
-            if (sub == kF3Cands) mine = out.best64[row];
-            const int e = find_event(ev_lo, k, row / N);
-            lo = ev_lo[e] * N;
-            hi = ev_lo[e + 1] * N;
-            s0 = ev_out_off[e];
-            s1 = ev_out_off[e + 1];
-            is_rest = row >= lo && row < hi;                  // else a token of no event: its scratch is not this call's
-            if (is_rest && sub < count && count <= kF3Cands) mine = ca.list[(size_t)row * (kF3Cands + 1) + sub];
+    int e = 0, lo = 0, hi = 0, s0 = 0, s1 = 0;
+    if (is_rest) {
+        e = find_event(ev_lo, k, row / N);
+        lo = ev_lo[e] * N;
+        hi = ev_lo[e + 1] * N;
+        s0 = ev_out_off[e];
+        s1 = ev_out_off[e + 1];
+        is_rest = row >= lo && row < hi;                      // else a token of no event: its scratch is not this call's
+    }
+    // a row of zeros: its products are zeros, and best64 has the first key with one
+    const bool zeros = inv >= kF3TinyInv && !(count & kF3NonZero), all = is_rest && count > kF3Cands && !zeros;
+    int n = best ? 1 : 0;
+    if (is_rest && !zeros && count > 0 && !all) {
+        unsigned long long* list = ca.list + (size_t)row * (kF3Cands + 1);
+        const float from = f3_value(best) - f3_margin(d) / inv;
+        n = 0;
+        for (int i0 = 0; i0 < count; i0 += 4) {               // those that are still within the margin move up
+            unsigned long long x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = i0 + u < count ? list[i0 + u] : 0ull;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (x[u] && f3_value(x[u]) >= from) list[n++] = x[u];
         }
-        const unsigned long long best = __shfl_sync(0xFFFFFFFFu, mine, lane | 7);
-        const bool cand = is_rest && mine && f3_value(mine) >= f3_value(best) - f3_margin(d) / inv;
-        const uint32_t set = (__ballot_sync(0xFFFFFFFFu, cand) >> (lane & 24)) & 0xFFu;
-        const bool all = count > kF3Cands, again = is_rest && (all || __popc(set) > 1);
-        int at = again && sub == 0 ? atomicAdd(&s_n, 1) : 0;
-        at = __shfl_sync(0xFFFFFFFFu, at, lane & 24);
-        if (again) {
-            F3Again& x = s_again[at];
-            if (sub == 0) { x.row = row; x.lo = lo; x.hi = hi; x.s0 = s0; x.s1 = s1; x.n = all ? 0 : __popc(set); }
-            if (cand) x.slot[__popc(set & ((1u << sub) - 1u))] = f3_slot(mine);
-        } else if (is_rest && sub == 0) {
-            f3_join(out, best ? f3_slot(best) : -1, row, lo, hi, s0, s1);
+        list[n++] = best;
+    }
+    const bool tile = all || (is_rest && n > kF3Few && s1 - s0 < kF3KeysPerCand * n), near = is_rest && !tile && n > 1;
+    const uint32_t nears = __ballot_sync(0xFFFFFFFFu, near), tiles = __ballot_sync(0xFFFFFFFFu, tile);
+    if (is_rest && !tile && !near) f3_join(out, best ? f3_slot(best) : -1, row, lo, hi, s0, s1);
+    if (near) {
+        const int first = __ffs(nears) - 1;
+        int at = lane == first ? atomicAdd(ag.n_near, __popc(nears)) : 0;
+        at = __shfl_sync(nears, at, first) + __popc(nears & ((1u << lane) - 1u));
+        ag.near[at] = make_int4(row, e, n, 0);
+    }
+    if (tile) {
+        const uint32_t same = __match_any_sync(tiles, e);
+        const int first = __ffs(same) - 1;
+        int at = lane == first ? atomicAdd(&ag.rows[e], __popc(same)) : 0;
+        at = __shfl_sync(same, at, first) + __popc(same & ((1u << lane) - 1u));
+        out.rest[lo + at] = row;
+        out.best64[row] = 0ull;
+        if (at % kF3AgainRows == 0) {
+            const unsigned long long units = (unsigned long long)((s1 - s0 + kF3AgainRows - 1) / kF3AgainRows);
+            const unsigned long long was = atomicAdd(ag.tiles, (1ull << kF3UnitBits) + units);
+            const int t = (int)(was >> kF3UnitBits);
+            ag.unit0[t] = (long long)(was & ((1ull << kF3UnitBits) - 1ull));
+            ag.event[t] = e;
+            ag.place[t] = lo + at;
+            ag.done[t] = 0;
         }
     }
-    __syncthreads();
-    for (int t = warp; t < s_n; t += kF3JoinWarps) {
-        const F3Again& x = s_again[t];
-        const int n4 = d >> 2, nc = x.n;
-        const float4* x4 = reinterpret_cast<const float4*>(feats + (size_t)x.row * d);
+}
+
+// A warp and its candidates' rows: lane j < nc <= G runs the chain of row `row` with row `key`.  Pieces of 16 float4s of the nc + 1
+// rows come by 16-byte asynchronous copies into a ring of the warp's own, at a pitch that puts the candidates into different banks.
+constexpr int kF3Piece = 16, kF3RingFloat4s = 4 * 9 * (kF3Piece + 1);   // four stages of 8 candidates, or two of 16
+template <int G>
+__device__ __forceinline__ float f3_chains(const float* __restrict__ feats, int d, int row, int key, int nc, float4* ring) {
+    constexpr int kPitch = kF3Piece + 1, kStage = (G + 1) * kPitch, S = G == 8 ? 4 : 2, kCopies = G / 2 + 1;
+    static_assert(S * kStage <= kF3RingFloat4s, "");
+    const int lane = threadIdx.x & 31, half = lane >> 4, col = lane & 15, n4 = d >> 2, pieces = (n4 + kF3Piece - 1) / kF3Piece;
+    const float4* src[kCopies];                               // rows half, half + 2, ...; row 0 is the token
+#pragma unroll
+    for (int i = 0; i < kCopies; ++i) {
+        const int r = half + 2 * i, other = __shfl_sync(0xFFFFFFFFu, key, max(r, 1) - 1);
+        src[i] = reinterpret_cast<const float4*>(feats + (size_t)(r == 0 ? row : other) * d) + col;
+    }
+    const uint32_t dst0 = sm100::smem_u32(ring + half * kPitch + col);
+    auto issue = [&](int p, int stage) {
+        if (p < pieces) {
+            const uint32_t bytes = p * kF3Piece + col < n4 ? 16u : 0u;   // past the row's end: zeros, which change nothing
+#pragma unroll
+            for (int i = 0; i < kCopies; ++i)
+                if (half + 2 * i <= nc)
+                    sm100::cp_async16_zfill(dst0 + (uint32_t)(stage * kStage + 2 * i * kPitch) * 16u, bytes ? src[i] + p * kF3Piece : src[i], bytes);
+        }
+        sm100::cp_async_commit();
+    };
+    __syncwarp();                                             // the ring is free
+#pragma unroll
+    for (int p = 0; p < S; ++p) issue(p, p);
+    float a = 0.f;
+    int stage = 0;
+    for (int p = 0; p < pieces; ++p) {
+        sm100::cp_async_wait<S - 1>();
+        __syncwarp();
+        if (lane < nc) {
+            const float4 *x = ring + stage * kStage, *y = x + (lane + 1) * kPitch;
+#pragma unroll
+            for (int i = 0; i < kF3Piece; ++i) {
+                const float4 u = x[i], v = y[i];
+                a = fmaf(u.w, v.w, fmaf(u.z, v.z, fmaf(u.y, v.y, fmaf(u.x, v.x, a))));
+            }
+        }
+        __syncwarp();
+        issue(p + S, stage);
+        stage = stage + 1 == S ? 0 : stage + 1;
+    }
+    sm100::cp_async_wait<0>();
+    return a;
+}
+// A warp's share of the tokens with a few near keys.
+__device__ __forceinline__ void f3_near(const float* __restrict__ feats, int d, int N, int Nv, const int32_t* ev_lo, const int32_t* ev_out_off,
+                                        const float* __restrict__ inv_norm, const TokenOut& out, const unsigned long long* cands, const F3Again& ag,
+                                        int first, int stride, float4* ring) {
+    const int lane = threadIdx.x & 31;
+    if (first >= Nv) return;
+    int4 x = ag.near[first];                                  // with the total, which says whether it is one
+    const int total = *ag.n_near;
+    for (int t = first; t < total;) {
+        const int n = x.z, e = x.y;
+        const int slot = lane < n ? f3_slot(cands[(size_t)x.x * (kF3Cands + 1) + lane]) : 0, row = lane < n ? out.out_src[slot] : x.x;
+        const float inv = inv_norm[row];
+        const int lo = ev_lo[e] * N, hi = ev_lo[e + 1] * N, s0 = ev_out_off[e], s1 = ev_out_off[e + 1];
         unsigned long long won = 0;
-        if (nc == 0) {                                        // a key of the event per lane
-            for (int s = x.s0 + lane; s < x.s1; s += 32) {
-                const int key = out.out_src[s];
-                const float4* y4 = reinterpret_cast<const float4*>(feats + (size_t)key * d);
-                float a = 0.f;
-#pragma unroll 4
-                for (int i = 0; i < n4; ++i) a = f3_chain4(__ldg(x4 + i), __ldg(y4 + i), a);
-                const float v = a * inv_norm[key];
-                if (v > -3.4e38f) {
-                    const unsigned long long p = f3_pack(v, s);
-                    won = p > won ? p : won;
-                }
-            }
-        } else {
-            const int slot = lane < nc ? x.slot[lane] : -1, key = lane < nc ? out.out_src[slot] : 0;
-            const float4* y4[kF3Cands + 1];
-#pragma unroll
-            for (int j = 0; j <= kF3Cands; ++j) y4[j] = reinterpret_cast<const float4*>(feats + (size_t)__shfl_sync(0xFFFFFFFFu, key, j) * d);
-            const float key_inv = lane < nc ? inv_norm[key] : 0.f;
-            constexpr int U = kF3JoinPiece / 32;
-            float4 next[kF3Cands + 2][U];
-            auto fetch = [&](int i0) {
-                const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int i = i0 + 32 * u + lane;
-                    next[0][u] = i < n4 ? __ldg(x4 + i) : zero;
-#pragma unroll
-                    for (int j = 0; j <= kF3Cands; ++j) next[j + 1][u] = j < nc && i < n4 ? __ldg(y4[j] + i) : zero;
-                }
-            };
-            fetch(0);
-            float a = 0.f;
-            for (int i0 = 0; i0 < n4; i0 += kF3JoinPiece) {
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j <= kF3Cands + 1; ++j)
-                    if (j <= nc) {
-#pragma unroll
-                        for (int u = 0; u < U; ++u) s_row[warp][j][32 * u + lane] = next[j][u];
-                    }
-                __syncwarp();
-                fetch(i0 + kF3JoinPiece);
-                if (lane < nc) {                              // (past the row's end: zeros, which change nothing)
-#pragma unroll 8
-                    for (int i = 0; i < kF3JoinPiece; ++i) a = f3_chain4(s_row[warp][0][i], s_row[warp][lane + 1][i], a);
-                }
-            }
-            if (lane < nc) {
-                const float v = a * key_inv;
-                if (v > -3.4e38f) won = f3_pack(v, slot);
-            }
+        for (int c = 0; c < n;) {
+            const bool few = n - c <= 8;
+            const int nc = min(few ? 8 : 16, n - c), other = __shfl_sync(0xFFFFFFFFu, row, (c + lane) & 31);
+            const float a = few ? f3_chains<8>(feats, d, x.x, other, nc, ring) : f3_chains<16>(feats, d, x.x, other, nc, ring);
+            const float v = __shfl_sync(0xFFFFFFFFu, a, (lane - c) & 31) * inv;
+            if (lane >= c && lane < c + nc && v > -3.4e38f) won = f3_pack(v, slot);
+            c += nc;
         }
         const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(won >> 32));
         const uint32_t low = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(won >> 32) == top ? (uint32_t)won : 0u);
-        if (lane == 0) f3_join(out, top ? (int)~low : -1, x.row, x.lo, x.hi, x.s0, x.s1);
+        if (lane == 0) f3_join(out, top ? (int)~low : -1, x.x, lo, hi, s0, s1);
+        t += stride;
+        if (t < total) x = ag.near[t];
     }
 }
 

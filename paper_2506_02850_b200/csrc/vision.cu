@@ -568,6 +568,10 @@ cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __res
 #undef METOK_EVENT_TOPK
 }
 
+}  // namespace metok
+#include "merge_f32.cuh"
+namespace metok {
+
 // --------------------------------------------------------------------------- //
 // Merge-assign on the CUDA cores (fp32 inputs; bf16 only when forced for debugging): fp32 products, added in
 // the order of the row, so every dot product is one chain of fused multiply-adds.
@@ -577,30 +581,56 @@ cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __res
 // products of a unit are SimtTile's.  Rows past a unit's end are copies of another row: nobody reads their results.
 // 16 x 169 tokens in two events, d = 1156: the call takes 99 us.  Larger problems go to merge_f32.cuh.
 // Units of one row meet in a 64-bit atomicMax as in the tensor-core kernel: larger value, then lower slot.
+//
+// kAgain: the tokens that merge_join_f32_kernel left (F3Again): first those with a few near keys, a warp each, then the tiles, of
+// which most calls have none; whoever does a tile's last chunk adds its tokens to the member lists.
 // --------------------------------------------------------------------------- //
-template <typename T, int PT>                       // PT x PT outputs per thread
+template <typename T, int PT, bool kAgain>          // PT x PT outputs per thread
 __global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? sa_ctas_per_sm(PT) : 4)
-merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_t* __restrict__ ev_lo, int k,
+merge_assign_simt_kernel(const T* __restrict__ feats, int Nv, int d, int N, const int32_t* __restrict__ ev_lo, int k,
                          const int32_t* __restrict__ ev_out_off, const int32_t* __restrict__ ev_unit_off,
-                         const float* __restrict__ inv_norm, int32_t* __restrict__ next, TokenOut out) {
+                         const float* __restrict__ inv_norm, int32_t* __restrict__ next, TokenOut out, const unsigned long long* cands, F3Again ag) {
     grid_dep_wait();
     const int32_t *out_src = out.out_src, *rest = out.rest;
     using Tile = SimtTile<T, PT>;
+    using Count = std::conditional_t<kAgain, long long, int>;
     constexpr int kSaTile = Tile::kTile, kCopies = Tile::kCopies;
-    __shared__ __align__(16) Tile tile;
+    static_assert(!kAgain || kSaTile == kF3AgainRows, "the tiles that merge_join_f32_kernel opens");
+    constexpr size_t kRing = kF3RingFloat4s * sizeof(float4);
+    __shared__ __align__(16) unsigned char s_mem[kAgain ? std::max(sizeof(Tile), kSaThreads / 32 * kRing) : sizeof(Tile)];
+    Tile& tile = *reinterpret_cast<Tile*>(s_mem);
     __shared__ float s_inv[kSaTile];
-    __shared__ int s_next;
+    __shared__ Count s_next;
+    __shared__ int s_last;
     const int tid = threadIdx.x, ty = tid >> 3, tx = tid & 7;
-    const int total = ev_unit_off[k];
+    if constexpr (kAgain)
+        f3_near(feats, d, N, Nv, ev_lo, ev_out_off, inv_norm, out, cands, ag, (int)blockIdx.x + (tid >> 5) * (int)gridDim.x,
+                (int)gridDim.x * (kSaThreads / 32), reinterpret_cast<float4*>(s_mem + (tid >> 5) * kRing));
+    const unsigned long long tiles = kAgain ? *ag.tiles : 0ull;
+    const Count total = kAgain ? (Count)(tiles & ((1ull << kF3UnitBits) - 1ull)) : (Count)ev_unit_off[k];
     const int row_chunks = d / Tile::CE, ksteps = Tile::steps(d);
     const uint32_t dst0 = tile.copy_dst();
-    for (int unit = blockIdx.x; unit < total; unit = s_next) {
-        const int e = find_event(ev_unit_off, k, unit);
-        const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0;
+    for (Count unit = blockIdx.x; unit < total; unit = s_next) {
+        int e, t = 0, local;
+        if constexpr (kAgain) {
+            for (int n = (int)(tiles >> kF3UnitBits); n > 1;) {   // of the n tiles from t on: the last with unit0 <= unit, 32 at a time
+                const int step = (n + 31) >> 5, at = (tid & 31) * step;
+                const uint32_t before = __ballot_sync(0xFFFFFFFFu, at < n && ag.unit0[t + at] <= unit);
+                const int skip = (31 - __clz(before)) * step;
+                t += skip;
+                n = min(step, n - skip);
+            }
+            e = ag.event[t];
+            local = (int)(unit - ag.unit0[t]);
+        } else {
+            e = find_event(ev_unit_off, k, unit);
+            local = unit - ev_unit_off[e];
+        }
+        const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0, lo = ev_lo[e] * N, hi = ev_lo[e + 1] * N;
         const int nchunks = (nk + kSaTile - 1) / kSaTile;
-        const int local = unit - ev_unit_off[e];
-        const int row_tile = local / nchunks, chunk = local - row_tile * nchunks;
-        const int row0 = ev_lo[e] * N + row_tile * kSaTile, row_end = ev_lo[e + 1] * N - nk;   // places in `rest`
+        const int row_tile = kAgain ? 0 : local / nchunks, chunk = local - row_tile * nchunks;
+        const int row0 = kAgain ? ag.place[t] : lo + row_tile * kSaTile;                   // places in `rest`
+        const int row_end = kAgain ? min(row0 + kSaTile, lo + ag.rows[e]) : hi - nk;
         const int key0 = s0 + chunk * kSaTile, key_end = s0 + nk;
         const uint4* src[kCopies];                  // where this thread's copies of the first stage read
 #pragma unroll
@@ -610,7 +640,13 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
             src[i] = reinterpret_cast<const uint4*>(feats) + (size_t)row * row_chunks + Tile::copy_chunk();
         }
         __syncthreads();                            // the unit before is done with s_inv and both stages
-        if (tid == 0) s_next = total > (int)gridDim.x ? (int)gridDim.x + atomicAdd(next, 1) : total;
+        if (tid == 0) {
+            s_next = total;
+            if (total > (Count)gridDim.x) {
+                if constexpr (kAgain) s_next = (Count)gridDim.x + (Count)atomicAdd(ag.next, 1ull);
+                else s_next = (Count)gridDim.x + atomicAdd(next, 1);
+            }
+        }
         if (tid < kSaTile) s_inv[tid] = key0 + tid < key_end ? inv_norm[out_src[key0 + tid]] : 0.f;
         float acc[PT][PT];
         tile.dots(src, row_chunks, ksteps, dst0, acc);
@@ -634,14 +670,22 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_
             if (tx == 0 && at < row_end && best_s != 0x7FFFFFFF)
                 atomicMax(&out.best64[rest[at]], ((unsigned long long)float_key(best_v) << 32) | (unsigned long long)(~(uint32_t)best_s));
         }
+        if constexpr (kAgain) {
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) s_last = atomicAdd(&ag.done[t], 1) == nchunks - 1;
+            __syncthreads();
+            if (s_last && row0 + tid < row_end) {
+                __threadfence();
+                const int row = rest[row0 + tid];
+                const unsigned long long best = __ldcg(&out.best64[row]);
+                f3_join(out, best ? f3_slot(best) : -1, row, lo, hi, s0, key_end);
+            }
+        }
     }
 }
 
-}  // namespace metok
-#include "merge_f32.cuh"
-namespace metok {
-
-// After it: every token that is no key token to its output.  (In the tensor-core kernel the CTA that does a row tile's last
+// After it, where it does all of the merge: every token that is no key token to its output.  (In the tensor-core kernel the CTA that does a row tile's last
 // chunk does this; here that cost 15 us at 61 frames, this kernel takes 5.)
 __global__ void __launch_bounds__(256)
 merge_join_kernel(int Nv, int N, const int32_t* __restrict__ ev_lo, int k, const int32_t* __restrict__ ev_out_off, TokenOut out) {
@@ -1466,8 +1510,9 @@ struct VisionWs {
     F3Planes planes;          // fp32 merge on the tensor cores; so are the candidates' lists and the hashes
     unsigned long long* cands;
     unsigned long long* key_hash;
+    F3Again again;
     int32_t *long_done, *avg_next, *unit_next;
-    int n_counters;           // the counters are cleared together: long, heavy, avg_next, unit_next and long_done
+    int n_counters;           // the counters are cleared together: long, heavy, avg_next, unit_next and long_done, again's tiles, next, n_near and rows
 };
 
 static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, bool merging, bool planes) {
@@ -1494,7 +1539,8 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
         w.ml.few = cv.take<int32_t>(n * kAvgFew);
         w.ml.heavy_slot = cv.take<int32_t>(n);
         w.ml.long_slot = cv.take<int32_t>(n);
-        w.n_counters = 5 + avg_long_cap(d) * avg_max_pieces(d);
+        const int n_avg = 5 + avg_long_cap(d) * avg_max_pieces(d), n_again = (n_avg + 1) & ~1;
+        w.n_counters = planes ? n_again + 5 + k : n_avg;
         w.ml.long_counter = cv.take<int32_t>((size_t)w.n_counters);
         w.ml.heavy_counter = w.ml.long_counter + 1;
         w.avg_next = w.ml.long_counter + 2;              // two: items, pieces
@@ -1506,6 +1552,16 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
             w.planes.b = cv.take<uint8_t>(f3_b_bytes(cap, k, d));
             w.cands = cv.take<unsigned long long>((size_t)Tn * N * (kF3Cands + 1));
             w.key_hash = cv.take<unsigned long long>(n);
+            const size_t tiles = f3_again_tiles((long long)Tn * N, k);
+            w.again.unit0 = cv.take<long long>(tiles);
+            w.again.event = cv.take<int32_t>(tiles);
+            w.again.place = cv.take<int32_t>(tiles);
+            w.again.done = cv.take<int32_t>(tiles);
+            w.again.tiles = reinterpret_cast<unsigned long long*>(w.ml.long_counter + n_again);
+            w.again.next = w.again.tiles + 1;
+            w.again.n_near = w.ml.long_counter + n_again + 4;
+            w.again.rows = w.again.n_near + 1;
+            w.again.near = cv.take<int4>((size_t)Tn * N);
         }
     }
     return w;
@@ -1735,8 +1791,14 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
                 METOK_LAUNCH_CHECK();
                 {
                     METOK_TIMED("merge_join_f32_kernel", st);
-                    launch_chained(merge_join_f32_kernel, dim3(ceil_div(Nv, 4 * kF3JoinWarps)), dim3(kF3JoinWarps * 32), 0, st, feats, Nv,
-                                   d, N, w.ev_lo, k, w.ev_out_off, inv_norm, to, cands);
+                    launch_chained(merge_join_f32_kernel, dim3(ceil_div(Nv, kF3JoinThreads)), dim3(kF3JoinThreads), 0, st, Nv, d, N, w.ev_lo,
+                                   k, w.ev_out_off, inv_norm, to, cands, w.again);
+                }
+                METOK_LAUNCH_CHECK();
+                {
+                    METOK_TIMED("merge_again_kernel", st);
+                    launch_chained(merge_assign_simt_kernel<float, 4, true>, dim3(kNumSMs * sa_ctas_per_sm(4)), dim3(kSaThreads), 0, st, feats,
+                                   Nv, d, N, w.ev_lo, k, w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to, w.cands, w.again);
                 }
                 METOK_LAUNCH_CHECK();
             }
@@ -1745,11 +1807,11 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
             {
                 METOK_TIMED("merge_assign_simt_kernel", st);
                 auto assign_units = [&](auto kernel) {
-                    launch_chained(kernel, dim3(kNumSMs * sa_ctas_per_sm(simt)), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
-                                   w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to);
+                    launch_chained(kernel, dim3(kNumSMs * sa_ctas_per_sm(simt)), dim3(kSaThreads), 0, st, feats, Nv, d, N, w.ev_lo, k,
+                                   w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to, w.cands, w.again);
                 };
-                if (simt == 2) assign_units(merge_assign_simt_kernel<T, 2>);
-                else assign_units(merge_assign_simt_kernel<T, 4>);
+                if (simt == 2) assign_units(merge_assign_simt_kernel<T, 2, false>);
+                else assign_units(merge_assign_simt_kernel<T, 4, false>);
             }
             METOK_LAUNCH_CHECK();
             {

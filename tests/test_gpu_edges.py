@@ -615,3 +615,110 @@ def test_fp32_merge_of_key_tokens_that_tie_but_are_no_copies(kind):
     assert np.array_equal(s, src)
     some = rest[::41]
     assert np.array_equal(a[some], _chains(tied[some], tied[src], norms[src]).argmax(1))
+
+
+def _fp32_merge_both_ways(V, norms, offs, score, keep=0.2):
+    """Assignment and features of one fp32 merge: with a workspace that has room for the planes, and on the CUDA cores without."""
+    import ctypes as c
+    T, N, d = V.shape
+    k, lib = len(offs) - 1, B.lib()
+    Vd, text, off = torch.from_numpy(V).cuda(), torch.ones(d, device="cuda"), torch.tensor(offs, dtype=torch.int32, device="cuda")
+    inv, score = torch.from_numpy(norms.astype(np.float32)).cuda(), torch.from_numpy(score.astype(np.float32)).cuda()
+    p = B.vision_params(0.5, keep, keep)
+    p.token_inv_norm = inv.data_ptr()
+    cap = B.metok_compress_vision_bound(T, N, k, p)
+    size = lambda q: lib.metok_compress_vision_workspace_bytes(B.F32, T, N, d, k, cap, c.byref(q))
+    small, full = size(B.vision_params(0.5, 0.001, 0.001)), size(p)
+    assert small < full
+    i32 = lambda n: torch.empty(n, dtype=torch.int32, device="cuda")
+    res = []
+    for n_bytes in (full, small):
+        ws = torch.randint(0, 256, (n_bytes,), dtype=torch.uint8, device="cuda")
+        feats, f32 = torch.empty((cap, d), device="cuda"), [torch.empty(n, device="cuda") for n in (T, k)]
+        src, event, members, assign, n_out = i32(cap), i32(cap), i32(cap), i32(T * N), i32(1)
+        is_key = torch.empty(k, dtype=torch.uint8, device="cuda")
+        assert lib.metok_compress_vision(Vd.data_ptr(), B.F32, T, N, d, off.data_ptr(), k, text.data_ptr(), c.byref(p), feats.data_ptr(),
+                                         src.data_ptr(), event.data_ptr(), members.data_ptr(), assign.data_ptr(), score.data_ptr(),
+                                         f32[0].data_ptr(), f32[1].data_ptr(), is_key.data_ptr(), n_out.data_ptr(), cap, ws.data_ptr(),
+                                         n_bytes, torch.cuda.current_stream().cuda_stream) == 0
+        torch.cuda.synchronize()
+        assert int(ws[:4].view(torch.int32).item()) == 0
+        n = int(n_out.item())
+        res.append((src[:n].cpu().numpy(), assign.cpu().numpy(), members[:n].cpu().numpy(), feats[:n].cpu().numpy()))
+    return res
+
+
+def _same_merge(got, want):
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b, equal_nan=a.dtype.kind == "f")
+
+
+# near keys of a token: eight a round of chains, then sixteen; 31 fit its list beside the best; beyond twelve keys of the event per candidate
+# (128, 416 and 736 keys here) the token goes to a tile of 32 with all keys
+@pytest.mark.parametrize("near", [2, 8, 9, 10, 11, 17, 24, 25, 31, 32, 33, 64])
+@pytest.mark.parametrize("tokens", [1, 33, 2000])
+def test_fp32_merge_of_many_near_keys(near, tokens):
+    T, N, offs = 40, 160, [0, 4, 17, 40]
+    V, inv, _ = _fp32_merge_case(seed=near, T=T)
+    rng = np.random.default_rng(near + tokens)
+    d = V.shape[1]
+    score = rng.standard_normal(len(V))
+    (src, *_), _ = _fp32_merge_both_ways(V.reshape(T, N, d), inv, offs, score)
+    event_of = lambda r: np.searchsorted(offs, r // N, side="right") - 1
+    rest = np.setdiff1d(np.arange(len(V)), src)
+    rest = rng.permutation(rest)[:tokens]
+    groups = [np.flatnonzero(event_of(src) == e) for e in range(3)]
+    groups = [[g[i:i + near] for i in range(0, len(g) - near + 1, near)] for g in groups]
+    for g in sum(groups, []):                                            # keys a few ulps from one another
+        V[src[g]] = V[src[g[0]]] * (1.0 + 2e-7 * rng.integers(-2, 3, (near, d))).astype(np.float32)
+    for r in rest:
+        own = groups[event_of(r)]
+        V[r] = V[src[own[rng.integers(len(own))][0]]] + 0.1 * V[r]
+    inv = 1.0 / np.sqrt((V.astype(np.float64) ** 2).sum(1))
+    got, want = _fp32_merge_both_ways(V.reshape(T, N, d), inv, offs, score)
+    _same_merge(got, want)
+
+
+def test_fp32_merge_of_zeros_and_of_rows_next_to_nothing():
+    """Rows of zeros (of either sign) are equally similar to every key; rows below the norms' clamp that are no zeros are not."""
+    T, N, offs = 40, 160, [0, 17, 40]
+    V, inv, _ = _fp32_merge_case(seed=31, T=T)
+    rng = np.random.default_rng(1)
+    d = V.shape[1]
+    score = rng.standard_normal(len(V))
+    V[rng.permutation(len(V))[:2000]] = 0.0
+    V[rng.permutation(len(V))[:50]] *= -0.0
+    V[rng.permutation(len(V))[:70]] *= np.float32(1e-30)
+    V[rng.permutation(len(V))[:40]] *= np.float32(1e-42)                 # subnormal: no bf16 number holds them
+    V[rng.permutation(len(V))[:5], 3] = np.nan
+    norm = np.sqrt((V.astype(np.float64) ** 2).sum(1))
+    inv = 1.0 / np.where(np.isnan(norm), 1e-8, np.maximum(norm, 1e-8))
+    got, want = _fp32_merge_both_ways(V.reshape(T, N, d), inv, offs, score)
+    _same_merge(got, want)
+    V[:] = 0.0
+    got, want = _fp32_merge_both_ways(V.reshape(T, N, d), np.full(len(V), 1e8), offs, score)
+    _same_merge(got, want)
+    assert (got[1][:17 * N] == 0).sum() == 17 * N - len(got[0][got[0] < 17 * N]) + 1
+
+
+def test_fp32_merge_of_still_video_takes_about_as_long_as_of_any():
+    """Frames that hardly differ, or are a third zeros, leave many near keys per token (measured: 1.2 and 1.05 times the usual call)."""
+    T, N, d = 61, 169, 1156
+    g = torch.Generator(device="cuda").manual_seed(3)
+    text, offs, p = torch.randn(d, device="cuda", generator=g), torch.tensor([0, T], dtype=torch.int32, device="cuda"), B.vision_params(0.5, 0.25, 0.25)
+    base, noise = torch.randn((1, N, d), device="cuda", generator=g), torch.randn((T, N, d), device="cuda", generator=g)
+    padded = base + 0.1 * noise
+    padded[:, ::3] = 0.0
+    times = []
+    for V in (base + 0.1 * noise, base + 0.001 * noise, padded):
+        B.metok_compress_vision(V, offs, text, p)
+        best = float("inf")
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            B.metok_compress_vision(V, offs, text, p)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        times.append(best)
+    assert max(times) < 4 * times[0], times
