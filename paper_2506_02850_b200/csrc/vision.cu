@@ -1627,8 +1627,11 @@ static int choose_simt_outputs(int Nv, int k, double keep) {
 // The planes take one and a half times the memory of the features, and the share of the key tokens as much again, so beyond kF3MaxBytes
 // the CUDA cores do it.
 constexpr size_t kF3MaxBytes = (size_t)1 << 30;
+static bool f3_fits(long long Nv, int k, int d, int cap) {
+    return d >= kF3MinD && f3_a_bytes(Nv, k, d) + f3_b_bytes(cap, k, d) <= kF3MaxBytes;
+}
 static int choose_f3(int Nv, int k, int d, int cap, double keep) {
-    if (d < kF3MinD || f3_a_bytes(Nv, k, d) + f3_b_bytes(cap, k, d) > kF3MaxBytes) return 0;
+    if (!f3_fits(Nv, k, d, cap)) return 0;
     const double m = (double)Nv / k, keys = std::max(1.0, keep * m), rest = m - keys;
     double best = 0.0;
     int best_bn = 0;
@@ -1894,7 +1897,7 @@ extern "C" size_t metok_compress_vision_workspace_bytes(int dtype, int T, int N,
     const bool merging = !(p && p->mode == METOK_MODE_POOL);
     bool planes = merging && dtype == METOK_F32 && !force_simt() && (long long)T * N <= 0x7FFFFFFFLL / 2;
     if (planes && p) planes = choose_f3(T * N, k, d, cap, p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey) > 0;
-    else if (planes) planes = f3_a_bytes((long long)T * N, k, d) + f3_b_bytes(cap, k, d) <= kF3MaxBytes;
+    else if (planes) planes = f3_fits((long long)T * N, k, d, cap);
     return vision_ws_bytes(T, N, k, d, cap, merging, planes);
 }
 

@@ -102,6 +102,20 @@ def test_compress_bound_and_workspace(lib):
     assert 0 < n < (1 << 30)
 
 
+@pytest.mark.parametrize("d", [8, 56, 64])
+def test_workspace_for_any_ratio_has_room_for_what_some_ratio_takes(lib, d):
+    """Without parameters the fp32 workspace holds the planes of the merge; rows narrower than 60 floats never have any."""
+    size = lambda p: lib.metok_compress_vision_workspace_bytes(B.F32, 61, 169, d, 7, 3000, p)
+    p = B.vision_params(0.5, 0.25, 0.25)
+    p.mode = B.MODE_TOPK_MERGE
+    of_ratios = []
+    for keep in (0.001, 0.1, 0.25, 0.5):
+        p.keep_key = p.keep_nonkey = keep
+        of_ratios.append(size(ctypes.byref(p)))
+    assert size(None) >= max(of_ratios)
+    assert (size(None) == min(of_ratios)) == (d < 60)
+
+
 def test_validation_rejects_before_any_launch(lib):
     """Bad arguments return INVALID_ARG / UNSUPPORTED / WORKSPACE without touching the GPU
     (see device_pointers for what the non-null pointers are)."""
