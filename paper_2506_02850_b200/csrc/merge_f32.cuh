@@ -2,15 +2,17 @@
 //
 // A float is the sum of three bf16 numbers, its leading, middle and trailing eight significant bits (x = h + m + l exactly,
 // by truncation), so a product of two floats is the sum of nine products of bf16 numbers, each exact in the tensor core's
-// fp32.  Six are made: hh, hm, mh, mm, hl, lh; the three left out (ml, lm, ll) are below 2^-23 of the product.  What would
-// lose precision is the accumulator, which the tensor core cuts off instead of rounding: the sums of hh are therefore taken
-// out of tensor memory after every two steps, four additions, and added up in registers with rounding, and the
-// other five, 2^-8 of the whole, have an accumulator of their own.
+// fp32.  Six are made: hh, hm, mh, mm, hl, lh; the three left out (ml, lm, ll) are below 2^-21 of the product, 2^-24.5 of it on
+// average, and have its sign: similarities near one are 4e-8 too low, all of them.  What would lose precision is the
+// accumulator, which the tensor core cuts off instead of rounding: the sums of hh are therefore taken out of tensor memory after
+// every two steps, four additions, and added up in registers with rounding, and the other five, 2^-8 of the whole, have an
+// accumulator of their own.
 //
-// Which key token is the most similar is decided by the fp32 chain all the same.  The tensor cores find, for every token, the key
-// with the largest similarity and the others that are within f3_margin of it; where there are any (a few per cent of the tokens
-// where frames differ by a tenth, nearly all in still video), these products are made again as one chain of fused multiply-adds and
-// the largest is taken: merge_join_f32_kernel lists such tokens and merge_assign_simt_kernel, which has the same chains, does them.
+// Which of several key tokens that are nearly alike is the most similar is decided by the fp32 chain all the same.  The tensor cores
+// find, for every token, the key with the largest similarity and the others that are within f3_margin of it; where there are any
+// (a few per cent of the tokens where frames differ by a tenth, nearly all in still video), these products are made again as one
+// chain of fused multiply-adds and the largest is taken: merge_join_f32_kernel lists such tokens and merge_assign_simt_kernel,
+// which has the same chains, does them.
 //
 // merge_planes_kernel writes the three planes of every token into the workspace, the tokens that are no key tokens and the key
 // tokens of an event apart, in the order and the swizzle in which a step's tiles lie in shared memory;
@@ -45,10 +47,13 @@ __host__ __device__ inline size_t f3_a_bytes(long long Nv, int k, int d) { retur
 __host__ __device__ inline size_t f3_b_bytes(long long cap, int k, int d) { return (size_t)(f3_group0(cap, k) + 1) * 16 * kF3RowBytes * f3_steps(d); }
 struct F3Planes { uint8_t *a, *b; };
 
-// The chain's error and the tensor cores' together, twice (for the two keys that are compared), with a factor of two to three to spare: the largest
-// errors of a cosine against 64 bits, chain + here: width 60: 6.3e-7 + 2.8e-7, margin 4.1e-6; 1156: 1.6e-6 + 5.7e-7, 1.5e-5;
-// 3580: 2.9e-6 + 9.6e-7, 2.5e-5.
-__device__ __forceinline__ float f3_margin(int d) { return 1.0e-6f + 4.0e-7f * sqrtf((float)d); }
+// The chain's error and the tensor cores' together, twice (for the two keys that are compared), and something to spare.  Measured, not
+// proven: the largest errors of a cosine against 64 bits are, chain + here, for Gaussian rows of very different size 6.3e-7 + 2.8e-7 at
+// width 60 (margin 4.1e-6), 1.6e-6 + 5.7e-7 at 1156 (3.8e-5), 2.9e-6 + 9.6e-7 at 3580 (1.2e-4), for uniform and rectified ones no
+// more; in rows of nearly equal elements all additions of a chain round one way and it is off by up to 9.1e-7, 1.7e-5 and 5.3e-5 (1.5e-8
+// times the width), which is what the second term is for.  (Without it such rows took other keys than on the CUDA cores; it costs
+// 0.3 us of 111 at 61 x 169 x 1156, 2.4 of 155 at 24 x 144 x 3584.)
+__device__ __forceinline__ float f3_margin(int d) { return 1.0e-6f + fmaxf(4.0e-7f * sqrtf((float)d), 3.2e-8f * (float)d); }
 // A token's candidates beside the best one so far (best64, whose packing they share): at most kF3Cands are listed, and a
 // count of kF3All or more stands for all keys of the event (a norm that is no finite number).  Key tokens that are copies
 // of one another (frames that repeat) would fill the lists: of those with the same similarity and the same hash the first counts.
@@ -455,8 +460,8 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
 // token with more than kF3Few candidates goes there if that outweighs the keys that are none.  Those whose list is full go there
 // too, and those with a norm that is no finite number.
 // The call with frames of an event that differ by 0.1 / 0.01 / 0.001 / 0.0001, with a third of the tokens zero and with tokens
-// that are all alike but for 0.001: 61 x 169 x 1156 in one event 275 / 317 / 331 / 1625 / 279 / 1650 us, on the CUDA cores 1346
-// whatever they are; in seven 118 / 121 / 144 / 175 / 118 / 332, on the CUDA cores 257.  What is left above the CUDA cores is the
+// that are all alike but for 0.001: 61 x 169 x 1156 in one event 275 / 315 / 417 / 1625 / 279 / 1650 us, on the CUDA cores 1346
+// whatever they are; in seven 119 / 125 / 168 / 176 / 118 / 332, on the CUDA cores 257.  What is left above the CUDA cores is the
 // planes and the products that decided nothing.
 constexpr int kF3JoinThreads = 128, kF3Few = 8, kF3KeysPerCand = 12;
 __device__ __forceinline__ void f3_join(const TokenOut& out, int slot, int row, int lo, int hi, int s0, int s1) {

@@ -1669,7 +1669,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     Carver cv(ws);
     const double keep = p->alpha * p->keep_key + (1.0 - p->alpha) * p->keep_nonkey;
     int f3_bn = kBf16 || p->mode != METOK_MODE_TOPK_MERGE || force_simt() ? 0 : choose_f3(Nv, k, d, cap, keep);
-    // a workspace sized for other ratios, for which there were no planes: the CUDA cores find the same assignment
+    // a workspace sized for other ratios, for which there were no planes: the CUDA cores do it (with the same assignment as far as f3_margin holds)
     if (f3_bn && ws_bytes < vision_ws_bytes(Tn, N, k, d, cap, true, true)) f3_bn = 0;
     VisionWs w = carve_vision(cv, Tn, N, k, d, cap, p->mode == METOK_MODE_TOPK_MERGE, f3_bn > 0);
     // (the status word and the scratch that must start cleared are written by event_plan_kernel)

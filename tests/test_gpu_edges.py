@@ -722,3 +722,23 @@ def test_fp32_merge_of_still_video_takes_about_as_long_as_of_any():
             best = min(best, a.elapsed_time(b))
         times.append(best)
     assert max(times) < 4 * times[0], times
+
+
+@pytest.mark.parametrize("d", [516, 1156, 3580])
+def test_fp32_merge_of_rows_whose_chains_round_one_way(d):
+    """Rows of nearly equal elements: every addition of a chain rounds the same way, so that it is off by up to 1.5e-8 times the
+    width, and the twelve such keys have cosines with a row of equal elements that differ by no more."""
+    rng = np.random.default_rng(d)
+    T, N, offs = 24, 160, [0, 24]
+    score = rng.standard_normal(T * N)
+    src = np.sort(np.argsort(-score)[:T * N // 5])
+    wave = np.where(np.arange(d) % 2 == 0, 1.0, -1.0)
+    V = np.repeat(rng.uniform(1.0, 2.0, (T * N, 1)), d, 1)
+    V[src] = rng.standard_normal((len(src), d))
+    for j in rng.permutation(src)[:12]:                                  # 1 - cos is half the wave's square
+        V[j] = rng.uniform(1.0, 2.0) * (1.0 + np.sqrt(rng.uniform(0.0, 6e-8 * d)) * wave)
+    V = V.astype(np.float32)
+    inv = 1.0 / np.sqrt((V.astype(np.float64) ** 2).sum(1))
+    got, want = _fp32_merge_both_ways(V.reshape(T, N, d), inv, offs, score)
+    assert np.array_equal(got[0], src)
+    _same_merge(got, want)
