@@ -6,7 +6,7 @@
 //
 // Fast path.  A source row at or beyond n is never written by anybody, so it can be
 // read at any time.  Only the first h rows of the list, h = #{i : keep[i] < n}, have
-// their source inside the destination region.  Those h rows are read, into registers or a
+// their source inside the destination region.  Those h rows are read, into shared memory or a
 // staging area in the workspace, by the CTAs of the slab's cluster before a cluster barrier behind
 // which every row is written.  With a keep ratio r about r*n rows are concerned.
 //
@@ -24,6 +24,7 @@
 
 #include "common.cuh"
 #include "launchers.h"
+#include "sm100.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -127,25 +128,22 @@ kv_check_lists_kernel(int S_cur, const int32_t* __restrict__ keep_idx, const int
 }
 
 // ---- fast path ------------------------------------------------------------------
-constexpr int kKvFastThreads = 256;
-constexpr int kKvFastUnroll = 8;          // 16-byte chunks in flight per thread
-constexpr int kKvCtasPerSm = 4;           // (64 registers)
+constexpr int kKvMoveWarps = 16;          // most warps of a CTA (64 registers, two such CTAs per SM)
+constexpr int kKvPieceBytes = 2048, kKvRing = 3;   // a warp's ring: pieces on their way
 constexpr int kKvMaxSplit = 8;            // most CTAs per slab, a cluster
 constexpr size_t kKvStageBudget = (size_t)128 << 20;   // bytes of workspace the staging area may take
 
-// First index of the ascending list keep[0..n) whose value is >= n; whole warp, 32-ary search.
-__device__ __forceinline__ int warp_lower_bound(const int32_t* __restrict__ keep, int n, int lane) {
-    int lo = 0, hi = n;                                   // answer in [lo, hi]
-    while (hi > lo) {
-        const int step = (hi - lo + 31) / 32;
-        const int idx = lo + lane * step;
-        const bool ge = idx < hi ? keep[idx] >= n : true;
-        const unsigned bal = __ballot_sync(0xFFFFFFFFu, ge);
-        const int f = bal ? __ffs(bal) - 1 : 32;          // first probe that is >= n; 32: none was
-        const int new_hi = f < 32 ? min(hi, lo + f * step) : hi;   // keep[new_hi] >= n (or new_hi == hi)
-        const int new_lo = f > 0 ? lo + (f - 1) * step + 1 : lo;   // the probe before it was < n
-        hi = new_hi;
-        lo = new_lo;
+// First index of [0, n) with f(index), which stays true from there on; n if there is none.  Whole warp, 32-ary search.
+template <typename F>
+__device__ __forceinline__ int warp_first(int n, int lane, F f) {
+    int lo = 0;
+    while (n > 0) {                                        // it lies in [lo, lo + n]
+        const int step = (n + 31) >> 5, at = lane * step + step - 1;
+        const uint32_t yes = __ballot_sync(0xFFFFFFFFu, at >= n ? true : f(lo + at));
+        if (!yes) return lo + n;
+        const int skip = (__ffs(yes) - 1) * step;
+        lo += skip;
+        n = min(step - 1, n - skip);
     }
     return lo;
 }
@@ -159,27 +157,31 @@ __device__ __forceinline__ SlabId slab_of(int slab, int Hkv) {
     return s;
 }
 
-// A cluster per slab moves the slab's rows; its CTAs take runs of 2048 pieces of 16 bytes in turn.  Rows whose
-// source lies at or beyond the new length (all but the first h) are never written before they are read.  The others are
-// read by everybody before anybody writes: those of a CTA's first run into registers, later ones into the staging area,
-// which the same thread reads again; then a cluster barrier, behind which the first run's loads of all rows land.
-// Records h per layer (-1: too many for the staging area, the general path takes the layer).
-// What bounds it is HBM, with scattered rows of 256 bytes.  Staging and copying as two kernels, the copy with four CTAs
-// per slab in one and a half waves, took (call, cold, us) for 28 layers x 4 heads of 18 432 + 64 rows, 6.5 / 15 / 30 / 50 %
-// kept: 52.2 / 98.3 / 196.6 / 469.0, this 46.0 / 87.0 / 185.3 / 472.1; 40 layers x 40 heads of 2751 rows 108.5 and 85.0, one
-// layer of one head of 63 606 rows 148.4 and 70.6.
-__global__ void __launch_bounds__(kKvFastThreads, kKvCtasPerSm)
+// A cluster per slab moves the slab's rows; the warps of its CTAs take pieces of up to kKvPieceBytes of consecutive destination rows in
+// turn.  Rows at the front that stay where they are (keep[i] == i: the first p) are left alone.  Rows whose source lies at or
+// beyond the new length (all from the h-th on) are never written before they are read.  The others are read by everybody before
+// anybody writes: those of a warp's first pieces into its ring, later ones into the staging area, which the same warp reads
+// again; then a cluster barrier, behind which a piece leaves by one bulk copy as soon as it has landed.
+// Records h per layer (-1: too many for the staging area, the general path takes the layer, before anything is read).
+// What bounds it is HBM, with scattered rows of 256 bytes.  Rows through registers, all CTAs of 256 threads resident to the end,
+// were a tenth slower, and other streams' kernels waited for the whole of it: an attention or selection CTA wants most of an SM.
+// The call, cold, with two kernels (stage, copy) / through registers / this, in us, 28 layers x 4 heads of 18 432 + 72 rows, 6.5 / 15 / 30 / 50 %
+// kept: 48.4 / 94.8 / 193.9 / 463.7; 43.6 / 86.0 / 183.2 / 469.8; 39.1 / 82.0 / 176.4 / 466.0.  40 layers x 40 heads of 2751 rows, 10 %:
+// 139.6; 117.5; 111.4.  One layer of one head of 63 614 rows: 69.8; 39.1; 26.8.  One 128-frame video with the call beside pruning
+// levels 2 and 3: 264.6; 268.5; 255.  The first of them with rings of 2 x 2 / 6 x 1 / 3 x 4 KB (eight warps) / 3 x 8 KB (four): 38.7 / 46.1 /
+// 41.5 / 40.2 against 36.6 warm.
+__global__ void __launch_bounds__(kKvMoveWarps * 32, 2)
 kv_move_kernel(KvPtrs ptrs, int layer0, int Hkv, int S_cap, int S_cur, int row_chunks,
                const int32_t* __restrict__ keep_idx, const int32_t* __restrict__ keep_len, int stage_rows,
                int32_t* __restrict__ haz, uint4* stage, const int32_t* __restrict__ valid,
                int n_layers, int32_t* __restrict__ status) {
     grid_dep_wait();
-    __shared__ int s_h;
+    extern __shared__ uint8_t kv_dyn[];
     const SlabId id = slab_of(blockIdx.y, Hkv);
-    const int layer = layer0 + id.ll;
-    const bool lead = blockIdx.x == 0 && id.which == 0 && id.head == 0 && threadIdx.x == 0;   // one thread per layer
-    // the call's status word: a rejected list (GIVEN policy) is an invalid argument
-    if (layer0 == 0 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    const int layer = layer0 + id.ll, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool lead = id.which == 0 && id.head == 0 && blockIdx.x == 0 && threadIdx.x == 0;
+    // the call's status: METOK_OK, or INVALID_ARG if any caller-given list failed its check
+    if (layer0 == 0 && blockIdx.y == 0 && blockIdx.x == 0 && threadIdx.x == 0) {
         int st = METOK_OK;
         if (valid)
             for (int l = 0; l < n_layers; ++l)
@@ -199,55 +201,107 @@ kv_move_kernel(KvPtrs ptrs, int layer0, int Hkv, int S_cap, int S_cur, int row_c
     uint4* base = reinterpret_cast<uint4*>(id.which ? ptrs.v[id.ll] : ptrs.k[id.ll]) +
                   (size_t)id.head * S_cap * row_chunks;
     uint4* stg = stage + ((size_t)(layer * 2 + id.which) * Hkv + id.head) * (size_t)stage_rows * row_chunks;
-    const int total = n * row_chunks;
-    constexpr int kStep = kKvFastThreads * kKvFastUnroll;
-    uint4 v[kKvFastUnroll];
-    unsigned some = 0;                                     // which of them there are to store
-    auto load = [&](int g0, int h) {
-        some = 0;
-#pragma unroll
-        for (int u = 0; u < kKvFastUnroll; ++u) {
-            const int gc = g0 + u * kKvFastThreads + threadIdx.x;
-            if (gc < total) {
-                const int i = gc / row_chunks, c = gc - i * row_chunks;
-                const int src = keep[i];
-                if (src != i) {
-                    v[u] = i < h ? stg[gc] : base[(size_t)src * row_chunks + c];
-                    some |= 1u << u;
+    const uint32_t ring = ((sm100::smem_u32(kv_dyn) + 127u) & ~127u) + (uint32_t)(warp * kKvRing * kKvPieceBytes);
+    // pieces: `rows` whole rows, or one of the `segs` parts of a row that is wider
+    constexpr int kPiece = kKvPieceBytes / 16;
+    const int rows = max(1, kPiece / row_chunks), segs = (row_chunks + kPiece - 1) / kPiece;
+    int p = 0;                                             // rows that stay
+    {
+        const bool too_many = stage_rows < n && keep[stage_rows] < n;   // h > stage_rows: uniform per cluster
+        const uint32_t stay = __ballot_sync(0xFFFFFFFFu, lane < n && keep[lane] == lane);
+        if (too_many) {
+            if (lead) haz[layer] = -1;
+            return;
+        }
+        p = stay == 0xFFFFFFFFu ? warp_first(n, lane, [&](int i) { return keep[i] > i; }) : __ffs(~stay) - 1;
+    }
+    const int pieces = ((n - p) + rows - 1) / rows * segs;
+    const int warps = blockDim.x >> 5, first = blockIdx.x * warps + warp, stride = gridDim.x * warps;
+    struct Piece { int row0, nrows, c0, nc; };
+    auto piece = [&](int q) {
+        Piece x;
+        const int g = q / segs, sg = q - g * segs;
+        x.row0 = p + g * rows;
+        x.nrows = min(rows, n - x.row0);
+        x.c0 = sg * kPiece;
+        x.nc = min(kPiece, row_chunks - x.c0);             // (all chunks where a piece is whole rows)
+        return x;
+    };
+    // the sources of a piece's first 32 rows, one per lane
+    auto sources = [&](int q) {
+        if (q >= pieces) return 0;
+        const int i = p + q / segs * rows + lane;
+        return i < n ? keep[i] : 0;
+    };
+    auto load = [&](int q, int src, int slot, int h) {
+        if (q < pieces) {
+            const Piece x = piece(q);
+            const uint32_t dst = ring + (uint32_t)(slot * kKvPieceBytes + lane * 16);
+            int r = lane / x.nc, c = lane - r * x.nc;
+            const int dr = 32 / x.nc, dc = 32 - dr * x.nc, total = x.nrows * x.nc;
+#pragma unroll 4
+            for (int t = 0; t < total; t += 32) {
+                int from = __shfl_sync(0xFFFFFFFFu, src, r & 31);
+                if (t + lane < total) {
+                    const int i = x.row0 + r;
+                    if (r >= 32) from = keep[i];
+                    const uint4* at = i < h ? stg + (size_t)i * row_chunks : base + (size_t)from * row_chunks;
+                    sm100::cp_async16_zfill(dst + (uint32_t)t * 16u, at + x.c0 + c, 16u);
                 }
+                r += dr;
+                c += dc;
+                if (c >= x.nc) { c -= x.nc; ++r; }
             }
         }
+        sm100::cp_async_commit();
     };
-    const int g_first = blockIdx.x * kStep, stride = gridDim.x * kStep;
-    load(g_first, 0);                                      // all from their sources
-    if (threadIdx.x < 32) {
-        const int h = warp_lower_bound(keep, n, threadIdx.x);
-        if (threadIdx.x == 0) s_h = h;
-    }
-    __syncthreads();
-    const int h = s_h;
-    if (lead) haz[layer] = h <= stage_rows ? h : -1;
-    if (h > stage_rows) return;                            // uniform per cluster
-    for (int gc = g_first + stride + (int)threadIdx.x, u = 0; gc < h * row_chunks;) {
-        const int i = gc / row_chunks, c = gc - i * row_chunks, src = keep[i];
-        if (src != i) stg[gc] = base[(size_t)src * row_chunks + c];
-        if (++u < kKvFastUnroll) {
-            gc += kKvFastThreads;
-        } else {
-            u = 0;
-            gc += stride - (kKvFastUnroll - 1) * kKvFastThreads;
+#pragma unroll 1
+    for (int k = 0; k < kKvRing; ++k) load(first + k * stride, sources(first + k * stride), k, 0);   // all from their sources
+    int ahead = sources(first + kKvRing * stride);
+    const int h = warp_first(n, lane, [&](int i) { return keep[i] >= n; });
+    if (lead) haz[layer] = h;
+    if (h > p) {
+#pragma unroll 1
+        for (int q = first + kKvRing * stride; q < pieces; q += stride) {
+            const Piece x = piece(q);
+            if (x.row0 >= h) break;
+            for (int t = lane; t < x.nrows * x.nc; t += 32) {
+                const int i = x.row0 + t / x.nc, c = x.c0 + t % x.nc;
+                if (i < h) stg[(size_t)i * row_chunks + c] = base[(size_t)keep[i] * row_chunks + c];
+            }
         }
+        sm100::cp_async_wait_all();
+        __syncwarp();
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    for (int g0 = g_first;;) {
-#pragma unroll
-        for (int u = 0; u < kKvFastUnroll; ++u)
-            if (some >> u & 1u) base[g0 + u * kKvFastThreads + threadIdx.x] = v[u];
-        g0 += stride;
-        if (g0 >= total) break;
-        load(g0, h);
+    if (gridDim.x > 1) {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
+        __syncthreads();
     }
+    int slot = 0;
+#pragma unroll 1
+    for (int q = first; q < pieces; q += stride) {
+        sm100::cp_async_wait<kKvRing - 2>();               // this piece has landed: kKvRing - 2 were asked for after it, and one more at first
+        sm100::fence_proxy_async();
+        __syncwarp();
+        const Piece x = piece(q);
+        if (lane == 0) {
+            sm100::bulk_store(base + (size_t)x.row0 * row_chunks + x.c0, ring + (uint32_t)slot * kKvPieceBytes, (uint32_t)(x.nrows * x.nc) * 16u);
+            sm100::bulk_commit();
+            sm100::bulk_wait_read<1>();                    // the piece before has left its slot
+        }
+        __syncwarp();
+        if (q != first) {
+            const int next = q + (kKvRing - 1) * stride;
+            const int src = ahead;
+            ahead = sources(next + stride);
+            load(next, src, slot == 0 ? kKvRing - 1 : slot - 1, h);
+        }
+        slot = slot + 1 == kKvRing ? 0 : slot + 1;
+    }
+    if (lane == 0) sm100::bulk_wait_all();
+    sm100::cp_async_wait_all();
 }
 
 // ---- general path -----------------------------------------------------------------
@@ -432,14 +486,17 @@ extern "C" int metok_kv_compact(void* const* k_layers, void* const* v_layers, in
         const int nl = (L - l0) < kKvMaxLayersPerLaunch ? (L - l0) : kKvMaxLayersPerLaunch;
         const KvPtrs ptrs = kv_ptrs(k_layers, v_layers, l0, nl);
         const int slabs = nl * 2 * Hkv;
-        // a cluster of as many CTAs per slab as keep all of them resident at once: two waves cost more than fewer loads in
-        // flight (224 slabs with clusters of four: 58.4 us instead of 46.0), and clusters that are no power of two leave SMs
-        // unused (192 slabs with clusters of three: 50.2 us instead of 44.6)
+        // a cluster of as many CTAs per slab as keep all of them resident at once (clusters that are no power of two leave SMs
+        // unused); where there are more slabs than places, smaller CTAs and more of them, so that one's reads run beside
+        // another's writes (3200 slabs of 311 rows: 125 us with 16 warps, 111 with four)
         int split = 1;
-        while (2 * split <= kKvMaxSplit && 2 * split * slabs <= kNumSMs * kKvCtasPerSm) split *= 2;
+        while (2 * split <= kKvMaxSplit && 2 * split * slabs <= 2 * kNumSMs) split *= 2;
+        const int warps = slabs <= 2 * kNumSMs ? kKvMoveWarps : slabs <= 4 * kNumSMs ? kKvMoveWarps / 2 : kKvMoveWarps / 4;
+        const size_t smem = (size_t)warps * kKvPieceBytes * kKvRing + 128;
+        METOK_ALLOW_SMEM(kv_move_kernel, smem);
         {
             METOK_TIMED("kv_move_kernel", st);
-            launch_chained_clusters(split, kv_move_kernel, dim3(split, slabs), dim3(kKvFastThreads), 0, st,
+            launch_chained_clusters(split, kv_move_kernel, dim3(split, slabs), dim3(warps * 32), smem, st,
                 ptrs, l0, Hkv, S_cap, S_cur, row_chunks, keep_idx, keep_len, w.stage_rows, w.haz, w.stage, valid, L,
                 w.status);
         }

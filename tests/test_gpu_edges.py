@@ -70,8 +70,8 @@ def test_kv_paper_rule_in_place(L, S_vis, vis_start, tail, l1, dh, dtype):
             assert torch.equal(x[:, :n], o[:, idx])
 
 
-@pytest.mark.parametrize("L,Hkv", [(1, 1), (10, 4), (10, 8), (38, 4)])             # clusters of 8, 4, 2 and 1 CTAs
-@pytest.mark.parametrize("S", [1, 129, 1100, 3000])                                # in registers, staged, and beyond the staging area
+@pytest.mark.parametrize("L,Hkv", [(1, 1), (10, 4), (10, 8), (38, 4)])             # clusters of 8, 2, 1 and 1 CTAs, the last of 8 warps
+@pytest.mark.parametrize("S", [1, 129, 1100, 3000])                                # in the rings, staged, and beyond the staging area
 @pytest.mark.parametrize("lists", ["dense", "some", "front", "back", "one", "all"])
 def test_kv_rows_given_move_in_place(L, Hkv, S, lists):
     g = torch.Generator().manual_seed(S + L)
@@ -99,6 +99,36 @@ def test_kv_rows_given_move_in_place(L, Hkv, S, lists):
         n = int(lens[l])
         assert torch.equal(cache[l, :, :, :n], want[l, :, :, :n])
         assert torch.equal(cache[l, :, :, S:], want[l, :, :, S:])                  # rows beyond the cache's length are not touched
+
+
+# rows of 16 to 4112 bytes: pieces of 128 rows, of 42, of 5, of one, rows in two and in three parts; clusters of 4 and CTAs of 4 warps
+@pytest.mark.parametrize("dh", [8, 24, 200, 1024, 1032, 2056])
+@pytest.mark.parametrize("L,Hkv,S", [(3, 1, 700), (9, 4, 100), (76, 4, 40)])
+@pytest.mark.parametrize("stay", [0, 5, 31, 32, 33])
+def test_kv_rows_of_any_width_behind_rows_that_stay(dh, L, Hkv, S, stay):
+    g = torch.Generator().manual_seed(dh + stay)
+    cache = torch.randint(-2 ** 15, 2 ** 15, (L, 2, Hkv, S + 1, dh), generator=g, dtype=torch.int16).cuda()
+    keep = torch.zeros((L, S), dtype=torch.int32)
+    lens = torch.zeros(L, dtype=torch.int32)
+    for l in range(L):
+        mask = torch.rand(S, generator=g) < (0.05, 0.3, 0.6)[l % 3]
+        mask[:stay], mask[stay] = True, False
+        rows = mask.nonzero().flatten().to(torch.int32)
+        keep[l, :len(rows)] = rows
+        lens[l] = len(rows)
+    want = cache.clone()
+    for l in range(L):
+        n = int(lens[l])
+        want[l, :, :, :n] = cache[l][:, :, keep[l, :n].long().cuda()]
+    kv = cache.view(torch.bfloat16)
+    r = B.metok_kv_compact([kv[l, 0] for l in range(L)], [kv[l, 1] for l in range(L)], S, B.KV_GIVEN, 0, 0,
+                           keep_idx=keep.cuda(), keep_len=lens.cuda())
+    torch.cuda.synchronize()
+    assert torch.equal(r["new_len"].cpu(), lens)
+    for l in range(L):
+        n = int(lens[l])
+        assert torch.equal(cache[l, :, :, :n], want[l, :, :, :n])
+        assert torch.equal(cache[l, :, :, S:], want[l, :, :, S:])
 
 
 @pytest.mark.parametrize("count", [15, 16, 17, 18, 127, 128, 129, 130, 300, 700])
