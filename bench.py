@@ -65,6 +65,7 @@ NCU_TRAFFIC_BYTES = {
     ("prefill3/class_topk_kernel", "frames128"): 67000,
     ("prefill3/gather_rows_kernel", "frames128"): 473088,
     ("kv/class_topk_kernel", "frames128"): 135680,
+    ("kv/kv_move_kernel", "frames128"): 99549000,
 }
 
 

@@ -852,9 +852,10 @@ __device__ __forceinline__ void schedule_check(const ScheduleHand& h) {
 
 // One level of a schedule: the class-wise selection of up to 81 920 items (as cs_topk_kernel), class and origin of every
 // survivor for the next level, and beside it the hidden rows of the level before.  CTAs 0 .. C - 1 select; each of the others runs
-// `workers` gather workers.  The selection is a chain of latencies in eight SMs or one and the gather is bound by memory, so
-// one hides the other (18 432 tokens, three levels: 8 + 16, 7.5 + 7.6 and 5 + 4 us one after the other, and 3 us for every
-// launch between that handed classes and origins on).
+// `workers` gather workers.  The selection is a chain of latencies in eight SMs or one and the gather is bound by memory.  What it
+// saves is the launches, 3 us for every one that handed classes and origins on; under ncu (18 432 tokens) the second level's launch
+// takes 21.6 us where its selection and the gather alone take 9 and 15, the third's 9.9 for 5 and 7.5: the gather's CTAs come in
+// the selection's clusters of eight and deal the rows out by a fixed stride, so those placed late end late.
 template <int IT, bool kCl>
 __global__ void __launch_bounds__(IT == kCsMaxItems ? kCsMaxItemsThreads : 1024)
 schedule_select_kernel(const float* __restrict__ sc, int n_vis, CsLayout lay, TopkBudgets budgets, int S, int vis_start,

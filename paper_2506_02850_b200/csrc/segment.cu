@@ -827,7 +827,7 @@ extern "C" int metok_segment_score_events(const void* feats, int dtype, int T, i
     if (dtype == METOK_F32) {
         if (nchunk <= 32 * 4) METOK_FS(float, 4);
         if (nchunk <= 32 * 8) METOK_FS(float, 8);
-        if (nchunk <= 32 * 10) METOK_FS(float, 10);              // four CTAs per SM, not three (61 x 169 x 1156: the encode path 136.5 -> 135.1 us)
+        if (nchunk <= 32 * 10) METOK_FS(float, 10);              // four CTAs per SM, not three (61 x 169 rows of 1028 / 1156 / 1280: 22.0 / 23.1 / 23.0 -> 20.5 / 21.5 / 21.4 us; 256 x 144 x 1280: 51.4 -> 44.9)
         METOK_FS(float, 16);
     }
     METOK_FS(__nv_bfloat16, 4);                                  // the bf16 kernel has no per-width variants

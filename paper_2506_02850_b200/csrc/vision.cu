@@ -685,8 +685,8 @@ merge_assign_simt_kernel(const T* __restrict__ feats, int Nv, int d, int N, cons
     }
 }
 
-// After it, where it does all of the merge: every token that is no key token to its output.  (In the tensor-core kernel the CTA that does a row tile's last
-// chunk does this; here that cost 15 us at 61 frames, this kernel takes 5.)
+// After it, where it does all of the merge: every token that is no key token to its output.  (In the bf16 tensor-core kernel the CTA
+// that does a row tile's last chunk does this; behind the chain of a unit that lengthened the launch by more than this one takes.)
 __global__ void __launch_bounds__(256)
 merge_join_kernel(int Nv, int N, const int32_t* __restrict__ ev_lo, int k, const int32_t* __restrict__ ev_out_off, TokenOut out) {
     grid_dep_wait();
@@ -1609,8 +1609,10 @@ static bool use_mma_path(int d) { return !force_simt() && d % 8 == 0; }
 // Outputs per thread (a side of the square) of the CUDA-core kernel, from the number of 64 x 64 units of the mean event.
 // Few of them leave SMs idle and last as long as one unit's chain of d steps: 16 x 16 units are then the fastest.  The whole
 // call with 16 x 16 / 32 x 32, at that many units: 169 tokens of 1156, 34 units 42 / 48 us, 57: 51 / 49, 103: 82 / 70; 100 tokens
-// of 512, 36: 29 / 32, 75: 39 / 42, 98: 48 / 44.  (Larger units would pay only for rows so short that fp32 stays on the CUDA
-// cores however many units there are.)
+// of 512, 36: 29 / 32, 75: 39 / 42, 98: 48 / 44.  Units of 64 x 64 wherever 740 to 888 of them fill a round of CTAs, in a launch of
+// their own that finds none elsewhere, matter only for rows so narrow that fp32 stays here however many units there are; the call
+// with that launch / without: rows of 20 floats, 612 such units 39.0 / 37.0 us, 735: 41.0 / 39.0; of 56, 740: 43.3 / 43.0, 888: 46.4 /
+// 49.2, 891: 50.7 / 49.2; of 32, 888: 39.8 / 41.2.  So there is none.
 static int choose_simt_outputs(int Nv, int k, double keep) {
     const double m = (double)Nv / k, keys = std::max(1.0, keep * m), units = ((m - keys) / 64 + 0.5) * (keys / 64 + 0.5) * k;
     return units < kNumSMs / 2 ? 2 : 4;
