@@ -11,8 +11,8 @@
 // Which of several key tokens that are nearly alike is the most similar is decided by the fp32 chain all the same.  The tensor cores
 // find, for every token, the key with the largest similarity and the others that are within f3_margin of it; where there are any
 // (a few per cent of the tokens where frames differ by a tenth, nearly all in still video), these products are made again as one
-// chain of fused multiply-adds and the largest is taken: merge_join_f32_kernel lists such tokens and merge_assign_simt_kernel,
-// which has the same chains, does them.
+// chain of fused multiply-adds and the largest is taken, by merge_join_f32_kernel, or for tokens with too many of them by
+// merge_assign_simt_kernel, which has the same chains.
 //
 // merge_planes_kernel writes the three planes of every token into the workspace, the tokens that are no key tokens and the key
 // tokens of an event apart, in the order and the swizzle in which a step's tiles lie in shared memory;
@@ -67,6 +67,7 @@ struct F3Cands {
     unsigned long long* list;                                 // [token][kF3Cands + 1]
     int32_t* count;                                           // [token], cleared with the merge's scratch
     unsigned long long* hash;                                 // [slot] of the key token's row and the inverse of its norm
+    int32_t *suspects, *n_suspects;                           // the tokens whose count is not zero
 };
 // A piece's share: two products of pairs of words, each word with a key of its own that depends on the place.  A thread's sum of
 // them is mixed once, so that the sums of different threads do not cancel.
@@ -88,20 +89,18 @@ __device__ __forceinline__ float f3_value(unsigned long long p) {
     return __uint_as_float(k & 0x80000000u ? k & 0x7FFFFFFFu : ~k);
 }
 __device__ __forceinline__ int f3_slot(unsigned long long p) { return (int)~(uint32_t)p; }
-__device__ __forceinline__ bool f3_push(const F3Cands& ca, int row, unsigned long long p) {   // false: the list is full
+__device__ __forceinline__ bool f3_push(const F3Cands& ca, int row, unsigned long long p, bool& fresh) {   // false: the list is full
     const int at = atomicAdd(&ca.count[row], 1);
+    fresh |= at == 0;
     if (at >= kF3Cands) return false;
     ca.list[(size_t)row * (kF3Cands + 1) + at] = p;
     return true;
 }
 
-// What merge_join_f32_kernel leaves to merge_assign_simt_kernel.  Tokens with a few near keys: `near`, their candidates (the best
-// one with them) in their lists.  Tokens to be done with all keys of their event: in `rest` (nobody
+// What merge_join_f32_kernel leaves to merge_assign_simt_kernel: tokens to be done with all keys of their event, in `rest` (nobody
 // reads what was there any more) from the event's first place on, in tiles of kF3AgainRows that are opened as they come.
 constexpr int kF3AgainRows = 32, kF3UnitBits = 40;
 struct F3Again {
-    int4* near;                                               // token, event, number of candidates
-    int32_t* n_near;
     int32_t* rows;                                            // [event]: tokens in tiles
     unsigned long long* tiles;                                // tiles << kF3UnitBits | units (tile x chunk of kF3AgainRows keys)
     unsigned long long* next;                                 // units taken beyond the first of every CTA
@@ -409,6 +408,7 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
             };
             for (int i = 0; i < nseg; ++i, ++seg) take(0u, smem_u32(&hfull_bar), (uint32_t)seg & 1u, smem_u32(&hempty_bar));
             take(kF3BN, smem_u32(&sfull_bar), (uint32_t)n & 1u, smem_u32(&sempty_bar));
+            bool fresh = false;                               // the first to find something beside the best key of its token
             if (ok && mine && row >= 0) {
                 float best_v = -3.4e38f, least = rinv;        // zero: a norm beyond the largest float, of the token or of a key
                 int best_c = -1;
@@ -420,13 +420,13 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
                     if (v > best_v) { best_v = v; best_c = c0 + j; }
                 }
                 const bool whole = least == 0.f || rinv >= kF3TinyInv;
-                if (whole) atomicOr(&ca.count[row], kF3All);
+                if (whole) fresh = (atomicOr(&ca.count[row], kF3All) & ~kF3NonZero) == 0;
                 if (best_c >= 0) {
                     const unsigned long long me = f3_pack(best_v, un.col0 + best_c), old = atomicMax(&out.best64[row], me);
                     const float old_v = old ? f3_value(old) : -3.4e38f, from = fmaxf(best_v, old_v) - margin / rinv;
                     bool room = !whole;
                     if (room && best_v >= from && old_v >= from && !(old_v == best_v && ca.hash[f3_slot(old)] == ca.hash[f3_slot(me)]))
-                        room = f3_push(ca, row, old > me ? me : old);
+                        room = f3_push(ca, row, old > me ? me : old, fresh);
                     uint32_t close[2] = {0u, 0u};             // the others of these columns
 #pragma unroll
                     for (int j = 0; j < 64; ++j)
@@ -440,10 +440,16 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
 #pragma unroll
                             for (int j = 32 * w; j < 32 * w + 32; ++j) v = c0 + j == c ? sum[j] : v;
                             if (c != best_c && c < un.cols && !(v == best_v && ca.hash[un.col0 + c] == ca.hash[f3_slot(me)]))
-                                room = f3_push(ca, row, f3_pack(v, un.col0 + c));
+                                room = f3_push(ca, row, f3_pack(v, un.col0 + c), fresh);
                         }
                     }
                 }
+            }
+            const uint32_t f = __ballot_sync(0xFFFFFFFFu, fresh);
+            if (f) {
+                int at = lane == 0 ? atomicAdd(ca.n_suspects, __popc(f)) : 0;
+                at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(f & ((1u << lane) - 1u));
+                if (fresh) ca.suspects[at] = row;
             }
         }
     }
@@ -451,100 +457,6 @@ merge_assign_f32_mma_kernel(int d, int N, const int32_t* ev_lo, int k, const int
     __syncthreads();
     if (warp == kF3EpiWarps + 1) tmem_dealloc(tmem_base, 512);
     if (threadIdx.x == 0 && s_abort) *status = METOK_ERR_TIMEOUT;
-}
-
-// The token's key where it is certain, and the token into that output's member list; the others are listed (F3Again).
-// Candidates are read by a warp per token, which tokens do not share: what bounds many of them is the reading of their rows.  A
-// tile reads all keys of the event, but for 32 tokens, and a key per token costs kF3KeysPerCand times less there (61 x 169 x 1156
-// in seven events, all tokens: nine candidates each 57 us, all 368 keys 205; 64 x 100 x 512: ten 23, all 250 keys 55); so a
-// token with more than kF3Few candidates goes there if that outweighs the keys that are none.  Those whose list is full go there
-// too, and those with a norm that is no finite number.
-// The call with frames of an event that differ by 0.1 / 0.01 / 0.001 / 0.0001, with a third of the tokens zero and with tokens
-// that are all alike but for 0.001: 61 x 169 x 1156 in one event 275 / 315 / 417 / 1625 / 279 / 1650 us, on the CUDA cores 1346
-// whatever they are; in seven 119 / 125 / 168 / 176 / 118 / 332, on the CUDA cores 257.  What is left above the CUDA cores is the
-// planes and the products that decided nothing.
-constexpr int kF3JoinThreads = 128, kF3Few = 8, kF3KeysPerCand = 12;
-__device__ __forceinline__ void f3_join(const TokenOut& out, int slot, int row, int lo, int hi, int s0, int s1) {
-    out.assign[row] = slot;
-    if (slot >= s0 && slot < s1) members_join(out.ml, slot, row, row - lo, hi - lo);
-}
-__global__ void __launch_bounds__(kF3JoinThreads)
-merge_join_f32_kernel(int Nv, int d, int N, const int32_t* ev_lo, int k, const int32_t* ev_out_off, const float* __restrict__ inv_norm,
-                      TokenOut out, F3Cands ca, F3Again ag) {
-    grid_dep_wait();
-    __shared__ int32_t s_lo[kF3Events + 1], s_out[kF3Events + 1];
-    const int row = blockIdx.x * kF3JoinThreads + threadIdx.x, lane = threadIdx.x & 31;
-    bool is_rest = row < Nv;
-    int count = 0;
-    float inv = 1.f;
-    unsigned long long best = 0;
-    if (is_rest) {                                            // (a key token's are not used)
-        count = ca.count[row];
-        inv = inv_norm[row];
-        best = out.best64[row];
-        is_rest = !out.is_key[row];
-    }
-    if (k <= kF3Events) {
-        for (int i = threadIdx.x; i <= k; i += kF3JoinThreads) {
-            s_lo[i] = ev_lo[i];
-            s_out[i] = ev_out_off[i];
-        }
-        __syncthreads();
-        ev_lo = s_lo;
-        ev_out_off = s_out;
-    }
-    int e = 0, lo = 0, hi = 0, s0 = 0, s1 = 0;
-    if (is_rest) {
-        e = find_event(ev_lo, k, row / N);
-        lo = ev_lo[e] * N;
-        hi = ev_lo[e + 1] * N;
-        s0 = ev_out_off[e];
-        s1 = ev_out_off[e + 1];
-        is_rest = row >= lo && row < hi;                      // else a token of no event: its scratch is not this call's
-    }
-    // a row of zeros: its products are zeros, and best64 has the first key with one
-    const bool zeros = inv >= kF3TinyInv && !(count & kF3NonZero), all = is_rest && count > kF3Cands && !zeros;
-    int n = best ? 1 : 0;
-    if (is_rest && !zeros && count > 0 && !all) {
-        unsigned long long* list = ca.list + (size_t)row * (kF3Cands + 1);
-        const float from = f3_value(best) - f3_margin(d) / inv;
-        n = 0;
-        for (int i0 = 0; i0 < count; i0 += 4) {               // those that are still within the margin move up
-            unsigned long long x[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = i0 + u < count ? list[i0 + u] : 0ull;
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (x[u] && f3_value(x[u]) >= from) list[n++] = x[u];
-        }
-        list[n++] = best;
-    }
-    const bool tile = all || (is_rest && n > kF3Few && s1 - s0 < kF3KeysPerCand * n), near = is_rest && !tile && n > 1;
-    const uint32_t nears = __ballot_sync(0xFFFFFFFFu, near), tiles = __ballot_sync(0xFFFFFFFFu, tile);
-    if (is_rest && !tile && !near) f3_join(out, best ? f3_slot(best) : -1, row, lo, hi, s0, s1);
-    if (near) {
-        const int first = __ffs(nears) - 1;
-        int at = lane == first ? atomicAdd(ag.n_near, __popc(nears)) : 0;
-        at = __shfl_sync(nears, at, first) + __popc(nears & ((1u << lane) - 1u));
-        ag.near[at] = make_int4(row, e, n, 0);
-    }
-    if (tile) {
-        const uint32_t same = __match_any_sync(tiles, e);
-        const int first = __ffs(same) - 1;
-        int at = lane == first ? atomicAdd(&ag.rows[e], __popc(same)) : 0;
-        at = __shfl_sync(same, at, first) + __popc(same & ((1u << lane) - 1u));
-        out.rest[lo + at] = row;
-        out.best64[row] = 0ull;
-        if (at % kF3AgainRows == 0) {
-            const unsigned long long units = (unsigned long long)((s1 - s0 + kF3AgainRows - 1) / kF3AgainRows);
-            const unsigned long long was = atomicAdd(ag.tiles, (1ull << kF3UnitBits) + units);
-            const int t = (int)(was >> kF3UnitBits);
-            ag.unit0[t] = (long long)(was & ((1ull << kF3UnitBits) - 1ull));
-            ag.event[t] = e;
-            ag.place[t] = lo + at;
-            ag.done[t] = 0;
-        }
-    }
 }
 
 // A warp and its candidates' rows: lane j < nc <= G runs the chain of row `row` with row `key`.  Pieces of 16 float4s of the nc + 1
@@ -595,33 +507,117 @@ __device__ __forceinline__ float f3_chains(const float* __restrict__ feats, int 
     sm100::cp_async_wait<0>();
     return a;
 }
-// A warp's share of the tokens with a few near keys.
-__device__ __forceinline__ void f3_near(const float* __restrict__ feats, int d, int N, int Nv, const int32_t* ev_lo, const int32_t* ev_out_off,
-                                        const float* __restrict__ inv_norm, const TokenOut& out, const unsigned long long* cands, const F3Again& ag,
-                                        int first, int stride, float4* ring) {
-    const int lane = threadIdx.x & 31;
-    if (first >= Nv) return;
-    int4 x = ag.near[first];                                  // with the total, which says whether it is one
-    const int total = *ag.n_near;
-    for (int t = first; t < total;) {
-        const int n = x.z, e = x.y;
-        const int slot = lane < n ? f3_slot(cands[(size_t)x.x * (kF3Cands + 1) + lane]) : 0, row = lane < n ? out.out_src[slot] : x.x;
+// Every token to its key, and into that output's member list.  The last CTAs take the tokens without any candidate beside the
+// best key, a thread each; the first ones take the others, a warp each: the candidates that are still within the margin of the best,
+// and if there are several, their chains.  What bounds it is latency, five dependent loads and a chain of d multiply-adds, and with
+// many candidates the reading of their rows, which tokens do not share.  A tile of merge_assign_simt_kernel reads all keys of the
+// event, but for 32 tokens, and a key per token costs kF3KeysPerCand times less there (61 x 169 x 1156 in seven events, all
+// tokens: nine candidates each 57 us, all 368 keys 205; 64 x 100 x 512: ten 23, all 250 keys 55); so a token with more than kF3Few
+// candidates is left to it if that outweighs the keys that are none.  So are those whose list is full, and those with a norm
+// that is no finite number.
+// The call with frames of an event that differ by 0.1 / 0.01 / 0.001 / 0.0001, with a third of the tokens zero and with tokens
+// that are all alike but for 0.001: 61 x 169 x 1156 in one event 271 / 337 / 446 / 1560 / 285 / 1578 us, on the CUDA cores 1346
+// whatever they are; in seven 118 / 129 / 167 / 177 / 122 / 326, on the CUDA cores 257.  What is left above the CUDA cores is the
+// planes and the products that decided nothing.
+constexpr int kF3JoinWarps = 4, kF3Few = 8, kF3KeysPerCand = 12;
+__device__ __forceinline__ void f3_join(const TokenOut& out, int slot, int row, int lo, int hi, int s0, int s1) {
+    out.assign[row] = slot;
+    if (slot >= s0 && slot < s1) members_join(out.ml, slot, row, row - lo, hi - lo);
+}
+__global__ void __launch_bounds__(kF3JoinWarps * 32, 4)
+merge_join_f32_kernel(const float* __restrict__ feats, int Nv, int d, int N, const int32_t* ev_lo, int k, const int32_t* ev_out_off,
+                      const float* __restrict__ inv_norm, TokenOut out, F3Cands ca, F3Again ag, int n_suspect_ctas) {
+    grid_dep_wait();
+    __shared__ int32_t s_lo[kF3Events + 1], s_out[kF3Events + 1];
+    __shared__ float4 s_ring[kF3JoinWarps][kF3RingFloat4s];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool certain = (int)blockIdx.x >= n_suspect_ctas;
+    const int first = certain ? ((int)blockIdx.x - n_suspect_ctas) * (kF3JoinWarps * 32) + (int)threadIdx.x
+                              : (int)blockIdx.x + warp * n_suspect_ctas;   // token, or place among the suspects
+    bool todo = first < Nv;
+    int row = first, count = 0, total = 0;
+    unsigned long long best = 0;
+    if (certain) {
+        if (todo) {                                           // (a key token's are not used)
+            count = ca.count[row];
+            best = out.best64[row];
+            todo = !out.is_key[row];
+        }
+        todo = todo && (count & ~kF3NonZero) == 0;
+    } else {
+        total = *ca.n_suspects;
+        row = todo ? ca.suspects[first] : 0;                  // with the total, which says whether it is one
+    }
+    if (k <= kF3Events) {
+        for (int i = threadIdx.x; i <= k; i += kF3JoinWarps * 32) {
+            s_lo[i] = ev_lo[i];
+            s_out[i] = ev_out_off[i];
+        }
+        __syncthreads();
+        ev_lo = s_lo;
+        ev_out_off = s_out;
+    }
+    if (certain) {
+        if (!todo) return;
+        const int e = find_event(ev_lo, k, row / N), lo = ev_lo[e] * N, hi = ev_lo[e + 1] * N;
+        if (row >= lo && row < hi)                            // else a token of no event: its scratch is not this call's
+            f3_join(out, best ? f3_slot(best) : -1, row, lo, hi, ev_out_off[e], ev_out_off[e + 1]);
+        return;
+    }
+    float4* ring = s_ring[warp];
+    for (int t = first; t < total; t += n_suspect_ctas * kF3JoinWarps) {
+        if (t != first) row = ca.suspects[t];
+        count = ca.count[row];
         const float inv = inv_norm[row];
-        const int lo = ev_lo[e] * N, hi = ev_lo[e + 1] * N, s0 = ev_out_off[e], s1 = ev_out_off[e + 1];
+        best = out.best64[row];
+        unsigned long long x = ca.list[(size_t)row * (kF3Cands + 1) + lane];   // beyond the count: whatever was there
+        const int e = find_event(ev_lo, k, row / N), lo = ev_lo[e] * N, hi = ev_lo[e + 1] * N, s0 = ev_out_off[e], s1 = ev_out_off[e + 1];
+        // a row of zeros: its products are zeros, and best64 has the first key with one
+        const bool zeros = inv >= kF3TinyInv && !(count & kF3NonZero), all = count > kF3Cands && !zeros;
+        if (all || zeros || lane > count) x = 0ull;
+        if (lane == (all || zeros ? 0 : count)) x = best;     // behind the candidates
+        const bool near = x && f3_value(x) >= f3_value(best) - f3_margin(d) / inv;
+        const uint32_t set = zeros ? 1u : __ballot_sync(0xFFFFFFFFu, near);
+        const int n = __popc(set);
+        if (all || (n > kF3Few && s1 - s0 < kF3KeysPerCand * n)) {
+            if (lane == 0) {
+                const int i = atomicAdd(&ag.rows[e], 1);
+                out.rest[lo + i] = row;
+                out.best64[row] = 0ull;
+                if (i % kF3AgainRows == 0) {
+                    const unsigned long long units = (unsigned long long)((s1 - s0 + kF3AgainRows - 1) / kF3AgainRows);
+                    const unsigned long long was = atomicAdd(ag.tiles, (1ull << kF3UnitBits) + units);
+                    const int at = (int)(was >> kF3UnitBits);
+                    ag.unit0[at] = (long long)(was & ((1ull << kF3UnitBits) - 1ull));
+                    ag.event[at] = e;
+                    ag.place[at] = lo + i;
+                    ag.done[at] = 0;
+                }
+            }
+            continue;
+        }
+        if (n <= 1) {
+            if (lane == 0) f3_join(out, best ? f3_slot(best) : -1, row, lo, hi, s0, s1);
+            continue;
+        }
+        int* slots = reinterpret_cast<int*>(ring);            // the candidates to the first lanes
+        __syncwarp();
+        if (near) slots[__popc(set & ((1u << lane) - 1u))] = f3_slot(x);
+        __syncwarp();
+        const int slot = lane < n ? slots[lane] : 0, key = lane < n ? out.out_src[slot] : row;
+        const float key_inv = inv_norm[key];
         unsigned long long won = 0;
         for (int c = 0; c < n;) {
             const bool few = n - c <= 8;
-            const int nc = min(few ? 8 : 16, n - c), other = __shfl_sync(0xFFFFFFFFu, row, (c + lane) & 31);
-            const float a = few ? f3_chains<8>(feats, d, x.x, other, nc, ring) : f3_chains<16>(feats, d, x.x, other, nc, ring);
-            const float v = __shfl_sync(0xFFFFFFFFu, a, (lane - c) & 31) * inv;
+            const int nc = min(few ? 8 : 16, n - c), other = __shfl_sync(0xFFFFFFFFu, key, (c + lane) & 31);
+            const float a = few ? f3_chains<8>(feats, d, row, other, nc, ring) : f3_chains<16>(feats, d, row, other, nc, ring);
+            const float v = __shfl_sync(0xFFFFFFFFu, a, (lane - c) & 31) * key_inv;
             if (lane >= c && lane < c + nc && v > -3.4e38f) won = f3_pack(v, slot);
             c += nc;
         }
         const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(won >> 32));
         const uint32_t low = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(won >> 32) == top ? (uint32_t)won : 0u);
-        if (lane == 0) f3_join(out, top ? (int)~low : -1, x.x, lo, hi, s0, s1);
-        t += stride;
-        if (t < total) x = ag.near[t];
+        if (lane == 0) f3_join(out, top ? (int)~low : -1, row, lo, hi, s0, s1);
     }
 }
 

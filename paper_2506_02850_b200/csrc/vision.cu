@@ -582,30 +582,25 @@ namespace metok {
 // 16 x 169 tokens in two events, d = 1156: the call takes 99 us.  Larger problems go to merge_f32.cuh.
 // Units of one row meet in a 64-bit atomicMax as in the tensor-core kernel: larger value, then lower slot.
 //
-// kAgain: the tokens that merge_join_f32_kernel left (F3Again): first those with a few near keys, a warp each, then the tiles, of
-// which most calls have none; whoever does a tile's last chunk adds its tokens to the member lists.
+// kAgain: the tokens that merge_join_f32_kernel left (F3Again), none in most calls; whoever does a tile's last chunk adds its
+// tokens to the member lists.
 // --------------------------------------------------------------------------- //
 template <typename T, int PT, bool kAgain>          // PT x PT outputs per thread
 __global__ void __launch_bounds__(kSaThreads, sizeof(T) == 4 ? sa_ctas_per_sm(PT) : 4)
-merge_assign_simt_kernel(const T* __restrict__ feats, int Nv, int d, int N, const int32_t* __restrict__ ev_lo, int k,
+merge_assign_simt_kernel(const T* __restrict__ feats, int d, int N, const int32_t* __restrict__ ev_lo, int k,
                          const int32_t* __restrict__ ev_out_off, const int32_t* __restrict__ ev_unit_off,
-                         const float* __restrict__ inv_norm, int32_t* __restrict__ next, TokenOut out, const unsigned long long* cands, F3Again ag) {
+                         const float* __restrict__ inv_norm, int32_t* __restrict__ next, TokenOut out, F3Again ag) {
     grid_dep_wait();
     const int32_t *out_src = out.out_src, *rest = out.rest;
     using Tile = SimtTile<T, PT>;
     using Count = std::conditional_t<kAgain, long long, int>;
     constexpr int kSaTile = Tile::kTile, kCopies = Tile::kCopies;
     static_assert(!kAgain || kSaTile == kF3AgainRows, "the tiles that merge_join_f32_kernel opens");
-    constexpr size_t kRing = kF3RingFloat4s * sizeof(float4);
-    __shared__ __align__(16) unsigned char s_mem[kAgain ? std::max(sizeof(Tile), kSaThreads / 32 * kRing) : sizeof(Tile)];
-    Tile& tile = *reinterpret_cast<Tile*>(s_mem);
+    __shared__ __align__(16) Tile tile;
     __shared__ float s_inv[kSaTile];
     __shared__ Count s_next;
     __shared__ int s_last;
     const int tid = threadIdx.x, ty = tid >> 3, tx = tid & 7;
-    if constexpr (kAgain)
-        f3_near(feats, d, N, Nv, ev_lo, ev_out_off, inv_norm, out, cands, ag, (int)blockIdx.x + (tid >> 5) * (int)gridDim.x,
-                (int)gridDim.x * (kSaThreads / 32), reinterpret_cast<float4*>(s_mem + (tid >> 5) * kRing));
     const unsigned long long tiles = kAgain ? *ag.tiles : 0ull;
     const Count total = kAgain ? (Count)(tiles & ((1ull << kF3UnitBits) - 1ull)) : (Count)ev_unit_off[k];
     const int row_chunks = d / Tile::CE, ksteps = Tile::steps(d);
@@ -1511,8 +1506,9 @@ struct VisionWs {
     unsigned long long* cands;
     unsigned long long* key_hash;
     F3Again again;
+    int32_t *suspects, *n_suspects;
     int32_t *long_done, *avg_next, *unit_next;
-    int n_counters;           // the counters are cleared together: long, heavy, avg_next, unit_next and long_done, again's tiles, next, n_near and rows
+    int n_counters;           // the counters are cleared together: long, heavy, avg_next, unit_next and long_done, again's tiles and next, n_suspects, again's rows
 };
 
 static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, bool merging, bool planes) {
@@ -1559,9 +1555,9 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
             w.again.done = cv.take<int32_t>(tiles);
             w.again.tiles = reinterpret_cast<unsigned long long*>(w.ml.long_counter + n_again);
             w.again.next = w.again.tiles + 1;
-            w.again.n_near = w.ml.long_counter + n_again + 4;
-            w.again.rows = w.again.n_near + 1;
-            w.again.near = cv.take<int4>((size_t)Tn * N);
+            w.n_suspects = w.ml.long_counter + n_again + 4;
+            w.again.rows = w.n_suspects + 1;
+            w.suspects = cv.take<int32_t>((size_t)Tn * N);
         }
     }
     return w;
@@ -1730,7 +1726,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     }
 
     const TokenOut to = {w.is_key, out_src, out_event, assign, w.rest, w.best64, w.tile_done, w.key_hash, w.ml};
-    const F3Cands cands = {w.cands, w.tile_done, w.key_hash};
+    const F3Cands cands = {w.cands, w.tile_done, w.key_hash, w.suspects, w.n_suspects};
     {
         // an event has at most Tn - (k - 1) frames if none is empty; cs_event_topk_long takes one that has more
         const long long longest = (long long)(Tn - (k - 1)) * N;
@@ -1796,14 +1792,15 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
                 METOK_LAUNCH_CHECK();
                 {
                     METOK_TIMED("merge_join_f32_kernel", st);
-                    launch_chained(merge_join_f32_kernel, dim3(ceil_div(Nv, kF3JoinThreads)), dim3(kF3JoinThreads), 0, st, Nv, d, N, w.ev_lo,
-                                   k, w.ev_out_off, inv_norm, to, cands, w.again);
+                    const int per = kF3JoinWarps * 32, suspect_ctas = std::min(kNumSMs * 4, ceil_div(Nv, kF3JoinWarps));
+                    launch_chained(merge_join_f32_kernel, dim3(suspect_ctas + ceil_div(Nv, per)), dim3(per), 0, st, feats, Nv, d, N, w.ev_lo, k,
+                                   w.ev_out_off, inv_norm, to, cands, w.again, suspect_ctas);
                 }
                 METOK_LAUNCH_CHECK();
                 {
                     METOK_TIMED("merge_again_kernel", st);
                     launch_chained(merge_assign_simt_kernel<float, 4, true>, dim3(kNumSMs * sa_ctas_per_sm(4)), dim3(kSaThreads), 0, st, feats,
-                                   Nv, d, N, w.ev_lo, k, w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to, w.cands, w.again);
+                                   d, N, w.ev_lo, k, w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to, w.again);
                 }
                 METOK_LAUNCH_CHECK();
             }
@@ -1812,8 +1809,8 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
             {
                 METOK_TIMED("merge_assign_simt_kernel", st);
                 auto assign_units = [&](auto kernel) {
-                    launch_chained(kernel, dim3(kNumSMs * sa_ctas_per_sm(simt)), dim3(kSaThreads), 0, st, feats, Nv, d, N, w.ev_lo, k,
-                                   w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to, w.cands, w.again);
+                    launch_chained(kernel, dim3(kNumSMs * sa_ctas_per_sm(simt)), dim3(kSaThreads), 0, st, feats, d, N, w.ev_lo, k,
+                                   w.ev_out_off, w.ev_unit_off, inv_norm, w.unit_next, to, w.again);
                 };
                 if (simt == 2) assign_units(merge_assign_simt_kernel<T, 2, false>);
                 else assign_units(merge_assign_simt_kernel<T, 4, false>);
