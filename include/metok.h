@@ -232,7 +232,7 @@ typedef struct metok_vision_params {
 
 /* TOPK_MERGE keeps a member list of 512 bytes per output in the workspace: about cap * 528 + T*N * 21 bytes, and
  * up to 32 MiB (4096*d bytes if that is more) for the sums of outputs with many members; fp32 calls that merge on
- * the tensor cores up to 1 GiB and some 280 bytes per token more.  Without these they take slower kernels. */
+ * the tensor cores up to 1 GiB and some 265 bytes per token more.  Without these they take slower kernels. */
 METOK_API int    metok_compress_vision_bound(int T, int N, int k, const metok_vision_params* p);
 METOK_API size_t metok_compress_vision_workspace_bytes(int dtype, int T, int N, int d, int k, int cap,
                                              const metok_vision_params* p);
