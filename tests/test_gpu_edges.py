@@ -272,6 +272,20 @@ def test_fp32_attention_scores_at_tile_edges(Hq, Hkv, Lt, dh, vis_start, n_vis):
     assert err < 1e-5, err
 
 
+@pytest.mark.parametrize("runs", [1, 2, 31, 32, 33, 64, 65, 128])
+def test_fp32_normalisers_of_any_number_of_runs(runs):
+    """One head and two queries: a run is one tile of 32 keys; a thread adds up every other run, sixteen at a time."""
+    rng = np.random.default_rng(runs)
+    S, Lt, dh = 32 * runs, 2, 8
+    Q = (2.0 * rng.standard_normal((1, Lt, dh))).astype(np.float32)
+    K = rng.standard_normal((1, S, dh)).astype(np.float32)
+    want = O.attention_scores(Q, K, 0, S - Lt, dh ** -0.5)
+    got = B.metok_attention_scores(torch.from_numpy(Q).cuda(), torch.from_numpy(K).cuda(), 0, S - Lt, dh ** -0.5)
+    torch.cuda.synchronize()
+    err = np.abs(got.double().cpu().numpy() - want).max() / want.max()
+    assert err < 1e-5, err
+
+
 @pytest.mark.parametrize("N", [1, 15, 16, 17, 33])
 @pytest.mark.parametrize("d,dtype", [(8, "bf16"), (520, "bf16"), (516, "f32")])
 def test_segmentation_by_mean_frames_around_sixteen_rows(N, d, dtype):
