@@ -369,8 +369,8 @@ cs_topk_kernel(const float* __restrict__ scores, size_t score_stride, const int3
     const CsSlice sl = cs_slice<IT>(n_vis, rank, C);
     float added[kPlanes ? IT : 1] = {};
     if constexpr (kPlanes) add_planes<IT>(pl, n_vis, sl.i_first, sl.i_hi, added);
-    auto load = [&](int i, float& v, int& c) {
-        v = kPlanes ? added[(i - sl.i_first) >> 5] : sc[i];
+    auto load = [&](int j, int i, float& v, int& c) {
+        v = kPlanes ? added[j] : sc[i];
         c = 0;
         if (!kOne) {
             c = token_group[i];
@@ -889,7 +889,7 @@ schedule_select_kernel(const float* __restrict__ sc, int n_vis, CsLayout lay, To
     if (rank == 0 && tid == 0) schedule_check(hand);
     const int32_t* group = hand.group;
     const CsSlice sl = cs_slice<IT>(n_vis, rank, C);
-    auto load = [&](int i, float& v, int& c) {
+    auto load = [&](int, int i, float& v, int& c) {
         v = sc[i];
         c = group[i];
         if (c >= 2) c = -1;

@@ -205,7 +205,7 @@ __device__ __forceinline__ void cs_sums(const uint32_t* hist, uint32_t* coarse, 
     }
 }
 
-// Decides which items are kept.  Item j of this thread is i = i_first + 32 j, j < IT, if i < i_hi; `load(i, v, c)`
+// Decides which items are kept.  Item j of this thread is i = i_first + 32 j, j < IT, if i < i_hi; `load(j, i, v, c)`
 // gives its score and class (c < 0: it takes no part).  On return bit j of the result says whether it is kept;
 // *before is the number of items kept before this warp's first one in the whole problem, *kept the number of all;
 // sm.total[g] is the number of items of class g.  All threads of the cluster (or CTA) call it, after cs_enter().
@@ -229,7 +229,7 @@ __device__ __forceinline__ uint32_t cs_select(CsShared& sm, unsigned char* dyn, 
         for (int j = 0; j < IT; ++j) {
             cls[j] = -1;
             v[j] = 0.f;
-            if (i_first + 32 * j < i_hi) load(i_first + 32 * j, v[j], cls[j]);
+            if (i_first + 32 * j < i_hi) load(j, i_first + 32 * j, v[j], cls[j]);
         }
         for (int b = tid; b < buckets / 4; b += nthr) reinterpret_cast<uint4*>(hist)[b] = make_uint4(0u, 0u, 0u, 0u);
         if (tid == 0) { sm.busy = 0; sm.before = 0; sm.kept = 0; }

@@ -98,9 +98,11 @@ __device__ __forceinline__ int find_event(const int32_t* __restrict__ off, int k
 // The offsets are the caller's memory: they are held to [0, Tn], and where they descend (events that overlap would want
 // more outputs than the caller has room for) an offset is raised to the largest before it and the call's status word says
 // METOK_ERR_INVALID_ARG.  Events of no frames are taken as they are: no key token, no output.
+// The shape of a merge unit: up to `rows` tokens that are no key token x up to `cols` key tokens of an event.
+struct MergeShape { int rows, cols; };
 struct PlanParams {
-    int Tn, N, k, n_key_events, event_agg, mode, tile_rows, chunk_cols;
-    int rows_with_keys;                         // the merge's row tiles run over all tokens of an event (1) or only over those that are no key token (0)
+    int Tn, N, k, n_key_events, event_agg, mode;
+    MergeShape shape;
     int grid, s1, s2, s1_nonkey, s2_nonkey;     // POOL: side of the token grid and the four strides
     double keep_key, keep_nonkey, beta;
     const uint8_t* key_given;                   // the caller's key events, or null
@@ -214,8 +216,8 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
     }
     __syncthreads();
     if (pp.mode == METOK_MODE_TOPK_MERGE) {
-        auto units = [&](int m, int b, int rows, int cols) {                 // row tiles x key chunks
-            return (m - (pp.rows_with_keys ? 0 : b) + rows - 1) / rows * ((b + cols - 1) / cols);
+        auto units = [&](int m, int b, const MergeShape& s) {                // row tiles x key chunks
+            return (m - b + s.rows - 1) / s.rows * ((b + s.cols - 1) / s.cols);
         };
         for (int e = tid; e < k; e += nthr) {
             const int m = (s_off[e + 1] - s_off[e]) * pp.N;
@@ -227,7 +229,7 @@ event_plan_kernel(const float* __restrict__ token_score, float* __restrict__ fra
             if (b > m) b = m;
             ev_budget[e] = (int)b;
             s_bud[e] = (int)b;
-            s_units[e] = units(m, (int)b, pp.tile_rows, pp.chunk_cols);
+            s_units[e] = units(m, (int)b, pp.shape);
         }
         __syncthreads();
         if (tid < 32) {                                     // offsets: one warp, 32 events at a time
@@ -519,49 +521,62 @@ __device__ __noinline__ void cs_event_topk_long(unsigned char* dyn, const float*
     }
 }
 
+// What a CTA reads before event_plan_kernel, the kernel before it, has completed: the caller's offsets and the token scores.
+// They were complete when that kernel let this one start; its own results are read after the wait.
+struct TopkEvent {
+    const float* token_score;
+    const int32_t *event_offsets, *ev_lo, *ev_budget, *ev_out_off;
+    int Tn, N;
+};
+
 template <int IT, bool kCl>
 __device__ __forceinline__ void
-cs_event_topk(CsShared& sm, unsigned char* dyn, const CsLayout& lay, const float* __restrict__ sc, int lo, int n, int e,
-              int budget, int slot0, int rank, const TokenOut& out) {
+cs_event_topk(CsShared& sm, unsigned char* dyn, const CsLayout& lay, const TopkEvent& ev, int f_lo, int f_hi, int e, int rank, const TokenOut& out) {
+    const int lo = f_lo * ev.N, n = (f_hi - f_lo) * ev.N;
+    const float* sc = ev.token_score + lo;
     const CsSlice sl = cs_slice<IT>(n, rank, kCl ? kCsMaxCluster : 1);
+    float score[IT];
+#pragma unroll
+    for (int j = 0; j < IT; ++j) score[j] = sl.i_first + 32 * j < sl.i_hi ? sc[sl.i_first + 32 * j] : 0.f;
+    grid_dep_wait();
+    const int budget = ev.ev_budget[e], slot0 = ev.ev_out_off[e];
+    if (ev.ev_lo[e] != f_lo || ev.ev_lo[e + 1] != f_hi) {   // offsets that descend, which event_plan_kernel has raised
+        const int lo2 = ev.ev_lo[e] * ev.N, n2 = ev.ev_lo[e + 1] * ev.N - lo2;
+        if (rank == 0 && n2 > 0) cs_event_topk_long(dyn, ev.token_score + lo2, lo2, n2, e, budget, slot0, out);
+        return;
+    }
+    if constexpr (kCl) cs_enter<true>();
     int before, kept;
     const uint32_t bits = cs_select<IT, kCl, true>(sm, dyn, lay, 1, &budget, rank, sl.i_first, sl.i_hi,
-                                                   [&](int i, float& v, int& c) { v = sc[i]; c = 0; }, &before, &kept);
+                                                   [&](int j, int, float& v, int& c) { v = score[j]; c = 0; }, &before, &kept);
     cs_for_items<IT>(bits, before, sl.i_first, sl.i_hi,
                      [&](int, int i, int place, bool key) { token_out(out, lo, n, i, e, slot0, place, key); });
 }
 
 template <int IT, bool kCl>
 __global__ void __launch_bounds__(IT == kCsMaxItems ? kCsMaxItemsThreads : 1024)
-cs_event_topk_kernel(const float* __restrict__ token_score, const int32_t* __restrict__ ev_lo, int N,
-                     const int32_t* __restrict__ ev_budget, const int32_t* __restrict__ ev_out_off, CsLayout lay,
-                     const __grid_constant__ TokenOut out) {
-    grid_dep_wait();
+cs_event_topk_kernel(TopkEvent ev, CsLayout lay, const __grid_constant__ TokenOut out) {
     __shared__ CsShared sm;
     extern __shared__ __align__(16) unsigned char sel_dyn[];
     constexpr int C = kCl ? kCsMaxCluster : 1;
     const int e = blockIdx.x / C, rank = blockIdx.x - e * C;
-    const int lo = ev_lo[e] * N, n = ev_lo[e + 1] * N - lo;
-    if (n <= 0) return;
-    const float* sc = token_score + lo;
-    const int budget = ev_budget[e], slot0 = ev_out_off[e];
-#define METOK_EVENT_TOPK(ITEMS, CLUSTER, RANK) \
-    cs_event_topk<ITEMS, CLUSTER>(sm, sel_dyn, lay, sc, lo, n, e, budget, slot0, RANK, out)
-    if (n > IT * C * (int)blockDim.x) {
-        if (rank == 0) cs_event_topk_long(sel_dyn, sc, lo, n, e, budget, slot0, out);
-        return;
-    }
+    const int f_lo = min(max(ev.event_offsets[e], 0), ev.Tn), f_hi = min(max(ev.event_offsets[e + 1], 0), ev.Tn);
+    const int n = (f_hi - f_lo) * ev.N;
+#define METOK_EVENT_TOPK(ITEMS, CLUSTER, RANK) cs_event_topk<ITEMS, CLUSTER>(sm, sel_dyn, lay, ev, f_lo, f_hi, e, RANK, out)
     // most events are much shorter than the longest possible one: the cluster's first CTA takes them alone
     const bool solo = !kCl || n <= min(kCsSolo, 4 * (int)blockDim.x);
+    if (n <= 0 || n > IT * C * (int)blockDim.x || (solo && rank > 0)) {
+        grid_dep_wait();
+        const int lo = ev.ev_lo[e] * ev.N, m = ev.ev_lo[e + 1] * ev.N - lo;   // not n only where offsets descend
+        if (rank == 0 && m > 0) cs_event_topk_long(sel_dyn, ev.token_score + lo, lo, m, e, ev.ev_budget[e], ev.ev_out_off[e], out);
+        return;
+    }
     if (solo) {
-        if (rank == 0) {
-            if (IT != 8 || n <= 4 * (int)blockDim.x) METOK_EVENT_TOPK(4, false, 0);
-            else METOK_EVENT_TOPK(8, false, 0);
-        }
+        if (IT != 8 || n <= 4 * (int)blockDim.x) METOK_EVENT_TOPK(4, false, 0);
+        else METOK_EVENT_TOPK(8, false, 0);
         return;
     }
     if constexpr (kCl) {
-        cs_enter<true>();
         if (IT == 4 || n <= 4 * C * (int)blockDim.x) METOK_EVENT_TOPK(4, true, rank);
         else METOK_EVENT_TOPK(IT, true, rank);
     }
@@ -698,59 +713,55 @@ merge_join_kernel(int Nv, int N, const int32_t* __restrict__ ev_lo, int k, const
 // --------------------------------------------------------------------------- //
 // Merge-assign on the tensor cores (bf16).
 //
-// Work unit = up to 256 consecutive token rows of one event x one chunk of the event's
-// key tokens (up to 256 columns; an event's keys are cut into equal chunks).  The two
-// 128-row halves of a unit are two accumulators in TMEM (2 x 256 columns) that share
-// every key tile brought into shared memory: the main loop is fed at a fixed rate per
-// SM, so what counts is the work done per byte loaded -- a 256 x 256 unit needs a third
-// fewer bytes per flop than a 128 x 256 one.  The units of all events form one list; a
-// persistent CTA takes every gridDim-th unit.
-//   warp 0   : TMA producer -- per 64-wide K step one 256x64 (or, for an event's last
-//              rows, 128x64) tile of V (rows are contiguous in V), 3-stage ring that
-//              runs on across units;
-//   warps 10-13: key producers -- the chunk's key rows are rows of V scattered over the
-//              event, so their 128-byte slices come by 16-byte asynchronous copies
-//              straight from V into the ring, written in the 128-byte swizzle the MMA
-//              expects (eight threads per row, sixteen rows per thread and K step); the
-//              copies of a stage report to the stage's barrier when they have landed;
-//   warp 1   : allocates TMEM, issues tcgen05.mma (M=128, N=16..256, K=16), two per K
-//              slice (one per row half), and commits to the ring / accumulator barriers;
-//   warps 2-9: epilogue, four warps per row half -- read the accumulator with
+// Work unit = up to 256 of an event's tokens that are no key token x one chunk of the event's key tokens (up to 256
+// columns; an event's keys are cut into equal chunks).  The two 128-row halves of a unit are two accumulators in TMEM
+// (2 x 256 columns) that share every key tile brought into shared memory: the main loop is fed at a fixed rate per SM,
+// so what counts is the work done per byte loaded -- a 256 x 256 unit needs a third fewer bytes per flop than a 128 x 256
+// one.  The units of all events form one list; a persistent CTA takes every gridDim-th unit.  choose_mma_shape
+// has the units' shape.
+//   warps 9-16: producers -- both operands of a unit are rows of V scattered over the event (the key tokens and the
+//              others), so the 128-byte slices of a 64-wide K step come by 16-byte asynchronous copies straight from V
+//              into a ring that runs on across units, written in the 128-byte swizzle the MMA expects (eight threads per
+//              row); the copies of a stage report to the stage's barrier when they have landed.  (With the token rows by
+//              TMA, as boxes of consecutive rows, a fifth of the products at a keep ratio of 0.2 was spent on key tokens;
+//              512 x 144 tokens of 1024 in 64 events: 138 us under ncu, 121 now);
+//   warp 0   : allocates TMEM, issues tcgen05.mma (M=128, N=16..256, K=16), two per K slice (one per row half), and
+//              commits to the ring / accumulator barriers;
+//   warps 1-8: epilogue, four warps per accumulator -- read it with
 //              tcgen05.ld, scale each column by 1/|key|, take the (value, slot) argmax of
 //              the thread's row over the chunk, and add the row's token to its output's member
-//              list once all chunks are known.
+//              list once all chunks are known.  Units of one half take the accumulators in turn, so that the argmax of one
+//              runs beside the next one's products.
 // Chunks of one row tile may be handled by different CTAs: a row's result is combined
 // with a 64-bit atomicMax on (order-preserving key of the value) << 32 | ~slot, which
 // does not depend on the order of arrival (larger value first, then the lower slot).
 // Every wait is bounded; on a timeout the CTA unwinds and writes METOK_ERR_TIMEOUT.
 // --------------------------------------------------------------------------- //
-constexpr int kMmaBM = 256, kMmaBK = 64, kMmaBN = 256, kMmaMaxStages = 6;
-constexpr int kMmaThreads = 448;
-constexpr int kMmaKeyThreads = 128;                        // warps 10-13
+constexpr int kMmaBK = 64, kMmaBN = 256, kMmaMaxStages = 6;
+constexpr int kMmaThreads = 544;
+constexpr int kMmaProducers = 256;                         // warps 9-16
 constexpr uint32_t kMmaRingBytes = 192 * 1024;
 constexpr int kMmaEvents = 512;                            // up to as many events' offsets are kept in shared memory
 constexpr size_t kMmaSmemBytes = kMmaRingBytes + 1024;
-// Unit shape of a launch: up to bm token rows (128 or 256) x up to bn keys (a multiple of 16), and what follows from it.
-struct MmaTile {
-    int bm, bn, stages;
-    uint32_t a_bytes, stage_bytes;
-};
 
-struct MergeUnit { int row_lo, row0, row_end, col0, nvalid, nchunks, slot0, slot_end; };   // the event's first row, the unit's rows; first key slot and number of keys; the event's chunks and slots
+// row_lo, row_end: the event's tokens; place0, place_end: its list of tokens that are no key token from the unit's first on;
+// col0, nvalid: the unit's first key slot and its number of keys; the event's chunks and slots
+struct MergeUnit { int row_lo, row_end, place0, place_end, col0, nvalid, nchunks, slot0, slot_end; };
 
 __device__ __forceinline__ MergeUnit merge_unit(int u, const int32_t* ev_unit_off,
                                                 const int32_t* ev_lo,
-                                                const int32_t* ev_out_off, int k, int N, const MmaTile& mt) {
+                                                const int32_t* ev_out_off, int k, int N, const MergeShape& ms) {
     const int e = find_event(ev_unit_off, k, u);
     const int s0 = ev_out_off[e], nk = ev_out_off[e + 1] - s0;
-    const int nchunks = (nk + mt.bn - 1) / mt.bn;
+    const int nchunks = (nk + ms.cols - 1) / ms.cols;
     const int cols = (((nk + nchunks - 1) / nchunks) + 15) & ~15;       // equal chunks, whole MMA columns
     const int local = u - ev_unit_off[e];
     const int tile = local / nchunks, c = local - tile * nchunks;
     MergeUnit m;
     m.row_lo = ev_lo[e] * N;
-    m.row0 = m.row_lo + tile * mt.bm;
     m.row_end = ev_lo[e + 1] * N;
+    m.place0 = m.row_lo + tile * ms.rows;
+    m.place_end = min(m.place0 + ms.rows, m.row_end - nk);
     m.col0 = s0 + c * cols;
     m.nvalid = min(cols, nk - c * cols);
     m.nchunks = nchunks;
@@ -760,20 +771,22 @@ __device__ __forceinline__ MergeUnit merge_unit(int u, const int32_t* ev_unit_of
 }
 
 __global__ void __launch_bounds__(kMmaThreads, 1)
-merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA_half,
-                        const __nv_bfloat16* __restrict__ feats, int d, int N,
+merge_assign_mma_kernel(const __nv_bfloat16* __restrict__ feats, int d, int N,
                         const int32_t* ev_lo, int k, const int32_t* ev_out_off,
-                        const int32_t* ev_unit_off, const float* __restrict__ inv_norm, MmaTile mt,
+                        const int32_t* ev_unit_off, MergeShape ms, const float* __restrict__ inv_norm,
                         TokenOut out, int32_t* __restrict__ status) {
-    grid_dep_wait();
     using namespace sm100;
     const int32_t* out_src = out.out_src;
     extern __shared__ uint8_t smem_dyn[];
-    __shared__ __align__(8) uint64_t full_bar[kMmaMaxStages], empty_bar[kMmaMaxStages], tfull_bar, tempty_bar, drain_bar;
+    __shared__ __align__(8) uint64_t full_bar[kMmaMaxStages], empty_bar[kMmaMaxStages], tfull_bar[2], tempty_bar[2], drain_bar;
     __shared__ uint32_t s_tmem_base;
-    __shared__ int s_abort, s_last;
-    __shared__ __align__(16) float s_keyinv[2][kMmaBN];
-    const int kMmaStages = mt.stages;
+    __shared__ int s_abort, s_last[2];
+    __shared__ __align__(16) float s_keyinv[2][2][kMmaBN];    // per accumulator, alternating: a slow warp may still read the last one
+    // The set-up, up to the wait, reads only what event_plan_kernel left, which was complete when the kernel after it, the choice of
+    // the key tokens, let this one start.  (Tensor memory may be taken then, too: that kernel's CTAs, all of which have started,
+    // need none.)
+    const uint32_t a_bytes = (uint32_t)ms.rows * kMmaBK * 2, stage_bytes = a_bytes + (uint32_t)ms.cols * kMmaBK * 2;
+    const int kMmaStages = min(kMmaMaxStages, (int)(kMmaRingBytes / stage_bytes));
 
     // The events' offsets: every role looks a unit up, in a chain of log2(k) + 2 dependent reads that the copies of a
     // unit's first stages wait for (400 x 100 tokens of 512 in 100 events: 86.7 us the whole path with the reads from
@@ -792,23 +805,24 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
         ev_out_off = s_off[2];
     }
     const int total_units = ev_unit_off[k];
-    if ((int)blockIdx.x >= total_units) return;
+    if ((int)blockIdx.x >= total_units) {
+        grid_dep_wait();
+        return;
+    }
     const int ksteps = (d + kMmaBK - 1) / kMmaBK;
     const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
 
     if (threadIdx.x == 0) {
-        // a stage is full when the tile of V has landed (one arrival with its byte count) and every
-        // key-producer thread's copies have (one arrival each)
-        for (int s = 0; s < kMmaStages; ++s) { mbar_init(smem_u32(&full_bar[s]), 1 + kMmaKeyThreads); mbar_init(smem_u32(&empty_bar[s]), 1); }
-        mbar_init(smem_u32(&tfull_bar), 1);
-        mbar_init(smem_u32(&tempty_bar), 8);
+        // a stage is full when every producer thread's copies have landed (one arrival each)
+        for (int s = 0; s < kMmaStages; ++s) { mbar_init(smem_u32(&full_bar[s]), kMmaProducers); mbar_init(smem_u32(&empty_bar[s]), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&tfull_bar[b]), 1); mbar_init(smem_u32(&tempty_bar[b]), 4); }
         mbar_init(smem_u32(&drain_bar), 1);
         s_abort = 0;
         mbar_fence_init();
     }
-    if (warp == 1) {
+    if (warp == 0) {
         tmem_alloc(smem_u32(&s_tmem_base), 512);
         tmem_relinquish();
     }
@@ -817,65 +831,34 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     tc_fence_after();
     const uint32_t tmem_base = s_tmem_base;
     volatile int* abort_flag = &s_abort;
+    grid_dep_wait();
 
-    // The loops of warps 0 and 1 run once per K step with nothing to hide their latency: stage and phase are counted (no
+    // Warp 0's loop runs once per K step with nothing to hide its latency: stage and phase are counted (no
     // division), addresses and descriptor words only move by adds, and the whole warp takes every step while one elected
     // thread issues, so that all of these stay in uniform registers.  (Inside a branch of lane 0 a step cost the issuing
     // thread some 1000 clocks, as long as its products: 250 for a wait that is over, 75 per product, 100 for the commit.  The
-    // launch, 32 x 144 tokens of 1024 / 128 x 144 of 3584 / 512 x 144 of 1024: 20.5 / 49.5 / 138.5 us, 18.9 / 47.3 / 129.2 now.)
+    // launch, 32 x 144 tokens of 1024 / 128 x 144 of 3584 / 512 x 144 of 1024: 20.5 / 49.5 / 138.5 us, 18.9 / 47.3 / 129.2 so.)
     const int units = __shfl_sync(0xFFFFFFFFu, total_units, 0);
     if (warp == 0) {
-        if (elect_one()) {
-            prefetch_tmap(&tmA);
-            prefetch_tmap(&tmA_half);
-        }
-        __syncwarp();
-        int s = 0, issued = 0;
-        uint32_t ph = 0;
-        bool ok = true;
-        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
-            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
-            const int row0 = __shfl_sync(0xFFFFFFFFu, mu.row0, 0), rows = __shfl_sync(0xFFFFFFFFu, mu.row_end, 0) - row0;
-            const bool two = mt.bm > 128 && rows > 128;                   // both row halves hold rows of the event
-            const CUtensorMap* a0 = two ? &tmA : &tmA_half;
-            const uint32_t tx = (two ? 256u : 128u) * kMmaBK * 2;
-            for (int ks = 0; ks < ksteps; ++ks) {
-                if (!mbar_wait_warp(smem_u32(&empty_bar[0]) + 8u * s, ph ^ 1u, abort_flag)) { ok = false; break; }
-                const uint32_t fb = smem_u32(&full_bar[0]) + 8u * s;
-                if (elect_one()) {
-                    mbar_arrive_expect_tx(fb, tx);
-                    if (!(dbg_withhold(status, kDbgMergeAssign) && blockIdx.x == 0 && issued == 0))   // debug builds: one copy never sent
-                        tma_load_2d(smem_base + (uint32_t)s * mt.stage_bytes, a0, ks * kMmaBK, row0, fb);
-                }
-                __syncwarp();
-                ++issued;
-                if (++s == kMmaStages) { s = 0; ph ^= 1u; }
-            }
-        }
-        if (!ok) {
-            // let the copies already issued land before the CTA's shared memory goes away
-            for (int back = 1; back <= kMmaStages && back <= issued; ++back) {
-                const int j = issued - back;
-                mbar_wait_warp(smem_u32(&full_bar[j % kMmaStages]), (uint32_t)(j / kMmaStages) & 1u, abort_flag);
-            }
-        }
-    } else if (warp == 1) {
-        int s = 0, n = 0;
+        int s = 0, n = 0;                                          // n: accumulators used so far
         uint32_t ph = 0;
         bool ok = true;
         const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tmem_base, 0);
         const uint32_t a_lo0 = desc_k128_lo(smem_base);
-        const uint32_t kStageWords = mt.stage_bytes >> 4, kBWords = mt.a_bytes >> 4;
+        const uint32_t kStageWords = stage_bytes >> 4, kBWords = a_bytes >> 4;
         constexpr uint32_t kHalfWords = (128 * kMmaBK * 2) >> 4;
-        for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++n) {
-            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
-            const bool two = mt.bm > 128 && __shfl_sync(0xFFFFFFFFu, mu.row_end - mu.row0, 0) > 128;
-            if (!mbar_wait_warp(smem_u32(&tempty_bar), ((uint32_t)n & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, ms);
+            const bool two = __shfl_sync(0xFFFFFFFFu, mu.place_end - mu.place0, 0) > 128;
+            const uint32_t b0 = (uint32_t)n & 1u, b1 = b0 ^ 1u;
+            if (!mbar_wait_warp(smem_u32(&tempty_bar[0]) + 8u * b0, ((uint32_t)(n >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+            if (two && !mbar_wait_warp(smem_u32(&tempty_bar[0]) + 8u * b1, ((uint32_t)((n + 1) >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
             tc_fence_after();
+            const uint32_t d0 = tmem + b0 * kMmaBN, d1 = tmem + b1 * kMmaBN;
             const uint32_t idesc = make_idesc_bf16(128, __shfl_sync(0xFFFFFFFFu, (mu.nvalid + 15) & ~15, 0));
             for (int ks = 0; ks < ksteps; ++ks) {
                 if (!mbar_wait_warp(smem_u32(&full_bar[0]) + 8u * s, ph, abort_flag)) { ok = false; break; }
-                fence_proxy_async();                             // the key rows were written by ordinary (non-bulk) copies
+                fence_proxy_async();                             // the rows were written by ordinary (non-bulk) copies
                 tc_fence_after();
                 const uint32_t a_lo = a_lo0 + (uint32_t)s * kStageWords, b_lo = a_lo + kBWords;
                 const uint32_t acc0 = ks != 0 ? 1u : 0u;
@@ -883,144 +866,160 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
                     if (two) {                                       // rows 128..255 of the tile: 16 KiB further on
 #pragma unroll
                         for (int kk = 0; kk < kMmaBK / 16; ++kk) {
-                            umma_bf16_words(tmem, a_lo + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
-                            umma_bf16_words(tmem + kMmaBN, a_lo + kHalfWords + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
+                            umma_bf16_words(d0, a_lo + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
+                            umma_bf16_words(d1, a_lo + kHalfWords + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
                         }
                     } else {
 #pragma unroll
                         for (int kk = 0; kk < kMmaBK / 16; ++kk)
-                            umma_bf16_words(tmem, a_lo + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
+                            umma_bf16_words(d0, a_lo + 2 * kk, b_lo + 2 * kk, idesc, kk ? 1u : acc0);
                     }
                     umma_commit(smem_u32(&empty_bar[0]) + 8u * s);   // frees the stage when these MMAs retire
                 }
                 __syncwarp();
                 if (++s == kMmaStages) { s = 0; ph ^= 1u; }
             }
-            if (ok && elect_one()) umma_commit(smem_u32(&tfull_bar));   // both accumulators of this unit complete
+            if (ok && elect_one()) {                                // the accumulators of this unit are complete
+                umma_commit(smem_u32(&tfull_bar[0]) + 8u * b0);
+                if (two) umma_commit(smem_u32(&tfull_bar[0]) + 8u * b1);
+            }
             __syncwarp();
+            n += two ? 2 : 1;
         }
         if (!ok) {                                             // wait until whatever was issued has retired
             if (elect_one()) umma_commit(smem_u32(&drain_bar));
             __syncwarp();
             mbar_wait_warp(smem_u32(&drain_bar), 0u, abort_flag);
         }
-    } else if (warp >= 10) {
-        // Key producers.  Thread pt copies 16-byte chunk c = pt % 8 of the rows r = pt / 8 + 16 i,
-        // i = 0..15, of the chunk's keys: eight consecutive threads read the 128 contiguous bytes of
-        // one row's K slice.  In the swizzled tile row r lies at r * 128 bytes and its chunk c at
-        // position c ^ (r % 8).  Rows past the chunk's keys up to the next multiple of 16 (the MMA's
-        // column count) are written as zeros; rows beyond are not touched.
-        const int pt = (int)threadIdx.x - 320, c = pt & 7, rsub = pt >> 3;
-        const uint32_t dst0 = smem_base + mt.a_bytes + (uint32_t)rsub * 128u + (uint32_t)((c ^ (rsub & 7)) << 4);   // (r % 8) == (rsub % 8)
+    } else if (warp >= 9) {
+        // Producers.  Thread pt copies 16-byte chunk c = pt % 8 of the rows r = pt / 8 + 32 i, i = 0..7, of the unit's tokens
+        // and of its keys: eight consecutive threads read the 128 contiguous bytes of one row's K slice.  In the swizzled tile
+        // row r lies at r * 128 bytes and its chunk c at position c ^ (r % 8).  Keys past the chunk's up to the next multiple
+        // of 16 (the MMA's column count) are written as zeros; token rows past the unit's are not touched (what their rows of
+        // the accumulator hold is not read).
+        const int pt = (int)threadIdx.x - 288, c = pt & 7, rsub = pt >> 3;
+        const uint32_t dst0 = smem_base + (uint32_t)rsub * 128u + (uint32_t)((c ^ (rsub & 7)) << 4);   // (r % 8) == (rsub % 8)
+        const long long all = (long long)ev_lo[k] * N;
+        const char* first = reinterpret_cast<const char*>(feats) + c * 16;
         int s = 0;
         uint32_t ph = 0;
-        bool ok = true;
+        bool ok = true, withheld = dbg_withhold(status, kDbgMergeAssign) && blockIdx.x == 0 && pt == 0;   // debug builds: one copy never reported
         for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
-            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
-            const int npad = (mu.nvalid + 15) & ~15;
-            const __nv_bfloat16* src[16];
+            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, ms);
+            const int rows = mu.place_end - mu.place0, npad = (mu.nvalid + 15) & ~15;
+            // Where the thread's copies of the next step read.  The pointers move on after a step's copies: a copy holds its
+            // address registers until it has been taken in.
+            const char *row[8], *key[8];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int r = rsub + 16 * i;
-                const int row = r < mu.nvalid ? (int)dbg_bound(out_src[mu.col0 + r], (long long)ev_lo[k] * N, status) : 0;
-                src[i] = feats + (size_t)row * d + c * 8;
+            for (int i = 0; i < 8; ++i) {
+                const int r = rsub + 32 * i;
+                row[i] = first + (r < rows ? (size_t)dbg_bound(out.rest[mu.place0 + r], all, status) * d * 2 : 0);
+                key[i] = first + (r < mu.nvalid ? (size_t)dbg_bound(out_src[mu.col0 + r], all, status) * d * 2 : 0);
             }
             for (int ks = 0; ks < ksteps; ++ks) {
                 if (!mbar_wait(smem_u32(&empty_bar[0]) + 8u * s, ph ^ 1u, abort_flag)) { ok = false; break; }
-                const uint32_t dst = dst0 + (uint32_t)s * mt.stage_bytes;
-                // a K slice that reaches past d (d is a multiple of 8, not of 64) reads zeros there
+                const uint32_t dst = dst0 + (uint32_t)s * stage_bytes;
+                // a K slice that reaches past d (d is a multiple of 8, not of 64; the last step) reads zeros there
                 const bool in_k = ks * kMmaBK + c * 8 < d;
+                const uint32_t full = in_k ? 16u : 0u;
+                if (!in_k) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int r = rsub + 16 * i;
-                    if (r < npad)
-                        cp_async16_zfill(dst + (uint32_t)i * 2048u, src[i] + (in_k ? ks * kMmaBK : 0),
-                                         (r < mu.nvalid && in_k) ? 16u : 0u);
+                    for (int i = 0; i < 8; ++i) row[i] = key[i] = first;
                 }
-                cp_async_arrive_noinc(smem_u32(&full_bar[0]) + 8u * s);   // arrives when this thread's copies have landed
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (rsub + 32 * i < rows) cp_async16_zfill(dst + (uint32_t)i * 4096u, row[i], full);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int r = rsub + 32 * i;
+                    if (r < npad) cp_async16_zfill(dst + a_bytes + (uint32_t)i * 4096u, key[i], r < mu.nvalid ? full : 0u);
+                }
+                if (!withheld) cp_async_arrive_noinc(smem_u32(&full_bar[0]) + 8u * s);   // arrives when this thread's copies have landed
+                withheld = false;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    row[i] += kMmaBK * 2;
+                    key[i] += kMmaBK * 2;
+                }
                 if (++s == kMmaStages) { s = 0; ph ^= 1u; }
             }
         }
         cp_async_wait_all();                                       // nothing may land after the CTA's shared memory is gone
     } else {
         const int grp = warp & 3;                                   // TMEM lanes 32*grp .. 32*grp+31
-        const int half = (warp - 2) >> 2;                           // row half = accumulator
-        const int et = (warp - 2) * 32 + lane;                      // 0..255 among the epilogue threads
+        const int buf = (warp - 1) >> 2;                            // this warp's accumulator
+        const int et = ((warp - 1) & 3) * 32 + lane;                // 0..127 among the accumulator's threads
         bool ok = true;
-        int n = 0;
-        for (int u = blockIdx.x; u < total_units; u += gridDim.x, ++n) {
-            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, mt);
-            const int b = n & 1;                                    // s_keyinv alternates: a slow warp may still read the last one
-            s_keyinv[b][et] = (et < mu.nvalid) ? inv_norm[out_src[mu.col0 + et]] : 0.f;
-            const int row = mu.row0 + half * 128 + grp * 32 + lane;
-            const bool is_key = row >= mu.row_end || out.is_key[row];   // on its way while the products are made
-            named_bar_sync(1, 256);
-            if (ok && !mbar_wait(smem_u32(&tfull_bar), (uint32_t)n & 1u, abort_flag)) ok = false;
+        int n = 0, mine = 0;                                        // accumulators used so far, and of them this one
+        for (int u = blockIdx.x; u < total_units; u += gridDim.x) {
+            const MergeUnit mu = merge_unit(u, ev_unit_off, ev_lo, ev_out_off, k, N, ms);
+            const bool two = mu.place_end - mu.place0 > 128;
+            const int half = two ? (buf ^ n) & 1 : 0;               // the row half in this accumulator
+            const bool has_half = two || (n & 1) == buf;
+            n += two ? 2 : 1;
+            if (!has_half) continue;
+            const int b = mine & 1;
+            const uint32_t tph = (uint32_t)mine & 1u;
+            ++mine;
+            for (int i = et; i < kMmaBN; i += 128) s_keyinv[buf][b][i] = i < mu.nvalid ? inv_norm[out_src[mu.col0 + i]] : 0.f;
+            const int place_first = mu.place0 + half * 128, place = place_first + grp * 32 + lane;
+            const bool has_row = place < mu.place_end;
+            const int row = has_row ? out.rest[place] : 0;          // on its way while the products are made
+            named_bar_sync(1 + buf, 128);
+            if (ok && !mbar_wait(smem_u32(&tfull_bar[0]) + 8u * buf, tph, abort_flag)) ok = false;
             ok = __all_sync(0xFFFFFFFFu, ok);                      // tcgen05.ld below is warp-collective
-            // the second accumulator of a short unit holds nothing
-            const bool mine = half == 0 || (mt.bm > 128 && mu.row_end - mu.row0 > 128);
             float best_v = -3.4e38f;
             int best_c = 0;
             if (ok) {
                 tc_fence_after();
-                if (mine) {
-                    // Row argmax.  An element costs an instruction or two: four products and their maximum, and only if
-                    // that beats the row's best are the four kept, so that the column is found once at the end (the
-                    // first column of the first group that reached the maximum, as a scan in column order finds it).
-                    const uint32_t t_row = tmem_base + ((uint32_t)(grp * 32) << 16) + (uint32_t)half * kMmaBN;
-                    float b0 = 0.f, b1 = 0.f, b2 = 0.f;
-                    uint32_t raw[2][32];
-                    auto fold = [&](int c0, const uint32_t (&r)[32]) {
-#pragma unroll
-                        for (int j = 0; j < 32; j += 4) {
-                            const float4 ki = *reinterpret_cast<const float4*>(&s_keyinv[b][c0 + j]);
-                            const float p0 = __uint_as_float(r[j]) * ki.x, p1 = __uint_as_float(r[j + 1]) * ki.y,
-                                        p2 = __uint_as_float(r[j + 2]) * ki.z, p3 = __uint_as_float(r[j + 3]) * ki.w;
-                            const float m4 = fmaxf(fmaxf(p0, p1), fmaxf(p2, p3));
-                            if (m4 > best_v) { best_v = m4; best_c = c0 + j; b0 = p0; b1 = p1; b2 = p2; }
-                        }
-                    };
-                    const int full = mu.nvalid & ~31;
-                    if (full > 0) tmem_ld32_issue(t_row, raw[0]);
+                // Row argmax.  An element costs an instruction or two: four products and their maximum, and only if
+                // that beats the row's best are the four kept, so that the column is found once at the end (the
+                // first column of the first group that reached the maximum, as a scan in column order finds it).
+                const uint32_t t_row = tmem_base + ((uint32_t)(grp * 32) << 16) + (uint32_t)buf * kMmaBN;
+                const float* keyinv = s_keyinv[buf][b];
+                float b0 = 0.f, b1 = 0.f, b2 = 0.f;
+                const int full = mu.nvalid & ~31;
 #pragma unroll 1
-                    for (int c0 = 0; c0 < full; c0 += 64) {         // the next 32 columns are fetched while these are reduced
-                        tmem_ld32_wait(raw[0]);
-                        if (c0 + 32 < full) tmem_ld32_issue(t_row + (uint32_t)c0 + 32u, raw[1]);
-                        fold(c0, raw[0]);
-                        if (c0 + 32 < full) {
-                            tmem_ld32_wait(raw[1]);
-                            if (c0 + 64 < full) tmem_ld32_issue(t_row + (uint32_t)c0 + 64u, raw[0]);
-                            fold(c0 + 32, raw[1]);
-                        }
-                    }
-                    if (best_v > -3.4e38f) best_c += b0 == best_v ? 0 : b1 == best_v ? 1 : b2 == best_v ? 2 : 3;
-                    if (full < mu.nvalid) {
-                        float v[32];
-                        tmem_ld32(t_row + (uint32_t)full, v);
+                for (int c0 = 0; c0 < full; c0 += 32) {
+                    uint32_t r[32];
+                    tmem_ld32_issue(t_row + (uint32_t)c0, r);
+                    tmem_ld32_wait(r);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const float val = v[j] * s_keyinv[b][(full + j) & (kMmaBN - 1)];
-                            if (full + j < mu.nvalid && val > best_v) { best_v = val; best_c = full + j; }
-                        }
+                    for (int j = 0; j < 32; j += 4) {
+                        const float4 ki = *reinterpret_cast<const float4*>(&keyinv[c0 + j]);
+                        const float p0 = __uint_as_float(r[j]) * ki.x, p1 = __uint_as_float(r[j + 1]) * ki.y,
+                                    p2 = __uint_as_float(r[j + 2]) * ki.z, p3 = __uint_as_float(r[j + 3]) * ki.w;
+                        const float m4 = fmaxf(fmaxf(p0, p1), fmaxf(p2, p3));
+                        if (m4 > best_v) { best_v = m4; best_c = c0 + j; b0 = p0; b1 = p1; b2 = p2; }
+                    }
+                }
+                if (best_v > -3.4e38f) best_c += b0 == best_v ? 0 : b1 == best_v ? 1 : b2 == best_v ? 2 : 3;
+                if (full < mu.nvalid) {
+                    float v[32];
+                    tmem_ld32(t_row + (uint32_t)full, v);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const float val = v[j] * keyinv[(full + j) & (kMmaBN - 1)];
+                        if (full + j < mu.nvalid && val > best_v) { best_v = val; best_c = full + j; }
                     }
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&tempty_bar));
+                if (lane == 0) mbar_arrive(smem_u32(&tempty_bar[0]) + 8u * buf);
             }
             // (a warp that gave up keeps meeting the others at the named barriers)
-            const bool have = ok && mine && !is_key;
+            const bool have = ok && has_row;
             int slot = mu.col0 + best_c;
             bool last = true;
             if (mu.nchunks > 1) {
-                // the chunks of a row tile meet in an order-independent maximum; whoever comes last has the result
+                // the chunks of a row half meet in an order-independent maximum; whoever comes last has the result
                 if (have)
                     atomicMax(&out.best64[row], ((unsigned long long)float_key(best_v) << 32) | (unsigned long long)(~(uint32_t)slot));
                 __threadfence();
-                named_bar_sync(1, 256);
-                if (et == 0) s_last = atomicAdd(&out.tile_done[mu.row0], 1) == mu.nchunks - 1;
-                named_bar_sync(1, 256);
-                last = s_last;
+                named_bar_sync(1 + buf, 128);
+                if (et == 0) s_last[buf] = atomicAdd(&out.tile_done[place_first], 1) == mu.nchunks - 1;
+                named_bar_sync(1 + buf, 128);
+                last = s_last[buf];
                 if (have && last) {
                     __threadfence();
                     slot = (int32_t)(~(uint32_t)(__ldcg(&out.best64[row]) & 0xFFFFFFFFull));
@@ -1039,7 +1038,7 @@ merge_assign_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, 512);
+    if (warp == 0) tmem_dealloc(tmem_base, 512);
     if (threadIdx.x == 0 && s_abort) *status = METOK_ERR_TIMEOUT;
 }
 
@@ -1350,7 +1349,6 @@ __device__ __forceinline__ void avg_long(AvgRing<R>& ring, const T* __restrict__
 template <typename T, int R>
 __global__ void __launch_bounds__(kAvgThreads, kAvgCtasPerSm)
 merge_avg_kernel(const T* __restrict__ feats, T* __restrict__ out_feats, AvgArgs ar) {
-    grid_dep_wait();
     using namespace sm100;
     constexpr int VN = 16 / sizeof(T), CH = AvgRing<R>::kChunks;
     extern __shared__ uint8_t avg_dyn[];
@@ -1373,6 +1371,7 @@ merge_avg_kernel(const T* __restrict__ feats, T* __restrict__ out_feats, AvgArgs
         mbar_fence_init();
     }
     __syncthreads();
+    grid_dep_wait();
     const int n_out = *ar.n_out, n_long = *ar.ml.long_counter, n_heavy = *ar.ml.heavy_counter;
     // the outputs with many members, a CTA per item: (part, output, piece), then (output, piece)
     const int per_part = n_long * ar.nseg, n_split = per_part * kAvgParts, n_items = n_split + n_heavy * ar.nseg;
@@ -1563,38 +1562,33 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
     return w;
 }
 
-// The shape of a merge unit.  An SM is fed about 118 KB per us from L2 and a tensor instruction of 128 x bn x 16 takes
-// bn * 0.27 ns (at least 24 ns), so large units do more per byte (256 x 256: 0.56 us per K block of 64 for 64 KB) --
+// The shape of a unit of the tensor-core merge.  An SM is fed about 118 KB per us from L2 and a tensor instruction of 128 x cols x
+// 16 takes cols * 0.27 ns (at least 24 ns), so large units do more per byte (256 x 256: 0.56 us per K block of 64 for 64 KB) --
 // but a launch lasts as long as the SM with the most of them, and with few events small units spread better: 32 frames
-// of 144 tokens in four events are 40 units of 256 x 173 or 76 of 128 x 173.  The shape with the
+// of 144 tokens in four events are 28 units of 256 x 173 or 119 of 128 x 115.  The shape with the
 // shortest estimated launch is taken; 1.5 us per unit for its start and its argmax.
 // The number of units is a guess from the mean event, with half as many key chunks again for the long ones, because the
-// offsets are on the device: for the shape taken, four in five of 400 calls drawn over 4 to 512 frames lie between 0.56 and
-// 1.33 of the real number (median 1.0).  It is too high where events are of like length (32 frames: 96 for 76 units of
-// 128 x 256; 128 frames: 148 for 112 of 256 x 256) and too low for Zipf lengths (512 frames: 591 for 1468).
-static MmaTile choose_mma_tile(int Nv, int k, int d, double keep) {
-    static const struct { int bm, bn; } shapes[] = {{256, 256}, {256, 128}, {128, 256}, {128, 128}, {128, 64}};
-    const int m = ceil_div(Nv, k), keys = std::max(1, (int)(keep * m)), ksteps = ceil_div(d, kMmaBK);
-    MmaTile best = {};
+// offsets are on the device.  (The exact number for eight shapes, in event_plan_kernel, chose no better on 32, 128 and 512 frames and made that
+// kernel 1.5 to 2 us longer.)
+static MergeShape choose_mma_shape(int Nv, int k, int d, double keep) {
+    static const MergeShape shapes[] = {{256, 256}, {256, 128}, {128, 256}, {128, 128}, {128, 64}};
+    const int m = ceil_div(Nv, k), keys = std::max(1, (int)(keep * m)), rest = std::max(1, m - keys), ksteps = ceil_div(d, kMmaBK);
+    MergeShape best = {};
     double best_us = 0.0;
     for (const auto& s : shapes) {
-        const int chunks = ceil_div(keys, s.bn), cols = (ceil_div(keys, chunks) + 15) & ~15;
-        const double units = k == 1 ? (double)ceil_div(Nv, s.bm) * chunks : ((double)Nv / s.bm + 0.5 * k) * (1.5 * keys / s.bn + 0.5);
-        const double fill = (s.bm + cols) * kMmaBK * 2 / 118e3, mma = (s.bm / 128) * 4 * std::max(0.024, cols * 0.272e-3);
+        const int chunks = ceil_div(keys, s.cols), cols = (ceil_div(keys, chunks) + 15) & ~15;
+        const double units = k == 1 ? (double)ceil_div(rest, s.rows) * chunks : k * ((double)rest / s.rows + 0.5) * (1.5 * keys / s.cols + 0.5);
+        const double fill = (s.rows + cols) * kMmaBK * 2 / 118e3, mma = (s.rows / 128) * 4 * std::max(0.024, cols * 0.272e-3);
         const double us = std::ceil(units / kNumSMs) * (ksteps * std::max(fill, mma) + 1.5);
-        if (best.bm == 0 || us < 0.97 * best_us) {                  // the larger one unless it is clearly slower
+        if (best.rows == 0 || us < 0.97 * best_us) {                // the larger one unless it is clearly slower
             best_us = us;
-            best.bm = s.bm;
-            best.bn = s.bn;
+            best = s;
         }
     }
-    best.a_bytes = (uint32_t)best.bm * kMmaBK * 2;
-    best.stage_bytes = best.a_bytes + (uint32_t)best.bn * kMmaBK * 2;
-    best.stages = std::min<int>(kMmaMaxStages, kMmaRingBytes / best.stage_bytes);
     return best;
 }
 
-// The tensor-core merge path needs bf16 rows that TMA can address (16-byte row pitch);
+// The tensor-core merge path needs bf16 rows of whole 16-byte pieces;
 // METOK_DEBUG_FORCE_SIMT=1 in the environment selects the CUDA-core kernels (debugging aid).
 static bool force_simt() {
     static const bool force = [] { const char* e = getenv("METOK_DEBUG_FORCE_SIMT"); return e && e[0] == '1'; }();
@@ -1683,14 +1677,12 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         }
         METOK_LAUNCH_CHECK();
     }
-    const MmaTile tile = choose_mma_tile(Nv, k, d, keep);
     const int simt = choose_simt_outputs(Nv, k, keep);
     PlanParams pp;
     pp.Tn = Tn; pp.N = N; pp.k = k;
     pp.n_key_events = min(k, ceilq(p->alpha * (double)k));
-    pp.event_agg = p->event_agg; pp.mode = p->mode; pp.tile_rows = mma ? tile.bm : f3_bn ? kF3BM : 8 * simt;
-    pp.chunk_cols = mma ? tile.bn : f3_bn ? f3_bn : 8 * simt;
-    pp.rows_with_keys = mma ? 1 : 0;
+    pp.event_agg = p->event_agg; pp.mode = p->mode;
+    pp.shape = mma ? choose_mma_shape(Nv, k, d, keep) : f3_bn ? MergeShape{kF3BM, f3_bn} : MergeShape{8 * simt, 8 * simt};
     pp.keep_key = p->keep_key; pp.keep_nonkey = p->keep_nonkey; pp.beta = p->beta;
     pp.key_given = p->key_events_given;
     pp.key_frames_given = p->key_frames_given;
@@ -1733,10 +1725,10 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         const CsPlan plan = cs_plan(longest);
         if (plan.fits) {
             const CsLayout lay = cs_layout(1, std::max(Nv / k, 2048));          // buckets for the mean event
+            const TopkEvent ev = {token_score, event_offsets, w.ev_lo, w.ev_budget, w.ev_out_off, Tn, N};
             METOK_TIMED("event_topk_kernel", st);
             auto launch = [&](auto kernel, int C, int threads) {
-                launch_chained_clusters(C, kernel, dim3(k * C), dim3(threads), lay.bytes, st, token_score, w.ev_lo, N, w.ev_budget,
-                                        w.ev_out_off, lay, to);
+                launch_chained_clusters(C, kernel, dim3(k * C), dim3(threads), lay.bytes, st, ev, lay, to);
             };
             // One CTA per event where that holds the longest one there can be.  Clusters, most of which come down to
             // their first CTA, cost nothing while all of them are resident at once; with more events (61 of them: 488
@@ -1759,17 +1751,12 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     }
 
     if (mma) {
-        CUtensorMap tmA, tmA_half;
-        int r2 = make_tmap_bf16_2d(&tmA, feats, (uint64_t)Nv, (uint64_t)d, kMmaBM);
-        if (r2 != METOK_OK) return r2;
-        r2 = make_tmap_bf16_2d(&tmA_half, feats, (uint64_t)Nv, (uint64_t)d, kMmaBM / 2);
-        if (r2 != METOK_OK) return r2;
         METOK_ALLOW_SMEM(merge_assign_mma_kernel, kMmaSmemBytes);
         {
             METOK_TIMED("merge_assign_mma_kernel", st);
-            launch_chained(merge_assign_mma_kernel, dim3(kNumSMs), dim3(kMmaThreads), kMmaSmemBytes, st, 
-                tmA, tmA_half, reinterpret_cast<const __nv_bfloat16*>(feats), d, N, w.ev_lo, k, w.ev_out_off, w.ev_unit_off, inv_norm,
-                tile, to, w.status);
+            launch_chained(merge_assign_mma_kernel, dim3(kNumSMs), dim3(kMmaThreads), kMmaSmemBytes, st,
+                reinterpret_cast<const __nv_bfloat16*>(feats), d, N, w.ev_lo, k, w.ev_out_off, w.ev_unit_off, pp.shape, inv_norm,
+                to, w.status);
         }
         METOK_LAUNCH_CHECK();
     } else {

@@ -239,6 +239,20 @@ def test_fp32_merge_units(T, N, k, d, keep):
     assert rep["assign_mismatches"] <= rep["assign_near_ties"]
 
 
+@pytest.mark.parametrize("N,d,keep,lens", [
+    (161, 64, 0.2, [1]), (162, 72, 0.2, [1]), (321, 8, 0.2, [1]), (322, 200, 0.2, [1, 2]),             # 128, 129, 256 and 257 tokens beside the keys
+    (40, 64, 1.0, [3, 1]), (40, 64, 0.01, [1, 7]), (1, 520, 0.5, [2, 1, 5]),                            # no other token, one key, hardly any token
+    (169, 136, 0.24, [40, 1, 9, 30]), (200, 1096, 0.45, [12, 20]),                                      # several chunks of keys per tile of rows
+    (4, 72, 0.5, [1] * 520 + [9]),                                                                      # more events than fit in shared memory
+])
+def test_bf16_merge_units(N, d, keep, lens):
+    rng = np.random.default_rng(N + d)
+    V, t = (torch.from_numpy(rng.standard_normal(n).astype(np.float32)).to(torch.bfloat16).float().numpy() for n in ((sum(lens), N, d), d))
+    rep = R.compress_case(V, t, np.concatenate([[0], np.cumsum(lens)]).astype(np.int32), "bf16", 0.5, keep, keep)
+    assert rep["key_mismatches"] <= rep["key_near_ties"]
+    assert rep["assign_mismatches"] <= rep["assign_near_ties"]
+
+
 @pytest.mark.parametrize("N,keep,lens,units", [
     (170, 0.25, [9, 12, 8, 11, 5], 612), (91, 0.25, [14, 41], 735), (84, 0.3, [24, 36], 740),        # 740 to 888 units of 64 x 64
     (87, 0.25, [7, 47, 15], 888), (126, 0.25, [4, 12, 22, 23], 891), (128, 0.25, [3, 1, 10, 27, 25], 1155),   # are done as such
