@@ -102,7 +102,7 @@ __device__ __forceinline__ int find_event(const int32_t* __restrict__ off, int k
 struct MergeShape { int rows, cols; };
 struct PlanParams {
     int Tn, N, k, n_key_events, event_agg, mode;
-    MergeShape shape;
+    MergeShape shape;                           // (the tensor-core merge of bf16 takes it only where there are more than kMmaEvents events)
     int grid, s1, s2, s1_nonkey, s2_nonkey;     // POOL: side of the token grid and the four strides
     double keep_key, keep_nonkey, beta;
     const uint8_t* key_given;                   // the caller's key events, or null
@@ -717,8 +717,8 @@ merge_join_kernel(int Nv, int N, const int32_t* __restrict__ ev_lo, int k, const
 // columns; an event's keys are cut into equal chunks).  The two 128-row halves of a unit are two accumulators in TMEM
 // (2 x 256 columns) that share every key tile brought into shared memory: the main loop is fed at a fixed rate per SM,
 // so what counts is the work done per byte loaded -- a 256 x 256 unit needs a third fewer bytes per flop than a 128 x 256
-// one.  The units of all events form one list; a persistent CTA takes every gridDim-th unit.  choose_mma_shape
-// has the units' shape.
+// one.  The units of all events form one list; a persistent CTA takes every gridDim-th unit.  The
+// kernel chooses the units' shape from the events' sizes (merge_shape).
 //   warps 9-16: producers -- both operands of a unit are rows of V scattered over the event (the key tokens and the
 //              others), so the 128-byte slices of a 64-wide K step come by 16-byte asynchronous copies straight from V
 //              into a ring that runs on across units, written in the 128-byte swizzle the MMA expects (eight threads per
@@ -743,6 +743,41 @@ constexpr int kMmaProducers = 256;                         // warps 9-16
 constexpr uint32_t kMmaRingBytes = 192 * 1024;
 constexpr int kMmaEvents = 512;                            // up to as many events' offsets are kept in shared memory
 constexpr size_t kMmaSmemBytes = kMmaRingBytes + 1024;
+
+// The shapes a unit may have, preferred ones first.  Large units do more per byte, but a launch lasts as long as the SM with the most
+// of them, and with few events small units spread better.
+constexpr int kMergeShapes = 8;
+__device__ __forceinline__ MergeShape merge_shape_at(int i) {
+    return {i < 5 ? 256 : 128, i < 5 ? 256 - 32 * i : i == 5 ? 256 : i == 6 ? 128 : 64};
+}
+// Estimated time of the launch with one of them, in us, by a warp, from the events' sizes.  In a step of 64 elements the tensor core takes
+// 0.27 ns per key and K slice of 16 for 128 rows (at least 24), the copies into the SM come at 118 KB per us, and its shared
+// memory takes 128 bytes a clock (written once; 128 rows are read with all of the keys); 1.5 us for a unit's start and its argmax.
+__device__ __forceinline__ float merge_launch_us(const MergeShape& ms, const int32_t* ev_lo, const int32_t* ev_out_off, int k, int N, int ksteps) {
+    const float per_row = 1.f / (float)ms.rows, per_col = 1.f / (float)ms.cols;
+    float n = 0.f, all = 0.f, most = 0.f;
+    for (int e = threadIdx.x & 31; e < k; e += 32) {
+        const int b = ev_out_off[e + 1] - ev_out_off[e], rest = (ev_lo[e + 1] - ev_lo[e]) * N - b;
+        if (rest <= 0) continue;
+        const float tiles = ceilf((float)rest * per_row), chunks = ceilf((float)b * per_col);
+        const float blocks = min(rest, ms.rows) > 128 ? 2.f : 1.f, cols = ceilf(__fdividef((float)b, chunks) * 0.0625f) * 16.f;
+        const float rows = 128.f * blocks + cols;
+        const float mma = blocks * fmaxf(0.096f, cols * 1.09e-3f), fill = rows * (128.f / 118e3f);
+        const float smem = rows * (128.f / 243e3f) + blocks * (16384.f / 243e3f + cols * (128.f / 243e3f));
+        const float us = (float)ksteps * fmaxf(mma, fmaxf(fill, smem)) + 1.5f;
+        n += tiles * chunks;
+        all += us * (tiles * chunks);
+        most = fmaxf(most, us);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        n += __shfl_xor_sync(0xFFFFFFFFu, n, o);
+        all += __shfl_xor_sync(0xFFFFFFFFu, all, o);
+        most = fmaxf(most, __shfl_xor_sync(0xFFFFFFFFu, most, o));
+    }
+    const float rounds = ceilf(n * (1.f / (float)kNumSMs));
+    return rounds <= 1.f ? most : rounds * __fdividef(all, n);
+}
 
 // row_lo, row_end: the event's tokens; place0, place_end: its list of tokens that are no key token from the unit's first on;
 // col0, nvalid: the unit's first key slot and its number of keys; the event's chunks and slots
@@ -785,17 +820,19 @@ merge_assign_mma_kernel(const __nv_bfloat16* __restrict__ feats, int d, int N,
     // The set-up, up to the wait, reads only what event_plan_kernel left, which was complete when the kernel after it, the choice of
     // the key tokens, let this one start.  (Tensor memory may be taken then, too: that kernel's CTAs, all of which have started,
     // need none.)
-    const uint32_t a_bytes = (uint32_t)ms.rows * kMmaBK * 2, stage_bytes = a_bytes + (uint32_t)ms.cols * kMmaBK * 2;
-    const int kMmaStages = min(kMmaMaxStages, (int)(kMmaRingBytes / stage_bytes));
+    const int ksteps = (d + kMmaBK - 1) / kMmaBK;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     // The events' offsets: every role looks a unit up, in a chain of log2(k) + 2 dependent reads that the copies of a
     // unit's first stages wait for (400 x 100 tokens of 512 in 100 events: 86.7 us the whole path with the reads from
     // global memory, 85.4 from shared memory; 127 x 174 of 1992 in 19: 193.5 and 192.6).
+    // With them every CTA chooses the units' shape and counts the units, while the kernel before runs: in event_plan_kernel,
+    // which everything waits for, that took 1.5 to 2 us.
     __shared__ int32_t s_off[3][kMmaEvents + 1];
+    __shared__ float s_cost[kMergeShapes];
     if (k <= kMmaEvents) {
         for (int i = threadIdx.x; i <= k; i += kMmaThreads) {
-            const int32_t a = ev_unit_off[i], b = ev_lo[i], c = ev_out_off[i];
-            s_off[0][i] = a;
+            const int32_t b = ev_lo[i], c = ev_out_off[i];
             s_off[1][i] = b;
             s_off[2][i] = c;
         }
@@ -803,15 +840,36 @@ merge_assign_mma_kernel(const __nv_bfloat16* __restrict__ feats, int d, int N,
         ev_unit_off = s_off[0];
         ev_lo = s_off[1];
         ev_out_off = s_off[2];
+        if (warp < kMergeShapes) {
+            const float us = merge_launch_us(merge_shape_at(warp), ev_lo, ev_out_off, k, N, ksteps);
+            if (lane == 0) s_cost[warp] = us;
+        }
+        __syncthreads();
+        int best = 0;
+#pragma unroll
+        for (int i = 1; i < kMergeShapes; ++i)
+            if (s_cost[i] < 0.97f * s_cost[best]) best = i;
+        ms = merge_shape_at(best);
+        if (warp == 0) {                                            // 32 events at a time
+            int before = 0;
+            for (int e0 = 0; e0 < k; e0 += 32) {
+                const int e = e0 + lane, b = e < k ? ev_out_off[e + 1] - ev_out_off[e] : 0, rest = e < k ? (ev_lo[e + 1] - ev_lo[e]) * N - b : 0;
+                const int u = (rest + ms.rows - 1) / ms.rows * ((b + ms.cols - 1) / ms.cols);
+                const int incl = cs_warp_scan(u, lane);
+                if (e < k) s_off[0][e] = before + incl - u;
+                before += __shfl_sync(0xFFFFFFFFu, incl, 31);
+            }
+            if (lane == 0) s_off[0][k] = before;
+        }
+        __syncthreads();
     }
+    const uint32_t a_bytes = (uint32_t)ms.rows * kMmaBK * 2, stage_bytes = a_bytes + (uint32_t)ms.cols * kMmaBK * 2;
+    const int kMmaStages = min(kMmaMaxStages, (int)(kMmaRingBytes / stage_bytes));
     const int total_units = ev_unit_off[k];
     if ((int)blockIdx.x >= total_units) {
         grid_dep_wait();
         return;
     }
-    const int ksteps = (d + kMmaBK - 1) / kMmaBK;
-    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-
     const uint32_t smem_base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
 
     if (threadIdx.x == 0) {
@@ -1562,32 +1620,6 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
     return w;
 }
 
-// The shape of a unit of the tensor-core merge.  An SM is fed about 118 KB per us from L2 and a tensor instruction of 128 x cols x
-// 16 takes cols * 0.27 ns (at least 24 ns), so large units do more per byte (256 x 256: 0.56 us per K block of 64 for 64 KB) --
-// but a launch lasts as long as the SM with the most of them, and with few events small units spread better: 32 frames
-// of 144 tokens in four events are 28 units of 256 x 173 or 119 of 128 x 115.  The shape with the
-// shortest estimated launch is taken; 1.5 us per unit for its start and its argmax.
-// The number of units is a guess from the mean event, with half as many key chunks again for the long ones, because the
-// offsets are on the device.  (The exact number for eight shapes, in event_plan_kernel, chose no better on 32, 128 and 512 frames and made that
-// kernel 1.5 to 2 us longer.)
-static MergeShape choose_mma_shape(int Nv, int k, int d, double keep) {
-    static const MergeShape shapes[] = {{256, 256}, {256, 128}, {128, 256}, {128, 128}, {128, 64}};
-    const int m = ceil_div(Nv, k), keys = std::max(1, (int)(keep * m)), rest = std::max(1, m - keys), ksteps = ceil_div(d, kMmaBK);
-    MergeShape best = {};
-    double best_us = 0.0;
-    for (const auto& s : shapes) {
-        const int chunks = ceil_div(keys, s.cols), cols = (ceil_div(keys, chunks) + 15) & ~15;
-        const double units = k == 1 ? (double)ceil_div(rest, s.rows) * chunks : k * ((double)rest / s.rows + 0.5) * (1.5 * keys / s.cols + 0.5);
-        const double fill = (s.rows + cols) * kMmaBK * 2 / 118e3, mma = (s.rows / 128) * 4 * std::max(0.024, cols * 0.272e-3);
-        const double us = std::ceil(units / kNumSMs) * (ksteps * std::max(fill, mma) + 1.5);
-        if (best.rows == 0 || us < 0.97 * best_us) {                // the larger one unless it is clearly slower
-            best_us = us;
-            best = s;
-        }
-    }
-    return best;
-}
-
 // The tensor-core merge path needs bf16 rows of whole 16-byte pieces;
 // METOK_DEBUG_FORCE_SIMT=1 in the environment selects the CUDA-core kernels (debugging aid).
 static bool force_simt() {
@@ -1682,7 +1714,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     pp.Tn = Tn; pp.N = N; pp.k = k;
     pp.n_key_events = min(k, ceilq(p->alpha * (double)k));
     pp.event_agg = p->event_agg; pp.mode = p->mode;
-    pp.shape = mma ? choose_mma_shape(Nv, k, d, keep) : f3_bn ? MergeShape{kF3BM, f3_bn} : MergeShape{8 * simt, 8 * simt};
+    pp.shape = mma ? MergeShape{256, 128} : f3_bn ? MergeShape{kF3BM, f3_bn} : MergeShape{8 * simt, 8 * simt};
     pp.keep_key = p->keep_key; pp.keep_nonkey = p->keep_nonkey; pp.beta = p->beta;
     pp.key_given = p->key_events_given;
     pp.key_frames_given = p->key_frames_given;
