@@ -253,6 +253,15 @@ def test_bf16_merge_units(N, d, keep, lens):
     assert rep["assign_mismatches"] <= rep["assign_near_ties"]
 
 
+@pytest.mark.parametrize("N,lens", [(1024, [64]), (1025, [64]), (800, [41, 1, 3]), (800, [1, 84, 1])])   # 65 536 tokens in the longest event there can be, and more
+def test_key_tokens_of_very_long_events(N, lens):
+    rng = np.random.default_rng(N + len(lens))
+    V, t = (torch.from_numpy(rng.standard_normal(n).astype(np.float32)).to(torch.bfloat16).float().numpy() for n in ((sum(lens), N, 8), 8))
+    rep = R.compress_case(V, t, np.concatenate([[0], np.cumsum(lens)]).astype(np.int32), "bf16", 0.5, 0.001, 0.001)
+    assert rep["key_mismatches"] <= rep["key_near_ties"]
+    assert rep["assign_mismatches"] <= rep["assign_near_ties"]
+
+
 @pytest.mark.parametrize("N,keep,lens,units", [
     (170, 0.25, [9, 12, 8, 11, 5], 612), (91, 0.25, [14, 41], 735), (84, 0.3, [24, 36], 740),        # 740 to 888 units of 64 x 64
     (87, 0.25, [7, 47, 15], 888), (126, 0.25, [4, 12, 22, 23], 891), (128, 0.25, [3, 1, 10, 27, 25], 1155),   # are done as such
