@@ -553,8 +553,9 @@ cs_event_topk(CsShared& sm, unsigned char* dyn, const CsLayout& lay, const TopkE
                      [&](int, int i, int place, bool key) { token_out(out, lo, n, i, e, slot0, place, key); });
 }
 
-template <int IT, bool kCl>
-__global__ void __launch_bounds__(IT == kCsMaxItems ? kCsMaxItemsThreads : 1024)
+constexpr int kTopkTwoThreads = 512;    // with kCsMaxItems items each; two CTAs of so many fit an SM
+template <int IT, bool kCl, int kThreads>
+__global__ void __launch_bounds__(kThreads, kThreads == kTopkTwoThreads ? 2 : 1)
 cs_event_topk_kernel(TopkEvent ev, CsLayout lay, const __grid_constant__ TokenOut out) {
     __shared__ CsShared sm;
     extern __shared__ __align__(16) unsigned char sel_dyn[];
@@ -1765,10 +1766,14 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
             // One CTA per event where that holds the longest one there can be.  Clusters, most of which come down to
             // their first CTA, cost nothing while all of them are resident at once; with more events (61 of them: 488
             // CTAs of 1024 threads, 9 us against 6) a CTA with eight items per thread is preferred as long as it can.
-            if (plan.C == 1) launch(cs_event_topk_kernel<4, false>, 1, plan.threads);
-            else if (longest <= 2 * kCsSolo && k * plan.C > kNumSMs) launch(cs_event_topk_kernel<8, false>, 1, 1024);
-            else if (plan.items == 4) launch(cs_event_topk_kernel<4, true>, plan.C, kCsSolo / 4);
-            else launch(cs_event_topk_kernel<kCsMaxItems, true>, plan.C, kCsMaxItemsThreads);
+            if (plan.C == 1) launch(cs_event_topk_kernel<4, false, 1024>, 1, plan.threads);
+            else if (longest <= 2 * kCsSolo && k * plan.C > kNumSMs) launch(cs_event_topk_kernel<8, false, 1024>, 1, 1024);
+            else if (plan.items == 4) launch(cs_event_topk_kernel<4, true, 1024>, plan.C, kCsSolo / 4);
+            // With so many registers a CTA has an SM to itself, and 64 events are four rounds of clusters; up to 65 536 tokens
+            // in the longest event the registers of two CTAs per SM do (512 x 144 tokens of 1024 in 64 events: the path 1.3 us of 217 shorter).
+            else if (longest <= (long long)kCsMaxItems * kCsMaxCluster * kTopkTwoThreads)
+                launch(cs_event_topk_kernel<kCsMaxItems, true, kTopkTwoThreads>, plan.C, kTopkTwoThreads);
+            else launch(cs_event_topk_kernel<kCsMaxItems, true, kCsMaxItemsThreads>, plan.C, kCsMaxItemsThreads);
         } else {
             // the cache is sized for the longest event there can be, the thread count for twice the mean
             const SelectLayout lay = select_layout(1, select_items_per_cta((long long)(Tn - (k - 1)) * N));
