@@ -562,18 +562,19 @@ seg_score_kernel(const T* __restrict__ feats, const T* __restrict__ text, int Tn
         dt = warp_sum(dt);
         dp = warp_sum(dp);
         const int i = f - f0;
-        if (lane == 0) {
-            if (f < f1) {
-                const float n = fmaxf(sqrtf(nn), kEps);
-                s_nn[(i >> 5) & 1][warp][i & 31] = mine ? nn : 0.f;
-                if (mine) {
-                    token_score[row] = dt / (n * tn);
-                    inv_norm[row] = 1.0f / n;
-                }
-            }
-            if (i > 0) s_dp[((i - 1) >> 5) & 1][warp][(i - 1) & 31] = mine ? dp : 0.f;   // dot of frames f-1 and f at position p
-        }
+        if (lane == 0 && i > 0) s_dp[((i - 1) >> 5) & 1][warp][(i - 1) & 31] = mine ? dp : 0.f;   // dot of frames f-1 and f at position p
+        // A block of 32 frames is complete with the dot that reaches into the next one, and is added up before anything of the
+        // next one is written: block c + 2's first entries, in the buffers of block c, then come after the barrier of block
+        // c + 1, and whoever adds up block c has read it before that barrier.
         if (i > 0 && (i & 31) == 0) flush();
+        if (lane == 0 && f < f1) {
+            const float n = fmaxf(sqrtf(nn), kEps);
+            s_nn[(i >> 5) & 1][warp][i & 31] = mine ? nn : 0.f;
+            if (mine) {
+                token_score[row] = dt / (n * tn);
+                inv_norm[row] = 1.0f / n;
+            }
+        }
 #pragma unroll
         for (int u = 0; u < kCH; ++u) cur[u] = nxt[u];
     }

@@ -225,6 +225,37 @@ def test_one_pass_segmentation_units(T, N, d):
     assert np.allclose(got["token_inv_norm"].cpu().numpy().reshape(T, N), 1.0 / norm, rtol=1e-5)
 
 
+# A warp takes a position and a run of frames, whose sums over four positions leave the CTA 32 frames at a time.  A run is the whole video
+# where there are more positions than half of the places for warps (4144, 2368, 2368 and 1776 with the four widths of rows), a
+# third of it where they are just below a third.
+@pytest.mark.parametrize("T,N,d", [
+    (1, 1, 4), (7, 5, 260), (40, 1, 8), (9, 2, 1284), (31, 2401, 4), (32, 2402, 8), (33, 2403, 4), (64, 2404, 4), (65, 2401, 12), (66, 2405, 4),
+    (96, 2402, 4), (97, 2403, 8), (200, 2401, 4), (34, 1185, 1284), (97, 1187, 1284), (67, 1186, 1028), (66, 1186, 516),      # one run
+    (96, 1380, 4), (192, 1377, 8), (195, 1379, 4), (291, 1378, 4), (96, 592, 1284), (194, 590, 1284), (200, 784, 1028),            # three
+    (385, 257, 1284), (3000, 170, 4),
+])
+def test_one_pass_segmentation_runs_in_fp32(T, N, d):
+    g = torch.Generator(device="cuda").manual_seed(T * N + d)
+    V = torch.randn((T, N, d), device="cuda", generator=g)
+    V[1:] += 0.5 * V[:-1]
+    t = torch.randn(d, device="cuda", generator=g)
+    got = B.metok_segment_score_events(V, 1, t)
+    norm = torch.empty((T, N), dtype=torch.float64, device="cuda")
+    score, dots = torch.empty_like(norm), torch.empty(max(T - 1, 0), dtype=torch.float64, device="cuda")
+    for f in range(T):
+        x = V[f].double()
+        norm[f] = x.norm(dim=1)
+        score[f] = x @ t.double() / (norm[f] * t.double().norm())
+        if f:
+            dots[f - 1] = (x * V[f - 1].double()).sum()
+    frame = (norm ** 2).sum(1).sqrt()
+    sims = dots / (frame[:-1] * frame[1:])
+    # sums of up to N d fp32 terms in short chains
+    assert torch.allclose(got["sims"][:T - 1].double(), sims, rtol=1e-5, atol=1e-6)
+    assert torch.allclose(got["token_score"].double().reshape(T, N), score, rtol=1e-5, atol=2e-6)
+    assert torch.allclose(got["token_inv_norm"].double().reshape(T, N), 1.0 / norm, rtol=1e-5)
+
+
 @pytest.mark.parametrize("T,N,k,d,keep", [(3, 5, 3, 4, 0.4), (8, 16, 2, 64, 0.5), (13, 127, 2, 36, 0.42), (61, 169, 7, 20, 0.25), (40, 225, 3, 20, 0.3)])
 def test_fp32_merge_units(T, N, k, d, keep):
     """Units of 16 x 16, 32 x 32 and 64 x 64, one round of CTAs and more."""
