@@ -464,8 +464,12 @@ namespace metok {
 
 constexpr int kFsThreads = 128;
 
-template <typename T, int kCH>
-__global__ void __launch_bounds__(kFsThreads, 3)
+// kTogether: the warps of a CTA take neighbouring positions of the same frames, and their norms and dots are added in the CTA, in
+// warp order, so that seg_finish has a quarter of the partial sums to read (169 of them for 61 frames: 9.3 us, 6.2 with 43); an
+// idle warp of a run's last CTA repeats the last position and counts nothing.  Otherwise every warp has a position and a run of
+// its own and leaves sums of its own.
+template <typename T, int kCH, bool kTogether>
+__global__ void __launch_bounds__(kFsThreads, kCH <= 4 ? 7 : kCH <= 10 ? 4 : 3)
 seg_score_kernel(const T* __restrict__ feats, const T* __restrict__ text, int Tn, int N, int d, int frames_per_warp,
                  float* __restrict__ part_dot, float* __restrict__ part_nrm, float* __restrict__ token_score,
                  float* __restrict__ inv_norm) {
@@ -494,16 +498,15 @@ seg_score_kernel(const T* __restrict__ feats, const T* __restrict__ text, int Tn
     }
     __syncthreads();
     const float tn = s_tn;
-    // The warps of a CTA take neighbouring positions of the same frames, and their norms and dots are added here, in warp order, so
-    // that seg_finish has a quarter of the partial sums to read (169 of them for 61 frames: 9.3 us, 6.2 with 43).  An idle
-    // warp repeats the last position and counts nothing.
     constexpr int kWarps = kFsThreads / 32;
-    __shared__ float s_nn[2][kWarps][32], s_dp[2][kWarps][32];   // of 32 frames each
-    const int pgroups = (N + kWarps - 1) / kWarps;
-    const int run = blockIdx.x / pgroups, pg = blockIdx.x - run * pgroups;
-    const bool mine = pg * kWarps + warp < N;
-    const int p = mine ? pg * kWarps + warp : N - 1;
+    __shared__ float s_nn[kTogether ? 2 : 1][kWarps][32], s_dp[kTogether ? 2 : 1][kWarps][32];   // of 32 frames each
+    const int pgroups = kTogether ? (N + kWarps - 1) / kWarps : N;
+    const int at = kTogether ? blockIdx.x : blockIdx.x * kWarps + warp;
+    const int run = at / pgroups, pg = at - run * pgroups;
+    const bool mine = !kTogether || pg * kWarps + warp < N;
+    const int p = !kTogether ? pg : mine ? pg * kWarps + warp : N - 1;
     const int f0 = run * frames_per_warp;
+    if (!kTogether && f0 >= Tn) return;                     // behind the last run
     const int f1 = min(Tn, f0 + frames_per_warp);           // own frames [f0, f1)
     const int f_last = min(Tn - 1, f1);                     // halo frame for the last dot
     const uint4* base = reinterpret_cast<const uint4*>(feats);
@@ -562,14 +565,18 @@ seg_score_kernel(const T* __restrict__ feats, const T* __restrict__ text, int Tn
         dt = warp_sum(dt);
         dp = warp_sum(dp);
         const int i = f - f0;
-        if (lane == 0 && i > 0) s_dp[((i - 1) >> 5) & 1][warp][(i - 1) & 31] = mine ? dp : 0.f;   // dot of frames f-1 and f at position p
+        if (lane == 0 && i > 0) {                           // dot of frames f-1 and f at position p
+            if constexpr (kTogether) s_dp[((i - 1) >> 5) & 1][warp][(i - 1) & 31] = mine ? dp : 0.f;
+            else part_dot[(size_t)p * Tn + (f - 1)] = dp;
+        }
         // A block of 32 frames is complete with the dot that reaches into the next one, and is added up before anything of the
         // next one is written: block c + 2's first entries, in the buffers of block c, then come after the barrier of block
         // c + 1, and whoever adds up block c has read it before that barrier.
-        if (i > 0 && (i & 31) == 0) flush();
+        if (kTogether && i > 0 && (i & 31) == 0) flush();
         if (lane == 0 && f < f1) {
             const float n = fmaxf(sqrtf(nn), kEps);
-            s_nn[(i >> 5) & 1][warp][i & 31] = mine ? nn : 0.f;
+            if constexpr (kTogether) s_nn[(i >> 5) & 1][warp][i & 31] = mine ? nn : 0.f;
+            else part_nrm[(size_t)p * Tn + f] = nn;
             if (mine) {
                 token_score[row] = dt / (n * tn);
                 inv_norm[row] = 1.0f / n;
@@ -578,7 +585,7 @@ seg_score_kernel(const T* __restrict__ feats, const T* __restrict__ text, int Tn
 #pragma unroll
         for (int u = 0; u < kCH; ++u) cur[u] = nxt[u];
     }
-    while (flushed * 32 < f1 - f0) flush();
+    while (kTogether && flushed * 32 < f1 - f0) flush();
 }
 
 // D += A * B for one m16n8k16 bf16 tile, fp32 accumulators; A is a 16-byte chunk as loaded.
@@ -796,11 +803,19 @@ static int launch_seg_score(const void* feats, const void* text, int Tn, int N, 
             part_dot, part_nrm, token_score, inv_norm);
     } else {
         const size_t smem_t = (size_t)d * sizeof(float) + (size_t)(kFsThreads / 32) * d * sizeof(T);
-        nslab = ceil_div(N, kFsThreads / 32);              // both kernels add the four positions of a CTA
-        const int rc = seg_score_runs(seg_score_kernel<T, kCH>, smem_t, Tn, nslab * (kFsThreads / 32), &fpw);
+        // Few positions are few partial sums: adding them in the CTA then costs more, at its end and in idle warps, than
+        // seg_finish gains.  The call with every warp alone / together, frames x positions x width: 400 x 1 x 2048 11.0 / 12.8 us,
+        // 300 x 17 x 1156 15.0 / 16.4, 300 x 29 x 1024 16.4 / 18.4, 300 x 32 x 1156 19.7 / 20.4, 61 x 41 x 1156 11.0 / 11.4,
+        // 150 x 49 x 1156 18.7 / 17.9, 61 x 61 x 1024 11.7 / 11.0, 61 x 169 x 1156 20.5 / 18.7.
+        constexpr int kWarps = kFsThreads / 32;
+        const bool together = N >= 48;
+        auto kernel = together ? seg_score_kernel<T, kCH, true> : seg_score_kernel<T, kCH, false>;
+        if (together) nslab = ceil_div(N, kWarps);
+        const int rc = seg_score_runs(kernel, smem_t, Tn, together ? nslab * kWarps : N, &fpw);
         if (rc != METOK_OK) return rc;
+        const int runs = ceil_div(Tn, fpw);
         METOK_TIMED("seg_score_kernel", st);
-        launch_chained(seg_score_kernel<T, kCH>, dim3(nslab * ceil_div(Tn, fpw)), dim3(kFsThreads), smem_t, st,
+        launch_chained(kernel, dim3(together ? nslab * runs : ceil_div(N * runs, kWarps)), dim3(kFsThreads), smem_t, st,
             reinterpret_cast<const T*>(feats), reinterpret_cast<const T*>(text), Tn, N, d, fpw, part_dot, part_nrm,
             token_score, inv_norm);
     }

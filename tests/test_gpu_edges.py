@@ -225,14 +225,15 @@ def test_one_pass_segmentation_units(T, N, d):
     assert np.allclose(got["token_inv_norm"].cpu().numpy().reshape(T, N), 1.0 / norm, rtol=1e-5)
 
 
-# A warp takes a position and a run of frames, whose sums over four positions leave the CTA 32 frames at a time.  A run is the whole video
+# A warp takes a position and a run of frames, whose sums over four positions leave the CTA 32 frames at a time (below 48 positions
+# every warp writes its own).  A run is the whole video
 # where there are more positions than half of the places for warps (4144, 2368, 2368 and 1776 with the four widths of rows), a
 # third of it where they are just below a third.
 @pytest.mark.parametrize("T,N,d", [
     (1, 1, 4), (7, 5, 260), (40, 1, 8), (9, 2, 1284), (31, 2401, 4), (32, 2402, 8), (33, 2403, 4), (64, 2404, 4), (65, 2401, 12), (66, 2405, 4),
     (96, 2402, 4), (97, 2403, 8), (200, 2401, 4), (34, 1185, 1284), (97, 1187, 1284), (67, 1186, 1028), (66, 1186, 516),      # one run
     (96, 1380, 4), (192, 1377, 8), (195, 1379, 4), (291, 1378, 4), (96, 592, 1284), (194, 590, 1284), (200, 784, 1028),            # three
-    (385, 257, 1284), (3000, 170, 4),
+    (385, 257, 1284), (3000, 170, 4), (3000, 47, 4), (3000, 49, 8), (70, 48, 516), (64, 47, 1028), (300, 45, 1284), (8192, 3, 4),
 ])
 def test_one_pass_segmentation_runs_in_fp32(T, N, d):
     g = torch.Generator(device="cuda").manual_seed(T * N + d)
