@@ -755,7 +755,8 @@ __device__ __forceinline__ MergeShape merge_shape_at(int i) {
 // 0.27 ns per key and K slice of 16 for 128 rows (at least 24), the copies into the SM come at 118 KB per us, and its shared
 // memory takes 128 bytes a clock (written once; 128 rows are read with all of the keys); 1.5 us for a unit's start and its argmax.
 __device__ __forceinline__ float merge_launch_us(const MergeShape& ms, const int32_t* ev_lo, const int32_t* ev_out_off, int k, int N, int ksteps) {
-    const float per_row = 1.f / (float)ms.rows, per_col = 1.f / (float)ms.cols;
+    // (1 / 224 rounds up, and 672 keys would be four chunks: a little less gives the integer division's count up to 2.6 million keys)
+    const float per_row = 1.f / (float)ms.rows, per_col = 0.9999998f / (float)ms.cols;
     float n = 0.f, all = 0.f, most = 0.f;
     for (int e = threadIdx.x & 31; e < k; e += 32) {
         const int b = ev_out_off[e + 1] - ev_out_off[e], rest = (ev_lo[e + 1] - ev_lo[e]) * N - b;
