@@ -748,12 +748,23 @@ constexpr size_t kMmaSmemBytes = kMmaRingBytes + 1024;
 // The shapes a unit may have, preferred ones first.  Large units do more per byte, but a launch lasts as long as the SM with the most
 // of them, and with few events small units spread better.
 constexpr int kMergeShapes = 8;
-__device__ __forceinline__ MergeShape merge_shape_at(int i) {
+__host__ __device__ __forceinline__ MergeShape merge_shape_at(int i) {
     return {i < 5 ? 256 : 128, i < 5 ? 256 - 32 * i : i == 5 ? 256 : i == 6 ? 128 : 64};
 }
-// Estimated time of the launch with one of them, in us, by a warp, from the events' sizes.  In a step of 64 elements the tensor core takes
+__host__ __device__ __forceinline__ int merge_stages(const MergeShape& ms) {
+    const int n = (int)(kMmaRingBytes / ((uint32_t)(ms.rows + ms.cols) * kMmaBK * 2));
+    return n < kMmaMaxStages ? n : kMmaMaxStages;
+}
+// Estimated time of a unit of one or two row halves and `cols` keys, in us.  In a step of 64 elements the tensor core takes
 // 0.27 ns per key and K slice of 16 for 128 rows (at least 24), the copies into the SM come at 118 KB per us, and its shared
 // memory takes 128 bytes a clock (written once; 128 rows are read with all of the keys); 1.5 us for a unit's start and its argmax.
+__host__ __device__ __forceinline__ float merge_unit_us(float blocks, float cols, int ksteps) {
+    const float rows = 128.f * blocks + cols;
+    const float mma = blocks * fmaxf(0.096f, cols * 1.09e-3f), fill = rows * (128.f / 118e3f);
+    const float smem = rows * (128.f / 243e3f) + blocks * (16384.f / 243e3f + cols * (128.f / 243e3f));
+    return (float)ksteps * fmaxf(mma, fmaxf(fill, smem)) + 1.5f;
+}
+// Of the launch with one of the shapes, by a warp, from the events' sizes.
 __device__ __forceinline__ float merge_launch_us(const MergeShape& ms, const int32_t* ev_lo, const int32_t* ev_out_off, int k, int N, int ksteps) {
     // (1 / 224 rounds up, and 672 keys would be four chunks: a little less gives the integer division's count up to 2.6 million keys)
     const float per_row = 1.f / (float)ms.rows, per_col = 0.9999998f / (float)ms.cols;
@@ -763,10 +774,7 @@ __device__ __forceinline__ float merge_launch_us(const MergeShape& ms, const int
         if (rest <= 0) continue;
         const float tiles = ceilf((float)rest * per_row), chunks = ceilf((float)b * per_col);
         const float blocks = min(rest, ms.rows) > 128 ? 2.f : 1.f, cols = ceilf(__fdividef((float)b, chunks) * 0.0625f) * 16.f;
-        const float rows = 128.f * blocks + cols;
-        const float mma = blocks * fmaxf(0.096f, cols * 1.09e-3f), fill = rows * (128.f / 118e3f);
-        const float smem = rows * (128.f / 243e3f) + blocks * (16384.f / 243e3f + cols * (128.f / 243e3f));
-        const float us = (float)ksteps * fmaxf(mma, fmaxf(fill, smem)) + 1.5f;
+        const float us = merge_unit_us(blocks, cols, ksteps);
         n += tiles * chunks;
         all += us * (tiles * chunks);
         most = fmaxf(most, us);
@@ -866,7 +874,7 @@ merge_assign_mma_kernel(const __nv_bfloat16* __restrict__ feats, int d, int N,
         __syncthreads();
     }
     const uint32_t a_bytes = (uint32_t)ms.rows * kMmaBK * 2, stage_bytes = a_bytes + (uint32_t)ms.cols * kMmaBK * 2;
-    const int kMmaStages = min(kMmaMaxStages, (int)(kMmaRingBytes / stage_bytes));
+    const int kMmaStages = merge_stages(ms);
     const int total_units = ev_unit_off[k];
     if ((int)blockIdx.x >= total_units) {
         grid_dep_wait();
@@ -1622,6 +1630,33 @@ static VisionWs carve_vision(Carver& cv, int Tn, int N, int k, int d, int cap, b
     return w;
 }
 
+// The shape of the units where there are more events than the merge's own choice holds.  The lengths are on the device: the estimate is
+// for events of half the mean length, the mean and one and a half times it.  Shapes within 3 % of the best are told apart by the bytes
+// that the ring has in flight, in the units of the mean event.  Events x tokens of each x width, keep, the call with units of 256 x 128
+// whatever the events are / so: 513 x 2160 x 256, 0.1 1043 / 857 us, 0.3 1618 / 1255; 520 x 1568 x 512, 0.1 942 / 813, 0.3 1384 / 1207;
+// 520 x 576 x 512, 0.3 662 / 629; 600 x 288 x 3584, 0.1 771 / 772, 0.5 1203 / 1167; 600 x 64 x 1024, 0.1 76.7 / 77.1;
+// 2000 x 144 x 1024, 0.3 439 / 439.
+static MergeShape choose_merge_shape(int Nv, int k, int d, double keep) {
+    const int ksteps = ceil_div(d, kMmaBK);
+    float us[kMergeShapes], best_us = 0.f;
+    int flight[kMergeShapes];
+    for (int i = 0; i < kMergeShapes; ++i) {
+        const MergeShape ms = merge_shape_at(i);
+        us[i] = 0.f;
+        for (int half = 1; half <= 3; ++half) {
+            const int m = std::max(2, (int)((long long)Nv * half / (2LL * k))), keys = std::min(m - 1, std::max(1, (int)(keep * m + 0.5))), rest = m - keys;
+            const int chunks = ceil_div(keys, ms.cols), cols = ceil_div(keys, 16 * chunks) * 16;
+            us[i] += (float)(ceil_div(rest, ms.rows) * chunks) * merge_unit_us(std::min(rest, ms.rows) > 128 ? 2.f : 1.f, (float)cols, ksteps);
+            if (half == 2) flight[i] = merge_stages(ms) * (std::min(rest, ms.rows) + cols);
+        }
+        if (i == 0 || us[i] < best_us) best_us = us[i];
+    }
+    int best = -1;
+    for (int i = 0; i < kMergeShapes; ++i)
+        if (us[i] <= 1.03f * best_us && (best < 0 || flight[i] > flight[best])) best = i;
+    return merge_shape_at(best);
+}
+
 // The tensor-core merge path needs bf16 rows of whole 16-byte pieces;
 // METOK_DEBUG_FORCE_SIMT=1 in the environment selects the CUDA-core kernels (debugging aid).
 static bool force_simt() {
@@ -1716,7 +1751,8 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
     pp.Tn = Tn; pp.N = N; pp.k = k;
     pp.n_key_events = min(k, ceilq(p->alpha * (double)k));
     pp.event_agg = p->event_agg; pp.mode = p->mode;
-    pp.shape = mma ? MergeShape{256, 128} : f3_bn ? MergeShape{kF3BM, f3_bn} : MergeShape{8 * simt, 8 * simt};
+    if (mma) pp.shape = k > kMmaEvents ? choose_merge_shape(Nv, k, d, keep) : MergeShape{256, 128};
+    else pp.shape = f3_bn ? MergeShape{kF3BM, f3_bn} : MergeShape{8 * simt, 8 * simt};
     pp.keep_key = p->keep_key; pp.keep_nonkey = p->keep_nonkey; pp.beta = p->beta;
     pp.key_given = p->key_events_given;
     pp.key_frames_given = p->key_frames_given;

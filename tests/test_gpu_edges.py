@@ -275,7 +275,8 @@ def test_fp32_merge_units(T, N, k, d, keep):
     (161, 64, 0.2, [1]), (162, 72, 0.2, [1]), (321, 8, 0.2, [1]), (322, 200, 0.2, [1, 2]),             # 128, 129, 256 and 257 tokens beside the keys
     (40, 64, 1.0, [3, 1]), (40, 64, 0.01, [1, 7]), (1, 520, 0.5, [2, 1, 5]),                            # no other token, one key, hardly any token
     (169, 136, 0.24, [40, 1, 9, 30]), (200, 1096, 0.45, [12, 20]),                                      # several chunks of keys per tile of rows
-    (4, 72, 0.5, [1] * 520 + [9]),                                                                      # more events than fit in shared memory
+    (4, 72, 0.5, [1] * 520 + [9]), (300, 72, 0.3, [1] * 514), (100, 8, 0.9, [1] * 520 + [40]),          # more events than fit in shared memory:
+                                                                                                        # units of 128 x 128, 256 x 256 and 128 x 256
 ])
 def test_bf16_merge_units(N, d, keep, lens):
     rng = np.random.default_rng(N + d)
