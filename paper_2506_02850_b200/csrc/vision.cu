@@ -578,7 +578,9 @@ cs_event_topk_kernel(TopkEvent ev, CsLayout lay, const __grid_constant__ TokenOu
         return;
     }
     if constexpr (kCl) {
+        // (events of 18 000 in clusters of 512 threads, the call with sixteen items for all of more than four / with eight: 102.6 / 97.6 us)
         if (IT == 4 || n <= 4 * C * (int)blockDim.x) METOK_EVENT_TOPK(4, true, rank);
+        else if (IT > 8 && n <= 8 * C * (int)blockDim.x) METOK_EVENT_TOPK(8, true, rank);
         else METOK_EVENT_TOPK(IT, true, rank);
     }
 #undef METOK_EVENT_TOPK
@@ -1806,9 +1808,11 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
             if (plan.C == 1) launch(cs_event_topk_kernel<4, false, 1024>, 1, plan.threads);
             else if (longest <= 2 * kCsSolo && k * plan.C > kNumSMs) launch(cs_event_topk_kernel<8, false, 1024>, 1, 1024);
             else if (plan.items == 4) launch(cs_event_topk_kernel<4, true, 1024>, plan.C, kCsSolo / 4);
-            // With so many registers a CTA has an SM to itself, and 64 events are four rounds of clusters; up to 65 536 tokens
-            // in the longest event the registers of two CTAs per SM do (512 x 144 tokens of 1024 in 64 events: the path 1.3 us of 217 shorter).
-            else if (longest <= (long long)kCsMaxItems * kCsMaxCluster * kTopkTwoThreads)
+            // With so many registers a CTA has an SM to itself, and the clusters of more than some fifteen events (a cluster's CTAs
+            // lie in one group of SMs) take several rounds; up to 65 536 tokens in the longest event the registers of two CTAs per SM
+            // do.  One per SM / two, frames x tokens of 8, the call: 200 x 196 in 2 events 125.7 / 134.5 us, 512 x 120 in 12
+            // 77.5 / 77.4, in 15 75.1 / 75.3, in 16 72.2 / 66.1, in 48 53.5 / 50.2; 512 x 144 of 1024 in 64 the path 218.4 / 217.1.
+            else if (k * plan.C > kNumSMs * 2 / 3 && longest <= (long long)kCsMaxItems * kCsMaxCluster * kTopkTwoThreads)
                 launch(cs_event_topk_kernel<kCsMaxItems, true, kTopkTwoThreads>, plan.C, kTopkTwoThreads);
             else launch(cs_event_topk_kernel<kCsMaxItems, true, kCsMaxItemsThreads>, plan.C, kCsMaxItemsThreads);
         } else {

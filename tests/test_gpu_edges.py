@@ -286,7 +286,11 @@ def test_bf16_merge_units(N, d, keep, lens):
     assert rep["assign_mismatches"] <= rep["assign_near_ties"]
 
 
-@pytest.mark.parametrize("N,lens", [(1024, [64]), (1025, [64]), (800, [41, 1, 3]), (800, [1, 84, 1])])   # 65 536 tokens in the longest event there can be, and more
+@pytest.mark.parametrize("N,lens", [
+    (1024, [64]), (1025, [64]), (800, [41, 1, 3]), (800, [1, 84, 1]),                       # 65 536 tokens in the longest event there can be, and more
+    (1024, [20, 21, 1]), (1024, [40, 39, 1]), (1024, [41, 38, 1]),                          # few events, CTAs of 640 threads with four, eight and sixteen items
+    (1024, [1] * 12 + [16, 17, 2]), (1024, [1] * 12 + [32, 20, 1]), (1024, [1] * 12 + [33, 20, 1]),   # more of them, 512 threads
+])
 def test_key_tokens_of_very_long_events(N, lens):
     rng = np.random.default_rng(N + len(lens))
     V, t = (torch.from_numpy(rng.standard_normal(n).astype(np.float32)).to(torch.bfloat16).float().numpy() for n in ((sum(lens), N, 8), 8))
