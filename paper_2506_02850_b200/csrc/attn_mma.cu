@@ -50,7 +50,7 @@ constexpr int kCsStages = 4;
 constexpr int kCsItems = 4;               // colsum: items whose normalisers are worked out at a time
 constexpr uint32_t kCsRingBytes = 216 * 1024;   // colsum: queries of two items and up to kCsStages key tiles
 constexpr int kStMinTiles = 2;            // fewest key tiles a stats CTA is started for
-constexpr int kCsMinTiles = 3;            // the same for colsum (on average), where a schedule's levels share the launch
+constexpr int kCsMinTiles = 3;            // the same for colsum (on average)
 
 struct AttnMmaDims {
     int Hq, Hkv, Lt, S, vis_start, n_vis, R;
@@ -80,9 +80,14 @@ __host__ AttnMmaDims make_mma_dims(int Hq, int Hkv, int Lt, int S, int vis_start
     dm.cs_t0 = vis_start / kCsBM;
     dm.cs_tiles = (vis_start + n_vis - 1) / kCsBM - dm.cs_t0 + 1;
     ns = kNumSMs / (Hkv * dm.cs_nchunk);
-    // A level scored alone: a CTA per key tile while they fit a round; the kernel is then as long as its set-up and a tile.  (With at
-    // least three tiles per CTA, so that other streams' kernels find room, the call took, heads / queries / keys: 14 / 24 / 6272
-    // 23.3 us and 21.6 so, 14 / 24 / 784 18.9 and 17.9, 28 / 64 / 784 21.8 and 19.6, 28 / 32 / 2048 21.4 and 19.3, 1 / 100 / 4096 19.6 and 18.0.)
+    // A level scored alone: at least kCsMinTiles key tiles per CTA, or fewer where the launch then still leaves five eighths of the SMs to
+    // other streams' kernels, for which a CTA that is mostly set-up is SM time lost.  Heads / queries / keys, one call (graph) and a
+    // pruning call of eight streams at once, with three tiles / one / so:
+    //   14 / 24 / 6272   13.8 / 11.6 / 12.7 us    6.4 / 7.7 / 6.7        28 / 64 / 1536   14.7 / 12.3 / 13.6    6.0 / 7.3 / 6.4
+    //   28 / 64 / 784    15.6 / 13.3 / 14.4       4.0 / 4.5 / 4.1        28 / 64 / 2160   14.8 / 12.9 / 14.8    8.2 / 10.2 / 8.2
+    //   14 / 24 / 784    14.0 / 12.0 / 12.0       3.3 / 3.0 / 3.0        14 / 24 / 2048   13.3 / 11.2 / 11.2    3.4 / 3.4 / 3.4
+    // Eight 128-frame videos at once, all calls: 96.1 / 95.4 / 96.1 M visual tokens/s.
+    ns = std::min(ns, std::max(ceil_div(dm.cs_tiles, kCsMinTiles), kNumSMs * 3 / 8 / (Hkv * dm.cs_nchunk)));
     if (ns < 1) ns = 1;
     if (ns > dm.cs_tiles) ns = dm.cs_tiles;
     dm.cs_per = ceil_div(dm.cs_tiles, ns);
