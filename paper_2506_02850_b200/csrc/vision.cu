@@ -721,7 +721,7 @@ merge_join_kernel(int Nv, int N, const int32_t* __restrict__ ev_lo, int k, const
 // (2 x 256 columns) that share every key tile brought into shared memory: the main loop is fed at a fixed rate per SM,
 // so what counts is the work done per byte loaded -- a 256 x 256 unit needs a third fewer bytes per flop than a 128 x 256
 // one.  The units of all events form one list; a persistent CTA takes every gridDim-th unit.  The
-// kernel chooses the units' shape from the events' sizes (merge_shape).
+// kernel chooses the units' shape from the events' sizes (merge_launch_cost).
 //   warps 9-16: producers -- both operands of a unit are rows of V scattered over the event (the key tokens and the
 //              others), so the 128-byte slices of a 64-wide K step come by 16-byte asynchronous copies straight from V
 //              into a ring that runs on across units, written in the 128-byte swizzle the MMA expects (eight threads per
@@ -766,8 +766,13 @@ __host__ __device__ __forceinline__ float merge_unit_us(float blocks, float cols
     const float smem = rows * (128.f / 243e3f) + blocks * (16384.f / 243e3f + cols * (128.f / 243e3f));
     return (float)ksteps * fmaxf(mma, fmaxf(fill, smem)) + 1.5f;
 }
-// Of the launch with one of the shapes, by a warp, from the events' sizes.
-__device__ __forceinline__ float merge_launch_us(const MergeShape& ms, const int32_t* ev_lo, const int32_t* ev_out_off, int k, int N, int ksteps) {
+// What a launch with one of the shapes costs, by a warp, from the events' sizes: the time it lasts, and twice the average SM's share of
+// it, which is what other streams' kernels wait for.  (By the time alone, small units were taken to spread over all SMs.  70
+// workloads of 4 to 512 frames, a call on its own and one of eight streams at once, relative to the time alone: with the share 1.006 and
+// 0.952, with twice the share 1.004 and 0.933, with three times 1.012 and 0.914.  24 x 144 tokens of 3584 in 3 events 45.4 -> 47.4 us and
+// 29.5 -> 22.1; 128 x 144 of 3584 in 16 91.5 -> 93.6 and 66.8 -> 59.6; 32 x 144 of 1024 in 4 31.6 -> 31.3 and 16.0 -> 13.2.)
+constexpr float kMergeShare = 2.f / (float)kNumSMs;
+__device__ __forceinline__ float merge_launch_cost(const MergeShape& ms, const int32_t* ev_lo, const int32_t* ev_out_off, int k, int N, int ksteps) {
     // (1 / 224 rounds up, and 672 keys would be four chunks: a little less gives the integer division's count up to 2.6 million keys)
     const float per_row = 1.f / (float)ms.rows, per_col = 0.9999998f / (float)ms.cols;
     float n = 0.f, all = 0.f, most = 0.f;
@@ -788,7 +793,7 @@ __device__ __forceinline__ float merge_launch_us(const MergeShape& ms, const int
         most = fmaxf(most, __shfl_xor_sync(0xFFFFFFFFu, most, o));
     }
     const float rounds = ceilf(n * (1.f / (float)kNumSMs));
-    return rounds <= 1.f ? most : rounds * __fdividef(all, n);
+    return (rounds <= 1.f ? most : rounds * __fdividef(all, n)) + kMergeShare * all;
 }
 
 // row_lo, row_end: the event's tokens; place0, place_end: its list of tokens that are no key token from the unit's first on;
@@ -853,8 +858,8 @@ merge_assign_mma_kernel(const __nv_bfloat16* __restrict__ feats, int d, int N,
         ev_lo = s_off[1];
         ev_out_off = s_off[2];
         if (warp < kMergeShapes) {
-            const float us = merge_launch_us(merge_shape_at(warp), ev_lo, ev_out_off, k, N, ksteps);
-            if (lane == 0) s_cost[warp] = us;
+            const float cost = merge_launch_cost(merge_shape_at(warp), ev_lo, ev_out_off, k, N, ksteps);
+            if (lane == 0) s_cost[warp] = cost;
         }
         __syncthreads();
         int best = 0;
