@@ -47,15 +47,20 @@ NCU_TRAFFIC_BYTES = {
     ("segment/seg_score_kernel", "frames128"): 136150000,
     ("segment/seg_finish_kernel", "frames128"): 61952,
     ("compress/event_plan_kernel", "frames128"): 133376,
-    ("compress/merge_avg_kernel", "frames128"): 140182000,
+    ("compress/event_topk_kernel", "frames128"): 140288,
+    ("compress/merge_assign_mma_kernel", "frames128"): 137002000,
+    ("compress/merge_avg_kernel", "frames128"): 140925000,
     ("prefill1/attn_stats_mma_kernel", "frames128"): 19441152,
+    ("prefill1/attn_colsum_mma_kernel", "frames128"): 19508480,
     ("prefill1/attn_score_reduce_kernel", "frames128"): 599040,
     ("prefill1/class_topk_kernel", "frames128"): 211968,
-    ("prefill1/gather_rows_kernel", "frames128"): 55006000,
+    ("prefill1/gather_rows_kernel", "frames128"): 54023000,
     ("prefill2/attn_stats_mma_kernel", "frames128"): 7497472,
+    ("prefill2/attn_colsum_mma_kernel", "frames128"): 7580928,
     ("prefill2/class_topk_kernel", "frames128"): 310000,
     ("prefill2/gather_rows_kernel", "frames128"): 15964672,
     ("prefill3/attn_stats_mma_kernel", "frames128"): 2778880,
+    ("prefill3/attn_colsum_mma_kernel", "frames128"): 2804736,
     ("prefill3/attn_score_reduce_kernel", "frames128"): 79000,
     ("prefill3/class_topk_kernel", "frames128"): 67000,
     ("prefill3/gather_rows_kernel", "frames128"): 473088,

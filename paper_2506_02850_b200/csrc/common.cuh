@@ -51,10 +51,14 @@ struct KernelTimer {
 #define METOK_TIMED(name, st) ::metok::KernelTimer _metok_kt(name, st)
 
 // Launch with programmatic stream serialisation: the grid may be scheduled while the kernel before it
-// on the stream is still draining, and every one of its CTAs calls grid_dep_wait() before it touches
-// memory, which returns once that kernel has completed and its writes are visible.  Because every CTA
-// of every kernel launched this way waits first, completion of a kernel implies completion of all
-// kernels before it on the stream.  The launch error is picked up by METOK_LAUNCH_CHECK().
+// on the stream is still draining, and every one of its CTAs calls grid_dep_wait(), which returns once
+// that kernel has completed and its writes are visible, and which only then lets the next kernel be
+// scheduled.  So every CTA waits before it ends and before its first write to global memory, and
+// completion of a kernel implies completion of all kernels before it on the stream.  Before the wait a
+// CTA may read what was complete when the kernel before it was let go, that is, what kernels before
+// THAT one (or the caller) have written; and it may take tensor memory if the kernel before it takes
+// none.  Most kernels wait first; cs_event_topk_kernel, merge_assign_mma_kernel and merge_avg_kernel do
+// not.  The launch error is picked up by METOK_LAUNCH_CHECK().
 // `cluster` > 1 launches clusters of that many CTAs along x.
 template <typename... P, typename... A>
 inline void launch_chained_clusters(int cluster, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
@@ -81,8 +85,8 @@ inline void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t sme
 }
 
 #ifdef __CUDACC__
-// First statements of a kernel launched by launch_chained(): wait for the kernel before it, then let
-// the kernel after it be scheduled as soon as all CTAs of this one have started.
+// In a kernel launched by launch_chained(): wait for the kernel before it, then let the kernel after it
+// be scheduled as soon as all CTAs of this one have come here or ended.
 __device__ __forceinline__ void grid_dep_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

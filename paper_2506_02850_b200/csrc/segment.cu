@@ -434,10 +434,11 @@ extern "C" int metok_segment_events(const void* feats, int dtype, int T, int N, 
 // metok_segment_score_events: segmentation and the per-token text relevance of Eq. 5
 // in ONE pass over V: per token row its squared norm, its dot product with the text
 // embedding and its dot product with the same position's row of the previous frame.
-// Token score and 1/norm are final in the kernel; the per-(position, frame) norms and
-// dots are added over the positions by seg_finish in a fixed order.
+// Token score and 1/norm are final in the kernel; the norms and dots of a frame leave it as sums over four
+// neighbouring positions (of single positions in fp32 where there are few), which seg_finish adds up in a fixed order.
 //
-// fp32 rows (seg_score_kernel): a warp owns one token position and a run of frames, holds
+// fp32 rows (seg_score_kernel): a warp owns one token position and a run of frames (from 48 positions on the
+// four warps of a CTA neighbouring positions and the same frames), holds
 // the row in registers (the next row's loads in flight meanwhile) and the previous row in
 // shared memory, and takes the three sums with multiply-adds.
 //
