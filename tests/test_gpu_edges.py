@@ -188,6 +188,21 @@ def test_attention_scores_whose_logits_grow_along_the_keys(Hq, Hkv, Lt, dh, n_vi
     assert err < 2e-4, err
 
 
+@pytest.mark.parametrize("n_vis,start", [(128 * 5 + 17, 100), (128 * 6, 0), (128 * 6 + 1, 0), (128 * 18, 0), (128 * 18 + 1, 127)])
+def test_attention_scores_with_one_two_and_three_key_tiles_per_cta(n_vis, start):
+    """Eight KV heads: six CTAs each leave five eighths of the SMs; 6, 6, 7, 18 and 19 tiles of 128 keys, some short ones at the ends."""
+    H, Lt, dh = 8, 4, 64
+    rng = np.random.default_rng(n_vis)
+    Q = rng.standard_normal((H, Lt, dh)).astype(np.float32)
+    K = rng.standard_normal((H, start + n_vis + Lt, dh)).astype(np.float32)
+    Qb, Kb = (torch.from_numpy(x).to(torch.bfloat16) for x in (Q, K))
+    want = O.attention_scores(Qb.float().numpy(), Kb.float().numpy(), start, n_vis, dh ** -0.5)
+    got = B.metok_attention_scores(Qb.cuda(), Kb.cuda(), start, n_vis, dh ** -0.5)
+    torch.cuda.synchronize()
+    err = np.abs(got.double().cpu().numpy() - want).max() / want.max()  # fp32 logits of exact products, sums in short chains
+    assert err < 2e-4, err
+
+
 @pytest.mark.parametrize("octaves", [50, 100, 128, 129, 130, 200, 255, 300, 400])
 @pytest.mark.parametrize("part", [0, 3])
 def test_attention_scores_with_one_key_far_above_the_first_tile(octaves, part):
