@@ -347,9 +347,9 @@ def test_fp32_attention_scores_at_tile_edges(Hq, Hkv, Lt, dh, vis_start, n_vis):
     assert err < 1e-5, err
 
 
-@pytest.mark.parametrize("runs", [1, 2, 31, 32, 33, 64, 65, 128])
+@pytest.mark.parametrize("runs", [1, 2, 7, 8, 9, 31, 32, 33, 64, 65, 128])
 def test_fp32_normalisers_of_any_number_of_runs(runs):
-    """One head and two queries: a run is one tile of 32 keys; a thread adds up every other run, sixteen at a time."""
+    """One head and two queries: a run is one tile of 32 keys; a thread adds up every other run, sixteen at a time or, up to eight runs, four."""
     rng = np.random.default_rng(runs)
     S, Lt, dh = 32 * runs, 2, 8
     Q = (2.0 * rng.standard_normal((1, Lt, dh))).astype(np.float32)
