@@ -1666,6 +1666,17 @@ static MergeShape choose_merge_shape(int Nv, int k, int d, double keep) {
     return merge_shape_at(best);
 }
 
+// CTAs of the merge: no more than there can be units of the smallest shape where no event is empty (with more units a CTA takes several).
+// A CTA has an SM to itself and chooses the shape and counts the units before it knows whether it has one, so that in small calls
+// idle CTAs kept other streams from the SMs.  With 148 CTAs always / so, a call of eight streams at once and on its own: 9 frames x 39
+// tokens 4.5 -> 3.2 us, 18.8 -> 19.1; 32 x 21 in 11 events 5.0 -> 3.7, 19.7 -> 20.2; 6 x 147 x 1096 7.3 -> 5.9, 26.8 -> 26.9.
+static int merge_ctas(int Tn, int N, int k, const metok_vision_params* p) {
+    const double keep = std::max(p->keep_key, p->keep_nonkey), Nv = (double)Tn * N, longest = (double)(Tn - (k - 1)) * N;
+    // sum of ceil(x) ceil(y) <= sum of x y + x + y + 1, x = tokens / 128, y = keys / 64
+    const double tiles = Nv / 128, chunks = (keep * Nv + k) / 64, both = tiles * (keep * longest + 1) / 64;
+    return (int)std::min<double>(kNumSMs, both + tiles + chunks + k + 1);
+}
+
 // The tensor-core merge path needs bf16 rows of whole 16-byte pieces;
 // METOK_DEBUG_FORCE_SIMT=1 in the environment selects the CUDA-core kernels (debugging aid).
 static bool force_simt() {
@@ -1841,7 +1852,7 @@ static int launch_vision(const void* feats_, int Tn, int N, int d, const int32_t
         METOK_ALLOW_SMEM(merge_assign_mma_kernel, kMmaSmemBytes);
         {
             METOK_TIMED("merge_assign_mma_kernel", st);
-            launch_chained(merge_assign_mma_kernel, dim3(kNumSMs), dim3(kMmaThreads), kMmaSmemBytes, st,
+            launch_chained(merge_assign_mma_kernel, dim3(merge_ctas(Tn, N, k, p)), dim3(kMmaThreads), kMmaSmemBytes, st,
                 reinterpret_cast<const __nv_bfloat16*>(feats), d, N, w.ev_lo, k, w.ev_out_off, w.ev_unit_off, pp.shape, inv_norm,
                 to, w.status);
         }
